@@ -134,9 +134,9 @@ int pre_anticipate_static(int32_t n_instances, int32_t horizon, const int32_t* d
  * *d_n_requests is a DEVICE int64, read at the start and written at the end of the batch.
  *
  * Two kernels implement the call with identical results (pre_route_select picks one).  The summary
- * kernel keeps four numbers per row (largest cell, largest cell + step and where it sits, cell 0)
+ * kernel keeps a few numbers per row (largest cell + step and where it sits, cell 0)
  * that give the peak of almost every row for any arrival without reading the row, scans the few
- * rows they leave undecided, routes with a single block and waits for nobody; it takes the batch
+ * rows they leave undecided and routes with a single block; it takes the batch
  * when the context's instances fit its shared memory, every value stays below 2^32 during the
  * batch and the batch (with the waiting requests of pre_route_admit) has fewer than 2^26 entries,
  * which it checks on the device.  Otherwise the scanning kernel routes: it reads every cell
@@ -310,7 +310,7 @@ int pre_status(pre_ctx* ctx, void* stream);
 int pre_last_cuda_error(const pre_ctx* ctx);
 
 /* Which kernel routes the batches of pre_route_batch and pre_route_admit on this context: PRE_ROUTE_AUTO (default:
- * the summary kernel when the shape fits it and beta and t_mem * M are whole numbers - its fast case -, the
+ * the summary kernel when the shape fits it, the
  * scanning kernel otherwise or when the summary kernel declines a batch), PRE_ROUTE_SCAN (always the scanning kernel), PRE_ROUTE_SUMMARY (as
  * AUTO, but PRE_ESIZE here when the shape does not fit the summary kernel).  Results do not
  * depend on it. */

@@ -36,7 +36,6 @@ void release(pre_ctx* c) {
     cudaFree(c->d_fused_base);
     cudaFree(c->d_fused_sync);
     cudaFree(c->d_rs_summary);
-    cudaFree(c->d_rs_jtop);
     cudaFree(c->d_rs_over);
     cudaFree(c->d_rs_guard);
     cudaFree(c->d_rs_handled);
@@ -121,7 +120,6 @@ int pre_create(const pre_config* cfg, pre_ctx** out) {
     if (e == cudaSuccess) e = alloc_zero(&c->d_rs_handled, 1);
     if (e == cudaSuccess && c->route_summary_smem) {
         e = alloc_zero(&c->d_rs_summary, (size_t)2 * I);
-        if (e == cudaSuccess) e = alloc_zero(&c->d_rs_jtop, (size_t)I);
         if (e == cudaSuccess) e = alloc_zero(&c->d_rs_over, (size_t)I);
     }
     if (e != cudaSuccess) {

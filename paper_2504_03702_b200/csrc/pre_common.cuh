@@ -68,8 +68,7 @@ struct pre_ctx {
     int route_path;                 // PRE_ROUTE_AUTO / _SCAN / _SUMMARY
     size_t route_summary_smem;
     size_t route_summary_smem_admit;    // the same for the kernel with the admission queue
-    unsigned long long* d_rs_summary;   // [I] {token count, largest cell, largest cell + step, cell 0} per row (16 bytes)
-    uint32_t* d_rs_jtop;            // [I] the first step of a row's largest cell + step
+    unsigned long long* d_rs_summary;   // [I] {token count, largest cell + step, its first step, cell 0} per row (16 bytes)
     int32_t* d_rs_over;             // [I] steps of a row above the overload level (admission queue)
     unsigned long long* d_rs_guard; // [8] what the summarising kernel found (largest cell, totals of the batch, ...)
     int* d_rs_handled;              // 1 when the summary kernel routed the last batch, 0 when it left it to the scanning kernel

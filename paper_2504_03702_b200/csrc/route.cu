@@ -1038,16 +1038,8 @@ static void fill_route_args(RouteArgs& a, pre_ctx* ctx, const int32_t* arr_promp
     a.queue_capacity = 0; a.queue_choice = nullptr; a.hot = 0; a.many = 0.0;
 }
 
-// PRE_ROUTE_AUTO takes the summary kernel when its scores are whole numbers (beta and t_mem * M whole: one
-// integer pass per arrival); with binary64 scores its chains of binary64 operations leave it level with the
-// scanning kernel (measured: 2.83 against 3.12 us per arrival on 4,096 x 2,048 instances x steps, 2.57 against
-// 2.43 on 1,024 x 1,024), so it runs them only when it is selected outright.
-static bool pre_route_summary_wanted(const pre_ctx* ctx) {
-    if (ctx->route_path == PRE_ROUTE_SCAN) return false;
-    if (ctx->route_path == PRE_ROUTE_SUMMARY) return true;
-    const double beta = ctx->cfg.beta, theta = ctx->theta;
-    return beta == floor(beta) && theta == floor(theta) && beta <= 1048576.0 && theta < 1073741824.0;
-}
+// The summary kernel wherever the shape fits it, unless the scanning kernel was selected.
+static bool pre_route_summary_wanted(const pre_ctx* ctx) { return ctx->route_path != PRE_ROUTE_SCAN; }
 
 cudaError_t pre_launch_route(pre_ctx* ctx, const int32_t* arr_prompt, const int32_t* arr_predicted,
                              int64_t n_arrivals, int64_t* curves, int64_t* queued_p, int64_t* current_d,

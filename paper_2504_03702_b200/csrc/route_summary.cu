@@ -3,40 +3,37 @@
 // The score of an arrival (P, D) against a row c[0..H) needs one number of the row, the peak
 // of the map with the arrival's ramp added (Sec. 4.3.1 update), Dc = min(D, H):
 //     peak = max( max_{j<Dc}(c[j] + P + j),  max_{j>=Dc} c[j] ).
-// Four numbers per row decide it without reading the row in almost every case:
-//     top  = max_j (c[j] + j)          jtop = the first step where that maximum is taken
-//     rmax = max_j c[j]                c0   = c[0]
+// A few numbers per row decide it without reading the row in almost every case:
+//     top = max_j (c[j] + j)      jtop = no step below which the maximum is first taken      c0 = c[0]
 //   * Dc > jtop:  the ramp covers the step of the maximum, so max_{j<Dc}(c[j]+j) = top; and
 //                 P + top >= c[j] for every j, so   peak = P + top   exactly;
-//   * otherwise:  max(rmax, P + c0) <= peak <= P + top   (the ramp covers step 0; top bounds every step).
-// In maps of requests that are being decoded the occupancy falls as requests finish, the maximum
-// of c[j] + j sits at the first steps, and the first case is the rule.  The kernel never relies on
-// that: a row that is only bounded and could hold the smallest score is scanned cell by cell.
+//   * always:     P + c0 <= peak <= P + top  (the ramp covers step 0; top bounds every step);
+//   * P + top <= theta: no penalty whatever the peak is.
+// In maps of requests that are being decoded the occupancy falls as requests finish and the maximum of c[j] + j
+// sits at the first steps.  The kernel never relies on that: a row that is only bounded and could hold the
+// smallest score is scanned cell by cell.
 //
 // Two kernels per batch:
-//   pre_summarise_rows   one pass over the maps: the four numbers of every row, the rows' token
+//   pre_summarise_rows   one pass over the maps: the numbers of every row, the rows' token
 //                        counts (queued_p + current_d) and the guards that tell whether 32-bit
 //                        arithmetic stays exact for the whole batch;
-//   pre_route_summaries  routes the batch with ONE block: summaries in shared memory, no exchange
-//                        between blocks, hence no device-side wait on another block anywhere.
-//
-// pre_route_summaries works in rounds, one arrival and two block barriers per round, three groups of warps:
-//   score warps:  every row's score for the arrival from its summary; the warp's smallest score by a
-//                 warp reduction, the block's smallest (score, row) by a shared-memory atomic minimum
-//                 (whole-number scores) or one (score, row) per warp (binary64 scores);
-//   control warp: before the first barrier it writes the last decision's outputs, takes the pending
-//                 rows' lower bounds and walks to the next well-formed arrival; between the barriers
-//                 it decides: the pass's best row unless a pending row could do better;
-//   fold warps:   add an arrival to its row in the map (Sec. 4.3.1 update) and take the row's new
-//                 summary in the same pass - RS_LAG rounds after the decision, so that the row's
-//                 cells can be fetched a round ahead and no decision waits for a fold.
-// The instances' token counts (Sec. 4.3.3: queued prompt tokens, tokens being decoded) are brought up
-// to date once, after the last round, from the new table rows.
-// Between its decision and its fold a row is "pending": it is left out of the scoring pass and
-// represented by a lower bound of its score (its token count is exact at once; the cell that
-// held `top` only grows).  A pending row whose lower bound could win makes the round a stall:
-// nothing is decided, the folds go on, and the arrival is decided once the row is exact again.
-// The decisions are therefore the same as with every fold done at once.
+//   pre_route_summaries  routes the batch with ONE block whose warps have different jobs:
+//     deciding warp  takes the arrivals one by one.  It holds rows in registers (token count a and penalty key), takes
+//                    every row's score for the arrival, the smallest by two warp reductions, and updates the winner in
+//                    place: no other warp is in this chain.  Up to 256 instances it holds all rows.  Beyond, it holds
+//                    the at most 128 rows of a list, and a table that bounds the scores of all other rows from below:
+//                    while the best row of the list beats that bound it is the best row of all.
+//     list warps     (3, beyond 256 instances) build the next list while the present one is being used up: the rows
+//                    whose score is within a margin of the smallest one for any of eight prompt lengths, and the
+//                    bounds of the rest.  Scores only grow during a batch, so a list that is a little behind is valid.
+//     folding warps  (12) add each routed request to its row (Sec. 4.3.1 update) and take the row's new
+//                    numbers in the same pass, one warp per request; they also scan single rows for the deciding warp;
+//     io warp        reads the arrivals ahead of the decisions and writes the results behind them.
+//   Warps 0, 4, 8, ... share one of the SM's four schedulers.  The deciding warp is warp 0, the io warp warp 4, and the
+//   others of that scheduler have nothing to do: the chain of dependent instructions of warp 0 is the time of the batch.
+// Nothing in that chain waits for a fold: a row between its decision and the end of its fold is "pending" and takes
+// part with a lower bound (its token count is exact at once, its top grows by at least P).  Only when a pending row has
+// the smallest score the warp waits for that fold.  The decisions are therefore the same as with every fold done at once.
 #include "pre_common.cuh"
 
 #include <math_constants.h>
@@ -45,76 +42,28 @@
 
 namespace {
 
-constexpr int RS_FOLD_WARPS = 8;
-constexpr int RS_FOLD_THREADS = 32 * RS_FOLD_WARPS;
-constexpr int RS_CONTROL_WARP = RS_FOLD_WARPS;     // the warp after the fold warps decides; the score warps follow it
-constexpr int RS_MAX_SCORE_WARPS = 10;      // 640 threads with the fold and control warps: 96 registers per thread, no spills
-constexpr int RS_MAX_THREADS = RS_FOLD_THREADS + 32 + 32 * RS_MAX_SCORE_WARPS;
-#ifndef PRE_RS_LAG
-#define PRE_RS_LAG 3
-#endif
-constexpr int RS_LAG = PRE_RS_LAG;         // rounds between a decision and the fold of its row
-constexpr int RS_PENDING = RS_LAG + 1;     // rows that can be pending at once (and row slots in shared memory)
-// Distance between the binary32 estimate of a score and the binary64 score, relative to
-// estimate + 2 * beta * theta: eight roundings of 2^-24 each on terms that add up to at most that
-// (2^-21), taken four times as large.
-constexpr float RS_EPS = 1.9073486328125e-06f;   // 2^-19
-constexpr int RS_ROWS_PER_LANE = 16;       // rows of one score lane at most (the host picks the score warps accordingly)
+constexpr int RS_WARPS = 20;
+constexpr int RS_THREADS = 32 * RS_WARPS;
+constexpr int RS_IO_WARP = 4;
+constexpr int RS_FOLD_WARPS = 12;           // warps 1-3, 5-7, 9-11, 13-15
+constexpr int RS_LIST_WARP = 17;            // 17, 18, 19
+constexpr int RS_LIST_THREADS = 96;
+constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
+constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
+constexpr int RS_LIST_ROWS = 128;           // rows of a list (4 per lane)
+constexpr int RS_PROBES = 8;                // prompt lengths for which a list has the best rows
+// A row whose top lies further out is treated as only bounded (by c0): `jmax`, the largest jtop of the other rows, decides
+// which arrivals take the quick way (Dc > jmax).
+constexpr int RS_NEAR_DIRECT = 128, RS_NEAR_LISTS = 32;
+constexpr int RS_MAX_ROWS = 10240;          // instances up to which the context offers this router (shared memory: 20 bytes each),
+constexpr int RS_MAX_BINARY64_ROWS = 5120;  // and with binary64 scores
 constexpr int SUM_THREADS = 256;
-// whole-number scores: token count of a row that is left out of the pass (pending, or padding)
-constexpr unsigned int RS_OUT = 0xc0000000u;
-
-// named barriers (0 is __syncthreads)
+constexpr unsigned int RS_SPIN_LIMIT = 1u << 24;   // polls of shared memory (some 0.5 s) before a wait inside the block is abandoned
+constexpr int RS_NO_ROW = 0x7fffffff;
 
 // guard words written by the summarising kernel
 constexpr int GUARD_MAX_CELL = 0, GUARD_MAX_BASE = 1, GUARD_BAD = 2, GUARD_SUM_RAMP = 3, GUARD_SUM_TOKENS = 4,
-              GUARD_MAX_PD = 5, GUARD_MAX_JTOP = 6;
-
-struct __align__(16) Item {
-    int P, D, Dc;
-    int k;   // index in the batch; -1: the batch has ended
-};
-
-// {token count, rmax, top, c0} of a row; jtop is kept beside it
-typedef uint4 RowSummary;
-
-// A row between its decision and its fold.
-struct __align__(16) Pending {
-    int row;                 // -1: free
-    int P, D, Dc;            // the arrival that goes into it
-    unsigned int tokens;     // token count with the arrival (exact)
-    unsigned int top_lb;     // cell jw + jw with the arrival added: a lower bound of the new top
-    unsigned int jw;         // the step of that cell (the old jtop)
-    unsigned int rmax;       // old largest cell: a lower bound of the new one
-    unsigned int c0;         // cell 0 with the arrival added (exact)
-    unsigned int unused[3];  // (three 16-byte stores write an entry)
-};
-
-__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
-    const unsigned int d = (unsigned int)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ unsigned int warp_max_u32(unsigned int v) {
-    #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, off));
-    return v;
-}
-
-
-// Score of one instance, binary64, every operation rounded on its own (the sums of whole
-// numbers below 2^53 are exact, so adding the two token counts first changes nothing).
-__device__ __forceinline__ double summary_score(unsigned int tokens, unsigned int peak, int P, int D, double theta,
-                                                double beta) {
-    double over = __dsub_rn((double)peak, theta);
-    if (over < 0.0) over = 0.0;
-    const double l = (double)((unsigned long long)tokens + (unsigned long long)P + (unsigned long long)D);
-    return __dadd_rn(l, __dmul_rn(beta, over));
-}
-
-__device__ __forceinline__ bool better_row(double s, int i, double bs, int bi) {
-    return s < bs || (s == bs && i < bi);
-}
+              GUARD_MAX_PD = 5;
 
 struct SumArgs {
     const int64_t* curves;
@@ -124,8 +73,7 @@ struct SumArgs {
     const int32_t* arr_predicted;
     long long n_arrivals;
     int I, H;
-    RowSummary* summary;
-    uint32_t* jtop;
+    uint4* summary;                // {token count, top, step of the top, cell 0} per row
     unsigned long long* guard;
     // admission queue (pre_route_admit): steps above the overload level per row, the waiting requests' totals
     int32_t* over;                 // NULL: not wanted
@@ -174,11 +122,9 @@ __global__ void __launch_bounds__(SUM_THREADS) pre_summarise_rows(const SumArgs 
             const long long tok = q + d;
             const bool ok = q >= 0 && d >= 0 && q <= 0xffffffffLL && d <= 0xffffffffLL && tok <= 0xffffffffLL;
             if (!ok) bad = true;
-            a.summary[row] = make_uint4(ok ? (unsigned int)tok : 0u, rmax, t, (unsigned int)src[0]);
-            a.jtop[row] = jt;
+            a.summary[row] = make_uint4(ok ? (unsigned int)tok : 0u, t, jt, (unsigned int)src[0]);
             if (ok) atomicMax(a.guard + GUARD_MAX_BASE, (unsigned long long)tok);
             if (rmax) atomicMax(a.guard + GUARD_MAX_CELL, (unsigned long long)rmax);
-            if (jt) atomicMax(a.guard + GUARD_MAX_JTOP, (unsigned long long)jt);
         }
     }
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.guard + GUARD_BAD, 1ull);
@@ -233,12 +179,10 @@ struct RouteSumArgs {
     double* score;
     int I, H;
     double theta, beta;
-    const RowSummary* summary0;
-    const uint32_t* jtop0;
+    const uint4* summary0;
     const unsigned long long* guard;
     int* status;
     int* handled;   // 1: this kernel routed the batch; 0: the scanning kernel has to
-    int score_warps;
     // admission queue (ADMIT kernels only): a ring of waiting requests, entry q at (head + q) mod capacity
     int32_t* queue_prompt;
     int32_t* queue_predicted;
@@ -251,93 +195,837 @@ struct RouteSumArgs {
     const int32_t* over0;          // [I] steps above the level per row, from the summarising kernel
 };
 
+// Rows in shared memory (structure of arrays):
+//   rec    {token count, key}: the key is top (jtop below the near limit) or c0 (beyond: RS_FAR), a lower bound while the
+//          row is pending; whole-number scores keep token count + beta * (key - theta) in its place
+//   flags  jtop | RS_NOT_OVER (ADMIT: the row was not overloaded when it was last folded) | RS_FAR, or RS_PENDING
+//          (written last when a fold ends)
+//   top, c0  as of the last fold
+constexpr unsigned int RS_PENDING = 0x80000000u, RS_FAR = 0x40000000u, RS_NOT_OVER = 0x20000000u, RS_JTOP = 0xffffu;
+struct Rows {
+    uint2* rec;
+    unsigned int* flags;
+    unsigned int* top;
+    unsigned int* c0;
+};
+constexpr size_t RS_ROW_BYTES = sizeof(uint2) + 3 * sizeof(unsigned int);
 
-// CPT: cells of the folded row per fold thread (H <= CPT * RS_FOLD_THREADS).
-// VEC: H is even, so 16-byte accesses to the rows are legal.
-// The block has RS_FOLD_WARPS fold warps, the control warp and a.score_warps score warps.
-// ADMIT adds the admission queue of Sec. 4.3.3: the requests that were waiting come first; a request that
-// finds every instance overloaded (the scaler's criterion of Sec. 4.3.2: more than `many` steps of the
-// row above `hot`) is not routed and the batch stops there: what is left waits or is turned away.
-// KIND: which scores the instantiation takes, chosen by the host from beta and theta (measured: with both kinds in
-// one kernel and the choice made at run time the whole-number rounds take 6 % longer, 8 % with the queue):
-//   RS_WHOLE      whole-number scores (beta and theta whole numbers); the kernel declines the batch when the
-//                 device-side bounds do not keep every score below 2^30;
-//   RS_WHOLE_BIG  the same for more than RS_ROWS_PER_LANE rows per score lane (contexts of more than 5,120
-//                 instances): the pass goes on beyond its unrolled part;
-//   RS_BINARY64   binary64 scores, RS_ROWS_PER_LANE rows per score lane at most.
-constexpr int RS_WHOLE = 0, RS_WHOLE_BIG = 1, RS_BINARY64 = 2;
-template <int CPT, bool VEC, bool ADMIT, int KIND>
-__global__ void __launch_bounds__(RS_MAX_THREADS, 1) pre_route_summaries(const RouteSumArgs a) {
-    constexpr bool BIG = KIND == RS_WHOLE_BIG;
-    constexpr bool whole = KIND != RS_BINARY64;
+struct RsShared {
+    // what the deciding warp tells the folding warps and the io warp, read with one access
+    uint4 ctl;                              // {decisions made, scans asked for, 1: no more of either, 1: a wait was abandoned}
+    int4 items[RS_ITEMS];                   // {P, D, -, index in the batch} of the requests to route, in order
+    int4 jobs[RS_ITEMS];                    // {row, P, D, whole-number score} of the decisions
+    double score[RS_ITEMS];                 // their binary64 scores
+    int4 table[2][32];                      // by code of the prompt: {bounds of the rows outside the list}
+    int list_row[2][RS_LIST_ROWS];
+    int list_n[2];
+    unsigned int bucket_a[32], bucket_b[32];   // (list warps) smallest keys of the rows outside the list
+    int probe_t[RS_PROBES];                 // (list warps) smallest scores at the probes
+    int list_count;
+    unsigned int list_met;                  // (list warps) arrivals at their meetings
+    unsigned int lists_wanted, lists_ready;
+    unsigned int done[RS_FOLD_WARPS];       // the next decision each folding warp will fold
+    unsigned int scans_done[RS_FOLD_WARPS];
+    int scan_row[32];
+    unsigned int peak[32];
+    int scan_P, scan_Dc, scan_n;
+    unsigned int jmax;                      // largest jtop of the rows that are not far
+    unsigned int items_ready;               // items written so far
+    unsigned int items_end;                 // 1: there will be no more
+    unsigned int not_over;                  // ADMIT: rows that turned out not to be overloaded, a running count
+    int blocked;                            // ADMIT: a request found every instance overloaded ...
+    long long blocked_k;                    // ... this one
+    int mode;                               // 0: decline the batch
+    long long n0;
+    int first_bad, first_full;              // the first items dropped as malformed / for a full table
+    int warp_ok[RS_WARPS];                  // (the tail of ADMIT)
+    long long joined;
+    int any_bad;
+};
+
+__device__ __forceinline__ unsigned int smem_u32(const void* p) { return (unsigned int)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p) {
+    unsigned int v;
+    asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release(unsigned int* p, unsigned int v) {
+    asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ unsigned int ld_volatile(const unsigned int* p) {
+    unsigned int v;
+    asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 ld_volatile2(const uint2* p) {
+    uint2 v;
+    asm volatile("ld.volatile.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 ld_volatile4(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void acquire_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
+
+// A wait of a whole warp on words that other warps of this block write.  False: abandoned, here or elsewhere.
+template <typename Cond>
+__device__ __forceinline__ bool rs_wait(RsShared& sh, Cond&& ready, unsigned int nap = 0) {
+    for (unsigned int polls = 0; !__all_sync(0xffffffffu, ready()); ++polls) {   // (all lanes take the same way)
+        if ((polls & 255u) == 255u && __any_sync(0xffffffffu, ld_volatile(&sh.ctl.w) != 0)) return false;
+        if (polls > RS_SPIN_LIMIT) { st_release(&sh.ctl.w, 1u); return false; }
+        if (nap) __nanosleep(nap);
+    }
+    return true;
+}
+
+// ---- Scores.  Whole-number scores (beta and theta whole numbers, every possible score below 2^30: each binary64
+// operation is exact and the score is the same number in 32-bit integer arithmetic, taken here without the arrival's
+// own P + D), and binary64 scores (each operation rounded on its own; bounds of the rows outside the list in binary32,
+// rounded down).
+// S: a score.  X: what is kept per row beside the token count.  K: bounds.
+template <bool WHOLE> struct Scores;
+
+template <> struct Scores<true> {
+    typedef unsigned int S;
+    typedef int K;
+    static __device__ __forceinline__ S none() { return 0xffffffffu; }
+    static __device__ __forceinline__ K no_a() { return 0x60000000; }
+    static __device__ __forceinline__ K no_b() { return 0x3fffffff; }    // (room for beta * P on top)
+    static __device__ __forceinline__ K lowest() { return -0x40000000; }
+    int theta, beta, code_base;
+    __device__ __forceinline__ void start(double theta_d, double beta_d, unsigned long long peak_bound, int mean) {
+        beta = (int)beta_d;
+        // a threshold above every peak of the batch is as good as any other: the penalty is never paid
+        theta = theta_d > (double)peak_bound ? (int)(peak_bound + 1) : (int)theta_d;
+        code_base = __float_as_int(fmaxf((float)mean * (1.0f / 32.0f) * (float)beta, 1.0f)) >> 21;
+    }
+    __device__ __forceinline__ unsigned int key(unsigned int tokens, unsigned int t) const {
+        return tokens + (unsigned int)(beta * ((int)t - theta));
+    }
+    static __device__ __forceinline__ uint2 absent() { return make_uint2((unsigned int)no_a(), (unsigned int)no_b()); }
+    // codes of prompt lengths, and of the prompt length at which a row starts to pay: monotone, so different codes decide
+    // which is larger.  Four per octave.
+    __device__ __forceinline__ int code(float v) const { return min(max((__float_as_int(v) >> 21) - code_base + 1, 1), 31); }
+    __device__ __forceinline__ int prompt_code(int p) const { return code((float)(beta * p)); }
+    __device__ __forceinline__ int row_code(uint2 r) const {    // 0: pays for every prompt length
+        const int z = (int)(r.x - r.y);
+        return z < 0 ? 0 : code((float)z);
+    }
+    static __device__ __forceinline__ K row_a(uint2 r) { return (int)r.x; }
+    __device__ __forceinline__ K row_b(uint2 r) const { return (int)r.y; }
+    __device__ __forceinline__ K probe(int p) const { return (int)min((long long)beta * p, 0x3fffffffLL); }     // what a prompt of p tokens adds to a row's b
+    static __device__ __forceinline__ K plus(K b, K bp) { return b + bp; }
+    static __device__ __forceinline__ unsigned int order(K v) { return (unsigned int)v ^ 0x80000000u; }
+    static __device__ __forceinline__ K unorder(unsigned int v) { return (int)(v ^ 0x80000000u); }
+    static __device__ __forceinline__ int bits(K v) { return v; }
+    static __device__ __forceinline__ K from_bits(int v) { return v; }
+    static __device__ __forceinline__ K from_margin(int m) { return m; }
+    // one arrival
+    int bp, limit;
+    unsigned int pd;
+    __device__ __forceinline__ void arrival(int P, int D) { bp = beta * P; limit = theta - P; pd = (unsigned int)P + (unsigned int)D; }
+    __device__ __forceinline__ K arrival_bp() const { return bp; }
+    __device__ __forceinline__ S value(uint2 r) const { return (unsigned int)max((int)r.x, (int)r.y + bp); }
+    // the row after it has received the arrival: a lower bound, exact in its token count.  covers: the ramp reaches the key's step
+    __device__ __forceinline__ uint2 with_arrival(uint2 r, bool covers) const {
+        return make_uint2(r.x + pd, r.y + pd + (covers ? (unsigned int)bp : 0u));
+    }
+    __device__ __forceinline__ bool no_penalty(unsigned int top) const { return limit >= 0 && top <= (unsigned int)limit; }
+    // from a top (or c0), from a peak
+    __device__ __forceinline__ S of_top(unsigned int tokens, unsigned int top) const { return tokens + (unsigned int)(beta * max((int)top - limit, 0)); }
+    __device__ __forceinline__ S of_peak(unsigned int tokens, unsigned int peak) const { return tokens + (unsigned int)(beta * max((int)peak - theta, 0)); }
+    static __device__ __forceinline__ S warp_min(S s) { return __reduce_min_sync(0xffffffffu, s); }
+    __device__ __forceinline__ bool beats(S s, K bound) const { return (int)s < bound; }
+    __device__ __forceinline__ int job_score(S s) const { return (int)s; }
+};
+
+// Score of one instance, binary64, every operation rounded on its own (the sums of whole
+// numbers below 2^53 are exact, so adding the two token counts first changes nothing).
+__device__ __forceinline__ double summary_score(unsigned int tokens, unsigned int peak, double pd, double theta, double beta) {
+    double over = __dsub_rn((double)peak, theta);
+    if (over < 0.0) over = 0.0;
+    return __dadd_rn((double)tokens + pd, __dmul_rn(beta, over));
+}
+
+template <> struct Scores<false> {
+    typedef double S;
+    typedef float K;
+    static __device__ __forceinline__ S none() { return CUDART_INF; }
+    static __device__ __forceinline__ K no_a() { return CUDART_INF_F; }
+    static __device__ __forceinline__ K no_b() { return CUDART_INF_F; }
+    static __device__ __forceinline__ K lowest() { return -CUDART_INF_F; }
+    double theta, beta, slack;
+    int code_base;
+    __device__ __forceinline__ void start(double theta_d, double beta_d, unsigned long long, int mean) {
+        theta = theta_d; beta = beta_d;
+        // The bounds are real numbers taken with roundings in binary64 before they are rounded down: each of at most eight
+        // operations is off by 2^-53 of values below 2^33 * (1 + beta) + beta * theta; sixteen times that.
+        slack = (8589934592.0 * (1.0 + beta) + beta * theta) * (128.0 * 1.1102230246251565e-16);
+        code_base = __float_as_int(fmaxf((float)mean * (1.0f / 32.0f), 1.0f)) >> 21;
+    }
+    __device__ __forceinline__ unsigned int key(unsigned int, unsigned int t) const { return t; }
+    static __device__ __forceinline__ uint2 absent() { return make_uint2(0xffffffffu, 0u); }   // (masked by the row number)
+    __device__ __forceinline__ int code(float v) const { return min(max((__float_as_int(v) >> 21) - code_base + 1, 1), 31); }
+    __device__ __forceinline__ int prompt_code(int p) const { return code((float)p); }
+    __device__ __forceinline__ int row_code(uint2 r) const {
+        const double z = theta - (double)r.y;
+        return z < 0.0 ? 0 : code(__double2float_rn(z));
+    }
+    static __device__ __forceinline__ K row_a(uint2 r) { return __uint2float_rd(r.x); }
+    __device__ __forceinline__ K row_b(uint2 r) const { return __double2float_rd((double)r.x + beta * ((double)r.y - theta)); }
+    __device__ __forceinline__ K probe(int p) const { return __double2float_rd(beta * (double)p); }
+    static __device__ __forceinline__ K plus(K b, K bp) { return __fadd_rd(b, bp); }
+    static __device__ __forceinline__ unsigned int order(K v) {
+        const unsigned int x = __float_as_uint(v);
+        return x ^ ((unsigned int)((int)x >> 31) | 0x80000000u);
+    }
+    static __device__ __forceinline__ K unorder(unsigned int x) { return __uint_as_float(x ^ ((x >> 31) ? 0x80000000u : 0xffffffffu)); }
+    static __device__ __forceinline__ int bits(K v) { return __float_as_int(v); }
+    static __device__ __forceinline__ K from_bits(int v) { return __int_as_float(v); }
+    static __device__ __forceinline__ K from_margin(int m) { return (float)m; }
+    int P;
+    double pd;
+    float bp;
+    __device__ __forceinline__ void arrival(int p, int d) { P = p; pd = (double)p + (double)d; bp = probe(p); }
+    __device__ __forceinline__ K arrival_bp() const { return bp; }
+    __device__ __forceinline__ S value(uint2 r) const { return summary_score(r.x, r.y + (unsigned int)P, pd, theta, beta); }
+    __device__ __forceinline__ uint2 with_arrival(uint2 r, bool covers) const {
+        return make_uint2(r.x + (unsigned int)pd, r.y + (covers ? (unsigned int)P : 0u));
+    }
+    __device__ __forceinline__ bool no_penalty(unsigned int top) const { return !((double)(top + (unsigned int)P) > theta); }
+    __device__ __forceinline__ S of_top(unsigned int tokens, unsigned int top) const { return summary_score(tokens, top + (unsigned int)P, pd, theta, beta); }
+    __device__ __forceinline__ S of_peak(unsigned int tokens, unsigned int peak) const { return summary_score(tokens, peak, pd, theta, beta); }
+    static __device__ __forceinline__ S warp_min(S s) {   // scores are >= 0: ordered by their bits
+        const unsigned int hi = (unsigned int)__double2hiint(s), lo = (unsigned int)__double2loint(s);
+        const unsigned int mh = __reduce_min_sync(0xffffffffu, hi);
+        const unsigned int ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : 0xffffffffu);
+        return __hiloint2double((int)mh, (int)ml);
+    }
+    __device__ __forceinline__ bool beats(S s, K bound) const { return __double2float_ru(s - pd + slack) < bound; }
+    __device__ __forceinline__ int job_score(S) const { return 0; }
+};
+
+// ---- folding warps.  A warp adds a decided arrival to its row and takes the row's new numbers in the same pass, or takes
+// the peak the row would have with the arrival.  16-byte accesses when H is even (a lane holds two neighbouring cells, the
+// warp 512 contiguous bytes), eight in flight per lane.  Other warps of this block wrote the row before: the loads
+// come after the acquire of the job, and no other block touches the maps meanwhile.
+template <bool VEC, bool ADMIT, bool FOLD>
+__device__ __forceinline__ void rs_row_pass(const RouteSumArgs& a, int64_t* row, int P, int Dc, unsigned int& top, unsigned int& jtop,
+                                            unsigned int& c0, unsigned int& peak, int& above) {
+    constexpr int BATCH = 8;                        // loads in flight
+    constexpr int PER = VEC ? 2 : 1;                // cells per load
+    constexpr int STEP = 32 * PER;                  // cells per warp access
+    const int lane = threadIdx.x & 31, H = a.H;
+    const int hot_all = (ADMIT && a.hot < 0) ? 1 : 0;   // the overload level against 32-bit cells
+    const unsigned int hot = a.hot < 0 ? 0u : (a.hot > 0xffffffffLL ? 0xffffffffu : (unsigned int)a.hot);
+    top = jtop = c0 = peak = 0;
+    above = 0;
+    #pragma unroll 1
+    for (int base = 0; base < H; base += BATCH * STEP) {
+        unsigned int c[BATCH * PER];
+        #pragma unroll
+        for (int u = 0; u < BATCH; ++u) {
+            const int j = base + u * STEP + lane * PER;
+            if (VEC) {
+                longlong2 v = make_longlong2(0, 0);
+                if (j < H) v = *reinterpret_cast<const longlong2*>(row + j);
+                c[2 * u] = (unsigned int)v.x; c[2 * u + 1] = (unsigned int)v.y;
+            } else {
+                c[u] = j < H ? (unsigned int)row[j] : 0u;
+            }
+        }
+        #pragma unroll
+        for (int u = 0; u < BATCH; ++u) {
+            const int j = base + u * STEP + lane * PER;
+            if (j < Dc) {
+                #pragma unroll
+                for (int e = 0; e < PER; ++e)
+                    if (j + e < Dc) c[PER * u + e] += (unsigned int)(P + j + e);
+                if (FOLD) {   // (a pair whose second cell lies past the ramp writes that cell back unchanged)
+                    if (VEC) *reinterpret_cast<longlong2*>(row + j) = make_longlong2((long long)c[2 * u], (long long)c[2 * u + 1]);
+                    else row[j] = (long long)c[u];
+                }
+            }
+            if (j < H) {
+                if (FOLD) {
+                    unsigned int t = c[PER * u] + (unsigned int)j;
+                    if (VEC) t = max(t, c[2 * u + 1] + (unsigned int)(j + 1));
+                    if (ADMIT) {
+                        #pragma unroll
+                        for (int e = 0; e < PER; ++e) above += hot_all | (c[PER * u + e] > hot);
+                    }
+                    if (t > top) { top = t; jtop = (unsigned int)(j + PER - 1); }
+                } else {
+                    peak = max(peak, c[PER * u]);
+                    if (VEC) peak = max(peak, c[2 * u + 1]);
+                }
+            }
+        }
+        if (base == 0) c0 = c[0];
+    }
+}
+
+template <bool VEC, bool ADMIT, bool WHOLE>
+__device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int me, int near_steps) {
+    const int lane = threadIdx.x & 31, H = a.H;
+    unsigned int scans = 0;
+    unsigned int top, jtop, c0, peak;
+    int above;
+    for (unsigned int n = me;;) {
+        uint4 ctl;
+        if (!rs_wait(sh, [&] {
+                ctl = ld_volatile4(&sh.ctl);
+                return (int)(ctl.x - n) > 0 || ctl.y != scans || ctl.z != 0;
+            }))
+            return;
+        acquire_cta();
+        ctl = ld_volatile4(&sh.ctl);
+        if (__any_sync(0xffffffffu, (int)(ctl.x - n) > 0)) {
+            const int4 job = sh.jobs[n % RS_ITEMS];
+            const int w = job.x, P = job.y, Dc = job.z < H ? job.z : H;
+            rs_row_pass<VEC, ADMIT, true>(a, a.curves + (size_t)w * H, P, Dc, top, jtop, c0, peak, above);
+            const unsigned int t = __reduce_max_sync(0xffffffffu, top);
+            jtop = __reduce_min_sync(0xffffffffu, top == t ? jtop : 0xffffffffu);
+            if (ADMIT) above = __reduce_add_sync(0xffffffffu, above);
+            __syncwarp();   // every lane's cells before the row is handed on
+            if (lane == 0) {
+                const bool far = jtop >= (unsigned int)near_steps;
+                const bool not_over = ADMIT && !((double)above > a.many);
+                if (!far && jtop > ld_volatile(&sh.jmax)) atomicMax(&sh.jmax, jtop);
+                rows.top[w] = t;
+                rows.c0[w] = c0;
+                rows.rec[w].y = sc.key(rows.rec[w].x, far ? c0 : t);
+                if (not_over) atomicAdd(&sh.not_over, 1u);
+                st_release(&rows.flags[w], jtop | (far ? RS_FAR : 0u) | (not_over ? RS_NOT_OVER : 0u));
+                st_release(&sh.done[me], n + RS_FOLD_WARPS);
+            }
+            n += RS_FOLD_WARPS;
+            __syncwarp();
+        } else if (__any_sync(0xffffffffu, ctl.y != scans)) {
+            scans = ctl.y;
+            const int count = sh.scan_n;
+            for (int x = me; x < count; x += RS_FOLD_WARPS) {
+                rs_row_pass<VEC, ADMIT, false>(a, a.curves + (size_t)sh.scan_row[x] * H, sh.scan_P, sh.scan_Dc, top, jtop, c0, peak, above);
+                peak = __reduce_max_sync(0xffffffffu, peak);
+                if (lane == 0) sh.peak[x] = peak;
+            }
+            __syncwarp();
+            if (lane == 0) st_release(&sh.scans_done[me], scans);
+        } else {
+            return;
+        }
+    }
+}
+
+// ---- io warp: arrivals ahead of the decisions, results behind them
+template <bool ADMIT, bool WHOLE>
+__device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, long long q_head, int waiting, int items, int room) {
+    const int lane = threadIdx.x & 31;
+    const long long n0 = sh.n0;
+    auto put_result = [&](int k, int c, double s) {
+        if (ADMIT && k < waiting) a.queue_choice[k] = c;
+        else {
+            a.choice[k - waiting] = c;
+            if (a.score) a.score[k - waiting] = s;
+        }
+    };
+    int cursor = 0;                 // items of the batch looked at
+    unsigned int entered = 0;       // requests found among them
+    unsigned int written = 0;       // results written out
+    int first_bad = 0x7fffffff, first_full = 0x7fffffff;
+    for (;;) {
+        while (cursor < items && entered - written <= RS_ITEMS - 32) {
+            const int k = cursor + lane;
+            int P = -1, D = 0;
+            if (k < items) {
+                if (ADMIT && k < waiting) {
+                    const long long at = (q_head + k) % a.queue_capacity;
+                    P = a.queue_prompt[at]; D = a.queue_predicted[at];
+                } else {
+                    P = a.arr_prompt[k - waiting]; D = a.arr_predicted[k - waiting];
+                }
+            }
+            const bool ok = P >= 0 && D >= 1 && P <= PRE_FIELD_MAX && D <= PRE_FIELD_MAX;
+            const unsigned int vote = __ballot_sync(0xffffffffu, ok);
+            const unsigned int slot = entered + __popc(vote & ((1u << lane) - 1u));
+            if (ok && slot < (unsigned int)room) sh.items[slot % RS_ITEMS] = make_int4(P, D, 0, k);
+            else if (k < items) {
+                put_result(k, -1, 0.0);
+                if (!ok) first_bad = min(first_bad, k); else first_full = min(first_full, k);
+            }
+            entered = min(entered + __popc(vote), (unsigned int)room);
+            cursor += 32;
+            __syncwarp();
+            if (lane == 0) st_release(&sh.items_ready, entered);
+        }
+        if (cursor >= items && lane == 0) st_release(&sh.items_end, 1u);
+        const uint4 ctl = ld_volatile4(&sh.ctl);
+        const bool last = __any_sync(0xffffffffu, ctl.z != 0);
+        acquire_cta();
+        const unsigned int decided = __shfl_sync(0xffffffffu, ld_volatile(&sh.ctl.x), 0);   // (final when `last`)
+        while (decided - written >= 32 || (last && written != decided)) {
+            const unsigned int e = written + lane;
+            if (e < decided) {
+                const int4 job = sh.jobs[e % RS_ITEMS];
+                const int w = job.x;
+                const long long at = n0 + e;
+                a.prompt[at] = job.y; a.generated[at] = 0; a.predicted[at] = job.z; a.instance[at] = w;
+                const double s = WHOLE ? (double)((unsigned int)job.w + (unsigned int)job.y + (unsigned int)job.z) : sh.score[e % RS_ITEMS];
+                put_result(sh.items[e % RS_ITEMS].w, w, s);
+                atomicAdd(reinterpret_cast<unsigned long long*>(a.queued_p + w), (unsigned long long)job.y);
+                atomicAdd(reinterpret_cast<unsigned long long*>(a.current_d + w), (unsigned long long)job.z);
+            }
+            written = min(written + 32u, decided);
+            __syncwarp();
+        }
+        if (last || __any_sync(0xffffffffu, ctl.w != 0)) break;
+        __nanosleep(100);
+    }
+    first_bad = __reduce_min_sync(0xffffffffu, first_bad);
+    first_full = __reduce_min_sync(0xffffffffu, first_full);
+    if (lane == 0) { sh.first_bad = first_bad; sh.first_full = first_full; }
+}
+
+// ---- list warps.  A list holds the rows whose score for one of RS_PROBES prompt lengths lies within a margin of the
+// smallest score known for it; the margin follows the list's room.  The other rows are bounded by 32 buckets: bucket x
+// holds the smallest token count and the smallest b of the rows whose row_code is x.  For an arrival of code q the rows
+// of codes above q pay no penalty (score = a), those below q do (score = b + beta * P), and those of code q either
+// (score = the larger, hence at least the larger of the two smallest): four numbers per code.
+template <bool WHOLE>
+__device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int I, int mean) {
+    typedef typename Scores<WHOLE>::K K;
+    constexpr unsigned int FULL = 0xffffffffu;
+    const int t = threadIdx.x - RS_LIST_WARP * 32, lane = threadIdx.x & 31;
+    const bool leader = t < 32;
+    unsigned int met = 0;
+    auto team = [&]() -> bool {   // the three warps meet (false: abandoned)
+        met += RS_LIST_THREADS / 32;
+        __syncwarp();
+        acquire_cta();
+        if (lane == 0) atomicAdd(&sh.list_met, 1u);
+        return rs_wait(sh, [&] { return (int)(ld_acquire(&sh.list_met) - met) >= 0; });
+    };
+    auto score_at = [&](uint2 r, K bp) { return max(Scores<WHOLE>::row_a(r), Scores<WHOLE>::plus(sc.row_b(r), bp)); };
+    // probes: shares of the mean prompt (+ ramp) of the batch, from nothing to several times it
+    int probe_p = 0;
+    {
+        const float share[RS_PROBES] = {0.0f, 0.08f, 0.17f, 0.3f, 0.5f, 0.9f, 1.5f, 2.5f};
+        #pragma unroll
+        for (int x = 0; x < RS_PROBES; ++x)
+            if (lane == x) probe_p = (int)((float)mean * share[x]);
+    }
+    K bp[RS_PROBES];
+    #pragma unroll
+    for (int x = 0; x < RS_PROBES; ++x) bp[x] = sc.probe(__shfl_sync(FULL, probe_p, x));
+    int margin = max(mean / 16, 8);
+    for (unsigned int n = 1;; ++n) {
+        bool go = false;
+        if (!rs_wait(sh, [&] {
+                const uint4 ctl = ld_volatile4(&sh.ctl);
+                go = ld_acquire(&sh.lists_wanted) >= n;
+                return go || ctl.z != 0;
+            }, 20))
+            return;
+        go = __any_sync(FULL, ld_acquire(&sh.lists_wanted) >= n);
+        if (!go) return;     // (all three warps: nothing is asked for after the last decision)
+        const int old = (n + 1) & 1, now = n & 1;
+        // the smallest score known per probe: the rows of the present list, and (kept in probe_t) the others' bound
+        if (!team()) return;
+        K least[RS_PROBES];
+        #pragma unroll
+        for (int x = 0; x < RS_PROBES; ++x) least[x] = Scores<WHOLE>::from_bits(0x7f000000);
+        const int old_n = n == 1 ? 0 : sh.list_n[old];
+        const int known_n = n == 1 ? I : old_n;                      // (the first list: all rows)
+        for (int x = t; x < known_n; x += RS_LIST_THREADS) {
+            const uint2 r = ld_volatile2(rows.rec + (n == 1 ? x : sh.list_row[old][x]));
+            #pragma unroll
+            for (int p = 0; p < RS_PROBES; ++p) least[p] = min(least[p], score_at(r, bp[p]));
+        }
+        #pragma unroll
+        for (int p = 0; p < RS_PROBES; ++p) {
+            const unsigned int v = __reduce_min_sync(FULL, Scores<WHOLE>::order(least[p]));
+            if (lane == 0) atomicMin(reinterpret_cast<unsigned int*>(&sh.probe_t[p]), v);
+        }
+        for (int tries = 0;; ++tries) {
+            if (leader) { sh.bucket_a[lane] = 0xffffffffu; sh.bucket_b[lane] = 0xffffffffu; }
+            if (t == 0) sh.list_count = 0;
+            if (!team()) return;
+            K limit[RS_PROBES];
+            #pragma unroll
+            for (int p = 0; p < RS_PROBES; ++p)
+                limit[p] = tries < 8 ? Scores<WHOLE>::unorder((unsigned int)sh.probe_t[p]) + Scores<WHOLE>::from_margin(margin)
+                                     : Scores<WHOLE>::from_bits(0xbf800000);   // (below every score: an empty list is a list, too)
+            K hot_b = Scores<WHOLE>::from_bits(0x7f000000), cold_a = hot_b;
+            for (int base = 0; base < I; base += RS_LIST_THREADS) {
+                const int i = base + t;
+                const bool in = i < I;
+                const uint2 r = in ? ld_volatile2(rows.rec + i) : make_uint2(0u, 0u);
+                const K ra = Scores<WHOLE>::row_a(r), rb = sc.row_b(r);
+                bool take = false;
+                #pragma unroll
+                for (int p = 0; p < RS_PROBES; ++p) take |= max(ra, Scores<WHOLE>::plus(rb, bp[p])) <= limit[p];
+                take &= in;
+                const unsigned int vote = __ballot_sync(FULL, take);
+                if (vote) {
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(&sh.list_count, __popc(vote));
+                    at = __shfl_sync(FULL, at, 0) + __popc(vote & ((1u << lane) - 1u));
+                    if (take && at < RS_LIST_ROWS) sh.list_row[now][at] = i;
+                }
+                if (in && !take) {
+                    const int c = sc.row_code(r);
+                    if (c == 0) hot_b = min(hot_b, rb);
+                    else if (c == 31) cold_a = min(cold_a, ra);
+                    else {
+                        atomicMin(&sh.bucket_a[c], Scores<WHOLE>::order(ra));
+                        atomicMin(&sh.bucket_b[c], Scores<WHOLE>::order(rb));
+                    }
+                }
+            }
+            const unsigned int hb = __reduce_min_sync(FULL, Scores<WHOLE>::order(hot_b));
+            const unsigned int ca = __reduce_min_sync(FULL, Scores<WHOLE>::order(cold_a));
+            if (lane == 0) { atomicMin(&sh.bucket_b[0], hb); atomicMin(&sh.bucket_a[31], ca); }
+            if (!team()) return;
+            const int count = sh.list_count;
+            if (count > RS_LIST_ROWS) { margin = max(margin / 2, 1); if (tries > 4) margin = 0; if (!team()) return; continue; }
+            if (leader) {
+                // (a key that no row has set is out of reach; rows of code 31 count as paying nothing only for smaller codes,
+                // so their b joins in with the bound "at least the token count")
+                const unsigned int ua = sh.bucket_a[lane], ub = sh.bucket_b[lane];
+                const K ka = ua == 0xffffffffu ? Scores<WHOLE>::no_a() : min(Scores<WHOLE>::unorder(ua), Scores<WHOLE>::no_a());
+                const K kb = ub == 0xffffffffu ? Scores<WHOLE>::no_b() : min(Scores<WHOLE>::unorder(ub), Scores<WHOLE>::no_b());
+                K above_a = ka, below_b = kb;
+                #pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const K x = Scores<WHOLE>::from_bits(__shfl_down_sync(FULL, Scores<WHOLE>::bits(above_a), off));
+                    const K y = Scores<WHOLE>::from_bits(__shfl_up_sync(FULL, Scores<WHOLE>::bits(below_b), off));
+                    if (lane + off < 32) above_a = min(above_a, x);
+                    if (lane >= off) below_b = min(below_b, y);
+                }
+                above_a = Scores<WHOLE>::from_bits(__shfl_down_sync(FULL, Scores<WHOLE>::bits(above_a), 1));
+                below_b = Scores<WHOLE>::from_bits(__shfl_up_sync(FULL, Scores<WHOLE>::bits(below_b), 1));
+                if (lane == 31) above_a = Scores<WHOLE>::no_a();
+                if (lane == 0) below_b = Scores<WHOLE>::no_b();
+                // code 31: its own rows by their token count alone (no b is kept for them)
+                sh.table[now][lane] = make_int4(Scores<WHOLE>::bits(above_a), Scores<WHOLE>::bits(below_b), Scores<WHOLE>::bits(ka),
+                                                Scores<WHOLE>::bits(lane == 31 ? Scores<WHOLE>::lowest() : kb));
+                __syncwarp();
+                if (lane < RS_PROBES) {
+                    const int4 e = sh.table[now][sc.prompt_code(probe_p)];
+                    const K x = sc.probe(probe_p);
+                    const K b = min(min(Scores<WHOLE>::from_bits(e.x), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(e.y), x)),
+                                    max(Scores<WHOLE>::from_bits(e.z), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(e.w), x)));
+                    sh.probe_t[lane] = (int)Scores<WHOLE>::order(b);
+                }
+                if (lane == 0) sh.list_n[now] = count;
+                __syncwarp();
+                if (lane == 0) st_release(&sh.lists_ready, n);
+            }
+            if (count < RS_LIST_ROWS * 3 / 5) margin = min(margin + margin / 2 + 1, 1 << 24);
+            break;
+        }
+    }
+}
+
+// ---- deciding warp.  KS: rows per lane.  LISTS: they are a list's, else all rows.
+template <int KS, bool LISTS, bool ADMIT, bool WHOLE>
+__device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, Scores<WHOLE> sc) {
+    typedef typename Scores<WHOLE>::S S;
+    typedef typename Scores<WHOLE>::K K;
+    constexpr unsigned int FULL = 0xffffffffu;
+    constexpr unsigned int REFRESH = KS <= 2 ? 2 : 4;   // (all rows held: decisions between two looks at the pending ones)
+    const int lane = threadIdx.x & 31, I = a.I, H = a.H, n_groups = (I + 31) / 32;
+    unsigned int ready = 0;          // items known to be there
+    unsigned int taken_over = 0;     // ADMIT: decisions for rows that were known not to be overloaded
+    unsigned int scans = 0;
+    bool lost = false;
+
+    // ---- the rows held by the lane
+    int row[KS];
+    uint2 rec[KS];
+    unsigned int marked = 0;         // bit k: row k is pending, or far (its key is only a lower bound)
+    auto load_rows = [&]() {
+        marked = 0;
+        #pragma unroll
+        for (int k = 0; k < KS; ++k) {
+            rec[k] = Scores<WHOLE>::absent();
+            if (row[k] != RS_NO_ROW) {
+                const unsigned int f = ld_volatile(rows.flags + row[k]);   // first: it is written last
+                rec[k] = ld_volatile2(rows.rec + row[k]);
+                if (f & (RS_PENDING | RS_FAR)) marked |= 1u << k;
+            }
+        }
+    };
+    unsigned int list = 0;           // the list held
+    unsigned int since = 0, half = 0;   // decisions with it, and after how many the next one is asked for
+    bool asked = false;
+    auto ask_for_list = [&]() {
+        if (!asked && lane == 0) st_release(&sh.lists_wanted, list + 1);
+        asked = true;
+    };
+    auto next_list = [&]() {
+        ask_for_list();
+        if (!rs_wait(sh, [&] { return ld_acquire(&sh.lists_ready) > list; })) { lost = true; return; }
+        ++list;
+        asked = false;
+        const int n = sh.list_n[list & 1];
+        #pragma unroll
+        for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < n ? sh.list_row[list & 1][k * 32 + lane] : RS_NO_ROW;
+        load_rows();
+        since = 0;
+        half = max(n / 2, 4);
+    };
+    if (LISTS) {
+        next_list();
+    } else {
+        #pragma unroll
+        for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < I ? k * 32 + lane : RS_NO_ROW;
+        load_rows();
+    }
+    auto all_folded = [&](unsigned int e) {   // every decision before e has reached its row
+        return __all_sync(FULL, lane >= RS_FOLD_WARPS || (int)(ld_acquire(&sh.done[lane < RS_FOLD_WARPS ? lane : 0]) - e) >= 0);
+    };
+
+    int4 next = make_int4(0, 0, 0, 0);
+    bool have_next = false;
+    unsigned int e = 0;
+    for (; !lost; ++e) {
+        // ---- the next item: fetched while the one before it was decided, if it was there
+        int4 it = next;
+        if (!have_next) {
+            if (e >= ready) {
+                bool end = false;
+                if (!rs_wait(sh, [&] {
+                        end = __any_sync(FULL, ld_acquire(&sh.items_end) != 0);    // (before the count: the count is then final)
+                        ready = __shfl_sync(FULL, ld_acquire(&sh.items_ready), 0);
+                        return ready > e || end;
+                    }))
+                    break;
+                if (ready <= e) break;
+            }
+            it = sh.items[e % RS_ITEMS];
+        }
+        have_next = e + 1 < ready;
+        if (have_next) next = sh.items[(e + 1) % RS_ITEMS];
+        const int P = it.x, D = it.y, Dc = D < H ? D : H;
+        sc.arrival(P, D);
+        if ((e & 31u) == 0) {   // room in the ring of jobs for the next 32 decisions
+            if (!rs_wait(sh, [&] { return lane >= RS_FOLD_WARPS || (int)(e + 32 - ld_acquire(&sh.done[lane < RS_FOLD_WARPS ? lane : 0])) <= RS_ITEMS; }))
+                break;
+        }
+        if (ADMIT) {
+            // every instance overloaded?  While one is known not to be, the request is routed; else the folds under way decide.
+            if (__any_sync(FULL, ld_volatile(&sh.not_over) == taken_over)) {
+                if (!rs_wait(sh, [&] { const bool free_again = ld_volatile(&sh.not_over) != taken_over, all = all_folded(e); return free_again || all; })) break;
+                if (__all_sync(FULL, ld_acquire(&sh.not_over) == taken_over)) {   // the request is not routed: the batch stops here
+                    if (lane == 0) { sh.blocked = 1; sh.blocked_k = it.w; }
+                    break;
+                }
+            }
+        }
+        S best;
+        int win;
+        bool quick;
+        unsigned int jmax;
+        for (int lists_tried = 0;;) {
+            // ---- the best of the rows held, lowest row first
+            jmax = ld_volatile(&sh.jmax);    // (after the rows were read)
+            S v[KS];
+            #pragma unroll
+            for (int k = 0; k < KS; ++k) {
+                v[k] = sc.value(rec[k]);
+                if (!WHOLE && row[k] == RS_NO_ROW) v[k] = Scores<WHOLE>::none();
+            }
+            S m = v[0];
+            #pragma unroll
+            for (int k = 1; k < KS; ++k) m = v[k] < m ? v[k] : m;
+            best = Scores<WHOLE>::warp_min(m);
+            int r = RS_NO_ROW;
+            #pragma unroll
+            for (int k = 0; k < KS; ++k) r = v[k] == best ? min(r, row[k]) : r;
+            win = __reduce_min_sync(FULL, r);
+            bool mine = false;               // the lane's winner is marked
+            #pragma unroll
+            for (int k = 0; k < KS; ++k) mine |= row[k] == win && ((marked >> k) & 1u);
+            const bool stop = __any_sync(FULL, mine);
+            quick = (unsigned int)Dc > jmax;
+            if (!quick) break;
+            if (LISTS) {
+                const int4 b = sh.table[list & 1][sc.prompt_code(P)];
+                const K bp = sc.arrival_bp();
+                const K bound = min(min(Scores<WHOLE>::from_bits(b.x), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(b.y), bp)),
+                                    max(Scores<WHOLE>::from_bits(b.z), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(b.w), bp)));
+                if (win == RS_NO_ROW || !sc.beats(best, bound)) {   // a row outside the list could do as well
+                    if (lists_tried == 2) { quick = false; break; }
+                    ++lists_tried;
+                    next_list();
+                    if (lost) break;
+                    continue;
+                }
+            }
+            if (!stop) break;
+            // the winner is pending, or was when its lane last looked, or is far
+            if (!rs_wait(sh, [&] { return !(ld_acquire(rows.flags + win) & RS_PENDING); })) { lost = true; break; }
+            if (__any_sync(FULL, (ld_volatile(rows.flags + win) & RS_FAR) != 0)) {
+                // (far: its token count is its score where it pays no penalty)
+                if (!__all_sync(FULL, sc.no_penalty(ld_volatile(rows.top + win)))) quick = false;
+                break;
+            }
+            load_rows();
+        }
+        if (lost) break;
+        if (!quick) {
+            // ---- short arrivals and rows that have to be scanned: all rows.  First those with exact scores ...
+            auto look = [&](int i, S& s, unsigned int& tokens) {   // whether row i's score is exact, and the score (else a lower bound)
+                bool exact = false;
+                s = Scores<WHOLE>::none();
+                tokens = 0;
+                if (i < I) {
+                    const unsigned int f = ld_volatile(rows.flags + i);      // first: it is written last
+                    const uint2 q = ld_volatile2(rows.rec + i);
+                    const unsigned int top = ld_volatile(rows.top + i);
+                    const bool full = !(f & RS_PENDING) && Dc > (int)(f & RS_JTOP);
+                    tokens = q.x;
+                    s = sc.of_top(q.x, full ? top : ld_volatile(rows.c0 + i));   // (c0 of a pending row: at least the old one)
+                    exact = full || (!(f & RS_PENDING) && sc.no_penalty(top));
+                }
+                return exact;
+            };
+            best = Scores<WHOLE>::none();
+            win = RS_NO_ROW;
+            S mine = Scores<WHOLE>::none();
+            int mine_row = RS_NO_ROW;
+            for (int g = 0; g < n_groups; ++g) {
+                S s;
+                unsigned int tokens;
+                const int i = g * 32 + lane;
+                const bool ok = look(i, s, tokens);
+                if (ok && s < mine) { mine = s; mine_row = i; }   // a lane's rows ascend
+            }
+            auto take = [&]() {   // the warp's smallest of (mine, mine_row), against the best so far
+                const S smallest = Scores<WHOLE>::warp_min(mine);
+                const int r = __reduce_min_sync(FULL, mine == smallest ? mine_row : RS_NO_ROW);
+                if (smallest < best || (smallest == best && r < win)) { best = smallest; win = r; }
+            };
+            take();
+            // ... then those whose bound could beat the best: their folds are waited for, and they are scanned
+            for (int g = 0; g < n_groups; ++g) {
+                S s;
+                unsigned int tokens;
+                const int i = g * 32 + lane;
+                bool ok = look(i, s, tokens);
+                bool todo = i < I && (s < best || (s == best && i < win));   // (a fold may have ended since the first pass)
+                if (!__any_sync(FULL, todo)) continue;
+                if (!rs_wait(sh, [&] { return !todo || !(ld_acquire(rows.flags + i) & RS_PENDING); })) { lost = true; break; }
+                ok = look(i, s, tokens);
+                mine = todo && ok ? s : Scores<WHOLE>::none();
+                mine_row = todo && ok ? i : RS_NO_ROW;
+                take();
+                todo = todo && !ok && (s < best || (s == best && i < win));
+                const unsigned int which = __ballot_sync(FULL, todo);
+                if (!which) continue;
+                const int slot = __popc(which & ((1u << lane) - 1u));
+                if (todo) sh.scan_row[slot] = i;
+                if (lane == 0) { sh.scan_P = P; sh.scan_Dc = Dc; sh.scan_n = __popc(which); }
+                ++scans;
+                __syncwarp();
+                if (lane == 0) st_release(&sh.ctl.y, scans);
+                if (!rs_wait(sh, [&] { return lane >= RS_FOLD_WARPS || ld_acquire(&sh.scans_done[lane < RS_FOLD_WARPS ? lane : 0]) == scans; })) { lost = true; break; }
+                mine = todo ? sc.of_peak(tokens, sh.peak[slot]) : Scores<WHOLE>::none();
+                mine_row = todo ? i : RS_NO_ROW;
+                take();
+                __syncwarp();
+            }
+            if (lost) break;
+            if (win >= I) win = 0;   // (no score is finite: beta or theta beyond binary64's range)
+        }
+        // ---- the decision: row `win`.  It is pending from now on: exact token count, a lower bound of its key.
+        unsigned int before = 0;
+        if (ADMIT) before = ld_volatile(rows.flags + win);
+        const bool covers = (unsigned int)Dc > jmax;
+        bool writes = false;
+        uint2 mine = make_uint2(0u, 0u);
+        if (!quick) {            // (the row may not be one of those held)
+            mine = sc.with_arrival(ld_volatile2(rows.rec + win), covers);
+            writes = lane == 0;
+        }
+        #pragma unroll
+        for (int k = 0; k < KS; ++k) {
+            if (row[k] == win) {
+                if (quick) { mine = sc.with_arrival(rec[k], covers); writes = true; }
+                rec[k] = mine;
+                marked |= 1u << k;
+            }
+        }
+        if (!quick) __syncwarp();
+        if (writes) {
+            rows.rec[win] = mine;
+            rows.flags[win] = RS_PENDING;
+            sh.jobs[e % RS_ITEMS] = make_int4(win, P, D, sc.job_score(best));
+            if (!WHOLE) sh.score[e % RS_ITEMS] = (double)best;
+            st_release(&sh.ctl.x, e + 1u);
+        }
+        __syncwarp();
+        if (ADMIT) taken_over += (before & RS_NOT_OVER) ? 1u : 0u;
+        if (LISTS) {
+            if (++since == half) ask_for_list();
+        } else if ((e & (REFRESH - 1)) == REFRESH - 1) {
+            #pragma unroll
+            for (int k = 0; k < KS; ++k) {
+                if ((marked >> k) & 1u) {
+                    const unsigned int f = ld_volatile(rows.flags + row[k]);
+                    const uint2 q = ld_volatile2(rows.rec + row[k]);
+                    if (!(f & RS_PENDING)) {
+                        rec[k] = q;
+                        if (!(f & RS_FAR)) marked &= ~(1u << k);
+                    }
+                }
+            }
+        }
+    }
+    __syncwarp();
+    if (lane == 0) st_release(&sh.ctl.z, 1u);
+}
+
+template <int KS, bool LISTS, bool ADMIT, bool WHOLE>
+__global__ void __launch_bounds__(RS_THREADS, 1) pre_route_summaries(const RouteSumArgs a) {
     extern __shared__ __align__(16) unsigned char rs_smem[];
+    __shared__ __align__(16) RsShared sh;
     const int I = a.I, H = a.H;
-    const int Ip = (I + 31) & ~31;
-    uint2* tt = reinterpret_cast<uint2*>(rs_smem);          // [Ip] {token count (RS_OUT: left out of the pass), top}
-    uint2* aux = tt + Ip;                                   // [Ip] {rmax, c0}
-    uint32_t* jst = reinterpret_cast<uint32_t*>(aux + Ip);  // [Ip] jtop
-    int* over = reinterpret_cast<int*>(jst + Ip);           // [Ip] ADMIT: steps of the row above the overload level
-    __shared__ Item sh_item[2];             // the arrival to decide, by round parity
-    __shared__ int sh_decided[2];           // whether the round decided its arrival
-    __shared__ Pending pend[RS_PENDING];
-    __shared__ unsigned long long sh_wkey[2][RS_MAX_SCORE_WARPS];   // binary64 scores: the warps' best rows, score bits
-    __shared__ unsigned long long sh_best[2];   // whole-number scores: the smallest score << 32 | row of all warps (atomic minimum)
-    __shared__ int sh_wrow[2][RS_MAX_SCORE_WARPS];
-    __shared__ uint4 sh_fold[RS_FOLD_WARPS];   // per fold warp {rmax, top, jtop, -}
-    __shared__ unsigned int sh_jmax;        // no row's jtop is larger
-    __shared__ int sh_mode;                 // 0: decline the batch
-    __shared__ long long sh_n0;
-    __shared__ int sh_arr_p[64], sh_arr_d[64];   // the arrivals around the walker's position
-    __shared__ int sh_n_over;               // ADMIT: rows known to be overloaded
-    __shared__ int sh_blocked;              // ADMIT: a request found every instance overloaded ...
-    __shared__ long long sh_blocked_k;      // ... this one
-    __shared__ int sh_warp_ok[RS_MAX_THREADS / 32];   // (the tail of ADMIT)
-    __shared__ long long sh_joined;
-    __shared__ int sh_any_bad;
+    Rows rows;
+    rows.rec = reinterpret_cast<uint2*>(rs_smem);
+    rows.flags = reinterpret_cast<unsigned int*>(rows.rec + I);
+    rows.top = rows.flags + I;
+    rows.c0 = rows.top + I;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nsw = a.score_warps, nst = 32 * nsw, nthreads = RS_FOLD_THREADS + 32 + nst;
-    const double theta = a.theta, beta = a.beta;
+    const int near_steps = LISTS ? RS_NEAR_LISTS : RS_NEAR_DIRECT;
+    const unsigned long long mc = a.guard[GUARD_MAX_CELL], mb = a.guard[GUARD_MAX_BASE], ramps = a.guard[GUARD_SUM_RAMP];
+    // every cell, every cell + step with a prompt added, and every token count stay below 2^32 all batch long
+    const unsigned long long peak_bound = mc + ramps + (unsigned long long)H + (unsigned long long)PRE_FIELD_MAX;
     if (tid == 0) {
-        const unsigned long long mc = a.guard[GUARD_MAX_CELL], mb = a.guard[GUARD_MAX_BASE];
-        // every cell, every cell + step with a prompt added, and every token count stay below 2^32 all batch long
-        const unsigned long long peak_bound = mc + a.guard[GUARD_SUM_RAMP] + (unsigned long long)H + (unsigned long long)PRE_FIELD_MAX;
         const unsigned long long token_bound = mb + a.guard[GUARD_SUM_TOKENS];
-        // (and the batch is short enough for the round counters below to be 32-bit numbers)
-        const bool ok = a.guard[GUARD_BAD] == 0 && peak_bound <= 0xffffffffull && token_bound < (unsigned long long)RS_OUT &&
+        // (and the batch is short enough for 32-bit counters)
+        const bool ok = a.guard[GUARD_BAD] == 0 && peak_bound <= 0xffffffffull && token_bound <= 0xffffffffull &&
                         a.n_arrivals + (ADMIT ? a.queue_capacity : 0) < (1ll << 26);
-        // Whole-number scores: with beta and theta whole numbers every term of the score is a whole number
-        // below 2^53, each binary64 operation is exact, and the score is the same number in integer
-        // arithmetic; it is taken in 32 bits when even the largest possible score stays below 2^30.
-        bool exact = ok && beta == floor(beta) && theta == floor(theta) && beta <= 1048576.0 && theta < 1073741824.0;
-        if (exact) exact = token_bound + a.guard[GUARD_MAX_PD] + (unsigned long long)beta * peak_bound < (1ull << 30);
-        sh_mode = ok && (exact || !whole) ? 1 : 0;
-        sh_n0 = *a.n_requests;
-        sh_jmax = (unsigned int)a.guard[GUARD_MAX_JTOP];
-        for (int x = 0; x < RS_PENDING; ++x) pend[x].row = -1;
-        sh_best[0] = sh_best[1] = 0xffffffffffffffffull;
-        sh_n_over = 0;
-        sh_blocked = 0;
-        sh_blocked_k = 0;
-        sh_joined = 0;
-        sh_any_bad = 0;
+        // (whole-number scores: the host has seen to beta and theta)
+        const bool exact = !WHOLE || token_bound + a.guard[GUARD_MAX_PD] + (unsigned long long)a.beta * peak_bound < (1ull << 30);
+        sh.mode = ok && exact ? 1 : 0;
+        sh.n0 = *a.n_requests;
+        sh.ctl = make_uint4(0u, 0u, 0u, 0u);
+        sh.items_ready = sh.items_end = sh.not_over = sh.jmax = 0;
+        sh.lists_wanted = sh.lists_ready = sh.list_met = 0;
+        sh.list_n[0] = sh.list_n[1] = 0;
+        sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0;
     }
+    if (tid < RS_FOLD_WARPS) { sh.done[tid] = (unsigned int)tid; sh.scans_done[tid] = 0; }
+    if (tid < RS_PROBES) sh.probe_t[tid] = -1;
     __syncthreads();
-    if (sh_mode == 0) {
+    if (sh.mode == 0) {
         if (tid == 0) *a.handled = 0;
         return;
-    }
-    const unsigned int beta_i = whole ? (unsigned int)beta : 0u;
-    const int theta_i = whole ? (int)theta : 0;
-    for (int i = tid; i < Ip; i += nthreads) {
-        const RowSummary q = i < I ? a.summary0[i] : make_uint4(RS_OUT, 0, 0, 0);
-        tt[i] = make_uint2(q.x, q.z);
-        aux[i] = make_uint2(q.y, q.w);
-        jst[i] = i < I ? a.jtop0[i] : 0u;
-        if (ADMIT) {
-            over[i] = i < I ? a.over0[i] : 0;
-            if (i < I && (double)over[i] > a.many) atomicAdd(&sh_n_over, 1);
-        }
     }
     // ADMIT: the requests that were waiting when the call was made come first, then the arrivals
     long long q_head = 0, q_len = 0;
@@ -349,509 +1037,54 @@ __global__ void __launch_bounds__(RS_MAX_THREADS, 1) pre_route_summaries(const R
         if (q_len > a.queue_capacity) q_len = a.queue_capacity;
     }
     const long long n_items = q_len + a.n_arrivals;
-    // where the result of item k goes
-    auto put_result = [&](long long k, int c, double sc) {
-        if (ADMIT && k < q_len) a.queue_choice[k] = c;
-        else {
-            a.choice[k - q_len] = c;
-            if (a.score) a.score[k - q_len] = sc;
+    const unsigned long long mean_l = ramps / (unsigned long long)(n_items > 0 ? n_items : 1);
+    const int mean = mean_l < (1ull << 22) ? (int)mean_l : 1 << 22;     // prompt + ramp of a typical request
+    Scores<WHOLE> sc;
+    sc.start(a.theta, a.beta, peak_bound, mean);
+    {
+        unsigned int jmax = 0;
+        int free_rows = 0;
+        for (int i = tid; i < I; i += RS_THREADS) {
+            const uint4 q = a.summary0[i];
+            const bool far = q.z >= (unsigned int)near_steps;
+            if (!far) jmax = max(jmax, q.z);
+            const bool not_over = ADMIT && !((double)a.over0[i] > a.many);
+            free_rows += not_over;
+            rows.rec[i] = make_uint2(q.x, sc.key(q.x, far ? q.w : q.y));
+            rows.flags[i] = q.z | (far ? RS_FAR : 0u) | (not_over ? RS_NOT_OVER : 0u);
+            rows.top[i] = q.y;
+            rows.c0[i] = q.w;
         }
-    };
-    const long long n0 = sh_n0;
-    long long room = a.max_requests - n0;
-    if (room < 0) room = 0;
-    const float thetaf = (float)theta, betaf = (float)beta;
-    const float c0f = 2.0f * betaf * thetaf;
-
-    // ---- the walker turns the batch into the sequence of requests that are really routed;
-    // malformed arrivals and those beyond the table's room are answered on the spot.  The deciding
-    // warp runs it, all lanes alike; the arrivals come through a ring of two 32-entry chunks in shared
-    // memory, each chunk copied while the one before it is being used.
-    auto copy_chunk = [&](long long first) {
-        const long long k = first + lane;
-        if (k < a.n_arrivals) {
-            cp_async4(&sh_arr_p[k & 63], a.arr_prompt + k);
-            cp_async4(&sh_arr_d[k & 63], a.arr_predicted + k);
+        jmax = __reduce_max_sync(0xffffffffu, jmax);
+        if (lane == 0 && jmax) atomicMax(&sh.jmax, jmax);
+        if (ADMIT) {
+            free_rows = __reduce_add_sync(0xffffffffu, free_rows);
+            if (lane == 0 && free_rows) atomicAdd(&sh.not_over, (unsigned int)free_rows);
         }
-        cp_async_commit();
-    };
-    // (32-bit numbers: the batch has fewer than 2^26 items, or the kernel has declined it above)
-    const int items = (int)n_items, waiting = (int)q_len;
-    const int room_i = room > 0x7fffffffLL ? 0x7fffffff : (int)room;
-    int cursor = 0, entered = 0;   // (control warp, all lanes alike) items looked at, requests found
-    int first_bad = 0x7fffffff, first_full = 0x7fffffff;   // the first items dropped as malformed / for a full table
-    auto walk_next = [&]() {
-        Item it;
-        it.P = it.D = it.Dc = 0;
-        it.k = -1;
-        while (cursor < items) {
-            int P, D;
-            if (ADMIT && cursor < waiting) {
-                const long long at = (q_head + cursor) % a.queue_capacity;
-                P = a.queue_prompt[at];
-                D = a.queue_predicted[at];
-            } else {
-                const int ac = cursor - waiting;
-                if ((ac & 31) == 0) {   // a new chunk: its copy was started a chunk ago; start the next one
-                    asm volatile("cp.async.wait_group 0;" ::: "memory");
-                    __syncwarp();
-                    copy_chunk(ac + 32);
-                }
-                P = sh_arr_p[ac & 63];
-                D = sh_arr_d[ac & 63];
-            }
-            const bool bad = P < 0 || D < 1 || P > PRE_FIELD_MAX || D > PRE_FIELD_MAX;
-            if (bad || entered >= room_i) {
-                if (bad && cursor < first_bad) first_bad = cursor;
-                if (!bad && cursor < first_full) first_full = cursor;
-                if (lane == 0) put_result(cursor, -1, 0.0);
-                ++cursor;
-                continue;
-            }
-            it.P = P; it.D = D; it.Dc = D < H ? D : H; it.k = cursor;
-            ++cursor; ++entered;
-            break;
-        }
-        return it;
-    };
-    // (control warp) the last decision, not yet written out
-    int out_w = -1, out_k = 0, out_P = 0, out_D = 0;
-    long long out_slot = 0;
-    double out_score = 0.0;
-    // (the instance's two token counts are brought up to date after the last round, from the new table rows)
-    auto flush_outputs = [&]() {
-        if (out_w < 0) return;
-        if (lane == 0) { a.prompt[out_slot] = out_P; a.generated[out_slot] = 0; }
-        if (lane == 1) { a.predicted[out_slot] = out_D; a.instance[out_slot] = out_w; }
-        if (lane == 2) put_result(out_k, out_w, out_score);
-        out_w = -1;
-    };
-    Item nxt;               // (control warp) the arrival after the one being decided, walked to ahead of time
-    bool have_nxt = false;
-    nxt.P = nxt.D = nxt.Dc = 0; nxt.k = -1;
-    if (warp == RS_CONTROL_WARP) {
-        copy_chunk(0);
-        const Item first = walk_next();
-        if (lane == 0) sh_item[0] = first;
     }
+    const long long room = a.max_requests - sh.n0;
     __syncthreads();
 
-    const int sw_id = warp - RS_FOLD_WARPS - 1;   // score warps
-    // ADMIT: the overload level against 32-bit cells (a negative level: every cell is above it)
-    const int hot_all = (ADMIT && a.hot < 0) ? 1 : 0;
-    const unsigned int hot_u = a.hot < 0 ? 0u : (a.hot > 0xffffffffLL ? 0xffffffffu : (unsigned int)a.hot);
-    // fold warps: thread t holds cells 2t, 2t+1, then the same 2 * RS_FOLD_THREADS further on (16-byte accesses, a warp
-    // reads 512 contiguous bytes); without 16-byte accesses cells t, t + RS_FOLD_THREADS, ...
-    auto cell = [&](int u) { return VEC ? 2 * tid + (u >> 1) * (2 * RS_FOLD_THREADS) + (u & 1) : tid + u * RS_FOLD_THREADS; };
-    unsigned int c[CPT], cn[CPT];              // fold warps: the row being folded, the row fetched for the next fold
-    int fetched = -1;                          // the row in cn[]
-    // literal scan of one row by a warp: the peak with the arrival (P, Dc) added
-    auto scan_row = [&](int i, int P, int Dc) {
-        const int64_t* src = a.curves + (size_t)i * H;
-        unsigned int pk = 0;
-        if (VEC) {
-            for (int j = 2 * lane; j < H; j += 64) {
-                const longlong2 v = __ldcg(reinterpret_cast<const longlong2*>(src + j));
-                pk = max(pk, (unsigned int)v.x + (j < Dc ? (unsigned int)(P + j) : 0u));
-                pk = max(pk, (unsigned int)v.y + (j + 1 < Dc ? (unsigned int)(P + j + 1) : 0u));
-            }
-        } else {
-            for (int j = lane; j < H; j += 32)
-                pk = max(pk, (unsigned int)__ldcg(src + j) + (j < Dc ? (unsigned int)(P + j) : 0u));
-        }
-        return __reduce_max_sync(0xffffffffu, pk);
-    };
-    auto fetch = [&](int row, unsigned int* dst) {
-        const int64_t* src = a.curves + (size_t)row * H;
-        if (VEC) {
-            #pragma unroll
-            for (int u = 0; u < CPT; u += 2) {
-                longlong2 v = make_longlong2(0, 0);
-                if (cell(u) < H) v = __ldcg(reinterpret_cast<const longlong2*>(src + cell(u)));
-                dst[u] = (unsigned int)v.x; dst[u + 1] = (unsigned int)v.y;
-            }
-        } else {
-            #pragma unroll
-            for (int u = 0; u < CPT; ++u) dst[u] = cell(u) < H ? (unsigned int)__ldcg(src + cell(u)) : 0u;
-        }
-    };
-    auto whole_over = [&](unsigned int peak) { return (int)peak > theta_i ? peak - (unsigned int)theta_i : 0u; };
-
-    int ndec = 0, nfold = 0;   // decisions made, folds done: every thread keeps them
-    bool stalled = false;
-    bool blocked = false;            // ADMIT: a request found every instance overloaded: no more decisions, the folds go on
-    // Every arrival is decided after at most RS_PENDING stalled rounds and folded RS_LAG rounds later:
-    // the loop below ends by itself.  The limit only keeps a mistake in that reasoning from spinning.
-    const int round_limit = (int)((n_items + 2) * (RS_PENDING + 2) + 64);
-    bool overrun = false;
-    for (int round = 0;; ++round) {
-        if (round > round_limit) { overrun = true; break; }
-        const int par = round & 1;
-        const Item it = sh_item[par];
-        const bool have = it.k >= 0 && !blocked;
-        if (!have && nfold == ndec) break;
-        const bool do_fold = nfold < ndec && (ndec - nfold >= RS_LAG || !have || stalled);
-        unsigned int pend_lb_i = 0xffffffffu;   // (control warp) lower bound of pending entry nfold + lane for this arrival
-        double pend_lb_d = CUDART_INF;
-        int pend_row = -1;
-        bool pend_uncertain = false;   // ADMIT: that row was not overloaded when it was decided; its fold may change that
-        if (warp == RS_CONTROL_WARP) {
-            // =============================== control warp, while the pass runs ===============================
-            // what does not depend on the pass: the last decision's outputs, the pending rows' lower
-            // bounds, the arrival after this one
-            flush_outputs();
-            if (lane == 0) sh_best[par ^ 1] = 0xffffffffffffffffull;   // the next round's minimum starts afresh
-            if (have) {
-                const int d = nfold + lane;
-                if (lane < RS_PENDING && d < ndec) {
-                    const Pending p = pend[d % RS_PENDING];
-                    const unsigned int peak_lb = (unsigned int)it.Dc > p.jw ? (unsigned int)it.P + p.top_lb
-                                                                             : max(p.rmax, (unsigned int)it.P + p.c0);
-                    pend_row = p.row;
-                    pend_uncertain = ADMIT && p.unused[0] == 0u;
-                    if (whole) pend_lb_i = p.tokens + beta_i * whole_over(peak_lb);   // (without the arrival's own P + D, like the pass)
-                    else pend_lb_d = summary_score(p.tokens, peak_lb, it.P, it.D, theta, beta);
-                }
-                if (!have_nxt) { nxt = walk_next(); have_nxt = true; }
-            }
-        } else if (warp > RS_CONTROL_WARP) {
-            // =============================== score warps: every row's score for arrival `it` ===============================
-            if (have) {
-                const int P = it.P, D = it.D, Dc = it.Dc;
-                const unsigned int PD = (unsigned int)P + (unsigned int)D;
-                if (whole) {
-                    unsigned int best = 0xffffffffu;   // scores without the arrival's own P + D
-                    int brow = 0x7fffffff;
-                    const int K = P - theta_i;
-                    if ((unsigned int)Dc > sh_jmax) {
-                        // every row's summary gives its peak: two words per row
-                        // (a trip count known to the compiler, unrolled by eight: measured against a run-time trip
-                        // count and against 4 and 16)
-                        #pragma unroll 8
-                        for (int u = 0; u < RS_ROWS_PER_LANE; ++u) {
-                            const int i = sw_id * 32 + lane + u * nst;
-                            if (i < Ip) {
-                                const uint2 q = tt[i];
-                                const unsigned int t = q.x + beta_i * (unsigned int)max((int)q.y + K, 0);
-                                if (t < best) { best = t; brow = i; }
-                            }
-                        }
-                        if (BIG) {   // the lane's rows beyond those
-                            for (int i = sw_id * 32 + lane + RS_ROWS_PER_LANE * nst; i < Ip; i += nst) {
-                                const uint2 q = tt[i];
-                                const unsigned int t = q.x + beta_i * (unsigned int)max((int)q.y + K, 0);
-                                if (t < best) { best = t; brow = i; }
-                            }
-                        }
-                    } else {
-                        // Some rows are only bounded.  First the smallest upper bound among the warp's rows
-                        // (every row's score is at most the score with peak P + top): no row whose lower
-                        // bound exceeds it can hold the smallest score.  Then the rows: exact ones compete,
-                        // bounded ones that pass that test are scanned by the warp.
-                        unsigned int reach = 0xffffffffu;
-                        for (int i = sw_id * 32 + lane; i < Ip; i += nst) {
-                            const uint2 q = tt[i];
-                            reach = min(reach, q.x + beta_i * (unsigned int)max((int)q.y + K, 0));
-                        }
-                        reach = __reduce_min_sync(0xffffffffu, reach);
-                        for (int base = sw_id * 32; base < Ip; base += nst) {
-                            const int i = base + lane;
-                            const uint2 q = tt[i];
-                            bool undecided = false;
-                            if (q.x != RS_OUT) {
-                                if ((unsigned int)Dc > jst[i]) {
-                                    const unsigned int t = q.x + beta_i * (unsigned int)max((int)q.y + K, 0);
-                                    if (t < best) { best = t; brow = i; }
-                                } else {
-                                    const uint2 x = aux[i];
-                                    undecided = q.x + beta_i * whole_over(max(x.x, (unsigned int)P + x.y)) <= min(best, reach);
-                                }
-                            }
-                            unsigned int todo = __ballot_sync(0xffffffffu, undecided);
-                            while (todo) {
-                                const int src = __ffs(todo) - 1;
-                                todo &= todo - 1;
-                                const int row = base + src;
-                                const unsigned int t = tt[row].x + beta_i * whole_over(scan_row(row, P, Dc));
-                                if (lane == src && t < best) { best = t; brow = row; }   // a lane's rows ascend
-                            }
-                        }
-                    }
-                    // The smallest (score, row) of all score warps: the warp's smallest score by a warp reduction, then
-                    // the lanes that hold it (one, but for ties) take the block's minimum of score << 32 | row.
-                    const unsigned int wbest = __reduce_min_sync(0xffffffffu, best);
-                    if (best == wbest && wbest < RS_OUT) atomicMin(&sh_best[par], ((unsigned long long)best << 32) | (unsigned int)brow);
-                } else {
-                    // Binary64 scores, per warp.  First every row's score in binary32: a lower and an upper
-                    // estimate (the same number when the summary gives the peak exactly), kept in registers.
-                    // The warp's smallest upper estimate bounds which of its rows can hold its smallest score;
-                    // only those get the binary64 score (each operation rounded on its own), and a row that is
-                    // only bounded and passes the test is scanned.  The warps' exact best rows are compared by
-                    // the deciding warp, so the block's best row is found without a barrier among the warps.
-                    auto estimate = [&](unsigned int tokens, unsigned int peak) {
-                        return fmaf(betaf, fmaxf((float)peak - thetaf, 0.0f), (float)(tokens + PD));
-                    };
-                    float est[RS_ROWS_PER_LANE];
-                    float umin = 3.402823466e38f;
-                    const bool all_exact = (unsigned int)Dc > sh_jmax;   // every row's summary gives its peak: two words per row
-                    if (all_exact) {
-                        #pragma unroll
-                        for (int u = 0; u < RS_ROWS_PER_LANE; ++u) {
-                            const int i = sw_id * 32 + lane + u * nst;
-                            est[u] = CUDART_INF_F;
-                            if (i < Ip) {
-                                const uint2 q = tt[i];
-                                if (q.x != RS_OUT) est[u] = estimate(q.x, (unsigned int)P + q.y);
-                            }
-                            umin = fminf(umin, est[u]);
-                        }
-                    } else {
-                        #pragma unroll
-                        for (int u = 0; u < RS_ROWS_PER_LANE; ++u) {
-                            const int i = sw_id * 32 + lane + u * nst;
-                            est[u] = CUDART_INF_F;
-                            if (i < Ip) {
-                                const uint2 q = tt[i];
-                                if (q.x != RS_OUT) {
-                                    const unsigned int up = (unsigned int)P + q.y;
-                                    const uint2 x = aux[i];
-                                    const unsigned int lo = (unsigned int)Dc > jst[i] ? up : max(x.x, (unsigned int)P + x.y);
-                                    umin = fminf(umin, estimate(q.x, up));
-                                    est[u] = estimate(q.x, lo);
-                                }
-                            }
-                        }
-                    }
-                    // estimates are >= 0 and never NaN here (fminf drops a NaN): their bit patterns order like the values
-                    const float E = __uint_as_float(0xffffffffu - warp_max_u32(0xffffffffu - __float_as_uint(umin)));
-                    // lower_m * (1 - eps) <= E * (1 + eps) + 2 * eps * c0 for the row m of the warp's smallest score
-                    const float T = fmaf(E, 1.0f + RS_EPS, 2.0f * RS_EPS * c0f) * (1.0f + 3.0f * RS_EPS);
-                    double dbs = CUDART_INF;
-                    int dbi = 0x7fffffff;
-                    bool bounded = false;   // a row of this lane passes the test but its summary only bounds its peak
-                    #pragma unroll
-                    for (int u = 0; u < RS_ROWS_PER_LANE; ++u) {
-                        if (!(est[u] > T)) {   // (never for a row that is left out: its estimate is infinite ... unless T is)
-                            const int i = sw_id * 32 + lane + u * nst;
-                            const uint2 q = i < Ip ? tt[i] : make_uint2(RS_OUT, 0u);
-                            if (q.x != RS_OUT) {
-                                if (all_exact || (unsigned int)Dc > jst[i]) {
-                                    const double sc = summary_score(q.x, (unsigned int)P + q.y, P, D, theta, beta);
-                                    if (better_row(sc, i, dbs, dbi)) { dbs = sc; dbi = i; }
-                                } else {
-                                    bounded = true;
-                                }
-                            }
-                        }
-                    }
-                    if (__any_sync(0xffffffffu, bounded)) {   // rare: the rows again, the bounded ones that pass are scanned
-                        for (int base = sw_id * 32; base < Ip; base += nst) {
-                            const int i = base + lane;
-                            const uint2 q = tt[i];
-                            bool undecided = false;
-                            if (q.x != RS_OUT && !((unsigned int)Dc > jst[i])) {
-                                const uint2 x = aux[i];
-                                undecided = !(estimate(q.x, max(x.x, (unsigned int)P + x.y)) > T);
-                            }
-                            unsigned int todo = __ballot_sync(0xffffffffu, undecided);
-                            while (todo) {
-                                const int src = __ffs(todo) - 1;
-                                todo &= todo - 1;
-                                const int row = base + src;
-                                const double sc = summary_score(tt[row].x, scan_row(row, P, Dc), P, D, theta, beta);
-                                if (lane == src && better_row(sc, row, dbs, dbi)) { dbs = sc; dbi = row; }
-                            }
-                        }
-                    }
-                    // the warp's smallest (score, row): scores are >= 0, their bit patterns order like the values
-                    unsigned long long key = (unsigned long long)__double_as_longlong(dbs);
-                    int wrow = dbi;
-                    #pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) {
-                        const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, off);
-                        const int r2 = __shfl_xor_sync(0xffffffffu, wrow, off);
-                        if (k2 < key || (k2 == key && r2 < wrow)) { key = k2; wrow = r2; }
-                    }
-                    if (lane == 0) {
-                        sh_wkey[par][sw_id] = key;
-                        sh_wrow[par][sw_id] = wrow;
-                    }
-                }
-            }
-        } else if (do_fold) {
-            // =============================== fold warps: entry nfold goes into its row ===============================
-            const Pending p = pend[nfold % RS_PENDING];
-            const int w = p.row, P = p.P, Dc = p.Dc;
-            int64_t* grow = a.curves + (size_t)w * H;
-            if (fetched == w) {
-                #pragma unroll
-                for (int u = 0; u < CPT; ++u) c[u] = cn[u];
-            } else {
-                fetch(w, c);
-            }
-            // the row of the next entry, when it is known already, is fetched while this fold runs
-            fetched = -1;
-            if (CPT <= 8 && nfold + 1 < ndec) {   // (registers allowing)
-                fetched = pend[(nfold + 1) % RS_PENDING].row;
-                fetch(fetched, cn);
-            }
-            #pragma unroll
-            for (int u = 0; u < CPT; ++u)
-                if (cell(u) < Dc) c[u] += (unsigned int)(P + cell(u));
-            if (VEC) {
-                #pragma unroll
-                for (int u = 0; u < CPT; u += 2)   // (a pair whose second cell lies past the ramp writes that cell back unchanged)
-                    if (cell(u) < Dc) *reinterpret_cast<longlong2*>(grow + cell(u)) = make_longlong2((long long)c[u], (long long)c[u + 1]);
-            } else {
-                #pragma unroll
-                for (int u = 0; u < CPT; ++u)
-                    if (cell(u) < Dc) grow[cell(u)] = (long long)c[u];
-            }
-            unsigned int rmax = 0, top = 0, jtop = 0xffffffffu;
-            int above = 0;
-            #pragma unroll
-            for (int u = 0; u < CPT; ++u) {   // a thread's steps ascend with u
-                const int j = cell(u);
-                if (j < H) {
-                    if (ADMIT) above += hot_all | (c[u] > hot_u);
-                    rmax = max(rmax, c[u]);
-                    const unsigned int t = c[u] + (unsigned int)j;
-                    if (t > top) { top = t; jtop = (unsigned int)j; }   // (a lane whose cells + steps are all 0 names no step)
-                }
-            }
-            // the warp's largest cell, largest cell + step and the first step that has it (warp reductions: the fold
-            // warps are the longest chain of a round, and a butterfly of shuffles is three times as many instructions)
-            rmax = __reduce_max_sync(0xffffffffu, rmax);
-            const unsigned int wt = __reduce_max_sync(0xffffffffu, top);   // (a lane without cells has top 0 and no step)
-            const unsigned int wj = __reduce_min_sync(0xffffffffu, top == wt ? jtop : 0xffffffffu);
-            if (ADMIT) above = __reduce_add_sync(0xffffffffu, above);
-            if (lane == 0) sh_fold[warp] = make_uint4(rmax, wt, wj, (unsigned int)above);
-        }
-        __syncthreads();   // the pass and the fold's per-warp maxima are complete
-        if (warp == RS_CONTROL_WARP) {
-            if (have) {
-                // ---- the decision.  The pass's best row wins unless a pending row could do better.
-                const int P = it.P, D = it.D, Dc = it.Dc;
-                const unsigned int PD = (unsigned int)P + (unsigned int)D;
-                double b1s = CUDART_INF;   // binary64 path: the pass's best score
-                unsigned int b1i = 0xffffffffu;   // whole-number path: the same without the arrival's own P + D
-                int b1r = -1;
-                if (whole) {
-                    // the score warps took the minimum over all of them already
-                    const unsigned long long key = sh_best[par];
-                    if (key != 0xffffffffffffffffull) { b1i = (unsigned int)(key >> 32); b1r = (int)(unsigned int)key; }
-                } else {   // binary64 scores: (score bits, row) pairs, smallest first, by shuffles
-                    unsigned long long key = lane < nsw ? sh_wkey[par][lane] : 0xffffffffffffffffull;
-                    int row = lane < nsw ? sh_wrow[par][lane] : 0x7fffffff;
-                    for (int off = 1; off < nsw; off <<= 1) {
-                        const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, off);
-                        const int r2 = __shfl_xor_sync(0xffffffffu, row, off);
-                        if (k2 < key || (k2 == key && r2 < row)) { key = k2; row = r2; }
-                    }
-                    key = __shfl_sync(0xffffffffu, key, 0);   // lanes beyond the warps' count hold no result of their own
-                    row = __shfl_sync(0xffffffffu, row, 0);
-                    if (row != 0x7fffffff) {
-                        b1s = __longlong_as_double((long long)key);
-                        b1r = row;
-                    }
-                }
-                bool stall = b1r < 0;
-                if (pend_row >= 0) {
-                    const bool could_win = whole ? (pend_lb_i < b1i || (pend_lb_i == b1i && pend_row < b1r))
-                                                 : better_row(pend_lb_d, pend_row, b1s, b1r);
-                    if (pend_row == b1r || could_win) stall = true;
-                }
-                stall = __any_sync(0xffffffffu, stall);
-                if (ADMIT) {
-                    // every instance overloaded?  Rows are counted once their state is known; a pending row that was
-                    // not overloaded when it was decided may have become so.
-                    const int uncertain = __popc(__ballot_sync(0xffffffffu, pend_uncertain));
-                    const int n_over = sh_n_over;
-                    if (n_over >= I) {   // the request is not routed: the batch stops here
-                        stall = true;
-                        if (lane == 0) { sh_blocked = 1; sh_blocked_k = it.k; }
-                    } else if (n_over + uncertain >= I) {
-                        stall = true;
-                    }
-                }
-                if (!stall) {
-                    // the row is pending from now on: exact token count, bounds for the rest
-                    const int w = b1r;
-                    if (lane == 0) {
-                        const uint2 q = tt[w], x = aux[w];
-                        const unsigned int jw = jst[w];
-                        uint4* dst = reinterpret_cast<uint4*>(&pend[ndec % RS_PENDING]);
-                        dst[0] = make_uint4((unsigned int)w, (unsigned int)P, (unsigned int)D, (unsigned int)Dc);
-                        dst[1] = make_uint4(q.x + PD, q.y + ((int)jw < Dc ? (unsigned int)P + jw : 0u), jw, x.x);
-                        dst[2] = make_uint4(x.y + (unsigned int)P, (ADMIT && (double)over[w] > a.many) ? 1u : 0u, 0u, 0u);
-                        tt[w] = make_uint2(RS_OUT, 0u);
-                        *reinterpret_cast<uint4*>(&sh_item[par ^ 1]) = make_uint4((unsigned int)nxt.P, (unsigned int)nxt.D, (unsigned int)nxt.Dc, (unsigned int)nxt.k);
-                    }
-                    // what the outside sees of the decision is written while the next pass runs
-                    out_w = w; out_k = it.k; out_P = P; out_D = D; out_slot = n0 + ndec;
-                    out_score = whole ? (double)(b1i + PD) : b1s;
-                    have_nxt = false;
-                } else if (lane == 0) {
-                    sh_item[par ^ 1] = it;
-                }
-                if (lane == 0) {
-                    sh_decided[par] = stall ? 0 : 1;
-                }
-            } else if (lane == 0) {
-                sh_item[par ^ 1] = it;   // the batch has ended; the remaining folds go on
-            }
-        } else if (tid == 0 && do_fold) {
-            // ---- the folded row's new summary; the row takes part in the next pass again
-            const Pending p = pend[nfold % RS_PENDING];
-            unsigned int rmax = 0, top = 0, jtop = 0xffffffffu;
-            int above = 0;
-            #pragma unroll
-            for (int x = 0; x < RS_FOLD_WARPS; ++x) {   // the first step at which the largest cell + step is taken
-                const uint4 q = sh_fold[x];
-                above += (int)q.w;
-                rmax = max(rmax, q.x);
-                if (q.z != 0xffffffffu && (jtop == 0xffffffffu || q.y > top || (q.y == top && q.z < jtop))) { top = q.y; jtop = q.z; }
-            }
-            if (jtop == 0xffffffffu) jtop = 0u;
-            aux[p.row] = make_uint2(rmax, c[0]);
-            jst[p.row] = jtop;
-            if (jtop > sh_jmax) sh_jmax = jtop;
-            if (ADMIT) {
-                const bool was = (double)over[p.row] > a.many;
-                over[p.row] = above;
-                if (!was && (double)above > a.many) sh_n_over += 1;
-            }
-            tt[p.row] = make_uint2(p.tokens, top);
-        }
-        __syncthreads();
-        if (have) {
-            stalled = sh_decided[par] == 0;
-            if (!stalled) ++ndec;
-        } else {
-            stalled = false;
-        }
-        if (do_fold) ++nfold;
-        if (ADMIT && sh_blocked) blocked = true;
+    if (warp == 0) {
+        rs_decide_loop<KS, LISTS, ADMIT, WHOLE>(a, sh, rows, sc);
+    } else if (warp == RS_IO_WARP) {
+        rs_io_loop<ADMIT, WHOLE>(a, sh, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
+    } else if (warp >= RS_LIST_WARP) {
+        if (LISTS) rs_list_loop<WHOLE>(sh, rows, sc, I, mean);
+    } else if ((warp & 3) != 0) {
+        const int me = (warp >> 2) * 3 + (warp & 3) - 1;
+        if ((H & 1) == 0) rs_fold_loop<true, ADMIT, WHOLE>(a, sh, rows, sc, me, near_steps);
+        else rs_fold_loop<false, ADMIT, WHOLE>(a, sh, rows, sc, me, near_steps);
     }
-    if (warp == RS_CONTROL_WARP) flush_outputs();
-    if (overrun && tid == 0) atomicOr(a.status, PRE_ST_TIMEOUT);
-    // Every routed request adds its prompt to its instance's queued tokens and its predicted length to the tokens
-    // being decoded (Sec. 4.3.3): one reduction each per new table row, by the whole block, instead of two
-    // reductions in every round's chain.
     __syncthreads();
-    for (int i = tid; i < ndec; i += nthreads) {
-        const int w = a.instance[n0 + i];
-        atomicAdd(reinterpret_cast<unsigned long long*>(a.queued_p + w), (unsigned long long)a.prompt[n0 + i]);
-        atomicAdd(reinterpret_cast<unsigned long long*>(a.current_d + w), (unsigned long long)a.predicted[n0 + i]);
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    // what the walker noted beyond a blocked request is decided again below and does not count here
-    const long long decided = (ADMIT && blocked) ? sh_blocked_k : n_items;
-    if (tid == RS_FOLD_THREADS) {   // the control warp kept the walker's notes
-        *a.n_requests = n0 + ndec;
-        int flags = 0;
-        if (first_bad < decided) flags |= PRE_ST_BADREQ;
-        if (first_full < decided) flags |= PRE_ST_CAPACITY;
+    const bool blocked = ADMIT && sh.blocked;
+    const long long decided = blocked ? sh.blocked_k : n_items;
+    if (tid == 0) {
+        *a.n_requests = sh.n0 + sh.ctl.x;
+        // (what was noted beyond a blocked request is decided again below and does not count here)
+        int flags = sh.ctl.w ? PRE_ST_TIMEOUT : 0;
+        if (sh.first_bad < decided) flags |= PRE_ST_BADREQ;
+        if (sh.first_full < decided) flags |= PRE_ST_CAPACITY;
         if (flags) atomicOr(a.status, flags);
         *a.handled = 1;
     }
@@ -862,20 +1095,20 @@ __global__ void __launch_bounds__(RS_MAX_THREADS, 1) pre_route_summaries(const R
         __syncthreads();
         const long long stop = decided;
         const long long left = stop < q_len ? q_len - stop : 0;          // waiting entries that stay
-        for (long long k = stop + tid; k < q_len; k += nthreads) a.queue_choice[k] = -2;
+        for (long long k = stop + tid; k < q_len; k += RS_THREADS) a.queue_choice[k] = -2;
         const long long a0 = (stop > q_len ? stop : q_len) - q_len;      // first arrival that was not decided
-        const int nw = nthreads >> 5;
-        for (long long base = a0; base < a.n_arrivals; base += nthreads) {
+        const int nw = RS_WARPS;
+        for (long long base = a0; base < a.n_arrivals; base += RS_THREADS) {
             const long long i = base + tid;
             int P = -1, D = 0;
             if (i < a.n_arrivals) { P = a.arr_prompt[i]; D = a.arr_predicted[i]; }
             const bool ok = i < a.n_arrivals && !(P < 0 || D < 1 || P > PRE_FIELD_MAX || D > PRE_FIELD_MAX);
             const unsigned int vote = __ballot_sync(0xffffffffu, ok);
-            if (lane == 0) sh_warp_ok[warp] = __popc(vote);
+            if (lane == 0) sh.warp_ok[warp] = __popc(vote);
             __syncthreads();
-            long long rank = sh_joined + __popc(vote & ((1u << lane) - 1u));
+            long long rank = sh.joined + __popc(vote & ((1u << lane) - 1u));
             int total = 0;
-            for (int x = 0; x < nw; ++x) { if (x < warp) rank += sh_warp_ok[x]; total += sh_warp_ok[x]; }
+            for (int x = 0; x < nw; ++x) { if (x < warp) rank += sh.warp_ok[x]; total += sh.warp_ok[x]; }
             if (i < a.n_arrivals) {
                 int c = -1;
                 if (ok) {
@@ -888,21 +1121,21 @@ __global__ void __launch_bounds__(RS_MAX_THREADS, 1) pre_route_summaries(const R
                         c = -3;
                     }
                 } else {
-                    sh_any_bad = 1;
+                    sh.any_bad = 1;
                 }
                 a.choice[i] = c;
                 if (a.score) a.score[i] = 0.0;
             }
             __syncthreads();
-            if (tid == 0) sh_joined += total;
+            if (tid == 0) sh.joined += total;
             __syncthreads();
         }
         if (tid == 0) {
-            long long joined = sh_joined;
+            long long joined = sh.joined;
             if (left + joined > a.queue_capacity) joined = a.queue_capacity - left;
             a.queue_state[0] = a.queue_capacity > 0 ? (q_head + (q_len - left)) % a.queue_capacity : 0;
             a.queue_state[1] = left + joined;
-            if (blocked && sh_any_bad) atomicOr(a.status, PRE_ST_BADREQ);
+            if (blocked && sh.any_bad) atomicOr(a.status, PRE_ST_BADREQ);
         }
     }
 }
@@ -911,18 +1144,7 @@ __global__ void __launch_bounds__(RS_MAX_THREADS, 1) pre_route_summaries(const R
 
 // ---- host side
 
-static size_t summaries_smem_bytes(int I, bool admit) {
-    const size_t Ip = (size_t)((I + 31) & ~31);
-    return Ip * (2 * sizeof(uint2) + sizeof(uint32_t) + (admit ? sizeof(int) : 0));
-}
-
-// Score warps: sixteen rows per score thread up to RS_MAX_SCORE_WARPS warps, more rows per thread beyond (measured:
-// 4,096 instances are fastest with 8 score warps, 1,024 with 2 to 4; more warps lengthen the block barriers more
-// than they shorten the pass, and a block of more than 640 threads leaves 64 registers per thread: 70 % slower).
-static int summaries_score_warps(int I) {
-    int w = (I + RS_ROWS_PER_LANE * 32 - 1) / (RS_ROWS_PER_LANE * 32);
-    return w < 1 ? 1 : (w > RS_MAX_SCORE_WARPS ? RS_MAX_SCORE_WARPS : w);
-}
+static size_t summaries_smem_bytes(int I) { return (size_t)((I + 3) & ~3) * RS_ROW_BYTES; }
 
 // beta and theta = t_mem * M whole numbers of moderate size: the scores can be taken in whole-number arithmetic
 static bool summaries_whole_numbers(const pre_ctx* ctx) {
@@ -930,40 +1152,35 @@ static bool summaries_whole_numbers(const pre_ctx* ctx) {
     return beta == floor(beta) && theta == floor(theta) && beta <= 1048576.0 && theta < 1073741824.0;
 }
 
-template <int CPT, bool ADMIT, int KIND>
-static const void* summaries_kernel(bool vec) {
-    return vec ? (const void*)pre_route_summaries<CPT, true, ADMIT, KIND> : (const void*)pre_route_summaries<CPT, false, ADMIT, KIND>;
+// All rows in the deciding warp's registers while that is at most eight per lane, a list of 128 beyond (a list costs a
+// look at its bounds per arrival and a share of the next list: about what four more rows per lane cost).
+template <bool ADMIT, bool WHOLE>
+static const void* summaries_kernel(int I) {
+    if (I <= 32) return (const void*)pre_route_summaries<1, false, ADMIT, WHOLE>;
+    if (I <= 64) return (const void*)pre_route_summaries<2, false, ADMIT, WHOLE>;
+    if (I <= 128) return (const void*)pre_route_summaries<4, false, ADMIT, WHOLE>;
+    if (I <= RS_DIRECT_ROWS) return (const void*)pre_route_summaries<8, false, ADMIT, WHOLE>;
+    return (const void*)pre_route_summaries<4, true, ADMIT, WHOLE>;
 }
-template <bool ADMIT, int KIND>
-static const void* summaries_kernel_of_kind(int H) {
-    const bool vec = (H & 1) == 0;
-    if (H <= 4 * RS_FOLD_THREADS) return summaries_kernel<4, ADMIT, KIND>(vec);
-    if (H <= 8 * RS_FOLD_THREADS) return summaries_kernel<8, ADMIT, KIND>(vec);
-    if (H <= 16 * RS_FOLD_THREADS) return summaries_kernel<16, ADMIT, KIND>(vec);
-    return summaries_kernel<32, ADMIT, KIND>(vec);
-}
-// nullptr: no instantiation takes this context (binary64 scores with more than RS_ROWS_PER_LANE rows per score lane)
 template <bool ADMIT>
 static const void* summaries_kernel_for(const pre_ctx* ctx) {
-    const int H = ctx->cfg.horizon, I = ctx->cfg.n_instances;
-    const bool big = I > RS_ROWS_PER_LANE * 32 * RS_MAX_SCORE_WARPS;
-    if (summaries_whole_numbers(ctx))
-        return big ? summaries_kernel_of_kind<ADMIT, RS_WHOLE_BIG>(H) : summaries_kernel_of_kind<ADMIT, RS_WHOLE>(H);
-    return big ? nullptr : summaries_kernel_of_kind<ADMIT, RS_BINARY64>(H);
+    const int I = ctx->cfg.n_instances;
+    return summaries_whole_numbers(ctx) ? summaries_kernel<ADMIT, true>(I) : summaries_kernel<ADMIT, false>(I);
 }
 
 template <bool ADMIT>
 static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* smem_out) {
     const int I = ctx->cfg.n_instances;
     *smem_out = 0;
+    if (I > (summaries_whole_numbers(ctx) ? RS_MAX_ROWS : RS_MAX_BINARY64_ROWS)) return cudaSuccess;
     const void* fn = summaries_kernel_for<ADMIT>(ctx);
-    if (fn == nullptr) return cudaSuccess;
     cudaFuncAttributes attr;
     cudaError_t e = cudaFuncGetAttributes(&attr, fn);
     if (e != cudaSuccess) return e;
-    const size_t smem = summaries_smem_bytes(I, ADMIT);
+    const size_t smem = summaries_smem_bytes(I);
     if (smem + attr.sharedSizeBytes + 256 > limit) return cudaSuccess;   // too many instances
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the limit is shared by every context of the process: always the device maximum)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(limit - attr.sharedSizeBytes));
     if (e != cudaSuccess) return e;
     *smem_out = smem;
     return cudaSuccess;
@@ -972,7 +1189,6 @@ static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* s
 cudaError_t pre_route_summary_configure(pre_ctx* ctx) {
     ctx->route_summary_smem = 0;
     ctx->route_summary_smem_admit = 0;
-    if (ctx->cfg.horizon > 32 * RS_FOLD_THREADS) return cudaSuccess;
     cudaDeviceProp prop;
     cudaError_t e = cudaGetDeviceProperties(&prop, ctx->device);
     if (e != cudaSuccess) return e;
@@ -994,8 +1210,8 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
     p.curves = curves; p.queued_p = queued_p; p.current_d = current_d;
     p.arr_prompt = arr_prompt; p.arr_predicted = arr_predicted; p.n_arrivals = n_arrivals;
     p.I = I; p.H = H;
-    p.summary = reinterpret_cast<RowSummary*>(ctx->d_rs_summary);
-    p.jtop = ctx->d_rs_jtop; p.guard = ctx->d_rs_guard;
+    p.summary = reinterpret_cast<uint4*>(ctx->d_rs_summary);
+    p.guard = ctx->d_rs_guard;
     p.over = nullptr; p.hot = 0; p.queue_prompt = nullptr; p.queue_predicted = nullptr; p.queue_entry = nullptr;
     p.queue_capacity = 0;
     a.arr_prompt = arr_prompt; a.arr_predicted = arr_predicted; a.n_arrivals = n_arrivals;
@@ -1005,9 +1221,8 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
     a.choice = choice; a.score = score;
     a.I = I; a.H = H;
     a.theta = ctx->theta; a.beta = ctx->cfg.beta;
-    a.summary0 = p.summary; a.jtop0 = p.jtop; a.guard = p.guard;
+    a.summary0 = p.summary; a.guard = p.guard;
     a.status = ctx->d_status; a.handled = ctx->d_rs_handled;
-    a.score_warps = summaries_score_warps(I);
     a.queue_prompt = nullptr; a.queue_predicted = nullptr; a.queue_state = nullptr; a.queue_entry = nullptr;
     a.queue_capacity = 0; a.queue_choice = nullptr; a.hot = 0; a.many = 0.0; a.over0 = nullptr;
 }
@@ -1022,7 +1237,7 @@ static cudaError_t launch_summary_kernels(pre_ctx* ctx, const SumArgs& p, const 
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     void* params[] = {(void*)&a};
-    return cudaLaunchKernel(summaries_kernel_for<ADMIT>(ctx), dim3(1), dim3(RS_FOLD_THREADS + 32 + 32 * a.score_warps), params,
+    return cudaLaunchKernel(summaries_kernel_for<ADMIT>(ctx), dim3(1), dim3(RS_THREADS), params,
                             ADMIT ? ctx->route_summary_smem_admit : ctx->route_summary_smem, s);
 }
 
