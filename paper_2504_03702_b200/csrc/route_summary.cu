@@ -213,7 +213,8 @@ constexpr size_t RS_ROW_BYTES = sizeof(uint2) + 3 * sizeof(unsigned int);
 struct RsShared {
     // what the deciding warp tells the folding warps and the io warp, read with one access
     uint4 ctl;                              // {decisions made, scans asked for, 1: no more of either, 1: a wait was abandoned}
-    int4 items[RS_ITEMS];                   // {P, D, -, index in the batch} of the requests to route, in order
+    int4 items[RS_ITEMS];                   // {P, D, min(D, H) | code of P << 16, what P adds to a row's b} of the requests, in order
+    int item_at[RS_ITEMS];                  // and their indices in the batch
     int4 jobs[RS_ITEMS];                    // {row, P, D, whole-number score} of the decisions
     double score[RS_ITEMS];                 // their binary64 scores
     int4 table[2][32];                      // by code of the prompt: {bounds of the rows outside the list}
@@ -325,7 +326,7 @@ template <> struct Scores<true> {
     // one arrival
     int bp, limit;
     unsigned int pd;
-    __device__ __forceinline__ void arrival(int P, int D) { bp = beta * P; limit = theta - P; pd = (unsigned int)P + (unsigned int)D; }
+    __device__ __forceinline__ void arrival(int4 it) { bp = it.w; limit = theta - it.x; pd = (unsigned int)it.x + (unsigned int)it.y; }
     __device__ __forceinline__ K arrival_bp() const { return bp; }
     __device__ __forceinline__ S value(uint2 r) const { return (unsigned int)max((int)r.x, (int)r.y + bp); }
     // the row after it has received the arrival: a lower bound, exact in its token count.  covers: the ramp reaches the key's step
@@ -388,7 +389,7 @@ template <> struct Scores<false> {
     int P;
     double pd;
     float bp;
-    __device__ __forceinline__ void arrival(int p, int d) { P = p; pd = (double)p + (double)d; bp = probe(p); }
+    __device__ __forceinline__ void arrival(int4 it) { P = it.x; pd = (double)it.x + (double)it.y; bp = __int_as_float(it.w); }
     __device__ __forceinline__ K arrival_bp() const { return bp; }
     __device__ __forceinline__ S value(uint2 r) const { return summary_score(r.x, r.y + (unsigned int)P, pd, theta, beta); }
     __device__ __forceinline__ uint2 with_arrival(uint2 r, bool covers) const {
@@ -521,7 +522,7 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
 
 // ---- io warp: arrivals ahead of the decisions, results behind them
 template <bool ADMIT, bool WHOLE>
-__device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, long long q_head, int waiting, int items, int room) {
+__device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, const Scores<WHOLE>& sc, long long q_head, int waiting, int items, int room) {
     const int lane = threadIdx.x & 31;
     const long long n0 = sh.n0;
     auto put_result = [&](int k, int c, double s) {
@@ -550,8 +551,10 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
             const bool ok = P >= 0 && D >= 1 && P <= PRE_FIELD_MAX && D <= PRE_FIELD_MAX;
             const unsigned int vote = __ballot_sync(0xffffffffu, ok);
             const unsigned int slot = entered + __popc(vote & ((1u << lane) - 1u));
-            if (ok && slot < (unsigned int)room) sh.items[slot % RS_ITEMS] = make_int4(P, D, 0, k);
-            else if (k < items) {
+            if (ok && slot < (unsigned int)room) {
+                sh.items[slot % RS_ITEMS] = make_int4(P, D, (D < a.H ? D : a.H) | (sc.prompt_code(P) << 16), Scores<WHOLE>::bits(sc.probe(P)));
+                sh.item_at[slot % RS_ITEMS] = k;
+            } else if (k < items) {
                 put_result(k, -1, 0.0);
                 if (!ok) first_bad = min(first_bad, k); else first_full = min(first_full, k);
             }
@@ -573,7 +576,7 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
                 const long long at = n0 + e;
                 a.prompt[at] = job.y; a.generated[at] = 0; a.predicted[at] = job.z; a.instance[at] = w;
                 const double s = WHOLE ? (double)((unsigned int)job.w + (unsigned int)job.y + (unsigned int)job.z) : sh.score[e % RS_ITEMS];
-                put_result(sh.items[e % RS_ITEMS].w, w, s);
+                put_result(sh.item_at[e % RS_ITEMS], w, s);
                 atomicAdd(reinterpret_cast<unsigned long long*>(a.queued_p + w), (unsigned long long)job.y);
                 atomicAdd(reinterpret_cast<unsigned long long*>(a.current_d + w), (unsigned long long)job.z);
             }
@@ -730,31 +733,36 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
 }
 
 // ---- deciding warp.  KS: rows per lane.  LISTS: they are a list's, else all rows.
+// What bounds it: the latency of one chain of dependent instructions per arrival (two warp reductions, some ten integer
+// operations) and the fetching of its instructions, so the usual way through the loop is one straight piece of code with a
+// single branch to everything unusual.
 template <int KS, bool LISTS, bool ADMIT, bool WHOLE>
 __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, Scores<WHOLE> sc) {
     typedef typename Scores<WHOLE>::S S;
     typedef typename Scores<WHOLE>::K K;
     constexpr unsigned int FULL = 0xffffffffu;
-    constexpr unsigned int REFRESH = KS <= 2 ? 2 : 4;   // (all rows held: decisions between two looks at the pending ones)
-    const int lane = threadIdx.x & 31, I = a.I, H = a.H, n_groups = (I + 31) / 32;
-    unsigned int ready = 0;          // items known to be there
+    // decisions between two looks at items, room in the ring of jobs and (all rows held) pending rows
+    constexpr unsigned int CHUNK = LISTS ? 32 : 4 * KS;
+    const int lane = threadIdx.x & 31, I = a.I, n_groups = (I + 31) / 32;
+    const int lane_f = lane < RS_FOLD_WARPS ? lane : 0;
     unsigned int taken_over = 0;     // ADMIT: decisions for rows that were known not to be overloaded
     unsigned int scans = 0;
     bool lost = false;
 
-    // ---- the rows held by the lane
-    int row[KS];
+    // ---- the rows held by the lane: 2 * row + 1 if it is marked (pending when the lane last looked, or far: its key is
+    // only a lower bound), and what the row table has for it
+    unsigned int row[KS];
     uint2 rec[KS];
-    unsigned int marked = 0;         // bit k: row k is pending, or far (its key is only a lower bound)
+    constexpr unsigned int NO_ROW = 2u * (unsigned int)RS_NO_ROW;
     auto load_rows = [&]() {
-        marked = 0;
         #pragma unroll
         for (int k = 0; k < KS; ++k) {
             rec[k] = Scores<WHOLE>::absent();
-            if (row[k] != RS_NO_ROW) {
-                const unsigned int f = ld_volatile(rows.flags + row[k]);   // first: it is written last
-                rec[k] = ld_volatile2(rows.rec + row[k]);
-                if (f & (RS_PENDING | RS_FAR)) marked |= 1u << k;
+            if (row[k] != NO_ROW) {
+                const unsigned int i = row[k] >> 1;
+                const unsigned int f = ld_volatile(rows.flags + i);   // first: it is written last
+                rec[k] = ld_volatile2(rows.rec + i);
+                row[k] = 2 * i + ((f & (RS_PENDING | RS_FAR)) ? 1u : 0u);
             }
         }
     };
@@ -772,7 +780,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         asked = false;
         const int n = sh.list_n[list & 1];
         #pragma unroll
-        for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < n ? sh.list_row[list & 1][k * 32 + lane] : RS_NO_ROW;
+        for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < n ? 2u * (unsigned int)sh.list_row[list & 1][k * 32 + lane] : NO_ROW;
         load_rows();
         since = 0;
         half = max(n / 2, 4);
@@ -781,207 +789,200 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         next_list();
     } else {
         #pragma unroll
-        for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < I ? k * 32 + lane : RS_NO_ROW;
-        load_rows();
+        for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < I ? 2u * (unsigned int)(k * 32 + lane) : NO_ROW;
     }
-    auto all_folded = [&](unsigned int e) {   // every decision before e has reached its row
-        return __all_sync(FULL, lane >= RS_FOLD_WARPS || (int)(ld_acquire(&sh.done[lane < RS_FOLD_WARPS ? lane : 0]) - e) >= 0);
+    // the smallest score of the rows held, and the lowest row that has it (as in `row`)
+    auto best_held = [&](S& best) {
+        S v[KS];
+        #pragma unroll
+        for (int k = 0; k < KS; ++k) {
+            v[k] = sc.value(rec[k]);
+            if (!WHOLE && row[k] == NO_ROW) v[k] = Scores<WHOLE>::none();
+        }
+        S m = v[0];
+        #pragma unroll
+        for (int k = 1; k < KS; ++k) m = v[k] < m ? v[k] : m;
+        best = Scores<WHOLE>::warp_min(m);
+        unsigned int r = NO_ROW;
+        #pragma unroll
+        for (int k = 0; k < KS; ++k) r = v[k] == best ? min(r, row[k]) : r;
+        return __reduce_min_sync(FULL, r);
     };
-
-    int4 next = make_int4(0, 0, 0, 0);
-    bool have_next = false;
-    unsigned int e = 0;
-    for (; !lost; ++e) {
-        // ---- the next item: fetched while the one before it was decided, if it was there
-        int4 it = next;
-        if (!have_next) {
-            if (e >= ready) {
-                bool end = false;
-                if (!rs_wait(sh, [&] {
-                        end = __any_sync(FULL, ld_acquire(&sh.items_end) != 0);    // (before the count: the count is then final)
-                        ready = __shfl_sync(FULL, ld_acquire(&sh.items_ready), 0);
-                        return ready > e || end;
-                    }))
-                    break;
-                if (ready <= e) break;
+    auto bound_of_others = [&](int code) -> K {
+        const int4 b = sh.table[list & 1][code];
+        const K bp = sc.arrival_bp();
+        return min(min(Scores<WHOLE>::from_bits(b.x), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(b.y), bp)),
+                   max(Scores<WHOLE>::from_bits(b.z), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(b.w), bp)));
+    };
+    // ADMIT: every instance overloaded?  While one is known not to be, the request is routed; else the folds under way decide.
+    auto all_folded = [&](unsigned int e) {
+        return __all_sync(FULL, lane >= RS_FOLD_WARPS || (int)(ld_acquire(&sh.done[lane_f]) - e) >= 0);
+    };
+    // the decision `w` (as in `row`) for item e with score `best`: the row is pending from now on, with its exact token
+    // count and a lower bound of its key
+    auto commit = [&](unsigned int e, int4 it, unsigned int w, S best, bool covers, bool held) {
+        unsigned int before = 0;
+        if (ADMIT) before = ld_volatile(rows.flags + (w >> 1));
+        bool writes = false;
+        uint2 now = make_uint2(0u, 0u);
+        if (!held) {             // (the row may not be one of those held)
+            now = sc.with_arrival(ld_volatile2(rows.rec + (w >> 1)), covers);
+            writes = lane == 0;
+            __syncwarp();
+        }
+        #pragma unroll
+        for (int k = 0; k < KS; ++k) {
+            if (held ? row[k] == w : (row[k] >> 1) == (w >> 1)) {
+                if (held) { now = sc.with_arrival(rec[k], covers); writes = true; }
+                rec[k] = now;
+                row[k] |= 1u;
             }
-            it = sh.items[e % RS_ITEMS];
         }
-        have_next = e + 1 < ready;
-        if (have_next) next = sh.items[(e + 1) % RS_ITEMS];
-        const int P = it.x, D = it.y, Dc = D < H ? D : H;
-        sc.arrival(P, D);
-        if ((e & 31u) == 0) {   // room in the ring of jobs for the next 32 decisions
-            if (!rs_wait(sh, [&] { return lane >= RS_FOLD_WARPS || (int)(e + 32 - ld_acquire(&sh.done[lane < RS_FOLD_WARPS ? lane : 0])) <= RS_ITEMS; }))
-                break;
+        if (writes) {
+            rows.rec[w >> 1] = now;
+            rows.flags[w >> 1] = RS_PENDING;
+            sh.jobs[e % RS_ITEMS] = make_int4((int)(w >> 1), it.x, it.y, sc.job_score(best));
+            if (!WHOLE) sh.score[e % RS_ITEMS] = (double)best;
+            st_release(&sh.ctl.x, e + 1u);
         }
+        if (ADMIT) taken_over += (before & RS_NOT_OVER) ? 1u : 0u;
+    };
+    // Everything unusual about item e.  False: the batch ends here.
+    auto unusual = [&](unsigned int e, int4 it) -> bool {
+        const int P = it.x, Dc = it.z & 0xffff;
         if (ADMIT) {
-            // every instance overloaded?  While one is known not to be, the request is routed; else the folds under way decide.
             if (__any_sync(FULL, ld_volatile(&sh.not_over) == taken_over)) {
-                if (!rs_wait(sh, [&] { const bool free_again = ld_volatile(&sh.not_over) != taken_over, all = all_folded(e); return free_again || all; })) break;
+                if (!rs_wait(sh, [&] { const bool free_again = ld_volatile(&sh.not_over) != taken_over, all = all_folded(e); return free_again || all; })) { lost = true; return false; }
                 if (__all_sync(FULL, ld_acquire(&sh.not_over) == taken_over)) {   // the request is not routed: the batch stops here
-                    if (lane == 0) { sh.blocked = 1; sh.blocked_k = it.w; }
-                    break;
+                    if (lane == 0) { sh.blocked = 1; sh.blocked_k = sh.item_at[e % RS_ITEMS]; }
+                    return false;
                 }
             }
         }
         S best;
-        int win;
-        bool quick;
-        unsigned int jmax;
         for (int lists_tried = 0;;) {
-            // ---- the best of the rows held, lowest row first
-            jmax = ld_volatile(&sh.jmax);    // (after the rows were read)
-            S v[KS];
-            #pragma unroll
-            for (int k = 0; k < KS; ++k) {
-                v[k] = sc.value(rec[k]);
-                if (!WHOLE && row[k] == RS_NO_ROW) v[k] = Scores<WHOLE>::none();
+            const unsigned int jmax = ld_volatile(&sh.jmax);    // (after the rows were read)
+            if ((unsigned int)Dc <= jmax) break;
+            const unsigned int w = best_held(best);
+            if (LISTS && (w == NO_ROW || !sc.beats(best, bound_of_others(it.z >> 16)))) {   // a row outside the list could do as well
+                if (lists_tried == 2) break;
+                ++lists_tried;
+                next_list();
+                if (lost) return false;
+                continue;
             }
-            S m = v[0];
-            #pragma unroll
-            for (int k = 1; k < KS; ++k) m = v[k] < m ? v[k] : m;
-            best = Scores<WHOLE>::warp_min(m);
-            int r = RS_NO_ROW;
-            #pragma unroll
-            for (int k = 0; k < KS; ++k) r = v[k] == best ? min(r, row[k]) : r;
-            win = __reduce_min_sync(FULL, r);
-            bool mine = false;               // the lane's winner is marked
-            #pragma unroll
-            for (int k = 0; k < KS; ++k) mine |= row[k] == win && ((marked >> k) & 1u);
-            const bool stop = __any_sync(FULL, mine);
-            quick = (unsigned int)Dc > jmax;
-            if (!quick) break;
-            if (LISTS) {
-                const int4 b = sh.table[list & 1][sc.prompt_code(P)];
-                const K bp = sc.arrival_bp();
-                const K bound = min(min(Scores<WHOLE>::from_bits(b.x), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(b.y), bp)),
-                                    max(Scores<WHOLE>::from_bits(b.z), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(b.w), bp)));
-                if (win == RS_NO_ROW || !sc.beats(best, bound)) {   // a row outside the list could do as well
-                    if (lists_tried == 2) { quick = false; break; }
-                    ++lists_tried;
-                    next_list();
-                    if (lost) break;
-                    continue;
-                }
-            }
-            if (!stop) break;
-            // the winner is pending, or was when its lane last looked, or is far
-            if (!rs_wait(sh, [&] { return !(ld_acquire(rows.flags + win) & RS_PENDING); })) { lost = true; break; }
-            if (__any_sync(FULL, (ld_volatile(rows.flags + win) & RS_FAR) != 0)) {
+            if (w & 1u) {
+                if (!rs_wait(sh, [&] { return !(ld_acquire(rows.flags + (w >> 1)) & RS_PENDING); })) { lost = true; return false; }
+                if (!__any_sync(FULL, (ld_volatile(rows.flags + (w >> 1)) & RS_FAR) != 0)) { load_rows(); continue; }
                 // (far: its token count is its score where it pays no penalty)
-                if (!__all_sync(FULL, sc.no_penalty(ld_volatile(rows.top + win)))) quick = false;
-                break;
+                if (!__all_sync(FULL, sc.no_penalty(ld_volatile(rows.top + (w >> 1))))) break;
             }
-            load_rows();
+            commit(e, it, w, best, true, true);
+            return true;
         }
-        if (lost) break;
-        if (!quick) {
-            // ---- short arrivals and rows that have to be scanned: all rows.  First those with exact scores ...
-            auto look = [&](int i, S& s, unsigned int& tokens) {   // whether row i's score is exact, and the score (else a lower bound)
-                bool exact = false;
-                s = Scores<WHOLE>::none();
-                tokens = 0;
-                if (i < I) {
-                    const unsigned int f = ld_volatile(rows.flags + i);      // first: it is written last
-                    const uint2 q = ld_volatile2(rows.rec + i);
-                    const unsigned int top = ld_volatile(rows.top + i);
-                    const bool full = !(f & RS_PENDING) && Dc > (int)(f & RS_JTOP);
-                    tokens = q.x;
-                    s = sc.of_top(q.x, full ? top : ld_volatile(rows.c0 + i));   // (c0 of a pending row: at least the old one)
-                    exact = full || (!(f & RS_PENDING) && sc.no_penalty(top));
-                }
-                return exact;
-            };
-            best = Scores<WHOLE>::none();
-            win = RS_NO_ROW;
-            S mine = Scores<WHOLE>::none();
-            int mine_row = RS_NO_ROW;
-            for (int g = 0; g < n_groups; ++g) {
-                S s;
-                unsigned int tokens;
-                const int i = g * 32 + lane;
-                const bool ok = look(i, s, tokens);
-                if (ok && s < mine) { mine = s; mine_row = i; }   // a lane's rows ascend
+        // ---- short arrivals and rows that have to be scanned: all rows.  First those with exact scores ...
+        auto look = [&](int i, S& s, unsigned int& tokens) {   // whether row i's score is exact, and the score (else a lower bound)
+            bool exact = false;
+            s = Scores<WHOLE>::none();
+            tokens = 0;
+            if (i < I) {
+                const unsigned int f = ld_volatile(rows.flags + i);      // first: it is written last
+                const uint2 q = ld_volatile2(rows.rec + i);
+                const unsigned int top = ld_volatile(rows.top + i);
+                const bool full = !(f & RS_PENDING) && Dc > (int)(f & RS_JTOP);
+                tokens = q.x;
+                s = sc.of_top(q.x, full ? top : ld_volatile(rows.c0 + i));   // (c0 of a pending row: at least the old one)
+                exact = full || (!(f & RS_PENDING) && sc.no_penalty(top));
             }
-            auto take = [&]() {   // the warp's smallest of (mine, mine_row), against the best so far
-                const S smallest = Scores<WHOLE>::warp_min(mine);
-                const int r = __reduce_min_sync(FULL, mine == smallest ? mine_row : RS_NO_ROW);
-                if (smallest < best || (smallest == best && r < win)) { best = smallest; win = r; }
-            };
+            return exact;
+        };
+        best = Scores<WHOLE>::none();
+        int win = RS_NO_ROW;
+        S mine = Scores<WHOLE>::none();
+        int mine_row = RS_NO_ROW;
+        for (int g = 0; g < n_groups; ++g) {
+            S s;
+            unsigned int tokens;
+            const int i = g * 32 + lane;
+            const bool ok = look(i, s, tokens);
+            if (ok && s < mine) { mine = s; mine_row = i; }   // a lane's rows ascend
+        }
+        auto take = [&]() {   // the warp's smallest of (mine, mine_row), against the best so far
+            const S smallest = Scores<WHOLE>::warp_min(mine);
+            const int r = __reduce_min_sync(FULL, mine == smallest ? mine_row : RS_NO_ROW);
+            if (smallest < best || (smallest == best && r < win)) { best = smallest; win = r; }
+        };
+        take();
+        // ... then those whose bound could beat the best: their folds are waited for, and they are scanned
+        for (int g = 0; g < n_groups; ++g) {
+            S s;
+            unsigned int tokens;
+            const int i = g * 32 + lane;
+            bool ok = look(i, s, tokens);
+            bool todo = i < I && (s < best || (s == best && i < win));   // (a fold may have ended since the first pass)
+            if (!__any_sync(FULL, todo)) continue;
+            if (!rs_wait(sh, [&] { return !todo || !(ld_acquire(rows.flags + i) & RS_PENDING); })) { lost = true; return false; }
+            ok = look(i, s, tokens);
+            mine = todo && ok ? s : Scores<WHOLE>::none();
+            mine_row = todo && ok ? i : RS_NO_ROW;
             take();
-            // ... then those whose bound could beat the best: their folds are waited for, and they are scanned
-            for (int g = 0; g < n_groups; ++g) {
-                S s;
-                unsigned int tokens;
-                const int i = g * 32 + lane;
-                bool ok = look(i, s, tokens);
-                bool todo = i < I && (s < best || (s == best && i < win));   // (a fold may have ended since the first pass)
-                if (!__any_sync(FULL, todo)) continue;
-                if (!rs_wait(sh, [&] { return !todo || !(ld_acquire(rows.flags + i) & RS_PENDING); })) { lost = true; break; }
-                ok = look(i, s, tokens);
-                mine = todo && ok ? s : Scores<WHOLE>::none();
-                mine_row = todo && ok ? i : RS_NO_ROW;
-                take();
-                todo = todo && !ok && (s < best || (s == best && i < win));
-                const unsigned int which = __ballot_sync(FULL, todo);
-                if (!which) continue;
-                const int slot = __popc(which & ((1u << lane) - 1u));
-                if (todo) sh.scan_row[slot] = i;
-                if (lane == 0) { sh.scan_P = P; sh.scan_Dc = Dc; sh.scan_n = __popc(which); }
-                ++scans;
-                __syncwarp();
-                if (lane == 0) st_release(&sh.ctl.y, scans);
-                if (!rs_wait(sh, [&] { return lane >= RS_FOLD_WARPS || ld_acquire(&sh.scans_done[lane < RS_FOLD_WARPS ? lane : 0]) == scans; })) { lost = true; break; }
-                mine = todo ? sc.of_peak(tokens, sh.peak[slot]) : Scores<WHOLE>::none();
-                mine_row = todo ? i : RS_NO_ROW;
-                take();
-                __syncwarp();
-            }
-            if (lost) break;
-            if (win >= I) win = 0;   // (no score is finite: beta or theta beyond binary64's range)
+            todo = todo && !ok && (s < best || (s == best && i < win));
+            const unsigned int which = __ballot_sync(FULL, todo);
+            if (!which) continue;
+            const int slot = __popc(which & ((1u << lane) - 1u));
+            if (todo) sh.scan_row[slot] = i;
+            if (lane == 0) { sh.scan_P = P; sh.scan_Dc = Dc; sh.scan_n = __popc(which); }
+            ++scans;
+            __syncwarp();
+            if (lane == 0) st_release(&sh.ctl.y, scans);
+            if (!rs_wait(sh, [&] { return lane >= RS_FOLD_WARPS || ld_acquire(&sh.scans_done[lane_f]) == scans; })) { lost = true; return false; }
+            mine = todo ? sc.of_peak(tokens, sh.peak[slot]) : Scores<WHOLE>::none();
+            mine_row = todo ? i : RS_NO_ROW;
+            take();
+            __syncwarp();
         }
-        // ---- the decision: row `win`.  It is pending from now on: exact token count, a lower bound of its key.
-        unsigned int before = 0;
-        if (ADMIT) before = ld_volatile(rows.flags + win);
-        const bool covers = (unsigned int)Dc > jmax;
-        bool writes = false;
-        uint2 mine = make_uint2(0u, 0u);
-        if (!quick) {            // (the row may not be one of those held)
-            mine = sc.with_arrival(ld_volatile2(rows.rec + win), covers);
-            writes = lane == 0;
+        if (win >= I) win = 0;   // (no score is finite: beta or theta beyond binary64's range)
+        // (the ramp reaches every row's key if it is longer than the largest jtop known before the rows were read)
+        commit(e, it, 2u * (unsigned int)win, best, false, false);
+        return true;
+    };
+
+    unsigned int e = 0, ready = 0;   // decisions made, items known to be there
+    bool more = !lost;
+    while (more) {
+        if (e >= ready) {
+            bool end = false;
+            if (!rs_wait(sh, [&] {
+                    end = __any_sync(FULL, ld_acquire(&sh.items_end) != 0);    // (before the count: the count is then final)
+                    ready = __shfl_sync(FULL, ld_acquire(&sh.items_ready), 0);
+                    return ready > e || end;
+                }))
+                break;
+            if (ready <= e) break;
         }
-        #pragma unroll
-        for (int k = 0; k < KS; ++k) {
-            if (row[k] == win) {
-                if (quick) { mine = sc.with_arrival(rec[k], covers); writes = true; }
-                rec[k] = mine;
-                marked |= 1u << k;
-            }
-        }
-        if (!quick) __syncwarp();
-        if (writes) {
-            rows.rec[win] = mine;
-            rows.flags[win] = RS_PENDING;
-            sh.jobs[e % RS_ITEMS] = make_int4(win, P, D, sc.job_score(best));
-            if (!WHOLE) sh.score[e % RS_ITEMS] = (double)best;
-            st_release(&sh.ctl.x, e + 1u);
-        }
-        __syncwarp();
-        if (ADMIT) taken_over += (before & RS_NOT_OVER) ? 1u : 0u;
-        if (LISTS) {
-            if (++since == half) ask_for_list();
-        } else if ((e & (REFRESH - 1)) == REFRESH - 1) {
-            #pragma unroll
-            for (int k = 0; k < KS; ++k) {
-                if ((marked >> k) & 1u) {
-                    const unsigned int f = ld_volatile(rows.flags + row[k]);
-                    const uint2 q = ld_volatile2(rows.rec + row[k]);
-                    if (!(f & RS_PENDING)) {
-                        rec[k] = q;
-                        if (!(f & RS_FAR)) marked &= ~(1u << k);
-                    }
-                }
+        const unsigned int stop = min(ready, e + CHUNK);
+        if (!rs_wait(sh, [&] { return lane >= RS_FOLD_WARPS || (int)(stop - ld_acquire(&sh.done[lane_f])) <= RS_ITEMS; })) break;
+        if (!LISTS) load_rows();
+        else if (since >= half) ask_for_list();
+        since += stop - e;
+        int4 next = sh.items[e % RS_ITEMS];
+        for (; e < stop; ++e) {
+            const int4 it = next;
+            next = sh.items[(e + 1) % RS_ITEMS];      // (beyond the items that are there: not used)
+            const unsigned int jmax = ld_volatile(&sh.jmax);    // (after the rows were read)
+            unsigned int free_rows = 1;
+            if (ADMIT) free_rows = ld_volatile(&sh.not_over) - taken_over;
+            sc.arrival(it);
+            K bound = K(0);
+            if (LISTS) bound = bound_of_others(it.z >> 16);
+            S best;
+            const unsigned int w = best_held(best);
+            const bool usual = !(w & 1u) && (unsigned int)(it.z & 0xffff) > jmax && free_rows != 0 && (!LISTS || sc.beats(best, bound));
+            if (__builtin_expect(__all_sync(FULL, usual), 1)) {
+                commit(e, it, w, best, true, true);
+            } else if (!unusual(e, it)) {
+                more = false;
+                break;
             }
         }
     }
@@ -1068,7 +1069,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1) pre_route_summaries(const Route
     if (warp == 0) {
         rs_decide_loop<KS, LISTS, ADMIT, WHOLE>(a, sh, rows, sc);
     } else if (warp == RS_IO_WARP) {
-        rs_io_loop<ADMIT, WHOLE>(a, sh, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
+        rs_io_loop<ADMIT, WHOLE>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
     } else if (warp >= RS_LIST_WARP) {
         if (LISTS) rs_list_loop<WHOLE>(sh, rows, sc, I, mean);
     } else if ((warp & 3) != 0) {
