@@ -51,6 +51,7 @@ constexpr int RS_LIST_THREADS = 96;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
 constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
 constexpr int RS_LIST_ROWS = 128;           // rows of a list (4 per lane)
+constexpr int RS_NEAR_ROWS = 512;           // rows a list warp keeps for a closer look at once
 constexpr int RS_PROBES = 8;                // prompt lengths for which a list has the best rows
 // A row whose top lies further out is treated as only bounded (by c0): `jmax`, the largest jtop of the other rows, decides
 // which arrivals take the quick way (Dc > jmax).
@@ -222,6 +223,7 @@ struct RsShared {
     int list_n[2];
     unsigned int bucket_a[32], bucket_b[32];   // (list warps) smallest keys of the rows outside the list
     int probe_t[RS_PROBES];                 // (list warps) smallest scores at the probes
+    unsigned short near_row[RS_LIST_THREADS / 32][RS_NEAR_ROWS];
     int list_count;
     unsigned int list_met;                  // (list warps) arrivals at their meetings
     unsigned int lists_wanted, lists_ready;
@@ -267,6 +269,21 @@ __device__ __forceinline__ uint4 ld_volatile4(const uint4* p) {
     uint4 v;
     asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem_u32(p)) : "memory");
     return v;
+}
+// Stores under a predicate: in the deciding warp a branch around a store costs more than ten other instructions.
+__device__ __forceinline__ void st_if(bool p, unsigned int* at, unsigned int v) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.u32 [%1], %2; }" ::"r"((unsigned int)p), "r"(smem_u32(at)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_if(bool p, uint2* at, uint2 v) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.v2.u32 [%1], {%2, %3}; }" ::"r"((unsigned int)p), "r"(smem_u32(at)),
+                 "r"(v.x), "r"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_if(bool p, int4* at, int4 v) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.v4.u32 [%1], {%2, %3, %4, %5}; }" ::"r"((unsigned int)p), "r"(smem_u32(at)),
+                 "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ void st_if(bool p, double* at, double v) {
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.f64 [%1], %2; }" ::"r"((unsigned int)p), "r"(smem_u32(at)), "d"(v) : "memory");
 }
 __device__ __forceinline__ void acquire_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 
@@ -468,7 +485,7 @@ __device__ __forceinline__ void rs_row_pass(const RouteSumArgs& a, int64_t* row,
     }
 }
 
-template <bool VEC, bool ADMIT, bool WHOLE>
+template <bool VEC, bool ADMIT, bool WHOLE, bool LISTS>
 __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int me, int near_steps) {
     const int lane = threadIdx.x & 31, H = a.H;
     unsigned int scans = 0;
@@ -479,7 +496,7 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
         if (!rs_wait(sh, [&] {
                 ctl = ld_volatile4(&sh.ctl);
                 return (int)(ctl.x - n) > 0 || ctl.y != scans || ctl.z != 0;
-            }))
+            }, LISTS ? 40 : 0))    // (the list warps need the issue slots)
             return;
         acquire_cta();
         ctl = ld_volatile4(&sh.ctl);
@@ -596,32 +613,38 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
 // holds the smallest token count and the smallest b of the rows whose row_code is x.  For an arrival of code q the rows
 // of codes above q pay no penalty (score = a), those below q do (score = b + beta * P), and those of code q either
 // (score = the larger, hence at least the larger of the two smallest): four numbers per code.
+// The probes: shares of the mean prompt (+ ramp) of the batch, from nothing to several times it.
+__device__ __forceinline__ int rs_probe(int mean, int x) {
+    const float share[RS_PROBES] = {0.0f, 0.08f, 0.17f, 0.3f, 0.5f, 0.9f, 1.5f, 2.5f};
+    return (int)((float)mean * share[x]);
+}
 template <bool WHOLE>
-__device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int I, int mean) {
+__device__ __forceinline__ typename Scores<WHOLE>::K rs_score_at(const Scores<WHOLE>& sc, uint2 r, typename Scores<WHOLE>::K bp) {
+    return max(Scores<WHOLE>::row_a(r), Scores<WHOLE>::plus(sc.row_b(r), bp));
+}
+template <bool WHOLE>
+__device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int I, int mean, int longest_p) {
     typedef typename Scores<WHOLE>::K K;
     constexpr unsigned int FULL = 0xffffffffu;
     const int t = threadIdx.x - RS_LIST_WARP * 32, lane = threadIdx.x & 31;
     const bool leader = t < 32;
     unsigned int met = 0;
-    auto team = [&]() -> bool {   // the three warps meet (false: abandoned)
+    auto over = [&] { return __any_sync(FULL, ld_volatile(&sh.ctl.z) != 0); };
+    auto team = [&]() -> bool {   // the three warps meet (false: abandoned, or the last decision has been made)
         met += RS_LIST_THREADS / 32;
         __syncwarp();
         acquire_cta();
         if (lane == 0) atomicAdd(&sh.list_met, 1u);
-        return rs_wait(sh, [&] { return (int)(ld_acquire(&sh.list_met) - met) >= 0; });
+        return rs_wait(sh, [&] { return (int)(ld_acquire(&sh.list_met) - met) >= 0 || ld_volatile(&sh.ctl.z) != 0; }) && !over();
     };
-    auto score_at = [&](uint2 r, K bp) { return max(Scores<WHOLE>::row_a(r), Scores<WHOLE>::plus(sc.row_b(r), bp)); };
-    // probes: shares of the mean prompt (+ ramp) of the batch, from nothing to several times it
     int probe_p = 0;
-    {
-        const float share[RS_PROBES] = {0.0f, 0.08f, 0.17f, 0.3f, 0.5f, 0.9f, 1.5f, 2.5f};
-        #pragma unroll
-        for (int x = 0; x < RS_PROBES; ++x)
-            if (lane == x) probe_p = (int)((float)mean * share[x]);
-    }
     K bp[RS_PROBES];
     #pragma unroll
-    for (int x = 0; x < RS_PROBES; ++x) bp[x] = sc.probe(__shfl_sync(FULL, probe_p, x));
+    for (int x = 0; x < RS_PROBES; ++x) {
+        if (lane == x) probe_p = rs_probe(mean, x);
+        bp[x] = sc.probe(rs_probe(mean, x));
+    }
+    const K longest = sc.probe(longest_p);     // what the longest prompt of the batch adds
     int margin = max(mean / 16, 8);
     for (unsigned int n = 1;; ++n) {
         bool go = false;
@@ -636,57 +659,94 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
         const int old = (n + 1) & 1, now = n & 1;
         // the smallest score known per probe: the rows of the present list, and (kept in probe_t) the others' bound
         if (!team()) return;
-        K least[RS_PROBES];
-        #pragma unroll
-        for (int x = 0; x < RS_PROBES; ++x) least[x] = Scores<WHOLE>::from_bits(0x7f000000);
-        const int old_n = n == 1 ? 0 : sh.list_n[old];
-        const int known_n = n == 1 ? I : old_n;                      // (the first list: all rows)
-        for (int x = t; x < known_n; x += RS_LIST_THREADS) {
-            const uint2 r = ld_volatile2(rows.rec + (n == 1 ? x : sh.list_row[old][x]));
+        if (n > 1) {   // (the first list: probe_t was set when the rows were loaded)
+            K least[RS_PROBES];
             #pragma unroll
-            for (int p = 0; p < RS_PROBES; ++p) least[p] = min(least[p], score_at(r, bp[p]));
-        }
-        #pragma unroll
-        for (int p = 0; p < RS_PROBES; ++p) {
-            const unsigned int v = __reduce_min_sync(FULL, Scores<WHOLE>::order(least[p]));
-            if (lane == 0) atomicMin(reinterpret_cast<unsigned int*>(&sh.probe_t[p]), v);
+            for (int x = 0; x < RS_PROBES; ++x) least[x] = Scores<WHOLE>::from_bits(0x7f000000);
+            const int old_n = sh.list_n[old];
+            for (int x = t; x < old_n; x += RS_LIST_THREADS) {
+                const uint2 r = ld_volatile2(rows.rec + sh.list_row[old][x]);
+                #pragma unroll
+                for (int p = 0; p < RS_PROBES; ++p) least[p] = min(least[p], rs_score_at(sc, r, bp[p]));
+            }
+            #pragma unroll
+            for (int p = 0; p < RS_PROBES; ++p) {
+                const unsigned int v = __reduce_min_sync(FULL, Scores<WHOLE>::order(least[p]));
+                if (lane == 0) atomicMin(reinterpret_cast<unsigned int*>(&sh.probe_t[p]), v);
+            }
         }
         for (int tries = 0;; ++tries) {
             if (leader) { sh.bucket_a[lane] = 0xffffffffu; sh.bucket_b[lane] = 0xffffffffu; }
             if (t == 0) sh.list_count = 0;
             if (!team()) return;
-            K limit[RS_PROBES];
+            // A row is in the list if for some probe its token count is at most limit_a and its b at most limit_b.
+            // Rows beyond far_a or far_b are out of reach of this list: the two limits bound them, and they are dropped by
+            // two comparisons.
+            K limit_a[RS_PROBES], limit_b[RS_PROBES];
+            K far_a = Scores<WHOLE>::lowest();
             #pragma unroll
-            for (int p = 0; p < RS_PROBES; ++p)
-                limit[p] = tries < 8 ? Scores<WHOLE>::unorder((unsigned int)sh.probe_t[p]) + Scores<WHOLE>::from_margin(margin)
-                                     : Scores<WHOLE>::from_bits(0xbf800000);   // (below every score: an empty list is a list, too)
+            for (int p = 0; p < RS_PROBES; ++p) {
+                limit_a[p] = tries < 8 ? Scores<WHOLE>::unorder((unsigned int)sh.probe_t[p]) + Scores<WHOLE>::from_margin(margin)
+                                       : Scores<WHOLE>::lowest();   // (an empty list is a list, too)
+                limit_b[p] = limit_a[p] - bp[p];
+                far_a = max(far_a, limit_a[p]);
+            }
+            const K far_b = limit_a[0];
+            far_a = min(Scores<WHOLE>::plus(far_a, longest), Scores<WHOLE>::no_a());
             K hot_b = Scores<WHOLE>::from_bits(0x7f000000), cold_a = hot_b;
-            for (int base = 0; base < I; base += RS_LIST_THREADS) {
-                const int i = base + t;
-                const bool in = i < I;
-                const uint2 r = in ? ld_volatile2(rows.rec + i) : make_uint2(0u, 0u);
-                const K ra = Scores<WHOLE>::row_a(r), rb = sc.row_b(r);
-                bool take = false;
-                #pragma unroll
-                for (int p = 0; p < RS_PROBES; ++p) take |= max(ra, Scores<WHOLE>::plus(rb, bp[p])) <= limit[p];
-                take &= in;
-                const unsigned int vote = __ballot_sync(FULL, take);
-                if (vote) {
-                    int at = 0;
-                    if (lane == 0) at = atomicAdd(&sh.list_count, __popc(vote));
-                    at = __shfl_sync(FULL, at, 0) + __popc(vote & ((1u << lane) - 1u));
-                    if (take && at < RS_LIST_ROWS) sh.list_row[now][at] = i;
-                }
-                if (in && !take) {
-                    const int c = sc.row_code(r);
-                    if (c == 0) hot_b = min(hot_b, rb);
-                    else if (c == 31) cold_a = min(cold_a, ra);
-                    else {
-                        atomicMin(&sh.bucket_a[c], Scores<WHOLE>::order(ra));
-                        atomicMin(&sh.bucket_b[c], Scores<WHOLE>::order(rb));
+            constexpr int AT_ONCE = 4;      // rows a thread has on their way
+            unsigned short* near = sh.near_row[t >> 5];
+            int n_near = 0;
+            auto sort_near = [&]() {        // the rows that were not dropped: into the list or into a bucket
+                __syncwarp();
+                for (int x = lane; x - lane < n_near; x += 32) {
+                    const bool in = x < n_near;
+                    const int i = in ? near[x] : 0;
+                    const uint2 r = ld_volatile2(rows.rec + i);
+                    const K ra = Scores<WHOLE>::row_a(r), rb = sc.row_b(r);
+                    bool take = false;
+                    #pragma unroll
+                    for (int p = 0; p < RS_PROBES; ++p) take |= ra <= limit_a[p] && rb <= limit_b[p];
+                    take &= in;
+                    const unsigned int vote = __ballot_sync(FULL, take);
+                    if (vote) {
+                        int at = 0;
+                        if (lane == 0) at = atomicAdd(&sh.list_count, __popc(vote));
+                        at = __shfl_sync(FULL, at, 0) + __popc(vote & ((1u << lane) - 1u));
+                        if (take && at < RS_LIST_ROWS) sh.list_row[now][at] = i;
+                    }
+                    if (in && !take) {
+                        const int c = sc.row_code(r);
+                        if (c == 0) hot_b = min(hot_b, rb);
+                        else if (c == 31) cold_a = min(cold_a, ra);
+                        else {
+                            atomicMin(&sh.bucket_a[c], Scores<WHOLE>::order(ra));
+                            atomicMin(&sh.bucket_b[c], Scores<WHOLE>::order(rb));
+                        }
                     }
                 }
+                __syncwarp();
+                n_near = 0;
+            };
+            for (int base = 0; base < I; base += AT_ONCE * RS_LIST_THREADS) {
+                if (over()) return;
+                uint2 r[AT_ONCE];
+                #pragma unroll
+                for (int u = 0; u < AT_ONCE; ++u) {
+                    const int i = base + u * RS_LIST_THREADS + t;
+                    if (i < I) r[u] = ld_volatile2(rows.rec + i);
+                }
+                #pragma unroll
+                for (int u = 0; u < AT_ONCE; ++u) {
+                    const int i = base + u * RS_LIST_THREADS + t;
+                    const bool keep = i < I && !(sc.row_b(r[u]) > far_b) && !(Scores<WHOLE>::row_a(r[u]) > far_a);
+                    const unsigned int vote = __ballot_sync(FULL, keep);
+                    if (keep) near[n_near + __popc(vote & ((1u << lane) - 1u))] = (unsigned short)i;
+                    n_near += __popc(vote);
+                }
+                if (n_near > RS_NEAR_ROWS - AT_ONCE * 32) sort_near();
             }
+            sort_near();
             const unsigned int hb = __reduce_min_sync(FULL, Scores<WHOLE>::order(hot_b));
             const unsigned int ca = __reduce_min_sync(FULL, Scores<WHOLE>::order(cold_a));
             if (lane == 0) { atomicMin(&sh.bucket_b[0], hb); atomicMin(&sh.bucket_a[31], ca); }
@@ -699,7 +759,7 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
                 const unsigned int ua = sh.bucket_a[lane], ub = sh.bucket_b[lane];
                 const K ka = ua == 0xffffffffu ? Scores<WHOLE>::no_a() : min(Scores<WHOLE>::unorder(ua), Scores<WHOLE>::no_a());
                 const K kb = ub == 0xffffffffu ? Scores<WHOLE>::no_b() : min(Scores<WHOLE>::unorder(ub), Scores<WHOLE>::no_b());
-                K above_a = ka, below_b = kb;
+                K above_a = min(ka, far_a), below_b = min(kb, far_b);
                 #pragma unroll
                 for (int off = 1; off < 32; off <<= 1) {
                     const K x = Scores<WHOLE>::from_bits(__shfl_down_sync(FULL, Scores<WHOLE>::bits(above_a), off));
@@ -709,8 +769,8 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
                 }
                 above_a = Scores<WHOLE>::from_bits(__shfl_down_sync(FULL, Scores<WHOLE>::bits(above_a), 1));
                 below_b = Scores<WHOLE>::from_bits(__shfl_up_sync(FULL, Scores<WHOLE>::bits(below_b), 1));
-                if (lane == 31) above_a = Scores<WHOLE>::no_a();
-                if (lane == 0) below_b = Scores<WHOLE>::no_b();
+                if (lane == 31) above_a = far_a;
+                if (lane == 0) below_b = far_b;
                 // code 31: its own rows by their token count alone (no b is kept for them)
                 sh.table[now][lane] = make_int4(Scores<WHOLE>::bits(above_a), Scores<WHOLE>::bits(below_b), Scores<WHOLE>::bits(ka),
                                                 Scores<WHOLE>::bits(lane == 31 ? Scores<WHOLE>::lowest() : kb));
@@ -743,6 +803,8 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     constexpr unsigned int FULL = 0xffffffffu;
     // decisions between two looks at items, room in the ring of jobs and (all rows held) pending rows
     constexpr unsigned int CHUNK = LISTS ? 32 : 4 * KS;
+    // decisions made known to the folding warps at once (few rows: soon)
+    constexpr unsigned int PUBLISH = LISTS ? 4 : (KS >= 4 ? 2 : 1);
     const int lane = threadIdx.x & 31, I = a.I, n_groups = (I + 31) / 32;
     const int lane_f = lane < RS_FOLD_WARPS ? lane : 0;
     unsigned int taken_over = 0;     // ADMIT: decisions for rows that were known not to be overloaded
@@ -767,7 +829,6 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         }
     };
     unsigned int list = 0;           // the list held
-    unsigned int since = 0, half = 0;   // decisions with it, and after how many the next one is asked for
     bool asked = false;
     auto ask_for_list = [&]() {
         if (!asked && lane == 0) st_release(&sh.lists_wanted, list + 1);
@@ -782,8 +843,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         #pragma unroll
         for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < n ? 2u * (unsigned int)sh.list_row[list & 1][k * 32 + lane] : NO_ROW;
         load_rows();
-        since = 0;
-        half = max(n / 2, 4);
+        ask_for_list();     // (a list takes about as long as one lasts)
     };
     if (LISTS) {
         next_list();
@@ -791,8 +851,8 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         #pragma unroll
         for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < I ? 2u * (unsigned int)(k * 32 + lane) : NO_ROW;
     }
-    // the smallest score of the rows held, and the lowest row that has it (as in `row`)
-    auto best_held = [&](S& best) {
+    // the smallest score of the rows held, and the lane's lowest row that has it (as in `row`)
+    auto best_of_lane = [&](S& best) {
         S v[KS];
         #pragma unroll
         for (int k = 0; k < KS; ++k) {
@@ -806,7 +866,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         unsigned int r = NO_ROW;
         #pragma unroll
         for (int k = 0; k < KS; ++k) r = v[k] == best ? min(r, row[k]) : r;
-        return __reduce_min_sync(FULL, r);
+        return r;
     };
     auto bound_of_others = [&](int code) -> K {
         const int4 b = sh.table[list & 1][code];
@@ -820,36 +880,37 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     };
     // the decision `w` (as in `row`) for item e with score `best`: the row is pending from now on, with its exact token
     // count and a lower bound of its key
+    auto publish = [&](unsigned int n) {
+        __syncwarp();
+        if (lane == 0) st_release(&sh.ctl.x, n);
+    };
     auto commit = [&](unsigned int e, int4 it, unsigned int w, S best, bool covers, bool held) {
         unsigned int before = 0;
         if (ADMIT) before = ld_volatile(rows.flags + (w >> 1));
-        bool writes = false;
-        uint2 now = make_uint2(0u, 0u);
-        if (!held) {             // (the row may not be one of those held)
-            now = sc.with_arrival(ld_volatile2(rows.rec + (w >> 1)), covers);
-            writes = lane == 0;
-            __syncwarp();
-        }
-        #pragma unroll
-        for (int k = 0; k < KS; ++k) {
-            if (held ? row[k] == w : (row[k] >> 1) == (w >> 1)) {
-                if (held) { now = sc.with_arrival(rec[k], covers); writes = true; }
-                rec[k] = now;
-                row[k] |= 1u;
+        if (held) {
+            #pragma unroll
+            for (int k = 0; k < KS; ++k) {
+                const bool hit = row[k] == w;
+                if (hit) { rec[k] = sc.with_arrival(rec[k], covers); row[k] |= 1u; }
+                st_if(hit, rows.rec + (w >> 1), rec[k]);
             }
+        } else {                 // (the row may not be one of those held)
+            const uint2 now = sc.with_arrival(ld_volatile2(rows.rec + (w >> 1)), covers);
+            __syncwarp();
+            #pragma unroll
+            for (int k = 0; k < KS; ++k)
+                if ((row[k] >> 1) == (w >> 1)) { rec[k] = now; row[k] |= 1u; }
+            st_if(lane == 0, rows.rec + (w >> 1), now);
         }
-        if (writes) {
-            rows.rec[w >> 1] = now;
-            rows.flags[w >> 1] = RS_PENDING;
-            sh.jobs[e % RS_ITEMS] = make_int4((int)(w >> 1), it.x, it.y, sc.job_score(best));
-            if (!WHOLE) sh.score[e % RS_ITEMS] = (double)best;
-            st_release(&sh.ctl.x, e + 1u);
-        }
+        st_if(lane == 0, rows.flags + (w >> 1), RS_PENDING);
+        st_if(lane == 0, sh.jobs + e % RS_ITEMS, make_int4((int)(w >> 1), it.x, it.y, sc.job_score(best)));
+        if (!WHOLE) st_if(lane == 0, sh.score + e % RS_ITEMS, (double)best);
         if (ADMIT) taken_over += (before & RS_NOT_OVER) ? 1u : 0u;
     };
     // Everything unusual about item e.  False: the batch ends here.
     auto unusual = [&](unsigned int e, int4 it) -> bool {
         const int P = it.x, Dc = it.z & 0xffff;
+        publish(e);
         if (ADMIT) {
             if (__any_sync(FULL, ld_volatile(&sh.not_over) == taken_over)) {
                 if (!rs_wait(sh, [&] { const bool free_again = ld_volatile(&sh.not_over) != taken_over, all = all_folded(e); return free_again || all; })) { lost = true; return false; }
@@ -863,7 +924,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         for (int lists_tried = 0;;) {
             const unsigned int jmax = ld_volatile(&sh.jmax);    // (after the rows were read)
             if ((unsigned int)Dc <= jmax) break;
-            const unsigned int w = best_held(best);
+            const unsigned int w = __reduce_min_sync(FULL, best_of_lane(best));
             if (LISTS && (w == NO_ROW || !sc.beats(best, bound_of_others(it.z >> 16)))) {   // a row outside the list could do as well
                 if (lists_tried == 2) break;
                 ++lists_tried;
@@ -900,6 +961,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         int win = RS_NO_ROW;
         S mine = Scores<WHOLE>::none();
         int mine_row = RS_NO_ROW;
+        #pragma unroll 4
         for (int g = 0; g < n_groups; ++g) {
             S s;
             unsigned int tokens;
@@ -963,28 +1025,28 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         const unsigned int stop = min(ready, e + CHUNK);
         if (!rs_wait(sh, [&] { return lane >= RS_FOLD_WARPS || (int)(stop - ld_acquire(&sh.done[lane_f])) <= RS_ITEMS; })) break;
         if (!LISTS) load_rows();
-        else if (since >= half) ask_for_list();
-        since += stop - e;
         int4 next = sh.items[e % RS_ITEMS];
         for (; e < stop; ++e) {
             const int4 it = next;
             next = sh.items[(e + 1) % RS_ITEMS];      // (beyond the items that are there: not used)
             const unsigned int jmax = ld_volatile(&sh.jmax);    // (after the rows were read)
-            unsigned int free_rows = 1;
-            if (ADMIT) free_rows = ld_volatile(&sh.not_over) - taken_over;
+            bool odd = (unsigned int)(it.z & 0xffff) <= jmax;
+            if (ADMIT) odd |= ld_volatile(&sh.not_over) == taken_over;
             sc.arrival(it);
             K bound = K(0);
             if (LISTS) bound = bound_of_others(it.z >> 16);
             S best;
-            const unsigned int w = best_held(best);
-            const bool usual = !(w & 1u) && (unsigned int)(it.z & 0xffff) > jmax && free_rows != 0 && (!LISTS || sc.beats(best, bound));
-            if (__builtin_expect(__all_sync(FULL, usual), 1)) {
-                commit(e, it, w, best, true, true);
-            } else if (!unusual(e, it)) {
-                more = false;
-                break;
+            const unsigned int r = best_of_lane(best);
+            if (LISTS) odd |= !sc.beats(best, bound);
+            const unsigned int w = __reduce_min_sync(FULL, odd ? 1u : r);     // (odd: like a marked row)
+            if (__builtin_expect(w & 1u, 0)) {
+                if (!unusual(e, it)) { more = false; break; }
+                continue;
             }
+            commit(e, it, w, best, true, true);
+            if (PUBLISH == 1 || (e & (PUBLISH - 1)) == PUBLISH - 1) publish(e + 1);
         }
+        publish(e);
     }
     __syncwarp();
     if (lane == 0) st_release(&sh.ctl.z, 1u);
@@ -994,6 +1056,7 @@ template <int KS, bool LISTS, bool ADMIT, bool WHOLE>
 __global__ void __launch_bounds__(RS_THREADS, 1) pre_route_summaries(const RouteSumArgs a) {
     extern __shared__ __align__(16) unsigned char rs_smem[];
     __shared__ __align__(16) RsShared sh;
+    typedef typename Scores<WHOLE>::K K;
     const int I = a.I, H = a.H;
     Rows rows;
     rows.rec = reinterpret_cast<uint2*>(rs_smem);
@@ -1045,19 +1108,33 @@ __global__ void __launch_bounds__(RS_THREADS, 1) pre_route_summaries(const Route
     {
         unsigned int jmax = 0;
         int free_rows = 0;
+        K least[LISTS ? RS_PROBES : 1];      // the smallest score per probe, for the first list
+        if (LISTS)
+            #pragma unroll
+            for (int p = 0; p < RS_PROBES; ++p) least[LISTS ? p : 0] = Scores<WHOLE>::from_bits(0x7f000000);
         for (int i = tid; i < I; i += RS_THREADS) {
             const uint4 q = a.summary0[i];
             const bool far = q.z >= (unsigned int)near_steps;
             if (!far) jmax = max(jmax, q.z);
             const bool not_over = ADMIT && !((double)a.over0[i] > a.many);
             free_rows += not_over;
-            rows.rec[i] = make_uint2(q.x, sc.key(q.x, far ? q.w : q.y));
+            const uint2 rec = make_uint2(q.x, sc.key(q.x, far ? q.w : q.y));
+            rows.rec[i] = rec;
+            if (LISTS)
+                #pragma unroll
+                for (int p = 0; p < RS_PROBES; ++p) least[LISTS ? p : 0] = min(least[LISTS ? p : 0], rs_score_at(sc, rec, sc.probe(rs_probe(mean, p))));
             rows.flags[i] = q.z | (far ? RS_FAR : 0u) | (not_over ? RS_NOT_OVER : 0u);
             rows.top[i] = q.y;
             rows.c0[i] = q.w;
         }
         jmax = __reduce_max_sync(0xffffffffu, jmax);
         if (lane == 0 && jmax) atomicMax(&sh.jmax, jmax);
+        if (LISTS)
+            #pragma unroll
+            for (int p = 0; p < RS_PROBES; ++p) {
+                const unsigned int v = __reduce_min_sync(0xffffffffu, Scores<WHOLE>::order(least[LISTS ? p : 0]));
+                if (lane == 0) atomicMin(reinterpret_cast<unsigned int*>(&sh.probe_t[p]), v);
+            }
         if (ADMIT) {
             free_rows = __reduce_add_sync(0xffffffffu, free_rows);
             if (lane == 0 && free_rows) atomicAdd(&sh.not_over, (unsigned int)free_rows);
@@ -1071,11 +1148,11 @@ __global__ void __launch_bounds__(RS_THREADS, 1) pre_route_summaries(const Route
     } else if (warp == RS_IO_WARP) {
         rs_io_loop<ADMIT, WHOLE>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
     } else if (warp >= RS_LIST_WARP) {
-        if (LISTS) rs_list_loop<WHOLE>(sh, rows, sc, I, mean);
+        if (LISTS) rs_list_loop<WHOLE>(sh, rows, sc, I, mean, a.guard[GUARD_MAX_PD] < (1ull << 29) ? (int)a.guard[GUARD_MAX_PD] : 1 << 29);
     } else if ((warp & 3) != 0) {
         const int me = (warp >> 2) * 3 + (warp & 3) - 1;
-        if ((H & 1) == 0) rs_fold_loop<true, ADMIT, WHOLE>(a, sh, rows, sc, me, near_steps);
-        else rs_fold_loop<false, ADMIT, WHOLE>(a, sh, rows, sc, me, near_steps);
+        if ((H & 1) == 0) rs_fold_loop<true, ADMIT, WHOLE, LISTS>(a, sh, rows, sc, me, near_steps);
+        else rs_fold_loop<false, ADMIT, WHOLE, LISTS>(a, sh, rows, sc, me, near_steps);
     }
     __syncthreads();
     const bool blocked = ADMIT && sh.blocked;
