@@ -37,6 +37,10 @@ void release(pre_ctx* c) {
     cudaFree(c->d_fused_sync);
     cudaFree(c->d_rs_summary);
     cudaFree(c->d_rs_over);
+    cudaFree(c->d_rs_near);
+    cudaFree(c->d_rs_far);
+    cudaFree(c->d_rs_applied);
+    cudaFree(c->d_rs_ramps);
     cudaFree(c->d_rs_guard);
     cudaFree(c->d_rs_handled);
     delete c;
@@ -121,6 +125,10 @@ int pre_create(const pre_config* cfg, pre_ctx** out) {
     if (e == cudaSuccess && c->route_summary_smem) {
         e = alloc_zero(&c->d_rs_summary, (size_t)2 * I);
         if (e == cudaSuccess) e = alloc_zero(&c->d_rs_over, (size_t)I);
+        if (e == cudaSuccess) e = alloc_zero(&c->d_rs_near, (size_t)64 * I);
+        if (e == cudaSuccess) e = alloc_zero(&c->d_rs_far, (size_t)32 * I);
+        if (e == cudaSuccess) e = alloc_zero(&c->d_rs_applied, (size_t)cfg->max_requests);
+        if (e == cudaSuccess) e = alloc_zero(&c->d_rs_ramps, 2);
     }
     if (e != cudaSuccess) {
         const bool oom = (e == cudaErrorMemoryAllocation);

@@ -68,9 +68,13 @@ struct pre_ctx {
     int route_path;                 // PRE_ROUTE_AUTO / _SCAN / _SUMMARY
     size_t route_summary_smem;
     size_t route_summary_smem_admit;    // the same for the kernel with the admission queue
-    unsigned long long* d_rs_summary;   // [I] {token count, largest cell + step, its first step, cell 0} per row (16 bytes)
+    unsigned long long* d_rs_summary;   // [I] {token count, largest cell + step, its first step, the same of the first steps} per row (16 bytes)
+    unsigned int* d_rs_near;        // [I][64] a row's first cells during a batch
+    unsigned int* d_rs_far;         // [I][32] bounds of cell + step of the others
+    unsigned char* d_rs_applied;    // [max_requests] 1: the map has this request of the batch already (zero between calls)
+    long long* d_rs_ramps;          // {first table row, rows} whose ramps the maps lack after the routing kernel
     int32_t* d_rs_over;             // [I] steps of a row above the overload level (admission queue)
-    unsigned long long* d_rs_guard; // [8] what the summarising kernel found (largest cell, totals of the batch, ...)
+    unsigned long long* d_rs_guard; // [8] what the summarising kernel found (largest cell, totals of the batch, ...; zero between calls)
     int* d_rs_handled;              // 1 when the summary kernel routed the last batch, 0 when it left it to the scanning kernel
 };
 

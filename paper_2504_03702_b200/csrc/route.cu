@@ -138,7 +138,9 @@ struct RouteArgs {
     unsigned int* abort_key;    // 0xffffffff - (smallest exchange number at which a block's wait ran out); 0: none
     unsigned int* abort_count;  // blocks that have given up
     unsigned int spin_limit;    // polls before a wait is declared lost
-    const int* done_elsewhere;  // when set and non-zero: the batch has been routed by the summary kernel, nothing to do
+    const int* done_elsewhere;  // when set and non-zero: the batch has been routed by the summary kernel; what is left to do is
+    const long long* ramps;     // the ramps of these table rows {first, rows},
+    unsigned char* applied;     // but for those marked here (the marks are taken back)
     int max_rows;       // ceil(I / G)
     size_t resident_bytes;  // shared memory per block left for resident rows
     // admission queue (ADMIT kernels only): a ring of waiting requests, entry q at (head + q) mod capacity
@@ -345,6 +347,33 @@ __device__ __forceinline__ void inspect_row_chunks(const int64_t* __restrict__ r
     *max_lo = m;
 }
 
+// The map update of Sec. 4.3.1 for the requests that the summary kernel has routed, by the whole grid: integer
+// reductions, so their order does not matter.  A warp takes one table row at a time, or eight when there are many, and each
+// of them with consecutive lanes on consecutive cells.
+__device__ __forceinline__ void add_ramps(const RouteArgs& a) {
+    const int lane = threadIdx.x & 31, H = a.H;
+    const long long first = a.ramps[0], count = a.ramps[1];
+    const long long warps = (long long)gridDim.x * ROUTE_WARPS, me = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const int each = count > 8 * warps ? 8 : 1;
+    for (long long base = me * each; base < count; base += warps * each) {
+        const long long k = base + lane;
+        int P = 0, len = 0, w = 0;
+        if (lane < each && k < count) {
+            if (a.applied[k]) a.applied[k] = 0;
+            else {
+                P = a.prompt[first + k]; w = a.instance[first + k];
+                const int D = a.predicted[first + k];
+                len = D < H ? D : H;
+            }
+        }
+        for (int src = 0; src < each; ++src) {
+            const int p = __shfl_sync(0xffffffffu, P, src), n = __shfl_sync(0xffffffffu, len, src);
+            unsigned long long* row = reinterpret_cast<unsigned long long*>(a.curves) + (size_t)__shfl_sync(0xffffffffu, w, src) * H;
+            for (int j = lane; j < n; j += 32) atomicAdd(row + j, (unsigned long long)(p + j));
+        }
+    }
+}
+
 // ADMIT adds the admission queue of Sec. 4.3.3: every block keeps, for its rows, the number of
 // steps above the overload level (the scaler's criterion of Sec. 4.3.2) and publishes with its
 // best row whether all its rows are overloaded; when all blocks say so the request that was
@@ -384,7 +413,10 @@ __global__ void __launch_bounds__(ROUTE_THREADS, 1) pre_route_persistent(const R
     __shared__ int sh_all_over[2];        // ADMIT: every block reported all its rows overloaded (by exchange parity)
     constexpr int RS_RESIDENT = 1, RS_WIDE = 2;
 
-    if (a.done_elsewhere && *a.done_elsewhere) return;   // the same word for every block; nobody writes it meanwhile
+    if (a.done_elsewhere && *a.done_elsewhere) {   // the same word for every block; nobody writes it meanwhile
+        if (!ADMIT) add_ramps(a);
+        return;
+    }
     const int G = gridDim.x, b = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int I = a.I, H = a.H;
@@ -1031,7 +1063,7 @@ static void fill_route_args(RouteArgs& a, pre_ctx* ctx, const int32_t* arr_promp
     a.abort_key = reinterpret_cast<unsigned int*>(ctx->d_abort + 1);
     a.abort_count = reinterpret_cast<unsigned int*>(ctx->d_abort + 2);
     a.spin_limit = ctx->spin_limit;
-    a.done_elsewhere = nullptr;
+    a.done_elsewhere = nullptr; a.ramps = ctx->d_rs_ramps; a.applied = ctx->d_rs_applied;
     a.max_rows = (a.I + ctx->route_blocks - 1) / ctx->route_blocks;
     a.resident_bytes = ctx->route_resident_bytes;
     a.queue_prompt = nullptr; a.queue_predicted = nullptr; a.queue_state = nullptr; a.queue_entry = nullptr;
@@ -1056,8 +1088,10 @@ cudaError_t pre_launch_route(pre_ctx* ctx, const int32_t* arr_prompt, const int3
                                      generated, predicted, instance, n_requests, choice, score, s);
         if (e != cudaSuccess) return e;
     }
-    e = cudaMemsetAsync(ctx->d_abort, 0, 3 * sizeof(int), s);   // flag, agreed exchange, blocks met
-    if (e != cudaSuccess) return e;
+    if (!summaries) {    // (else the summary kernel clears them when it declines)
+        e = cudaMemsetAsync(ctx->d_abort, 0, 3 * sizeof(int), s);   // flag, agreed exchange, blocks met
+        if (e != cudaSuccess) return e;
+    }
     RouteArgs a;
     fill_route_args(a, ctx, arr_prompt, arr_predicted, n_arrivals, curves, queued_p, current_d, prompt, generated,
                     predicted, instance, n_requests, choice, score);
@@ -1074,10 +1108,7 @@ cudaError_t pre_launch_route_admit(pre_ctx* ctx, const int32_t* arr_prompt, cons
                                    int64_t* queued_p, int64_t* current_d, int32_t* prompt, int32_t* generated,
                                    int32_t* predicted, int32_t* instance, int64_t* n_requests, int32_t* choice,
                                    double* score, cudaStream_t s) {
-    // The kernel's blocks read the queue's head and length while block 0 may already be writing the
-    // new ones: they read a copy taken here, in stream order.
-    cudaError_t e = cudaMemcpyAsync(ctx->d_queue_entry, queue_state, 2 * sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     // For a whole number c, c > x holds exactly when c > floor(x): the per-cell test is done on integers.
     double hot = floor(overload_level * (double)ctx->cfg.capacity_tokens);
     if (hot > 9.2e18) hot = 9.2e18;
@@ -1092,8 +1123,13 @@ cudaError_t pre_launch_route_admit(pre_ctx* ctx, const int32_t* arr_prompt, cons
                                            s);
         if (e != cudaSuccess) return e;
     }
-    e = cudaMemsetAsync(ctx->d_abort, 0, 3 * sizeof(int), s);
-    if (e != cudaSuccess) return e;
+    if (!summaries) {
+        // The kernel's blocks read the queue's head and length while block 0 may already be writing the
+        // new ones: they read a copy taken here, in stream order.
+        e = cudaMemcpyAsync(ctx->d_queue_entry, queue_state, 2 * sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_abort, 0, 3 * sizeof(int), s);
+        if (e != cudaSuccess) return e;
+    }
     RouteArgs a;
     fill_route_args(a, ctx, arr_prompt, arr_predicted, n_arrivals, curves, queued_p, current_d, prompt, generated,
                     predicted, instance, n_requests, choice, score);

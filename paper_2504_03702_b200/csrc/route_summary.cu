@@ -3,34 +3,41 @@
 // The score of an arrival (P, D) against a row c[0..H) needs one number of the row, the peak
 // of the map with the arrival's ramp added (Sec. 4.3.1 update), Dc = min(D, H):
 //     peak = max( max_{j<Dc}(c[j] + P + j),  max_{j>=Dc} c[j] ).
-// A few numbers per row decide it without reading the row in almost every case:
-//     top = max_j (c[j] + j)      jtop = no step below which the maximum is first taken      c0 = c[0]
+// Two numbers per row decide it without reading the row in almost every case:
+//     top = max_j (c[j] + j)      jtop = no step below which the maximum is first taken
 //   * Dc > jtop:  the ramp covers the step of the maximum, so max_{j<Dc}(c[j]+j) = top; and
 //                 P + top >= c[j] for every j, so   peak = P + top   exactly;
-//   * always:     P + c0 <= peak <= P + top  (the ramp covers step 0; top bounds every step);
+//   * always:     top - jtop <= peak <= P + top;
 //   * P + top <= theta: no penalty whatever the peak is.
 // In maps of requests that are being decoded the occupancy falls as requests finish and the maximum of c[j] + j
 // sits at the first steps.  The kernel never relies on that: a row that is only bounded and could hold the
 // smallest score is scanned cell by cell.
 //
-// Two kernels per batch:
+// A routed arrival changes its row's cells, but what the next decisions need of them is top and jtop.  So a row is kept as
+// its first 64 cells (exact) and, per stretch of the other steps, an upper bound of c[j] + j: adding an arrival to those
+// costs one access by one warp.  While no stretch's bound exceeds the largest of the first steps, top and jtop are exact
+// ("near" rows); the map itself receives all ramps of the batch at the end, in one pass by the whole GPU.  When a bound does
+// exceed it, the row is brought up to date cell by cell and its numbers are taken afresh; a row whose maximum really lies
+// beyond the first steps ("full" rows) gets its ramps at once, as do all rows when the admission queue counts cells.
+//
+// Two kernels per batch, and a third for the ramps (pre_route_persistent of route.cu, when it has nothing to route):
 //   pre_summarise_rows   one pass over the maps: the numbers of every row, the rows' token
 //                        counts (queued_p + current_d) and the guards that tell whether 32-bit
 //                        arithmetic stays exact for the whole batch;
 //   pre_route_summaries  routes the batch with ONE block whose warps have different jobs:
-//     deciding warp  takes the arrivals one by one.  It holds rows in registers (token count a and penalty key), takes
+//     deciding warp  takes the arrivals one by one.  It holds rows in registers (two keys each), takes
 //                    every row's score for the arrival, the smallest by two warp reductions, and updates the winner in
 //                    place: no other warp is in this chain.  Up to 256 instances it holds all rows.  Beyond, it holds
 //                    the at most 128 rows of a list, and a table that bounds the scores of all other rows from below:
 //                    while the best row of the list beats that bound it is the best row of all.
-//     list warps     (3, beyond 256 instances) build the next list while the present one is being used up: the rows
+//     list warps     (beyond 256 instances) build the next list while the present one is being used up: the rows
 //                    whose score is within a margin of the smallest one for any of eight prompt lengths, and the
 //                    bounds of the rest.  Scores only grow during a batch, so a list that is a little behind is valid.
-//     folding warps  (12) add each routed request to its row (Sec. 4.3.1 update) and take the row's new
-//                    numbers in the same pass, one warp per request; they also scan single rows for the deciding warp;
+//     folding warps  add each routed request to its row's numbers, one warp per request; they also scan single rows for
+//                    the deciding warp;
 //     io warp        reads the arrivals ahead of the decisions and writes the results behind them.
-//   Warps 0, 4, 8, ... share one of the SM's four schedulers.  The deciding warp is warp 0, the io warp warp 4, and the
-//   others of that scheduler have nothing to do: the chain of dependent instructions of warp 0 is the time of the batch.
+//   Warps 0, 4, 8, ... share one of the SM's four schedulers.  The deciding warp is warp 0 and the others of that scheduler
+//   have nothing to do: the chain of dependent instructions of warp 0 is the time of the batch.
 // Nothing in that chain waits for a fold: a row between its decision and the end of its fold is "pending" and takes
 // part with a lower bound (its token count is exact at once, its top grows by at least P).  Only when a pending row has
 // the smallest score the warp waits for that fold.  The decisions are therefore the same as with every fold done at once.
@@ -39,96 +46,173 @@
 #include <math_constants.h>
 
 #include <cmath>
+#include <type_traits>
 
 namespace {
 
-constexpr int RS_WARPS = 20;
-constexpr int RS_THREADS = 32 * RS_WARPS;
-constexpr int RS_IO_WARP = 4;
-constexpr int RS_FOLD_WARPS = 12;           // warps 1-3, 5-7, 9-11, 13-15
-constexpr int RS_LIST_WARP = 17;            // 17, 18, 19
-constexpr int RS_LIST_THREADS = 96;
+constexpr int RS_MAX_FOLD_WARPS = 11;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
 constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
 constexpr int RS_LIST_ROWS = 128;           // rows of a list (4 per lane)
-constexpr int RS_NEAR_ROWS = 512;           // rows a list warp keeps for a closer look at once
+constexpr int RS_NEAR_ROWS = 2304;          // rows the list warps keep for a closer look at once
 constexpr int RS_PROBES = 8;                // prompt lengths for which a list has the best rows
-// A row whose top lies further out is treated as only bounded (by c0): `jmax`, the largest jtop of the other rows, decides
-// which arrivals take the quick way (Dc > jmax).
-constexpr int RS_NEAR_DIRECT = 128, RS_NEAR_LISTS = 32;
-constexpr int RS_MAX_ROWS = 10240;          // instances up to which the context offers this router (shared memory: 20 bytes each),
+constexpr int RS_NEAR = 64;                 // steps kept exactly; the rest in 32 stretches of whole chunks of as many steps
+// A row whose top lies further out than this is "far": the deciding warp has only a lower bound of its score, and the
+// arrivals that take its quick way are those that reach the largest jtop of the other rows.
+constexpr int RS_LIMIT = 32;
+constexpr int RS_MAX_ROWS = 10240;          // instances up to which the context offers this router (shared memory),
 constexpr int RS_MAX_BINARY64_ROWS = 5120;  // and with binary64 scores
 constexpr int SUM_THREADS = 256;
 constexpr unsigned int RS_SPIN_LIMIT = 1u << 24;   // polls of shared memory (some 0.5 s) before a wait inside the block is abandoned
-constexpr int RS_NO_ROW = 0x7fffffff;
+constexpr int RS_NO_ROW = 0x3fffffff;
+constexpr unsigned int RS_GIVEN = 0x40000000u;
+constexpr unsigned int FULL_MASK = 0xffffffffu;
 
-// guard words written by the summarising kernel
+// guard words written by the summarising kernel; the routing kernel clears them for the next call
 constexpr int GUARD_MAX_CELL = 0, GUARD_MAX_BASE = 1, GUARD_BAD = 2, GUARD_SUM_RAMP = 3, GUARD_SUM_TOKENS = 4,
-              GUARD_MAX_PD = 5;
+              GUARD_MAX_PD = 5, GUARD_SUM_BASE = 6, GUARDS = 7;
+
+// What a warp finds out about a row in one pass: lane l has cells 2l and 2l+1 of the first 64 and the largest c[j] + j of
+// stretch l (0: no such stretch).
+struct RowNumbers {
+    unsigned int near0, near1, far;
+    unsigned int top, jtop;      // all lanes alike
+    unsigned int peak;           // largest cell, with the ramp
+    int above;                   // cells above the overload level
+    bool bad;                    // a cell (or cell + step) outside [0, 2^32)
+};
+
+__device__ __forceinline__ int far_chunks(int H) { return max(1, (((H + RS_NEAR - 1) / RS_NEAR - 1) + 31) / 32); }   // chunks per stretch
+
+// One pass over a row by one warp.  RAMP: with the arrival (P, Dc) added; STORE: and written back.  16-byte accesses when H
+// is even (a lane holds two neighbouring cells, the warp 512 contiguous bytes), eight in flight per lane.
+// CHECK: the cells may hold anything.
+template <bool RAMP, bool STORE, bool COUNT, bool CHECK>
+__device__ __forceinline__ RowNumbers row_pass(int64_t* row, int H, int P, int Dc, long long hot) {
+    constexpr int BATCH = 8;
+    const int lane = threadIdx.x & 31;
+    const bool vec = (H & 1) == 0;
+    const int per = far_chunks(H);
+    RowNumbers n;
+    n.near0 = n.near1 = n.far = n.peak = 0;
+    n.above = 0;
+    n.bad = false;
+    unsigned int top = 0, jtop = 0;
+    #pragma unroll 1
+    for (int base = 0; base < H; base += BATCH * RS_NEAR) {
+        long long v[2 * BATCH];
+        #pragma unroll
+        for (int u = 0; u < BATCH; ++u) {
+            const int j = base + u * RS_NEAR + 2 * lane;
+            v[2 * u] = v[2 * u + 1] = 0;
+            if (vec) {
+                if (j < H) {
+                    const longlong2 q = CHECK ? __ldcs(reinterpret_cast<const longlong2*>(row + j)) : *reinterpret_cast<const longlong2*>(row + j);
+                    v[2 * u] = q.x; v[2 * u + 1] = q.y;
+                }
+            } else {
+                if (j < H) v[2 * u] = row[j];
+                if (j + 1 < H) v[2 * u + 1] = row[j + 1];
+            }
+        }
+        #pragma unroll
+        for (int u = 0; u < BATCH; ++u) {
+            const int first = base + u * RS_NEAR, j = first + 2 * lane;
+            if (first >= H) break;
+            if (CHECK) n.bad |= ((v[2 * u] | v[2 * u + 1]) >> 32) != 0;
+            unsigned int c0 = (unsigned int)v[2 * u], c1 = (unsigned int)v[2 * u + 1];
+            if (RAMP && j < Dc) {
+                c0 += (unsigned int)(P + j);
+                if (j + 1 < Dc) c1 += (unsigned int)(P + j + 1);
+                if (STORE) {   // (a pair whose second cell lies past the ramp writes that cell back unchanged)
+                    if (vec) *reinterpret_cast<longlong2*>(row + j) = make_longlong2((long long)c0, (long long)c1);
+                    else {
+                        row[j] = (long long)c0;
+                        if (j + 1 < Dc) row[j + 1] = (long long)c1;
+                    }
+                }
+            }
+            const unsigned int t0 = j < H ? c0 + (unsigned int)j : 0u, t1 = j + 1 < H ? c1 + (unsigned int)(j + 1) : 0u;
+            if (CHECK) n.bad |= (j < H && t0 < c0) || (j + 1 < H && t1 < c1);
+            if (COUNT) n.above += (j < H && (long long)c0 > hot) + (j + 1 < H && (long long)c1 > hot);
+            n.peak = max(n.peak, max(c0, c1));
+            const unsigned int t = max(t0, t1);
+            if (t > top) { top = t; jtop = (unsigned int)(j + 1 < H ? j + 1 : j); }   // a lane's steps ascend
+            if (first == 0) { n.near0 = c0; n.near1 = c1; }
+            else {
+                const unsigned int m = __reduce_max_sync(FULL_MASK, t);
+                if (lane == (first / RS_NEAR - 1) / per) n.far = max(n.far, m);
+            }
+        }
+    }
+    n.top = __reduce_max_sync(FULL_MASK, top);
+    n.jtop = __reduce_min_sync(FULL_MASK, top == n.top ? jtop : 0xffffffffu);
+    n.peak = __reduce_max_sync(FULL_MASK, n.peak);
+    if (COUNT) n.above = __reduce_add_sync(FULL_MASK, n.above);
+    return n;
+}
 
 struct SumArgs {
-    const int64_t* curves;
+    int64_t* curves;
     const int64_t* queued_p;
     const int64_t* current_d;
     const int32_t* arr_prompt;
     const int32_t* arr_predicted;
     long long n_arrivals;
     int I, H;
-    uint4* summary;                // {token count, top, step of the top, cell 0} per row
+    uint4* summary;                // {token count, top, jtop | step of the next << 16, largest c[j] + j of the first steps} per row
+    uint2* near;                   // [I][32] the first 64 cells
+    unsigned int* far;             // [I][32] the stretches
     unsigned long long* guard;
     // admission queue (pre_route_admit): steps above the overload level per row, the waiting requests' totals
     int32_t* over;                 // NULL: not wanted
     long long hot;
     const int32_t* queue_prompt;
     const int32_t* queue_predicted;
-    const int64_t* queue_entry;    // {head, length} as they were when the call was made
+    const int64_t* queue_state;    // {head, length}
     long long queue_capacity;
 };
 
-// One warp per row.
+// The largest c[j] + j of the steps below RS_LIMIT, from the first cells, and no step below which it is first taken.
+__device__ __forceinline__ unsigned int first_top(unsigned int near0, unsigned int near1, int H, unsigned int& step) {
+    const int j = 2 * (threadIdx.x & 31), end = H < RS_LIMIT ? H : RS_LIMIT;
+    const unsigned int t = max(j < end ? near0 + (unsigned int)j : 0u, j + 1 < end ? near1 + (unsigned int)(j + 1) : 0u);
+    const unsigned int top = __reduce_max_sync(FULL_MASK, t);
+    step = __reduce_min_sync(FULL_MASK, t == top && j < end ? (unsigned int)(j + 1 < end ? j + 1 : j) : 0xffffffffu);
+    return top;
+}
+
+// One warp per row; block totals of the guards in shared memory first.
 __global__ void __launch_bounds__(SUM_THREADS) pre_summarise_rows(const SumArgs a) {
+    __shared__ unsigned long long sh_guard[GUARDS];
     const int tid = threadIdx.x, lane = tid & 31;
     const int row = blockIdx.x * (SUM_THREADS / 32) + (tid >> 5);
     const int H = a.H;
+    if (tid < GUARDS) sh_guard[tid] = 0;
+    __syncthreads();
     bool bad = false;
     if (row < a.I) {
-        const int64_t* src = a.curves + (size_t)row * H;
-        unsigned int rmax = 0, top = 0, jtop = 0;
-        int above = 0;
-        auto take = [&](long long v, int j) {
-            above += v > a.hot;
-            bad |= (v < 0) || (v > 0xffffffffLL);
-            const unsigned int c = (unsigned int)v;
-            rmax = max(rmax, c);
-            const unsigned long long t = (unsigned long long)c + (unsigned long long)j;
-            if (t > 0xffffffffull) bad = true;
-            if ((unsigned int)t > top) { top = (unsigned int)t; jtop = (unsigned int)j; }   // a lane's steps ascend
-        };
-        if ((H & 1) == 0) {
-            for (int j = 2 * lane; j < H; j += 64) {
-                const longlong2 v = __ldcs(reinterpret_cast<const longlong2*>(src + j));
-                take(v.x, j);
-                take(v.y, j + 1);
-            }
-        } else {
-            for (int j = lane; j < H; j += 32) take(__ldcs(src + j), j);
-        }
-        rmax = __reduce_max_sync(0xffffffffu, rmax);
-        const unsigned int t = __reduce_max_sync(0xffffffffu, top);
-        const unsigned int jt = __reduce_min_sync(0xffffffffu, top == t ? jtop : 0xffffffffu);
-        above = __reduce_add_sync(0xffffffffu, above);
-        if (lane == 0 && a.over) a.over[row] = above;
+        const RowNumbers n = row_pass<false, false, true, true>(a.curves + (size_t)row * H, H, 0, 0, a.hot);
+        unsigned int step;
+        const unsigned int first = first_top(n.near0, n.near1, H, step);
+        bad = n.bad;
+        a.near[(size_t)row * 32 + lane] = make_uint2(n.near0, n.near1);
+        a.far[(size_t)row * 32 + lane] = n.far;
         if (lane == 0) {
+            if (a.over) a.over[row] = n.above;
             const long long q = a.queued_p[row], d = a.current_d[row];
             const long long tok = q + d;
             const bool ok = q >= 0 && d >= 0 && q <= 0xffffffffLL && d <= 0xffffffffLL && tok <= 0xffffffffLL;
             if (!ok) bad = true;
-            a.summary[row] = make_uint4(ok ? (unsigned int)tok : 0u, t, jt, (unsigned int)src[0]);
-            if (ok) atomicMax(a.guard + GUARD_MAX_BASE, (unsigned long long)tok);
-            if (rmax) atomicMax(a.guard + GUARD_MAX_CELL, (unsigned long long)rmax);
+            a.summary[row] = make_uint4(ok ? (unsigned int)tok : 0u, n.top, n.jtop | (step << 16), first);
+            if (ok) {
+                atomicMax(sh_guard + GUARD_MAX_BASE, (unsigned long long)tok);
+                atomicAdd(sh_guard + GUARD_SUM_BASE, (unsigned long long)tok);
+            }
+            atomicMax(sh_guard + GUARD_MAX_CELL, (unsigned long long)n.peak);
         }
     }
-    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.guard + GUARD_BAD, 1ull);
+    if (__any_sync(FULL_MASK, bad) && lane == 0) atomicOr(sh_guard + GUARD_BAD, 1ull);
     // the arrivals' own totals: what the batch can add to a cell (ramps) and to a row's token count
     unsigned long long ramp = 0, tokens = 0;
     unsigned int max_pd = 0;
@@ -141,7 +225,7 @@ __global__ void __launch_bounds__(SUM_THREADS) pre_summarise_rows(const SumArgs 
     for (long long k = (long long)blockIdx.x * SUM_THREADS + tid; k < a.n_arrivals; k += (long long)gridDim.x * SUM_THREADS)
         count(a.arr_prompt[k], a.arr_predicted[k]);
     if (a.queue_capacity > 0) {   // the waiting requests are routed before the arrivals
-        long long q_head = a.queue_entry[0], q_len = a.queue_entry[1];
+        long long q_head = a.queue_state[0], q_len = a.queue_state[1];
         if (q_head < 0 || q_head >= a.queue_capacity) q_head = 0;
         if (q_len < 0) q_len = 0;
         if (q_len > a.queue_capacity) q_len = a.queue_capacity;
@@ -152,14 +236,23 @@ __global__ void __launch_bounds__(SUM_THREADS) pre_summarise_rows(const SumArgs 
     }
     #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-        ramp += __shfl_xor_sync(0xffffffffu, ramp, off);
-        tokens += __shfl_xor_sync(0xffffffffu, tokens, off);
+        ramp += __shfl_xor_sync(FULL_MASK, ramp, off);
+        tokens += __shfl_xor_sync(FULL_MASK, tokens, off);
     }
-    max_pd = __reduce_max_sync(0xffffffffu, max_pd);
+    max_pd = __reduce_max_sync(FULL_MASK, max_pd);
     if (lane == 0 && (ramp | tokens)) {
-        atomicAdd(a.guard + GUARD_SUM_RAMP, ramp);
-        atomicAdd(a.guard + GUARD_SUM_TOKENS, tokens);
-        atomicMax(a.guard + GUARD_MAX_PD, (unsigned long long)max_pd);
+        atomicAdd(sh_guard + GUARD_SUM_RAMP, ramp);
+        atomicAdd(sh_guard + GUARD_SUM_TOKENS, tokens);
+        atomicMax(sh_guard + GUARD_MAX_PD, (unsigned long long)max_pd);
+    }
+    __syncthreads();
+    if (tid < GUARDS) {
+        const unsigned long long v = sh_guard[tid];
+        if (v) {
+            if (tid == GUARD_BAD) atomicOr(a.guard + tid, v);
+            else if (tid == GUARD_SUM_RAMP || tid == GUARD_SUM_TOKENS || tid == GUARD_SUM_BASE) atomicAdd(a.guard + tid, v);
+            else atomicMax(a.guard + tid, v);
+        }
     }
 }
 
@@ -181,14 +274,19 @@ struct RouteSumArgs {
     int I, H;
     double theta, beta;
     const uint4* summary0;
-    const unsigned long long* guard;
+    uint2* near;                   // [I][32], [I][32]: see SumArgs
+    unsigned int* far;
+    unsigned char* applied;        // [max_requests] 1: the map has this request of the batch already (zero between calls)
+    unsigned long long* guard;
     int* status;
-    int* handled;   // 1: this kernel routed the batch; 0: the scanning kernel has to
+    int* give_up;                  // three words that the scanning kernel finds cleared
+    int* handled;                  // 1: this kernel routed the batch; 0: the scanning kernel has to
+    long long* ramps;              // {first table row, rows} whose ramps the maps still lack
     // admission queue (ADMIT kernels only): a ring of waiting requests, entry q at (head + q) mod capacity
     int32_t* queue_prompt;
     int32_t* queue_predicted;
     int64_t* queue_state;          // {head, length}, rewritten at the end
-    const int64_t* queue_entry;    // the same two words as they were when the call was made
+    int64_t* queue_entry;          // a copy of the two words for the scanning kernel
     long long queue_capacity;
     int32_t* queue_choice;         // results for the entries that were waiting at entry
     long long hot;                 // floor(overload_level * M): a cell counts when it is above
@@ -197,51 +295,57 @@ struct RouteSumArgs {
 };
 
 // Rows in shared memory (structure of arrays):
-//   rec    {token count, key}: the key is top (jtop below the near limit) or c0 (beyond: RS_FAR), a lower bound while the
-//          row is pending; whole-number scores keep token count + beta * (key - theta) in its place
-//   flags  jtop | RS_NOT_OVER (ADMIT: the row was not overloaded when it was last folded) | RS_FAR, or RS_PENDING
-//          (written last when a fold ends)
-//   top, c0  as of the last fold
-constexpr unsigned int RS_PENDING = 0x80000000u, RS_FAR = 0x40000000u, RS_NOT_OVER = 0x20000000u, RS_JTOP = 0xffffu;
+//   rec    {a, b}, even: the score of an arrival is at least max(a, b + what its prompt adds), and that but for the rounding
+//          of the keys unless the row is far or pending
+//   state  jtop | RS_FAR | RS_FULL | RS_DEFERRED (the map lacks ramps) | RS_NOT_OVER (ADMIT: the row was not overloaded when it
+//          was last folded)
+//   top, tok   top and token count (whole-number scores: half of a)
+//   pending  1 from the decision for the row to the end of its fold; cleared last
+constexpr unsigned int RS_FAR = 0x40000000u, RS_NOT_OVER = 0x20000000u, RS_FULL = 0x10000000u, RS_DEFERRED = 0x08000000u, RS_JTOP = 0xffffu;
 struct Rows {
-    uint2* rec;
-    unsigned int* flags;
+    int2* rec;
+    unsigned int* state;
     unsigned int* top;
-    unsigned int* c0;
+    unsigned int* pending;
+    unsigned int* tok;
 };
-constexpr size_t RS_ROW_BYTES = sizeof(uint2) + 3 * sizeof(unsigned int);
 
 struct RsShared {
     // what the deciding warp tells the folding warps and the io warp, read with one access
     uint4 ctl;                              // {decisions made, scans asked for, 1: no more of either, 1: a wait was abandoned}
-    int4 items[RS_ITEMS];                   // {P, D, min(D, H) | code of P << 16, what P adds to a row's b} of the requests, in order
-    int item_at[RS_ITEMS];                  // and their indices in the batch
-    int4 jobs[RS_ITEMS];                    // {row, P, D, whole-number score} of the decisions
-    double score[RS_ITEMS];                 // their binary64 scores
+    int4 items[RS_ITEMS];                   // of the requests to route, in order: {what P adds to b, P + D as a key, less one, min(D, H)
+                                            // (0: not for the quick way), offset of P's entry in the table}
+    int2 raw[RS_ITEMS];                     // {P, D}
+    int item_at[RS_ITEMS];                  // their indices in the batch
+    uint2 jobs[RS_ITEMS];                   // decisions: {row | RS_GIVEN if the peak is given, peak}
+    double score[RS_ITEMS];                 // their scores, from the folding warps
     int4 table[2][32];                      // by code of the prompt: {bounds of the rows outside the list}
     int list_row[2][RS_LIST_ROWS];
     int list_n[2];
     unsigned int bucket_a[32], bucket_b[32];   // (list warps) smallest keys of the rows outside the list
-    int probe_t[RS_PROBES];                 // (list warps) smallest scores at the probes
-    unsigned short near_row[RS_LIST_THREADS / 32][RS_NEAR_ROWS];
+    unsigned int probe_t[RS_PROBES];        // (list warps) smallest scores at the probes
+    unsigned short near_row[RS_NEAR_ROWS];
     int list_count;
     unsigned int list_met;                  // (list warps) arrivals at their meetings
     unsigned int lists_wanted, lists_ready;
-    unsigned int done[RS_FOLD_WARPS];       // the next decision each folding warp will fold
-    unsigned int scans_done[RS_FOLD_WARPS];
+    unsigned int done[RS_MAX_FOLD_WARPS];   // the next decision each folding warp will fold
+    unsigned int scans_done[RS_MAX_FOLD_WARPS];
+    unsigned short slow_group[(RS_MAX_ROWS + 31) / 32 + 4];   // (deciding warp) groups of 32 rows to look at again
     int scan_row[32];
     unsigned int peak[32];
     int scan_P, scan_Dc, scan_n;
-    unsigned int jmax;                      // largest jtop of the rows that are not far
+    unsigned int jmax;                      // largest step that a row's b stands for
     unsigned int items_ready;               // items written so far
     unsigned int items_end;                 // 1: there will be no more
-    unsigned int not_over;                  // ADMIT: rows that turned out not to be overloaded, a running count
+    unsigned int written;                   // results written so far
+    unsigned int flush;                     // ... and as many are asked for
+    unsigned int not_over;                  // ADMIT: rows that are not overloaded, as far as folded
     int blocked;                            // ADMIT: a request found every instance overloaded ...
     long long blocked_k;                    // ... this one
     int mode;                               // 0: decline the batch
     long long n0;
     int first_bad, first_full;              // the first items dropped as malformed / for a full table
-    int warp_ok[RS_WARPS];                  // (the tail of ADMIT)
+    int warp_ok[32];                        // (the tail of ADMIT)
     long long joined;
     int any_bad;
 };
@@ -260,8 +364,8 @@ __device__ __forceinline__ unsigned int ld_volatile(const unsigned int* p) {
     asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
     return v;
 }
-__device__ __forceinline__ uint2 ld_volatile2(const uint2* p) {
-    uint2 v;
+__device__ __forceinline__ int2 ld_volatile2(const int2* p) {
+    int2 v;
     asm volatile("ld.volatile.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(smem_u32(p)) : "memory");
     return v;
 }
@@ -270,94 +374,23 @@ __device__ __forceinline__ uint4 ld_volatile4(const uint4* p) {
     asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem_u32(p)) : "memory");
     return v;
 }
-// Stores under a predicate: in the deciding warp a branch around a store costs more than ten other instructions.
-__device__ __forceinline__ void st_if(bool p, unsigned int* at, unsigned int v) {
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.u32 [%1], %2; }" ::"r"((unsigned int)p), "r"(smem_u32(at)), "r"(v) : "memory");
-}
-__device__ __forceinline__ void st_if(bool p, uint2* at, uint2 v) {
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.v2.u32 [%1], {%2, %3}; }" ::"r"((unsigned int)p), "r"(smem_u32(at)),
-                 "r"(v.x), "r"(v.y) : "memory");
-}
-__device__ __forceinline__ void st_if(bool p, int4* at, int4 v) {
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.v4.u32 [%1], {%2, %3, %4, %5}; }" ::"r"((unsigned int)p), "r"(smem_u32(at)),
-                 "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-__device__ __forceinline__ void st_if(bool p, double* at, double v) {
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.f64 [%1], %2; }" ::"r"((unsigned int)p), "r"(smem_u32(at)), "d"(v) : "memory");
+__device__ __forceinline__ int4 ld_table(unsigned int at) {
+    int4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at));
+    return v;
 }
 __device__ __forceinline__ void acquire_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 
 // A wait of a whole warp on words that other warps of this block write.  False: abandoned, here or elsewhere.
 template <typename Cond>
 __device__ __forceinline__ bool rs_wait(RsShared& sh, Cond&& ready, unsigned int nap = 0) {
-    for (unsigned int polls = 0; !__all_sync(0xffffffffu, ready()); ++polls) {   // (all lanes take the same way)
-        if ((polls & 255u) == 255u && __any_sync(0xffffffffu, ld_volatile(&sh.ctl.w) != 0)) return false;
+    for (unsigned int polls = 0; !__all_sync(FULL_MASK, ready()); ++polls) {   // (all lanes take the same way)
+        if ((polls & 255u) == 255u && __any_sync(FULL_MASK, ld_volatile(&sh.ctl.w) != 0)) return false;
         if (polls > RS_SPIN_LIMIT) { st_release(&sh.ctl.w, 1u); return false; }
         if (nap) __nanosleep(nap);
     }
     return true;
 }
-
-// ---- Scores.  Whole-number scores (beta and theta whole numbers, every possible score below 2^30: each binary64
-// operation is exact and the score is the same number in 32-bit integer arithmetic, taken here without the arrival's
-// own P + D), and binary64 scores (each operation rounded on its own; bounds of the rows outside the list in binary32,
-// rounded down).
-// S: a score.  X: what is kept per row beside the token count.  K: bounds.
-template <bool WHOLE> struct Scores;
-
-template <> struct Scores<true> {
-    typedef unsigned int S;
-    typedef int K;
-    static __device__ __forceinline__ S none() { return 0xffffffffu; }
-    static __device__ __forceinline__ K no_a() { return 0x60000000; }
-    static __device__ __forceinline__ K no_b() { return 0x3fffffff; }    // (room for beta * P on top)
-    static __device__ __forceinline__ K lowest() { return -0x40000000; }
-    int theta, beta, code_base;
-    __device__ __forceinline__ void start(double theta_d, double beta_d, unsigned long long peak_bound, int mean) {
-        beta = (int)beta_d;
-        // a threshold above every peak of the batch is as good as any other: the penalty is never paid
-        theta = theta_d > (double)peak_bound ? (int)(peak_bound + 1) : (int)theta_d;
-        code_base = __float_as_int(fmaxf((float)mean * (1.0f / 32.0f) * (float)beta, 1.0f)) >> 21;
-    }
-    __device__ __forceinline__ unsigned int key(unsigned int tokens, unsigned int t) const {
-        return tokens + (unsigned int)(beta * ((int)t - theta));
-    }
-    static __device__ __forceinline__ uint2 absent() { return make_uint2((unsigned int)no_a(), (unsigned int)no_b()); }
-    // codes of prompt lengths, and of the prompt length at which a row starts to pay: monotone, so different codes decide
-    // which is larger.  Four per octave.
-    __device__ __forceinline__ int code(float v) const { return min(max((__float_as_int(v) >> 21) - code_base + 1, 1), 31); }
-    __device__ __forceinline__ int prompt_code(int p) const { return code((float)(beta * p)); }
-    __device__ __forceinline__ int row_code(uint2 r) const {    // 0: pays for every prompt length
-        const int z = (int)(r.x - r.y);
-        return z < 0 ? 0 : code((float)z);
-    }
-    static __device__ __forceinline__ K row_a(uint2 r) { return (int)r.x; }
-    __device__ __forceinline__ K row_b(uint2 r) const { return (int)r.y; }
-    __device__ __forceinline__ K probe(int p) const { return (int)min((long long)beta * p, 0x3fffffffLL); }     // what a prompt of p tokens adds to a row's b
-    static __device__ __forceinline__ K plus(K b, K bp) { return b + bp; }
-    static __device__ __forceinline__ unsigned int order(K v) { return (unsigned int)v ^ 0x80000000u; }
-    static __device__ __forceinline__ K unorder(unsigned int v) { return (int)(v ^ 0x80000000u); }
-    static __device__ __forceinline__ int bits(K v) { return v; }
-    static __device__ __forceinline__ K from_bits(int v) { return v; }
-    static __device__ __forceinline__ K from_margin(int m) { return m; }
-    // one arrival
-    int bp, limit;
-    unsigned int pd;
-    __device__ __forceinline__ void arrival(int4 it) { bp = it.w; limit = theta - it.x; pd = (unsigned int)it.x + (unsigned int)it.y; }
-    __device__ __forceinline__ K arrival_bp() const { return bp; }
-    __device__ __forceinline__ S value(uint2 r) const { return (unsigned int)max((int)r.x, (int)r.y + bp); }
-    // the row after it has received the arrival: a lower bound, exact in its token count.  covers: the ramp reaches the key's step
-    __device__ __forceinline__ uint2 with_arrival(uint2 r, bool covers) const {
-        return make_uint2(r.x + pd, r.y + pd + (covers ? (unsigned int)bp : 0u));
-    }
-    __device__ __forceinline__ bool no_penalty(unsigned int top) const { return limit >= 0 && top <= (unsigned int)limit; }
-    // from a top (or c0), from a peak
-    __device__ __forceinline__ S of_top(unsigned int tokens, unsigned int top) const { return tokens + (unsigned int)(beta * max((int)top - limit, 0)); }
-    __device__ __forceinline__ S of_peak(unsigned int tokens, unsigned int peak) const { return tokens + (unsigned int)(beta * max((int)peak - theta, 0)); }
-    static __device__ __forceinline__ S warp_min(S s) { return __reduce_min_sync(0xffffffffu, s); }
-    __device__ __forceinline__ bool beats(S s, K bound) const { return (int)s < bound; }
-    __device__ __forceinline__ int job_score(S s) const { return (int)s; }
-};
 
 // Score of one instance, binary64, every operation rounded on its own (the sums of whole
 // numbers below 2^53 are exact, so adding the two token counts first changes nothing).
@@ -367,166 +400,219 @@ __device__ __forceinline__ double summary_score(unsigned int tokens, unsigned in
     return __dadd_rn((double)tokens + pd, __dmul_rn(beta, over));
 }
 
-template <> struct Scores<false> {
-    typedef double S;
-    typedef float K;
-    static __device__ __forceinline__ S none() { return CUDART_INF; }
-    static __device__ __forceinline__ K no_a() { return CUDART_INF_F; }
-    static __device__ __forceinline__ K no_b() { return CUDART_INF_F; }
-    static __device__ __forceinline__ K lowest() { return -CUDART_INF_F; }
-    double theta, beta, slack;
-    int code_base;
-    __device__ __forceinline__ void start(double theta_d, double beta_d, unsigned long long, int mean) {
+// ---- Scores.  The keys are even 32-bit whole numbers: a = token count, b = token count + beta * (top - theta), in units of
+// one half (WHOLE) or less; an arrival of P tokens scores max(a, b + beta * P) plus its own P + D, which is left out.
+//   WHOLE: beta and theta are whole numbers and every possible score is below 2^29: each binary64 operation of the score
+//   is exact and the keys give the same number.
+//   Otherwise the keys are the same real numbers times 2^shift, rounded down, doubled, and cut at RS_CUT: for rows that are
+//   neither far nor pending half the key value lies within 4 of 2^shift times the score (two roundings down of less than one
+//   each, and those of binary64, below 2^-10 in these units), so a row whose key value is more than 8 above the smallest one
+//   does not have the smallest score; what is left is compared in binary64, each operation rounded on its own.
+// Odd keys belong to rows whose keys are only lower bounds (one less than the bound).
+constexpr int RS_CUT = 1 << 29, RS_ABSENT = 0x60000000, RS_LOWEST = -(1 << 30), RS_TOP_KEY = 0x3ffffffe;
+template <bool WHOLE> struct Scores {
+    static constexpr int SLACK = WHOLE ? 0 : 8;
+    double theta, beta, unit;
+    int theta_i, beta_i, shift, code_base;
+    __device__ __forceinline__ void start(double theta_d, double beta_d, unsigned long long peak_bound, unsigned long long max_pd,
+                                          unsigned long long typical_tokens, int mean) {
         theta = theta_d; beta = beta_d;
-        // The bounds are real numbers taken with roundings in binary64 before they are rounded down: each of at most eight
-        // operations is off by 2^-53 of values below 2^33 * (1 + beta) + beta * theta; sixteen times that.
-        slack = (8589934592.0 * (1.0 + beta) + beta * theta) * (128.0 * 1.1102230246251565e-16);
-        code_base = __float_as_int(fmaxf((float)mean * (1.0f / 32.0f), 1.0f)) >> 21;
+        beta_i = theta_i = shift = 0;
+        unit = 1.0;
+        if (WHOLE) {
+            beta_i = (int)beta_d;
+            // a threshold above every peak of the batch is as good as any other: the penalty is never paid
+            theta_i = theta_d > (double)peak_bound ? (int)(peak_bound + 1) : (int)theta_d;
+        } else {
+            // seven binary digits, fewer for long requests or many tokens
+            shift = 7;
+            while (shift > 0 && ((double)max_pd * (1.0 + beta) * (double)(2 << shift) > 16777216.0 ||
+                                 (typical_tokens << shift) > (unsigned long long)(RS_CUT / 8)))
+                --shift;
+            unit = (double)(1 << shift);
+        }
+        code_base = __float_as_int(fmaxf((float)mean * (1.0f / 32.0f) * (float)beta * (float)(2.0 * unit), 1.0f)) >> 21;
     }
-    __device__ __forceinline__ unsigned int key(unsigned int, unsigned int t) const { return t; }
-    static __device__ __forceinline__ uint2 absent() { return make_uint2(0xffffffffu, 0u); }   // (masked by the row number)
+    __device__ __forceinline__ int key_a(unsigned int tokens) const {
+        return WHOLE ? 2 * (int)tokens : (int)min((unsigned long long)tokens << (shift + 1), (unsigned long long)RS_CUT);
+    }
+    __device__ __forceinline__ int key_b(unsigned int tokens, unsigned int t) const {
+        if (WHOLE) return 2 * ((int)tokens + beta_i * ((int)t - theta_i));
+        return 2 * min(max(__double2int_rd(((double)tokens + beta * ((double)t - theta)) * unit), RS_LOWEST / 2), RS_CUT / 2);
+    }
+    __device__ __forceinline__ int key_p(int P) const {      // what a prompt adds to b
+        if (WHOLE) return (int)min(2ll * beta_i * P, (long long)RS_TOP_KEY);
+        return 2 * min(__double2int_rd(beta * (double)P * unit), RS_CUT / 2);
+    }
+    __device__ __forceinline__ int key_pd(int P, int D) const {
+        return WHOLE ? 2 * (P + D) : (int)min((long long)(P + D) << (shift + 1), (long long)RS_CUT);
+    }
+    // whether the keys of 32 such arrivals in a row stay below their cut
+    __device__ __forceinline__ bool usual(int kp, int kpd) const { return WHOLE || kp + kpd <= 16777216; }
+    __device__ __forceinline__ unsigned int tokens_of(const Rows& rows, int i) const { return WHOLE ? (unsigned int)rows.rec[i].x >> 1 : rows.tok[i]; }
+    // Codes of what a prompt adds, and of what a row lacks to pay a penalty: monotone, so different codes decide which is
+    // larger.  Four per octave.  0 (rows): pays for every prompt.
     __device__ __forceinline__ int code(float v) const { return min(max((__float_as_int(v) >> 21) - code_base + 1, 1), 31); }
-    __device__ __forceinline__ int prompt_code(int p) const { return code((float)p); }
-    __device__ __forceinline__ int row_code(uint2 r) const {
-        const double z = theta - (double)r.y;
-        return z < 0.0 ? 0 : code(__double2float_rn(z));
+    __device__ __forceinline__ int row_code(int2 r) const {
+        const int z = r.x - r.y;
+        return z < 0 ? 0 : code((float)z);
     }
-    static __device__ __forceinline__ K row_a(uint2 r) { return __uint2float_rd(r.x); }
-    __device__ __forceinline__ K row_b(uint2 r) const { return __double2float_rd((double)r.x + beta * ((double)r.y - theta)); }
-    __device__ __forceinline__ K probe(int p) const { return __double2float_rd(beta * (double)p); }
-    static __device__ __forceinline__ K plus(K b, K bp) { return __fadd_rd(b, bp); }
-    static __device__ __forceinline__ unsigned int order(K v) {
-        const unsigned int x = __float_as_uint(v);
-        return x ^ ((unsigned int)((int)x >> 31) | 0x80000000u);
+    // the score (without P + D where WHOLE) for a given peak
+    typedef typename std::conditional<WHOLE, unsigned int, double>::type S;
+    static __device__ __forceinline__ S none() { return WHOLE ? (S)0xffffffffu : (S)CUDART_INF; }
+    __device__ __forceinline__ S of_peak(unsigned int tokens, unsigned int peak, int P, int D) const {
+        if constexpr (WHOLE) return tokens + (unsigned int)(beta_i * max((int)peak - theta_i, 0));
+        else return summary_score(tokens, peak, (double)P + (double)D, theta, beta);
     }
-    static __device__ __forceinline__ K unorder(unsigned int x) { return __uint_as_float(x ^ ((x >> 31) ? 0x80000000u : 0xffffffffu)); }
-    static __device__ __forceinline__ int bits(K v) { return __float_as_int(v); }
-    static __device__ __forceinline__ K from_bits(int v) { return __int_as_float(v); }
-    static __device__ __forceinline__ K from_margin(int m) { return (float)m; }
-    int P;
-    double pd;
-    float bp;
-    __device__ __forceinline__ void arrival(int4 it) { P = it.x; pd = (double)it.x + (double)it.y; bp = __int_as_float(it.w); }
-    __device__ __forceinline__ K arrival_bp() const { return bp; }
-    __device__ __forceinline__ S value(uint2 r) const { return summary_score(r.x, r.y + (unsigned int)P, pd, theta, beta); }
-    __device__ __forceinline__ uint2 with_arrival(uint2 r, bool covers) const {
-        return make_uint2(r.x + (unsigned int)pd, r.y + (covers ? (unsigned int)P : 0u));
-    }
-    __device__ __forceinline__ bool no_penalty(unsigned int top) const { return !((double)(top + (unsigned int)P) > theta); }
-    __device__ __forceinline__ S of_top(unsigned int tokens, unsigned int top) const { return summary_score(tokens, top + (unsigned int)P, pd, theta, beta); }
-    __device__ __forceinline__ S of_peak(unsigned int tokens, unsigned int peak) const { return summary_score(tokens, peak, pd, theta, beta); }
+    __device__ __forceinline__ bool no_penalty(unsigned int top, int P) const { return !((double)(top + (unsigned int)P) > theta); }
     static __device__ __forceinline__ S warp_min(S s) {   // scores are >= 0: ordered by their bits
-        const unsigned int hi = (unsigned int)__double2hiint(s), lo = (unsigned int)__double2loint(s);
-        const unsigned int mh = __reduce_min_sync(0xffffffffu, hi);
-        const unsigned int ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : 0xffffffffu);
-        return __hiloint2double((int)mh, (int)ml);
+        if constexpr (WHOLE) return __reduce_min_sync(FULL_MASK, s);
+        else {
+            const unsigned int hi = (unsigned int)__double2hiint(s), lo = (unsigned int)__double2loint(s);
+            const unsigned int mh = __reduce_min_sync(FULL_MASK, hi);
+            const unsigned int ml = __reduce_min_sync(FULL_MASK, hi == mh ? lo : 0xffffffffu);
+            return __hiloint2double((int)mh, (int)ml);
+        }
     }
-    __device__ __forceinline__ bool beats(S s, K bound) const { return __double2float_ru(s - pd + slack) < bound; }
-    __device__ __forceinline__ int job_score(S) const { return 0; }
+};
+__device__ __forceinline__ unsigned int ordered(int v) { return (unsigned int)v ^ 0x80000000u; }
+__device__ __forceinline__ int unordered(unsigned int v) { return (int)(v ^ 0x80000000u); }
+
+// ---- folding warps
+template <bool ADMIT, bool WHOLE>
+struct Folder {
+    const RouteSumArgs& a;
+    RsShared& sh;
+    const Rows& rows;
+    const Scores<WHOLE>& sc;
+
+    __device__ __forceinline__ void store_numbers(int w, const RowNumbers& n) {
+        a.near[(size_t)w * 32 + (threadIdx.x & 31)] = make_uint2(n.near0, n.near1);
+        a.far[(size_t)w * 32 + (threadIdx.x & 31)] = n.far;
+    }
+    // Brings the map's row up to date with the requests of the batch below `upto` whose ramps it lacks.
+    __device__ __forceinline__ bool catch_up(int w, unsigned int upto) {
+        const int lane = threadIdx.x & 31, H = a.H;
+        if (lane == 0) atomicMax(&sh.flush, upto);
+        if (!rs_wait(sh, [&] { return (int)(ld_acquire(&sh.written) - upto) >= 0; })) return false;
+        const long long n0 = sh.n0;
+        int64_t* row = a.curves + (size_t)w * H;
+        for (unsigned int base = 0; base < upto; base += 32) {
+            const unsigned int k = base + lane;
+            const bool mine = k < upto && a.instance[n0 + k] == w && a.applied[k] == 0;
+            if (mine) a.applied[k] = 1;
+            int P = 0, D = 0;
+            if (mine) { P = a.prompt[n0 + k]; D = a.predicted[n0 + k]; }
+            for (unsigned int todo = __ballot_sync(FULL_MASK, mine); todo; todo &= todo - 1) {
+                const int src = __ffs(todo) - 1;
+                const int p = __shfl_sync(FULL_MASK, P, src), d = __shfl_sync(FULL_MASK, D, src);
+                for (int j = lane; j < (d < H ? d : H); j += 32) row[j] += p + j;
+            }
+        }
+        __syncwarp();
+        return true;
+    }
+    // Decision e: its row's new numbers.
+    __device__ __forceinline__ bool fold(unsigned int e) {
+        const int lane = threadIdx.x & 31, H = a.H;
+        const uint2 job = sh.jobs[e % RS_ITEMS];
+        const int2 pd = sh.raw[e % RS_ITEMS];
+        const int w = (int)(job.x & ~RS_GIVEN), P = pd.x, D = pd.y, Dc = D < H ? D : H;
+        const unsigned int state = rows.state[w], old_top = rows.top[w];
+        const unsigned int tokens = sc.tokens_of(rows, w);
+        if (lane == 0)
+            sh.score[e % RS_ITEMS] = summary_score(tokens, (job.x & RS_GIVEN) ? job.y : old_top + (unsigned int)P, (double)P + (double)D, a.theta, a.beta);
+        RowNumbers n;
+        bool full = ADMIT || (state & RS_FULL) != 0, deferred = !ADMIT && (state & RS_DEFERRED) != 0;
+        if (!full) {
+            const uint2 q = a.near[(size_t)w * 32 + lane];
+            n.near0 = q.x; n.near1 = q.y;
+            n.far = a.far[(size_t)w * 32 + lane];
+            const int j = 2 * lane, steps = far_chunks(H) * RS_NEAR, lo = RS_NEAR + lane * steps;
+            if (j < Dc) n.near0 += (unsigned int)(P + j);
+            if (j + 1 < Dc) n.near1 += (unsigned int)(P + j + 1);
+            if (lo < Dc) n.far += (unsigned int)(P + min(Dc, lo + steps) - 1);
+            store_numbers(w, n);
+            const unsigned int t = max(j < H ? n.near0 + (unsigned int)j : 0u, j + 1 < H ? n.near1 + (unsigned int)(j + 1) : 0u);
+            n.top = __reduce_max_sync(FULL_MASK, t);
+            n.jtop = __reduce_min_sync(FULL_MASK, t == n.top ? (unsigned int)(j + 1 < H ? j + 1 : j) : 0xffffffffu);
+            full = __any_sync(FULL_MASK, n.far > n.top);
+            if (!full) deferred = true;
+        }
+        if (full) {
+            if (deferred && !catch_up(w, e)) return false;
+            deferred = false;
+            n = row_pass<true, true, ADMIT, false>(a.curves + (size_t)w * H, H, P, Dc, a.hot);
+            if (!ADMIT) {
+                store_numbers(w, n);
+                if (lane == 0) a.applied[e] = 1;
+                full = n.jtop >= (unsigned int)RS_NEAR;
+            }
+        }
+        const bool far = n.jtop >= (unsigned int)RS_LIMIT;
+        unsigned int key_top = n.top, key_step = n.jtop;
+        if (far) key_top = first_top(n.near0, n.near1, H, key_step);
+        __syncwarp();   // every lane's cells before the row is handed on
+        if (lane == 0) {
+            const bool not_over = ADMIT && !((double)n.above > a.many);
+            if (key_step > ld_volatile(&sh.jmax)) atomicMax(&sh.jmax, key_step);
+            const unsigned int now = tokens + (unsigned int)P + (unsigned int)D;
+            rows.top[w] = n.top;
+            if (!WHOLE) rows.tok[w] = now;
+            rows.rec[w] = make_int2(sc.key_a(now), sc.key_b(now, key_top));
+            rows.state[w] = n.jtop | (far ? RS_FAR : 0u) | (full ? RS_FULL : 0u) | (deferred ? RS_DEFERRED : 0u) | (not_over ? RS_NOT_OVER : 0u);
+            if (ADMIT && (state & RS_NOT_OVER) && !not_over) atomicSub(&sh.not_over, 1u);
+            st_release(&rows.pending[w], 0u);
+        }
+        return true;
+    }
+    // The peak row w would have with the arrival (P, Dc); the row is not pending.
+    __device__ __forceinline__ bool scan(int w, int P, int Dc, unsigned int decided, unsigned int& peak) {
+        const int lane = threadIdx.x & 31, H = a.H;
+        if (!ADMIT && (rows.state[w] & RS_DEFERRED)) {
+            // the first cells, and what bounds the others: enough when Dc ends among the first and none of the others can be larger
+            const uint2 q = a.near[(size_t)w * 32 + lane];
+            const int j = 2 * lane, lo = RS_NEAR + lane * far_chunks(H) * RS_NEAR;
+            const unsigned int u = a.far[(size_t)w * 32 + lane];
+            peak = __reduce_max_sync(FULL_MASK, max(q.x + (j < Dc ? (unsigned int)(P + j) : 0u), q.y + (j + 1 < Dc ? (unsigned int)(P + j + 1) : 0u)));
+            const bool others = Dc > RS_NEAR || u > peak + (unsigned int)(u ? lo : 0);
+            if (!__any_sync(FULL_MASK, others)) return true;
+            if (!catch_up(w, decided)) return false;
+            const RowNumbers n = row_pass<false, false, false, false>(a.curves + (size_t)w * H, H, 0, 0, 0);
+            store_numbers(w, n);
+            __syncwarp();
+            if (lane == 0) rows.state[w] &= ~RS_DEFERRED;     // (its numbers stay what they are: they were exact)
+        }
+        peak = row_pass<true, false, false, false>(a.curves + (size_t)w * H, H, P, Dc, 0).peak;
+        return true;
+    }
 };
 
-// ---- folding warps.  A warp adds a decided arrival to its row and takes the row's new numbers in the same pass, or takes
-// the peak the row would have with the arrival.  16-byte accesses when H is even (a lane holds two neighbouring cells, the
-// warp 512 contiguous bytes), eight in flight per lane.  Other warps of this block wrote the row before: the loads
-// come after the acquire of the job, and no other block touches the maps meanwhile.
-template <bool VEC, bool ADMIT, bool FOLD>
-__device__ __forceinline__ void rs_row_pass(const RouteSumArgs& a, int64_t* row, int P, int Dc, unsigned int& top, unsigned int& jtop,
-                                            unsigned int& c0, unsigned int& peak, int& above) {
-    constexpr int BATCH = 8;                        // loads in flight
-    constexpr int PER = VEC ? 2 : 1;                // cells per load
-    constexpr int STEP = 32 * PER;                  // cells per warp access
-    const int lane = threadIdx.x & 31, H = a.H;
-    const int hot_all = (ADMIT && a.hot < 0) ? 1 : 0;   // the overload level against 32-bit cells
-    const unsigned int hot = a.hot < 0 ? 0u : (a.hot > 0xffffffffLL ? 0xffffffffu : (unsigned int)a.hot);
-    top = jtop = c0 = peak = 0;
-    above = 0;
-    #pragma unroll 1
-    for (int base = 0; base < H; base += BATCH * STEP) {
-        unsigned int c[BATCH * PER];
-        #pragma unroll
-        for (int u = 0; u < BATCH; ++u) {
-            const int j = base + u * STEP + lane * PER;
-            if (VEC) {
-                longlong2 v = make_longlong2(0, 0);
-                if (j < H) v = *reinterpret_cast<const longlong2*>(row + j);
-                c[2 * u] = (unsigned int)v.x; c[2 * u + 1] = (unsigned int)v.y;
-            } else {
-                c[u] = j < H ? (unsigned int)row[j] : 0u;
-            }
-        }
-        #pragma unroll
-        for (int u = 0; u < BATCH; ++u) {
-            const int j = base + u * STEP + lane * PER;
-            if (j < Dc) {
-                #pragma unroll
-                for (int e = 0; e < PER; ++e)
-                    if (j + e < Dc) c[PER * u + e] += (unsigned int)(P + j + e);
-                if (FOLD) {   // (a pair whose second cell lies past the ramp writes that cell back unchanged)
-                    if (VEC) *reinterpret_cast<longlong2*>(row + j) = make_longlong2((long long)c[2 * u], (long long)c[2 * u + 1]);
-                    else row[j] = (long long)c[u];
-                }
-            }
-            if (j < H) {
-                if (FOLD) {
-                    unsigned int t = c[PER * u] + (unsigned int)j;
-                    if (VEC) t = max(t, c[2 * u + 1] + (unsigned int)(j + 1));
-                    if (ADMIT) {
-                        #pragma unroll
-                        for (int e = 0; e < PER; ++e) above += hot_all | (c[PER * u + e] > hot);
-                    }
-                    if (t > top) { top = t; jtop = (unsigned int)(j + PER - 1); }
-                } else {
-                    peak = max(peak, c[PER * u]);
-                    if (VEC) peak = max(peak, c[2 * u + 1]);
-                }
-            }
-        }
-        if (base == 0) c0 = c[0];
-    }
-}
-
-template <bool VEC, bool ADMIT, bool WHOLE, bool LISTS>
-__device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int me, int near_steps) {
-    const int lane = threadIdx.x & 31, H = a.H;
+template <int FOLD_WARPS, bool ADMIT, bool WHOLE, bool LISTS>
+__device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int me) {
+    const int lane = threadIdx.x & 31;
+    Folder<ADMIT, WHOLE> f{a, sh, rows, sc};
     unsigned int scans = 0;
-    unsigned int top, jtop, c0, peak;
-    int above;
     for (unsigned int n = me;;) {
         uint4 ctl;
         if (!rs_wait(sh, [&] {
                 ctl = ld_volatile4(&sh.ctl);
                 return (int)(ctl.x - n) > 0 || ctl.y != scans || ctl.z != 0;
-            }, LISTS ? 40 : 0))    // (the list warps need the issue slots)
+            }, LISTS ? 20 : 0))    // (the list warps need the issue slots)
             return;
         acquire_cta();
         ctl = ld_volatile4(&sh.ctl);
-        if (__any_sync(0xffffffffu, (int)(ctl.x - n) > 0)) {
-            const int4 job = sh.jobs[n % RS_ITEMS];
-            const int w = job.x, P = job.y, Dc = job.z < H ? job.z : H;
-            rs_row_pass<VEC, ADMIT, true>(a, a.curves + (size_t)w * H, P, Dc, top, jtop, c0, peak, above);
-            const unsigned int t = __reduce_max_sync(0xffffffffu, top);
-            jtop = __reduce_min_sync(0xffffffffu, top == t ? jtop : 0xffffffffu);
-            if (ADMIT) above = __reduce_add_sync(0xffffffffu, above);
-            __syncwarp();   // every lane's cells before the row is handed on
-            if (lane == 0) {
-                const bool far = jtop >= (unsigned int)near_steps;
-                const bool not_over = ADMIT && !((double)above > a.many);
-                if (!far && jtop > ld_volatile(&sh.jmax)) atomicMax(&sh.jmax, jtop);
-                rows.top[w] = t;
-                rows.c0[w] = c0;
-                rows.rec[w].y = sc.key(rows.rec[w].x, far ? c0 : t);
-                if (not_over) atomicAdd(&sh.not_over, 1u);
-                st_release(&rows.flags[w], jtop | (far ? RS_FAR : 0u) | (not_over ? RS_NOT_OVER : 0u));
-                st_release(&sh.done[me], n + RS_FOLD_WARPS);
-            }
-            n += RS_FOLD_WARPS;
+        if (__any_sync(FULL_MASK, (int)(ctl.x - n) > 0)) {
+            if (!f.fold(n)) return;
+            n += FOLD_WARPS;
+            if (lane == 0) st_release(&sh.done[me], n);
             __syncwarp();
-        } else if (__any_sync(0xffffffffu, ctl.y != scans)) {
+        } else if (__any_sync(FULL_MASK, ctl.y != scans)) {
             scans = ctl.y;
             const int count = sh.scan_n;
-            for (int x = me; x < count; x += RS_FOLD_WARPS) {
-                rs_row_pass<VEC, ADMIT, false>(a, a.curves + (size_t)sh.scan_row[x] * H, sh.scan_P, sh.scan_Dc, top, jtop, c0, peak, above);
-                peak = __reduce_max_sync(0xffffffffu, peak);
+            for (int x = me; x < count; x += FOLD_WARPS) {
+                unsigned int peak = 0;
+                if (!f.scan(sh.scan_row[x], sh.scan_P, sh.scan_Dc, ctl.x, peak)) return;
                 if (lane == 0) sh.peak[x] = peak;
             }
             __syncwarp();
@@ -537,8 +623,8 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
     }
 }
 
-// ---- io warp: arrivals ahead of the decisions, results behind them
-template <bool ADMIT, bool WHOLE>
+// ---- io warp: arrivals ahead of the decisions, results behind the folds
+template <int FOLD_WARPS, bool ADMIT, bool WHOLE>
 __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, const Scores<WHOLE>& sc, long long q_head, int waiting, int items, int room) {
     const int lane = threadIdx.x & 31;
     const long long n0 = sh.n0;
@@ -566,10 +652,12 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
                 }
             }
             const bool ok = P >= 0 && D >= 1 && P <= PRE_FIELD_MAX && D <= PRE_FIELD_MAX;
-            const unsigned int vote = __ballot_sync(0xffffffffu, ok);
+            const unsigned int vote = __ballot_sync(FULL_MASK, ok);
             const unsigned int slot = entered + __popc(vote & ((1u << lane) - 1u));
             if (ok && slot < (unsigned int)room) {
-                sh.items[slot % RS_ITEMS] = make_int4(P, D, (D < a.H ? D : a.H) | (sc.prompt_code(P) << 16), Scores<WHOLE>::bits(sc.probe(P)));
+                const int kp = sc.key_p(P), kpd = sc.key_pd(P, D);
+                sh.items[slot % RS_ITEMS] = make_int4(kp, kpd - 1, sc.usual(kp, kpd) ? (D < a.H ? D : a.H) : 0, 16 * sc.code((float)kp));
+                sh.raw[slot % RS_ITEMS] = make_int2(P, D);
                 sh.item_at[slot % RS_ITEMS] = k;
             } else if (k < items) {
                 put_result(k, -1, 0.0);
@@ -582,70 +670,74 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
         }
         if (cursor >= items && lane == 0) st_release(&sh.items_end, 1u);
         const uint4 ctl = ld_volatile4(&sh.ctl);
-        const bool last = __any_sync(0xffffffffu, ctl.z != 0);
+        const bool last = __any_sync(FULL_MASK, ctl.z != 0);
         acquire_cta();
-        const unsigned int decided = __shfl_sync(0xffffffffu, ld_volatile(&sh.ctl.x), 0);   // (final when `last`)
-        while (decided - written >= 32 || (last && written != decided)) {
+        const unsigned int decided = __shfl_sync(FULL_MASK, ld_volatile(&sh.ctl.x), 0);   // (final when `last`)
+        // folded: every decision below the smallest of the folding warps' next ones
+        const unsigned int next = ld_acquire(&sh.done[lane < FOLD_WARPS ? lane : 0]);
+        const unsigned int folded = min(decided, written + __reduce_min_sync(FULL_MASK, next - written));
+        const unsigned int flush = __shfl_sync(FULL_MASK, ld_volatile(&sh.flush), 0);
+        while (folded - written >= 32 || (folded != written && (last || (int)(flush - written) > 0))) {
             const unsigned int e = written + lane;
-            if (e < decided) {
-                const int4 job = sh.jobs[e % RS_ITEMS];
-                const int w = job.x;
+            if (e < folded) {
+                const int w = (int)(sh.jobs[e % RS_ITEMS].x & ~RS_GIVEN);
+                const int2 pd = sh.raw[e % RS_ITEMS];
                 const long long at = n0 + e;
-                a.prompt[at] = job.y; a.generated[at] = 0; a.predicted[at] = job.z; a.instance[at] = w;
-                const double s = WHOLE ? (double)((unsigned int)job.w + (unsigned int)job.y + (unsigned int)job.z) : sh.score[e % RS_ITEMS];
-                put_result(sh.item_at[e % RS_ITEMS], w, s);
-                atomicAdd(reinterpret_cast<unsigned long long*>(a.queued_p + w), (unsigned long long)job.y);
-                atomicAdd(reinterpret_cast<unsigned long long*>(a.current_d + w), (unsigned long long)job.z);
+                a.prompt[at] = pd.x; a.generated[at] = 0; a.predicted[at] = pd.y; a.instance[at] = w;
+                put_result(sh.item_at[e % RS_ITEMS], w, sh.score[e % RS_ITEMS]);
+                atomicAdd(reinterpret_cast<unsigned long long*>(a.queued_p + w), (unsigned long long)pd.x);
+                atomicAdd(reinterpret_cast<unsigned long long*>(a.current_d + w), (unsigned long long)pd.y);
             }
-            written = min(written + 32u, decided);
+            written = min(written + 32u, folded);
             __syncwarp();
+            if (lane == 0) st_release(&sh.written, written);
         }
-        if (last || __any_sync(0xffffffffu, ctl.w != 0)) break;
+        if (last && written == decided) break;
+        if (__any_sync(FULL_MASK, ctl.w != 0)) break;
         __nanosleep(100);
     }
-    first_bad = __reduce_min_sync(0xffffffffu, first_bad);
-    first_full = __reduce_min_sync(0xffffffffu, first_full);
+    first_bad = __reduce_min_sync(FULL_MASK, first_bad);
+    first_full = __reduce_min_sync(FULL_MASK, first_full);
     if (lane == 0) { sh.first_bad = first_bad; sh.first_full = first_full; }
 }
 
-// ---- list warps.  A list holds the rows whose score for one of RS_PROBES prompt lengths lies within a margin of the
-// smallest score known for it; the margin follows the list's room.  The other rows are bounded by 32 buckets: bucket x
-// holds the smallest token count and the smallest b of the rows whose row_code is x.  For an arrival of code q the rows
-// of codes above q pay no penalty (score = a), those below q do (score = b + beta * P), and those of code q either
-// (score = the larger, hence at least the larger of the two smallest): four numbers per code.
+// ---- list warps.  A list holds the rows whose key value for one of RS_PROBES prompt lengths lies within a margin of the
+// smallest one known for it; the margin follows the list's room.  The other rows are bounded by 32 buckets: bucket x
+// holds the smallest a and the smallest b of the rows whose row_code is x.  For an arrival of code q the rows
+// of codes above q pay no penalty (value = a), those below q do (value = b + beta * P), and those of code q either
+// (value = the larger, hence at least the larger of the two smallest): four numbers per code.
 // The probes: shares of the mean prompt (+ ramp) of the batch, from nothing to several times it.
 __device__ __forceinline__ int rs_probe(int mean, int x) {
     const float share[RS_PROBES] = {0.0f, 0.08f, 0.17f, 0.3f, 0.5f, 0.9f, 1.5f, 2.5f};
     return (int)((float)mean * share[x]);
 }
-template <bool WHOLE>
-__device__ __forceinline__ typename Scores<WHOLE>::K rs_score_at(const Scores<WHOLE>& sc, uint2 r, typename Scores<WHOLE>::K bp) {
-    return max(Scores<WHOLE>::row_a(r), Scores<WHOLE>::plus(sc.row_b(r), bp));
-}
-template <bool WHOLE>
-__device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int I, int mean, int longest_p) {
-    typedef typename Scores<WHOLE>::K K;
-    constexpr unsigned int FULL = 0xffffffffu;
-    const int t = threadIdx.x - RS_LIST_WARP * 32, lane = threadIdx.x & 31;
+
+template <int LIST_WARPS, bool WHOLE>
+__device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int I, int mean, int longest, int t) {
+    constexpr int THREADS = 32 * LIST_WARPS, NEAR_ROOM = RS_NEAR_ROWS / LIST_WARPS;
+    constexpr int FAR_KEY = 0x7f000000, AT_ONCE = 4;      // AT_ONCE: rows a thread has on their way
+    static_assert(NEAR_ROOM >= 2 * 32 * AT_ONCE, "");
+    const int lane = threadIdx.x & 31;
     const bool leader = t < 32;
     unsigned int met = 0;
-    auto over = [&] { return __any_sync(FULL, ld_volatile(&sh.ctl.z) != 0); };
-    auto team = [&]() -> bool {   // the three warps meet (false: abandoned, or the last decision has been made)
-        met += RS_LIST_THREADS / 32;
+    auto over = [&] { return __any_sync(FULL_MASK, ld_volatile(&sh.ctl.z) != 0); };
+    auto team = [&]() -> bool {   // the list warps meet (false: abandoned, or the last decision has been made)
+        met += LIST_WARPS;
         __syncwarp();
         acquire_cta();
         if (lane == 0) atomicAdd(&sh.list_met, 1u);
         return rs_wait(sh, [&] { return (int)(ld_acquire(&sh.list_met) - met) >= 0 || ld_volatile(&sh.ctl.z) != 0; }) && !over();
     };
-    int probe_p = 0;
-    K bp[RS_PROBES];
+    int probe_key = 0;
+    int bp[RS_PROBES];
     #pragma unroll
     for (int x = 0; x < RS_PROBES; ++x) {
-        if (lane == x) probe_p = rs_probe(mean, x);
-        bp[x] = sc.probe(rs_probe(mean, x));
+        bp[x] = sc.key_p(rs_probe(mean, x));
+        if (lane == x) probe_key = bp[x];
     }
-    const K longest = sc.probe(longest_p);     // what the longest prompt of the batch adds
-    int margin = max(mean / 16, 8);
+    int margin = max(sc.key_a((unsigned int)mean) / 16, 8);
+    const int least_margin = max(sc.key_a(1u), 1);
+    unsigned short* near = sh.near_row + (t >> 5) * NEAR_ROOM;
     for (unsigned int n = 1;; ++n) {
         bool go = false;
         if (!rs_wait(sh, [&] {
@@ -654,342 +746,356 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
                 return go || ctl.z != 0;
             }, 20))
             return;
-        go = __any_sync(FULL, ld_acquire(&sh.lists_wanted) >= n);
-        if (!go) return;     // (all three warps: nothing is asked for after the last decision)
+        go = __any_sync(FULL_MASK, ld_acquire(&sh.lists_wanted) >= n);
+        if (!go) return;     // (nothing is asked for after the last decision)
         const int old = (n + 1) & 1, now = n & 1;
-        // the smallest score known per probe: the rows of the present list, and (kept in probe_t) the others' bound
+        // the smallest value known per probe: the rows of the present list, and (kept in probe_t) the others' bound
         if (!team()) return;
         if (n > 1) {   // (the first list: probe_t was set when the rows were loaded)
-            K least[RS_PROBES];
-            #pragma unroll
-            for (int x = 0; x < RS_PROBES; ++x) least[x] = Scores<WHOLE>::from_bits(0x7f000000);
             const int old_n = sh.list_n[old];
-            for (int x = t; x < old_n; x += RS_LIST_THREADS) {
-                const uint2 r = ld_volatile2(rows.rec + sh.list_row[old][x]);
+            if (t - lane < old_n) {
+                int least[RS_PROBES];
                 #pragma unroll
-                for (int p = 0; p < RS_PROBES; ++p) least[p] = min(least[p], rs_score_at(sc, r, bp[p]));
-            }
-            #pragma unroll
-            for (int p = 0; p < RS_PROBES; ++p) {
-                const unsigned int v = __reduce_min_sync(FULL, Scores<WHOLE>::order(least[p]));
-                if (lane == 0) atomicMin(reinterpret_cast<unsigned int*>(&sh.probe_t[p]), v);
+                for (int x = 0; x < RS_PROBES; ++x) least[x] = FAR_KEY;
+                for (int x = t; x < old_n; x += THREADS) {
+                    const int2 r = ld_volatile2(rows.rec + sh.list_row[old][x]);
+                    #pragma unroll
+                    for (int p = 0; p < RS_PROBES; ++p) least[p] = min(least[p], max(r.x, r.y + bp[p]));
+                }
+                #pragma unroll
+                for (int p = 0; p < RS_PROBES; ++p) {
+                    const int v = __reduce_min_sync(FULL_MASK, least[p]);
+                    if (lane == 0) atomicMin(&sh.probe_t[p], ordered(v));
+                }
             }
         }
         for (int tries = 0;; ++tries) {
             if (leader) { sh.bucket_a[lane] = 0xffffffffu; sh.bucket_b[lane] = 0xffffffffu; }
             if (t == 0) sh.list_count = 0;
             if (!team()) return;
-            // A row is in the list if for some probe its token count is at most limit_a and its b at most limit_b.
+            // A row is in the list if for some probe its a is at most limit_a and its b at most limit_b.
             // Rows beyond far_a or far_b are out of reach of this list: the two limits bound them, and they are dropped by
             // two comparisons.
-            K limit_a[RS_PROBES], limit_b[RS_PROBES];
-            K far_a = Scores<WHOLE>::lowest();
+            int limit_a[RS_PROBES], limit_b[RS_PROBES];
+            int far_a = RS_LOWEST;
             #pragma unroll
             for (int p = 0; p < RS_PROBES; ++p) {
-                limit_a[p] = tries < 8 ? Scores<WHOLE>::unorder((unsigned int)sh.probe_t[p]) + Scores<WHOLE>::from_margin(margin)
-                                       : Scores<WHOLE>::lowest();   // (an empty list is a list, too)
+                limit_a[p] = tries < 8 ? unordered(sh.probe_t[p]) + margin : RS_LOWEST;   // (an empty list is a list, too)
                 limit_b[p] = limit_a[p] - bp[p];
                 far_a = max(far_a, limit_a[p]);
             }
-            const K far_b = limit_a[0];
-            far_a = min(Scores<WHOLE>::plus(far_a, longest), Scores<WHOLE>::no_a());
-            K hot_b = Scores<WHOLE>::from_bits(0x7f000000), cold_a = hot_b;
-            constexpr int AT_ONCE = 4;      // rows a thread has on their way
-            unsigned short* near = sh.near_row[t >> 5];
+            const int far_b = limit_a[0];
+            far_a = (int)min((long long)far_a + longest, (long long)RS_ABSENT);
+            int hot_b = FAR_KEY, cold_a = FAR_KEY;
             int n_near = 0;
             auto sort_near = [&]() {        // the rows that were not dropped: into the list or into a bucket
                 __syncwarp();
                 for (int x = lane; x - lane < n_near; x += 32) {
                     const bool in = x < n_near;
                     const int i = in ? near[x] : 0;
-                    const uint2 r = ld_volatile2(rows.rec + i);
-                    const K ra = Scores<WHOLE>::row_a(r), rb = sc.row_b(r);
+                    const int2 r = ld_volatile2(rows.rec + i);
                     bool take = false;
                     #pragma unroll
-                    for (int p = 0; p < RS_PROBES; ++p) take |= ra <= limit_a[p] && rb <= limit_b[p];
+                    for (int p = 0; p < RS_PROBES; ++p) take |= r.x <= limit_a[p] && r.y <= limit_b[p];
                     take &= in;
-                    const unsigned int vote = __ballot_sync(FULL, take);
+                    const unsigned int vote = __ballot_sync(FULL_MASK, take);
                     if (vote) {
                         int at = 0;
                         if (lane == 0) at = atomicAdd(&sh.list_count, __popc(vote));
-                        at = __shfl_sync(FULL, at, 0) + __popc(vote & ((1u << lane) - 1u));
+                        at = __shfl_sync(FULL_MASK, at, 0) + __popc(vote & ((1u << lane) - 1u));
                         if (take && at < RS_LIST_ROWS) sh.list_row[now][at] = i;
                     }
                     if (in && !take) {
                         const int c = sc.row_code(r);
-                        if (c == 0) hot_b = min(hot_b, rb);
-                        else if (c == 31) cold_a = min(cold_a, ra);
+                        if (c == 0) hot_b = min(hot_b, r.y);
+                        else if (c == 31) cold_a = min(cold_a, r.x);
                         else {
-                            atomicMin(&sh.bucket_a[c], Scores<WHOLE>::order(ra));
-                            atomicMin(&sh.bucket_b[c], Scores<WHOLE>::order(rb));
+                            atomicMin(&sh.bucket_a[c], ordered(r.x));
+                            atomicMin(&sh.bucket_b[c], ordered(r.y));
                         }
                     }
                 }
                 __syncwarp();
                 n_near = 0;
             };
-            for (int base = 0; base < I; base += AT_ONCE * RS_LIST_THREADS) {
+            for (int base = 0; base < I; base += AT_ONCE * THREADS) {
                 if (over()) return;
-                uint2 r[AT_ONCE];
+                int2 r[AT_ONCE];
                 #pragma unroll
                 for (int u = 0; u < AT_ONCE; ++u) {
-                    const int i = base + u * RS_LIST_THREADS + t;
+                    const int i = base + u * THREADS + t;
                     if (i < I) r[u] = ld_volatile2(rows.rec + i);
                 }
                 #pragma unroll
                 for (int u = 0; u < AT_ONCE; ++u) {
-                    const int i = base + u * RS_LIST_THREADS + t;
-                    const bool keep = i < I && !(sc.row_b(r[u]) > far_b) && !(Scores<WHOLE>::row_a(r[u]) > far_a);
-                    const unsigned int vote = __ballot_sync(FULL, keep);
+                    const int i = base + u * THREADS + t;
+                    const bool keep = i < I && r[u].y <= far_b && r[u].x <= far_a;
+                    const unsigned int vote = __ballot_sync(FULL_MASK, keep);
                     if (keep) near[n_near + __popc(vote & ((1u << lane) - 1u))] = (unsigned short)i;
                     n_near += __popc(vote);
                 }
-                if (n_near > RS_NEAR_ROWS - AT_ONCE * 32) sort_near();
+                if (n_near > NEAR_ROOM - AT_ONCE * 32) sort_near();
             }
             sort_near();
-            const unsigned int hb = __reduce_min_sync(FULL, Scores<WHOLE>::order(hot_b));
-            const unsigned int ca = __reduce_min_sync(FULL, Scores<WHOLE>::order(cold_a));
-            if (lane == 0) { atomicMin(&sh.bucket_b[0], hb); atomicMin(&sh.bucket_a[31], ca); }
+            const int hb = __reduce_min_sync(FULL_MASK, hot_b), ca = __reduce_min_sync(FULL_MASK, cold_a);
+            if (lane == 0) { atomicMin(&sh.bucket_b[0], ordered(hb)); atomicMin(&sh.bucket_a[31], ordered(ca)); }
             if (!team()) return;
             const int count = sh.list_count;
-            if (count > RS_LIST_ROWS) { margin = max(margin / 2, 1); if (tries > 4) margin = 0; if (!team()) return; continue; }
+            if (count > RS_LIST_ROWS) { margin = max(margin / 2, least_margin); if (tries > 4) margin = 0; if (!team()) return; continue; }
             if (leader) {
-                // (a key that no row has set is out of reach; rows of code 31 count as paying nothing only for smaller codes,
-                // so their b joins in with the bound "at least the token count")
-                const unsigned int ua = sh.bucket_a[lane], ub = sh.bucket_b[lane];
-                const K ka = ua == 0xffffffffu ? Scores<WHOLE>::no_a() : min(Scores<WHOLE>::unorder(ua), Scores<WHOLE>::no_a());
-                const K kb = ub == 0xffffffffu ? Scores<WHOLE>::no_b() : min(Scores<WHOLE>::unorder(ub), Scores<WHOLE>::no_b());
-                K above_a = min(ka, far_a), below_b = min(kb, far_b);
+                // (a key that no row has set is out of reach; rows of code 31 count by their a alone, no b is kept for them)
+                const int ka = unordered(min(sh.bucket_a[lane], ordered(RS_ABSENT)));
+                const int kb = unordered(min(sh.bucket_b[lane], ordered(RS_TOP_KEY)));     // (room for beta * P on top)
+                int above_a = min(ka, far_a), below_b = min(kb, far_b);
                 #pragma unroll
                 for (int off = 1; off < 32; off <<= 1) {
-                    const K x = Scores<WHOLE>::from_bits(__shfl_down_sync(FULL, Scores<WHOLE>::bits(above_a), off));
-                    const K y = Scores<WHOLE>::from_bits(__shfl_up_sync(FULL, Scores<WHOLE>::bits(below_b), off));
+                    const int x = __shfl_down_sync(FULL_MASK, above_a, off), y = __shfl_up_sync(FULL_MASK, below_b, off);
                     if (lane + off < 32) above_a = min(above_a, x);
                     if (lane >= off) below_b = min(below_b, y);
                 }
-                above_a = Scores<WHOLE>::from_bits(__shfl_down_sync(FULL, Scores<WHOLE>::bits(above_a), 1));
-                below_b = Scores<WHOLE>::from_bits(__shfl_up_sync(FULL, Scores<WHOLE>::bits(below_b), 1));
+                above_a = __shfl_down_sync(FULL_MASK, above_a, 1);
+                below_b = __shfl_up_sync(FULL_MASK, below_b, 1);
                 if (lane == 31) above_a = far_a;
                 if (lane == 0) below_b = far_b;
-                // code 31: its own rows by their token count alone (no b is kept for them)
-                sh.table[now][lane] = make_int4(Scores<WHOLE>::bits(above_a), Scores<WHOLE>::bits(below_b), Scores<WHOLE>::bits(ka),
-                                                Scores<WHOLE>::bits(lane == 31 ? Scores<WHOLE>::lowest() : kb));
+                sh.table[now][lane] = make_int4(above_a, below_b, ka, lane == 31 ? RS_LOWEST : kb);
                 __syncwarp();
                 if (lane < RS_PROBES) {
-                    const int4 e = sh.table[now][sc.prompt_code(probe_p)];
-                    const K x = sc.probe(probe_p);
-                    const K b = min(min(Scores<WHOLE>::from_bits(e.x), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(e.y), x)),
-                                    max(Scores<WHOLE>::from_bits(e.z), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(e.w), x)));
-                    sh.probe_t[lane] = (int)Scores<WHOLE>::order(b);
+                    const int4 e = sh.table[now][sc.code((float)probe_key)];
+                    sh.probe_t[lane] = ordered(min(min(e.x, e.y + probe_key), max(e.z, e.w + probe_key)));
                 }
                 if (lane == 0) sh.list_n[now] = count;
                 __syncwarp();
                 if (lane == 0) st_release(&sh.lists_ready, n);
             }
-            if (count < RS_LIST_ROWS * 3 / 5) margin = min(margin + margin / 2 + 1, 1 << 24);
+            if (count < RS_LIST_ROWS * 3 / 5) margin = min(margin + margin / 2 + 1, 1 << 27);
             break;
         }
     }
 }
 
 // ---- deciding warp.  KS: rows per lane.  LISTS: they are a list's, else all rows.
-// What bounds it: the latency of one chain of dependent instructions per arrival (two warp reductions, some ten integer
-// operations) and the fetching of its instructions, so the usual way through the loop is one straight piece of code with a
-// single branch to everything unusual.
-template <int KS, bool LISTS, bool ADMIT, bool WHOLE>
-__device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, Scores<WHOLE> sc) {
+// What bounds it: the latency of one chain of dependent instructions per arrival (two warp reductions and some ten integer
+// operations) and the number of its instructions, so the usual way through the loop has a single branch, to everything
+// unusual, and what need not be in the chain (scores, token counts, the tables) is done by the folding warps.
+template <int KS, bool LISTS, int FOLD_WARPS, bool ADMIT, bool WHOLE>
+__device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc) {
     typedef typename Scores<WHOLE>::S S;
-    typedef typename Scores<WHOLE>::K K;
-    constexpr unsigned int FULL = 0xffffffffu;
-    // decisions between two looks at items, room in the ring of jobs and (all rows held) pending rows
+    constexpr int SLACK = Scores<WHOLE>::SLACK;
+    // decisions between two looks at items and at the rows that were pending
     constexpr unsigned int CHUNK = LISTS ? 32 : 4 * KS;
     // decisions made known to the folding warps at once (few rows: soon)
     constexpr unsigned int PUBLISH = LISTS ? 4 : (KS >= 4 ? 2 : 1);
-    const int lane = threadIdx.x & 31, I = a.I, n_groups = (I + 31) / 32;
-    const int lane_f = lane < RS_FOLD_WARPS ? lane : 0;
-    unsigned int taken_over = 0;     // ADMIT: decisions for rows that were known not to be overloaded
+    const int lane = threadIdx.x & 31, I = a.I, H = a.H, n_groups = (I + 31) / 32;
+    const int lane_f = lane < FOLD_WARPS ? lane : 0;
     unsigned int scans = 0;
     bool lost = false;
 
-    // ---- the rows held by the lane: 2 * row + 1 if it is marked (pending when the lane last looked, or far: its key is
-    // only a lower bound), and what the row table has for it
-    unsigned int row[KS];
-    uint2 rec[KS];
-    constexpr unsigned int NO_ROW = 2u * (unsigned int)RS_NO_ROW;
-    auto load_rows = [&]() {
+    // ---- the rows held by the lane, ascending, and their keys: odd for a row that is marked (pending when the lane last
+    // looked, or far: its keys are only lower bounds)
+    int row[KS], ra[KS], rb[KS];
+    constexpr int NO_ROW = RS_NO_ROW, ODD = -1, NONE = -2;   // (ODD, NONE: of the step before, see below)
+    int jmax = 0;        // an arrival whose ramp is longer than this reaches the step of every row's b
+    auto refresh = [&]() {   // the marked rows that are not pending any more
         #pragma unroll
         for (int k = 0; k < KS; ++k) {
-            rec[k] = Scores<WHOLE>::absent();
-            if (row[k] != NO_ROW) {
-                const unsigned int i = row[k] >> 1;
-                const unsigned int f = ld_volatile(rows.flags + i);   // first: it is written last
-                rec[k] = ld_volatile2(rows.rec + i);
-                row[k] = 2 * i + ((f & (RS_PENDING | RS_FAR)) ? 1u : 0u);
+            if (ra[k] & 1) {
+                const bool pending = ld_volatile(rows.pending + row[k]) != 0;    // first: it is cleared last
+                const int2 r = ld_volatile2(rows.rec + row[k]);
+                const int far = (ld_volatile(rows.state + row[k]) & RS_FAR) ? 1 : 0;
+                if (!pending) { ra[k] = r.x - far; rb[k] = r.y - far; }
             }
         }
+        jmax = (int)ld_volatile(&sh.jmax);    // (after the rows were read)
+    };
+    auto held_pending = [&]() {
+        unsigned int m = 0;
+        #pragma unroll
+        for (int k = 0; k < KS; ++k)
+            if (row[k] != NO_ROW && ld_acquire(rows.pending + row[k])) m |= 1u << k;
+        return m;
+    };
+    auto all_folded = [&](unsigned int e) {   // every decision before e has reached its row
+        return __all_sync(FULL_MASK, (int)(ld_acquire(&sh.done[lane_f]) - e) >= 0);
+    };
+    auto publish = [&](unsigned int n) {
+        __syncwarp();
+        if (lane == 0) st_release(&sh.ctl.x, n);
     };
     unsigned int list = 0;           // the list held
+    unsigned int table = smem_u32(sh.table[0]);
     bool asked = false;
     auto ask_for_list = [&]() {
         if (!asked && lane == 0) st_release(&sh.lists_wanted, list + 1);
         asked = true;
     };
-    auto next_list = [&]() {
+    auto next_list = [&](unsigned int e) {
         ask_for_list();
         if (!rs_wait(sh, [&] { return ld_acquire(&sh.lists_ready) > list; })) { lost = true; return; }
         ++list;
         asked = false;
+        table = smem_u32(sh.table[list & 1]);
         const int n = sh.list_n[list & 1];
         #pragma unroll
-        for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < n ? 2u * (unsigned int)sh.list_row[list & 1][k * 32 + lane] : NO_ROW;
-        load_rows();
+        for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < n ? sh.list_row[list & 1][k * 32 + lane] : NO_ROW;
+        #pragma unroll
+        for (int i = 1; i < KS; ++i)
+            #pragma unroll
+            for (int k = KS - 1; k >= i; --k) {
+                const int x = min(row[k - 1], row[k]);
+                row[k] = max(row[k - 1], row[k]);
+                row[k - 1] = x;
+            }
+        #pragma unroll
+        for (int k = 0; k < KS; ++k) { ra[k] = row[k] != NO_ROW ? RS_ABSENT - 1 : RS_ABSENT; rb[k] = RS_LOWEST; }
+        if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return; }
+        refresh();
         ask_for_list();     // (a list takes about as long as one lasts)
     };
     if (LISTS) {
-        next_list();
+        next_list(0);
     } else {
         #pragma unroll
-        for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < I ? 2u * (unsigned int)(k * 32 + lane) : NO_ROW;
-    }
-    // the smallest score of the rows held, and the lane's lowest row that has it (as in `row`)
-    auto best_of_lane = [&](S& best) {
-        S v[KS];
-        #pragma unroll
         for (int k = 0; k < KS; ++k) {
-            v[k] = sc.value(rec[k]);
-            if (!WHOLE && row[k] == NO_ROW) v[k] = Scores<WHOLE>::none();
+            row[k] = k * 32 + lane < I ? k * 32 + lane : NO_ROW;
+            ra[k] = row[k] != NO_ROW ? RS_ABSENT - 1 : RS_ABSENT; rb[k] = RS_LOWEST;
         }
-        S m = v[0];
-        #pragma unroll
-        for (int k = 1; k < KS; ++k) m = v[k] < m ? v[k] : m;
-        best = Scores<WHOLE>::warp_min(m);
-        unsigned int r = NO_ROW;
-        #pragma unroll
-        for (int k = 0; k < KS; ++k) r = v[k] == best ? min(r, row[k]) : r;
-        return r;
+        refresh();
+    }
+    auto bound_of = [&](int4 b, int kp) { return min(min(b.x, b.y + kp), max(b.z, b.w + kp)); };
+    // a decision told to the folding warps: job `w` (a row, and RS_GIVEN with a peak) for item e; NONE: nothing is told
+    const unsigned int at_pending = smem_u32(rows.pending), at_jobs = smem_u32(sh.jobs), at_items = smem_u32(sh.items), at_ctl = smem_u32(&sh.ctl);
+    auto tell = [&](unsigned int e, int row_of, int w, unsigned int peak) {
+        asm volatile("{ .reg .pred p; setp.eq.s32 p, %0, 0; setp.ne.and.s32 p, %1, -2, p; @p st.shared.u32 [%2], 1; @p st.shared.v2.u32 [%3], {%1, %4}; }"
+                     ::"r"(lane), "r"(w), "r"(at_pending + 4u * (unsigned int)row_of), "r"(at_jobs + 8u * (e % RS_ITEMS)), "r"(peak) : "memory");
     };
-    auto bound_of_others = [&](int code) -> K {
-        const int4 b = sh.table[list & 1][code];
-        const K bp = sc.arrival_bp();
-        return min(min(Scores<WHOLE>::from_bits(b.x), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(b.y), bp)),
-                   max(Scores<WHOLE>::from_bits(b.z), Scores<WHOLE>::plus(Scores<WHOLE>::from_bits(b.w), bp)));
+    auto release = [&](unsigned int n) {
+        asm volatile("{ .reg .pred p; setp.eq.s32 p, %0, 0; @p st.release.cta.shared.u32 [%1], %2; }" ::"r"(lane), "r"(at_ctl), "r"(n) : "memory");
     };
-    // ADMIT: every instance overloaded?  While one is known not to be, the request is routed; else the folds under way decide.
-    auto all_folded = [&](unsigned int e) {
-        return __all_sync(FULL, lane >= RS_FOLD_WARPS || (int)(ld_acquire(&sh.done[lane_f]) - e) >= 0);
-    };
-    // the decision `w` (as in `row`) for item e with score `best`: the row is pending from now on, with its exact token
-    // count and a lower bound of its key
-    auto publish = [&](unsigned int n) {
-        __syncwarp();
-        if (lane == 0) st_release(&sh.ctl.x, n);
-    };
-    auto commit = [&](unsigned int e, int4 it, unsigned int w, S best, bool covers, bool held) {
-        unsigned int before = 0;
-        if (ADMIT) before = ld_volatile(rows.flags + (w >> 1));
-        if (held) {
+    // Everything unusual about item e.
+    auto unusual = [&](unsigned int e) {
+        const int4 it = sh.items[e % RS_ITEMS];
+        const int2 pd = sh.raw[e % RS_ITEMS];
+        const int P = pd.x, D = pd.y, Dc = D < H ? D : H, kp = it.x, kpd = it.y;
+        publish(e);
+        for (int lists_tried = 0;;) {
+            refresh();
+            if (it.z <= jmax) break;
+            // the rows that can have the smallest score: those within the slack of the smallest value of a row that is not marked
+            int v[KS], least = RS_ABSENT;
             #pragma unroll
             for (int k = 0; k < KS; ++k) {
-                const bool hit = row[k] == w;
-                if (hit) { rec[k] = sc.with_arrival(rec[k], covers); row[k] |= 1u; }
-                st_if(hit, rows.rec + (w >> 1), rec[k]);
+                v[k] = max(ra[k], rb[k] + kp);
+                if (!(ra[k] & 1)) least = min(least, v[k]);
             }
-        } else {                 // (the row may not be one of those held)
-            const uint2 now = sc.with_arrival(ld_volatile2(rows.rec + (w >> 1)), covers);
-            __syncwarp();
+            const int reach = __reduce_min_sync(FULL_MASK, least) + SLACK;
+            if (reach >= (WHOLE ? RS_ABSENT : RS_CUT)) {   // no row to measure by, or one whose keys are cut
+                const unsigned int before = held_pending();
+                if (__any_sync(FULL_MASK, before != 0)) {
+                    if (!rs_wait(sh, [&] { return __any_sync(FULL_MASK, held_pending() != before) != 0; })) { lost = true; return; }
+                    continue;
+                }
+                if (!LISTS) break;
+            }
+            if (LISTS && reach >= bound_of(ld_table(table + it.w), kp)) {   // a row outside the list could do as well
+                if (lists_tried == 2) break;
+                ++lists_tried;
+                next_list(e);
+                if (lost) return;
+                continue;
+            }
+            S mine = Scores<WHOLE>::none();
+            int mine_row = NO_ROW;
+            bool wait = false, scan = false;
+            #pragma unroll
+            for (int k = 0; k < KS; ++k) {
+                if (v[k] <= reach && row[k] != NO_ROW) {
+                    const int i = row[k];
+                    if (ld_volatile(rows.pending + i)) wait = true;
+                    else {
+                        const unsigned int top = ld_volatile(rows.top + i), jt = ld_volatile(rows.state + i) & RS_JTOP;
+                        const unsigned int tokens = WHOLE ? (unsigned int)ld_volatile2(rows.rec + i).x >> 1 : ld_volatile(rows.tok + i);
+                        if (Dc > (int)jt || sc.no_penalty(top, P)) {
+                            const S s = sc.of_peak(tokens, top + (unsigned int)P, P, D);
+                            if (s < mine || (s == mine && i < mine_row)) { mine = s; mine_row = i; }
+                        } else scan = true;
+                    }
+                }
+            }
+            if (__any_sync(FULL_MASK, wait)) {
+                if (!rs_wait(sh, [&] {
+                        bool open = false;
+                        #pragma unroll
+                        for (int k = 0; k < KS; ++k)
+                            if (v[k] <= reach && row[k] != NO_ROW) open |= ld_acquire(rows.pending + row[k]) != 0;
+                        return !open;
+                    })) { lost = true; return; }
+                continue;
+            }
+            if (__any_sync(FULL_MASK, scan)) break;
+            const S best = Scores<WHOLE>::warp_min(mine);
+            const int win = __reduce_min_sync(FULL_MASK, mine == best ? mine_row : NO_ROW);
+            if (win >= I) break;
             #pragma unroll
             for (int k = 0; k < KS; ++k)
-                if ((row[k] >> 1) == (w >> 1)) { rec[k] = now; row[k] |= 1u; }
-            st_if(lane == 0, rows.rec + (w >> 1), now);
+                if (row[k] == win) {
+                    const int marked = ra[k] & 1;
+                    ra[k] += kpd + marked;
+                    rb[k] += kpd + (marked ? 1 : kp);
+                }
+            tell(e, win, win, 0u);
+            return;
         }
-        st_if(lane == 0, rows.flags + (w >> 1), RS_PENDING);
-        st_if(lane == 0, sh.jobs + e % RS_ITEMS, make_int4((int)(w >> 1), it.x, it.y, sc.job_score(best)));
-        if (!WHOLE) st_if(lane == 0, sh.score + e % RS_ITEMS, (double)best);
-        if (ADMIT) taken_over += (before & RS_NOT_OVER) ? 1u : 0u;
-    };
-    // Everything unusual about item e.  False: the batch ends here.
-    auto unusual = [&](unsigned int e, int4 it) -> bool {
-        const int P = it.x, Dc = it.z & 0xffff;
-        publish(e);
-        if (ADMIT) {
-            if (__any_sync(FULL, ld_volatile(&sh.not_over) == taken_over)) {
-                if (!rs_wait(sh, [&] { const bool free_again = ld_volatile(&sh.not_over) != taken_over, all = all_folded(e); return free_again || all; })) { lost = true; return false; }
-                if (__all_sync(FULL, ld_acquire(&sh.not_over) == taken_over)) {   // the request is not routed: the batch stops here
-                    if (lane == 0) { sh.blocked = 1; sh.blocked_k = sh.item_at[e % RS_ITEMS]; }
-                    return false;
+        // ---- short arrivals and rows that have to be scanned: all rows, with every fold done.  First those with exact scores ...
+        if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return; }
+        acquire_cta();
+        auto look = [&](int i, S& s, unsigned int& tokens, unsigned int& peak) {   // whether row i's score is exact, and the score (else a lower bound)
+            s = Scores<WHOLE>::none();
+            tokens = peak = 0;
+            if (i >= I) return true;
+            const unsigned int top = rows.top[i], jt = rows.state[i] & RS_JTOP;
+            tokens = sc.tokens_of(rows, i);
+            const bool exact = Dc > (int)jt || sc.no_penalty(top, P);
+            peak = exact ? top + (unsigned int)P : top - jt;     // (jt is at most one step beyond the maximum's)
+            s = sc.of_peak(tokens, peak, P, D);
+            return exact;
+        };
+        S best = Scores<WHOLE>::none(), mine = best;
+        int win = RS_NO_ROW, mine_row = RS_NO_ROW, n_again = 0;
+        unsigned int mine_peak = 0, win_peak = 0;
+        for (int g0 = 0; g0 < n_groups; g0 += 4) {
+            S s[4];
+            unsigned int tokens, peak[4];
+            bool ok[4];
+            #pragma unroll
+            for (int u = 0; u < 4; ++u) ok[u] = look((g0 + u) * 32 + lane, s[u], tokens, peak[u]);
+            #pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (ok[u] && s[u] < mine) { mine = s[u]; mine_row = (g0 + u) * 32 + lane; mine_peak = peak[u]; }   // a lane's rows ascend
+                if (__any_sync(FULL_MASK, !ok[u])) {
+                    if (lane == 0) sh.slow_group[n_again] = (unsigned short)(g0 + u);
+                    ++n_again;
                 }
             }
         }
-        S best;
-        for (int lists_tried = 0;;) {
-            const unsigned int jmax = ld_volatile(&sh.jmax);    // (after the rows were read)
-            if ((unsigned int)Dc <= jmax) break;
-            const unsigned int w = __reduce_min_sync(FULL, best_of_lane(best));
-            if (LISTS && (w == NO_ROW || !sc.beats(best, bound_of_others(it.z >> 16)))) {   // a row outside the list could do as well
-                if (lists_tried == 2) break;
-                ++lists_tried;
-                next_list();
-                if (lost) return false;
-                continue;
-            }
-            if (w & 1u) {
-                if (!rs_wait(sh, [&] { return !(ld_acquire(rows.flags + (w >> 1)) & RS_PENDING); })) { lost = true; return false; }
-                if (!__any_sync(FULL, (ld_volatile(rows.flags + (w >> 1)) & RS_FAR) != 0)) { load_rows(); continue; }
-                // (far: its token count is its score where it pays no penalty)
-                if (!__all_sync(FULL, sc.no_penalty(ld_volatile(rows.top + (w >> 1))))) break;
-            }
-            commit(e, it, w, best, true, true);
-            return true;
-        }
-        // ---- short arrivals and rows that have to be scanned: all rows.  First those with exact scores ...
-        auto look = [&](int i, S& s, unsigned int& tokens) {   // whether row i's score is exact, and the score (else a lower bound)
-            bool exact = false;
-            s = Scores<WHOLE>::none();
-            tokens = 0;
-            if (i < I) {
-                const unsigned int f = ld_volatile(rows.flags + i);      // first: it is written last
-                const uint2 q = ld_volatile2(rows.rec + i);
-                const unsigned int top = ld_volatile(rows.top + i);
-                const bool full = !(f & RS_PENDING) && Dc > (int)(f & RS_JTOP);
-                tokens = q.x;
-                s = sc.of_top(q.x, full ? top : ld_volatile(rows.c0 + i));   // (c0 of a pending row: at least the old one)
-                exact = full || (!(f & RS_PENDING) && sc.no_penalty(top));
-            }
-            return exact;
-        };
-        best = Scores<WHOLE>::none();
-        int win = RS_NO_ROW;
-        S mine = Scores<WHOLE>::none();
-        int mine_row = RS_NO_ROW;
-        #pragma unroll 4
-        for (int g = 0; g < n_groups; ++g) {
-            S s;
-            unsigned int tokens;
-            const int i = g * 32 + lane;
-            const bool ok = look(i, s, tokens);
-            if (ok && s < mine) { mine = s; mine_row = i; }   // a lane's rows ascend
-        }
+        __syncwarp();
         auto take = [&]() {   // the warp's smallest of (mine, mine_row), against the best so far
             const S smallest = Scores<WHOLE>::warp_min(mine);
-            const int r = __reduce_min_sync(FULL, mine == smallest ? mine_row : RS_NO_ROW);
-            if (smallest < best || (smallest == best && r < win)) { best = smallest; win = r; }
+            const int r = __reduce_min_sync(FULL_MASK, mine == smallest ? mine_row : RS_NO_ROW);
+            if (smallest < best || (smallest == best && r < win)) {
+                best = smallest; win = r;
+                const unsigned int who = __ballot_sync(FULL_MASK, mine == smallest && mine_row == r);
+                win_peak = __shfl_sync(FULL_MASK, mine_peak, __ffs(who) - 1);
+            }
         };
         take();
-        // ... then those whose bound could beat the best: their folds are waited for, and they are scanned
-        for (int g = 0; g < n_groups; ++g) {
+        // ... then those whose bound could beat the best: they are scanned
+        for (int x = 0; x < n_again; ++x) {
             S s;
-            unsigned int tokens;
-            const int i = g * 32 + lane;
-            bool ok = look(i, s, tokens);
-            bool todo = i < I && (s < best || (s == best && i < win));   // (a fold may have ended since the first pass)
-            if (!__any_sync(FULL, todo)) continue;
-            if (!rs_wait(sh, [&] { return !todo || !(ld_acquire(rows.flags + i) & RS_PENDING); })) { lost = true; return false; }
-            ok = look(i, s, tokens);
-            mine = todo && ok ? s : Scores<WHOLE>::none();
-            mine_row = todo && ok ? i : RS_NO_ROW;
-            take();
-            todo = todo && !ok && (s < best || (s == best && i < win));
-            const unsigned int which = __ballot_sync(FULL, todo);
+            unsigned int tokens, peak;
+            const int i = (int)sh.slow_group[x] * 32 + lane;
+            const bool ok = look(i, s, tokens, peak);
+            const bool todo = !ok && (s < best || (s == best && i < win));
+            const unsigned int which = __ballot_sync(FULL_MASK, todo);
             if (!which) continue;
             const int slot = __popc(which & ((1u << lane) - 1u));
             if (todo) sh.scan_row[slot] = i;
@@ -997,105 +1103,208 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             ++scans;
             __syncwarp();
             if (lane == 0) st_release(&sh.ctl.y, scans);
-            if (!rs_wait(sh, [&] { return lane >= RS_FOLD_WARPS || ld_acquire(&sh.scans_done[lane_f]) == scans; })) { lost = true; return false; }
-            mine = todo ? sc.of_peak(tokens, sh.peak[slot]) : Scores<WHOLE>::none();
-            mine_row = todo ? i : RS_NO_ROW;
+            if (!rs_wait(sh, [&] { return ld_acquire(&sh.scans_done[lane_f]) == scans; })) { lost = true; return; }
+            mine = Scores<WHOLE>::none();
+            mine_row = RS_NO_ROW;
+            if (todo) {
+                mine_peak = sh.peak[slot];
+                mine = sc.of_peak(tokens, mine_peak, P, D);
+                mine_row = i;
+            }
             take();
             __syncwarp();
         }
-        if (win >= I) win = 0;   // (no score is finite: beta or theta beyond binary64's range)
-        // (the ramp reaches every row's key if it is longer than the largest jtop known before the rows were read)
-        commit(e, it, 2u * (unsigned int)win, best, false, false);
-        return true;
+        if (win >= I) { win = 0; win_peak = 0; }   // (no score is finite: beta or theta beyond binary64's range)
+        #pragma unroll
+        for (int k = 0; k < KS; ++k)
+            if (row[k] == win) {      // (a lower bound, odd)
+                ra[k] = (min(ra[k] + kpd + 1, RS_CUT) - 1) | 1;
+                rb[k] = (min(rb[k] + kpd + 1, RS_CUT) - 1) | 1;
+            }
+        tell(e, win, win | (int)RS_GIVEN, win_peak);
     };
 
     unsigned int e = 0, ready = 0;   // decisions made, items known to be there
-    bool more = !lost;
-    while (more) {
+    while (!lost) {     // (every way out has published what was decided)
         if (e >= ready) {
             bool end = false;
             if (!rs_wait(sh, [&] {
-                    end = __any_sync(FULL, ld_acquire(&sh.items_end) != 0);    // (before the count: the count is then final)
-                    ready = __shfl_sync(FULL, ld_acquire(&sh.items_ready), 0);
+                    end = __any_sync(FULL_MASK, ld_acquire(&sh.items_end) != 0);    // (before the count: the count is then final)
+                    ready = __shfl_sync(FULL_MASK, ld_acquire(&sh.items_ready), 0);
                     return ready > e || end;
                 }))
                 break;
             if (ready <= e) break;
         }
-        const unsigned int stop = min(ready, e + CHUNK);
-        if (!rs_wait(sh, [&] { return lane >= RS_FOLD_WARPS || (int)(stop - ld_acquire(&sh.done[lane_f])) <= RS_ITEMS; })) break;
-        if (!LISTS) load_rows();
-        int4 next = sh.items[e % RS_ITEMS];
-        for (; e < stop; ++e) {
-            const int4 it = next;
-            next = sh.items[(e + 1) % RS_ITEMS];      // (beyond the items that are there: not used)
-            const unsigned int jmax = ld_volatile(&sh.jmax);    // (after the rows were read)
-            bool odd = (unsigned int)(it.z & 0xffff) <= jmax;
-            if (ADMIT) odd |= ld_volatile(&sh.not_over) == taken_over;
-            sc.arrival(it);
-            K bound = K(0);
-            if (LISTS) bound = bound_of_others(it.z >> 16);
-            S best;
-            const unsigned int r = best_of_lane(best);
-            if (LISTS) odd |= !sc.beats(best, bound);
-            const unsigned int w = __reduce_min_sync(FULL, odd ? 1u : r);     // (odd: like a marked row)
-            if (__builtin_expect(w & 1u, 0)) {
-                if (!unusual(e, it)) { more = false; break; }
-                continue;
+        unsigned int stop = min(ready, e + CHUNK);
+        if (ADMIT) {
+            // Every instance overloaded?  Each decision not folded yet may have taken one more over the level; while fewer of
+            // those are under way than rows are known not to be overloaded, the request is routed.
+            int spare = 0;
+            if (!rs_wait(sh, [&] {
+                    const int next = __reduce_min_sync(FULL_MASK, (int)(ld_acquire(&sh.done[lane_f]) - e));
+                    const int open = next < 0 ? -next : 0;
+                    spare = (int)__shfl_sync(FULL_MASK, ld_acquire(&sh.not_over), 0) - open;
+                    return spare > 0 || open == 0;
+                }))
+                break;
+            if (spare <= 0) {   // the request is not routed: the batch stops here
+                if (lane == 0) { sh.blocked = 1; sh.blocked_k = sh.item_at[e % RS_ITEMS]; }
+                break;
             }
-            commit(e, it, w, best, true, true);
-            if (PUBLISH == 1 || (e & (PUBLISH - 1)) == PUBLISH - 1) publish(e + 1);
+            stop = min(stop, e + (unsigned int)spare);
         }
+        refresh();
+        // The usual way.  What was decided at one step is checked and told at the next, while the reduction over its scores is
+        // under way: the branch and the stores would else be waited for (measured in this loop alone, four rows per lane:
+        // 232 cycles with them in the step, 158 with them a step later, four steps per trip and the keys marked in their last bit).
+        int4 it = sh.items[e % RS_ITEMS];
+        int4 others = make_int4(0, 0, 0, 0);
+        if (LISTS) others = ld_table(table + it.w);
+        int w = NONE;        // the decision of the step before; ODD: that was not the usual case
+        auto scores = [&](int kp, int (&v)[KS]) {    // of the rows held; returns the lane's smallest
+            #pragma unroll
+            for (int k = 0; k < KS; ++k) v[k] = __viaddmax_s32(rb[k], kp, ra[k]);
+            int least = v[0];
+            #pragma unroll
+            for (int k = 1; k + 1 < KS; k += 2) least = __vimin3_s32(least, v[k], v[k + 1]);
+            return KS % 2 ? least : min(least, v[KS - 1]);
+        };
+        // u: e modulo 4 where that is known.  False: the step before was not the usual case, nothing has been done.
+        auto step = [&](unsigned int e, unsigned int trip, int u, bool publishes) -> bool {
+            const int kp = it.x, kpd = it.y, kpb = kpd + kp;
+            int v[KS];
+            const int best = __reduce_min_sync(FULL_MASK, scores(kp, v));
+            if (w == ODD) return false;
+            tell(u > 0 ? trip + u - 1 : e - 1, w, w, 0u);
+            if (publishes) release(e);
+            int bound = it.z > jmax ? (WHOLE ? RS_ABSENT : RS_CUT) : RS_LOWEST;
+            if (LISTS) bound = __vimin3_s32(bound, __viaddmin_s32(others.y, kp, others.x), __viaddmax_s32(others.w, kp, others.z));
+            it = ld_table(at_items + 16u * (u >= 0 && u < 3 ? (trip + u + 1) : (e + 1) % RS_ITEMS));      // (beyond the items that are there: not used)
+            int mine = NO_ROW;
+            if (WHOLE) {
+                #pragma unroll
+                for (int k = KS - 1; k >= 0; --k) mine = v[k] == best ? row[k] : mine;
+            } else {     // more than one row that can be the best: not the usual case
+                int many = 0;
+                #pragma unroll
+                for (int k = KS - 1; k >= 0; --k)
+                    if (v[k] <= best + SLACK) { mine = row[k]; ++many; }
+                if (many > 1) mine = ODD;
+            }
+            if (best + SLACK >= bound || (best & 1)) mine = ODD;
+            w = __reduce_min_sync(FULL_MASK, mine);
+            if (!WHOLE) {
+                const int last = __reduce_max_sync(FULL_MASK, mine == NO_ROW ? ODD : mine);
+                if (last != w) w = ODD;
+            }
+            if (LISTS) others = ld_table(table + it.w);
+            #pragma unroll
+            for (int k = 0; k < KS; ++k)
+                if (row[k] == w) { ra[k] += kpd; rb[k] += kpb; }
+            return true;
+        };
+        // (everything unusual in one place, away from the loop: inlined in it the way around it cost 15 cycles a step)
+        for (;;) {
+            bool usual = true;
+            while (e < stop) {
+                if ((e & 3u) == 0 && e + 4 <= stop) {
+                    const unsigned int trip = e % RS_ITEMS;
+                    usual = step(e, trip, 0, true);
+                    if (!usual) break;
+                    ++e;
+                    usual = step(e, trip, 1, PUBLISH == 1);
+                    if (!usual) break;
+                    ++e;
+                    usual = step(e, trip, 2, PUBLISH <= 2);
+                    if (!usual) break;
+                    ++e;
+                    usual = step(e, trip, 3, PUBLISH == 1);
+                    if (!usual) break;
+                    ++e;
+                } else {
+                    usual = step(e, 0u, -1, true);
+                    if (!usual) break;
+                    ++e;
+                }
+            }
+            if (usual && w != ODD) break;
+            unusual(e - 1);
+            w = NONE;
+            if (lost || e >= stop) break;
+            if (LISTS) others = ld_table(table + it.w);
+        }
+        tell(e - 1, w, w, 0u);
+        if (lost) break;
         publish(e);
     }
     __syncwarp();
     if (lane == 0) st_release(&sh.ctl.z, 1u);
 }
 
+// Folding and list warps, warps and threads of the instantiations.
+template <bool LISTS, bool ADMIT> struct Shape {
+    static constexpr int FOLD = ADMIT ? 11 : (LISTS ? 6 : 5), LIST = LISTS ? (ADMIT ? 3 : 8) : 0;
+    static constexpr int WARPS = 4 * ((FOLD + 1 + LIST + 2) / 3), THREADS = 32 * WARPS;
+};
+
 template <int KS, bool LISTS, bool ADMIT, bool WHOLE>
-__global__ void __launch_bounds__(RS_THREADS, 1) pre_route_summaries(const RouteSumArgs a) {
+__global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_summaries(const RouteSumArgs a) {
+    typedef Shape<LISTS, ADMIT> Sp;
+    constexpr int THREADS = Sp::THREADS;
     extern __shared__ __align__(16) unsigned char rs_smem[];
     __shared__ __align__(16) RsShared sh;
-    typedef typename Scores<WHOLE>::K K;
     const int I = a.I, H = a.H;
     Rows rows;
-    rows.rec = reinterpret_cast<uint2*>(rs_smem);
-    rows.flags = reinterpret_cast<unsigned int*>(rows.rec + I);
-    rows.top = rows.flags + I;
-    rows.c0 = rows.top + I;
+    rows.rec = reinterpret_cast<int2*>(rs_smem);
+    rows.state = reinterpret_cast<unsigned int*>(rows.rec + I);
+    rows.top = rows.state + I;
+    rows.pending = rows.top + I;
+    rows.tok = rows.pending + I;     // (binary64 scores only)
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int near_steps = LISTS ? RS_NEAR_LISTS : RS_NEAR_DIRECT;
-    const unsigned long long mc = a.guard[GUARD_MAX_CELL], mb = a.guard[GUARD_MAX_BASE], ramps = a.guard[GUARD_SUM_RAMP];
+    // (the warp's number by a shuffle: the compiler then knows that the roles part between warps and not within one, and
+    // leaves out what would bring the lanes of a warp together again: 157 instead of 202 cycles for a step of the deciding warp)
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(FULL_MASK, tid >> 5, 0);
+    const unsigned long long mc = a.guard[GUARD_MAX_CELL], mb = a.guard[GUARD_MAX_BASE], ramps = a.guard[GUARD_SUM_RAMP],
+                             tokens_in = a.guard[GUARD_SUM_TOKENS], max_pd = a.guard[GUARD_MAX_PD], base_sum = a.guard[GUARD_SUM_BASE];
     // every cell, every cell + step with a prompt added, and every token count stay below 2^32 all batch long
-    const unsigned long long peak_bound = mc + ramps + (unsigned long long)H + (unsigned long long)PRE_FIELD_MAX;
+    // (the ramps of the batch bound what an arrival that is not routed yet can add, too)
+    const unsigned long long peak_bound = mc + ramps + (unsigned long long)H;
     if (tid == 0) {
-        const unsigned long long token_bound = mb + a.guard[GUARD_SUM_TOKENS];
+        const unsigned long long token_bound = mb + tokens_in;
         // (and the batch is short enough for 32-bit counters)
         const bool ok = a.guard[GUARD_BAD] == 0 && peak_bound <= 0xffffffffull && token_bound <= 0xffffffffull &&
                         a.n_arrivals + (ADMIT ? a.queue_capacity : 0) < (1ll << 26);
         // (whole-number scores: the host has seen to beta and theta)
-        const bool exact = !WHOLE || token_bound + a.guard[GUARD_MAX_PD] + (unsigned long long)a.beta * peak_bound < (1ull << 30);
+        const bool exact = !WHOLE || token_bound + max_pd + (unsigned long long)a.beta * (peak_bound + 1) < (1ull << 29);
         sh.mode = ok && exact ? 1 : 0;
         sh.n0 = *a.n_requests;
         sh.ctl = make_uint4(0u, 0u, 0u, 0u);
-        sh.items_ready = sh.items_end = sh.not_over = sh.jmax = 0;
+        sh.items_ready = sh.items_end = sh.not_over = sh.jmax = sh.written = sh.flush = 0;
         sh.lists_wanted = sh.lists_ready = sh.list_met = 0;
         sh.list_n[0] = sh.list_n[1] = 0;
         sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0;
     }
-    if (tid < RS_FOLD_WARPS) { sh.done[tid] = (unsigned int)tid; sh.scans_done[tid] = 0; }
-    if (tid < RS_PROBES) sh.probe_t[tid] = -1;
-    __syncthreads();
-    if (sh.mode == 0) {
-        if (tid == 0) *a.handled = 0;
-        return;
-    }
+    for (int i = tid; i < RS_ITEMS; i += THREADS) sh.items[i] = make_int4(0, 0, 0, 0);    // (an item is fetched before it is known to be there)
+    if (tid < RS_MAX_FOLD_WARPS) { sh.done[tid] = (unsigned int)tid; sh.scans_done[tid] = 0; }
+    if (tid < RS_PROBES) sh.probe_t[tid] = 0xffffffffu;
     // ADMIT: the requests that were waiting when the call was made come first, then the arrivals
     long long q_head = 0, q_len = 0;
+    if (ADMIT && a.queue_capacity > 0) {
+        q_head = a.queue_state[0];
+        q_len = a.queue_state[1];
+    }
+    __syncthreads();
+    if (tid < GUARDS) a.guard[tid] = 0;    // ready for the next call
+    if (sh.mode == 0) {
+        if (tid == 0) {
+            *a.handled = 0;
+            if (ADMIT) { a.queue_entry[0] = a.queue_state[0]; a.queue_entry[1] = a.queue_state[1]; }
+        }
+        if (tid < 3) a.give_up[tid] = 0;
+        return;
+    }
     if (ADMIT && a.queue_capacity > 0) {   // kept inside the ring whatever the two words hold
-        q_head = a.queue_entry[0];
-        q_len = a.queue_entry[1];
         if (q_head < 0 || q_head >= a.queue_capacity) q_head = 0;
         if (q_len < 0) q_len = 0;
         if (q_len > a.queue_capacity) q_len = a.queue_capacity;
@@ -1104,61 +1313,64 @@ __global__ void __launch_bounds__(RS_THREADS, 1) pre_route_summaries(const Route
     const unsigned long long mean_l = ramps / (unsigned long long)(n_items > 0 ? n_items : 1);
     const int mean = mean_l < (1ull << 22) ? (int)mean_l : 1 << 22;     // prompt + ramp of a typical request
     Scores<WHOLE> sc;
-    sc.start(a.theta, a.beta, peak_bound, mean);
+    sc.start(a.theta, a.beta, peak_bound, max_pd, (base_sum + tokens_in) / (unsigned long long)I, mean);
     {
         unsigned int jmax = 0;
         int free_rows = 0;
-        K least[LISTS ? RS_PROBES : 1];      // the smallest score per probe, for the first list
+        int least[LISTS ? RS_PROBES : 1];      // the smallest value per probe, for the first list
         if (LISTS)
             #pragma unroll
-            for (int p = 0; p < RS_PROBES; ++p) least[LISTS ? p : 0] = Scores<WHOLE>::from_bits(0x7f000000);
-        for (int i = tid; i < I; i += RS_THREADS) {
+            for (int p = 0; p < RS_PROBES; ++p) least[LISTS ? p : 0] = 0x7f000000;
+        for (int i = tid; i < I; i += THREADS) {
             const uint4 q = a.summary0[i];
-            const bool far = q.z >= (unsigned int)near_steps;
-            if (!far) jmax = max(jmax, q.z);
+            const unsigned int jtop = q.z & 0xffffu, step = q.z >> 16;
+            const bool far = jtop >= (unsigned int)RS_LIMIT;
+            jmax = max(jmax, far ? step : jtop);
             const bool not_over = ADMIT && !((double)a.over0[i] > a.many);
             free_rows += not_over;
-            const uint2 rec = make_uint2(q.x, sc.key(q.x, far ? q.w : q.y));
+            const int2 rec = make_int2(sc.key_a(q.x), sc.key_b(q.x, far ? q.w : q.y));
             rows.rec[i] = rec;
+            rows.state[i] = jtop | (far ? RS_FAR : 0u) | (jtop >= (unsigned int)RS_NEAR ? RS_FULL : 0u) | (not_over ? RS_NOT_OVER : 0u);
+            rows.top[i] = q.y;
+            rows.pending[i] = 0;
+            if (!WHOLE) rows.tok[i] = q.x;
             if (LISTS)
                 #pragma unroll
-                for (int p = 0; p < RS_PROBES; ++p) least[LISTS ? p : 0] = min(least[LISTS ? p : 0], rs_score_at(sc, rec, sc.probe(rs_probe(mean, p))));
-            rows.flags[i] = q.z | (far ? RS_FAR : 0u) | (not_over ? RS_NOT_OVER : 0u);
-            rows.top[i] = q.y;
-            rows.c0[i] = q.w;
+                for (int p = 0; p < RS_PROBES; ++p) least[LISTS ? p : 0] = min(least[LISTS ? p : 0], max(rec.x, rec.y + sc.key_p(rs_probe(mean, p))));
         }
-        jmax = __reduce_max_sync(0xffffffffu, jmax);
+        jmax = __reduce_max_sync(FULL_MASK, jmax);
         if (lane == 0 && jmax) atomicMax(&sh.jmax, jmax);
         if (LISTS)
             #pragma unroll
             for (int p = 0; p < RS_PROBES; ++p) {
-                const unsigned int v = __reduce_min_sync(0xffffffffu, Scores<WHOLE>::order(least[LISTS ? p : 0]));
-                if (lane == 0) atomicMin(reinterpret_cast<unsigned int*>(&sh.probe_t[p]), v);
+                const int v = __reduce_min_sync(FULL_MASK, least[LISTS ? p : 0]);
+                if (lane == 0) atomicMin(&sh.probe_t[p], ordered(v));
             }
         if (ADMIT) {
-            free_rows = __reduce_add_sync(0xffffffffu, free_rows);
+            free_rows = __reduce_add_sync(FULL_MASK, free_rows);
             if (lane == 0 && free_rows) atomicAdd(&sh.not_over, (unsigned int)free_rows);
         }
     }
     const long long room = a.max_requests - sh.n0;
     __syncthreads();
 
+    const int role = (warp >> 2) * 3 + (warp & 3) - 1;      // (of the warps that are not on the deciding warp's scheduler)
     if (warp == 0) {
-        rs_decide_loop<KS, LISTS, ADMIT, WHOLE>(a, sh, rows, sc);
-    } else if (warp == RS_IO_WARP) {
-        rs_io_loop<ADMIT, WHOLE>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
-    } else if (warp >= RS_LIST_WARP) {
-        if (LISTS) rs_list_loop<WHOLE>(sh, rows, sc, I, mean, a.guard[GUARD_MAX_PD] < (1ull << 29) ? (int)a.guard[GUARD_MAX_PD] : 1 << 29);
+        rs_decide_loop<KS, LISTS, Sp::FOLD, ADMIT, WHOLE>(a, sh, rows, sc);
     } else if ((warp & 3) != 0) {
-        const int me = (warp >> 2) * 3 + (warp & 3) - 1;
-        if ((H & 1) == 0) rs_fold_loop<true, ADMIT, WHOLE, LISTS>(a, sh, rows, sc, me, near_steps);
-        else rs_fold_loop<false, ADMIT, WHOLE, LISTS>(a, sh, rows, sc, me, near_steps);
+        if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, WHOLE, LISTS>(a, sh, rows, sc, role);
+        else if (role == Sp::FOLD)
+            rs_io_loop<Sp::FOLD, ADMIT, WHOLE>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
+        else if (LISTS && role <= Sp::FOLD + Sp::LIST)
+            rs_list_loop<LISTS ? Sp::LIST : 3, WHOLE>(sh, rows, sc, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
     }
     __syncthreads();
     const bool blocked = ADMIT && sh.blocked;
     const long long decided = blocked ? sh.blocked_k : n_items;
     if (tid == 0) {
         *a.n_requests = sh.n0 + sh.ctl.x;
+        a.ramps[0] = sh.n0;
+        a.ramps[1] = ADMIT ? 0 : (long long)sh.ctl.x;
         // (what was noted beyond a blocked request is decided again below and does not count here)
         int flags = sh.ctl.w ? PRE_ST_TIMEOUT : 0;
         if (sh.first_bad < decided) flags |= PRE_ST_BADREQ;
@@ -1173,10 +1385,10 @@ __global__ void __launch_bounds__(RS_THREADS, 1) pre_route_summaries(const Route
         __syncthreads();
         const long long stop = decided;
         const long long left = stop < q_len ? q_len - stop : 0;          // waiting entries that stay
-        for (long long k = stop + tid; k < q_len; k += RS_THREADS) a.queue_choice[k] = -2;
+        for (long long k = stop + tid; k < q_len; k += THREADS) a.queue_choice[k] = -2;
         const long long a0 = (stop > q_len ? stop : q_len) - q_len;      // first arrival that was not decided
-        const int nw = RS_WARPS;
-        for (long long base = a0; base < a.n_arrivals; base += RS_THREADS) {
+        const int nw = Sp::WARPS;
+        for (long long base = a0; base < a.n_arrivals; base += THREADS) {
             const long long i = base + tid;
             int P = -1, D = 0;
             if (i < a.n_arrivals) { P = a.arr_prompt[i]; D = a.arr_predicted[i]; }
@@ -1222,8 +1434,6 @@ __global__ void __launch_bounds__(RS_THREADS, 1) pre_route_summaries(const Route
 
 // ---- host side
 
-static size_t summaries_smem_bytes(int I) { return (size_t)((I + 3) & ~3) * RS_ROW_BYTES; }
-
 // beta and theta = t_mem * M whole numbers of moderate size: the scores can be taken in whole-number arithmetic
 static bool summaries_whole_numbers(const pre_ctx* ctx) {
     const double beta = ctx->cfg.beta, theta = ctx->theta;
@@ -1255,7 +1465,7 @@ static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* s
     cudaFuncAttributes attr;
     cudaError_t e = cudaFuncGetAttributes(&attr, fn);
     if (e != cudaSuccess) return e;
-    const size_t smem = summaries_smem_bytes(I);
+    const size_t smem = (size_t)I * (sizeof(int2) + (summaries_whole_numbers(ctx) ? 3 : 4) * sizeof(unsigned int));
     if (smem + attr.sharedSizeBytes + 256 > limit) return cudaSuccess;   // too many instances
     // (the limit is shared by every context of the process: always the device maximum)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(limit - attr.sharedSizeBytes));
@@ -1267,12 +1477,12 @@ static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* s
 cudaError_t pre_route_summary_configure(pre_ctx* ctx) {
     ctx->route_summary_smem = 0;
     ctx->route_summary_smem_admit = 0;
-    cudaDeviceProp prop;
-    cudaError_t e = cudaGetDeviceProperties(&prop, ctx->device);
+    int limit = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
     if (e != cudaSuccess) return e;
-    e = summaries_configure_one<false>(ctx, (size_t)prop.sharedMemPerBlockOptin, &ctx->route_summary_smem);
+    e = summaries_configure_one<false>(ctx, (size_t)limit, &ctx->route_summary_smem);
     if (e != cudaSuccess) return e;
-    return summaries_configure_one<true>(ctx, (size_t)prop.sharedMemPerBlockOptin, &ctx->route_summary_smem_admit);
+    return summaries_configure_one<true>(ctx, (size_t)limit, &ctx->route_summary_smem_admit);
 }
 
 bool pre_route_summary_fits(const pre_ctx* ctx) { return ctx->route_summary_smem != 0 && ctx->d_rs_summary != nullptr; }
@@ -1290,7 +1500,8 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
     p.I = I; p.H = H;
     p.summary = reinterpret_cast<uint4*>(ctx->d_rs_summary);
     p.guard = ctx->d_rs_guard;
-    p.over = nullptr; p.hot = 0; p.queue_prompt = nullptr; p.queue_predicted = nullptr; p.queue_entry = nullptr;
+    p.near = reinterpret_cast<uint2*>(ctx->d_rs_near); p.far = ctx->d_rs_far;
+    p.over = nullptr; p.hot = 0; p.queue_prompt = nullptr; p.queue_predicted = nullptr; p.queue_state = nullptr;
     p.queue_capacity = 0;
     a.arr_prompt = arr_prompt; a.arr_predicted = arr_predicted; a.n_arrivals = n_arrivals;
     a.curves = curves; a.queued_p = queued_p; a.current_d = current_d;
@@ -1299,8 +1510,8 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
     a.choice = choice; a.score = score;
     a.I = I; a.H = H;
     a.theta = ctx->theta; a.beta = ctx->cfg.beta;
-    a.summary0 = p.summary; a.guard = p.guard;
-    a.status = ctx->d_status; a.handled = ctx->d_rs_handled;
+    a.summary0 = p.summary; a.guard = p.guard; a.near = p.near; a.far = p.far; a.applied = ctx->d_rs_applied;
+    a.status = ctx->d_status; a.handled = ctx->d_rs_handled; a.give_up = ctx->d_abort; a.ramps = ctx->d_rs_ramps;
     a.queue_prompt = nullptr; a.queue_predicted = nullptr; a.queue_state = nullptr; a.queue_entry = nullptr;
     a.queue_capacity = 0; a.queue_choice = nullptr; a.hot = 0; a.many = 0.0; a.over0 = nullptr;
 }
@@ -1308,14 +1519,12 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
 template <bool ADMIT>
 static cudaError_t launch_summary_kernels(pre_ctx* ctx, const SumArgs& p, const RouteSumArgs& a, cudaStream_t s) {
     const int I = ctx->cfg.n_instances;
-    cudaError_t e = cudaMemsetAsync(ctx->d_rs_guard, 0, 8 * sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
     const int rows_per_block = SUM_THREADS / 32;
     pre_summarise_rows<<<(I + rows_per_block - 1) / rows_per_block, SUM_THREADS, 0, s>>>(p);
-    e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     void* params[] = {(void*)&a};
-    return cudaLaunchKernel(summaries_kernel_for<ADMIT>(ctx), dim3(1), dim3(RS_THREADS), params,
+    return cudaLaunchKernel(summaries_kernel_for<ADMIT>(ctx), dim3(1), dim3(I > RS_DIRECT_ROWS ? Shape<true, ADMIT>::THREADS : Shape<false, ADMIT>::THREADS), params,
                             ADMIT ? ctx->route_summary_smem_admit : ctx->route_summary_smem, s);
 }
 
@@ -1330,7 +1539,7 @@ cudaError_t pre_launch_route_summary(pre_ctx* ctx, const int32_t* arr_prompt, co
     return launch_summary_kernels<false>(ctx, p, a, s);
 }
 
-// The queue's head and length must have been copied to ctx->d_queue_entry on the stream before this call.
+// (When the kernel declines the batch it leaves the queue's head and length in ctx->d_queue_entry for the scanning kernel.)
 cudaError_t pre_launch_route_summary_admit(pre_ctx* ctx, const int32_t* arr_prompt, const int32_t* arr_predicted,
                                            int64_t n_arrivals, long long hot, double many, int32_t* queue_prompt,
                                            int32_t* queue_predicted, int64_t* queue_state, int64_t queue_capacity,
@@ -1343,7 +1552,7 @@ cudaError_t pre_launch_route_summary_admit(pre_ctx* ctx, const int32_t* arr_prom
     fill_summary_args(ctx, p, a, arr_prompt, arr_predicted, n_arrivals, curves, queued_p, current_d, prompt, generated,
                       predicted, instance, n_requests, choice, score);
     p.over = ctx->d_rs_over; p.hot = hot;
-    p.queue_prompt = queue_prompt; p.queue_predicted = queue_predicted; p.queue_entry = ctx->d_queue_entry;
+    p.queue_prompt = queue_prompt; p.queue_predicted = queue_predicted; p.queue_state = queue_state;
     p.queue_capacity = queue_capacity;
     a.queue_prompt = queue_prompt; a.queue_predicted = queue_predicted; a.queue_state = queue_state;
     a.queue_entry = ctx->d_queue_entry; a.queue_capacity = queue_capacity; a.queue_choice = queue_choice;
