@@ -9,6 +9,8 @@ from __future__ import annotations
 import ctypes as C
 import os
 
+import torch
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libpreserve_b200.so")
 
@@ -61,6 +63,8 @@ def _load():
 
 
 lib = _load()
+_raw_stream = torch._C._cuda_getCurrentRawStream
+_device = torch._C._cuda_getDevice
 
 
 class PreError(RuntimeError):
@@ -79,8 +83,8 @@ def _ptr(t):
 
 
 def _stream():
-    import torch
-    return torch.cuda.current_stream().cuda_stream
+    """torch's current stream on the current device, without building a Stream object for it."""
+    return _raw_stream(_device())
 
 
 def pre_strerror(code: int) -> str:

@@ -712,6 +712,8 @@ size_t pre_chunk_table_words(int n_tiles, int max_chunks) {
 cudaError_t pre_launch_anticipate(pre_ctx* ctx, const int32_t* prompt, const int32_t* generated,
                                   const int32_t* predicted, const int32_t* instance, int64_t n,
                                   int64_t* curves, int64_t* current_d, cudaStream_t s) {
+    if (pre_small_build_fits(ctx, n))
+        return pre_launch_anticipate_small(ctx, prompt, generated, predicted, instance, n, curves, current_d, s);
     if (pre_fused_fits(ctx, n))
         return pre_launch_anticipate_fused(ctx, prompt, generated, predicted, instance, n, curves, current_d, s);
     const int I = ctx->cfg.n_instances, H = ctx->cfg.horizon, T = ctx->tile_rows, nt = ctx->n_tiles;

@@ -116,6 +116,7 @@ int pre_create(const pre_config* cfg, pre_ctx** out) {
     if (e == cudaSuccess) e = alloc_zero(&c->d_queue_entry, 2);
     c->spin_limit = PRE_DEFAULT_SPIN_LIMIT;
     if (e == cudaSuccess) e = pre_anticipate_configure(c);
+    if (e == cudaSuccess) e = pre_small_build_configure(c);
     if (e == cudaSuccess) e = pre_fused_configure(c);
     if (e == cudaSuccess) e = pre_route_configure(c);
     if (e == cudaSuccess) e = alloc_zero(&c->d_slots, (size_t)32 * c->route_blocks);

@@ -52,6 +52,8 @@ struct pre_ctx {
     long long* d_scaler_partial;    // [16 * n_sm][3] block totals of the kernels that sum the scaler's signals
     unsigned int* d_scaler_done;    // blocks of that kernel that have finished (zero between calls)
     unsigned int* d_ring_done;      // the same for the kernel that advances a ring of maps
+    size_t small_build_smem;        // build of small tables: 0 when this shape does not use it
+    int64_t small_build_rows;       // and the largest table it takes
     // fused (single-launch) build: 0 blocks when this shape does not use it
     int fused_grid;
     size_t fused_smem;
@@ -138,6 +140,11 @@ int pre_tile_threads(int tile_rows, int horizon);
 int pre_sort_max_chunks(int64_t max_requests, int n_sm);
 size_t pre_chunk_table_words(int n_tiles, int max_chunks);
 cudaError_t pre_anticipate_configure(pre_ctx* ctx);
+cudaError_t pre_small_build_configure(pre_ctx* ctx);   // sets ctx->small_build_smem
+bool pre_small_build_fits(const pre_ctx* ctx, int64_t n);
+cudaError_t pre_launch_anticipate_small(pre_ctx* ctx, const int32_t* prompt, const int32_t* generated,
+                                        const int32_t* predicted, const int32_t* instance, int64_t n,
+                                        int64_t* curves, int64_t* current_d, cudaStream_t s);
 cudaError_t pre_fused_configure(pre_ctx* ctx);   // sets ctx->fused_grid (0: this shape keeps the two-kernel build)
 bool pre_fused_fits(const pre_ctx* ctx, int64_t n);
 int64_t pre_fused_max_rows(const pre_ctx* ctx);

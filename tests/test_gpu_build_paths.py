@@ -128,3 +128,20 @@ def test_table_beyond_the_single_launch_build():
     check(st, table_of(wl, info[3]), n_inst, h, "single launch at its largest table")
     check(st, table_of(wl), n_inst, h, "two-kernel build again")
     st.close()
+
+
+@pytest.mark.parametrize("n_inst,h,n", [(1, 1, 1), (1, 255, 3), (7, 256, 4), (8, 257, 130), (149, 511, 2047), (300, 33, 16383),
+                                        (64, 256, 16384), (64, 256, 16385), (2, 8192, 500), (296, 8192, 900)])
+def test_tables_on_both_sides_of_the_small_build(n_inst, h, n):
+    """Up to 16,384 rows every block looks through the whole table for its own rows; segments of 256 cells."""
+    wl = W.make_random(400 + n % 89, n_inst, h, n, 0, max_prompt=2 ** 27, max_output=2 * h + 3)
+    st = DeviceState(n_inst, h, 1000, n)
+    check(st, table_of(wl), n_inst, h, "sums beyond 32 bits")
+    wl.instance[n // 2] = n_inst if n > 1 else 0            # malformed: skipped and reported
+    st.load_requests(*table_of(wl))
+    st.anticipate()
+    assert st.status() == (B.PRE_EBADREQ if n > 1 else B.PRE_OK)
+    keep = np.arange(n) != n // 2 if n > 1 else np.ones(n, bool)
+    want_c, want_d = expect(*(c[keep] for c in table_of(wl)), n_inst, h)
+    assert (st.curves.cpu().numpy() == want_c).all() and (st.current_d.cpu().numpy() == want_d).all()
+    st.close()
