@@ -347,31 +347,39 @@ __device__ __forceinline__ void inspect_row_chunks(const int64_t* __restrict__ r
     *max_lo = m;
 }
 
-// The map update of Sec. 4.3.1 for the requests that the summary kernel has routed, by the whole grid: integer
-// reductions, so their order does not matter.  A warp takes one table row at a time, or eight when there are many, and each
-// of them with consecutive lanes on consecutive cells.
-__device__ __forceinline__ void add_ramps(const RouteArgs& a) {
-    const int lane = threadIdx.x & 31, H = a.H;
-    const long long first = a.ramps[0], count = a.ramps[1];
-    const long long warps = (long long)gridDim.x * ROUTE_WARPS, me = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+// The map update of Sec. 4.3.1 for the requests that the summary kernel has routed (table rows ramps[0] ... + ramps[1], but
+// for those marked as applied, whose marks are taken back), by a whole grid of blocks of `block_warps` warps: integer
+// reductions, so their order does not matter.  A warp takes one table row at a time, or eight when there are many, and
+// each of them with consecutive lanes on consecutive cells.
+__device__ __forceinline__ void add_ramps(const long long* ramps, unsigned char* applied, const int32_t* prompt, const int32_t* predicted,
+                                          const int32_t* instance, int64_t* curves, int H, int block_warps) {
+    const int lane = threadIdx.x & 31;
+    const long long first = ramps[0], count = ramps[1];
+    const long long warps = (long long)gridDim.x * block_warps, me = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     const int each = count > 8 * warps ? 8 : 1;
     for (long long base = me * each; base < count; base += warps * each) {
         const long long k = base + lane;
         int P = 0, len = 0, w = 0;
         if (lane < each && k < count) {
-            if (a.applied[k]) a.applied[k] = 0;
+            if (applied[k]) applied[k] = 0;
             else {
-                P = a.prompt[first + k]; w = a.instance[first + k];
-                const int D = a.predicted[first + k];
+                P = prompt[first + k]; w = instance[first + k];
+                const int D = predicted[first + k];
                 len = D < H ? D : H;
             }
         }
         for (int src = 0; src < each; ++src) {
             const int p = __shfl_sync(0xffffffffu, P, src), n = __shfl_sync(0xffffffffu, len, src);
-            unsigned long long* row = reinterpret_cast<unsigned long long*>(a.curves) + (size_t)__shfl_sync(0xffffffffu, w, src) * H;
+            unsigned long long* row = reinterpret_cast<unsigned long long*>(curves) + (size_t)__shfl_sync(0xffffffffu, w, src) * H;
             for (int j = lane; j < n; j += 32) atomicAdd(row + j, (unsigned long long)(p + j));
         }
     }
+}
+constexpr int RAMP_THREADS = 256;
+__global__ void __launch_bounds__(RAMP_THREADS)
+pre_add_ramps(const long long* ramps, unsigned char* applied, const int32_t* prompt, const int32_t* predicted,
+              const int32_t* instance, int64_t* curves, int H) {
+    add_ramps(ramps, applied, prompt, predicted, instance, curves, H, RAMP_THREADS / 32);
 }
 
 // ADMIT adds the admission queue of Sec. 4.3.3: every block keeps, for its rows, the number of
@@ -414,7 +422,7 @@ __global__ void __launch_bounds__(ROUTE_THREADS, 1) pre_route_persistent(const R
     constexpr int RS_RESIDENT = 1, RS_WIDE = 2;
 
     if (a.done_elsewhere && *a.done_elsewhere) {   // the same word for every block; nobody writes it meanwhile
-        if (!ADMIT) add_ramps(a);
+        if (!ADMIT) add_ramps(a.ramps, a.applied, a.prompt, a.predicted, a.instance, a.curves, a.H, ROUTE_WARPS);
         return;
     }
     const int G = gridDim.x, b = blockIdx.x;
@@ -1073,6 +1081,14 @@ static void fill_route_args(RouteArgs& a, pre_ctx* ctx, const int32_t* arr_promp
 // The summary kernel wherever the shape fits it, unless the scanning kernel was selected.
 static bool pre_route_summary_wanted(const pre_ctx* ctx) { return ctx->route_path != PRE_ROUTE_SCAN; }
 
+cudaError_t pre_launch_add_ramps(pre_ctx* ctx, int64_t n_arrivals, const int32_t* prompt, const int32_t* predicted,
+                                 const int32_t* instance, int64_t* curves, cudaStream_t s) {
+    long long blocks = (n_arrivals + RAMP_THREADS / 32 - 1) / (RAMP_THREADS / 32);     // a warp per row
+    if (blocks > 8LL * ctx->n_sm) blocks = 8LL * ctx->n_sm;
+    pre_add_ramps<<<(int)blocks, RAMP_THREADS, 0, s>>>(ctx->d_rs_ramps, ctx->d_rs_applied, prompt, predicted, instance, curves, ctx->cfg.horizon);
+    return cudaGetLastError();
+}
+
 cudaError_t pre_launch_route(pre_ctx* ctx, const int32_t* arr_prompt, const int32_t* arr_predicted,
                              int64_t n_arrivals, int64_t* curves, int64_t* queued_p, int64_t* current_d,
                              int32_t* prompt, int32_t* generated, int32_t* predicted, int32_t* instance,
@@ -1086,7 +1102,7 @@ cudaError_t pre_launch_route(pre_ctx* ctx, const int32_t* arr_prompt, const int3
     if (summaries) {
         e = pre_launch_route_summary(ctx, arr_prompt, arr_predicted, n_arrivals, curves, queued_p, current_d, prompt,
                                      generated, predicted, instance, n_requests, choice, score, s);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || pre_route_summary_alone(ctx)) return e;
     }
     if (!summaries) {    // (else the summary kernel clears them when it declines)
         e = cudaMemsetAsync(ctx->d_abort, 0, 3 * sizeof(int), s);   // flag, agreed exchange, blocks met
@@ -1121,7 +1137,7 @@ cudaError_t pre_launch_route_admit(pre_ctx* ctx, const int32_t* arr_prompt, cons
                                            queue_predicted, queue_state, queue_capacity, queue_choice, curves, queued_p,
                                            current_d, prompt, generated, predicted, instance, n_requests, choice, score,
                                            s);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || pre_route_summary_alone(ctx)) return e;
     }
     if (!summaries) {
         // The kernel's blocks read the queue's head and length while block 0 may already be writing the

@@ -65,6 +65,8 @@ constexpr int RS_MAX_BINARY64_ROWS = 5120;  // and with binary64 scores
 constexpr int SUM_THREADS = 256;
 constexpr unsigned int RS_SPIN_LIMIT = 1u << 24;   // polls of shared memory (some 0.5 s) before a wait inside the block is abandoned
 constexpr int RS_NO_ROW = 0x3fffffff;
+constexpr long long RS_ALONE_CELLS = 32768;        // small shapes: cells of the maps,
+constexpr long long RS_OWN_RAMP_CELLS = 65536;     // and arrivals x steps up to which the routing block adds the ramps
 constexpr unsigned int RS_GIVEN = 0x40000000u;
 constexpr unsigned int FULL_MASK = 0xffffffffu;
 
@@ -182,54 +184,25 @@ __device__ __forceinline__ unsigned int first_top(unsigned int near0, unsigned i
     return top;
 }
 
-// One warp per row; block totals of the guards in shared memory first.
-__global__ void __launch_bounds__(SUM_THREADS) pre_summarise_rows(const SumArgs a) {
-    __shared__ unsigned long long sh_guard[GUARDS];
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int row = blockIdx.x * (SUM_THREADS / 32) + (tid >> 5);
-    const int H = a.H;
-    if (tid < GUARDS) sh_guard[tid] = 0;
-    __syncthreads();
-    bool bad = false;
-    if (row < a.I) {
-        const RowNumbers n = row_pass<false, false, true, true>(a.curves + (size_t)row * H, H, 0, 0, a.hot);
-        unsigned int step;
-        const unsigned int first = first_top(n.near0, n.near1, H, step);
-        bad = n.bad;
-        a.near[(size_t)row * 32 + lane] = make_uint2(n.near0, n.near1);
-        a.far[(size_t)row * 32 + lane] = n.far;
-        if (lane == 0) {
-            if (a.over) a.over[row] = n.above;
-            const long long q = a.queued_p[row], d = a.current_d[row];
-            const long long tok = q + d;
-            const bool ok = q >= 0 && d >= 0 && q <= 0xffffffffLL && d <= 0xffffffffLL && tok <= 0xffffffffLL;
-            if (!ok) bad = true;
-            a.summary[row] = make_uint4(ok ? (unsigned int)tok : 0u, n.top, n.jtop | (step << 16), first);
-            if (ok) {
-                atomicMax(sh_guard + GUARD_MAX_BASE, (unsigned long long)tok);
-                atomicAdd(sh_guard + GUARD_SUM_BASE, (unsigned long long)tok);
-            }
-            atomicMax(sh_guard + GUARD_MAX_CELL, (unsigned long long)n.peak);
-        }
-    }
-    if (__any_sync(FULL_MASK, bad) && lane == 0) atomicOr(sh_guard + GUARD_BAD, 1ull);
-    // the arrivals' own totals: what the batch can add to a cell (ramps) and to a row's token count
+// The arrivals' own totals: what the batch can add to a cell (ramps) and to a row's token count.
+template <typename Args>
+__device__ __forceinline__ void batch_totals(const Args& a, long long first, long long stride, unsigned long long* guard) {
     unsigned long long ramp = 0, tokens = 0;
     unsigned int max_pd = 0;
     auto count = [&](int P, int D) {
         if (P < 0 || D < 1 || P > PRE_FIELD_MAX || D > PRE_FIELD_MAX) return;
-        ramp += (unsigned long long)P + (unsigned long long)(D < H ? D : H);
+        ramp += (unsigned long long)P + (unsigned long long)(D < a.H ? D : a.H);
         tokens += (unsigned long long)P + (unsigned long long)D;
         max_pd = max(max_pd, (unsigned int)P + (unsigned int)D);
     };
-    for (long long k = (long long)blockIdx.x * SUM_THREADS + tid; k < a.n_arrivals; k += (long long)gridDim.x * SUM_THREADS)
+    for (long long k = first; k < a.n_arrivals; k += stride)
         count(a.arr_prompt[k], a.arr_predicted[k]);
     if (a.queue_capacity > 0) {   // the waiting requests are routed before the arrivals
         long long q_head = a.queue_state[0], q_len = a.queue_state[1];
         if (q_head < 0 || q_head >= a.queue_capacity) q_head = 0;
         if (q_len < 0) q_len = 0;
         if (q_len > a.queue_capacity) q_len = a.queue_capacity;
-        for (long long k = (long long)blockIdx.x * SUM_THREADS + tid; k < q_len; k += (long long)gridDim.x * SUM_THREADS) {
+        for (long long k = first; k < q_len; k += stride) {
             const long long at = (q_head + k) % a.queue_capacity;
             count(a.queue_prompt[at], a.queue_predicted[at]);
         }
@@ -240,11 +213,51 @@ __global__ void __launch_bounds__(SUM_THREADS) pre_summarise_rows(const SumArgs 
         tokens += __shfl_xor_sync(FULL_MASK, tokens, off);
     }
     max_pd = __reduce_max_sync(FULL_MASK, max_pd);
-    if (lane == 0 && (ramp | tokens)) {
-        atomicAdd(sh_guard + GUARD_SUM_RAMP, ramp);
-        atomicAdd(sh_guard + GUARD_SUM_TOKENS, tokens);
-        atomicMax(sh_guard + GUARD_MAX_PD, (unsigned long long)max_pd);
+    if ((threadIdx.x & 31) == 0 && (ramp | tokens)) {
+        atomicAdd(guard + GUARD_SUM_RAMP, ramp);
+        atomicAdd(guard + GUARD_SUM_TOKENS, tokens);
+        atomicMax(guard + GUARD_MAX_PD, (unsigned long long)max_pd);
     }
+}
+
+// One row by one warp: its first cells and stretches, the guards, and for lane 0 the summary {token count, top,
+// jtop | step of the next << 16, largest c[j] + j of the first steps} and the number of cells above the overload level.
+template <typename Args, typename Put>
+__device__ __forceinline__ void summarise_row(const Args& a, int row, unsigned long long* guard, Put&& put) {
+    const int lane = threadIdx.x & 31, H = a.H;
+    const RowNumbers n = row_pass<false, false, true, true>(a.curves + (size_t)row * H, H, 0, 0, a.hot);
+    unsigned int step;
+    const unsigned int first = first_top(n.near0, n.near1, H, step);
+    bool bad = n.bad;
+    a.near[(size_t)row * 32 + lane] = make_uint2(n.near0, n.near1);
+    a.far[(size_t)row * 32 + lane] = n.far;
+    if (lane == 0) {
+        const long long q = a.queued_p[row], d = a.current_d[row];
+        const long long tok = q + d;
+        const bool ok = q >= 0 && d >= 0 && q <= 0xffffffffLL && d <= 0xffffffffLL && tok <= 0xffffffffLL;
+        if (!ok) bad = true;
+        put(make_uint4(ok ? (unsigned int)tok : 0u, n.top, n.jtop | (step << 16), first), n.above);
+        if (ok) {
+            atomicMax(guard + GUARD_MAX_BASE, (unsigned long long)tok);
+            atomicAdd(guard + GUARD_SUM_BASE, (unsigned long long)tok);
+        }
+        atomicMax(guard + GUARD_MAX_CELL, (unsigned long long)n.peak);
+    }
+    if (__any_sync(FULL_MASK, bad) && lane == 0) atomicOr(guard + GUARD_BAD, 1ull);
+}
+
+// One warp per row; block totals of the guards in shared memory first.
+__global__ void __launch_bounds__(SUM_THREADS) pre_summarise_rows(const SumArgs a) {
+    __shared__ unsigned long long sh_guard[GUARDS];
+    const int tid = threadIdx.x;
+    const int row = blockIdx.x * (SUM_THREADS / 32) + (tid >> 5);
+    if (tid < GUARDS) sh_guard[tid] = 0;
+    __syncthreads();
+    if (row < a.I) summarise_row(a, row, sh_guard, [&](const uint4& q, int above) {
+        a.summary[row] = q;
+        if (a.over) a.over[row] = above;
+    });
+    batch_totals(a, (long long)blockIdx.x * SUM_THREADS + tid, (long long)gridDim.x * SUM_THREADS, sh_guard);
     __syncthreads();
     if (tid < GUARDS) {
         const unsigned long long v = sh_guard[tid];
@@ -281,6 +294,8 @@ struct RouteSumArgs {
     int* status;
     int* give_up;                  // three words that the scanning kernel finds cleared
     int* handled;                  // 1: this kernel routed the batch; 0: the scanning kernel has to
+    int alone;                     // small shapes: nothing is launched before or after this kernel, but for the ramps where
+    int own_ramps;                 // this kernel does not add them itself
     long long* ramps;              // {first table row, rows} whose ramps the maps still lack
     // admission queue (ADMIT kernels only): a ring of waiting requests, entry q at (head + q) mod capacity
     int32_t* queue_prompt;
@@ -1242,6 +1257,91 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     if (lane == 0) st_release(&sh.ctl.z, 1u);
 }
 
+// The batch cell by cell in 64 bits, by the whole block: small shapes whose numbers could leave 32 bits.
+template <bool ADMIT>
+__device__ __noinline__ void rs_literal(const RouteSumArgs& a, RsShared& sh, long long q_head, long long waiting, long long n_items) {
+    __shared__ double best_s[32];
+    __shared__ int best_i[32], n_over[32];
+    __shared__ int win;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5, I = a.I, H = a.H;
+    unsigned int routed = 0;
+    for (long long k = 0; k < n_items; ++k) {
+        int P, D;
+        if (k < waiting) {
+            const long long at = (q_head + k) % a.queue_capacity;
+            P = a.queue_prompt[at]; D = a.queue_predicted[at];
+        } else {
+            P = a.arr_prompt[k - waiting]; D = a.arr_predicted[k - waiting];
+        }
+        const bool bad = P < 0 || D < 1 || P > PRE_FIELD_MAX || D > PRE_FIELD_MAX, full = sh.n0 + routed >= a.max_requests;
+        auto put_result = [&](int c, double s) {
+            if (k < waiting) a.queue_choice[k] = c;
+            else {
+                a.choice[k - waiting] = c;
+                if (a.score) a.score[k - waiting] = s;
+            }
+        };
+        if (bad || full) {
+            if (tid == 0) {
+                put_result(-1, 0.0);
+                int* first = bad ? &sh.first_bad : &sh.first_full;
+                if (k < *first) *first = (int)k;
+            }
+            continue;
+        }
+        const int Dc = D < H ? D : H;
+        double bs = CUDART_INF;
+        int bi = 0x7fffffff, over = 0;
+        for (int row = warp; row < I; row += warps) {
+            const int64_t* src = a.curves + (size_t)row * H;
+            long long peak = -0x7fffffffffffffffLL - 1;
+            int above = 0;
+            for (int j = lane; j < H; j += 32) {
+                const long long c = __ldcg(src + j), v = j < Dc ? c + P + j : c;
+                peak = v > peak ? v : peak;
+                above += c > a.hot;
+            }
+            #pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                const long long other = __shfl_xor_sync(FULL_MASK, peak, off);
+                peak = other > peak ? other : peak;
+            }
+            if (ADMIT) over += (double)__reduce_add_sync(FULL_MASK, above) > a.many;
+            double excess = __dsub_rn((double)peak, a.theta);
+            if (excess < 0.0) excess = 0.0;
+            const double s = __dadd_rn(__dadd_rn((double)(__ldcg(a.queued_p + row) + P), (double)(__ldcg(a.current_d + row) + D)), __dmul_rn(a.beta, excess));
+            if (s < bs || bi == 0x7fffffff) { bs = s; bi = row; }       // a warp's rows ascend
+        }
+        if (lane == 0) { best_s[warp] = bs; best_i[warp] = bi; n_over[warp] = over; }
+        __syncthreads();
+        if (tid == 0) {
+            int all = n_over[0];
+            for (int x = 1; x < warps; ++x) {
+                all += n_over[x];
+                if (best_i[x] < I && (best_s[x] < bs || (best_s[x] == bs && best_i[x] < bi))) { bs = best_s[x]; bi = best_i[x]; }
+            }
+            win = bi;
+            if (ADMIT && all == I) {   // the request is not routed: the batch stops here
+                win = -1;
+                sh.blocked = 1; sh.blocked_k = k;
+            } else {
+                const long long at = sh.n0 + routed;
+                a.prompt[at] = P; a.generated[at] = 0; a.predicted[at] = D; a.instance[at] = bi;
+                a.queued_p[bi] += P;
+                a.current_d[bi] += D;
+                put_result(bi, bs);
+            }
+        }
+        __syncthreads();
+        if (win < 0) break;
+        for (int j = tid; j < Dc; j += blockDim.x) a.curves[(size_t)win * H + j] += P + j;
+        ++routed;
+        __syncthreads();
+    }
+    if (tid == 0) sh.ctl.x = routed;
+    __syncthreads();
+}
+
 // Folding and list warps, warps and threads of the instantiations.
 template <bool LISTS, bool ADMIT> struct Shape {
     static constexpr int FOLD = ADMIT ? 11 : (LISTS ? 6 : 5), LIST = LISTS ? (ADMIT ? 3 : 8) : 0;
@@ -1265,15 +1365,31 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     // (the warp's number by a shuffle: the compiler then knows that the roles part between warps and not within one, and
     // leaves out what would bring the lanes of a warp together again: 157 instead of 202 cycles for a step of the deciding warp)
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(FULL_MASK, tid >> 5, 0);
-    const unsigned long long mc = a.guard[GUARD_MAX_CELL], mb = a.guard[GUARD_MAX_BASE], ramps = a.guard[GUARD_SUM_RAMP],
-                             tokens_in = a.guard[GUARD_SUM_TOKENS], max_pd = a.guard[GUARD_MAX_PD], base_sum = a.guard[GUARD_SUM_BASE];
+    __shared__ unsigned long long sh_guard[GUARDS];
+    const bool alone = !LISTS && a.alone;
+    if (alone) {     // small shapes: what pre_summarise_rows does (kept in the rows' words until the keys' units are known)
+        if (tid < GUARDS) sh_guard[tid] = 0;
+        __syncthreads();
+        for (int i = warp; i < I; i += Sp::WARPS)
+            summarise_row(a, i, sh_guard, [&](const uint4& q, int above) {
+                rows.rec[i] = make_int2((int)q.x, (int)q.w);
+                rows.top[i] = q.y;
+                rows.state[i] = q.z;
+                rows.pending[i] = (unsigned int)above;
+            });
+        batch_totals(a, tid, THREADS, sh_guard);
+        __syncthreads();
+    }
+    const unsigned long long* guard = alone ? sh_guard : a.guard;
+    const unsigned long long mc = guard[GUARD_MAX_CELL], mb = guard[GUARD_MAX_BASE], ramps = guard[GUARD_SUM_RAMP],
+                             tokens_in = guard[GUARD_SUM_TOKENS], max_pd = guard[GUARD_MAX_PD], base_sum = guard[GUARD_SUM_BASE];
     // every cell, every cell + step with a prompt added, and every token count stay below 2^32 all batch long
     // (the ramps of the batch bound what an arrival that is not routed yet can add, too)
     const unsigned long long peak_bound = mc + ramps + (unsigned long long)H;
     if (tid == 0) {
         const unsigned long long token_bound = mb + tokens_in;
         // (and the batch is short enough for 32-bit counters)
-        const bool ok = a.guard[GUARD_BAD] == 0 && peak_bound <= 0xffffffffull && token_bound <= 0xffffffffull &&
+        const bool ok = guard[GUARD_BAD] == 0 && peak_bound <= 0xffffffffull && token_bound <= 0xffffffffull &&
                         a.n_arrivals + (ADMIT ? a.queue_capacity : 0) < (1ll << 26);
         // (whole-number scores: the host has seen to beta and theta)
         const bool exact = !WHOLE || token_bound + max_pd + (unsigned long long)a.beta * (peak_bound + 1) < (1ull << 29);
@@ -1284,6 +1400,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         sh.lists_wanted = sh.lists_ready = sh.list_met = 0;
         sh.list_n[0] = sh.list_n[1] = 0;
         sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0;
+        sh.first_bad = sh.first_full = 0x7fffffff;
     }
     for (int i = tid; i < RS_ITEMS; i += THREADS) sh.items[i] = make_int4(0, 0, 0, 0);    // (an item is fetched before it is known to be there)
     if (tid < RS_MAX_FOLD_WARPS) { sh.done[tid] = (unsigned int)tid; sh.scans_done[tid] = 0; }
@@ -1295,8 +1412,8 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         q_len = a.queue_state[1];
     }
     __syncthreads();
-    if (tid < GUARDS) a.guard[tid] = 0;    // ready for the next call
-    if (sh.mode == 0) {
+    if (tid < GUARDS && !alone) a.guard[tid] = 0;    // ready for the next call
+    if (sh.mode == 0 && !alone) {
         if (tid == 0) {
             *a.handled = 0;
             if (ADMIT) { a.queue_entry[0] = a.queue_state[0]; a.queue_entry[1] = a.queue_state[1]; }
@@ -1310,6 +1427,9 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         if (q_len > a.queue_capacity) q_len = a.queue_capacity;
     }
     const long long n_items = q_len + a.n_arrivals;
+    if (sh.mode == 0) {
+        rs_literal<ADMIT>(a, sh, q_head, q_len, n_items);
+    } else {
     const unsigned long long mean_l = ramps / (unsigned long long)(n_items > 0 ? n_items : 1);
     const int mean = mean_l < (1ull << 22) ? (int)mean_l : 1 << 22;     // prompt + ramp of a typical request
     Scores<WHOLE> sc;
@@ -1322,11 +1442,19 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
             #pragma unroll
             for (int p = 0; p < RS_PROBES; ++p) least[LISTS ? p : 0] = 0x7f000000;
         for (int i = tid; i < I; i += THREADS) {
-            const uint4 q = a.summary0[i];
+            uint4 q;
+            int above = 0;
+            if (alone) {
+                q = make_uint4((unsigned int)rows.rec[i].x, rows.top[i], rows.state[i], (unsigned int)rows.rec[i].y);
+                above = (int)rows.pending[i];
+            } else {
+                q = a.summary0[i];
+                if (ADMIT) above = a.over0[i];
+            }
             const unsigned int jtop = q.z & 0xffffu, step = q.z >> 16;
             const bool far = jtop >= (unsigned int)RS_LIMIT;
             jmax = max(jmax, far ? step : jtop);
-            const bool not_over = ADMIT && !((double)a.over0[i] > a.many);
+            const bool not_over = ADMIT && !((double)above > a.many);
             free_rows += not_over;
             const int2 rec = make_int2(sc.key_a(q.x), sc.key_b(q.x, far ? q.w : q.y));
             rows.rec[i] = rec;
@@ -1365,18 +1493,31 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
             rs_list_loop<LISTS ? Sp::LIST : 3, WHOLE>(sh, rows, sc, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
     }
     __syncthreads();
+    }
     const bool blocked = ADMIT && sh.blocked;
     const long long decided = blocked ? sh.blocked_k : n_items;
     if (tid == 0) {
         *a.n_requests = sh.n0 + sh.ctl.x;
         a.ramps[0] = sh.n0;
-        a.ramps[1] = ADMIT ? 0 : (long long)sh.ctl.x;
+        a.ramps[1] = ADMIT || sh.mode == 0 || a.own_ramps ? 0 : (long long)sh.ctl.x;
         // (what was noted beyond a blocked request is decided again below and does not count here)
         int flags = sh.ctl.w ? PRE_ST_TIMEOUT : 0;
         if (sh.first_bad < decided) flags |= PRE_ST_BADREQ;
         if (sh.first_full < decided) flags |= PRE_ST_CAPACITY;
         if (flags) atomicOr(a.status, flags);
         *a.handled = 1;
+    }
+    if (!LISTS && !ADMIT && a.own_ramps && sh.mode != 0) {     // few ramps: added here
+        for (unsigned int e = warp; e < sh.ctl.x; e += Sp::WARPS) {
+            const long long at = sh.n0 + e;
+            if (a.applied[e]) {
+                if (lane == 0) a.applied[e] = 0;
+                continue;
+            }
+            const int P = a.prompt[at], D = a.predicted[at];
+            unsigned long long* row = reinterpret_cast<unsigned long long*>(a.curves) + (size_t)a.instance[at] * H;
+            for (int j = lane; j < (D < H ? D : H); j += 32) atomicAdd(row + j, (unsigned long long)(P + j));
+        }
     }
     if (ADMIT) {
         // Everything from the blocked request on: a request that was waiting keeps its place; an arrival joins
@@ -1490,6 +1631,13 @@ bool pre_route_summary_admit_fits(const pre_ctx* ctx) {
     return ctx->route_summary_smem_admit != 0 && ctx->d_rs_summary != nullptr && ctx->d_rs_over != nullptr;
 }
 
+// Small shapes: the routing block summarises the rows itself and takes what it would decline cell by cell, so that a batch is
+// one launch (or two: the ramps of a longer batch go to the whole GPU).  A launch costs 4 us of the stream here; reading
+// 32,768 cells by one block costs 3.
+bool pre_route_summary_alone(const pre_ctx* ctx) {
+    return ctx->cfg.n_instances <= RS_DIRECT_ROWS && (long long)ctx->cfg.n_instances * ctx->cfg.horizon <= RS_ALONE_CELLS;
+}
+
 static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const int32_t* arr_prompt,
                               const int32_t* arr_predicted, int64_t n_arrivals, int64_t* curves, int64_t* queued_p,
                               int64_t* current_d, int32_t* prompt, int32_t* generated, int32_t* predicted,
@@ -1512,6 +1660,8 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
     a.theta = ctx->theta; a.beta = ctx->cfg.beta;
     a.summary0 = p.summary; a.guard = p.guard; a.near = p.near; a.far = p.far; a.applied = ctx->d_rs_applied;
     a.status = ctx->d_status; a.handled = ctx->d_rs_handled; a.give_up = ctx->d_abort; a.ramps = ctx->d_rs_ramps;
+    a.alone = pre_route_summary_alone(ctx) ? 1 : 0;
+    a.own_ramps = a.alone && n_arrivals * (long long)H <= RS_OWN_RAMP_CELLS ? 1 : 0;
     a.queue_prompt = nullptr; a.queue_predicted = nullptr; a.queue_state = nullptr; a.queue_entry = nullptr;
     a.queue_capacity = 0; a.queue_choice = nullptr; a.hot = 0; a.many = 0.0; a.over0 = nullptr;
 }
@@ -1519,13 +1669,18 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
 template <bool ADMIT>
 static cudaError_t launch_summary_kernels(pre_ctx* ctx, const SumArgs& p, const RouteSumArgs& a, cudaStream_t s) {
     const int I = ctx->cfg.n_instances;
-    const int rows_per_block = SUM_THREADS / 32;
-    pre_summarise_rows<<<(I + rows_per_block - 1) / rows_per_block, SUM_THREADS, 0, s>>>(p);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    if (!a.alone) {
+        const int rows_per_block = SUM_THREADS / 32;
+        pre_summarise_rows<<<(I + rows_per_block - 1) / rows_per_block, SUM_THREADS, 0, s>>>(p);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     void* params[] = {(void*)&a};
-    return cudaLaunchKernel(summaries_kernel_for<ADMIT>(ctx), dim3(1), dim3(I > RS_DIRECT_ROWS ? Shape<true, ADMIT>::THREADS : Shape<false, ADMIT>::THREADS), params,
+    e = cudaLaunchKernel(summaries_kernel_for<ADMIT>(ctx), dim3(1), dim3(I > RS_DIRECT_ROWS ? Shape<true, ADMIT>::THREADS : Shape<false, ADMIT>::THREADS), params,
                             ADMIT ? ctx->route_summary_smem_admit : ctx->route_summary_smem, s);
+    if (e == cudaSuccess && !ADMIT && a.alone && !a.own_ramps) e = pre_launch_add_ramps(ctx, a.n_arrivals, a.prompt, a.predicted, a.instance, a.curves, s);
+    return e;
 }
 
 cudaError_t pre_launch_route_summary(pre_ctx* ctx, const int32_t* arr_prompt, const int32_t* arr_predicted,
