@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(ROUTE_THREADS, 1) pre_route_persistent(const R
     constexpr int RS_RESIDENT = 1, RS_WIDE = 2;
 
     if (a.done_elsewhere && *a.done_elsewhere) {   // the same word for every block; nobody writes it meanwhile
-        if (!ADMIT) add_ramps(a.ramps, a.applied, a.prompt, a.predicted, a.instance, a.curves, a.H, ROUTE_WARPS);
+        add_ramps(a.ramps, a.applied, a.prompt, a.predicted, a.instance, a.curves, a.H, ROUTE_WARPS);
         return;
     }
     const int G = gridDim.x, b = blockIdx.x;

@@ -18,7 +18,8 @@
 // costs one access by one warp.  While no stretch's bound exceeds the largest of the first steps, top and jtop are exact
 // ("near" rows); the map itself receives all ramps of the batch at the end, in one pass by the whole GPU.  When a bound does
 // exceed it, the row is brought up to date cell by cell and its numbers are taken afresh; a row whose maximum really lies
-// beyond the first steps ("full" rows) gets its ramps at once, as do all rows when the admission queue counts cells.
+// beyond the first steps ("full" rows) gets its ramps at once, as does a row that the bounds leave undecided between overloaded
+// and not (admission queue).
 //
 // Two kernels per batch, and a third for the ramps (pre_route_persistent of route.cu, when it has nothing to route):
 //   pre_summarise_rows   one pass over the maps: the numbers of every row, the rows' token
@@ -50,7 +51,7 @@
 
 namespace {
 
-constexpr int RS_MAX_FOLD_WARPS = 11;
+constexpr int RS_MAX_FOLD_WARPS = 6;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
 constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
 constexpr int RS_LIST_ROWS = 128;           // rows of a list (4 per lane)
@@ -65,7 +66,8 @@ constexpr int RS_MAX_BINARY64_ROWS = 5120;  // and with binary64 scores
 constexpr int SUM_THREADS = 256;
 constexpr unsigned int RS_SPIN_LIMIT = 1u << 24;   // polls of shared memory (some 0.5 s) before a wait inside the block is abandoned
 constexpr int RS_NO_ROW = 0x3fffffff;
-constexpr long long RS_ALONE_CELLS = 32768;        // small shapes: cells of the maps,
+constexpr int RS_ALONE_ROWS = 64;                  // small shapes: instances,
+constexpr long long RS_ALONE_CELLS = 32768;        // cells of the maps,
 constexpr long long RS_OWN_RAMP_CELLS = 65536;     // and arrivals x steps up to which the routing block adds the ramps
 constexpr unsigned int RS_GIVEN = 0x40000000u;
 constexpr unsigned int FULL_MASK = 0xffffffffu;
@@ -220,17 +222,17 @@ __device__ __forceinline__ void batch_totals(const Args& a, long long first, lon
     }
 }
 
-// One row by one warp: its first cells and stretches, the guards, and for lane 0 the summary {token count, top,
+// One row by one warp: its first cells and stretches (to `near`, `far`), the guards, and for lane 0 the summary {token count, top,
 // jtop | step of the next << 16, largest c[j] + j of the first steps} and the number of cells above the overload level.
 template <typename Args, typename Put>
-__device__ __forceinline__ void summarise_row(const Args& a, int row, unsigned long long* guard, Put&& put) {
+__device__ __forceinline__ void summarise_row(const Args& a, int row, uint2* near, unsigned int* far, unsigned long long* guard, Put&& put) {
     const int lane = threadIdx.x & 31, H = a.H;
     const RowNumbers n = row_pass<false, false, true, true>(a.curves + (size_t)row * H, H, 0, 0, a.hot);
     unsigned int step;
     const unsigned int first = first_top(n.near0, n.near1, H, step);
     bool bad = n.bad;
-    a.near[(size_t)row * 32 + lane] = make_uint2(n.near0, n.near1);
-    a.far[(size_t)row * 32 + lane] = n.far;
+    near[(size_t)row * 32 + lane] = make_uint2(n.near0, n.near1);
+    far[(size_t)row * 32 + lane] = n.far;
     if (lane == 0) {
         const long long q = a.queued_p[row], d = a.current_d[row];
         const long long tok = q + d;
@@ -253,7 +255,7 @@ __global__ void __launch_bounds__(SUM_THREADS) pre_summarise_rows(const SumArgs 
     const int row = blockIdx.x * (SUM_THREADS / 32) + (tid >> 5);
     if (tid < GUARDS) sh_guard[tid] = 0;
     __syncthreads();
-    if (row < a.I) summarise_row(a, row, sh_guard, [&](const uint4& q, int above) {
+    if (row < a.I) summarise_row(a, row, a.near, a.far, sh_guard, [&](const uint4& q, int above) {
         a.summary[row] = q;
         if (a.over) a.over[row] = above;
     });
@@ -312,8 +314,8 @@ struct RouteSumArgs {
 // Rows in shared memory (structure of arrays):
 //   rec    {a, b}, even: the score of an arrival is at least max(a, b + what its prompt adds), and that but for the rounding
 //          of the keys unless the row is far or pending
-//   state  jtop | RS_FAR | RS_FULL | RS_DEFERRED (the map lacks ramps) | RS_NOT_OVER (ADMIT: the row was not overloaded when it
-//          was last folded)
+//   state  jtop | RS_FAR | RS_FULL | RS_DEFERRED (the map lacks ramps) | RS_NOT_OVER (ADMIT: the row is not overloaded, as
+//          far as folded)
 //   top, tok   top and token count (whole-number scores: half of a)
 //   pending  1 from the decision for the row to the end of its fold; cleared last
 constexpr unsigned int RS_FAR = 0x40000000u, RS_NOT_OVER = 0x20000000u, RS_FULL = 0x10000000u, RS_DEFERRED = 0x08000000u, RS_JTOP = 0xffffu;
@@ -505,6 +507,13 @@ struct Folder {
         a.near[(size_t)w * 32 + (threadIdx.x & 31)] = make_uint2(n.near0, n.near1);
         a.far[(size_t)w * 32 + (threadIdx.x & 31)] = n.far;
     }
+    // At most so many cells are above the overload level: the first ones counted, a stretch whole if its bound is above.
+    __device__ __forceinline__ int most_above(const RowNumbers& n) {
+        const int lane = threadIdx.x & 31, H = a.H, j = 2 * lane, steps = far_chunks(H) * RS_NEAR, lo = RS_NEAR + lane * steps;
+        int above = (j < H && (long long)n.near0 > a.hot) + (j + 1 < H && (long long)n.near1 > a.hot);
+        if (lo < H && (long long)n.far - lo > a.hot) above += min(steps, H - lo);
+        return __reduce_add_sync(FULL_MASK, above);
+    }
     // Brings the map's row up to date with the requests of the batch below `upto` whose ramps it lacks.
     __device__ __forceinline__ bool catch_up(int w, unsigned int upto) {
         const int lane = threadIdx.x & 31, H = a.H;
@@ -538,7 +547,8 @@ struct Folder {
         if (lane == 0)
             sh.score[e % RS_ITEMS] = summary_score(tokens, (job.x & RS_GIVEN) ? job.y : old_top + (unsigned int)P, (double)P + (double)D, a.theta, a.beta);
         RowNumbers n;
-        bool full = ADMIT || (state & RS_FULL) != 0, deferred = !ADMIT && (state & RS_DEFERRED) != 0;
+        bool full = (state & RS_FULL) != 0, deferred = (state & RS_DEFERRED) != 0;
+        bool not_over = ADMIT && (state & RS_NOT_OVER) != 0;      // (once a row is overloaded it stays so: cells only grow)
         if (!full) {
             const uint2 q = a.near[(size_t)w * 32 + lane];
             n.near0 = q.x; n.near1 = q.y;
@@ -551,25 +561,23 @@ struct Folder {
             const unsigned int t = max(j < H ? n.near0 + (unsigned int)j : 0u, j + 1 < H ? n.near1 + (unsigned int)(j + 1) : 0u);
             n.top = __reduce_max_sync(FULL_MASK, t);
             n.jtop = __reduce_min_sync(FULL_MASK, t == n.top ? (unsigned int)(j + 1 < H ? j + 1 : j) : 0xffffffffu);
-            full = __any_sync(FULL_MASK, n.far > n.top);
+            full = __any_sync(FULL_MASK, n.far > n.top) || (not_over && (double)most_above(n) > a.many);
             if (!full) deferred = true;
         }
         if (full) {
             if (deferred && !catch_up(w, e)) return false;
             deferred = false;
             n = row_pass<true, true, ADMIT, false>(a.curves + (size_t)w * H, H, P, Dc, a.hot);
-            if (!ADMIT) {
-                store_numbers(w, n);
-                if (lane == 0) a.applied[e] = 1;
-                full = n.jtop >= (unsigned int)RS_NEAR;
-            }
+            store_numbers(w, n);
+            if (lane == 0) a.applied[e] = 1;
+            not_over = not_over && !((double)n.above > a.many);
+            full = n.jtop >= (unsigned int)RS_NEAR || (not_over && (double)most_above(n) > a.many);
         }
         const bool far = n.jtop >= (unsigned int)RS_LIMIT;
         unsigned int key_top = n.top, key_step = n.jtop;
         if (far) key_top = first_top(n.near0, n.near1, H, key_step);
         __syncwarp();   // every lane's cells before the row is handed on
         if (lane == 0) {
-            const bool not_over = ADMIT && !((double)n.above > a.many);
             if (key_step > ld_volatile(&sh.jmax)) atomicMax(&sh.jmax, key_step);
             const unsigned int now = tokens + (unsigned int)P + (unsigned int)D;
             rows.top[w] = n.top;
@@ -584,7 +592,7 @@ struct Folder {
     // The peak row w would have with the arrival (P, Dc); the row is not pending.
     __device__ __forceinline__ bool scan(int w, int P, int Dc, unsigned int decided, unsigned int& peak) {
         const int lane = threadIdx.x & 31, H = a.H;
-        if (!ADMIT && (rows.state[w] & RS_DEFERRED)) {
+        if (rows.state[w] & RS_DEFERRED) {
             // the first cells, and what bounds the others: enough when Dc ends among the first and none of the others can be larger
             const uint2 q = a.near[(size_t)w * 32 + lane];
             const int j = 2 * lane, lo = RS_NEAR + lane * far_chunks(H) * RS_NEAR;
@@ -616,7 +624,7 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
             }, LISTS ? 20 : 0))    // (the list warps need the issue slots)
             return;
         acquire_cta();
-        ctl = ld_volatile4(&sh.ctl);
+        if (__all_sync(FULL_MASK, (int)(ctl.x - n) <= 0)) ctl = ld_volatile4(&sh.ctl);
         if (__any_sync(FULL_MASK, (int)(ctl.x - n) > 0)) {
             if (!f.fold(n)) return;
             n += FOLD_WARPS;
@@ -1344,7 +1352,7 @@ __device__ __noinline__ void rs_literal(const RouteSumArgs& a, RsShared& sh, lon
 
 // Folding and list warps, warps and threads of the instantiations.
 template <bool LISTS, bool ADMIT> struct Shape {
-    static constexpr int FOLD = ADMIT ? 11 : (LISTS ? 6 : 5), LIST = LISTS ? (ADMIT ? 3 : 8) : 0;
+    static constexpr int FOLD = LISTS ? 6 : 5, LIST = LISTS ? 8 : 0;
     static constexpr int WARPS = 4 * ((FOLD + 1 + LIST + 2) / 3), THREADS = 32 * WARPS;
 };
 
@@ -1371,7 +1379,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         if (tid < GUARDS) sh_guard[tid] = 0;
         __syncthreads();
         for (int i = warp; i < I; i += Sp::WARPS)
-            summarise_row(a, i, sh_guard, [&](const uint4& q, int above) {
+            summarise_row(a, i, a.near, a.far, sh_guard, [&](const uint4& q, int above) {
                 rows.rec[i] = make_int2((int)q.x, (int)q.w);
                 rows.top[i] = q.y;
                 rows.state[i] = q.z;
@@ -1490,7 +1498,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         else if (role == Sp::FOLD)
             rs_io_loop<Sp::FOLD, ADMIT, WHOLE>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
         else if (LISTS && role <= Sp::FOLD + Sp::LIST)
-            rs_list_loop<LISTS ? Sp::LIST : 3, WHOLE>(sh, rows, sc, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
+            rs_list_loop<LISTS ? Sp::LIST : 8, WHOLE>(sh, rows, sc, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
     }
     __syncthreads();
     }
@@ -1499,7 +1507,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     if (tid == 0) {
         *a.n_requests = sh.n0 + sh.ctl.x;
         a.ramps[0] = sh.n0;
-        a.ramps[1] = ADMIT || sh.mode == 0 || a.own_ramps ? 0 : (long long)sh.ctl.x;
+        a.ramps[1] = sh.mode == 0 || a.own_ramps ? 0 : (long long)sh.ctl.x;
         // (what was noted beyond a blocked request is decided again below and does not count here)
         int flags = sh.ctl.w ? PRE_ST_TIMEOUT : 0;
         if (sh.first_bad < decided) flags |= PRE_ST_BADREQ;
@@ -1507,7 +1515,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         if (flags) atomicOr(a.status, flags);
         *a.handled = 1;
     }
-    if (!LISTS && !ADMIT && a.own_ramps && sh.mode != 0) {     // few ramps: added here
+    if (!LISTS && a.own_ramps && sh.mode != 0) {     // few ramps: added here
         for (unsigned int e = warp; e < sh.ctl.x; e += Sp::WARPS) {
             const long long at = sh.n0 + e;
             if (a.applied[e]) {
@@ -1632,10 +1640,10 @@ bool pre_route_summary_admit_fits(const pre_ctx* ctx) {
 }
 
 // Small shapes: the routing block summarises the rows itself and takes what it would decline cell by cell, so that a batch is
-// one launch (or two: the ramps of a longer batch go to the whole GPU).  A launch costs 4 us of the stream here; reading
-// 32,768 cells by one block costs 3.
+// one launch (or two: the ramps of a longer batch go to the whole GPU).  A launch costs 4 us of the stream here; the block's
+// warps take 0.8 us per row (64 rows: as long as the launch; 256 rows: 25 us more than it).
 bool pre_route_summary_alone(const pre_ctx* ctx) {
-    return ctx->cfg.n_instances <= RS_DIRECT_ROWS && (long long)ctx->cfg.n_instances * ctx->cfg.horizon <= RS_ALONE_CELLS;
+    return ctx->cfg.n_instances <= RS_ALONE_ROWS && (long long)ctx->cfg.n_instances * ctx->cfg.horizon <= RS_ALONE_CELLS;
 }
 
 static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const int32_t* arr_prompt,
@@ -1679,7 +1687,7 @@ static cudaError_t launch_summary_kernels(pre_ctx* ctx, const SumArgs& p, const 
     void* params[] = {(void*)&a};
     e = cudaLaunchKernel(summaries_kernel_for<ADMIT>(ctx), dim3(1), dim3(I > RS_DIRECT_ROWS ? Shape<true, ADMIT>::THREADS : Shape<false, ADMIT>::THREADS), params,
                             ADMIT ? ctx->route_summary_smem_admit : ctx->route_summary_smem, s);
-    if (e == cudaSuccess && !ADMIT && a.alone && !a.own_ramps) e = pre_launch_add_ramps(ctx, a.n_arrivals, a.prompt, a.predicted, a.instance, a.curves, s);
+    if (e == cudaSuccess && a.alone && !a.own_ramps) e = pre_launch_add_ramps(ctx, a.n_arrivals + a.queue_capacity, a.prompt, a.predicted, a.instance, a.curves, s);
     return e;
 }
 
@@ -1712,5 +1720,6 @@ cudaError_t pre_launch_route_summary_admit(pre_ctx* ctx, const int32_t* arr_prom
     a.queue_prompt = queue_prompt; a.queue_predicted = queue_predicted; a.queue_state = queue_state;
     a.queue_entry = ctx->d_queue_entry; a.queue_capacity = queue_capacity; a.queue_choice = queue_choice;
     a.hot = hot; a.many = many; a.over0 = ctx->d_rs_over;
+    a.own_ramps = a.alone && (n_arrivals + queue_capacity) * (long long)a.H <= RS_OWN_RAMP_CELLS ? 1 : 0;
     return launch_summary_kernels<true>(ctx, p, a, s);
 }
