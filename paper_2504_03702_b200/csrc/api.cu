@@ -28,6 +28,7 @@ void release(pre_ctx* c) {
     cudaFree(c->d_slots);
     cudaFree(c->d_enter);
     cudaFree(c->d_active);
+    cudaFree(c->d_tally);
     cudaFree(c->d_scaler_partial);
     cudaFree(c->d_scaler_done);
     cudaFree(c->d_ring_done);
@@ -109,7 +110,8 @@ int pre_create(const pre_config* cfg, pre_ctx** out) {
     if (e == cudaSuccess) e = alloc_zero(&c->d_fused_base, (size_t)c->n_tiles + 1);
     if (e == cudaSuccess) e = alloc_zero(&c->d_fused_sync, 8);
     if (e == cudaSuccess) e = alloc_zero(&c->d_enter, (size_t)I);
-    if (e == cudaSuccess) e = alloc_zero(&c->d_active, (size_t)I);
+    if (e == cudaSuccess) e = alloc_zero(&c->d_active, (size_t)I + 1);
+    if (e == cudaSuccess) e = alloc_zero(&c->d_tally, 3);
     if (e == cudaSuccess) e = alloc_zero(&c->d_scaler_partial, (size_t)16 * c->n_sm * 3);
     if (e == cudaSuccess) e = alloc_zero(&c->d_scaler_done, 1);
     if (e == cudaSuccess) e = alloc_zero(&c->d_ring_done, 1);

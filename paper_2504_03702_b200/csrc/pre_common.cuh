@@ -48,7 +48,8 @@ struct pre_ctx {
     unsigned long long* d_records;  // [max_requests]
     unsigned long long* d_slots;    // [2][G][16] routing exchange, one 128-byte line per block and parity
     unsigned long long* d_enter;    // [I] tokens entering the window at step H-1 (zero between calls)
-    unsigned int* d_active;         // [I] live requests per instance (zero between calls)
+    unsigned int* d_active;         // [I, rounded up to even] live requests per instance (zero between calls)
+    unsigned long long* d_tally;    // [3] events of the refinement (zero between calls)
     long long* d_scaler_partial;    // [16 * n_sm][3] block totals of the kernels that sum the scaler's signals
     unsigned int* d_scaler_done;    // blocks of that kernel that have finished (zero between calls)
     unsigned int* d_ring_done;      // the same for the kernel that advances a ring of maps
@@ -156,6 +157,15 @@ cudaError_t pre_launch_anticipate_fused(pre_ctx* ctx, const int32_t* prompt, con
                                         int64_t* curves, int64_t* current_d, cudaStream_t s);
 cudaError_t pre_fused_reset(pre_ctx* ctx, cudaStream_t s);   // after a wait ran out
 constexpr unsigned int PRE_DEFAULT_SPIN_LIMIT = 1u << 22;
+
+// Adds a block's counts per instance to the global ones, two counts per 64-bit addition (a count stays below 2^31, so
+// nothing carries over): every block adds every instance's count, which is 1.2 million additions with 4,096 instances.
+__device__ __forceinline__ void pre_flush_counts(const unsigned int* sh, unsigned int* global, int I) {
+    for (int i = 2 * threadIdx.x; i < I; i += 2 * blockDim.x) {
+        const unsigned int lo = sh[i], hi = i + 1 < I ? sh[i + 1] : 0u;
+        if (lo | hi) atomicAdd(reinterpret_cast<unsigned long long*>(global + i), ((unsigned long long)hi << 32) | lo);
+    }
+}
 
 __device__ __forceinline__ bool pre_request_ok(int32_t P, int32_t g, int32_t D, int32_t inst, int32_t I) {
     return P >= 0 && g >= 0 && D >= 1 && inst >= 0 && inst < I;

@@ -68,10 +68,7 @@ pre_step_requests(const int32_t* __restrict__ prompt, int32_t* __restrict__ gene
     }
     if (use_sh) {
         __syncthreads();
-        for (int i = threadIdx.x; i < I; i += blockDim.x) {
-            const unsigned int c = sh_active[i];
-            if (c) atomicAdd(&active[i], c);
-        }
+        pre_flush_counts(sh_active, active, I);
     }
     if (any_bad) atomicOr(status, PRE_ST_BADREQ);
 }

@@ -38,7 +38,7 @@ pre_tick_requests(const int32_t* __restrict__ prompt, int32_t* __restrict__ gene
                   const int32_t* __restrict__ instance, const int32_t* __restrict__ actual,
                   const int64_t* __restrict__ n_requests, long long max_requests, int I, int H,
                   int64_t* __restrict__ curves, int64_t* __restrict__ current_d, unsigned int* __restrict__ active,
-                  unsigned long long* __restrict__ enter, unsigned long long* __restrict__ counts,
+                  unsigned long long* __restrict__ enter, unsigned long long* __restrict__ tally,
                   long long* __restrict__ summary, int* __restrict__ status) {
     extern __shared__ unsigned int sh_active[];
     __shared__ unsigned int sh_tally[3];
@@ -84,7 +84,7 @@ pre_tick_requests(const int32_t* __restrict__ prompt, int32_t* __restrict__ gene
             }
         }
         int32_t g1[4];
-        bool moved = false;
+        bool moved = false, refined = false;
         #pragma unroll
         for (int e = 0; e < 4; ++e) {
             g1[e] = g[e];
@@ -131,23 +131,21 @@ pre_tick_requests(const int32_t* __restrict__ prompt, int32_t* __restrict__ gene
             }
             if (kind != 0) {
                 D[e] = new_d;
-                moved = true;
+                refined = true;
                 const long long delta = kind == 1 ? -(long long)steps : (long long)steps;
                 atomicAdd(reinterpret_cast<unsigned long long*>(current_d + inst[e]), (unsigned long long)delta);
                 if (kind == 1) ++n_early; else ++n_ext;
             }
         }
-        if (moved) {
-            if (vec && r0 + 4 <= n) {
-                *reinterpret_cast<int4*>(generated + r0) = make_int4(g1[0], g1[1], g1[2], g1[3]);
-                if (actual) *reinterpret_cast<int4*>(predicted + r0) = make_int4(D[0], D[1], D[2], D[3]);
-            } else {
-                #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if (r0 + e < n) {
-                        generated[r0 + e] = g1[e];
-                        if (actual) predicted[r0 + e] = D[e];
-                    }
+        if (vec && r0 + 4 <= n) {
+            if (moved) *reinterpret_cast<int4*>(generated + r0) = make_int4(g1[0], g1[1], g1[2], g1[3]);
+            if (refined) *reinterpret_cast<int4*>(predicted + r0) = make_int4(D[0], D[1], D[2], D[3]);
+        } else if (moved || refined) {
+            #pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (r0 + e < n) {
+                    generated[r0 + e] = g1[e];
+                    if (refined) predicted[r0 + e] = D[e];
                 }
             }
         }
@@ -161,14 +159,9 @@ pre_tick_requests(const int32_t* __restrict__ prompt, int32_t* __restrict__ gene
         if (n_bad) atomicAdd(&sh_tally[2], n_bad);
     }
     __syncthreads();
-    if (use_sh) {
-        for (int i = threadIdx.x; i < I; i += blockDim.x) {
-            const unsigned int c = sh_active[i];
-            if (c) atomicAdd(&active[i], c);
-        }
-    }
+    if (use_sh) pre_flush_counts(sh_active, active, I);
     if (threadIdx.x < 3 && sh_tally[threadIdx.x]) {
-        if (counts) atomicAdd(&counts[threadIdx.x], (unsigned long long)sh_tally[threadIdx.x]);
+        atomicAdd(&tally[threadIdx.x], (unsigned long long)sh_tally[threadIdx.x]);
         if (threadIdx.x == 2) atomicOr(status, PRE_ST_BADREQ);
     }
     if (any_bad) atomicOr(status, PRE_ST_BADREQ);
@@ -180,7 +173,12 @@ __global__ void __launch_bounds__(SHIFT_THREADS)
 pre_tick_shift(int64_t* __restrict__ curves, int64_t* __restrict__ queued_p, int64_t* __restrict__ current_d,
                unsigned int* __restrict__ active, unsigned long long* __restrict__ enter, int I, int H,
                long long hot, double many, double idle, int32_t* __restrict__ over_count,
-               int64_t* __restrict__ row_max, long long* __restrict__ summary) {
+               int64_t* __restrict__ row_max, long long* __restrict__ summary, unsigned long long* __restrict__ tally,
+               int64_t* __restrict__ counts) {
+    if (blockIdx.x == 0 && threadIdx.x < 3) {     // what the table pass counted, and zero for the next call
+        if (counts) counts[threadIdx.x] = (int64_t)tally[threadIdx.x];
+        tally[threadIdx.x] = 0;
+    }
     __shared__ int sh_cnt[2][SHIFT_WARPS];          // per-warp partials of a row, by parity of the block's row count:
     __shared__ long long sh_max[2][SHIFT_WARPS];    // thread 0 adds them up one row later, after the barrier that ends the row
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -251,10 +249,6 @@ cudaError_t pre_launch_tick(pre_ctx* ctx, int32_t* prompt, int32_t* generated, i
                             int64_t* current_d, double overload_level, double overload_share, double idle_level,
                             int32_t* over_count, int64_t* row_max, int64_t* summary, int64_t* counts, cudaStream_t s) {
     const int I = ctx->cfg.n_instances, H = ctx->cfg.horizon;
-    if (counts) {
-        cudaError_t e = cudaMemsetAsync(counts, 0, 3 * sizeof(int64_t), s);
-        if (e != cudaSuccess) return e;
-    }
     const size_t smem = I <= PRE_SMEM_BINS ? (size_t)I * sizeof(unsigned int) : 0;
     long long want = (ctx->cfg.max_requests + TICK_THREADS * 4 - 1) / (TICK_THREADS * 4);
     // two blocks per SM: every block flushes its live counts with one global atomic per instance
@@ -262,7 +256,7 @@ cudaError_t pre_launch_tick(pre_ctx* ctx, int32_t* prompt, int32_t* generated, i
     if (grid < 1) grid = 1;
     pre_tick_requests<<<grid, TICK_THREADS, smem, s>>>(prompt, generated, predicted, instance, actual, n_requests,
                                                       ctx->cfg.max_requests, I, H, curves, current_d, ctx->d_active,
-                                                      ctx->d_enter, reinterpret_cast<unsigned long long*>(counts),
+                                                      ctx->d_enter, ctx->d_tally,
                                                       reinterpret_cast<long long*>(summary), ctx->d_status);
     // For a whole number c, c > x holds exactly when c > floor(x): the per-cell test is done on integers.
     double hot_d = floor(overload_level * (double)ctx->cfg.capacity_tokens);
@@ -273,6 +267,6 @@ cudaError_t pre_launch_tick(pre_ctx* ctx, int32_t* prompt, int32_t* generated, i
     int sgrid = I < 16 * ctx->n_sm ? I : 16 * ctx->n_sm;
     pre_tick_shift<<<sgrid, SHIFT_THREADS, 0, s>>>(curves, queued_p, current_d, ctx->d_active, ctx->d_enter, I, H,
                                                   (long long)hot_d, many, idle, over_count, row_max,
-                                                  reinterpret_cast<long long*>(summary));
+                                                  reinterpret_cast<long long*>(summary), ctx->d_tally, counts);
     return cudaGetLastError();
 }
