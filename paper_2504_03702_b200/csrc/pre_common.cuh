@@ -167,6 +167,24 @@ __device__ __forceinline__ void pre_flush_counts(const unsigned int* sh, unsigne
     }
 }
 
+// Two kernels of one call, the second launched while the first still runs: its blocks take their places as the first one's
+// leave, and wait there until the first has finished and its writes are visible.  (A launch behind a finished kernel
+// costs the stream 1 to 2 us.)  The first kernel says pre_let_next_start(), the second pre_wait_for_previous() before it
+// touches memory.
+__device__ __forceinline__ void pre_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pre_wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... Params, typename... Args>
+cudaError_t pre_launch_behind(void (*kernel)(Params...), int grid, int block, size_t smem, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned int)grid); cfg.blockDim = dim3((unsigned int)block);
+    cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 __device__ __forceinline__ bool pre_request_ok(int32_t P, int32_t g, int32_t D, int32_t inst, int32_t I) {
     return P >= 0 && g >= 0 && D >= 1 && inst >= 0 && inst < I;
 }

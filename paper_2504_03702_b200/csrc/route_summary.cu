@@ -251,6 +251,7 @@ __device__ __forceinline__ void summarise_row(const Args& a, int row, uint2* nea
 // One warp per row; block totals of the guards in shared memory first.
 __global__ void __launch_bounds__(SUM_THREADS) pre_summarise_rows(const SumArgs a) {
     __shared__ unsigned long long sh_guard[GUARDS];
+    pre_let_next_start();
     const int tid = threadIdx.x;
     const int row = blockIdx.x * (SUM_THREADS / 32) + (tid >> 5);
     if (tid < GUARDS) sh_guard[tid] = 0;
@@ -1375,6 +1376,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(FULL_MASK, tid >> 5, 0);
     __shared__ unsigned long long sh_guard[GUARDS];
     const bool alone = !LISTS && a.alone;
+    if (!alone) pre_wait_for_previous();
     if (alone) {     // small shapes: what pre_summarise_rows does (kept in the rows' words until the keys' units are known)
         if (tid < GUARDS) sh_guard[tid] = 0;
         __syncthreads();
@@ -1684,9 +1686,16 @@ static cudaError_t launch_summary_kernels(pre_ctx* ctx, const SumArgs& p, const 
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    void* params[] = {(void*)&a};
-    e = cudaLaunchKernel(summaries_kernel_for<ADMIT>(ctx), dim3(1), dim3(I > RS_DIRECT_ROWS ? Shape<true, ADMIT>::THREADS : Shape<false, ADMIT>::THREADS), params,
-                            ADMIT ? ctx->route_summary_smem_admit : ctx->route_summary_smem, s);
+    typedef void (*Kernel)(const RouteSumArgs);
+    const Kernel kernel = reinterpret_cast<Kernel>(const_cast<void*>(summaries_kernel_for<ADMIT>(ctx)));
+    const int threads = I > RS_DIRECT_ROWS ? Shape<true, ADMIT>::THREADS : Shape<false, ADMIT>::THREADS;
+    const size_t smem = ADMIT ? ctx->route_summary_smem_admit : ctx->route_summary_smem;
+    if (a.alone) {
+        kernel<<<1, threads, smem, s>>>(a);
+        e = cudaGetLastError();
+    } else {
+        e = pre_launch_behind(kernel, 1, threads, smem, s, a);
+    }
     if (e == cudaSuccess && a.alone && !a.own_ramps) e = pre_launch_add_ramps(ctx, a.n_arrivals + a.queue_capacity, a.prompt, a.predicted, a.instance, a.curves, s);
     return e;
 }

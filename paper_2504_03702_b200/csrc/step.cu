@@ -20,6 +20,7 @@ pre_step_requests(const int32_t* __restrict__ prompt, int32_t* __restrict__ gene
                   unsigned int* __restrict__ active, unsigned long long* __restrict__ enter,
                   int* __restrict__ status) {
     extern __shared__ unsigned int sh_active[];
+    pre_let_next_start();
     const bool use_sh = I <= PRE_SMEM_BINS;
     long long n = *n_requests;
     if (n > max_requests) n = max_requests;
@@ -78,6 +79,7 @@ pre_step_requests(const int32_t* __restrict__ prompt, int32_t* __restrict__ gene
 __global__ void __launch_bounds__(SHIFT_THREADS)
 pre_step_shift(int64_t* __restrict__ curves, int64_t* __restrict__ queued_p, int64_t* __restrict__ current_d,
                unsigned int* __restrict__ active, unsigned long long* __restrict__ enter, int I, int H) {
+    pre_wait_for_previous();
     for (int row = blockIdx.x; row < I; row += gridDim.x) {
         int64_t* rp = curves + (size_t)row * H;
         const long long last = (long long)enter[row];
@@ -130,6 +132,6 @@ cudaError_t pre_launch_step(pre_ctx* ctx, int32_t* prompt, int32_t* generated, i
     cudaError_t e = pre_launch_step_requests(ctx, prompt, generated, predicted, instance, n_requests, H, s);
     if (e != cudaSuccess) return e;
     int sgrid = I < 16 * ctx->n_sm ? I : 16 * ctx->n_sm;
-    pre_step_shift<<<sgrid, SHIFT_THREADS, 0, s>>>(curves, queued_p, current_d, ctx->d_active, ctx->d_enter, I, H);
-    return cudaGetLastError();
+    return pre_launch_behind(pre_step_shift, sgrid, SHIFT_THREADS, 0, s, curves, queued_p, current_d, ctx->d_active,
+                             ctx->d_enter, I, H);
 }

@@ -42,6 +42,7 @@ pre_tick_requests(const int32_t* __restrict__ prompt, int32_t* __restrict__ gene
                   long long* __restrict__ summary, int* __restrict__ status) {
     extern __shared__ unsigned int sh_active[];
     __shared__ unsigned int sh_tally[3];
+    pre_let_next_start();
     const bool use_sh = I <= PRE_SMEM_BINS;
     long long n = *n_requests;
     if (n > max_requests) n = max_requests;
@@ -175,6 +176,7 @@ pre_tick_shift(int64_t* __restrict__ curves, int64_t* __restrict__ queued_p, int
                long long hot, double many, double idle, int32_t* __restrict__ over_count,
                int64_t* __restrict__ row_max, long long* __restrict__ summary, unsigned long long* __restrict__ tally,
                int64_t* __restrict__ counts) {
+    pre_wait_for_previous();
     if (blockIdx.x == 0 && threadIdx.x < 3) {     // what the table pass counted, and zero for the next call
         if (counts) counts[threadIdx.x] = (int64_t)tally[threadIdx.x];
         tally[threadIdx.x] = 0;
@@ -265,8 +267,9 @@ cudaError_t pre_launch_tick(pre_ctx* ctx, int32_t* prompt, int32_t* generated, i
     const double many = overload_share * (double)H;
     const double idle = idle_level * (double)ctx->cfg.capacity_tokens;
     int sgrid = I < 16 * ctx->n_sm ? I : 16 * ctx->n_sm;
-    pre_tick_shift<<<sgrid, SHIFT_THREADS, 0, s>>>(curves, queued_p, current_d, ctx->d_active, ctx->d_enter, I, H,
-                                                  (long long)hot_d, many, idle, over_count, row_max,
-                                                  reinterpret_cast<long long*>(summary), ctx->d_tally, counts);
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return pre_launch_behind(pre_tick_shift, sgrid, SHIFT_THREADS, 0, s, curves, queued_p, current_d, ctx->d_active,
+                             ctx->d_enter, I, H, (long long)hot_d, many, idle, over_count, row_max,
+                             reinterpret_cast<long long*>(summary), ctx->d_tally, counts);
 }
