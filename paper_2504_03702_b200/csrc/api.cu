@@ -73,16 +73,17 @@ int pre_create(const pre_config* cfg, pre_ctx** out) {
     c->theta = cfg->t_mem * (double)cfg->capacity_tokens;
 
     cudaError_t e = cudaGetDevice(&c->device);
-    cudaDeviceProp prop;
-    if (e == cudaSuccess) e = cudaGetDeviceProperties(&prop, c->device);
+    // (single attributes: a whole cudaDeviceProp takes 2.5 ms to fill)
+    int smem_limit = 0;
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
     if (e != cudaSuccess) { delete c; return PRE_ECUDA; }
-    c->n_sm = prop.multiProcessorCount;
 
     const int I = cfg->n_instances, H = cfg->horizon;
     const int t = pre_tile_rows_for(I, H, c->n_sm);
     c->tile_rows = t;
     c->n_tiles = (I + t - 1) / t;
-    if (pre_tile_smem_bytes(t, H) > (size_t)prop.sharedMemPerBlockOptin) { delete c; return PRE_EINVAL; }
+    if (pre_tile_smem_bytes(t, H) > (size_t)smem_limit) { delete c; return PRE_EINVAL; }
 
     e = alloc_zero(&c->d_status, 8);     // status | give-up flag, agreed exchange, blocks met | . | exchange counter
     c->d_abort = c->d_status ? c->d_status + 1 : nullptr;

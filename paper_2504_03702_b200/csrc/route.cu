@@ -1042,10 +1042,10 @@ cudaError_t pre_route_configure(pre_ctx* ctx) {
     const int I = ctx->cfg.n_instances;
     const int G = ctx->n_sm < I ? ctx->n_sm : I;  // one block per SM, never more blocks than rows
     const int max_rows = (I + G - 1) / G;
-    cudaDeviceProp prop;
-    cudaError_t e = cudaGetDeviceProperties(&prop, ctx->device);
+    int smem_limit = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&smem_limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
     if (e != cudaSuccess) return e;
-    const size_t limit = (size_t)prop.sharedMemPerBlockOptin;
+    const size_t limit = (size_t)smem_limit;
     e = configure_one<false>(ctx, G, max_rows, limit, &ctx->route_smem, &ctx->route_resident_bytes);
     if (e != cudaSuccess) return e;
     e = configure_one<true>(ctx, G, max_rows, limit, &ctx->route_smem_admit, &ctx->route_resident_bytes_admit);

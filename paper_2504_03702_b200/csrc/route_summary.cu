@@ -54,7 +54,8 @@ namespace {
 constexpr int RS_MAX_FOLD_WARPS = 6;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
 constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
-constexpr int RS_LIST_ROWS = 128;           // rows of a list (4 per lane)
+constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lane, 8 beyond RS_LONG_LISTS instances)
+constexpr int RS_LONG_LISTS = 2048;
 constexpr int RS_NEAR_ROWS = 2304;          // rows the list warps keep for a closer look at once
 constexpr int RS_PROBES = 8;                // prompt lengths for which a list has the best rows
 constexpr int RS_NEAR = 64;                 // steps kept exactly; the rest in 32 stretches of whole chunks of as many steps
@@ -736,7 +737,7 @@ __device__ __forceinline__ int rs_probe(int mean, int x) {
     return (int)((float)mean * share[x]);
 }
 
-template <int LIST_WARPS, bool WHOLE>
+template <int LIST_WARPS, int ROOM, bool WHOLE>
 __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int I, int mean, int longest, int t) {
     constexpr int THREADS = 32 * LIST_WARPS, NEAR_ROOM = RS_NEAR_ROWS / LIST_WARPS;
     constexpr int FAR_KEY = 0x7f000000, AT_ONCE = 4;      // AT_ONCE: rows a thread has on their way
@@ -827,7 +828,7 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
                         int at = 0;
                         if (lane == 0) at = atomicAdd(&sh.list_count, __popc(vote));
                         at = __shfl_sync(FULL_MASK, at, 0) + __popc(vote & ((1u << lane) - 1u));
-                        if (take && at < RS_LIST_ROWS) sh.list_row[now][at] = i;
+                        if (take && at < ROOM) sh.list_row[now][at] = i;
                     }
                     if (in && !take) {
                         const int c = sc.row_code(r);
@@ -865,7 +866,7 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
             if (lane == 0) { atomicMin(&sh.bucket_b[0], ordered(hb)); atomicMin(&sh.bucket_a[31], ordered(ca)); }
             if (!team()) return;
             const int count = sh.list_count;
-            if (count > RS_LIST_ROWS) { margin = max(margin / 2, least_margin); if (tries > 4) margin = 0; if (!team()) return; continue; }
+            if (count > ROOM) { margin = max(margin / 2, least_margin); if (tries > 4) margin = 0; if (!team()) return; continue; }
             if (leader) {
                 // (a key that no row has set is out of reach; rows of code 31 count by their a alone, no b is kept for them)
                 const int ka = unordered(min(sh.bucket_a[lane], ordered(RS_ABSENT)));
@@ -891,7 +892,7 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
                 __syncwarp();
                 if (lane == 0) st_release(&sh.lists_ready, n);
             }
-            if (count < RS_LIST_ROWS * 3 / 5) margin = min(margin + margin / 2 + 1, 1 << 27);
+            if (count < ROOM * 3 / 5) margin = min(margin + margin / 2 + 1, 1 << 27);
             break;
         }
     }
@@ -1001,6 +1002,15 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         const int2 pd = sh.raw[e % RS_ITEMS];
         const int P = pd.x, D = pd.y, Dc = D < H ? D : H, kp = it.x, kpd = it.y;
         publish(e);
+        auto received = [&](int win) {     // the arrival's ramp reaches the step of the row's b
+            #pragma unroll
+            for (int k = 0; k < KS; ++k)
+                if (row[k] == win) {
+                    const int marked = ra[k] & 1;
+                    ra[k] += kpd + marked;
+                    rb[k] += kpd + (marked ? 1 : kp);
+                }
+        };
         for (int lists_tried = 0;;) {
             refresh();
             if (it.z <= jmax) break;
@@ -1059,19 +1069,36 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             const S best = Scores<WHOLE>::warp_min(mine);
             const int win = __reduce_min_sync(FULL_MASK, mine == best ? mine_row : NO_ROW);
             if (win >= I) break;
-            #pragma unroll
-            for (int k = 0; k < KS; ++k)
-                if (row[k] == win) {
-                    const int marked = ra[k] & 1;
-                    ra[k] += kpd + marked;
-                    rb[k] += kpd + (marked ? 1 : kp);
-                }
+            received(win);
             tell(e, win, win, 0u);
             return;
         }
         // ---- short arrivals and rows that have to be scanned: all rows, with every fold done.  First those with exact scores ...
         if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return; }
         acquire_cta();
+        jmax = (int)ld_volatile(&sh.jmax);
+        if (WHOLE && it.z > jmax) {
+            // no list covers it, but its ramp reaches every row's step: the keys give the scores of all rows that are not far
+            // (4,096 rows: 3,000 cycles, 28,000 for what follows)
+            int least = RS_ABSENT, least_row = RS_NO_ROW;
+            for (int g0 = 0; g0 < n_groups; g0 += 8) {
+                int2 r[8];
+                #pragma unroll
+                for (int u = 0; u < 8; ++u) r[u] = (g0 + u) * 32 + lane < I ? rows.rec[(g0 + u) * 32 + lane] : make_int2(RS_ABSENT, RS_LOWEST);
+                #pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int v = __viaddmax_s32(r[u].y, kp, r[u].x);
+                    if (v < least) { least = v; least_row = (g0 + u) * 32 + lane; }     // a lane's rows ascend
+                }
+            }
+            const int best = __reduce_min_sync(FULL_MASK, least);
+            const int win = __reduce_min_sync(FULL_MASK, least == best ? least_row : RS_NO_ROW);
+            if (win < I && !__any_sync(FULL_MASK, (rows.state[win] & RS_FAR) != 0)) {
+                received(win);
+                tell(e, win, win, 0u);
+                return;
+            }
+        }
         auto look = [&](int i, S& s, unsigned int& tokens, unsigned int& peak) {   // whether row i's score is exact, and the score (else a lower bound)
             s = Scores<WHOLE>::none();
             tokens = peak = 0;
@@ -1423,7 +1450,8 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     }
     __syncthreads();
     if (tid < GUARDS && !alone) a.guard[tid] = 0;    // ready for the next call
-    if (sh.mode == 0 && !alone) {
+    const int mode = __shfl_sync(FULL_MASK, sh.mode, 0);     // (all threads alike, and known to be)
+    if (mode == 0 && !alone) {
         if (tid == 0) {
             *a.handled = 0;
             if (ADMIT) { a.queue_entry[0] = a.queue_state[0]; a.queue_entry[1] = a.queue_state[1]; }
@@ -1437,7 +1465,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         if (q_len > a.queue_capacity) q_len = a.queue_capacity;
     }
     const long long n_items = q_len + a.n_arrivals;
-    if (sh.mode == 0) {
+    if (mode == 0) {
         rs_literal<ADMIT>(a, sh, q_head, q_len, n_items);
     } else {
     const unsigned long long mean_l = ramps / (unsigned long long)(n_items > 0 ? n_items : 1);
@@ -1500,7 +1528,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         else if (role == Sp::FOLD)
             rs_io_loop<Sp::FOLD, ADMIT, WHOLE>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
         else if (LISTS && role <= Sp::FOLD + Sp::LIST)
-            rs_list_loop<LISTS ? Sp::LIST : 8, WHOLE>(sh, rows, sc, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
+            rs_list_loop<LISTS ? Sp::LIST : 8, 32 * KS, WHOLE>(sh, rows, sc, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
     }
     __syncthreads();
     }
@@ -1509,7 +1537,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     if (tid == 0) {
         *a.n_requests = sh.n0 + sh.ctl.x;
         a.ramps[0] = sh.n0;
-        a.ramps[1] = sh.mode == 0 || a.own_ramps ? 0 : (long long)sh.ctl.x;
+        a.ramps[1] = mode == 0 || a.own_ramps ? 0 : (long long)sh.ctl.x;
         // (what was noted beyond a blocked request is decided again below and does not count here)
         int flags = sh.ctl.w ? PRE_ST_TIMEOUT : 0;
         if (sh.first_bad < decided) flags |= PRE_ST_BADREQ;
@@ -1517,7 +1545,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         if (flags) atomicOr(a.status, flags);
         *a.handled = 1;
     }
-    if (!LISTS && a.own_ramps && sh.mode != 0) {     // few ramps: added here
+    if (!LISTS && a.own_ramps && mode != 0) {     // few ramps: added here
         for (unsigned int e = warp; e < sh.ctl.x; e += Sp::WARPS) {
             const long long at = sh.n0 + e;
             if (a.applied[e]) {
@@ -1599,7 +1627,8 @@ static const void* summaries_kernel(int I) {
     if (I <= 64) return (const void*)pre_route_summaries<2, false, ADMIT, WHOLE>;
     if (I <= 128) return (const void*)pre_route_summaries<4, false, ADMIT, WHOLE>;
     if (I <= RS_DIRECT_ROWS) return (const void*)pre_route_summaries<8, false, ADMIT, WHOLE>;
-    return (const void*)pre_route_summaries<4, true, ADMIT, WHOLE>;
+    if (I <= RS_LONG_LISTS) return (const void*)pre_route_summaries<4, true, ADMIT, WHOLE>;
+    return (const void*)pre_route_summaries<8, true, ADMIT, WHOLE>;
 }
 template <bool ADMIT>
 static const void* summaries_kernel_for(const pre_ctx* ctx) {
