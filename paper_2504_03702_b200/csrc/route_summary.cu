@@ -1076,24 +1076,33 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         // ---- short arrivals and rows that have to be scanned: all rows, with every fold done.  First those with exact scores ...
         if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return; }
         acquire_cta();
-        jmax = (int)ld_volatile(&sh.jmax);
-        if (WHOLE && it.z > jmax) {
-            // no list covers it, but its ramp reaches every row's step: the keys give the scores of all rows that are not far
-            // (4,096 rows: 3,000 cycles, 28,000 for what follows)
+        if (WHOLE) {
+            // The keys give the scores of the rows that are not far and whose step the ramp reaches; the others are bounded from
+            // below by the cell that holds their top.  (4,096 rows: 3,000 cycles; 28,000 for what follows.)
             int least = RS_ABSENT, least_row = RS_NO_ROW;
             for (int g0 = 0; g0 < n_groups; g0 += 8) {
                 int2 r[8];
-                #pragma unroll
-                for (int u = 0; u < 8; ++u) r[u] = (g0 + u) * 32 + lane < I ? rows.rec[(g0 + u) * 32 + lane] : make_int2(RS_ABSENT, RS_LOWEST);
+                unsigned int s[8];
                 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    const int v = __viaddmax_s32(r[u].y, kp, r[u].x);
-                    if (v < least) { least = v; least_row = (g0 + u) * 32 + lane; }     // a lane's rows ascend
+                    const int i = (g0 + u) * 32 + lane;
+                    r[u] = i < I ? rows.rec[i] : make_int2(RS_ABSENT, RS_LOWEST);
+                    s[u] = i < I ? rows.state[i] : 0u;
+                }
+                #pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int jt = (int)(s[u] & RS_JTOP);
+                    const int add = (s[u] & RS_FAR) ? RS_LOWEST : (Dc > jt ? kp : -2 * sc.beta_i * jt);
+                    const int v = (s[u] & RS_FAR) ? r[u].x : max(r[u].x, r[u].y + add);
+                    const bool exact = !(s[u] & RS_FAR) && Dc > jt;
+                    // (bit 30 of the row: only a bound)
+                    if (v < least) { least = v; least_row = ((g0 + u) * 32 + lane) | (exact ? 0 : (int)RS_GIVEN); }     // a lane's rows ascend
                 }
             }
             const int best = __reduce_min_sync(FULL_MASK, least);
-            const int win = __reduce_min_sync(FULL_MASK, least == best ? least_row : RS_NO_ROW);
-            if (win < I && !__any_sync(FULL_MASK, (rows.state[win] & RS_FAR) != 0)) {
+            const int win = __reduce_min_sync(FULL_MASK, least == best ? (least_row & ~(int)RS_GIVEN) : RS_NO_ROW);
+            // (rows of the same value that are only bounded need a closer look)
+            if (win < I && !__any_sync(FULL_MASK, least == best && (least_row & (int)RS_GIVEN))) {
                 received(win);
                 tell(e, win, win, 0u);
                 return;
