@@ -284,3 +284,56 @@ def test_admission_queue_on_the_summary_kernel(beta, level):
     assert -2 in seen and -3 in seen and any(v >= 0 for v in seen) and any(v <= -10 for v in seen), \
         "the case was meant to route, queue, turn away and route out of the queue"
     st.close()
+
+
+@pytest.mark.parametrize("n_inst,h,n_arr", [(1, 32768 // 4, 9), (64, 512, 128), (64, 512, 129), (65, 504, 70), (128, 40, 300),
+                                            (129, 65, 300), (256, 64, 400), (257, 63, 400), (2048, 9, 300), (2049, 70, 300)])
+@pytest.mark.parametrize("beta", [1.0, 0.75])
+def test_both_sides_of_every_layout_of_the_deciding_warp(n_inst, h, n_arr, beta):
+    """One launch or three, ramps by the routing block or by the whole grid, one to eight rows per lane, all rows or a list."""
+    wl = W.make_random(500 + n_inst % 97, n_inst, h, 12 * n_inst, 0, max_prompt=300, max_output=2 * h + 9, beta=beta)
+    rng = np.random.default_rng(20)
+    ap = rng.integers(0, 300, n_arr).astype(np.int32)
+    ad = rng.integers(1, 2 * h + 9, n_arr).astype(np.int32)
+    wl.max_requests = 12 * n_inst + n_arr
+    route_and_compare(wl, ap, ad, batches=2)
+
+
+@pytest.mark.parametrize("n_inst,h", [(3, 700), (40, 900), (300, 260)])
+@pytest.mark.parametrize("beta", [1.0, 0.5])
+@pytest.mark.parametrize("queue", [False, True])
+def test_rows_whose_largest_cell_moves_beyond_the_first_steps(n_inst, h, beta, queue):
+    """Long requests with short prompts on maps that fall slowly: the bounds of the later steps overtake the first ones again
+    and again, rows are brought up to date in the middle of a batch, turn full and near again, and are counted cell by cell."""
+    n = 4 * n_inst
+    wl = W.make_random(520 + n_inst % 7, n_inst, h, n, 0, max_prompt=6000, max_output=h, beta=beta)
+    wl.generated[:] = 0
+    rng = np.random.default_rng(21)
+    n_arr = 900
+    ap = np.where(rng.random(n_arr) < 0.3, rng.integers(2000, 6000, n_arr), rng.integers(0, 40, n_arr)).astype(np.int32)
+    ad = np.where(rng.random(n_arr) < 0.4, rng.integers(1, 70, n_arr), rng.integers(h // 2, 2 * h, n_arr)).astype(np.int32)
+    wl.max_requests = n + n_arr
+    st = DeviceState.from_workload(wl)
+    st.select_router(B.ROUTE_SUMMARY)
+    ref = oracle.State.from_workload(wl)
+    st.anticipate()
+    ref.anticipate()
+    if queue:
+        st.make_queue(50)
+        ref.make_queue(50)
+    for lo in range(0, n_arr, 300):
+        p, d = ap[lo:lo + 300], ad[lo:lo + 300]
+        if queue:
+            _, c, s = st.route_admit(dev(p), dev(d), overload_level=2.0, overload_share=0.3)
+            _, wc, ws = ref.route_admit(p, d, overload_level=2.0, overload_share=0.3)
+        else:
+            c, s = st.route_batch(dev(p), dev(d))
+            wc, ws = ref.route_batch(p, d)
+        got = c.cpu().numpy()
+        assert (got == wc).all(), f"first difference at arrival {lo + int(np.argmax(got != wc))}"
+        assert_scores_close(s.cpu().numpy(), ws, wc)
+        assert_state_equal(st, ref, f"after arrival {lo + 300}")
+        st.step()
+        ref.step()
+    assert st.status() == B.PRE_OK
+    st.close()
