@@ -42,18 +42,18 @@ METRIC_STREAM = "routes/sec over the whole stream (decode step + routing of the 
 # its figure is below the algorithmic bytes.  pre_step: its two kernels added.
 # profiles/ncu_full_tick_scaler_refine_config3.txt: refinement and the fused tick (two kernels added).
 ROUTE_DRAM_READ = {3: 67322880}
-# profiles/ncu_dram_route_summary_kernels_config3_full_batch.txt: both kernels of the summary router on the full
+# profiles/ncu_dram_route_summary_kernels_config3_full_batch.txt: the three kernels of the summary router on the full
 # batch (the traffic does not grow in proportion to the batch, so the figure is used for the full batch only)
-ROUTE_SUMMARY_DRAM_TRAFFIC = {(3, 65536): 67724288 + 116224 + 55949824 + 5290240}
+ROUTE_SUMMARY_DRAM_TRAFFIC = {(3, 65536): 67732992 + 165120 + 2322176 + 50707456 + 2891264}
 # warp instructions per arrival of pre_route_summaries (smsp__inst_executed.sum of the 2,048-arrival capture in
-# profiles/ncu_full_step_kernels_config3_2048_arrivals.txt: 9,365,991 / 2,048)
-ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL = {3: 9365991 / 2048}
+# profiles/ncu_full_step_kernels_config3_2048_arrivals.txt: 1,565,269 / 2,048)
+ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL = {3: 1565269 / 2048}
 ROUTE_DRAM_WRITE_PER_ARRIVAL = {3: 679168 / 256}
-ANTICIPATE_DRAM_TRAFFIC = {3: 33808640 + 21654272}
-STEP_DRAM_TRAFFIC = {3: 33668864 + 67196416 + 8912640}
+ANTICIPATE_DRAM_TRAFFIC = {3: 33812992 + 19587328}
+STEP_DRAM_TRAFFIC = {3: 33670144 + 67196928 + 9366528}
 SCALER_DRAM_TRAFFIC = {3: 67127552 + 291584}   # profiles/ncu_full_scaler_rows_config3.txt
 REFINE_DRAM_TRAFFIC = {3: 44151040 + 25344}
-TICK_DRAM_TRAFFIC = {3: 44137216 + 46080 + 67199744 + 9207552}
+TICK_DRAM_TRAFFIC = {3: 44338688 + 45568 + 67200512 + 9501440}
 
 
 def measured_peak_gbs():
@@ -656,50 +656,35 @@ def route_scan_roofline(wl, index, t_route_ms, n_arrivals, map_max, layout, rout
 
 
 def route_summary_roofline(wl, index, t_route_ms, n_arrivals, clocks):
-    """The summary routing kernel.  One block on one SM: per arrival it reads the rows' summaries from shared
-    memory (8 bytes per instance), reads and rewrites the receiving row in the map (16 bytes per step), and is
-    bound by the latency of its rounds (two block barriers and the dependent steps of a decision), not by any
-    bandwidth.  Where the instructions per arrival are known from an ncu capture the roof quoted is the instruction
-    issue of the ONE SM the block runs on, else that SM's shared-memory bandwidth."""
+    """The summary router: rows' numbers, the routing block, the batch's ramps.  The routing block is bound by the chain of
+    dependent instructions of its deciding warp, not by any bandwidth; where the instructions per arrival are known from an
+    ncu capture the roof quoted is the instruction issue of the ONE SM the block runs on."""
     i, h = wl.n_instances, wl.horizon
-    ip = (i + 31) // 32 * 32
     mhz = clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or 1965.0
-    peak = 128 * mhz * 1e6 / 1e9
     sec = t_route_ms * 1e-3
-    smem_bytes = 8 * ip * n_arrivals
-    achieved = smem_bytes / sec / 1e9
     literal = n_arrivals * (8 * i * h + 16 * h + 16 * i)
     traffic = ROUTE_SUMMARY_DRAM_TRAFFIC.get((index, n_arrivals))
     hbm_peak, kind = measured_peak_gbs()
-    out = {
-        "traffic": traffic, "kernel": "pre_summarise_rows + pre_route_summaries", "us_per_arrival": sec * 1e6 / n_arrivals,
-        "bytes_of_shared_memory_read_per_arrival": 8 * ip, "bytes_of_map_read_and_written_per_arrival": 16 * h,
-        "smem_gbs": achieved, "smem_peak_gbs_of_the_one_sm": peak, "smem_frac": achieved / peak,
+    inst = ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL.get(index)
+    # 4 warp instructions per clock of the SM
+    issue_peak = 4 * mhz * 1e6 / 1e9
+    issued = None if inst is None else inst * n_arrivals / sec / 1e9
+    return {
+        "traffic": traffic, "kernel": "pre_summarise_rows + pre_route_summaries + pre_route_persistent (ramps)",
+        "us_per_arrival": sec * 1e6 / n_arrivals, "cycles_per_arrival": sec * mhz * 1e6 / n_arrivals,
         "scan_equivalent_gbs": literal / sec / 1e9,
         "hbm_frac_of_captured_traffic": None if traffic is None else traffic / sec / 1e9 / hbm_peak,
-        "limiter": "latency: every arrival is one round of the block (two block barriers, the scoring pass, the "
-                   "dependent steps of the decision); neither a memory nor the instruction issue is saturated",
-        "note": "the kernel decides from four numbers per row instead of scanning the maps (identical decisions) and "
-                "runs as ONE block; smem_* = bytes of row summaries read from shared memory over time against 128 "
-                f"B/clk x {mhz:.0f} MHz of the one SM it occupies; scan_equivalent_gbs is the literal formulation's 8 "
-                "bytes per cell and arrival over time, a convenience number that is not memory traffic; traffic = DRAM "
-                f"bytes of both kernels from the ncu capture of this batch ({kind} HBM peak {hbm_peak:.0f} GB/s for "
-                "hbm_frac_of_captured_traffic)"}
-    inst = ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL.get(index)
-    if inst is not None:
-        # not memory-bound: the roof is the instruction issue of the SM the block runs on, 4 warp instructions per clock
-        issue_peak = 4 * mhz * 1e6 / 1e9
-        issued = inst * n_arrivals / sec / 1e9
-        out.update({"bound": "alu", "achieved": issued, "peak": issue_peak, "unit": "G warp-instructions/s",
-                    "frac": issued / issue_peak,
-                    "peak_kind": f"derived: 1 SM x 4 schedulers x 1 warp instruction per clock x {mhz:.0f} MHz (SM clock "
-                                 "sampled during the timed region)",
-                    "warp_instructions_per_arrival": inst})
-    else:
-        out.update({"bound": "smem", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                    "peak_kind": f"derived: 1 SM x 128 B/clk x {mhz:.0f} MHz (the kernel is one block; SM clock sampled "
-                                 "during the timed region)"})
-    return out
+        "limiter": "latency: arrivals are decided one after another by one warp (two warp reductions and some ten dependent "
+                   "instructions each); neither a memory nor the instruction issue is saturated",
+        "note": "decisions are taken from two numbers per row instead of scanning the maps (identical decisions), by ONE block; "
+                "scan_equivalent_gbs is the literal formulation's 8 bytes per cell and arrival over time, a convenience "
+                "number that is not memory traffic; traffic = DRAM bytes of the call's kernels from the ncu capture of this "
+                f"batch ({kind} HBM peak {hbm_peak:.0f} GB/s for hbm_frac_of_captured_traffic)",
+        "bound": "alu", "achieved": issued, "peak": issue_peak, "unit": "G warp-instructions/s",
+        "frac": None if issued is None else issued / issue_peak,
+        "peak_kind": f"derived: 1 SM x 4 schedulers x 1 warp instruction per clock x {mhz:.0f} MHz (SM clock sampled during "
+                     "the timed region)",
+        "warp_instructions_per_arrival": inst}
 
 
 def main():
