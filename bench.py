@@ -751,7 +751,7 @@ def main():
             "vs_baseline": None, "dtype": "int64+f64", "data": "synthetic",
             "config": dict(config_dict(wl, 4), parallelism=f"{world} independent replica(s), one per GPU"),
             "ticks_per_s": rs["ticks"] / (rs["total_ms"] * 1e-3), "stream": rs,
-            "parity_checked": rs["parity_checked"], "gpu_launches": 3 * rs["ticks"] + 1, "clocks": clocks,
+            "parity_checked": rs["parity_checked"], "gpu_launches": 5 * rs["ticks"] + 1, "clocks": clocks,
             "roofline": {"bound": "smem", "achieved": None, "peak": None, "unit": "GB/s", "frac": None, "traffic": None,
                          "kernel": "pre_route_persistent",
                          "note": "per-tick batches of about 4,096 arrivals; see the one-shot configurations for the roofs"},
