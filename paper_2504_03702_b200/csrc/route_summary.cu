@@ -1394,7 +1394,7 @@ template <bool LISTS, bool ADMIT> struct Shape {
 };
 
 template <int KS, bool LISTS, bool ADMIT, bool WHOLE>
-__global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_summaries(const RouteSumArgs a) {
+__global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_summaries(const __grid_constant__ RouteSumArgs a) {
     typedef Shape<LISTS, ADMIT> Sp;
     constexpr int THREADS = Sp::THREADS;
     extern __shared__ __align__(16) unsigned char rs_smem[];

@@ -287,7 +287,8 @@ def test_admission_queue_on_the_summary_kernel(beta, level):
 
 
 @pytest.mark.parametrize("n_inst,h,n_arr", [(1, 32768 // 4, 9), (64, 512, 128), (64, 512, 129), (65, 504, 70), (128, 40, 300),
-                                            (129, 65, 300), (256, 64, 400), (257, 63, 400), (2048, 9, 300), (2049, 70, 300)])
+                                            (129, 65, 300), (256, 64, 400), (257, 63, 400), (2048, 9, 300), (2049, 70, 300),
+                                            (257, 63, 24), (2049, 70, 12), (2500, 128, 25)])
 @pytest.mark.parametrize("beta", [1.0, 0.75])
 def test_both_sides_of_every_layout_of_the_deciding_warp(n_inst, h, n_arr, beta):
     """One launch or three, ramps by the routing block or by the whole grid, one to eight rows per lane, all rows or a list."""
