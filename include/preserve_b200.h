@@ -140,14 +140,15 @@ int pre_anticipate_static(int32_t n_instances, int32_t horizon, const int32_t* d
  * when the context's instances fit its shared memory, every value stays below 2^32 during the
  * batch and the batch (with the waiting requests of pre_route_admit) has fewer than 2^26 entries,
  * which it checks on the device.  Otherwise the scanning kernel routes: it reads every cell
- * for every arrival, its blocks exchange their best instances through device memory and wait
- * for one another a bounded number of polls.  If such a wait runs out (PRE_ETIMEOUT from
- * pre_status; it should never happen on a GPU that runs the kernel alone), the blocks agree on
- * the last arrival that every one of them had scored: arrivals up to that one are routed exactly
- * as above (maps, queued_p, current_d, table and *d_n_requests all include them and nothing
- * else), every later arrival gets PRE_CHOICE_DROPPED and score 0, and the context stays usable.
- * Only if the blocks cannot even meet to agree (a second, much longer bounded wait) may the maps
- * hold one request more than the table; rebuild them with pre_anticipate then. */
+ * for every arrival, and its blocks exchange their best instances through device memory.
+ * The scanning kernel's blocks wait for one another, and the summary kernel's warps do, a bounded number
+ * of polls.  If such a wait runs out (PRE_ETIMEOUT from pre_status; it should never happen on a GPU that
+ * runs the kernel alone), the batch ends with the last arrival that had been decided (scanning kernel: the
+ * last one that every block had scored): arrivals up to that one are routed exactly as above (maps,
+ * queued_p, current_d, table and *d_n_requests all include them and nothing else), every later arrival
+ * gets PRE_CHOICE_DROPPED and score 0, and the context stays usable.
+ * Only if the scanning kernel's blocks cannot even meet to agree (a second, much longer bounded wait) may
+ * the maps hold one request more than the table; rebuild them with pre_anticipate then. */
 int pre_route_batch(pre_ctx* ctx, const int32_t* d_arr_prompt, const int32_t* d_arr_predicted,
                     int64_t n_arrivals, int64_t* d_curves, int64_t* d_queued_p, int64_t* d_current_d,
                     int32_t* d_prompt, int32_t* d_generated, int32_t* d_predicted, int32_t* d_instance,

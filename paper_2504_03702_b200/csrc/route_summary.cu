@@ -65,7 +65,8 @@ constexpr int RS_LIMIT = 32;
 constexpr int RS_MAX_ROWS = 10240;          // instances up to which the context offers this router (shared memory),
 constexpr int RS_MAX_BINARY64_ROWS = 5120;  // and with binary64 scores
 constexpr int SUM_THREADS = 256;
-constexpr unsigned int RS_SPIN_LIMIT = 1u << 24;   // polls of shared memory (some 0.5 s) before a wait inside the block is abandoned
+constexpr unsigned int RS_POLLS = 4;        // polls of shared memory per poll of the context's limit (together some 0.5 s) before a wait
+                                            // inside the block is abandoned
 constexpr int RS_NO_ROW = 0x3fffffff;
 constexpr int RS_ALONE_ROWS = 64;                  // small shapes: instances,
 constexpr long long RS_ALONE_CELLS = 32768;        // cells of the maps,
@@ -298,6 +299,7 @@ struct RouteSumArgs {
     int* status;
     int* give_up;                  // three words that the scanning kernel finds cleared
     int* handled;                  // 1: this kernel routed the batch; 0: the scanning kernel has to
+    unsigned int spin_limit;       // polls before a wait is declared lost
     int alone;                     // small shapes: nothing is launched before or after this kernel, but for the ramps where
     int own_ramps;                 // this kernel does not add them itself
     long long* ramps;              // {first table row, rows} whose ramps the maps still lack
@@ -358,6 +360,8 @@ struct RsShared {
     unsigned int items_end;                 // 1: there will be no more
     unsigned int written;                   // results written so far
     unsigned int flush;                     // ... and as many are asked for
+    int cursor;                             // items of the batch that the io warp has looked at (when it has ended)
+    unsigned int spin_limit;
     unsigned int not_over;                  // ADMIT: rows that are not overloaded, as far as folded
     int blocked;                            // ADMIT: a request found every instance overloaded ...
     long long blocked_k;                    // ... this one
@@ -405,7 +409,7 @@ template <typename Cond>
 __device__ __forceinline__ bool rs_wait(RsShared& sh, Cond&& ready, unsigned int nap = 0) {
     for (unsigned int polls = 0; !__all_sync(FULL_MASK, ready()); ++polls) {   // (all lanes take the same way)
         if ((polls & 255u) == 255u && __any_sync(FULL_MASK, ld_volatile(&sh.ctl.w) != 0)) return false;
-        if (polls > RS_SPIN_LIMIT) { st_release(&sh.ctl.w, 1u); return false; }
+        if (polls >= sh.spin_limit) { st_release(&sh.ctl.w, 1u); return false; }
         if (nap) __nanosleep(nap);
     }
     return true;
@@ -723,7 +727,7 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
     }
     first_bad = __reduce_min_sync(FULL_MASK, first_bad);
     first_full = __reduce_min_sync(FULL_MASK, first_full);
-    if (lane == 0) { sh.first_bad = first_bad; sh.first_full = first_full; }
+    if (lane == 0) { sh.first_bad = first_bad; sh.first_full = first_full; sh.cursor = min(cursor, items); }
 }
 
 // ---- list warps.  A list holds the rows whose key value for one of RS_PROBES prompt lengths lies within a margin of the
@@ -1387,6 +1391,34 @@ __device__ __noinline__ void rs_literal(const RouteSumArgs& a, RsShared& sh, lon
     __syncthreads();
 }
 
+// After a wait that was abandoned: the results of the decisions that were told and that the io warp has not written.  A row has
+// at most one decision that is not folded, and as long as it is pending its numbers are those that the decision was made with.
+// The maps need nothing: they receive the ramps of every table row that is not marked as applied.  Returns the first item that
+// was not decided (the ones from there on that are malformed or find the table full have their results already, the same
+// as those that were not reached).
+template <bool ADMIT, bool WHOLE>
+__device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int waiting) {
+    const unsigned int told = sh.ctl.x;
+    for (unsigned int e = sh.written + threadIdx.x; e < told; e += blockDim.x) {
+        const uint2 job = sh.jobs[e % RS_ITEMS];
+        const int2 pd = sh.raw[e % RS_ITEMS];
+        const int w = (int)(job.x & ~RS_GIVEN), k = sh.item_at[e % RS_ITEMS];
+        const long long at = sh.n0 + e;
+        double s = sh.score[e % RS_ITEMS];
+        if (rows.pending[w])
+            s = summary_score(sc.tokens_of(rows, w), (job.x & RS_GIVEN) ? job.y : rows.top[w] + (unsigned int)pd.x, (double)pd.x + (double)pd.y, a.theta, a.beta);
+        a.prompt[at] = pd.x; a.generated[at] = 0; a.predicted[at] = pd.y; a.instance[at] = w;
+        if (ADMIT && k < waiting) a.queue_choice[k] = w;
+        else {
+            a.choice[k - waiting] = w;
+            if (a.score) a.score[k - waiting] = s;
+        }
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.queued_p + w), (unsigned long long)pd.x);
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.current_d + w), (unsigned long long)pd.y);
+    }
+    return sh.items_ready > told ? sh.item_at[told % RS_ITEMS] : sh.cursor;
+}
+
 // Folding and list warps, warps and threads of the instantiations.
 template <bool LISTS, bool ADMIT> struct Shape {
     static constexpr int FOLD = LISTS ? 6 : 5, LIST = LISTS ? 8 : 0;
@@ -1440,6 +1472,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         // (whole-number scores: the host has seen to beta and theta)
         const bool exact = !WHOLE || token_bound + max_pd + (unsigned long long)a.beta * (peak_bound + 1) < (1ull << 29);
         sh.mode = ok && exact ? 1 : 0;
+        sh.spin_limit = a.spin_limit; sh.cursor = 0;
         sh.n0 = *a.n_requests;
         sh.ctl = make_uint4(0u, 0u, 0u, 0u);
         sh.items_ready = sh.items_end = sh.not_over = sh.jmax = sh.written = sh.flush = 0;
@@ -1474,6 +1507,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         if (q_len > a.queue_capacity) q_len = a.queue_capacity;
     }
     const long long n_items = q_len + a.n_arrivals;
+    long long decided = n_items;     // items from here on were not decided
     if (mode == 0) {
         rs_literal<ADMIT>(a, sh, q_head, q_len, n_items);
     } else {
@@ -1540,14 +1574,24 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
             rs_list_loop<LISTS ? Sp::LIST : 8, 32 * KS, WHOLE>(sh, rows, sc, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
     }
     __syncthreads();
+    if (sh.ctl.w) {     // (all threads alike: nobody writes it any more)
+        decided = rs_settle<ADMIT, WHOLE>(a, sh, rows, sc, (int)q_len);
+        __syncthreads();
     }
-    const bool blocked = ADMIT && sh.blocked;
-    const long long decided = blocked ? sh.blocked_k : n_items;
+    }
+    const bool blocked = ADMIT && sh.blocked, dropped = !blocked && decided < n_items;
+    if (blocked) decided = sh.blocked_k;
+    if (!ADMIT && dropped)
+        for (long long k = decided + tid; k < n_items; k += THREADS) {
+            a.choice[k] = PRE_CHOICE_DROPPED;
+            if (a.score) a.score[k] = 0.0;
+        }
     if (tid == 0) {
         *a.n_requests = sh.n0 + sh.ctl.x;
         a.ramps[0] = sh.n0;
         a.ramps[1] = mode == 0 || a.own_ramps ? 0 : (long long)sh.ctl.x;
-        // (what was noted beyond a blocked request is decided again below and does not count here)
+        // (what was noted beyond a blocked request is decided again below, what was noted beyond the last decision is dropped: neither
+        // counts here)
         int flags = sh.ctl.w ? PRE_ST_TIMEOUT : 0;
         if (sh.first_bad < decided) flags |= PRE_ST_BADREQ;
         if (sh.first_full < decided) flags |= PRE_ST_CAPACITY;
@@ -1569,7 +1613,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     if (ADMIT) {
         // Everything from the blocked request on: a request that was waiting keeps its place; an arrival joins
         // the tail of the queue while there is room and is turned away otherwise (a malformed arrival is
-        // dropped).  Nothing else reads or writes these arrays any more.
+        // dropped).  After a wait that was abandoned the arrivals are dropped.  Nothing else reads or writes these arrays any more.
         __syncthreads();
         const long long stop = decided;
         const long long left = stop < q_len ? q_len - stop : 0;          // waiting entries that stay
@@ -1580,7 +1624,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
             const long long i = base + tid;
             int P = -1, D = 0;
             if (i < a.n_arrivals) { P = a.arr_prompt[i]; D = a.arr_predicted[i]; }
-            const bool ok = i < a.n_arrivals && !(P < 0 || D < 1 || P > PRE_FIELD_MAX || D > PRE_FIELD_MAX);
+            const bool ok = i < a.n_arrivals && !dropped && !(P < 0 || D < 1 || P > PRE_FIELD_MAX || D > PRE_FIELD_MAX);
             const unsigned int vote = __ballot_sync(0xffffffffu, ok);
             if (lane == 0) sh.warp_ok[warp] = __popc(vote);
             __syncthreads();
@@ -1708,6 +1752,7 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
     a.theta = ctx->theta; a.beta = ctx->cfg.beta;
     a.summary0 = p.summary; a.guard = p.guard; a.near = p.near; a.far = p.far; a.applied = ctx->d_rs_applied;
     a.status = ctx->d_status; a.handled = ctx->d_rs_handled; a.give_up = ctx->d_abort; a.ramps = ctx->d_rs_ramps;
+    a.spin_limit = ctx->spin_limit > 0xffffffffu / RS_POLLS ? 0xffffffffu : RS_POLLS * ctx->spin_limit;
     a.alone = pre_route_summary_alone(ctx) ? 1 : 0;
     a.own_ramps = a.alone && n_arrivals * (long long)H <= RS_OWN_RAMP_CELLS ? 1 : 0;
     a.queue_prompt = nullptr; a.queue_predicted = nullptr; a.queue_state = nullptr; a.queue_entry = nullptr;
