@@ -361,7 +361,8 @@ struct RsShared {
     unsigned int written;                   // results written so far
     unsigned int flush;                     // ... and as many are asked for
     int cursor;                             // items of the batch that the io warp has looked at (when it has ended)
-    unsigned int spin_limit;
+    unsigned int spin_limit, idle_limit;
+    unsigned int beat;                      // moves while a warp is busy with something long that others wait for
     unsigned int not_over;                  // ADMIT: rows that are not overloaded, as far as folded
     int blocked;                            // ADMIT: a request found every instance overloaded ...
     long long blocked_k;                    // ... this one
@@ -405,11 +406,18 @@ __device__ __forceinline__ int4 ld_table(unsigned int at) {
 __device__ __forceinline__ void acquire_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 
 // A wait of a whole warp on words that other warps of this block write.  False: abandoned, here or elsewhere.
-template <typename Cond>
+// What counts against the limit is time in which nothing moves.  IDLE: nothing is owed to this warp, it waits for work; that
+// there is none as long as the deciding warp gets on without is no reason to give up.
+template <bool IDLE = false, typename Cond>
 __device__ __forceinline__ bool rs_wait(RsShared& sh, Cond&& ready, unsigned int nap = 0) {
+    unsigned int seen = 0;
     for (unsigned int polls = 0; !__all_sync(FULL_MASK, ready()); ++polls) {   // (all lanes take the same way)
-        if ((polls & 255u) == 255u && __any_sync(FULL_MASK, ld_volatile(&sh.ctl.w) != 0)) return false;
-        if (polls >= sh.spin_limit) { st_release(&sh.ctl.w, 1u); return false; }
+        if ((polls & 255u) == 255u) {
+            if (__any_sync(FULL_MASK, ld_volatile(&sh.ctl.w) != 0)) return false;
+            const unsigned int now = __shfl_sync(FULL_MASK, ld_volatile(&sh.beat) + (IDLE ? ld_volatile(&sh.ctl.x) : 0u), 0);
+            if (now != seen) { seen = now; polls = 0; }
+        }
+        if (polls >= (IDLE ? sh.idle_limit : sh.spin_limit)) { st_release(&sh.ctl.w, 1u); return false; }
         if (nap) __nanosleep(nap);
     }
     return true;
@@ -528,6 +536,7 @@ struct Folder {
         const long long n0 = sh.n0;
         int64_t* row = a.curves + (size_t)w * H;
         for (unsigned int base = 0; base < upto; base += 32) {
+            if ((base & 1023u) == 0 && lane == 0) atomicAdd(&sh.beat, 1u);
             const unsigned int k = base + lane;
             const bool mine = k < upto && a.instance[n0 + k] == w && a.applied[k] == 0;
             if (mine) a.applied[k] = 1;
@@ -624,7 +633,7 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
     unsigned int scans = 0;
     for (unsigned int n = me;;) {
         uint4 ctl;
-        if (!rs_wait(sh, [&] {
+        if (!rs_wait<true>(sh, [&] {
                 ctl = ld_volatile4(&sh.ctl);
                 return (int)(ctl.x - n) > 0 || ctl.y != scans || ctl.z != 0;
             }, LISTS ? 20 : 0))    // (the list warps need the issue slots)
@@ -668,6 +677,7 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
     unsigned int entered = 0;       // requests found among them
     unsigned int written = 0;       // results written out
     int first_bad = 0x7fffffff, first_full = 0x7fffffff;
+    unsigned int quiet = 0, seen = 0;      // rounds of this loop in which nothing has moved
     for (;;) {
         while (cursor < items && entered - written <= RS_ITEMS - 32) {
             const int k = cursor + lane;
@@ -695,7 +705,7 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
             entered = min(entered + __popc(vote), (unsigned int)room);
             cursor += 32;
             __syncwarp();
-            if (lane == 0) st_release(&sh.items_ready, entered);
+            if (lane == 0) { st_release(&sh.items_ready, entered); atomicAdd(&sh.beat, 1u); }
         }
         if (cursor >= items && lane == 0) st_release(&sh.items_end, 1u);
         const uint4 ctl = ld_volatile4(&sh.ctl);
@@ -723,6 +733,10 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
         }
         if (last && written == decided) break;
         if (__any_sync(FULL_MASK, ctl.w != 0)) break;
+        const unsigned int now = decided + written + (unsigned int)cursor + __shfl_sync(FULL_MASK, ld_volatile(&sh.beat), 0);
+        quiet = now != seen ? 0u : quiet + 1u;
+        seen = now;
+        if (quiet >= sh.idle_limit) { st_release(&sh.ctl.w, 1u); break; }
         __nanosleep(100);
     }
     first_bad = __reduce_min_sync(FULL_MASK, first_bad);
@@ -769,7 +783,7 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
     unsigned short* near = sh.near_row + (t >> 5) * NEAR_ROOM;
     for (unsigned int n = 1;; ++n) {
         bool go = false;
-        if (!rs_wait(sh, [&] {
+        if (!rs_wait<true>(sh, [&] {
                 const uint4 ctl = ld_volatile4(&sh.ctl);
                 go = ld_acquire(&sh.lists_wanted) >= n;
                 return go || ctl.z != 0;
@@ -1472,7 +1486,9 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         // (whole-number scores: the host has seen to beta and theta)
         const bool exact = !WHOLE || token_bound + max_pd + (unsigned long long)a.beta * (peak_bound + 1) < (1ull << 29);
         sh.mode = ok && exact ? 1 : 0;
-        sh.spin_limit = a.spin_limit; sh.cursor = 0;
+        sh.spin_limit = a.spin_limit;
+        sh.idle_limit = max(a.spin_limit < (1u << 27) ? 16u * a.spin_limit : 0xffffffffu, 1u << 22);
+        sh.cursor = 0; sh.beat = 0;
         sh.n0 = *a.n_requests;
         sh.ctl = make_uint4(0u, 0u, 0u, 0u);
         sh.items_ready = sh.items_end = sh.not_over = sh.jmax = sh.written = sh.flush = 0;

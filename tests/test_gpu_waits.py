@@ -131,6 +131,33 @@ def test_summary_router_wait_that_runs_out_keeps_a_routed_prefix(n_inst, h, beta
     st.close()
 
 
+def test_warps_that_have_nothing_to_do_are_not_lost():
+    """Arrivals of one token for which no list is asked for, and a long run of malformed ones that reach nobody: both take many
+    times the limit, and nothing is owed to the warps that wait meanwhile."""
+    n_inst, h = 900, 64
+    n = 8 * n_inst
+    wl = W.make_random(33, n_inst, h, n, 0, max_prompt=300, max_output=h)
+    rng = np.random.default_rng(33)
+    short, bad = 3000, 300000
+    ap = rng.integers(0, 300, short + bad + 50).astype(np.int32)
+    ad = np.ones(short + bad + 50, np.int32)
+    ad[short:short + bad] = 0
+    wl.max_requests = n + short + 50
+    st = DeviceState.from_workload(wl)
+    st.select_router(B.ROUTE_SUMMARY)
+    ref = oracle.State.from_workload(wl)
+    st.anticipate()
+    ref.anticipate()
+    B.pre_test_set_spin_limit(st.ctx, 4096)
+    choice, score = st.route_batch(dev(ap), dev(ad))
+    assert st.status() == B.PRE_EBADREQ, "a warp that waited for work gave the batch up"
+    want_c, want_s = ref.route_batch(ap, ad, fast=True)
+    assert (choice.cpu().numpy() == want_c).all()
+    assert_scores_close(score.cpu().numpy(), want_s, want_c)
+    assert_state_equal(st, ref)
+    st.close()
+
+
 @pytest.mark.parametrize("n_inst,h,beta", SUMMARY_SHAPES)
 @pytest.mark.parametrize("polls", [0, 20])
 def test_summary_admission_router_wait_that_runs_out(n_inst, h, beta, polls):
