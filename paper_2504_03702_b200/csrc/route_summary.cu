@@ -1148,7 +1148,8 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             for (int u = 0; u < 4; ++u) ok[u] = look((g0 + u) * 32 + lane, s[u], tokens, peak[u]);
             #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (ok[u] && s[u] < mine) { mine = s[u]; mine_row = (g0 + u) * 32 + lane; mine_peak = peak[u]; }   // a lane's rows ascend
+                // (a lane's rows ascend; the first counts whatever its score, which may be infinite)
+                if (ok[u] && (s[u] < mine || (mine_row == RS_NO_ROW && (g0 + u) * 32 + lane < I))) { mine = s[u]; mine_row = (g0 + u) * 32 + lane; mine_peak = peak[u]; }
                 if (__any_sync(FULL_MASK, !ok[u])) {
                     if (lane == 0) sh.slow_group[n_again] = (unsigned short)(g0 + u);
                     ++n_again;
@@ -1192,7 +1193,6 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             take();
             __syncwarp();
         }
-        if (win >= I) { win = 0; win_peak = 0; }   // (no score is finite: beta or theta beyond binary64's range)
         #pragma unroll
         for (int k = 0; k < KS; ++k)
             if (row[k] == win) {      // (a lower bound, odd)

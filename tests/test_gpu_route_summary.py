@@ -169,6 +169,30 @@ def test_whole_number_scores_that_could_reach_2_to_the_30_go_to_the_scanning_ker
     assert ref.curves.max() * 4096.0 > 2.0 ** 30, "the case was meant to pass the whole-number bound"
 
 
+@pytest.mark.parametrize("n_inst,h", [(5, 16), (40, 900), (300, 24)])
+def test_scores_beyond_binary64(n_inst, h):
+    """A penalty coefficient of 1e308: a row that pays has an infinite score, and when all rows do, the first one wins with it."""
+    wl = W.make_random(98, n_inst, h, 4 * n_inst, 0, max_prompt=200, max_output=h, capacity=2000, beta=1e308)
+    rng = np.random.default_rng(16)
+    n_arr = 8 * n_inst
+    ap = rng.integers(50, 400, n_arr).astype(np.int32)
+    ad = rng.integers(1, 2 * h, n_arr).astype(np.int32)
+    wl.max_requests = 4 * n_inst + n_arr
+    st = DeviceState.from_workload(wl)
+    st.select_router(B.ROUTE_SUMMARY)
+    ref = oracle.State.from_workload(wl)
+    st.anticipate()
+    ref.anticipate()
+    choice, score = st.route_batch(dev(ap), dev(ad))
+    want_c, want_s = ref.route_batch(ap, ad)
+    assert np.isfinite(want_s[0]) and np.isinf(want_s[-1]), "the case was meant to run from finite scores to infinite ones"
+    assert (choice.cpu().numpy() == want_c).all()
+    assert (score.cpu().numpy() == want_s).all()
+    assert_state_equal(st, ref)
+    assert st.status() == B.PRE_OK
+    st.close()
+
+
 def test_selecting_the_kernel():
     wl = W.make_random(93, 20000, 4, 100, 0)
     st = DeviceState.from_workload(wl)
