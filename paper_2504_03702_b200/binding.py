@@ -63,8 +63,9 @@ def _load():
 
 
 lib = _load()
-_raw_stream = torch._C._cuda_getCurrentRawStream
-_device = torch._C._cuda_getDevice
+# (torch's own wrappers build a Stream object, 3 us per call; a torch without these two entry points takes the wrappers)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 class PreError(RuntimeError):
@@ -84,6 +85,8 @@ def _ptr(t):
 
 def _stream():
     """torch's current stream on the current device, without building a Stream object for it."""
+    if _raw_stream is None or _device is None:
+        return torch.cuda.current_stream().cuda_stream
     return _raw_stream(_device())
 
 

@@ -2,6 +2,8 @@
 import ctypes as C
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -72,3 +74,14 @@ def test_missing_library_is_loud(binding, tmp_path, monkeypatch):
     mod = importlib.util.module_from_spec(spec)
     with pytest.raises(ImportError, match="no CPU fallback"):
         spec.loader.exec_module(mod)
+
+
+def test_binding_without_torchs_raw_stream_entry_points(binding):
+    """A torch without them (built without CUDA) can import the binding; the stream then comes from the public wrapper."""
+    code = ("import torch\n"
+            "for n in ('_cuda_getCurrentRawStream', '_cuda_getDevice'):\n"
+            "    if hasattr(torch._C, n): delattr(torch._C, n)\n"
+            "from paper_2504_03702_b200 import binding as B\n"
+            "torch.cuda.current_stream = lambda: type('S', (), {'cuda_stream': 77})()\n"
+            "assert B._stream() == 77\n")
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
