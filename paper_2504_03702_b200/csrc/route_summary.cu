@@ -938,7 +938,12 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     int row[KS], ra[KS], rb[KS];
     constexpr int NO_ROW = RS_NO_ROW, ODD = -1, NONE = -2;   // (ODD, NONE: of the step before, see below)
     int jmax = 0;        // an arrival whose ramp is longer than this reaches the step of every row's b
-    auto refresh = [&]() {   // the marked rows that are not pending any more
+    // The marked rows that are not pending any more.  The loads are no acquires: what this warp needs of a fold lies in shared memory
+    // and is read after `pending`, in order.  That the next folding warp of the row sees the cells that the last one stored to
+    // device memory follows from all of them running on one SM (one L1, and the last one's release comes before its `pending`), not
+    // from a chain of acquires; a fence here would make it one, and costs 50 ns a look (64 instances, 1,024 arrivals: 199 -> 205 us;
+    // as acquiring loads 212, with the fence merged into the release of the decisions 204).
+    auto refresh = [&]() {
         #pragma unroll
         for (int k = 0; k < KS; ++k) {
             if (ra[k] & 1) {
