@@ -1414,9 +1414,9 @@ __device__ __noinline__ void rs_literal(const RouteSumArgs& a, RsShared& sh, lon
 // at most one decision that is not folded, and as long as it is pending its numbers are those that the decision was made with.
 // The maps need nothing: they receive the ramps of every table row that is not marked as applied.  Returns the first item that
 // was not decided (the ones from there on that are malformed or find the table full have their results already, the same
-// as those that were not reached).
+// as those that were not reached).  (`rows` and `sc` by value: by reference they would live on the stack of every thread.)
 template <bool ADMIT, bool WHOLE>
-__device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int waiting) {
+__device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const Rows rows, const Scores<WHOLE> sc, int waiting) {
     const unsigned int told = sh.ctl.x;
     for (unsigned int e = sh.written + threadIdx.x; e < told; e += blockDim.x) {
         const uint2 job = sh.jobs[e % RS_ITEMS];
