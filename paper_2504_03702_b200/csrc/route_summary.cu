@@ -34,8 +34,8 @@
 //     list warps     (beyond 256 instances) build the next list while the present one is being used up: the rows
 //                    whose score is within a margin of the smallest one for any of eight prompt lengths, and the
 //                    bounds of the rest.  Scores only grow during a batch, so a list that is a little behind is valid.
-//     folding warps  add each routed request to its row's numbers, one warp per request; they also scan single rows for
-//                    the deciding warp;
+//     folding warps  add each routed request to its row's numbers, one warp per request; an arrival that the rows held
+//                    leave undecided is decided by all of them together on all rows;
 //     io warp        reads the arrivals ahead of the decisions and writes the results behind them.
 //   Warps 0, 4, 8, ... share one of the SM's four schedulers.  The deciding warp is warp 0 and the others of that scheduler
 //   have nothing to do: the chain of dependent instructions of warp 0 is the time of the batch.
@@ -166,7 +166,7 @@ struct SumArgs {
     const int32_t* arr_predicted;
     long long n_arrivals;
     int I, H;
-    uint4* summary;                // {token count, top, jtop | step of the next << 16, largest c[j] + j of the first steps} per row
+    uint4* summary;                // {token count, top, jtop | step of the next << 16 | drop << 21, largest c[j] + j of the first steps} per row
     uint2* near;                   // [I][32] the first 64 cells
     unsigned int* far;             // [I][32] the stretches
     unsigned long long* guard;
@@ -224,8 +224,11 @@ __device__ __forceinline__ void batch_totals(const Args& a, long long first, lon
     }
 }
 
+// How much less than `top` the row's first cell is: 2047 stands for that much or more.
+__device__ __forceinline__ unsigned int drop_of(unsigned int top, unsigned int cell0) { return min(top - cell0, 2047u); }
+
 // One row by one warp: its first cells and stretches (to `near`, `far`), the guards, and for lane 0 the summary {token count, top,
-// jtop | step of the next << 16, largest c[j] + j of the first steps} and the number of cells above the overload level.
+// jtop | step of the next << 16 | drop << 21, largest c[j] + j of the first steps} and the number of cells above the overload level.
 template <typename Args, typename Put>
 __device__ __forceinline__ void summarise_row(const Args& a, int row, uint2* near, unsigned int* far, unsigned long long* guard, Put&& put) {
     const int lane = threadIdx.x & 31, H = a.H;
@@ -240,7 +243,8 @@ __device__ __forceinline__ void summarise_row(const Args& a, int row, uint2* nea
         const long long tok = q + d;
         const bool ok = q >= 0 && d >= 0 && q <= 0xffffffffLL && d <= 0xffffffffLL && tok <= 0xffffffffLL;
         if (!ok) bad = true;
-        put(make_uint4(ok ? (unsigned int)tok : 0u, n.top, n.jtop | (step << 16), first), n.above);
+        const unsigned int drop = drop_of(n.jtop >= (unsigned int)RS_LIMIT ? first : n.top, n.near0);
+        put(make_uint4(ok ? (unsigned int)tok : 0u, n.top, n.jtop | (step << 16) | (drop << 21), first), n.above);
         if (ok) {
             atomicMax(guard + GUARD_MAX_BASE, (unsigned long long)tok);
             atomicAdd(guard + GUARD_SUM_BASE, (unsigned long long)tok);
@@ -318,11 +322,13 @@ struct RouteSumArgs {
 // Rows in shared memory (structure of arrays):
 //   rec    {a, b}, even: the score of an arrival is at least max(a, b + what its prompt adds), and that but for the rounding
 //          of the keys unless the row is far or pending
-//   state  jtop | RS_FAR | RS_FULL | RS_DEFERRED (the map lacks ramps) | RS_NOT_OVER (ADMIT: the row is not overloaded, as
+//   state  jtop | drop << RS_DROP (the first cell is that much below the top that b stands for; RS_DROP_MAX: or more) | RS_FAR | RS_FULL | RS_DEFERRED (the map lacks ramps) | RS_NOT_OVER (ADMIT: the row is not overloaded, as
 //          far as folded)
 //   top, tok   top and token count (whole-number scores: half of a)
 //   pending  1 from the decision for the row to the end of its fold; cleared last
-constexpr unsigned int RS_FAR = 0x40000000u, RS_NOT_OVER = 0x20000000u, RS_FULL = 0x10000000u, RS_DEFERRED = 0x08000000u, RS_JTOP = 0xffffu;
+constexpr unsigned int RS_FAR = 0x40000000u, RS_NOT_OVER = 0x20000000u, RS_FULL = 0x10000000u, RS_DEFERRED = 0x08000000u, RS_JTOP = 0xffffu,
+                       RS_DROP_MAX = 2047u;
+constexpr int RS_DROP = 16;
 struct Rows {
     int2* rec;
     unsigned int* state;
@@ -333,7 +339,7 @@ struct Rows {
 
 struct RsShared {
     // what the deciding warp tells the folding warps and the io warp, read with one access
-    uint4 ctl;                              // {decisions made, scans asked for, 1: no more of either, 1: a wait was abandoned}
+    uint4 ctl;                              // {decisions made, arrivals for all rows, 1: no more of either, 1: a wait was abandoned}
     int4 items[RS_ITEMS];                   // of the requests to route, in order: {what P adds to b, P + D as a key, less one, min(D, H)
                                             // (0: not for the quick way), offset of P's entry in the table}
     int2 raw[RS_ITEMS];                     // {P, D}
@@ -350,11 +356,13 @@ struct RsShared {
     unsigned int list_met;                  // (list warps) arrivals at their meetings
     unsigned int lists_wanted, lists_ready;
     unsigned int done[RS_MAX_FOLD_WARPS];   // the next decision each folding warp will fold
-    unsigned int scans_done[RS_MAX_FOLD_WARPS];
-    unsigned short slow_group[(RS_MAX_ROWS + 31) / 32 + 4];   // (deciding warp) groups of 32 rows to look at again
-    int scan_row[32];
-    unsigned int peak[32];
-    int scan_P, scan_Dc, scan_n;
+    unsigned int looks_done[RS_MAX_FOLD_WARPS];
+    int look_P, look_D, look_closely;
+    int4 look_key[RS_MAX_FOLD_WARPS];       // smallest key of a warp's rows (odd: exact), the row, the next smallest key
+    unsigned int look_met, look_least;      // (a closer look) arrivals at the meetings; smallest key that a row has at most
+    unsigned long long look_score[2][RS_MAX_FOLD_WARPS];   // the smallest score of a warp's rows, before and after the scans, as its bits,
+    int look_row[2][RS_MAX_FOLD_WARPS];                    // the row that has it
+    unsigned int look_peak[2][RS_MAX_FOLD_WARPS];          // and its peak
     unsigned int jmax;                      // largest step that a row's b stands for
     unsigned int items_ready;               // items written so far
     unsigned int items_end;                 // 1: there will be no more
@@ -445,6 +453,7 @@ template <bool WHOLE> struct Scores {
     static constexpr int SLACK = WHOLE ? 0 : 8;
     double theta, beta, unit;
     int theta_i, beta_i, shift, code_base;
+    int slope;           // what a token less at the peak takes from b at most (0: too much)
     __device__ __forceinline__ void start(double theta_d, double beta_d, unsigned long long peak_bound, unsigned long long max_pd,
                                           unsigned long long typical_tokens, int mean) {
         theta = theta_d; beta = beta_d;
@@ -462,6 +471,8 @@ template <bool WHOLE> struct Scores {
                 --shift;
             unit = (double)(1 << shift);
         }
+        const double s = WHOLE ? 2.0 * beta : 2.0 * ceil(beta * unit);
+        slope = WHOLE || s <= 524288.0 ? (int)s : 0;
         code_base = __float_as_int(fmaxf((float)mean * (1.0f / 32.0f) * (float)beta * (float)(2.0 * unit), 1.0f)) >> 21;
     }
     __device__ __forceinline__ int key_a(unsigned int tokens) const {
@@ -478,6 +489,9 @@ template <bool WHOLE> struct Scores {
     __device__ __forceinline__ int key_pd(int P, int D) const {
         return WHOLE ? 2 * (P + D) : (int)min((long long)(P + D) << (shift + 1), (long long)RS_CUT);
     }
+    // The least that an arrival whose ramp may end before the step of the top, Dc <= jtop, adds to b: the first cell has its
+    // prompt, and unless the row is far the cell of the top has what it had; the ramp reaches all of the first steps, or not.
+    __device__ __forceinline__ int key_short(unsigned int state, int kp, int Dc) const;
     // whether the keys of 32 such arrivals in a row stay below their cut
     __device__ __forceinline__ bool usual(int kp, int kpd) const { return WHOLE || kp + kpd <= 16777216; }
     __device__ __forceinline__ unsigned int tokens_of(const Rows& rows, int i) const { return WHOLE ? (unsigned int)rows.rec[i].x >> 1 : rows.tok[i]; }
@@ -506,6 +520,13 @@ template <bool WHOLE> struct Scores {
         }
     }
 };
+template <bool WHOLE>
+__device__ __forceinline__ int Scores<WHOLE>::key_short(unsigned int state, int kp, int Dc) const {
+    const int drop = (int)((state >> RS_DROP) & RS_DROP_MAX), jt = (int)(state & RS_JTOP);
+    const int by_first = drop < (int)RS_DROP_MAX && slope ? kp - slope * drop : RS_LOWEST;
+    const int by_top = (state & RS_FAR) ? (Dc >= RS_LIMIT ? kp : RS_LOWEST) : (slope && jt < RS_LIMIT ? -slope * jt : RS_LOWEST);
+    return max(by_first, by_top);
+}
 __device__ __forceinline__ unsigned int ordered(int v) { return (unsigned int)v ^ 0x80000000u; }
 __device__ __forceinline__ int unordered(unsigned int v) { return (int)(v ^ 0x80000000u); }
 
@@ -598,7 +619,7 @@ struct Folder {
             rows.top[w] = n.top;
             if (!WHOLE) rows.tok[w] = now;
             rows.rec[w] = make_int2(sc.key_a(now), sc.key_b(now, key_top));
-            rows.state[w] = n.jtop | (far ? RS_FAR : 0u) | (full ? RS_FULL : 0u) | (deferred ? RS_DEFERRED : 0u) | (not_over ? RS_NOT_OVER : 0u);
+            rows.state[w] = n.jtop | (drop_of(key_top, n.near0) << RS_DROP) | (far ? RS_FAR : 0u) | (full ? RS_FULL : 0u) | (deferred ? RS_DEFERRED : 0u) | (not_over ? RS_NOT_OVER : 0u);
             if (ADMIT && (state & RS_NOT_OVER) && !not_over) atomicSub(&sh.not_over, 1u);
             st_release(&rows.pending[w], 0u);
         }
@@ -607,14 +628,14 @@ struct Folder {
     // The peak row w would have with the arrival (P, Dc); the row is not pending.
     __device__ __forceinline__ bool scan(int w, int P, int Dc, unsigned int decided, unsigned int& peak) {
         const int lane = threadIdx.x & 31, H = a.H;
+        // the first cells, and what bounds the others: enough when Dc ends among the first and none of the others can be larger
+        const uint2 q = a.near[(size_t)w * 32 + lane];
+        const int j = 2 * lane, lo = RS_NEAR + lane * far_chunks(H) * RS_NEAR;
+        const unsigned int u = a.far[(size_t)w * 32 + lane];
+        peak = __reduce_max_sync(FULL_MASK, max(q.x + (j < Dc ? (unsigned int)(P + j) : 0u), q.y + (j + 1 < Dc ? (unsigned int)(P + j + 1) : 0u)));
+        const bool others = Dc > RS_NEAR || u > peak + (unsigned int)(u ? lo : 0);
+        if (!__any_sync(FULL_MASK, others)) return true;
         if (rows.state[w] & RS_DEFERRED) {
-            // the first cells, and what bounds the others: enough when Dc ends among the first and none of the others can be larger
-            const uint2 q = a.near[(size_t)w * 32 + lane];
-            const int j = 2 * lane, lo = RS_NEAR + lane * far_chunks(H) * RS_NEAR;
-            const unsigned int u = a.far[(size_t)w * 32 + lane];
-            peak = __reduce_max_sync(FULL_MASK, max(q.x + (j < Dc ? (unsigned int)(P + j) : 0u), q.y + (j + 1 < Dc ? (unsigned int)(P + j + 1) : 0u)));
-            const bool others = Dc > RS_NEAR || u > peak + (unsigned int)(u ? lo : 0);
-            if (!__any_sync(FULL_MASK, others)) return true;
             if (!catch_up(w, decided)) return false;
             const RowNumbers n = row_pass<false, false, false, false>(a.curves + (size_t)w * H, H, 0, 0, 0);
             store_numbers(w, n);
@@ -626,16 +647,176 @@ struct Folder {
     }
 };
 
+// ---- an arrival on all rows, by the folding warps together: every fold is done, and the deciding warp waits.  First a look at the
+// rows' keys, each warp at its share; it decides unless the smallest one is only a bound or (binary64) others are as close as its
+// rounding.  A closer look takes the scores of the rows that can be the best, and scans those that are only bounded.
+// What bounds it: the hand-over and one or two passes over the rows' words in shared memory.  By the deciding warp alone the look at the
+// keys took 3,000 cycles with 4,096 rows, and the closer one, taken for all bounded rows and all binary64 scores, 28,000.
+template <int FOLD_WARPS, bool ADMIT, bool WHOLE>
+struct Look {
+    typedef typename Scores<WHOLE>::S S;
+    static constexpr int STRIDE = 32 * FOLD_WARPS;
+    const RouteSumArgs& a;
+    RsShared& sh;
+    const Rows& rows;
+    const Scores<WHOLE>& sc;
+    unsigned int met;
+
+    __device__ __forceinline__ void keys(int me) {
+        constexpr int AT_ONCE = 4;
+        const int lane = threadIdx.x & 31, I = a.I;
+        const int P = sh.look_P, D = sh.look_D, Dc = D < a.H ? D : a.H, kp = sc.key_p(P);
+        int least = 0x7fffffff, next = 0x7fffffff, least_row = RS_NO_ROW;
+        for (int base = 32 * me + lane; base - lane < I; base += AT_ONCE * STRIDE) {
+            int2 r[AT_ONCE];
+            unsigned int st[AT_ONCE];
+            #pragma unroll
+            for (int u = 0; u < AT_ONCE; ++u) {
+                const int i = base + u * STRIDE;
+                r[u] = i < I ? rows.rec[i] : make_int2(RS_ABSENT, RS_LOWEST);
+                st[u] = i < I ? rows.state[i] : RS_FAR | (RS_DROP_MAX << RS_DROP);
+            }
+            #pragma unroll
+            for (int u = 0; u < AT_ONCE; ++u) {
+                const bool reached = !(st[u] & RS_FAR) && Dc > (int)(st[u] & RS_JTOP);
+                const int v = max(r[u].x, r[u].y + (reached ? kp : sc.key_short(st[u], kp, Dc)));
+                const int key = v | (reached || (!(st[u] & RS_FAR) && r[u].y + kp <= r[u].x) ? 1 : 0);    // (or no penalty: the token count)
+                next = min(next, max(least, key));
+                if (key < least) { least = key; least_row = base + u * STRIDE; }      // a lane's rows ascend
+            }
+        }
+        const int best = __reduce_min_sync(FULL_MASK, least);
+        const int win = __reduce_min_sync(FULL_MASK, least == best ? least_row : RS_NO_ROW);
+        next = __reduce_min_sync(FULL_MASK, least_row == win ? next : least);
+        if (lane == 0) sh.look_key[me] = make_int4(best, win, next, 0);
+    }
+    // (deciding warp) The row that the keys decide for, or none.
+    __device__ __forceinline__ int decided_by_keys(int kp) const {
+        const int lane = threadIdx.x & 31, x = lane < FOLD_WARPS ? lane : 0;
+        const int4 k = sh.look_key[x];
+        const int best = __reduce_min_sync(FULL_MASK, k.x), win = __reduce_min_sync(FULL_MASK, k.x == best ? k.y : RS_NO_ROW);
+        const int next = __reduce_min_sync(FULL_MASK, k.y == win ? k.z : k.x);
+        if (!(best & 1) || win >= a.I) return RS_NO_ROW;
+        if (!WHOLE && (next <= best + Scores<WHOLE>::SLACK || best >= RS_CUT || kp >= RS_CUT)) return RS_NO_ROW;
+        return win;
+    }
+    // ---- the closer look
+    __device__ __forceinline__ void arrive() {
+        met += FOLD_WARPS;
+        __syncwarp();
+        acquire_cta();
+        if ((threadIdx.x & 31) == 0) atomicAdd(&sh.look_met, 1u);
+    }
+    __device__ __forceinline__ bool meet() {
+        return rs_wait(sh, [&] { return (int)(ld_acquire(&sh.look_met) - met) >= 0; });
+    }
+    // The least a row's key value can be, and in `most` the largest (but for the rounding of the keys).
+    __device__ __forceinline__ int least_key(int i, int kp, int Dc, int& most) {
+        const int2 r = rows.rec[i];
+        const unsigned int st = rows.state[i];
+        most = max(r.x, ((st & RS_FAR) ? sc.key_b(sc.tokens_of(rows, i), rows.top[i]) : r.y) + kp);
+        return Dc > (int)(st & RS_JTOP) ? most : max(r.x, r.y + sc.key_short(st, kp, Dc));
+    }
+    // The smallest of the warps' scores (lane l has that of warp l), the lowest row among equals.
+    __device__ __forceinline__ void smallest(int stage, S& best, int& win, unsigned int& peak) const {
+        const int lane = threadIdx.x & 31, x = lane < FOLD_WARPS ? lane : 0;
+        S s;
+        if constexpr (WHOLE) s = (S)sh.look_score[stage][x];
+        else s = __longlong_as_double((long long)sh.look_score[stage][x]);
+        const int r = sh.look_row[stage][x];
+        best = Scores<WHOLE>::warp_min(s);
+        win = __reduce_min_sync(FULL_MASK, s == best ? r : RS_NO_ROW);
+        peak = __shfl_sync(FULL_MASK, sh.look_peak[stage][x], __ffs(__ballot_sync(FULL_MASK, s == best && r == win)) - 1);
+    }
+    __device__ __forceinline__ void put(int stage, int me, S best, int win, unsigned int peak) {
+        if ((threadIdx.x & 31) != 0) return;
+        if constexpr (WHOLE) sh.look_score[stage][me] = best;
+        else sh.look_score[stage][me] = (unsigned long long)__double_as_longlong(best);
+        sh.look_row[stage][me] = win;
+        sh.look_peak[stage][me] = peak;
+    }
+    __device__ __forceinline__ bool closely(int me, unsigned int decided) {
+        static_assert((RS_MAX_ROWS + 32 * 6 - 1) / (32 * 6) <= 64, "a bit for each row of a lane");
+        const int lane = threadIdx.x & 31, I = a.I, first = 32 * me + lane;
+        const int P = sh.look_P, D = sh.look_D, Dc = D < a.H ? D : a.H, kp = sc.key_p(P);
+        int least = 0x7fffffff;
+        #pragma unroll 4
+        for (int i = first; i < I; i += STRIDE) {
+            int most;
+            least_key(i, kp, Dc, most);
+            least = min(least, most);
+        }
+        least = __reduce_min_sync(FULL_MASK, least);
+        if (lane == 0) atomicMin(&sh.look_least, ordered(least));
+        arrive();
+        if (!meet()) return false;
+        // (keys that are cut say nothing: then every row counts)
+        const int smallest_most = unordered(sh.look_least);
+        const int reach = !WHOLE && (smallest_most >= RS_CUT || kp >= RS_CUT) ? 0x7fffffff : smallest_most + Scores<WHOLE>::SLACK;
+        S mine = Scores<WHOLE>::none();
+        int mine_row = RS_NO_ROW, n = 0;
+        unsigned int mine_peak = 0;
+        unsigned long long open = 0;       // the lane's rows that are only bounded and could have the smallest score
+        #pragma unroll 2
+        for (int i = first; i < I; i += STRIDE, ++n) {
+            int most;
+            if (least_key(i, kp, Dc, most) > reach) continue;
+            const unsigned int top = rows.top[i];
+            if (Dc > (int)(rows.state[i] & RS_JTOP) || sc.no_penalty(top, P)) {
+                const S s = sc.of_peak(sc.tokens_of(rows, i), top + (unsigned int)P, P, D);
+                // (a lane's rows ascend; the first counts whatever its score, which may be infinite)
+                if (s < mine || mine_row == RS_NO_ROW) { mine = s; mine_row = i; mine_peak = top + (unsigned int)P; }
+            } else open |= 1ull << n;
+        }
+        S best = Scores<WHOLE>::warp_min(mine);
+        int win = __reduce_min_sync(FULL_MASK, mine == best ? mine_row : RS_NO_ROW);
+        unsigned int peak = __shfl_sync(FULL_MASK, mine_peak, __ffs(__ballot_sync(FULL_MASK, mine == best && mine_row == win)) - 1);
+        put(0, me, best, win, peak);
+        arrive();
+        if (__any_sync(FULL_MASK, open != 0)) {
+            if (!meet()) return false;
+            __syncwarp();
+            smallest(0, best, win, peak);
+            for (int x = 0; __any_sync(FULL_MASK, (open >> x) != 0); ++x) {
+                const int i = first + x * STRIDE;
+                bool todo = ((open >> x) & 1) != 0;
+                unsigned int tokens = 0;
+                if (todo) {
+                    const unsigned int top = rows.top[i], st = rows.state[i], drop = (st >> RS_DROP) & RS_DROP_MAX;
+                    unsigned int low = top - (st & RS_JTOP);
+                    if (!(st & RS_FAR) && drop < RS_DROP_MAX) low = max(low, top - drop + (unsigned int)P);
+                    tokens = sc.tokens_of(rows, i);
+                    const S s = sc.of_peak(tokens, low, P, D);
+                    todo = s < best || (s == best && i < win);
+                }
+                for (unsigned int which = __ballot_sync(FULL_MASK, todo); which; which &= which - 1) {
+                    const int src = __ffs(which) - 1, w = __shfl_sync(FULL_MASK, i, src);
+                    const unsigned int t = __shfl_sync(FULL_MASK, tokens, src);
+                    unsigned int p = 0;
+                    Folder<ADMIT, WHOLE> f{a, sh, rows, sc};
+                    if (!f.scan(w, P, Dc, decided, p)) return false;
+                    const S s = sc.of_peak(t, p, P, D);
+                    if (s < best || (s == best && w < win)) { best = s; win = w; peak = p; }
+                }
+                if (x == 63) break;
+            }
+        }
+        put(1, me, best, win, peak);
+        return true;
+    }
+};
+
 template <int FOLD_WARPS, bool ADMIT, bool WHOLE, bool LISTS>
 __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int me) {
     const int lane = threadIdx.x & 31;
     Folder<ADMIT, WHOLE> f{a, sh, rows, sc};
-    unsigned int scans = 0;
+    Look<FOLD_WARPS, ADMIT, WHOLE> look{a, sh, rows, sc, 0u};
+    unsigned int looks = 0;
     for (unsigned int n = me;;) {
         uint4 ctl;
         if (!rs_wait<true>(sh, [&] {
                 ctl = ld_volatile4(&sh.ctl);
-                return (int)(ctl.x - n) > 0 || ctl.y != scans || ctl.z != 0;
+                return (int)(ctl.x - n) > 0 || ctl.y != looks || ctl.z != 0;
             }, LISTS ? 20 : 0))    // (the list warps need the issue slots)
             return;
         acquire_cta();
@@ -645,16 +826,12 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
             n += FOLD_WARPS;
             if (lane == 0) st_release(&sh.done[me], n);
             __syncwarp();
-        } else if (__any_sync(FULL_MASK, ctl.y != scans)) {
-            scans = ctl.y;
-            const int count = sh.scan_n;
-            for (int x = me; x < count; x += FOLD_WARPS) {
-                unsigned int peak = 0;
-                if (!f.scan(sh.scan_row[x], sh.scan_P, sh.scan_Dc, ctl.x, peak)) return;
-                if (lane == 0) sh.peak[x] = peak;
-            }
+        } else if (__any_sync(FULL_MASK, ctl.y != looks)) {
+            looks = ctl.y;
+            if (!sh.look_closely) look.keys(me);
+            else if (!look.closely(me, ctl.x)) return;
             __syncwarp();
-            if (lane == 0) st_release(&sh.scans_done[me], scans);
+            if (lane == 0) st_release(&sh.looks_done[me], looks);
         } else {
             return;
         }
@@ -928,9 +1105,9 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     constexpr unsigned int CHUNK = LISTS ? 32 : 4 * KS;
     // decisions made known to the folding warps at once (few rows: soon)
     constexpr unsigned int PUBLISH = LISTS ? 4 : (KS >= 4 ? 2 : 1);
-    const int lane = threadIdx.x & 31, I = a.I, H = a.H, n_groups = (I + 31) / 32;
+    const int lane = threadIdx.x & 31, I = a.I, H = a.H;
     const int lane_f = lane < FOLD_WARPS ? lane : 0;
-    unsigned int scans = 0;
+    unsigned int looks = 0;
     bool lost = false;
 
     // ---- the rows held by the lane, ascending, and their keys: odd for a row that is marked (pending when the lane last
@@ -1096,108 +1273,37 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             tell(e, win, win, 0u);
             return;
         }
-        // ---- short arrivals and rows that have to be scanned: all rows, with every fold done.  First those with exact scores ...
+        // ---- short arrivals and rows that have to be scanned: all rows, with every fold done
         if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return; }
         acquire_cta();
-        if (WHOLE) {
-            // The keys give the scores of the rows that are not far and whose step the ramp reaches; the others are bounded from
-            // below by the cell that holds their top.  (4,096 rows: 3,000 cycles; 28,000 for what follows.)
-            int least = RS_ABSENT, least_row = RS_NO_ROW;
-            for (int g0 = 0; g0 < n_groups; g0 += 8) {
-                int2 r[8];
-                unsigned int s[8];
-                #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = (g0 + u) * 32 + lane;
-                    r[u] = i < I ? rows.rec[i] : make_int2(RS_ABSENT, RS_LOWEST);
-                    s[u] = i < I ? rows.state[i] : 0u;
-                }
-                #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int jt = (int)(s[u] & RS_JTOP);
-                    const int add = (s[u] & RS_FAR) ? RS_LOWEST : (Dc > jt ? kp : -2 * sc.beta_i * jt);
-                    const int v = (s[u] & RS_FAR) ? r[u].x : max(r[u].x, r[u].y + add);
-                    const bool exact = !(s[u] & RS_FAR) && Dc > jt;
-                    // (bit 30 of the row: only a bound)
-                    if (v < least) { least = v; least_row = ((g0 + u) * 32 + lane) | (exact ? 0 : (int)RS_GIVEN); }     // a lane's rows ascend
-                }
-            }
-            const int best = __reduce_min_sync(FULL_MASK, least);
-            const int win = __reduce_min_sync(FULL_MASK, least == best ? (least_row & ~(int)RS_GIVEN) : RS_NO_ROW);
-            // (rows of the same value that are only bounded need a closer look)
-            if (win < I && !__any_sync(FULL_MASK, least == best && (least_row & (int)RS_GIVEN))) {
-                received(win);
-                tell(e, win, win, 0u);
-                return;
-            }
-        }
-        auto look = [&](int i, S& s, unsigned int& tokens, unsigned int& peak) {   // whether row i's score is exact, and the score (else a lower bound)
-            s = Scores<WHOLE>::none();
-            tokens = peak = 0;
-            if (i >= I) return true;
-            const unsigned int top = rows.top[i], jt = rows.state[i] & RS_JTOP;
-            tokens = sc.tokens_of(rows, i);
-            const bool exact = Dc > (int)jt || sc.no_penalty(top, P);
-            peak = exact ? top + (unsigned int)P : top - jt;     // (jt is at most one step beyond the maximum's)
-            s = sc.of_peak(tokens, peak, P, D);
-            return exact;
-        };
-        S best = Scores<WHOLE>::none(), mine = best;
-        int win = RS_NO_ROW, mine_row = RS_NO_ROW, n_again = 0;
-        unsigned int mine_peak = 0, win_peak = 0;
-        for (int g0 = 0; g0 < n_groups; g0 += 4) {
-            S s[4];
-            unsigned int tokens, peak[4];
-            bool ok[4];
-            #pragma unroll
-            for (int u = 0; u < 4; ++u) ok[u] = look((g0 + u) * 32 + lane, s[u], tokens, peak[u]);
-            #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                // (a lane's rows ascend; the first counts whatever its score, which may be infinite)
-                if (ok[u] && (s[u] < mine || (mine_row == RS_NO_ROW && (g0 + u) * 32 + lane < I))) { mine = s[u]; mine_row = (g0 + u) * 32 + lane; mine_peak = peak[u]; }
-                if (__any_sync(FULL_MASK, !ok[u])) {
-                    if (lane == 0) sh.slow_group[n_again] = (unsigned short)(g0 + u);
-                    ++n_again;
-                }
-            }
-        }
-        __syncwarp();
-        auto take = [&]() {   // the warp's smallest of (mine, mine_row), against the best so far
-            const S smallest = Scores<WHOLE>::warp_min(mine);
-            const int r = __reduce_min_sync(FULL_MASK, mine == smallest ? mine_row : RS_NO_ROW);
-            if (smallest < best || (smallest == best && r < win)) {
-                best = smallest; win = r;
-                const unsigned int who = __ballot_sync(FULL_MASK, mine == smallest && mine_row == r);
-                win_peak = __shfl_sync(FULL_MASK, mine_peak, __ffs(who) - 1);
-            }
-        };
-        take();
-        // ... then those whose bound could beat the best: they are scanned
-        for (int x = 0; x < n_again; ++x) {
-            S s;
-            unsigned int tokens, peak;
-            const int i = (int)sh.slow_group[x] * 32 + lane;
-            const bool ok = look(i, s, tokens, peak);
-            const bool todo = !ok && (s < best || (s == best && i < win));
-            const unsigned int which = __ballot_sync(FULL_MASK, todo);
-            if (!which) continue;
-            const int slot = __popc(which & ((1u << lane) - 1u));
-            if (todo) sh.scan_row[slot] = i;
-            if (lane == 0) { sh.scan_P = P; sh.scan_Dc = Dc; sh.scan_n = __popc(which); }
-            ++scans;
+        const Look<FOLD_WARPS, ADMIT, WHOLE> look{a, sh, rows, sc, 0u};
+        auto folding_warps_look = [&](int closely) {
+            ++looks;
+            if (lane == 0) { sh.look_P = P; sh.look_D = D; sh.look_closely = closely; sh.look_least = 0xffffffffu; }
             __syncwarp();
-            if (lane == 0) st_release(&sh.ctl.y, scans);
-            if (!rs_wait(sh, [&] { return ld_acquire(&sh.scans_done[lane_f]) == scans; })) { lost = true; return; }
-            mine = Scores<WHOLE>::none();
-            mine_row = RS_NO_ROW;
-            if (todo) {
-                mine_peak = sh.peak[slot];
-                mine = sc.of_peak(tokens, mine_peak, P, D);
-                mine_row = i;
+            if (lane == 0) st_release(&sh.ctl.y, looks);
+            if (!rs_wait(sh, [&] { return ld_acquire(&sh.looks_done[lane_f]) == looks; })) lost = true;
+        };
+        folding_warps_look(0);
+        if (lost) return;
+        const int by_keys = look.decided_by_keys(kp);
+        const bool reached = by_keys < I && Dc > (int)(rows.state[by_keys] & RS_JTOP);
+        if (by_keys < I && (WHOLE || reached || sc.no_penalty(rows.top[by_keys], P))) {
+            if (reached) received(by_keys);
+            else {      // (it pays no penalty)
+                #pragma unroll
+                for (int k = 0; k < KS; ++k)
+                    if (row[k] == by_keys) { ra[k] = (ra[k] + kpd) | 1; rb[k] = (rb[k] + kpd) | 1; }
             }
-            take();
-            __syncwarp();
+            tell(e, by_keys, by_keys, 0u);
+            return;
         }
+        folding_warps_look(1);
+        if (lost) return;
+        S best;
+        int win;
+        unsigned int win_peak;
+        look.smallest(1, best, win, win_peak);
         #pragma unroll
         for (int k = 0; k < KS; ++k)
             if (row[k] == win) {      // (a lower bound, odd)
@@ -1497,13 +1603,13 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         sh.n0 = *a.n_requests;
         sh.ctl = make_uint4(0u, 0u, 0u, 0u);
         sh.items_ready = sh.items_end = sh.not_over = sh.jmax = sh.written = sh.flush = 0;
-        sh.lists_wanted = sh.lists_ready = sh.list_met = 0;
+        sh.lists_wanted = sh.lists_ready = sh.list_met = sh.look_met = 0;
         sh.list_n[0] = sh.list_n[1] = 0;
         sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0;
         sh.first_bad = sh.first_full = 0x7fffffff;
     }
     for (int i = tid; i < RS_ITEMS; i += THREADS) sh.items[i] = make_int4(0, 0, 0, 0);    // (an item is fetched before it is known to be there)
-    if (tid < RS_MAX_FOLD_WARPS) { sh.done[tid] = (unsigned int)tid; sh.scans_done[tid] = 0; }
+    if (tid < RS_MAX_FOLD_WARPS) { sh.done[tid] = (unsigned int)tid; sh.looks_done[tid] = 0; }
     if (tid < RS_PROBES) sh.probe_t[tid] = 0xffffffffu;
     // ADMIT: the requests that were waiting when the call was made come first, then the arrivals
     long long q_head = 0, q_len = 0;
@@ -1553,14 +1659,14 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
                 q = a.summary0[i];
                 if (ADMIT) above = a.over0[i];
             }
-            const unsigned int jtop = q.z & 0xffffu, step = q.z >> 16;
+            const unsigned int jtop = q.z & 0xffffu, step = (q.z >> 16) & 31u, drop = q.z >> 21;
             const bool far = jtop >= (unsigned int)RS_LIMIT;
             jmax = max(jmax, far ? step : jtop);
             const bool not_over = ADMIT && !((double)above > a.many);
             free_rows += not_over;
             const int2 rec = make_int2(sc.key_a(q.x), sc.key_b(q.x, far ? q.w : q.y));
             rows.rec[i] = rec;
-            rows.state[i] = jtop | (far ? RS_FAR : 0u) | (jtop >= (unsigned int)RS_NEAR ? RS_FULL : 0u) | (not_over ? RS_NOT_OVER : 0u);
+            rows.state[i] = jtop | (drop << RS_DROP) | (far ? RS_FAR : 0u) | (jtop >= (unsigned int)RS_NEAR ? RS_FULL : 0u) | (not_over ? RS_NOT_OVER : 0u);
             rows.top[i] = q.y;
             rows.pending[i] = 0;
             if (!WHOLE) rows.tok[i] = q.x;
