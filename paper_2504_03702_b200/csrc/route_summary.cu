@@ -57,6 +57,7 @@ constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding
 constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lane, 8 beyond RS_LONG_LISTS instances)
 constexpr int RS_LONG_LISTS = 2048;
 constexpr int RS_NEAR_ROWS = 2304;          // rows the list warps keep for a closer look at once
+constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding warp looks at their keys by itself (as fast at 4,096)
 constexpr int RS_PROBES = 8;                // prompt lengths for which a list has the best rows
 constexpr int RS_NEAR = 64;                 // steps kept exactly; the rest in 32 stretches of whole chunks of as many steps
 // A row whose top lies further out than this is "far": the deciding warp has only a lower bound of its score, and the
@@ -319,6 +320,9 @@ struct RouteSumArgs {
     const int32_t* over0;          // [I] steps above the level per row, from the summarising kernel
 };
 
+// What the deciding warp can ask of the folding warps: the peaks of some rows, or a look at all rows.
+constexpr int RS_SCANS = 0, RS_KEYS = 1, RS_CLOSELY = 2;
+
 // Rows in shared memory (structure of arrays):
 //   rec    {a, b}, even: the score of an arrival is at least max(a, b + what its prompt adds), and that but for the rounding
 //          of the keys unless the row is far or pending
@@ -357,8 +361,10 @@ struct RsShared {
     unsigned int lists_wanted, lists_ready;
     unsigned int done[RS_MAX_FOLD_WARPS];   // the next decision each folding warp will fold
     unsigned int looks_done[RS_MAX_FOLD_WARPS];
-    int look_P, look_D, look_closely;
+    int look_P, look_D, look_how;           // RS_SCANS, RS_KEYS or RS_CLOSELY
     int4 look_key[RS_MAX_FOLD_WARPS];       // smallest key of a warp's rows (odd: exact), the row, the next smallest key
+    int scan_n, scan_row[32];
+    unsigned int scan_peak[32];
     unsigned int look_met, look_least;      // (a closer look) arrivals at the meetings; smallest key that a row has at most
     unsigned long long look_score[2][RS_MAX_FOLD_WARPS];   // the smallest score of a warp's rows, before and after the scans, as its bits,
     int look_row[2][RS_MAX_FOLD_WARPS];                    // the row that has it
@@ -662,17 +668,18 @@ struct Look {
     const Scores<WHOLE>& sc;
     unsigned int met;
 
-    __device__ __forceinline__ void keys(int me) {
-        constexpr int AT_ONCE = 4;
+    // The rows from `start` on, 32 of every EACH: {smallest key, odd if exact; its row; the next smallest key}.
+    template <int EACH, int AT_ONCE>
+    __device__ __forceinline__ int4 keys(int start, int P, int D) const {
         const int lane = threadIdx.x & 31, I = a.I;
-        const int P = sh.look_P, D = sh.look_D, Dc = D < a.H ? D : a.H, kp = sc.key_p(P);
+        const int Dc = D < a.H ? D : a.H, kp = sc.key_p(P);
         int least = 0x7fffffff, next = 0x7fffffff, least_row = RS_NO_ROW;
-        for (int base = 32 * me + lane; base - lane < I; base += AT_ONCE * STRIDE) {
+        for (int base = start + lane; base - lane < I; base += AT_ONCE * EACH) {
             int2 r[AT_ONCE];
             unsigned int st[AT_ONCE];
             #pragma unroll
             for (int u = 0; u < AT_ONCE; ++u) {
-                const int i = base + u * STRIDE;
+                const int i = base + u * EACH;
                 r[u] = i < I ? rows.rec[i] : make_int2(RS_ABSENT, RS_LOWEST);
                 st[u] = i < I ? rows.state[i] : RS_FAR | (RS_DROP_MAX << RS_DROP);
             }
@@ -681,24 +688,28 @@ struct Look {
                 const bool reached = !(st[u] & RS_FAR) && Dc > (int)(st[u] & RS_JTOP);
                 const int v = max(r[u].x, r[u].y + (reached ? kp : sc.key_short(st[u], kp, Dc)));
                 const int key = v | (reached || (!(st[u] & RS_FAR) && r[u].y + kp <= r[u].x) ? 1 : 0);    // (or no penalty: the token count)
-                next = min(next, max(least, key));
-                if (key < least) { least = key; least_row = base + u * STRIDE; }      // a lane's rows ascend
+                if (!WHOLE) next = min(next, max(least, key));
+                if (key < least) { least = key; least_row = base + u * EACH; }      // a lane's rows ascend
             }
         }
         const int best = __reduce_min_sync(FULL_MASK, least);
         const int win = __reduce_min_sync(FULL_MASK, least == best ? least_row : RS_NO_ROW);
-        next = __reduce_min_sync(FULL_MASK, least_row == win ? next : least);
-        if (lane == 0) sh.look_key[me] = make_int4(best, win, next, 0);
+        if (!WHOLE) next = __reduce_min_sync(FULL_MASK, least_row == win ? next : least);
+        return make_int4(best, win, next, 0);
     }
-    // (deciding warp) The row that the keys decide for, or none.
-    __device__ __forceinline__ int decided_by_keys(int kp) const {
-        const int lane = threadIdx.x & 31, x = lane < FOLD_WARPS ? lane : 0;
-        const int4 k = sh.look_key[x];
+    // Whether such keys decide: a whole-number key that is exact does, one in binary64 if no other is as close as its rounding.
+    __device__ __forceinline__ bool decide(const int4& k, int kp, int P, int Dc) const {
+        if (!(k.x & 1) || k.y >= a.I) return false;
+        if (WHOLE) return true;
+        if (k.z <= k.x + Scores<WHOLE>::SLACK || k.x >= RS_CUT || kp >= RS_CUT) return false;
+        return Dc > (int)(rows.state[k.y] & RS_JTOP) || sc.no_penalty(rows.top[k.y], P);
+    }
+    // (deciding warp) The keys of all folding warps together.
+    __device__ __forceinline__ int4 all_keys() const {
+        const int lane = threadIdx.x & 31;
+        const int4 k = sh.look_key[lane < FOLD_WARPS ? lane : 0];
         const int best = __reduce_min_sync(FULL_MASK, k.x), win = __reduce_min_sync(FULL_MASK, k.x == best ? k.y : RS_NO_ROW);
-        const int next = __reduce_min_sync(FULL_MASK, k.y == win ? k.z : k.x);
-        if (!(best & 1) || win >= a.I) return RS_NO_ROW;
-        if (!WHOLE && (next <= best + Scores<WHOLE>::SLACK || best >= RS_CUT || kp >= RS_CUT)) return RS_NO_ROW;
-        return win;
+        return make_int4(best, win, __reduce_min_sync(FULL_MASK, k.y == win ? k.z : k.x), 0);
     }
     // ---- the closer look
     __device__ __forceinline__ void arrive() {
@@ -716,6 +727,12 @@ struct Look {
         const unsigned int st = rows.state[i];
         most = max(r.x, ((st & RS_FAR) ? sc.key_b(sc.tokens_of(rows, i), rows.top[i]) : r.y) + kp);
         return Dc > (int)(st & RS_JTOP) ? most : max(r.x, r.y + sc.key_short(st, kp, Dc));
+    }
+    // The least that row i's peak can be: the cell of its top, or the first cell with the prompt.
+    __device__ __forceinline__ unsigned int least_peak(int i, int P) const {
+        const unsigned int top = rows.top[i], st = rows.state[i], drop = (st >> RS_DROP) & RS_DROP_MAX;
+        const unsigned int low = top - (st & RS_JTOP);
+        return !(st & RS_FAR) && drop < RS_DROP_MAX ? max(low, top - drop + (unsigned int)P) : low;
     }
     // The smallest of the warps' scores (lane l has that of warp l), the lowest row among equals.
     __device__ __forceinline__ void smallest(int stage, S& best, int& win, unsigned int& peak) const {
@@ -782,11 +799,8 @@ struct Look {
                 bool todo = ((open >> x) & 1) != 0;
                 unsigned int tokens = 0;
                 if (todo) {
-                    const unsigned int top = rows.top[i], st = rows.state[i], drop = (st >> RS_DROP) & RS_DROP_MAX;
-                    unsigned int low = top - (st & RS_JTOP);
-                    if (!(st & RS_FAR) && drop < RS_DROP_MAX) low = max(low, top - drop + (unsigned int)P);
                     tokens = sc.tokens_of(rows, i);
-                    const S s = sc.of_peak(tokens, low, P, D);
+                    const S s = sc.of_peak(tokens, least_peak(i, P), P, D);
                     todo = s < best || (s == best && i < win);
                 }
                 for (unsigned int which = __ballot_sync(FULL_MASK, todo); which; which &= which - 1) {
@@ -828,8 +842,18 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
             __syncwarp();
         } else if (__any_sync(FULL_MASK, ctl.y != looks)) {
             looks = ctl.y;
-            if (!sh.look_closely) look.keys(me);
-            else if (!look.closely(me, ctl.x)) return;
+            const int how = sh.look_how;
+            if (!LISTS && how == RS_SCANS) {
+                const int P = sh.look_P, Dc = sh.look_D < a.H ? sh.look_D : a.H, count = sh.scan_n;
+                for (int x = me; x < count; x += FOLD_WARPS) {
+                    unsigned int peak = 0;
+                    if (!f.scan(sh.scan_row[x], P, Dc, ctl.x, peak)) return;
+                    if (lane == 0) sh.scan_peak[x] = peak;
+                }
+            } else if (LISTS && how == RS_KEYS) {
+                const int4 k = look.template keys<32 * FOLD_WARPS, 4>(32 * me, sh.look_P, sh.look_D);
+                if (lane == 0) sh.look_key[me] = k;
+            } else if (!look.closely(me, ctl.x)) return;
             __syncwarp();
             if (lane == 0) st_release(&sh.looks_done[me], looks);
         } else {
@@ -1201,6 +1225,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         const int4 it = sh.items[e % RS_ITEMS];
         const int2 pd = sh.raw[e % RS_ITEMS];
         const int P = pd.x, D = pd.y, Dc = D < H ? D : H, kp = it.x, kpd = it.y;
+        const Look<FOLD_WARPS, ADMIT, WHOLE> look{a, sh, rows, sc, 0u};
         publish(e);
         auto received = [&](int win) {     // the arrival's ramp reaches the step of the row's b
             #pragma unroll
@@ -1273,32 +1298,140 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             tell(e, win, win, 0u);
             return;
         }
-        // ---- short arrivals and rows that have to be scanned: all rows, with every fold done
-        if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return; }
-        acquire_cta();
-        const Look<FOLD_WARPS, ADMIT, WHOLE> look{a, sh, rows, sc, 0u};
-        auto folding_warps_look = [&](int closely) {
+        auto folding_warps_look = [&](int how) {
             ++looks;
-            if (lane == 0) { sh.look_P = P; sh.look_D = D; sh.look_closely = closely; sh.look_least = 0xffffffffu; }
+            if (lane == 0) { sh.look_P = P; sh.look_D = D; sh.look_how = how; sh.look_least = 0xffffffffu; }
             __syncwarp();
             if (lane == 0) st_release(&sh.ctl.y, looks);
             if (!rs_wait(sh, [&] { return ld_acquire(&sh.looks_done[lane_f]) == looks; })) lost = true;
         };
-        folding_warps_look(0);
-        if (lost) return;
-        const int by_keys = look.decided_by_keys(kp);
-        const bool reached = by_keys < I && Dc > (int)(rows.state[by_keys] & RS_JTOP);
-        if (by_keys < I && (WHOLE || reached || sc.no_penalty(rows.top[by_keys], P))) {
-            if (reached) received(by_keys);
-            else {      // (it pays no penalty)
+        // A held row takes the arrival without its ramp being known to reach the step of the row's b.
+        auto received_some = [&](int win) {
+            #pragma unroll
+            for (int k = 0; k < KS; ++k)
+                if (row[k] == win) { ra[k] = (ra[k] + kpd) | 1; rb[k] = (rb[k] + kpd) | 1; }
+        };
+        if (!LISTS) {
+            // ---- short arrivals and rows that are only bounded, among all rows: nothing is waited for but what can be the best
+            while (WHOLE || kp < RS_CUT) {
+                // The rows that can have the smallest score: those whose least value (a held row's keys grow with what it has received,
+                // the drop in its state is that of its last fold or a later one) is within the slack of the smallest one that a row
+                // has at most.
+                int v[KS], least = RS_ABSENT;
                 #pragma unroll
-                for (int k = 0; k < KS; ++k)
-                    if (row[k] == by_keys) { ra[k] = (ra[k] + kpd) | 1; rb[k] = (rb[k] + kpd) | 1; }
+                for (int k = 0; k < KS; ++k) {
+                    int add = kp, most = max(ra[k], rb[k] + kp);
+                    if (row[k] != NO_ROW) {
+                        const unsigned int st = ld_volatile(rows.state + row[k]);
+                        if ((st & RS_FAR) || Dc <= (int)(st & RS_JTOP)) add = sc.key_short(st, kp, Dc);
+                    }
+                    if (ra[k] & 1) {
+                        most = RS_ABSENT;
+                        if (!ld_acquire(rows.pending + row[k])) {
+                            const unsigned int tokens = sc.tokens_of(rows, row[k]);
+                            most = max(sc.key_a(tokens), sc.key_b(tokens, rows.top[row[k]]) + kp);
+                        }
+                    }
+                    v[k] = max(ra[k], rb[k] + add);
+                    least = min(least, most);
+                }
+                const int reach = __reduce_min_sync(FULL_MASK, least) + SLACK;
+                if (reach >= (WHOLE ? RS_ABSENT : RS_CUT)) {   // no row to measure by, or one whose keys are cut
+                    const unsigned int before = held_pending();
+                    if (!__any_sync(FULL_MASK, before != 0)) break;
+                    if (!rs_wait(sh, [&] { return __any_sync(FULL_MASK, held_pending() != before) != 0; })) { lost = true; return; }
+                    refresh();
+                    continue;
+                }
+                S mine = Scores<WHOLE>::none();
+                int mine_row = NO_ROW;
+                unsigned int open = 0, reached = 0;     // (of the lane's rows) only bounded; the ramp reaches the step of the top
+                bool wait = false;
+                #pragma unroll
+                for (int k = 0; k < KS; ++k) {
+                    if (v[k] <= reach && row[k] != NO_ROW) {
+                        const int i = row[k];
+                        if (ld_acquire(rows.pending + i)) wait = true;
+                        else {
+                            const unsigned int top = rows.top[i], jt = rows.state[i] & RS_JTOP;
+                            if (Dc > (int)jt) reached |= 1u << k;
+                            if (Dc > (int)jt || sc.no_penalty(top, P)) {
+                                const S s = sc.of_peak(sc.tokens_of(rows, i), top + (unsigned int)P, P, D);
+                                if (s < mine || (s == mine && i < mine_row)) { mine = s; mine_row = i; }
+                            } else open |= 1u << k;
+                        }
+                    }
+                }
+                if (__any_sync(FULL_MASK, wait)) {
+                    if (!rs_wait(sh, [&] {
+                            bool pending = false;
+                            #pragma unroll
+                            for (int k = 0; k < KS; ++k)
+                                if (v[k] <= reach && row[k] != NO_ROW) pending |= ld_acquire(rows.pending + row[k]) != 0;
+                            return !pending;
+                        })) { lost = true; return; }
+                    refresh();
+                    continue;
+                }
+                S best = Scores<WHOLE>::warp_min(mine);
+                int win = __reduce_min_sync(FULL_MASK, mine == best ? mine_row : NO_ROW);
+                unsigned int peak = 0;
+                bool scanned = false;
+                if (__any_sync(FULL_MASK, open != 0)) {    // bounded rows that could be better are scanned
+                    #pragma unroll 1
+                    for (int k = 0; k < KS; ++k) {
+                        const int i = k * 32 + lane;       // (all rows are held: row[k])
+                        bool todo = ((open >> k) & 1) != 0;
+                        unsigned int tokens = 0;
+                        if (todo) {
+                            tokens = sc.tokens_of(rows, i);
+                            const S s = sc.of_peak(tokens, look.least_peak(i, P), P, D);
+                            todo = s < best || (s == best && i < win);
+                        }
+                        const unsigned int which = __ballot_sync(FULL_MASK, todo);
+                        if (!which) continue;
+                        const int slot = __popc(which & ((1u << lane) - 1u));
+                        if (todo) sh.scan_row[slot] = i;
+                        if (lane == 0) sh.scan_n = __popc(which);
+                        folding_warps_look(RS_SCANS);
+                        if (lost) return;
+                        const unsigned int p = todo ? sh.scan_peak[slot] : 0u;
+                        const S s = todo ? sc.of_peak(tokens, p, P, D) : Scores<WHOLE>::none();
+                        const S smallest = Scores<WHOLE>::warp_min(s);
+                        const int r = __reduce_min_sync(FULL_MASK, todo && s == smallest ? i : NO_ROW);
+                        if (smallest < best || (smallest == best && r < win)) {
+                            best = smallest; win = r; scanned = true;
+                            peak = __shfl_sync(FULL_MASK, p, r & 31);
+                        }
+                        __syncwarp();
+                    }
+                }
+                if (win >= I) break;
+                if (!scanned && __any_sync(FULL_MASK, mine_row == win && ((reached >> (win >> 5)) & 1))) received(win);
+                else received_some(win);
+                tell(e, win, scanned ? win | (int)RS_GIVEN : win, peak);
+                return;
             }
-            tell(e, by_keys, by_keys, 0u);
-            return;
         }
-        folding_warps_look(1);
+        // ---- rows outside the list could do as well, or keys are cut: all rows, with every fold done
+        if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return; }
+        acquire_cta();
+        if (LISTS) {
+            int4 k;
+            if (I <= RS_OWN_LOOK) k = look.template keys<32, 8>(0, P, D);
+            else {
+                folding_warps_look(RS_KEYS);
+                if (lost) return;
+                k = look.all_keys();
+            }
+            if (look.decide(k, kp, P, Dc)) {
+                if (Dc > (int)(rows.state[k.y] & RS_JTOP)) received(k.y);
+                else received_some(k.y);      // (it pays no penalty)
+                tell(e, k.y, k.y, 0u);
+                return;
+            }
+        }
+        folding_warps_look(RS_CLOSELY);
         if (lost) return;
         S best;
         int win;
