@@ -57,7 +57,7 @@ constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding
 constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lane, 8 beyond RS_LONG_LISTS instances)
 constexpr int RS_LONG_LISTS = 2048;
 constexpr int RS_NEAR_ROWS = 2304;          // rows the list warps keep for a closer look at once
-constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding warp looks at their keys by itself (as fast at 4,096)
+constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding warp looks at their keys by itself
 constexpr int RS_PROBES = 8;                // prompt lengths for which a list has the best rows
 constexpr int RS_NEAR = 64;                 // steps kept exactly; the rest in 32 stretches of whole chunks of as many steps
 // A row whose top lies further out than this is "far": the deciding warp has only a lower bound of its score, and the
@@ -495,9 +495,10 @@ template <bool WHOLE> struct Scores {
     __device__ __forceinline__ int key_pd(int P, int D) const {
         return WHOLE ? 2 * (P + D) : (int)min((long long)(P + D) << (shift + 1), (long long)RS_CUT);
     }
-    // The least that an arrival whose ramp may end before the step of the top, Dc <= jtop, adds to b: the first cell has its
-    // prompt, and unless the row is far the cell of the top has what it had; the ramp reaches all of the first steps, or not.
-    __device__ __forceinline__ int key_short(unsigned int state, int kp, int Dc) const;
+    // The least that an arrival adds to b, and that but for the rounding when its ramp reaches the step of the top (`exact`).  Else
+    // the first cell has its prompt, and unless the row is far the cell of the top has what it had; or the ramp reaches all of
+    // the first steps.  (Selects and no branches: with them a row cost the looking warp 150 cycles.)
+    __device__ __forceinline__ int key_least(unsigned int state, int kp, int Dc, int& exact) const;
     // whether the keys of 32 such arrivals in a row stay below their cut
     __device__ __forceinline__ bool usual(int kp, int kpd) const { return WHOLE || kp + kpd <= 16777216; }
     __device__ __forceinline__ unsigned int tokens_of(const Rows& rows, int i) const { return WHOLE ? (unsigned int)rows.rec[i].x >> 1 : rows.tok[i]; }
@@ -527,11 +528,14 @@ template <bool WHOLE> struct Scores {
     }
 };
 template <bool WHOLE>
-__device__ __forceinline__ int Scores<WHOLE>::key_short(unsigned int state, int kp, int Dc) const {
-    const int drop = (int)((state >> RS_DROP) & RS_DROP_MAX), jt = (int)(state & RS_JTOP);
-    const int by_first = drop < (int)RS_DROP_MAX && slope ? kp - slope * drop : RS_LOWEST;
-    const int by_top = (state & RS_FAR) ? (Dc >= RS_LIMIT ? kp : RS_LOWEST) : (slope && jt < RS_LIMIT ? -slope * jt : RS_LOWEST);
-    return max(by_first, by_top);
+__device__ __forceinline__ int Scores<WHOLE>::key_least(unsigned int state, int kp, int Dc, int& exact) const {
+    const int drop = (int)((state >> RS_DROP) & RS_DROP_MAX), jt = (int)(state & RS_JTOP), near = (state & RS_FAR) ? 0 : 1;
+    const int no_drop = slope ? (int)RS_DROP_MAX : 0, far_add = Dc >= RS_LIMIT ? kp : RS_LOWEST, jt_max = slope ? RS_LIMIT : 0;
+    const int by_first = drop < no_drop ? kp - slope * drop : RS_LOWEST;
+    const int by_top = jt < jt_max ? -slope * jt : RS_LOWEST;
+    exact = near & (Dc > jt ? 1 : 0);
+    const int least = max(by_first, near ? by_top : far_add);
+    return exact ? kp : least;
 }
 __device__ __forceinline__ unsigned int ordered(int v) { return (unsigned int)v ^ 0x80000000u; }
 __device__ __forceinline__ int unordered(unsigned int v) { return (int)(v ^ 0x80000000u); }
@@ -685,11 +689,13 @@ struct Look {
             }
             #pragma unroll
             for (int u = 0; u < AT_ONCE; ++u) {
-                const bool reached = !(st[u] & RS_FAR) && Dc > (int)(st[u] & RS_JTOP);
-                const int v = max(r[u].x, r[u].y + (reached ? kp : sc.key_short(st[u], kp, Dc)));
-                const int key = v | (reached || (!(st[u] & RS_FAR) && r[u].y + kp <= r[u].x) ? 1 : 0);    // (or no penalty: the token count)
+                int exact;
+                const int add = sc.key_least(st[u], kp, Dc, exact), v = max(r[u].x, r[u].y + add);
+                const int free = ((st[u] & RS_FAR) ? 0 : 1) & (r[u].y + kp <= r[u].x ? 1 : 0);      // (no penalty: the token count)
+                const int key = v | exact | free;
                 if (!WHOLE) next = min(next, max(least, key));
-                if (key < least) { least = key; least_row = base + u * EACH; }      // a lane's rows ascend
+                least_row = key < least ? base + u * EACH : least_row;      // a lane's rows ascend
+                least = min(least, key);
             }
         }
         const int best = __reduce_min_sync(FULL_MASK, least);
@@ -726,7 +732,9 @@ struct Look {
         const int2 r = rows.rec[i];
         const unsigned int st = rows.state[i];
         most = max(r.x, ((st & RS_FAR) ? sc.key_b(sc.tokens_of(rows, i), rows.top[i]) : r.y) + kp);
-        return Dc > (int)(st & RS_JTOP) ? most : max(r.x, r.y + sc.key_short(st, kp, Dc));
+        int exact;
+        const int add = sc.key_least(st, kp, Dc, exact);
+        return Dc > (int)(st & RS_JTOP) ? most : max(r.x, r.y + add);
     }
     // The least that row i's peak can be: the cell of its top, or the first cell with the prompt.
     __device__ __forceinline__ unsigned int least_peak(int i, int P) const {
@@ -1320,11 +1328,8 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 int v[KS], least = RS_ABSENT;
                 #pragma unroll
                 for (int k = 0; k < KS; ++k) {
-                    int add = kp, most = max(ra[k], rb[k] + kp);
-                    if (row[k] != NO_ROW) {
-                        const unsigned int st = ld_volatile(rows.state + row[k]);
-                        if ((st & RS_FAR) || Dc <= (int)(st & RS_JTOP)) add = sc.key_short(st, kp, Dc);
-                    }
+                    int exact, most = max(ra[k], rb[k] + kp);
+                    const int add = sc.key_least(row[k] != NO_ROW ? ld_volatile(rows.state + row[k]) : 0u, kp, Dc, exact);
                     if (ra[k] & 1) {
                         most = RS_ABSENT;
                         if (!ld_acquire(rows.pending + row[k])) {
