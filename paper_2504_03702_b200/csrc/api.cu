@@ -40,6 +40,8 @@ void release(pre_ctx* c) {
     cudaFree(c->d_rs_over);
     cudaFree(c->d_rs_near);
     cudaFree(c->d_rs_far);
+    cudaFree(c->d_rs_link);
+    cudaFree(c->d_rs_newest);
     cudaFree(c->d_rs_applied);
     cudaFree(c->d_rs_ramps);
     cudaFree(c->d_rs_guard);
@@ -131,6 +133,8 @@ int pre_create(const pre_config* cfg, pre_ctx** out) {
         if (e == cudaSuccess) e = alloc_zero(&c->d_rs_over, (size_t)I);
         if (e == cudaSuccess) e = alloc_zero(&c->d_rs_near, (size_t)64 * I);
         if (e == cudaSuccess) e = alloc_zero(&c->d_rs_far, (size_t)32 * I);
+        if (e == cudaSuccess) e = alloc_zero(&c->d_rs_link, (size_t)cfg->max_requests);
+        if (e == cudaSuccess) e = alloc_zero(&c->d_rs_newest, (size_t)I);
         if (e == cudaSuccess) e = alloc_zero(&c->d_rs_applied, (size_t)cfg->max_requests);
         if (e == cudaSuccess) e = alloc_zero(&c->d_rs_ramps, 2);
     }

@@ -74,6 +74,8 @@ struct pre_ctx {
     unsigned long long* d_rs_summary;   // [I] {token count, largest cell + step, its first step, the same of the first steps} per row (16 bytes)
     unsigned int* d_rs_near;        // [I][64] a row's first cells during a batch
     unsigned int* d_rs_far;         // [I][32] bounds of cell + step of the others
+    unsigned int* d_rs_link;        // [max_requests] the requests of a batch chained per row
+    unsigned int* d_rs_newest;      // [I] where the chains begin
     unsigned char* d_rs_applied;    // [max_requests] 1: the map has this request of the batch already (zero between calls)
     long long* d_rs_ramps;          // {first table row, rows} whose ramps the maps lack after the routing kernel
     int32_t* d_rs_over;             // [I] steps of a row above the overload level (admission queue)

@@ -72,7 +72,7 @@ constexpr int RS_NO_ROW = 0x3fffffff;
 constexpr int RS_ALONE_ROWS = 64;                  // small shapes: instances,
 constexpr long long RS_ALONE_CELLS = 32768;        // cells of the maps,
 constexpr long long RS_OWN_RAMP_CELLS = 65536;     // and arrivals x steps up to which the routing block adds the ramps
-constexpr unsigned int RS_GIVEN = 0x40000000u;
+constexpr unsigned int RS_GIVEN = 0x40000000u, RS_NOBODY = 0xffffffffu;
 constexpr unsigned int FULL_MASK = 0xffffffffu;
 
 // guard words written by the summarising kernel; the routing kernel clears them for the next call
@@ -91,11 +91,31 @@ struct RowNumbers {
 
 __device__ __forceinline__ int far_chunks(int H) { return max(1, (((H + RS_NEAR - 1) / RS_NEAR - 1) + 31) / 32); }   // chunks per stretch
 
-// One pass over a row by one warp.  RAMP: with the arrival (P, Dc) added; STORE: and written back.  16-byte accesses when H
-// is even (a lane holds two neighbouring cells, the warp 512 contiguous bytes), eight in flight per lane.
-// CHECK: the cells may hold anything.
-template <bool RAMP, bool STORE, bool COUNT, bool CHECK>
-__device__ __forceinline__ RowNumbers row_pass(int64_t* row, int H, int P, int Dc, long long hot) {
+__device__ __forceinline__ longlong2 load_pair(const int64_t* p, bool ok, bool stream) {
+    longlong2 v;
+    if (stream) asm volatile("{ .reg .pred p; setp.ne.s32 p, %3, 0; mov.u64 %0, 0; mov.u64 %1, 0; @p ld.global.cs.v2.u64 {%0, %1}, [%2]; }" : "=l"(v.x), "=l"(v.y) : "l"(p), "r"((int)ok) : "memory");
+    else asm volatile("{ .reg .pred p; setp.ne.s32 p, %3, 0; mov.u64 %0, 0; mov.u64 %1, 0; @p ld.global.v2.u64 {%0, %1}, [%2]; }" : "=l"(v.x), "=l"(v.y) : "l"(p), "r"((int)ok) : "memory");
+    return v;
+}
+__device__ __forceinline__ long long load_one(const int64_t* p, bool ok) {
+    long long v;
+    asm volatile("{ .reg .pred p; setp.ne.s32 p, %2, 0; mov.u64 %0, 0; @p ld.global.u64 %0, [%1]; }" : "=l"(v) : "l"(p), "r"((int)ok) : "memory");
+    return v;
+}
+__device__ __forceinline__ void store_pair(int64_t* p, unsigned int c0, unsigned int c1, bool ok) {
+    asm volatile("{ .reg .pred p; setp.ne.s32 p, %3, 0; @p st.global.v2.u64 [%0], {%1, %2}; }" ::"l"(p), "l"((long long)c0), "l"((long long)c1), "r"((int)ok) : "memory");
+}
+__device__ __forceinline__ void store_one(int64_t* p, unsigned int c, bool ok) {
+    asm volatile("{ .reg .pred p; setp.ne.s32 p, %2, 0; @p st.global.u64 [%0], %1; }" ::"l"(p), "l"((long long)c), "r"((int)ok) : "memory");
+}
+
+// One pass over a row by one warp.  RAMP: with the ramps of `count` arrivals added, lane s having the s-th's (P, Dc), and written back
+// if `store`.  16-byte accesses when H is even (a lane holds two neighbouring cells, the warp 512 contiguous bytes), eight in
+// flight per lane.  CHECK: the cells may hold anything.
+// What bounds it is the latency of the row's cells (600 to 1,000 cycles from L2) and that of the warp's own instructions: all of
+// them are under predicates, the branches per 64 cells made it three times as long (1,024 cells: 8,800 cycles, 2,800 so).
+template <bool RAMP, bool COUNT, bool CHECK>
+__device__ __forceinline__ RowNumbers row_pass(int64_t* row, int H, int P, int Dc, int count, bool store, long long hot) {
     constexpr int BATCH = 8;
     const int lane = threadIdx.x & 31;
     const bool vec = (H & 1) == 0;
@@ -103,55 +123,80 @@ __device__ __forceinline__ RowNumbers row_pass(int64_t* row, int H, int P, int D
     RowNumbers n;
     n.near0 = n.near1 = n.far = n.peak = 0;
     n.above = 0;
-    n.bad = false;
-    unsigned int top = 0, jtop = 0;
+    unsigned int top = 0, jtop = 0, bad = 0;
+    const int longest = RAMP ? __reduce_max_sync(FULL_MASK, lane < count ? Dc : 0) : 0;
+    int stretch = -1, in_stretch = per - 1;     // of the chunk of 64 cells (the first one belongs to none)
     #pragma unroll 1
     for (int base = 0; base < H; base += BATCH * RS_NEAR) {
-        long long v[2 * BATCH];
+        unsigned int c[2 * BATCH];
+        {
+            longlong2 v[BATCH];
+            if (vec) {
+                #pragma unroll
+                for (int u = 0; u < BATCH; ++u) {
+                    const int j = base + u * RS_NEAR + 2 * lane;
+                    v[u] = load_pair(row + j, j < H, CHECK);
+                }
+            } else {
+                #pragma unroll
+                for (int u = 0; u < BATCH; ++u) {
+                    const int j = base + u * RS_NEAR + 2 * lane;
+                    v[u].x = load_one(row + j, j < H);
+                    v[u].y = load_one(row + j + 1, j + 1 < H);
+                }
+            }
+            #pragma unroll
+            for (int u = 0; u < BATCH; ++u) {
+                c[2 * u] = (unsigned int)v[u].x; c[2 * u + 1] = (unsigned int)v[u].y;
+                if (CHECK) bad |= (unsigned int)((unsigned long long)(v[u].x | v[u].y) >> 32);     // (cells beyond H are zero)
+            }
+        }
+        if (RAMP && base < longest) {
+            #pragma unroll 1
+            for (int s = 0; s < count; ++s) {
+                const int p = __shfl_sync(FULL_MASK, P, s), d = __shfl_sync(FULL_MASK, Dc, s);
+                #pragma unroll
+                for (int u = 0; u < BATCH; ++u) {
+                    const int j = base + u * RS_NEAR + 2 * lane;
+                    c[2 * u] += j < d ? (unsigned int)(p + j) : 0u;
+                    c[2 * u + 1] += j + 1 < d ? (unsigned int)(p + j + 1) : 0u;
+                }
+            }
+            if (store && vec) {      // (a cell behind the end of the ramps is written back unchanged)
+                #pragma unroll
+                for (int u = 0; u < BATCH; ++u) {
+                    const int j = base + u * RS_NEAR + 2 * lane;
+                    store_pair(row + j, c[2 * u], c[2 * u + 1], j < longest);
+                }
+            } else if (store) {
+                #pragma unroll
+                for (int u = 0; u < BATCH; ++u) {
+                    const int j = base + u * RS_NEAR + 2 * lane;
+                    store_one(row + j, c[2 * u], j < longest);
+                    store_one(row + j + 1, c[2 * u + 1], j + 1 < longest);
+                }
+            }
+        }
+        if (base == 0) { n.near0 = c[0]; n.near1 = c[1]; }
         #pragma unroll
         for (int u = 0; u < BATCH; ++u) {
             const int j = base + u * RS_NEAR + 2 * lane;
-            v[2 * u] = v[2 * u + 1] = 0;
-            if (vec) {
-                if (j < H) {
-                    const longlong2 q = CHECK ? __ldcs(reinterpret_cast<const longlong2*>(row + j)) : *reinterpret_cast<const longlong2*>(row + j);
-                    v[2 * u] = q.x; v[2 * u + 1] = q.y;
-                }
-            } else {
-                if (j < H) v[2 * u] = row[j];
-                if (j + 1 < H) v[2 * u + 1] = row[j + 1];
-            }
-        }
-        #pragma unroll
-        for (int u = 0; u < BATCH; ++u) {
-            const int first = base + u * RS_NEAR, j = first + 2 * lane;
-            if (first >= H) break;
-            if (CHECK) n.bad |= ((v[2 * u] | v[2 * u + 1]) >> 32) != 0;
-            unsigned int c0 = (unsigned int)v[2 * u], c1 = (unsigned int)v[2 * u + 1];
-            if (RAMP && j < Dc) {
-                c0 += (unsigned int)(P + j);
-                if (j + 1 < Dc) c1 += (unsigned int)(P + j + 1);
-                if (STORE) {   // (a pair whose second cell lies past the ramp writes that cell back unchanged)
-                    if (vec) *reinterpret_cast<longlong2*>(row + j) = make_longlong2((long long)c0, (long long)c1);
-                    else {
-                        row[j] = (long long)c0;
-                        if (j + 1 < Dc) row[j + 1] = (long long)c1;
-                    }
-                }
-            }
+            const unsigned int c0 = c[2 * u], c1 = c[2 * u + 1];
             const unsigned int t0 = j < H ? c0 + (unsigned int)j : 0u, t1 = j + 1 < H ? c1 + (unsigned int)(j + 1) : 0u;
-            if (CHECK) n.bad |= (j < H && t0 < c0) || (j + 1 < H && t1 < c1);
-            if (COUNT) n.above += (j < H && (long long)c0 > hot) + (j + 1 < H && (long long)c1 > hot);
+            if (CHECK) bad |= (j < H && t0 < c0 ? 1u : 0u) | (j + 1 < H && t1 < c1 ? 1u : 0u);
+            if (COUNT) n.above += (j < H && (long long)c0 > hot ? 1 : 0) + (j + 1 < H && (long long)c1 > hot ? 1 : 0);
             n.peak = max(n.peak, max(c0, c1));
-            const unsigned int t = max(t0, t1);
-            if (t > top) { top = t; jtop = (unsigned int)(j + 1 < H ? j + 1 : j); }   // a lane's steps ascend
-            if (first == 0) { n.near0 = c0; n.near1 = c1; }
-            else {
-                const unsigned int m = __reduce_max_sync(FULL_MASK, t);
-                if (lane == (first / RS_NEAR - 1) / per) n.far = max(n.far, m);
-            }
+            const unsigned int t = max(t0, t1), step = (unsigned int)(t0 == t ? j : j + 1);
+            jtop = t > top ? step : jtop;     // a lane's steps ascend
+            top = max(top, t);
+            const unsigned int m = __reduce_max_sync(FULL_MASK, t);
+            n.far = max(n.far, lane == stretch ? m : 0u);
+            const bool next = ++in_stretch >= per;
+            stretch += next ? 1 : 0;
+            in_stretch = next ? 0 : in_stretch;
         }
     }
+    n.bad = bad != 0;
     n.top = __reduce_max_sync(FULL_MASK, top);
     n.jtop = __reduce_min_sync(FULL_MASK, top == n.top ? jtop : 0xffffffffu);
     n.peak = __reduce_max_sync(FULL_MASK, n.peak);
@@ -233,7 +278,7 @@ __device__ __forceinline__ unsigned int drop_of(unsigned int top, unsigned int c
 template <typename Args, typename Put>
 __device__ __forceinline__ void summarise_row(const Args& a, int row, uint2* near, unsigned int* far, unsigned long long* guard, Put&& put) {
     const int lane = threadIdx.x & 31, H = a.H;
-    const RowNumbers n = row_pass<false, false, true, true>(a.curves + (size_t)row * H, H, 0, 0, a.hot);
+    const RowNumbers n = row_pass<false, true, true>(a.curves + (size_t)row * H, H, 0, 0, 0, false, a.hot);
     unsigned int step;
     const unsigned int first = first_top(n.near0, n.near1, H, step);
     bool bad = n.bad;
@@ -299,6 +344,8 @@ struct RouteSumArgs {
     const uint4* summary0;
     uint2* near;                   // [I][32], [I][32]: see SumArgs
     unsigned int* far;
+    unsigned int* link;            // [max_requests] per request of the batch the one that the same row got before,
+    unsigned int* newest;          // [I] and the newest one of each row, as far as written out (RS_NOBODY: none)
     unsigned char* applied;        // [max_requests] 1: the map has this request of the batch already (zero between calls)
     unsigned long long* guard;
     int* status;
@@ -376,7 +423,7 @@ struct RsShared {
     unsigned int flush;                     // ... and as many are asked for
     int cursor;                             // items of the batch that the io warp has looked at (when it has ended)
     unsigned int spin_limit, idle_limit;
-    unsigned int beat;                      // moves while a warp is busy with something long that others wait for
+    unsigned int beat;                      // moves while the io warp goes through arrivals
     unsigned int not_over;                  // ADMIT: rows that are not overloaded, as far as folded
     int blocked;                            // ADMIT: a request found every instance overloaded ...
     long long blocked_k;                    // ... this one
@@ -559,27 +606,48 @@ struct Folder {
         if (lo < H && (long long)n.far - lo > a.hot) above += min(steps, H - lo);
         return __reduce_add_sync(FULL_MASK, above);
     }
-    // Brings the map's row up to date with the requests of the batch below `upto` whose ramps it lacks.
-    __device__ __forceinline__ bool catch_up(int w, unsigned int upto) {
-        const int lane = threadIdx.x & 31, H = a.H;
-        if (lane == 0) atomicMax(&sh.flush, upto);
-        if (!rs_wait(sh, [&] { return (int)(ld_acquire(&sh.written) - upto) >= 0; })) return false;
+    // The requests of the batch whose ramps the map's row lacks, from the newest on: {P, min(D, H)} of up to ROOM of them, one per
+    // lane, marked as applied; `k` is the next one then.  The io warp keeps the requests of a row as a chain; behind the first one
+    // that is applied all are.  (Looked for among all requests of the batch they took longer the longer the batch was: 64 instances, 1,024
+    // arrivals, 5,000 cycles a time.)
+    template <int ROOM>
+    __device__ __forceinline__ int lacking(unsigned int& k, int& P, int& Dc) {
+        const int lane = threadIdx.x & 31;
         const long long n0 = sh.n0;
-        int64_t* row = a.curves + (size_t)w * H;
-        for (unsigned int base = 0; base < upto; base += 32) {
-            if ((base & 1023u) == 0 && lane == 0) atomicAdd(&sh.beat, 1u);
-            const unsigned int k = base + lane;
-            const bool mine = k < upto && a.instance[n0 + k] == w && a.applied[k] == 0;
-            if (mine) a.applied[k] = 1;
-            int P = 0, D = 0;
-            if (mine) { P = a.prompt[n0 + k]; D = a.predicted[n0 + k]; }
-            for (unsigned int todo = __ballot_sync(FULL_MASK, mine); todo; todo &= todo - 1) {
-                const int src = __ffs(todo) - 1;
-                const int p = __shfl_sync(FULL_MASK, P, src), d = __shfl_sync(FULL_MASK, D, src);
-                for (int j = lane; j < (d < H ? d : H); j += 32) row[j] += p + j;
-            }
+        int count = 0;
+        while (k != RS_NOBODY && count < ROOM) {
+            const int p = a.prompt[n0 + k], d = a.predicted[n0 + k], applied = a.applied[k];
+            const unsigned int next = a.link[k];
+            if (applied) { k = RS_NOBODY; break; }
+            __syncwarp();      // (all lanes have looked at the mark)
+            if (lane == count) { P = p; Dc = d < a.H ? d : a.H; a.applied[k] = 1; }
+            ++count;
+            k = next;
         }
-        __syncwarp();
+        return count;
+    }
+    // Brings the map's row up to date with the requests of the batch below `upto`, and with the arrival (P, Dc) as one more if `own`;
+    // false: abandoned.
+    __device__ __forceinline__ bool catch_up(int w, unsigned int upto, int P, int Dc, bool own, RowNumbers& n) {
+        const int lane = threadIdx.x & 31;
+        unsigned int k = RS_NOBODY;
+        if (rows.state[w] & RS_DEFERRED) {
+            if (lane == 0) atomicMax(&sh.flush, upto);
+            if (!rs_wait(sh, [&] { return (int)(ld_acquire(&sh.written) - upto) >= 0; })) return false;
+            k = __ldcg(a.newest + w);
+        }
+        int p = 0, d = 0;
+        for (bool more = true; more;) {
+            int count = lacking<31>(k, p, d);
+            more = k != RS_NOBODY;
+            if (!more && own) {
+                if (lane == count) { p = P; d = Dc; }
+                ++count;
+            }
+            n = row_pass<true, ADMIT, false>(a.curves + (size_t)w * a.H, a.H, p, d, count, true, a.hot);
+            __syncwarp();
+        }
+        store_numbers(w, n);
         return true;
     }
     // Decision e: its row's new numbers.
@@ -611,10 +679,8 @@ struct Folder {
             if (!full) deferred = true;
         }
         if (full) {
-            if (deferred && !catch_up(w, e)) return false;
+            if (!catch_up(w, e, P, Dc, true, n)) return false;
             deferred = false;
-            n = row_pass<true, true, ADMIT, false>(a.curves + (size_t)w * H, H, P, Dc, a.hot);
-            store_numbers(w, n);
             if (lane == 0) a.applied[e] = 1;
             not_over = not_over && !((double)n.above > a.many);
             full = n.jtop >= (unsigned int)RS_NEAR || (not_over && (double)most_above(n) > a.many);
@@ -646,13 +712,12 @@ struct Folder {
         const bool others = Dc > RS_NEAR || u > peak + (unsigned int)(u ? lo : 0);
         if (!__any_sync(FULL_MASK, others)) return true;
         if (rows.state[w] & RS_DEFERRED) {
-            if (!catch_up(w, decided)) return false;
-            const RowNumbers n = row_pass<false, false, false, false>(a.curves + (size_t)w * H, H, 0, 0, 0);
-            store_numbers(w, n);
+            RowNumbers n;
+            if (!catch_up(w, decided, 0, 0, false, n)) return false;
             __syncwarp();
             if (lane == 0) rows.state[w] &= ~RS_DEFERRED;     // (its numbers stay what they are: they were exact)
         }
-        peak = row_pass<true, false, false, false>(a.curves + (size_t)w * H, H, P, Dc, 0).peak;
+        peak = row_pass<true, ADMIT, false>(a.curves + (size_t)w * H, H, P, Dc, 1, false, a.hot).peak;
         return true;
     }
 };
@@ -926,12 +991,17 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
         const unsigned int folded = min(decided, written + __reduce_min_sync(FULL_MASK, next - written));
         const unsigned int flush = __shfl_sync(FULL_MASK, ld_volatile(&sh.flush), 0);
         while (folded - written >= 32 || (folded != written && (last || (int)(flush - written) > 0))) {
-            const unsigned int e = written + lane;
+            const unsigned int e = written + lane, some = __ballot_sync(FULL_MASK, e < folded);
             if (e < folded) {
                 const int w = (int)(sh.jobs[e % RS_ITEMS].x & ~RS_GIVEN);
                 const int2 pd = sh.raw[e % RS_ITEMS];
                 const long long at = n0 + e;
                 a.prompt[at] = pd.x; a.generated[at] = 0; a.predicted[at] = pd.y; a.instance[at] = w;
+                // (a row's requests in their order: those of this group by their lanes)
+                const unsigned int same = __match_any_sync(some, w), below = same & ((1u << lane) - 1u);
+                a.link[e] = below ? e - lane + (31 - __clz(below)) : __ldcg(a.newest + w);
+                __syncwarp(some);
+                if ((same >> lane) == 1u) __stcg(a.newest + w, e);
                 put_result(sh.item_at[e % RS_ITEMS], w, sh.score[e % RS_ITEMS]);
                 atomicAdd(reinterpret_cast<unsigned long long*>(a.queued_p + w), (unsigned long long)pd.x);
                 atomicAdd(reinterpret_cast<unsigned long long*>(a.current_d + w), (unsigned long long)pd.y);
@@ -1808,6 +1878,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
             rows.top[i] = q.y;
             rows.pending[i] = 0;
             if (!WHOLE) rows.tok[i] = q.x;
+            a.newest[i] = RS_NOBODY;
             if (LISTS)
                 #pragma unroll
                 for (int p = 0; p < RS_PROBES; ++p) least[LISTS ? p : 0] = min(least[LISTS ? p : 0], max(rec.x, rec.y + sc.key_p(rs_probe(mean, p))));
@@ -2015,7 +2086,7 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
     a.choice = choice; a.score = score;
     a.I = I; a.H = H;
     a.theta = ctx->theta; a.beta = ctx->cfg.beta;
-    a.summary0 = p.summary; a.guard = p.guard; a.near = p.near; a.far = p.far; a.applied = ctx->d_rs_applied;
+    a.summary0 = p.summary; a.guard = p.guard; a.near = p.near; a.far = p.far; a.applied = ctx->d_rs_applied; a.link = ctx->d_rs_link; a.newest = ctx->d_rs_newest;
     a.status = ctx->d_status; a.handled = ctx->d_rs_handled; a.give_up = ctx->d_abort; a.ramps = ctx->d_rs_ramps;
     a.spin_limit = ctx->spin_limit > 0xffffffffu / RS_POLLS ? 0xffffffffu : RS_POLLS * ctx->spin_limit;
     a.alone = pre_route_summary_alone(ctx) ? 1 : 0;

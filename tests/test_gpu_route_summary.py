@@ -362,3 +362,19 @@ def test_rows_whose_largest_cell_moves_beyond_the_first_steps(n_inst, h, beta, q
         ref.step()
     assert st.status() == B.PRE_OK
     st.close()
+
+
+@pytest.mark.parametrize("n_inst,h,beta", [(2, 500, 1.0), (3, 901, 0.75), (280, 400, 1.0)])
+def test_rows_brought_up_to_date_late_in_a_long_batch(n_inst, h, beta):
+    """Runs of requests that leave a row's largest cell among the first steps, more of them than a warp has lanes, between requests
+    that move it far out: the row then gets all ramps that its map lacks at once, several times in one batch."""
+    n = 6 * n_inst
+    wl = W.make_random(540 + n_inst, n_inst, h, n, 0, max_prompt=50, max_output=30, beta=beta, capacity=20000)
+    rng = np.random.default_rng(22)
+    ap, ad = [], []
+    for run in (45 * n_inst, 20 * n_inst, 70 * n_inst) if n_inst < 10 else (5 * n_inst, 4 * n_inst):
+        ap += [rng.integers(300, 900, run), rng.integers(0, 3, 12 * n_inst if n_inst < 10 else 3 * n_inst)]
+        ad += [rng.integers(40, 64, run), rng.integers(h - 40, 2 * h, len(ap[-1]))]
+    ap, ad = np.concatenate(ap).astype(np.int32), np.concatenate(ad).astype(np.int32)
+    wl.max_requests = n + len(ap)
+    route_and_compare(wl, ap, ad)
