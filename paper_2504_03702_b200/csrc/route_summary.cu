@@ -61,7 +61,8 @@ constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding war
 constexpr int RS_PROBES = 8;                // prompt lengths for which a list has the best rows
 constexpr int RS_NEAR = 64;                 // steps kept exactly; the rest in 32 stretches of whole chunks of as many steps
 // A row whose top lies further out than this is "far": the deciding warp has only a lower bound of its score, and the
-// arrivals that take its quick way are those that reach the largest jtop of the other rows.
+// arrivals that take its quick way are those that reach the largest jtop of the other rows.  A row that cannot pay a penalty for any arrival
+// of the batch is never far: its score is its token count, wherever its top lies, and an upper bound of the top shows it.
 constexpr int RS_LIMIT = 32;
 constexpr int RS_MAX_ROWS = 10240;          // instances up to which the context offers this router (shared memory),
 constexpr int RS_MAX_BINARY64_ROWS = 5120;  // and with binary64 scores
@@ -77,7 +78,7 @@ constexpr unsigned int FULL_MASK = 0xffffffffu;
 
 // guard words written by the summarising kernel; the routing kernel clears them for the next call
 constexpr int GUARD_MAX_CELL = 0, GUARD_MAX_BASE = 1, GUARD_BAD = 2, GUARD_SUM_RAMP = 3, GUARD_SUM_TOKENS = 4,
-              GUARD_MAX_PD = 5, GUARD_SUM_BASE = 6, GUARDS = 7;
+              GUARD_MAX_PD = 5, GUARD_SUM_BASE = 6, GUARD_MAX_P = 7, GUARDS = 8;
 
 // What a warp finds out about a row in one pass: lane l has cells 2l and 2l+1 of the first 64 and the largest c[j] + j of
 // stretch l (0: no such stretch).
@@ -238,12 +239,13 @@ __device__ __forceinline__ unsigned int first_top(unsigned int near0, unsigned i
 template <typename Args>
 __device__ __forceinline__ void batch_totals(const Args& a, long long first, long long stride, unsigned long long* guard) {
     unsigned long long ramp = 0, tokens = 0;
-    unsigned int max_pd = 0;
+    unsigned int max_pd = 0, max_p = 0;
     auto count = [&](int P, int D) {
         if (P < 0 || D < 1 || P > PRE_FIELD_MAX || D > PRE_FIELD_MAX) return;
         ramp += (unsigned long long)P + (unsigned long long)(D < a.H ? D : a.H);
         tokens += (unsigned long long)P + (unsigned long long)D;
         max_pd = max(max_pd, (unsigned int)P + (unsigned int)D);
+        max_p = max(max_p, (unsigned int)P);
     };
     for (long long k = first; k < a.n_arrivals; k += stride)
         count(a.arr_prompt[k], a.arr_predicted[k]);
@@ -263,10 +265,12 @@ __device__ __forceinline__ void batch_totals(const Args& a, long long first, lon
         tokens += __shfl_xor_sync(FULL_MASK, tokens, off);
     }
     max_pd = __reduce_max_sync(FULL_MASK, max_pd);
+    max_p = __reduce_max_sync(FULL_MASK, max_p);
     if ((threadIdx.x & 31) == 0 && (ramp | tokens)) {
         atomicAdd(guard + GUARD_SUM_RAMP, ramp);
         atomicAdd(guard + GUARD_SUM_TOKENS, tokens);
         atomicMax(guard + GUARD_MAX_PD, (unsigned long long)max_pd);
+        atomicMax(guard + GUARD_MAX_P, (unsigned long long)max_p);
     }
 }
 
@@ -375,7 +379,7 @@ constexpr int RS_SCANS = 0, RS_KEYS = 1, RS_CLOSELY = 2;
 //          of the keys unless the row is far or pending
 //   state  jtop | drop << RS_DROP (the first cell is that much below the top that b stands for; RS_DROP_MAX: or more) | RS_FAR | RS_FULL | RS_DEFERRED (the map lacks ramps) | RS_NOT_OVER (ADMIT: the row is not overloaded, as
 //          far as folded)
-//   top, tok   top and token count (whole-number scores: half of a)
+//   top, tok   top (or, jtop RS_JTOP, an upper bound for which no arrival of the batch pays) and token count (whole-number scores: half of a)
 //   pending  1 from the decision for the row to the end of its fold; cleared last
 constexpr unsigned int RS_FAR = 0x40000000u, RS_NOT_OVER = 0x20000000u, RS_FULL = 0x10000000u, RS_DEFERRED = 0x08000000u, RS_JTOP = 0xffffu,
                        RS_DROP_MAX = 2047u;
@@ -507,7 +511,8 @@ template <bool WHOLE> struct Scores {
     double theta, beta, unit;
     int theta_i, beta_i, shift, code_base;
     int slope;           // what a token less at the peak takes from b at most (0: too much)
-    __device__ __forceinline__ void start(double theta_d, double beta_d, unsigned long long peak_bound, unsigned long long max_pd,
+    unsigned int free_below;     // a row whose top is below pays no penalty, whatever arrival of the batch it gets
+    __device__ __forceinline__ void start(double theta_d, double beta_d, unsigned long long peak_bound, unsigned long long max_pd, unsigned long long max_p,
                                           unsigned long long typical_tokens, int mean) {
         theta = theta_d; beta = beta_d;
         beta_i = theta_i = shift = 0;
@@ -516,6 +521,7 @@ template <bool WHOLE> struct Scores {
             beta_i = (int)beta_d;
             // a threshold above every peak of the batch is as good as any other: the penalty is never paid
             theta_i = theta_d > (double)peak_bound ? (int)(peak_bound + 1) : (int)theta_d;
+            free_below = max_p <= (unsigned long long)theta_i ? (unsigned int)((unsigned long long)theta_i - max_p) + 1 : 0u;
         } else {
             // seven binary digits, fewer for long requests or many tokens
             shift = 7;
@@ -523,9 +529,12 @@ template <bool WHOLE> struct Scores {
                                  (typical_tokens << shift) > (unsigned long long)(RS_CUT / 8)))
                 --shift;
             unit = (double)(1 << shift);
+            const double most = floor(fmin(theta, 8.0e9)) - (double)max_p;
+            free_below = most < 0.0 ? 0u : most >= 4294967294.0 ? 0xffffffffu : (unsigned int)most + 1u;
         }
         const double s = WHOLE ? 2.0 * beta : 2.0 * ceil(beta * unit);
         slope = WHOLE || s <= 524288.0 ? (int)s : 0;
+        if (beta == 0.0) free_below = 0xffffffffu;
         code_base = __float_as_int(fmaxf((float)mean * (1.0f / 32.0f) * (float)beta * (float)(2.0 * unit), 1.0f)) >> 21;
     }
     __device__ __forceinline__ int key_a(unsigned int tokens) const {
@@ -563,7 +572,7 @@ template <bool WHOLE> struct Scores {
         if constexpr (WHOLE) return tokens + (unsigned int)(beta_i * max((int)peak - theta_i, 0));
         else return summary_score(tokens, peak, (double)P + (double)D, theta, beta);
     }
-    __device__ __forceinline__ bool no_penalty(unsigned int top, int P) const { return !((double)(top + (unsigned int)P) > theta); }
+    __device__ __forceinline__ bool no_penalty(unsigned int top, int P) const { return beta == 0.0 || !((double)(top + (unsigned int)P) > theta); }
     static __device__ __forceinline__ S warp_min(S s) {   // scores are >= 0: ordered by their bits
         if constexpr (WHOLE) return __reduce_min_sync(FULL_MASK, s);
         else {
@@ -675,7 +684,10 @@ struct Folder {
             const unsigned int t = max(j < H ? n.near0 + (unsigned int)j : 0u, j + 1 < H ? n.near1 + (unsigned int)(j + 1) : 0u);
             n.top = __reduce_max_sync(FULL_MASK, t);
             n.jtop = __reduce_min_sync(FULL_MASK, t == n.top ? (unsigned int)(j + 1 < H ? j + 1 : j) : 0xffffffffu);
-            full = __any_sync(FULL_MASK, n.far > n.top) || (not_over && (double)most_above(n) > a.many);
+            const bool beyond = __any_sync(FULL_MASK, n.far > n.top);
+            const unsigned int bound = beyond ? max(n.top, __reduce_max_sync(FULL_MASK, n.far)) : 0u;
+            full = (beyond && bound >= sc.free_below) || (not_over && (double)most_above(n) > a.many);
+            if (beyond && !full) { n.top = bound; n.jtop = RS_JTOP; }     // (enough for a row that pays no penalty)
             if (!full) deferred = true;
         }
         if (full) {
@@ -683,14 +695,14 @@ struct Folder {
             deferred = false;
             if (lane == 0) a.applied[e] = 1;
             not_over = not_over && !((double)n.above > a.many);
-            full = n.jtop >= (unsigned int)RS_NEAR || (not_over && (double)most_above(n) > a.many);
+            full = (n.jtop >= (unsigned int)RS_NEAR && n.top >= sc.free_below) || (not_over && (double)most_above(n) > a.many);
         }
-        const bool far = n.jtop >= (unsigned int)RS_LIMIT;
+        const bool pays = n.top >= sc.free_below, far = pays && n.jtop >= (unsigned int)RS_LIMIT;
         unsigned int key_top = n.top, key_step = n.jtop;
         if (far) key_top = first_top(n.near0, n.near1, H, key_step);
         __syncwarp();   // every lane's cells before the row is handed on
         if (lane == 0) {
-            if (key_step > ld_volatile(&sh.jmax)) atomicMax(&sh.jmax, key_step);
+            if (pays && key_step > ld_volatile(&sh.jmax)) atomicMax(&sh.jmax, key_step);
             const unsigned int now = tokens + (unsigned int)P + (unsigned int)D;
             rows.top[w] = n.top;
             if (!WHOLE) rows.tok[w] = now;
@@ -1793,7 +1805,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     }
     const unsigned long long* guard = alone ? sh_guard : a.guard;
     const unsigned long long mc = guard[GUARD_MAX_CELL], mb = guard[GUARD_MAX_BASE], ramps = guard[GUARD_SUM_RAMP],
-                             tokens_in = guard[GUARD_SUM_TOKENS], max_pd = guard[GUARD_MAX_PD], base_sum = guard[GUARD_SUM_BASE];
+                             tokens_in = guard[GUARD_SUM_TOKENS], max_pd = guard[GUARD_MAX_PD], max_p = guard[GUARD_MAX_P], base_sum = guard[GUARD_SUM_BASE];
     // every cell, every cell + step with a prompt added, and every token count stay below 2^32 all batch long
     // (the ramps of the batch bound what an arrival that is not routed yet can add, too)
     const unsigned long long peak_bound = mc + ramps + (unsigned long long)H;
@@ -1849,7 +1861,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     const unsigned long long mean_l = ramps / (unsigned long long)(n_items > 0 ? n_items : 1);
     const int mean = mean_l < (1ull << 22) ? (int)mean_l : 1 << 22;     // prompt + ramp of a typical request
     Scores<WHOLE> sc;
-    sc.start(a.theta, a.beta, peak_bound, max_pd, (base_sum + tokens_in) / (unsigned long long)I, mean);
+    sc.start(a.theta, a.beta, peak_bound, max_pd, max_p, (base_sum + tokens_in) / (unsigned long long)I, mean);
     {
         unsigned int jmax = 0;
         int free_rows = 0;
@@ -1868,13 +1880,13 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
                 if (ADMIT) above = a.over0[i];
             }
             const unsigned int jtop = q.z & 0xffffu, step = (q.z >> 16) & 31u, drop = q.z >> 21;
-            const bool far = jtop >= (unsigned int)RS_LIMIT;
-            jmax = max(jmax, far ? step : jtop);
+            const bool pays = q.y >= sc.free_below, far = pays && jtop >= (unsigned int)RS_LIMIT;
+            jmax = max(jmax, !pays ? 0u : far ? step : jtop);
             const bool not_over = ADMIT && !((double)above > a.many);
             free_rows += not_over;
             const int2 rec = make_int2(sc.key_a(q.x), sc.key_b(q.x, far ? q.w : q.y));
             rows.rec[i] = rec;
-            rows.state[i] = jtop | (drop << RS_DROP) | (far ? RS_FAR : 0u) | (jtop >= (unsigned int)RS_NEAR ? RS_FULL : 0u) | (not_over ? RS_NOT_OVER : 0u);
+            rows.state[i] = jtop | (drop << RS_DROP) | (far ? RS_FAR : 0u) | (pays && jtop >= (unsigned int)RS_NEAR ? RS_FULL : 0u) | (not_over ? RS_NOT_OVER : 0u);
             rows.top[i] = q.y;
             rows.pending[i] = 0;
             if (!WHOLE) rows.tok[i] = q.x;
