@@ -311,10 +311,10 @@ int pre_status(pre_ctx* ctx, void* stream);
 int pre_last_cuda_error(const pre_ctx* ctx);
 
 /* Which kernel routes the batches of pre_route_batch and pre_route_admit on this context: PRE_ROUTE_AUTO (default:
- * the summary kernel when the shape fits it, the
- * scanning kernel otherwise or when the summary kernel declines a batch), PRE_ROUTE_SCAN (always the scanning kernel), PRE_ROUTE_SUMMARY (as
- * AUTO, but PRE_ESIZE here when the shape does not fit the summary kernel).  Results do not
- * depend on it. */
+ * the summary kernel when the shape fits it, the scanning kernel otherwise or when the summary kernel declines a batch, because
+ * a value could leave its numbers or because the rows are such that the scanning kernel is faster), PRE_ROUTE_SCAN
+ * (always the scanning kernel), PRE_ROUTE_SUMMARY (the summary kernel whenever its numbers hold the batch; PRE_ESIZE here when the
+ * shape does not fit it).  Results do not depend on it. */
 #define PRE_ROUTE_AUTO    0
 #define PRE_ROUTE_SCAN    1
 #define PRE_ROUTE_SUMMARY 2

@@ -58,6 +58,11 @@ constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lan
 constexpr int RS_LONG_LISTS = 2048;
 constexpr int RS_NEAR_ROWS = 2304;          // rows the list warps keep for a closer look at once
 constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding warp looks at their keys by itself
+// Beyond RS_DIRECT_ROWS instances two kinds of batches cost this kernel more than the scanning one (which takes 2.4 us an arrival on 1,024 x
+// 1,024 whatever the rows): many far rows that may pay a penalty, whose arrivals need a look at all rows, scans, and folds of
+// whole rows (share of such rows, us: 28 % 2.0, 51 % 4.4, 58 % 5.4; with 512 x 40, 55 %, 1.3 against 2.3); and more rows that
+// share the smallest score than a list holds (empty services; 512 rows 2.7, 4,096 rows 42 against 3.1).
+constexpr int RS_FAR_SHARE = 3, RS_FAR_STEPS = 256;     // one row in so many, maps of more steps than that
 constexpr int RS_PROBES = 8;                // prompt lengths for which a list has the best rows
 constexpr int RS_NEAR = 64;                 // steps kept exactly; the rest in 32 stretches of whole chunks of as many steps
 // A row whose top lies further out than this is "far": the deciding warp has only a lower bound of its score, and the
@@ -356,6 +361,7 @@ struct RouteSumArgs {
     int* give_up;                  // three words that the scanning kernel finds cleared
     int* handled;                  // 1: this kernel routed the batch; 0: the scanning kernel has to
     unsigned int spin_limit;       // polls before a wait is declared lost
+    int may_decline;               // a batch that the scanning kernel routes faster is left to it
     int alone;                     // small shapes: nothing is launched before or after this kernel, but for the ramps where
     int own_ramps;                 // this kernel does not add them itself
     long long* ramps;              // {first table row, rows} whose ramps the maps still lack
@@ -421,6 +427,7 @@ struct RsShared {
     int look_row[2][RS_MAX_FOLD_WARPS];                    // the row that has it
     unsigned int look_peak[2][RS_MAX_FOLD_WARPS];          // and its peak
     unsigned int jmax;                      // largest step that a row's b stands for
+    unsigned int n_far, n_least;            // when the batch begins: far rows, rows with the smallest score for an empty prompt
     unsigned int items_ready;               // items written so far
     unsigned int items_end;                 // 1: there will be no more
     unsigned int written;                   // results written so far
@@ -1822,7 +1829,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         sh.cursor = 0; sh.beat = 0;
         sh.n0 = *a.n_requests;
         sh.ctl = make_uint4(0u, 0u, 0u, 0u);
-        sh.items_ready = sh.items_end = sh.not_over = sh.jmax = sh.written = sh.flush = 0;
+        sh.items_ready = sh.items_end = sh.not_over = sh.jmax = sh.n_far = sh.n_least = sh.written = sh.flush = 0;
         sh.lists_wanted = sh.lists_ready = sh.list_met = sh.look_met = 0;
         sh.list_n[0] = sh.list_n[1] = 0;
         sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0;
@@ -1840,14 +1847,14 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     __syncthreads();
     if (tid < GUARDS && !alone) a.guard[tid] = 0;    // ready for the next call
     const int mode = __shfl_sync(FULL_MASK, sh.mode, 0);     // (all threads alike, and known to be)
-    if (mode == 0 && !alone) {
+    auto decline = [&]() {
         if (tid == 0) {
             *a.handled = 0;
             if (ADMIT) { a.queue_entry[0] = a.queue_state[0]; a.queue_entry[1] = a.queue_state[1]; }
         }
         if (tid < 3) a.give_up[tid] = 0;
-        return;
-    }
+    };
+    if (mode == 0 && !alone) { decline(); return; }
     if (ADMIT && a.queue_capacity > 0) {   // kept inside the ring whatever the two words hold
         if (q_head < 0 || q_head >= a.queue_capacity) q_head = 0;
         if (q_len < 0) q_len = 0;
@@ -1863,7 +1870,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     Scores<WHOLE> sc;
     sc.start(a.theta, a.beta, peak_bound, max_pd, max_p, (base_sum + tokens_in) / (unsigned long long)I, mean);
     {
-        unsigned int jmax = 0;
+        unsigned int jmax = 0, n_far = 0;
         int free_rows = 0;
         int least[LISTS ? RS_PROBES : 1];      // the smallest value per probe, for the first list
         if (LISTS)
@@ -1882,6 +1889,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
             const unsigned int jtop = q.z & 0xffffu, step = (q.z >> 16) & 31u, drop = q.z >> 21;
             const bool pays = q.y >= sc.free_below, far = pays && jtop >= (unsigned int)RS_LIMIT;
             jmax = max(jmax, !pays ? 0u : far ? step : jtop);
+            n_far += far;
             const bool not_over = ADMIT && !((double)above > a.many);
             free_rows += not_over;
             const int2 rec = make_int2(sc.key_a(q.x), sc.key_b(q.x, far ? q.w : q.y));
@@ -1897,6 +1905,10 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         }
         jmax = __reduce_max_sync(FULL_MASK, jmax);
         if (lane == 0 && jmax) atomicMax(&sh.jmax, jmax);
+        if (LISTS) {
+            n_far = __reduce_add_sync(FULL_MASK, n_far);
+            if (lane == 0 && n_far) atomicAdd(&sh.n_far, n_far);
+        }
         if (LISTS)
             #pragma unroll
             for (int p = 0; p < RS_PROBES; ++p) {
@@ -1910,6 +1922,14 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     }
     const long long room = a.max_requests - sh.n0;
     __syncthreads();
+    if (LISTS && a.may_decline) {
+        unsigned int n_least = 0;
+        for (int i = tid; i < I; i += THREADS) n_least += max(rows.rec[i].x, rows.rec[i].y) <= unordered(sh.probe_t[0]) + Scores<WHOLE>::SLACK;
+        n_least = __reduce_add_sync(FULL_MASK, n_least);
+        if (lane == 0 && n_least) atomicAdd(&sh.n_least, n_least);
+        __syncthreads();
+        if ((H > RS_FAR_STEPS && sh.n_far > (unsigned int)(I / RS_FAR_SHARE)) || sh.n_least > 32u * KS) { decline(); return; }
+    }
 
     const int role = (warp >> 2) * 3 + (warp & 3) - 1;      // (of the warps that are not on the deciding warp's scheduler)
     if (warp == 0) {
@@ -2101,6 +2121,7 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
     a.summary0 = p.summary; a.guard = p.guard; a.near = p.near; a.far = p.far; a.applied = ctx->d_rs_applied; a.link = ctx->d_rs_link; a.newest = ctx->d_rs_newest;
     a.status = ctx->d_status; a.handled = ctx->d_rs_handled; a.give_up = ctx->d_abort; a.ramps = ctx->d_rs_ramps;
     a.spin_limit = ctx->spin_limit > 0xffffffffu / RS_POLLS ? 0xffffffffu : RS_POLLS * ctx->spin_limit;
+    a.may_decline = ctx->route_path == PRE_ROUTE_AUTO ? 1 : 0;
     a.alone = pre_route_summary_alone(ctx) ? 1 : 0;
     a.own_ramps = a.alone && n_arrivals * (long long)H <= RS_OWN_RAMP_CELLS ? 1 : 0;
     a.queue_prompt = nullptr; a.queue_predicted = nullptr; a.queue_state = nullptr; a.queue_entry = nullptr;

@@ -378,3 +378,47 @@ def test_rows_brought_up_to_date_late_in_a_long_batch(n_inst, h, beta):
     ap, ad = np.concatenate(ap).astype(np.int32), np.concatenate(ad).astype(np.int32)
     wl.max_requests = n + len(ap)
     route_and_compare(wl, ap, ad)
+
+
+def case_of(kind):
+    """Services on which summaries say little: empty ones, few requests per instance, all of them young, one-token arrivals."""
+    n_inst, h, per, beta = {"empty": (512, 512, 0, 1.0), "empty, binary64": (2000, 300, 0, 0.75), "few": (600, 700, 4, 1.0),
+                            "few, binary64": (600, 700, 4, 0.75), "young": (600, 700, 16, 1.0), "one token": (1024, 512, 64, 1.0)}[kind]
+    wl = W.make_random(560 + n_inst % 89, n_inst, h, per * n_inst, 0, max_prompt=2000, max_output=h + h // 2, beta=beta,
+                       capacity=None if per else 500001)
+    if kind == "young":
+        wl.generated[:] = 0
+    rng = np.random.default_rng(23)
+    ap = rng.integers(1, 2000, 1500).astype(np.int32)
+    ad = rng.integers(1, h + h // 2, 1500).astype(np.int32)
+    if kind == "one token":
+        ad[:] = 1
+    wl.max_requests = per * n_inst + 1500
+    return wl, ap, ad
+
+
+@pytest.mark.parametrize("kind", ["empty", "empty, binary64", "few", "few, binary64", "young", "one token"])
+def test_the_default_is_not_slower_than_the_scanning_kernel(kind):
+    """The library's choice against the kernel that reads every cell for every arrival, whose time does not depend on the rows: the best
+    of five calls each, with half as much again as room (the two differ by less than 2 % from call to call)."""
+    wl, ap, ad = case_of(kind)
+    st = DeviceState.from_workload(wl)
+    p, d = dev(ap), dev(ad)
+    best, choices = {}, {}
+    for path in (B.ROUTE_AUTO, B.ROUTE_SCAN):
+        st.select_router(path)
+        times = []
+        for _ in range(5):
+            st.n_requests.fill_(len(wl.prompt))
+            st.queued_p.zero_()
+            st.anticipate(len(wl.prompt))
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            choice, _ = st.route_batch(p, d)
+            t1.record()
+            torch.cuda.synchronize()
+            times.append(t0.elapsed_time(t1))
+        best[path], choices[path] = min(times), choice.cpu().numpy()
+    assert (choices[B.ROUTE_AUTO] == choices[B.ROUTE_SCAN]).all()
+    assert best[B.ROUTE_AUTO] <= 1.5 * best[B.ROUTE_SCAN], best
+    st.close()
