@@ -4,7 +4,7 @@
 // of the map with the arrival's ramp added (Sec. 4.3.1 update), Dc = min(D, H):
 //     peak = max( max_{j<Dc}(c[j] + P + j),  max_{j>=Dc} c[j] ).
 // Two numbers per row decide it without reading the row in almost every case:
-//     top = max_j (c[j] + j)      jtop = no step below which the maximum is first taken
+//     top = max_j (c[j] + j)      jtop = the step at which the maximum is first taken
 //   * Dc > jtop:  the ramp covers the step of the maximum, so max_{j<Dc}(c[j]+j) = top; and
 //                 P + top >= c[j] for every j, so   peak = P + top   exactly;
 //   * always:     top - jtop <= peak <= P + top;
@@ -68,7 +68,8 @@ constexpr int RS_NEAR = 64;                 // steps kept exactly; the rest in 3
 // A row whose top lies further out than this is "far": the deciding warp has only a lower bound of its score, and the
 // arrivals that take its quick way are those that reach the largest jtop of the other rows.  A row that cannot pay a penalty for any arrival
 // of the batch is never far: its score is its token count, wherever its top lies, and an upper bound of the top shows it.
-constexpr int RS_LIMIT = 32;
+constexpr int RS_LIMIT = 32;                // (maps of at most RS_NEAR steps have no far rows: most arrivals reach their last step)
+__device__ __forceinline__ unsigned int far_from(int H) { return H <= RS_NEAR ? RS_NEAR : RS_LIMIT; }
 constexpr int RS_MAX_ROWS = 10240;          // instances up to which the context offers this router (shared memory),
 constexpr int RS_MAX_BINARY64_ROWS = 5120;  // and with binary64 scores
 constexpr int SUM_THREADS = 256;
@@ -231,12 +232,12 @@ struct SumArgs {
     long long queue_capacity;
 };
 
-// The largest c[j] + j of the steps below RS_LIMIT, from the first cells, and no step below which it is first taken.
+// The largest c[j] + j of the steps below RS_LIMIT, from the first cells, and the step at which it is first taken.
 __device__ __forceinline__ unsigned int first_top(unsigned int near0, unsigned int near1, int H, unsigned int& step) {
     const int j = 2 * (threadIdx.x & 31), end = H < RS_LIMIT ? H : RS_LIMIT;
-    const unsigned int t = max(j < end ? near0 + (unsigned int)j : 0u, j + 1 < end ? near1 + (unsigned int)(j + 1) : 0u);
+    const unsigned int t0 = j < end ? near0 + (unsigned int)j : 0u, t = max(t0, j + 1 < end ? near1 + (unsigned int)(j + 1) : 0u);
     const unsigned int top = __reduce_max_sync(FULL_MASK, t);
-    step = __reduce_min_sync(FULL_MASK, t == top && j < end ? (unsigned int)(j + 1 < end ? j + 1 : j) : 0xffffffffu);
+    step = __reduce_min_sync(FULL_MASK, t == top && j < end ? (unsigned int)(t0 == t ? j : j + 1) : 0xffffffffu);
     return top;
 }
 
@@ -298,7 +299,7 @@ __device__ __forceinline__ void summarise_row(const Args& a, int row, uint2* nea
         const long long tok = q + d;
         const bool ok = q >= 0 && d >= 0 && q <= 0xffffffffLL && d <= 0xffffffffLL && tok <= 0xffffffffLL;
         if (!ok) bad = true;
-        const unsigned int drop = drop_of(n.jtop >= (unsigned int)RS_LIMIT ? first : n.top, n.near0);
+        const unsigned int drop = drop_of(n.jtop >= far_from(H) ? first : n.top, n.near0);
         put(make_uint4(ok ? (unsigned int)tok : 0u, n.top, n.jtop | (step << 16) | (drop << 21), first), n.above);
         if (ok) {
             atomicMax(guard + GUARD_MAX_BASE, (unsigned long long)tok);
@@ -593,7 +594,7 @@ template <bool WHOLE> struct Scores {
 template <bool WHOLE>
 __device__ __forceinline__ int Scores<WHOLE>::key_least(unsigned int state, int kp, int Dc, int& exact) const {
     const int drop = (int)((state >> RS_DROP) & RS_DROP_MAX), jt = (int)(state & RS_JTOP), near = (state & RS_FAR) ? 0 : 1;
-    const int no_drop = slope ? (int)RS_DROP_MAX : 0, far_add = Dc >= RS_LIMIT ? kp : RS_LOWEST, jt_max = slope ? RS_LIMIT : 0;
+    const int no_drop = slope ? (int)RS_DROP_MAX : 0, far_add = Dc >= RS_LIMIT ? kp : RS_LOWEST, jt_max = slope ? RS_NEAR : 0;
     const int by_first = drop < no_drop ? kp - slope * drop : RS_LOWEST;
     const int by_top = jt < jt_max ? -slope * jt : RS_LOWEST;
     exact = near & (Dc > jt ? 1 : 0);
@@ -688,9 +689,9 @@ struct Folder {
             if (j + 1 < Dc) n.near1 += (unsigned int)(P + j + 1);
             if (lo < Dc) n.far += (unsigned int)(P + min(Dc, lo + steps) - 1);
             store_numbers(w, n);
-            const unsigned int t = max(j < H ? n.near0 + (unsigned int)j : 0u, j + 1 < H ? n.near1 + (unsigned int)(j + 1) : 0u);
+            const unsigned int t0 = j < H ? n.near0 + (unsigned int)j : 0u, t = max(t0, j + 1 < H ? n.near1 + (unsigned int)(j + 1) : 0u);
             n.top = __reduce_max_sync(FULL_MASK, t);
-            n.jtop = __reduce_min_sync(FULL_MASK, t == n.top ? (unsigned int)(j + 1 < H ? j + 1 : j) : 0xffffffffu);
+            n.jtop = __reduce_min_sync(FULL_MASK, t == n.top && j < H ? (unsigned int)(t0 == t ? j : j + 1) : 0xffffffffu);
             const bool beyond = __any_sync(FULL_MASK, n.far > n.top);
             const unsigned int bound = beyond ? max(n.top, __reduce_max_sync(FULL_MASK, n.far)) : 0u;
             full = (beyond && bound >= sc.free_below) || (not_over && (double)most_above(n) > a.many);
@@ -704,7 +705,7 @@ struct Folder {
             not_over = not_over && !((double)n.above > a.many);
             full = (n.jtop >= (unsigned int)RS_NEAR && n.top >= sc.free_below) || (not_over && (double)most_above(n) > a.many);
         }
-        const bool pays = n.top >= sc.free_below, far = pays && n.jtop >= (unsigned int)RS_LIMIT;
+        const bool pays = n.top >= sc.free_below, far = pays && n.jtop >= far_from(H);
         unsigned int key_top = n.top, key_step = n.jtop;
         if (far) key_top = first_top(n.near0, n.near1, H, key_step);
         __syncwarp();   // every lane's cells before the row is handed on
@@ -1887,7 +1888,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
                 if (ADMIT) above = a.over0[i];
             }
             const unsigned int jtop = q.z & 0xffffu, step = (q.z >> 16) & 31u, drop = q.z >> 21;
-            const bool pays = q.y >= sc.free_below, far = pays && jtop >= (unsigned int)RS_LIMIT;
+            const bool pays = q.y >= sc.free_below, far = pays && jtop >= far_from(H);
             jmax = max(jmax, !pays ? 0u : far ? step : jtop);
             n_far += far;
             const bool not_over = ADMIT && !((double)above > a.many);
