@@ -126,7 +126,7 @@ cudaError_t pre_route_configure(pre_ctx* ctx);  // picks G and the shared-memory
 cudaError_t pre_route_summary_configure(pre_ctx* ctx);   // sets ctx->route_summary_smem (0: this shape keeps the scanning kernel)
 bool pre_route_summary_fits(const pre_ctx* ctx);
 bool pre_route_summary_admit_fits(const pre_ctx* ctx);
-bool pre_route_summary_alone(const pre_ctx* ctx);   // small shapes: nothing is launched behind the summary kernel
+bool pre_route_summary_alone(const pre_ctx* ctx, int64_t n_items);   // small shapes: nothing is launched behind the summary kernel
 cudaError_t pre_launch_add_ramps(pre_ctx* ctx, int64_t n_arrivals, const int32_t* prompt, const int32_t* predicted,
                                  const int32_t* instance, int64_t* curves, cudaStream_t s);
 cudaError_t pre_launch_route_summary_admit(pre_ctx* ctx, const int32_t* arr_prompt, const int32_t* arr_predicted,

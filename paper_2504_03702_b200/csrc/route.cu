@@ -1102,7 +1102,7 @@ cudaError_t pre_launch_route(pre_ctx* ctx, const int32_t* arr_prompt, const int3
     if (summaries) {
         e = pre_launch_route_summary(ctx, arr_prompt, arr_predicted, n_arrivals, curves, queued_p, current_d, prompt,
                                      generated, predicted, instance, n_requests, choice, score, s);
-        if (e != cudaSuccess || pre_route_summary_alone(ctx)) return e;
+        if (e != cudaSuccess || pre_route_summary_alone(ctx, n_arrivals)) return e;
     }
     if (!summaries) {    // (else the summary kernel clears them when it declines)
         e = cudaMemsetAsync(ctx->d_abort, 0, 3 * sizeof(int), s);   // flag, agreed exchange, blocks met
@@ -1137,7 +1137,7 @@ cudaError_t pre_launch_route_admit(pre_ctx* ctx, const int32_t* arr_prompt, cons
                                            queue_predicted, queue_state, queue_capacity, queue_choice, curves, queued_p,
                                            current_d, prompt, generated, predicted, instance, n_requests, choice, score,
                                            s);
-        if (e != cudaSuccess || pre_route_summary_alone(ctx)) return e;
+        if (e != cudaSuccess || pre_route_summary_alone(ctx, n_arrivals + queue_capacity)) return e;
     }
     if (!summaries) {
         // The kernel's blocks read the queue's head and length while block 0 may already be writing the

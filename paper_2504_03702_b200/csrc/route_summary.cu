@@ -2095,14 +2095,18 @@ bool pre_route_summary_admit_fits(const pre_ctx* ctx) {
 // Small shapes: the routing block summarises the rows itself and takes what it would decline cell by cell, so that a batch is
 // one launch (or two: the ramps of a longer batch go to the whole GPU).  A launch costs 4 us of the stream here; the block's
 // warps take 0.8 us per row (64 rows: as long as the launch; 256 rows: 25 us more than it).
-bool pre_route_summary_alone(const pre_ctx* ctx) {
-    return ctx->cfg.n_instances <= RS_ALONE_ROWS && (long long)ctx->cfg.n_instances * ctx->cfg.horizon <= RS_ALONE_CELLS;
+// Not for batches whose whole-number scores are likely to pass what the kernel takes (2^29; peaks are guessed at four capacities, requests
+// at 4,096 tokens): the one block takes them cell by cell, 11 us an arrival with 64 x 512 and beta = 1,000, the scanning kernel 2.3.
+bool pre_route_summary_alone(const pre_ctx* ctx, int64_t n_items) {
+    if (ctx->cfg.n_instances > RS_ALONE_ROWS || (long long)ctx->cfg.n_instances * ctx->cfg.horizon > RS_ALONE_CELLS) return false;
+    return !summaries_whole_numbers(ctx) ||
+           (1.0 + ctx->cfg.beta) * (4.0 * (double)ctx->cfg.capacity_tokens + 4096.0 * (double)n_items) < (double)(1 << 29);
 }
 
 static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const int32_t* arr_prompt,
                               const int32_t* arr_predicted, int64_t n_arrivals, int64_t* curves, int64_t* queued_p,
                               int64_t* current_d, int32_t* prompt, int32_t* generated, int32_t* predicted,
-                              int32_t* instance, int64_t* n_requests, int32_t* choice, double* score) {
+                              int32_t* instance, int64_t* n_requests, int32_t* choice, double* score, int64_t queue_capacity) {
     const int I = ctx->cfg.n_instances, H = ctx->cfg.horizon;
     p.curves = curves; p.queued_p = queued_p; p.current_d = current_d;
     p.arr_prompt = arr_prompt; p.arr_predicted = arr_predicted; p.n_arrivals = n_arrivals;
@@ -2123,8 +2127,8 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
     a.status = ctx->d_status; a.handled = ctx->d_rs_handled; a.give_up = ctx->d_abort; a.ramps = ctx->d_rs_ramps;
     a.spin_limit = ctx->spin_limit > 0xffffffffu / RS_POLLS ? 0xffffffffu : RS_POLLS * ctx->spin_limit;
     a.may_decline = ctx->route_path == PRE_ROUTE_AUTO ? 1 : 0;
-    a.alone = pre_route_summary_alone(ctx) ? 1 : 0;
-    a.own_ramps = a.alone && n_arrivals * (long long)H <= RS_OWN_RAMP_CELLS ? 1 : 0;
+    a.alone = pre_route_summary_alone(ctx, n_arrivals + queue_capacity) ? 1 : 0;
+    a.own_ramps = a.alone && (n_arrivals + queue_capacity) * (long long)H <= RS_OWN_RAMP_CELLS ? 1 : 0;
     a.queue_prompt = nullptr; a.queue_predicted = nullptr; a.queue_state = nullptr; a.queue_entry = nullptr;
     a.queue_capacity = 0; a.queue_choice = nullptr; a.hot = 0; a.many = 0.0; a.over0 = nullptr;
 }
@@ -2160,7 +2164,7 @@ cudaError_t pre_launch_route_summary(pre_ctx* ctx, const int32_t* arr_prompt, co
     SumArgs p;
     RouteSumArgs a;
     fill_summary_args(ctx, p, a, arr_prompt, arr_predicted, n_arrivals, curves, queued_p, current_d, prompt, generated,
-                      predicted, instance, n_requests, choice, score);
+                      predicted, instance, n_requests, choice, score, 0);
     return launch_summary_kernels<false>(ctx, p, a, s);
 }
 
@@ -2175,13 +2179,12 @@ cudaError_t pre_launch_route_summary_admit(pre_ctx* ctx, const int32_t* arr_prom
     SumArgs p;
     RouteSumArgs a;
     fill_summary_args(ctx, p, a, arr_prompt, arr_predicted, n_arrivals, curves, queued_p, current_d, prompt, generated,
-                      predicted, instance, n_requests, choice, score);
+                      predicted, instance, n_requests, choice, score, queue_capacity);
     p.over = ctx->d_rs_over; p.hot = hot;
     p.queue_prompt = queue_prompt; p.queue_predicted = queue_predicted; p.queue_state = queue_state;
     p.queue_capacity = queue_capacity;
     a.queue_prompt = queue_prompt; a.queue_predicted = queue_predicted; a.queue_state = queue_state;
     a.queue_entry = ctx->d_queue_entry; a.queue_capacity = queue_capacity; a.queue_choice = queue_choice;
     a.hot = hot; a.many = many; a.over0 = ctx->d_rs_over;
-    a.own_ramps = a.alone && (n_arrivals + queue_capacity) * (long long)a.H <= RS_OWN_RAMP_CELLS ? 1 : 0;
     return launch_summary_kernels<true>(ctx, p, a, s);
 }

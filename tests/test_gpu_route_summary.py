@@ -422,3 +422,33 @@ def test_the_default_is_not_slower_than_the_scanning_kernel(kind):
     assert (choices[B.ROUTE_AUTO] == choices[B.ROUTE_SCAN]).all()
     assert best[B.ROUTE_AUTO] <= 1.5 * best[B.ROUTE_SCAN], best
     st.close()
+
+
+@pytest.mark.parametrize("beta", [1.0, 0.75])
+@pytest.mark.parametrize("queue", [False, True])
+def test_small_shapes_whose_numbers_leave_32_bits_against_expectation(beta, queue):
+    """A small capacity promises small numbers, and one launch without the scanning kernel behind it; the maps hold cells above 2^32 all the
+    same, and the routing block takes the batch cell by cell."""
+    wl = W.make_random(99, 25, 40, 3000, 0, max_prompt=2 ** 27, max_output=60, capacity=1000, beta=beta)
+    rng = np.random.default_rng(17)
+    ap = rng.integers(2 ** 16, 2 ** 24, 80).astype(np.int32)
+    ad = rng.integers(1, 80, 80).astype(np.int32)
+    wl.max_requests = 3000 + 80
+    if not queue:
+        route_and_compare(wl, ap, ad)
+        return
+    st = DeviceState.from_workload(wl)
+    ref = oracle.State.from_workload(wl)
+    st.anticipate()
+    ref.anticipate()
+    st.make_queue(30)
+    ref.make_queue(30)
+    level = float(np.sort(ref.curves.max(axis=1))[-3]) / 1000
+    for lo in (0, 40):
+        qc, c, s = st.route_admit(dev(ap[lo:lo + 40]), dev(ad[lo:lo + 40]), overload_level=level, overload_share=0.0)
+        wqc, wc, ws = ref.route_admit(ap[lo:lo + 40], ad[lo:lo + 40], overload_level=level, overload_share=0.0)
+        assert (c.cpu().numpy() == wc).all() and (qc[:len(wqc)].cpu().numpy() == wqc).all()
+        assert_scores_close(s.cpu().numpy(), ws, wc)
+        assert st.queue_state.cpu().tolist() == ref.queue_state.tolist()
+    assert_state_equal(st, ref)
+    st.close()
