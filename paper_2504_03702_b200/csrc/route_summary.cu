@@ -513,6 +513,7 @@ __device__ __forceinline__ double summary_score(unsigned int tokens, unsigned in
 //   each, and those of binary64, below 2^-10 in these units), so a row whose key value is more than 8 above the smallest one
 //   does not have the smallest score; what is left is compared in binary64, each operation rounded on its own.
 // Odd keys belong to rows whose keys are only lower bounds (one less than the bound).
+constexpr int RS_LEAST_SHIFT = -20;
 constexpr int RS_CUT = 1 << 29, RS_ABSENT = 0x60000000, RS_LOWEST = -(1 << 30), RS_TOP_KEY = 0x3ffffffe;
 template <bool WHOLE> struct Scores {
     static constexpr int SLACK = WHOLE ? 0 : 8;
@@ -531,12 +532,14 @@ template <bool WHOLE> struct Scores {
             theta_i = theta_d > (double)peak_bound ? (int)(peak_bound + 1) : (int)theta_d;
             free_below = max_p <= (unsigned long long)theta_i ? (unsigned int)((unsigned long long)theta_i - max_p) + 1 : 0u;
         } else {
-            // seven binary digits, fewer for long requests or many tokens
+            // seven binary digits, fewer (below none: units of several tokens) for long requests, many tokens or a large beta
             shift = 7;
-            while (shift > 0 && ((double)max_pd * (1.0 + beta) * (double)(2 << shift) > 16777216.0 ||
-                                 (typical_tokens << shift) > (unsigned long long)(RS_CUT / 8)))
+            unit = 128.0;
+            while (shift > RS_LEAST_SHIFT && ((double)max_pd * (1.0 + beta) * 2.0 * unit > 16777216.0 ||
+                                              (double)typical_tokens * unit > (double)(RS_CUT / 8))) {
                 --shift;
-            unit = (double)(1 << shift);
+                unit *= 0.5;
+            }
             const double most = floor(fmin(theta, 8.0e9)) - (double)max_p;
             free_below = most < 0.0 ? 0u : most >= 4294967294.0 ? 0xffffffffu : (unsigned int)most + 1u;
         }
@@ -545,8 +548,11 @@ template <bool WHOLE> struct Scores {
         if (beta == 0.0) free_below = 0xffffffffu;
         code_base = __float_as_int(fmaxf((float)mean * (1.0f / 32.0f) * (float)beta * (float)(2.0 * unit), 1.0f)) >> 21;
     }
+    __device__ __forceinline__ int in_units(unsigned int tokens) const {
+        return (int)min(shift >= 0 ? (unsigned long long)tokens << shift : (unsigned long long)(tokens >> -shift), (unsigned long long)(RS_CUT / 2));
+    }
     __device__ __forceinline__ int key_a(unsigned int tokens) const {
-        return WHOLE ? 2 * (int)tokens : (int)min((unsigned long long)tokens << (shift + 1), (unsigned long long)RS_CUT);
+        return WHOLE ? 2 * (int)tokens : 2 * in_units(tokens);
     }
     __device__ __forceinline__ int key_b(unsigned int tokens, unsigned int t) const {
         if (WHOLE) return 2 * ((int)tokens + beta_i * ((int)t - theta_i));
@@ -557,7 +563,7 @@ template <bool WHOLE> struct Scores {
         return 2 * min(__double2int_rd(beta * (double)P * unit), RS_CUT / 2);
     }
     __device__ __forceinline__ int key_pd(int P, int D) const {
-        return WHOLE ? 2 * (P + D) : (int)min((long long)(P + D) << (shift + 1), (long long)RS_CUT);
+        return WHOLE ? 2 * (P + D) : 2 * in_units((unsigned int)P + (unsigned int)D);
     }
     // The least that an arrival adds to b, and that but for the rounding when its ramp reaches the step of the top (`exact`).  Else
     // the first cell has its prompt, and unless the row is far the cell of the top has what it had; or the ramp reaches all of

@@ -452,3 +452,15 @@ def test_small_shapes_whose_numbers_leave_32_bits_against_expectation(beta, queu
         assert st.queue_state.cpu().tolist() == ref.queue_state.tolist()
     assert_state_equal(st, ref)
     st.close()
+
+
+@pytest.mark.parametrize("beta", [1000.5, 1e5 + 0.5, 1e9 + 0.25, 1e15])
+@pytest.mark.parametrize("n_inst,h", [(40, 900), (300, 80), (2100, 30)])
+def test_large_fractional_penalties(n_inst, h, beta):
+    """Keys in units of several tokens: rows within the rounding are compared in binary64."""
+    wl = W.make_random(580 + n_inst % 89, n_inst, h, 10 * n_inst, 0, max_prompt=3000, max_output=h, beta=beta)
+    rng = np.random.default_rng(24)
+    ap = rng.integers(1, 3000, 500).astype(np.int32)
+    ad = rng.integers(1, 2 * h, 500).astype(np.int32)
+    wl.max_requests = 10 * n_inst + 500
+    route_and_compare(wl, ap, ad, batches=2)
