@@ -66,9 +66,9 @@ typedef struct pre_config {
     int64_t max_requests;    /* capacity of the request table arrays, >= 1, < 2^31 */
 } pre_config;
 
-/* Creates a context on the current CUDA device and allocates its scratch (8 bytes per
- * table slot, 8 bytes per instance, and one index word per build tile and 4,096 table
- * slots: a few MB).  *out is set only on success. */
+/* Creates a context on the current CUDA device and allocates its scratch (15 bytes per
+ * table slot, some 450 bytes per instance, and one index word per build tile and 4,096 table
+ * slots: a few MB to a few tens of MB).  *out is set only on success. */
 int pre_create(const pre_config* cfg, pre_ctx** out);
 
 /* Frees the scratch.  The caller must have synchronised the stream first. */

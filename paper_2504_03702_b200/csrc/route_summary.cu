@@ -29,13 +29,13 @@
 //     deciding warp  takes the arrivals one by one.  It holds rows in registers (two keys each), takes
 //                    every row's score for the arrival, the smallest by two warp reductions, and updates the winner in
 //                    place: no other warp is in this chain.  Up to 256 instances it holds all rows.  Beyond, it holds
-//                    the at most 128 rows of a list, and a table that bounds the scores of all other rows from below:
+//                    the at most 128 rows of a list (256 beyond 2,048 instances), and a table that bounds the scores of all other rows from below:
 //                    while the best row of the list beats that bound it is the best row of all.
 //     list warps     (beyond 256 instances) build the next list while the present one is being used up: the rows
 //                    whose score is within a margin of the smallest one for any of eight prompt lengths, and the
 //                    bounds of the rest.  Scores only grow during a batch, so a list that is a little behind is valid.
-//     folding warps  add each routed request to its row's numbers, one warp per request; an arrival that the rows held
-//                    leave undecided is decided by all of them together on all rows;
+//     folding warps  add each routed request to its row's numbers, one warp per request; they scan single rows for the
+//                    deciding warp, and decide an arrival on all rows together where the rows it holds leave it undecided;
 //     io warp        reads the arrivals ahead of the decisions and writes the results behind them.
 //   Warps 0, 4, 8, ... share one of the SM's four schedulers.  The deciding warp is warp 0 and the others of that scheduler
 //   have nothing to do: the chain of dependent instructions of warp 0 is the time of the batch.
@@ -2047,7 +2047,7 @@ static bool summaries_whole_numbers(const pre_ctx* ctx) {
     return beta == floor(beta) && theta == floor(theta) && beta <= 1048576.0 && theta < 1073741824.0;
 }
 
-// All rows in the deciding warp's registers while that is at most eight per lane, a list of 128 beyond (a list costs a
+// All rows in the deciding warp's registers while that is at most eight per lane, a list of 128 or 256 beyond (a list costs a
 // look at its bounds per arrival and a share of the next list: about what four more rows per lane cost).
 template <bool ADMIT, bool WHOLE>
 static const void* summaries_kernel(int I) {
