@@ -51,8 +51,10 @@
 
 namespace {
 
-constexpr int RS_MAX_FOLD_WARPS = 6;
+constexpr int RS_MAX_FOLD_WARPS = 8;
+constexpr int RS_LIST_WARPS = 6;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
+constexpr int RS_AHEAD = 8;                 // items that are fetched beyond the present one, at most
 constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
 constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lane, 8 beyond RS_LONG_LISTS instances)
 constexpr int RS_LONG_LISTS = 2048;
@@ -79,7 +81,7 @@ constexpr int RS_NO_ROW = 0x3fffffff;
 constexpr int RS_ALONE_ROWS = 64;                  // small shapes: instances,
 constexpr long long RS_ALONE_CELLS = 32768;        // cells of the maps,
 constexpr long long RS_OWN_RAMP_CELLS = 65536;     // and arrivals x steps up to which the routing block adds the ramps
-constexpr unsigned int RS_GIVEN = 0x40000000u, RS_NOBODY = 0xffffffffu;
+constexpr unsigned int RS_GIVEN = 0x40000000u, RS_BY_SLOT = 0x20000000u, RS_NOBODY = 0xffffffffu;
 constexpr unsigned int FULL_MASK = 0xffffffffu;
 
 // guard words written by the summarising kernel; the routing kernel clears them for the next call
@@ -387,7 +389,6 @@ constexpr int RS_SCANS = 0, RS_KEYS = 1, RS_CLOSELY = 2;
 //   state  jtop | drop << RS_DROP (the first cell is that much below the top that b stands for; RS_DROP_MAX: or more) | RS_FAR | RS_FULL | RS_DEFERRED (the map lacks ramps) | RS_NOT_OVER (ADMIT: the row is not overloaded, as
 //          far as folded)
 //   top, tok   top (or, jtop RS_JTOP, an upper bound for which no arrival of the batch pays) and token count (whole-number scores: half of a)
-//   pending  1 from the decision for the row to the end of its fold; cleared last
 constexpr unsigned int RS_FAR = 0x40000000u, RS_NOT_OVER = 0x20000000u, RS_FULL = 0x10000000u, RS_DEFERRED = 0x08000000u, RS_JTOP = 0xffffu,
                        RS_DROP_MAX = 2047u;
 constexpr int RS_DROP = 16;
@@ -395,27 +396,29 @@ struct Rows {
     int2* rec;
     unsigned int* state;
     unsigned int* top;
-    unsigned int* pending;
     unsigned int* tok;
 };
 
 struct RsShared {
     // what the deciding warp tells the folding warps and the io warp, read with one access
     uint4 ctl;                              // {decisions made, arrivals for all rows, 1: no more of either, 1: a wait was abandoned}
-    int4 items[RS_ITEMS];                   // of the requests to route, in order: {what P adds to b, P + D as a key, less one, min(D, H)
-                                            // (0: not for the quick way), offset of P's entry in the table}
+    int4 items[RS_ITEMS + RS_AHEAD];        // of the requests to route, in order: {what P adds to b, P + D as a key and the mark, min(D, H)
+                                            // (0: not for the quick way), offset of P's entry in the table}; both keys as in Held; the first ones
+                                            // once more behind the last
     int2 raw[RS_ITEMS];                     // {P, D}
     int item_at[RS_ITEMS];                  // their indices in the batch
-    uint2 jobs[RS_ITEMS];                   // decisions: {row | RS_GIVEN if the peak is given, peak}
-    double score[RS_ITEMS];                 // their scores, from the folding warps
+    uint2 jobs[RS_ITEMS];                   // decisions: {row, or until it is folded 2 * slot | list's parity << 16 | RS_BY_SLOT; RS_GIVEN if the peak is
+                                            // given, peak}
+    unsigned int pending[RS_LIST_ROWS];     // by slot of the row held: 1 from the decision for it to the end of its fold; cleared last
+    uint2 scored[RS_ITEMS];                 // {token count, peak} of their scores, from the folding warps
     int4 table[2][32];                      // by code of the prompt: {bounds of the rows outside the list}
     int list_row[2][RS_LIST_ROWS];
-    int list_n[2];
+    int list_n[2], list_base[2];
+    unsigned short list_seg[RS_LIST_WARPS][RS_LIST_ROWS];      // (list warps) each one's rows of the list, and their number
+    int list_take[RS_LIST_WARPS];
     unsigned int bucket_a[32], bucket_b[32];   // (list warps) smallest keys of the rows outside the list
     unsigned int probe_t[RS_PROBES];        // (list warps) smallest scores at the probes
     unsigned short near_row[RS_NEAR_ROWS];
-    int list_count;
-    unsigned int list_met;                  // (list warps) arrivals at their meetings
     unsigned int lists_wanted, lists_ready;
     unsigned int done[RS_MAX_FOLD_WARPS];   // the next decision each folding warp will fold
     unsigned int looks_done[RS_MAX_FOLD_WARPS];
@@ -513,6 +516,26 @@ __device__ __forceinline__ double summary_score(unsigned int tokens, unsigned in
 //   each, and those of binary64, below 2^-10 in these units), so a row whose key value is more than 8 above the smallest one
 //   does not have the smallest score; what is left is compared in binary64, each operation rounded on its own.
 // Odd keys belong to rows whose keys are only lower bounds (one less than the bound).
+//
+// The deciding warp holds its rows' keys in another form: relative to a base (the smallest score of any row for an empty prompt when the
+// rows or the list were taken; scores only grow), with the row's slot and its mark below:
+//     (key - base, cut at LIMIT either way) * 2^SLOT_BITS | 2 * slot | mark
+// Slots ascend with the rows, so ONE reduction gives the smallest score, the lowest row that has it (the paper's tie-break) and whether
+// that row is marked; a reduction for the score and one for the row took 37 cycles and a compare more (a step of the deciding warp alone,
+// two and four rows per lane: 127 and 139 cycles with two reductions, 65 and 85 with one).
+//   * A marked row's keys are lower bounds: if the bound is the smallest the arrival is settled outside the loop, and if it is not, the
+//     row is not the best one: among equal scores the mark counts less than the slot.
+//   * A key cut below is too large, but has no say: a < base of a row whose score is b, or b + beta * P <= base of one whose score is a,
+//     as what an arrival adds is at most ITEM and a row gets at most two before its keys are read again.
+//   * A key cut above, or a score from CUT on, is not decided on.
+template <int KS> struct Held {
+    static constexpr int SLOT_BITS = KS == 1 ? 5 : KS == 2 ? 6 : KS == 4 ? 7 : 8;
+    static_assert((1 << SLOT_BITS) == 32 * KS, "");
+    static constexpr int TAGS = (2 << SLOT_BITS) - 1, SLOT = TAGS - 1;
+    static constexpr int LIMIT = 1 << (30 - SLOT_BITS), CUT = LIMIT / 2, ITEM = LIMIT / 4;
+    static __device__ __forceinline__ int scaled(int key) { return key * (1 << SLOT_BITS); }
+    static __device__ __forceinline__ int relative(int key, int base) { return scaled(min(max(key - base, -LIMIT), LIMIT)); }
+};
 constexpr int RS_LEAST_SHIFT = -20;
 constexpr int RS_CUT = 1 << 29, RS_ABSENT = 0x60000000, RS_LOWEST = -(1 << 30), RS_TOP_KEY = 0x3ffffffe;
 template <bool WHOLE> struct Scores {
@@ -522,7 +545,7 @@ template <bool WHOLE> struct Scores {
     int slope;           // what a token less at the peak takes from b at most (0: too much)
     unsigned int free_below;     // a row whose top is below pays no penalty, whatever arrival of the batch it gets
     __device__ __forceinline__ void start(double theta_d, double beta_d, unsigned long long peak_bound, unsigned long long max_pd, unsigned long long max_p,
-                                          unsigned long long typical_tokens, int mean) {
+                                          unsigned long long typical_tokens, int mean, int item_limit) {
         theta = theta_d; beta = beta_d;
         beta_i = theta_i = shift = 0;
         unit = 1.0;
@@ -535,7 +558,8 @@ template <bool WHOLE> struct Scores {
             // seven binary digits, fewer (below none: units of several tokens) for long requests, many tokens or a large beta
             shift = 7;
             unit = 128.0;
-            while (shift > RS_LEAST_SHIFT && ((double)max_pd * (1.0 + beta) * 2.0 * unit > 16777216.0 ||
+            const double long_pd = fmin((double)max_pd, 16.0 * (double)mean + 16.0);      // (longer ones are left to the unusual way)
+            while (shift > RS_LEAST_SHIFT && (long_pd * (1.0 + beta) * 2.0 * unit > (double)item_limit ||
                                               (double)typical_tokens * unit > (double)(RS_CUT / 8))) {
                 --shift;
                 unit *= 0.5;
@@ -569,8 +593,6 @@ template <bool WHOLE> struct Scores {
     // the first cell has its prompt, and unless the row is far the cell of the top has what it had; or the ramp reaches all of
     // the first steps.  (Selects and no branches: with them a row cost the looking warp 150 cycles.)
     __device__ __forceinline__ int key_least(unsigned int state, int kp, int Dc, int& exact) const;
-    // whether the keys of 32 such arrivals in a row stay below their cut
-    __device__ __forceinline__ bool usual(int kp, int kpd) const { return WHOLE || kp + kpd <= 16777216; }
     __device__ __forceinline__ unsigned int tokens_of(const Rows& rows, int i) const { return WHOLE ? (unsigned int)rows.rec[i].x >> 1 : rows.tok[i]; }
     // Codes of what a prompt adds, and of what a row lacks to pay a penalty: monotone, so different codes decide which is
     // larger.  Four per octave.  0 (rows): pays for every prompt.
@@ -611,12 +633,19 @@ __device__ __forceinline__ unsigned int ordered(int v) { return (unsigned int)v 
 __device__ __forceinline__ int unordered(unsigned int v) { return (int)(v ^ 0x80000000u); }
 
 // ---- folding warps
-template <bool ADMIT, bool WHOLE>
+__device__ __forceinline__ unsigned int job_slot(unsigned int job) { return (job >> 1) & (RS_LIST_ROWS - 1); }
+template <bool LISTS>
+__device__ __forceinline__ int job_row(const RsShared& sh, unsigned int job) {
+    if (!(job & RS_BY_SLOT)) return (int)(job & ~RS_GIVEN);
+    return LISTS ? sh.list_row[(job >> 16) & 1][job_slot(job)] : (int)job_slot(job);
+}
+template <bool ADMIT, bool WHOLE, bool LISTS>
 struct Folder {
     const RouteSumArgs& a;
     RsShared& sh;
     const Rows& rows;
     const Scores<WHOLE>& sc;
+    int far_steps;      // steps of a stretch
 
     __device__ __forceinline__ void store_numbers(int w, const RowNumbers& n) {
         a.near[(size_t)w * 32 + (threadIdx.x & 31)] = make_uint2(n.near0, n.near1);
@@ -624,7 +653,7 @@ struct Folder {
     }
     // At most so many cells are above the overload level: the first ones counted, a stretch whole if its bound is above.
     __device__ __forceinline__ int most_above(const RowNumbers& n) {
-        const int lane = threadIdx.x & 31, H = a.H, j = 2 * lane, steps = far_chunks(H) * RS_NEAR, lo = RS_NEAR + lane * steps;
+        const int lane = threadIdx.x & 31, H = a.H, j = 2 * lane, steps = far_steps, lo = RS_NEAR + lane * steps;
         int above = (j < H && (long long)n.near0 > a.hot) + (j + 1 < H && (long long)n.near1 > a.hot);
         if (lo < H && (long long)n.far - lo > a.hot) above += min(steps, H - lo);
         return __reduce_add_sync(FULL_MASK, above);
@@ -678,22 +707,19 @@ struct Folder {
         const int lane = threadIdx.x & 31, H = a.H;
         const uint2 job = sh.jobs[e % RS_ITEMS];
         const int2 pd = sh.raw[e % RS_ITEMS];
-        const int w = (int)(job.x & ~RS_GIVEN), P = pd.x, D = pd.y, Dc = D < H ? D : H;
+        const int w = job_row<LISTS>(sh, job.x), P = pd.x, D = pd.y, Dc = D < H ? D : H;
+        const uint2 q = a.near[(size_t)w * 32 + lane];      // (on their way before anything else)
+        const unsigned int q_far = a.far[(size_t)w * 32 + lane];
         const unsigned int state = rows.state[w], old_top = rows.top[w];
         const unsigned int tokens = sc.tokens_of(rows, w);
-        if (lane == 0)
-            sh.score[e % RS_ITEMS] = summary_score(tokens, (job.x & RS_GIVEN) ? job.y : old_top + (unsigned int)P, (double)P + (double)D, a.theta, a.beta);
         RowNumbers n;
         bool full = (state & RS_FULL) != 0, deferred = (state & RS_DEFERRED) != 0;
         bool not_over = ADMIT && (state & RS_NOT_OVER) != 0;      // (once a row is overloaded it stays so: cells only grow)
         if (!full) {
-            const uint2 q = a.near[(size_t)w * 32 + lane];
-            n.near0 = q.x; n.near1 = q.y;
-            n.far = a.far[(size_t)w * 32 + lane];
-            const int j = 2 * lane, steps = far_chunks(H) * RS_NEAR, lo = RS_NEAR + lane * steps;
-            if (j < Dc) n.near0 += (unsigned int)(P + j);
-            if (j + 1 < Dc) n.near1 += (unsigned int)(P + j + 1);
-            if (lo < Dc) n.far += (unsigned int)(P + min(Dc, lo + steps) - 1);
+            const int j = 2 * lane, steps = far_steps, lo = RS_NEAR + lane * steps;
+            n.near0 = q.x + (j < Dc ? (unsigned int)(P + j) : 0u);
+            n.near1 = q.y + (j + 1 < Dc ? (unsigned int)(P + j + 1) : 0u);
+            n.far = q_far + (lo < Dc ? (unsigned int)(P + min(Dc, lo + steps) - 1) : 0u);
             store_numbers(w, n);
             const unsigned int t0 = j < H ? n.near0 + (unsigned int)j : 0u, t = max(t0, j + 1 < H ? n.near1 + (unsigned int)(j + 1) : 0u);
             n.top = __reduce_max_sync(FULL_MASK, t);
@@ -723,7 +749,9 @@ struct Folder {
             rows.rec[w] = make_int2(sc.key_a(now), sc.key_b(now, key_top));
             rows.state[w] = n.jtop | (drop_of(key_top, n.near0) << RS_DROP) | (far ? RS_FAR : 0u) | (full ? RS_FULL : 0u) | (deferred ? RS_DEFERRED : 0u) | (not_over ? RS_NOT_OVER : 0u);
             if (ADMIT && (state & RS_NOT_OVER) && !not_over) atomicSub(&sh.not_over, 1u);
-            st_release(&rows.pending[w], 0u);
+            sh.scored[e % RS_ITEMS] = make_uint2(tokens, (job.x & RS_GIVEN) ? job.y : old_top + (unsigned int)P);
+            sh.jobs[e % RS_ITEMS].x = (unsigned int)w | (job.x & RS_GIVEN);
+            if (job.x & RS_BY_SLOT) st_release(&sh.pending[job_slot(job.x)], 0u);
         }
         return true;
     }
@@ -732,7 +760,7 @@ struct Folder {
         const int lane = threadIdx.x & 31, H = a.H;
         // the first cells, and what bounds the others: enough when Dc ends among the first and none of the others can be larger
         const uint2 q = a.near[(size_t)w * 32 + lane];
-        const int j = 2 * lane, lo = RS_NEAR + lane * far_chunks(H) * RS_NEAR;
+        const int j = 2 * lane, lo = RS_NEAR + lane * far_steps;
         const unsigned int u = a.far[(size_t)w * 32 + lane];
         peak = __reduce_max_sync(FULL_MASK, max(q.x + (j < Dc ? (unsigned int)(P + j) : 0u), q.y + (j + 1 < Dc ? (unsigned int)(P + j + 1) : 0u)));
         const bool others = Dc > RS_NEAR || u > peak + (unsigned int)(u ? lo : 0);
@@ -753,7 +781,7 @@ struct Folder {
 // rounding.  A closer look takes the scores of the rows that can be the best, and scans those that are only bounded.
 // What bounds it: the hand-over and one or two passes over the rows' words in shared memory.  By the deciding warp alone the look at the
 // keys took 3,000 cycles with 4,096 rows, and the closer one, taken for all bounded rows and all binary64 scores, 28,000.
-template <int FOLD_WARPS, bool ADMIT, bool WHOLE>
+template <int FOLD_WARPS, bool ADMIT, bool WHOLE, bool LISTS>
 struct Look {
     typedef typename Scores<WHOLE>::S S;
     static constexpr int STRIDE = 32 * FOLD_WARPS;
@@ -852,7 +880,7 @@ struct Look {
         sh.look_peak[stage][me] = peak;
     }
     __device__ __forceinline__ bool closely(int me, unsigned int decided) {
-        static_assert((RS_MAX_ROWS + 32 * 6 - 1) / (32 * 6) <= 64, "a bit for each row of a lane");
+        static_assert((RS_MAX_ROWS + STRIDE - 1) / STRIDE <= 64 || !LISTS, "a bit for each row of a lane");
         const int lane = threadIdx.x & 31, I = a.I, first = 32 * me + lane;
         const int P = sh.look_P, D = sh.look_D, Dc = D < a.H ? D : a.H, kp = sc.key_p(P);
         int least = 0x7fffffff;
@@ -906,7 +934,7 @@ struct Look {
                     const int src = __ffs(which) - 1, w = __shfl_sync(FULL_MASK, i, src);
                     const unsigned int t = __shfl_sync(FULL_MASK, tokens, src);
                     unsigned int p = 0;
-                    Folder<ADMIT, WHOLE> f{a, sh, rows, sc};
+                    Folder<ADMIT, WHOLE, LISTS> f{a, sh, rows, sc, far_chunks(a.H) * RS_NEAR};
                     if (!f.scan(w, P, Dc, decided, p)) return false;
                     const S s = sc.of_peak(t, p, P, D);
                     if (s < best || (s == best && w < win)) { best = s; win = w; peak = p; }
@@ -922,8 +950,8 @@ struct Look {
 template <int FOLD_WARPS, bool ADMIT, bool WHOLE, bool LISTS>
 __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int me) {
     const int lane = threadIdx.x & 31;
-    Folder<ADMIT, WHOLE> f{a, sh, rows, sc};
-    Look<FOLD_WARPS, ADMIT, WHOLE> look{a, sh, rows, sc, 0u};
+    Folder<ADMIT, WHOLE, LISTS> f{a, sh, rows, sc, far_chunks(a.H) * RS_NEAR};
+    Look<FOLD_WARPS, ADMIT, WHOLE, LISTS> look{a, sh, rows, sc, 0u};
     unsigned int looks = 0;
     for (unsigned int n = me;;) {
         uint4 ctl;
@@ -962,7 +990,7 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
 }
 
 // ---- io warp: arrivals ahead of the decisions, results behind the folds
-template <int FOLD_WARPS, bool ADMIT, bool WHOLE>
+template <int KS, int FOLD_WARPS, bool ADMIT, bool WHOLE>
 __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, const Scores<WHOLE>& sc, long long q_head, int waiting, int items, int room) {
     const int lane = threadIdx.x & 31;
     const long long n0 = sh.n0;
@@ -995,7 +1023,10 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
             const unsigned int slot = entered + __popc(vote & ((1u << lane) - 1u));
             if (ok && slot < (unsigned int)room) {
                 const int kp = sc.key_p(P), kpd = sc.key_pd(P, D);
-                sh.items[slot % RS_ITEMS] = make_int4(kp, kpd - 1, sc.usual(kp, kpd) ? (D < a.H ? D : a.H) : 0, 16 * sc.code((float)kp));
+                const bool usual = kp <= Held<KS>::ITEM && kpd <= Held<KS>::ITEM - kp;
+                const int4 item = make_int4(usual ? Held<KS>::scaled(kp) : 0, (usual ? Held<KS>::scaled(kpd) : 0) + 1, usual ? (D < a.H ? D : a.H) : 0, 16 * sc.code((float)kp));
+                sh.items[slot % RS_ITEMS] = item;
+                if (slot % RS_ITEMS < RS_AHEAD) sh.items[RS_ITEMS + slot % RS_ITEMS] = item;
                 sh.raw[slot % RS_ITEMS] = make_int2(P, D);
                 sh.item_at[slot % RS_ITEMS] = k;
             } else if (k < items) {
@@ -1028,7 +1059,8 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
                 a.link[e] = below ? e - lane + (31 - __clz(below)) : __ldcg(a.newest + w);
                 __syncwarp(some);
                 if ((same >> lane) == 1u) __stcg(a.newest + w, e);
-                put_result(sh.item_at[e % RS_ITEMS], w, sh.score[e % RS_ITEMS]);
+                const uint2 of = sh.scored[e % RS_ITEMS];
+                put_result(sh.item_at[e % RS_ITEMS], w, summary_score(of.x, of.y, (double)pd.x + (double)pd.y, a.theta, a.beta));
                 atomicAdd(reinterpret_cast<unsigned long long*>(a.queued_p + w), (unsigned long long)pd.x);
                 atomicAdd(reinterpret_cast<unsigned long long*>(a.current_d + w), (unsigned long long)pd.y);
             }
@@ -1060,22 +1092,27 @@ __device__ __forceinline__ int rs_probe(int mean, int x) {
     return (int)((float)mean * share[x]);
 }
 
-template <int LIST_WARPS, int ROOM, bool WHOLE>
-__device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int I, int mean, int longest, int t) {
-    constexpr int THREADS = 32 * LIST_WARPS, NEAR_ROOM = RS_NEAR_ROWS / LIST_WARPS;
+__device__ __forceinline__ void prefetch_row(const uint2* near, const unsigned int* far, int row) {
+    asm volatile("prefetch.global.L1 [%0]; prefetch.global.L1 [%0 + 128]; prefetch.global.L1 [%1];" ::"l"(near + (size_t)row * 32), "l"(far + (size_t)row * 32));
+}
+
+template <int LIST_WARPS, int KS, bool WHOLE>
+__device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, const uint2* near_cells, const unsigned int* far_cells, int I, int mean, int longest, int t) {
+    constexpr int THREADS = 32 * LIST_WARPS, ROOM = 32 * KS, NEAR_ROOM = RS_NEAR_ROWS / LIST_WARPS;
     constexpr int FAR_KEY = 0x7f000000, AT_ONCE = 4;      // AT_ONCE: rows a thread has on their way
     static_assert(NEAR_ROOM >= 2 * 32 * AT_ONCE, "");
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, me = t >> 5;
     const bool leader = t < 32;
-    unsigned int met = 0;
     auto over = [&] { return __any_sync(FULL_MASK, ld_volatile(&sh.ctl.z) != 0); };
-    auto team = [&]() -> bool {   // the list warps meet (false: abandoned, or the last decision has been made)
-        met += LIST_WARPS;
+    // The list warps meet at a barrier of their own, and leave together if one of them has seen that the last decision is made.  (Polls of
+    // a counter took 500 cycles a meeting and the other warps' issue slots.)
+    auto meet = [&](bool stop) -> bool {
+        int leave;
         __syncwarp();
-        acquire_cta();
-        if (lane == 0) atomicAdd(&sh.list_met, 1u);
-        return rs_wait(sh, [&] { return (int)(ld_acquire(&sh.list_met) - met) >= 0 || ld_volatile(&sh.ctl.z) != 0; }) && !over();
+        asm volatile("{ .reg .pred p, q; setp.ne.s32 p, %1, 0; barrier.cta.red.or.pred q, 1, %2, p; selp.s32 %0, 1, 0, q; }" : "=r"(leave) : "r"((int)stop), "n"(THREADS) : "memory");
+        return leave != 0;
     };
+    auto empty_buckets = [&] { if (leader) { sh.bucket_a[lane] = 0xffffffffu; sh.bucket_b[lane] = 0xffffffffu; } };
     int probe_key = 0;
     int bp[RS_PROBES];
     #pragma unroll
@@ -1085,20 +1122,21 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
     }
     int margin = max(sc.key_a((unsigned int)mean) / 16, 8);
     const int least_margin = max(sc.key_a(1u), 1);
-    unsigned short* near = sh.near_row + (t >> 5) * NEAR_ROOM;
+    unsigned short* near = sh.near_row + me * NEAR_ROOM;
+    // (a warp has neighbouring rows: the list is put together in their order)
+    const int share = ((I + THREADS - 1) / THREADS) * 32, first = me * share, end = min(I, first + share);
     for (unsigned int n = 1;; ++n) {
-        bool go = false;
-        if (!rs_wait<true>(sh, [&] {
-                const uint4 ctl = ld_volatile4(&sh.ctl);
-                go = ld_acquire(&sh.lists_wanted) >= n;
-                return go || ctl.z != 0;
-            }, 20))
-            return;
-        go = __any_sync(FULL_MASK, ld_acquire(&sh.lists_wanted) >= n);
-        if (!go) return;     // (nothing is asked for after the last decision)
+        bool stop = false;
+        if (leader) {      // (one of them looks for work, the others wait for it)
+            stop = !rs_wait<true>(sh, [&] {
+                const unsigned int last = ld_volatile(&sh.ctl.z);
+                return ld_acquire(&sh.lists_wanted) >= n || last != 0;
+            }, 20);
+            stop = stop || !__any_sync(FULL_MASK, ld_acquire(&sh.lists_wanted) >= n);     // (nothing is asked for after the last decision)
+        }
+        if (meet(stop)) return;
         const int old = (n + 1) & 1, now = n & 1;
         // the smallest value known per probe: the rows of the present list, and (kept in probe_t) the others' bound
-        if (!team()) return;
         if (n > 1) {   // (the first list: probe_t was set when the rows were loaded)
             const int old_n = sh.list_n[old];
             if (t - lane < old_n) {
@@ -1110,17 +1148,17 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
                     #pragma unroll
                     for (int p = 0; p < RS_PROBES; ++p) least[p] = min(least[p], max(r.x, r.y + bp[p]));
                 }
+                int mine = 0;
                 #pragma unroll
                 for (int p = 0; p < RS_PROBES; ++p) {
                     const int v = __reduce_min_sync(FULL_MASK, least[p]);
-                    if (lane == 0) atomicMin(&sh.probe_t[p], ordered(v));
+                    mine = lane == p ? v : mine;
                 }
+                if (lane < RS_PROBES) atomicMin(&sh.probe_t[lane], ordered(mine));
             }
         }
+        if (meet(over())) return;
         for (int tries = 0;; ++tries) {
-            if (leader) { sh.bucket_a[lane] = 0xffffffffu; sh.bucket_b[lane] = 0xffffffffu; }
-            if (t == 0) sh.list_count = 0;
-            if (!team()) return;
             // A row is in the list if for some probe its a is at most limit_a and its b at most limit_b.
             // Rows beyond far_a or far_b are out of reach of this list: the two limits bound them, and they are dropped by
             // two comparisons.
@@ -1135,61 +1173,88 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
             const int far_b = limit_a[0];
             far_a = (int)min((long long)far_a + longest, (long long)RS_ABSENT);
             int hot_b = FAR_KEY, cold_a = FAR_KEY;
-            int n_near = 0;
+            int n_near = 0, n_take = 0;
             auto sort_near = [&]() {        // the rows that were not dropped: into the list or into a bucket
                 __syncwarp();
-                for (int x = lane; x - lane < n_near; x += 32) {
-                    const bool in = x < n_near;
-                    const int i = in ? near[x] : 0;
-                    const int2 r = ld_volatile2(rows.rec + i);
-                    bool take = false;
+                // (two rows a lane at once and no branches: what bounds this is the latency of a row's chain)
+                for (int x = lane; x - lane < n_near; x += 64) {
+                    int2 r[2];
+                    bool in[2], take[2], low[2];
+                    int i[2], c[2];
                     #pragma unroll
-                    for (int p = 0; p < RS_PROBES; ++p) take |= r.x <= limit_a[p] && r.y <= limit_b[p];
-                    take &= in;
-                    const unsigned int vote = __ballot_sync(FULL_MASK, take);
-                    if (vote) {
-                        int at = 0;
-                        if (lane == 0) at = atomicAdd(&sh.list_count, __popc(vote));
-                        at = __shfl_sync(FULL_MASK, at, 0) + __popc(vote & ((1u << lane) - 1u));
-                        if (take && at < ROOM) sh.list_row[now][at] = i;
+                    for (int u = 0; u < 2; ++u) { in[u] = x + 32 * u < n_near; i[u] = near[in[u] ? x + 32 * u : 0]; }
+                    #pragma unroll
+                    for (int u = 0; u < 2; ++u) r[u] = ld_volatile2(rows.rec + i[u]);
+                    #pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        take[u] = false;
+                        #pragma unroll
+                        for (int p = 0; p < RS_PROBES; ++p) take[u] |= r[u].x <= limit_a[p] && r[u].y <= limit_b[p];
+                        take[u] &= in[u];
+                        c[u] = sc.row_code(r[u]);
                     }
-                    if (in && !take) {
-                        const int c = sc.row_code(r);
-                        if (c == 0) hot_b = min(hot_b, r.y);
-                        else if (c == 31) cold_a = min(cold_a, r.x);
-                        else {
-                            atomicMin(&sh.bucket_a[c], ordered(r.x));
-                            atomicMin(&sh.bucket_b[c], ordered(r.y));
-                        }
+                    #pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const unsigned int vote = __ballot_sync(FULL_MASK, take[u]);
+                        const int at = n_take + __popc(vote & ((1u << lane) - 1u));
+                        if (take[u] && at < ROOM) sh.list_seg[me][at] = (unsigned short)i[u];
+                        n_take += __popc(vote);
+                        const bool left = in[u] && !take[u], middle = left && c[u] != 0 && c[u] != 31;
+                        hot_b = min(hot_b, left && c[u] == 0 ? r[u].y : FAR_KEY);
+                        cold_a = min(cold_a, left && c[u] == 31 ? r[u].x : FAR_KEY);
+                        low[u] = middle && (ordered(r[u].x) < ld_volatile(&sh.bucket_a[c[u]]) || ordered(r[u].y) < ld_volatile(&sh.bucket_b[c[u]]));
+                    }
+                    if (__any_sync(FULL_MASK, low[0] || low[1])) {      // (most rows change no bucket)
+                        #pragma unroll
+                        for (int u = 0; u < 2; ++u)
+                            if (low[u]) {
+                                atomicMin(&sh.bucket_a[c[u]], ordered(r[u].x));
+                                atomicMin(&sh.bucket_b[c[u]], ordered(r[u].y));
+                            }
                     }
                 }
                 __syncwarp();
                 n_near = 0;
             };
-            for (int base = 0; base < I; base += AT_ONCE * THREADS) {
-                if (over()) return;
+            for (int base = first; base < end; base += AT_ONCE * 32) {
                 int2 r[AT_ONCE];
                 #pragma unroll
                 for (int u = 0; u < AT_ONCE; ++u) {
-                    const int i = base + u * THREADS + t;
-                    if (i < I) r[u] = ld_volatile2(rows.rec + i);
+                    const int i = base + u * 32 + lane;
+                    r[u] = ld_volatile2(rows.rec + (i < end ? i : first));
                 }
+                const bool enough = over();
                 #pragma unroll
                 for (int u = 0; u < AT_ONCE; ++u) {
-                    const int i = base + u * THREADS + t;
-                    const bool keep = i < I && r[u].y <= far_b && r[u].x <= far_a;
+                    const int i = base + u * 32 + lane;
+                    const bool keep = i < end && r[u].y <= far_b && r[u].x <= far_a;
                     const unsigned int vote = __ballot_sync(FULL_MASK, keep);
                     if (keep) near[n_near + __popc(vote & ((1u << lane) - 1u))] = (unsigned short)i;
                     n_near += __popc(vote);
                 }
+                if (enough) break;
                 if (n_near > NEAR_ROOM - AT_ONCE * 32) sort_near();
             }
             sort_near();
             const int hb = __reduce_min_sync(FULL_MASK, hot_b), ca = __reduce_min_sync(FULL_MASK, cold_a);
-            if (lane == 0) { atomicMin(&sh.bucket_b[0], ordered(hb)); atomicMin(&sh.bucket_a[31], ordered(ca)); }
-            if (!team()) return;
-            const int count = sh.list_count;
-            if (count > ROOM) { margin = max(margin / 2, least_margin); if (tries > 4) margin = 0; if (!team()) return; continue; }
+            if (lane == 0) { atomicMin(&sh.bucket_b[0], ordered(hb)); atomicMin(&sh.bucket_a[31], ordered(ca)); sh.list_take[me] = n_take; }
+            if (meet(over())) return;
+            const int taken = lane < LIST_WARPS ? sh.list_take[lane] : 0, count = __reduce_add_sync(FULL_MASK, taken);
+            // (the margin that fills four fifths of the list, were its rows spread evenly)
+            const int fitting = (int)((float)margin * fmaxf(0.8f * ROOM / (float)max(count, 1), 0.25f));
+            if (count > ROOM) {
+                margin = max(min(fitting, margin / 2 + margin / 4), least_margin);
+                if (tries > 4) margin = 0;
+                empty_buckets();
+                if (meet(over())) return;
+                continue;
+            }
+            const int before = __reduce_add_sync(FULL_MASK, lane < me ? taken : 0);
+            for (int x = lane; x < n_take; x += 32) {
+                const int i = sh.list_seg[me][x];
+                sh.list_row[now][before + x] = i;
+                prefetch_row(near_cells, far_cells, i);     // (the folds of its rows: 280 cycles less)
+            }
             if (leader) {
                 // (a key that no row has set is out of reach; rows of code 31 count by their a alone, no b is kept for them)
                 const int ka = unordered(min(sh.bucket_a[lane], ordered(RS_ABSENT)));
@@ -1205,58 +1270,88 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
                 below_b = __shfl_up_sync(FULL_MASK, below_b, 1);
                 if (lane == 31) above_a = far_a;
                 if (lane == 0) below_b = far_b;
-                sh.table[now][lane] = make_int4(above_a, below_b, ka, lane == 31 ? RS_LOWEST : kb);
+                const int row_b = lane == 31 ? RS_LOWEST : kb;
+                // The entries as keys that the deciding warp holds: a row that wins by less than the rounding of its key does not beat them.
+                // (The base is a lower bound of every row's score, so an entry that is cut below is one, too.)
+                const int base = unordered(sh.probe_t[0]) & ~1;
+                auto entry = [&](int key) { return Held<KS>::relative(key, base) - 1 - Held<KS>::scaled(Scores<WHOLE>::SLACK); };
+                sh.table[now][lane] = make_int4(entry(above_a), entry(below_b), entry(ka), entry(row_b));
+                const int c = sc.code((float)probe_key);
+                const int ex = __shfl_sync(FULL_MASK, above_a, c), ey = __shfl_sync(FULL_MASK, below_b, c), ez = __shfl_sync(FULL_MASK, ka, c), ew = __shfl_sync(FULL_MASK, row_b, c);
                 __syncwarp();
-                if (lane < RS_PROBES) {
-                    const int4 e = sh.table[now][sc.code((float)probe_key)];
-                    sh.probe_t[lane] = ordered(min(min(e.x, e.y + probe_key), max(e.z, e.w + probe_key)));
-                }
-                if (lane == 0) sh.list_n[now] = count;
-                __syncwarp();
-                if (lane == 0) st_release(&sh.lists_ready, n);
+                if (lane < RS_PROBES) sh.probe_t[lane] = ordered(min(min(ex, ey + probe_key), max(ez, ew + probe_key)));
+                if (lane == 0) { sh.list_n[now] = count; sh.list_base[now] = base; }
+                empty_buckets();
             }
-            if (count < ROOM * 3 / 5) margin = min(margin + margin / 2 + 1, 1 << 27);
+            if (meet(over())) return;
+            if (t == 0) st_release(&sh.lists_ready, n);
+            margin = max(min(min(fitting, margin + margin / 2 + 1), 1 << 27), least_margin);
             break;
         }
     }
 }
 
 // ---- deciding warp.  KS: rows per lane.  LISTS: they are a list's, else all rows.
-// What bounds it: the latency of one chain of dependent instructions per arrival (two warp reductions and some ten integer
-// operations) and the number of its instructions, so the usual way through the loop has a single branch, to everything
-// unusual, and what need not be in the chain (scores, token counts, the tables) is done by the folding warps.
+// What bounds it: the latency of one chain of dependent instructions per arrival (a warp reduction, 23 cycles, and some eight integer
+// operations: 65 cycles with two rows per lane, in a kernel with nothing else) and, with four and eight rows per lane, the number of its
+// instructions (85 and 130).  So nothing else is in the loop: no branch (one per step cost 50 to 100 cycles; whether all steps were usual
+// is seen once per trip, which is taken back as far as they were not), items and bounds fetched two steps ahead, and what need not
+// be in the chain (scores, token counts, the tables) is done by the folding warps.
 template <int KS, bool LISTS, int FOLD_WARPS, bool ADMIT, bool WHOLE>
 __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc) {
     typedef typename Scores<WHOLE>::S S;
-    constexpr int SLACK = Scores<WHOLE>::SLACK;
+    typedef Held<KS> K;
+    constexpr int SLACK = Scores<WHOLE>::SLACK * (1 << K::SLOT_BITS);
+    // steps of a trip: decisions are made known to the folding warps by trips (few rows: soon)
+    constexpr int TRIP = KS <= 2 ? 2 : 4;
     // decisions between two looks at items and at the rows that were pending
     constexpr unsigned int CHUNK = LISTS ? 32 : 4 * KS;
-    // decisions made known to the folding warps at once (few rows: soon)
-    constexpr unsigned int PUBLISH = LISTS ? 4 : (KS >= 4 ? 2 : 1);
     const int lane = threadIdx.x & 31, I = a.I, H = a.H;
     const int lane_f = lane < FOLD_WARPS ? lane : 0;
     unsigned int looks = 0;
     bool lost = false;
 
-    // ---- the rows held by the lane, ascending, and their keys: odd for a row that is marked (pending when the lane last
-    // looked, or far: its keys are only lower bounds)
-    int row[KS], ra[KS], rb[KS];
-    constexpr int NO_ROW = RS_NO_ROW, ODD = -1, NONE = -2;   // (ODD, NONE: of the step before, see below)
+    // ---- the rows held by the lane, ascending, and their keys (see Held): marked when the row was pending when the lane last looked, or is
+    // far: its keys are only lower bounds
+    constexpr int NO_ROW = RS_NO_ROW, ABSENT = K::LIMIT * (1 << K::SLOT_BITS);
+    int list_row[LISTS ? KS : 1], ra[KS], rb[KS];
+    #pragma unroll
+    for (int k = 0; k < (LISTS ? KS : 1); ++k) list_row[k] = NO_ROW;
+    auto row = [&](int k) { return LISTS ? list_row[LISTS ? k : 0] : (k * 32 + lane < I ? k * 32 + lane : NO_ROW); };
+    auto tag = [&](int k) { return 64 * k + 2 * lane; };
+    unsigned int by_slot = RS_BY_SLOT;     // in the jobs told by slot
+    int base = 0, cut = 0;       // cut: the largest (odd) key that is not decided on, as the entries of the tables
     int jmax = 0;        // an arrival whose ramp is longer than this reaches the step of every row's b
+    auto take_base = [&](int b) {
+        base = b;
+        cut = (WHOLE ? K::CUT : min(K::CUT, RS_CUT - b)) * (1 << K::SLOT_BITS) - 1 - SLACK;
+    };
+    auto unread = [&]() {        // all rows present are marked, with keys that are below any
+        #pragma unroll
+        for (int k = 0; k < KS; ++k) { ra[k] = (row(k) != NO_ROW ? 1 : ABSENT) + tag(k); rb[k] = tag(k) - ABSENT + (row(k) != NO_ROW ? 1 : 0); }
+    };
     // The marked rows that are not pending any more.  The loads are no acquires: what this warp needs of a fold lies in shared memory
     // and is read after `pending`, in order.  That the next folding warp of the row sees the cells that the last one stored to
     // device memory follows from all of them running on one SM (one L1, and the last one's release comes before its `pending`), not
     // from a chain of acquires; a fence here would make it one, and costs 50 ns a look (64 instances, 1,024 arrivals: 199 -> 205 us;
     // as acquiring loads 212, with the fence merged into the release of the decisions 204).
     auto refresh = [&]() {
+        unsigned int pending[KS], state[KS];
+        int2 r[KS];
+        #pragma unroll
+        for (int k = 0; k < KS; ++k) pending[k] = ld_volatile(sh.pending + 32 * k + lane);    // first: it is cleared last
         #pragma unroll
         for (int k = 0; k < KS; ++k) {
-            if (ra[k] & 1) {
-                const bool pending = ld_volatile(rows.pending + row[k]) != 0;    // first: it is cleared last
-                const int2 r = ld_volatile2(rows.rec + row[k]);
-                const int far = (ld_volatile(rows.state + row[k]) & RS_FAR) ? 1 : 0;
-                if (!pending) { ra[k] = r.x - far; rb[k] = r.y - far; }
-            }
+            const int i = row(k) != NO_ROW ? row(k) : 0;
+            r[k] = ld_volatile2(rows.rec + i);
+            state[k] = ld_volatile(rows.state + i);
+        }
+        #pragma unroll
+        for (int k = 0; k < KS; ++k) {      // (selects: a branch per row took 130 cycles a row)
+            const bool read = (ra[k] & 1) != 0 && pending[k] == 0;
+            const int mark = tag(k) + ((state[k] & RS_FAR) ? 1 : 0), key_a = K::relative(r[k].x, base) + mark, key_b = K::relative(r[k].y, base) + mark;
+            ra[k] = read ? key_a : ra[k];
+            rb[k] = read ? key_b : rb[k];
         }
         jmax = (int)ld_volatile(&sh.jmax);    // (after the rows were read)
     };
@@ -1264,12 +1359,13 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         unsigned int m = 0;
         #pragma unroll
         for (int k = 0; k < KS; ++k)
-            if (row[k] != NO_ROW && ld_acquire(rows.pending + row[k])) m |= 1u << k;
+            if (row(k) != NO_ROW && ld_acquire(sh.pending + 32 * k + lane)) m |= 1u << k;
         return m;
     };
     auto all_folded = [&](unsigned int e) {   // every decision before e has reached its row
         return __all_sync(FULL_MASK, (int)(ld_acquire(&sh.done[lane_f]) - e) >= 0);
     };
+    const unsigned int at_pending = smem_u32(sh.pending), at_jobs = smem_u32(sh.jobs), at_items = smem_u32(sh.items);
     auto publish = [&](unsigned int n) {
         __syncwarp();
         if (lane == 0) st_release(&sh.ctl.x, n);
@@ -1289,118 +1385,161 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         table = smem_u32(sh.table[list & 1]);
         const int n = sh.list_n[list & 1];
         #pragma unroll
-        for (int k = 0; k < KS; ++k) row[k] = k * 32 + lane < n ? sh.list_row[list & 1][k * 32 + lane] : NO_ROW;
-        #pragma unroll
-        for (int i = 1; i < KS; ++i)
-            #pragma unroll
-            for (int k = KS - 1; k >= i; --k) {
-                const int x = min(row[k - 1], row[k]);
-                row[k] = max(row[k - 1], row[k]);
-                row[k - 1] = x;
-            }
-        #pragma unroll
-        for (int k = 0; k < KS; ++k) { ra[k] = row[k] != NO_ROW ? RS_ABSENT - 1 : RS_ABSENT; rb[k] = RS_LOWEST; }
+        for (int k = 0; k < KS; ++k) list_row[LISTS ? k : 0] = k * 32 + lane < n ? sh.list_row[list & 1][k * 32 + lane] : NO_ROW;
+        by_slot = RS_BY_SLOT | ((list & 1) << 16);
+        take_base(sh.list_base[list & 1]);
+        unread();
         if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return; }
         refresh();
         ask_for_list();     // (a list takes about as long as one lasts)
     };
+    // All rows held, none pending: a larger base, if there is one.
+    auto rebase = [&]() -> bool {
+        int least = 0x7fffffff;
+        #pragma unroll
+        for (int k = 0; k < KS; ++k)
+            if (row(k) != NO_ROW) {
+                const int2 r = ld_volatile2(rows.rec + row(k));
+                least = min(least, max(r.x, r.y));
+            }
+        least = __reduce_min_sync(FULL_MASK, least) & ~1;
+        if (least <= base) return false;
+        take_base(least);
+        unread();
+        refresh();
+        return true;
+    };
     if (LISTS) {
         next_list(0);
     } else {
-        #pragma unroll
-        for (int k = 0; k < KS; ++k) {
-            row[k] = k * 32 + lane < I ? k * 32 + lane : NO_ROW;
-            ra[k] = row[k] != NO_ROW ? RS_ABSENT - 1 : RS_ABSENT; rb[k] = RS_LOWEST;
-        }
+        take_base(unordered(sh.probe_t[0]) & ~1);
+        unread();
         refresh();
     }
-    auto bound_of = [&](int4 b, int kp) { return min(min(b.x, b.y + kp), max(b.z, b.w + kp)); };
-    // a decision told to the folding warps: job `w` (a row, and RS_GIVEN with a peak) for item e; NONE: nothing is told
-    const unsigned int at_pending = smem_u32(rows.pending), at_jobs = smem_u32(sh.jobs), at_items = smem_u32(sh.items), at_ctl = smem_u32(&sh.ctl);
-    auto tell = [&](unsigned int e, int row_of, int w, unsigned int peak) {
-        asm volatile("{ .reg .pred p; setp.eq.s32 p, %0, 0; setp.ne.and.s32 p, %1, -2, p; @p st.shared.u32 [%2], 1; @p st.shared.v2.u32 [%3], {%1, %4}; }"
-                     ::"r"(lane), "r"(w), "r"(at_pending + 4u * (unsigned int)row_of), "r"(at_jobs + 8u * (e % RS_ITEMS)), "r"(peak) : "memory");
+    // An entry of the bounds' table, for an arrival that adds kp: no row outside the list has a smaller key.
+    auto bound_of = [&](int4 b, int kp) { return min(__viaddmin_s32(b.y, kp, b.x), __viaddmax_s32(b.w, kp, b.z)); };
+    // Decisions told to the folding warps: those of `count` items from e on, lane u's row by the key that has won.
+    auto tell = [&](unsigned int e, int key, int count) {
+        asm volatile("{ .reg .pred p; setp.lt.s32 p, %0, %1; @p st.shared.u32 [%2], %3; @p st.shared.u32 [%4], 1; }"
+                     ::"r"(lane), "r"(count), "r"(at_jobs + 8u * ((e + lane) % RS_ITEMS)), "r"((unsigned int)(key & K::SLOT) | by_slot), "r"(at_pending + 2u * (unsigned int)(key & K::SLOT)) : "memory");
     };
-    auto release = [&](unsigned int n) {
-        asm volatile("{ .reg .pred p; setp.eq.s32 p, %0, 0; @p st.release.cta.shared.u32 [%1], %2; }" ::"r"(lane), "r"(at_ctl), "r"(n) : "memory");
+    auto tell_slot = [&](unsigned int e, int t, unsigned int given, unsigned int peak) {
+        __syncwarp();
+        if (lane == 0) { sh.pending[t >> 1] = 1; sh.jobs[e % RS_ITEMS] = make_uint2((unsigned int)t | by_slot | given, peak); }
+        __syncwarp();
     };
-    // Everything unusual about item e.
-    auto unusual = [&](unsigned int e) {
+    auto tell_row = [&](unsigned int e, int w, unsigned int given, unsigned int peak) {    // (a row that need not be held)
+        int t = -1;
+        #pragma unroll
+        for (int k = 0; k < KS; ++k)
+            if (row(k) == w) t = tag(k);
+        t = __reduce_max_sync(FULL_MASK, t);
+        if (t >= 0) tell_slot(e, t, given, peak);
+        else if (lane == 0) sh.jobs[e % RS_ITEMS] = make_uint2((unsigned int)w | given, peak);
+    };
+    // Everything unusual about item e.  False: not decided, but the keys are such that it may be usual now (or the batch is lost).
+    unsigned int tried_at = 0xffffffffu;      // the item for which `lists_tried` lists have been taken
+    int lists_tried = 0;
+    auto unusual = [&](unsigned int e) -> bool {
         const int4 it = sh.items[e % RS_ITEMS];
         const int2 pd = sh.raw[e % RS_ITEMS];
-        const int P = pd.x, D = pd.y, Dc = D < H ? D : H, kp = it.x, kpd = it.y;
-        const Look<FOLD_WARPS, ADMIT, WHOLE> look{a, sh, rows, sc, 0u};
+        const int P = pd.x, D = pd.y, Dc = D < H ? D : H, kp = sc.key_p(P), kpe = it.x;
+        const int kpde = K::scaled(min(sc.key_pd(P, D), K::ITEM));
+        const Look<FOLD_WARPS, ADMIT, WHOLE, LISTS> look{a, sh, rows, sc, 0u};
         publish(e);
-        auto received = [&](int win) {     // the arrival's ramp reaches the step of the row's b
+        auto received = [&](int t) {     // the arrival's ramp reaches the step of the row's b
             #pragma unroll
             for (int k = 0; k < KS; ++k)
-                if (row[k] == win) {
+                if (tag(k) == t) {
                     const int marked = ra[k] & 1;
-                    ra[k] += kpd + marked;
-                    rb[k] += kpd + (marked ? 1 : kp);
+                    ra[k] = (ra[k] + kpde) | 1;
+                    rb[k] = (rb[k] + kpde + (marked ? 0 : kpe)) | 1;
                 }
         };
-        for (int lists_tried = 0;;) {
-            refresh();
-            if (it.z <= jmax) break;
-            // the rows that can have the smallest score: those within the slack of the smallest value of a row that is not marked
-            int v[KS], least = RS_ABSENT;
+        if (tried_at != e) { tried_at = e; lists_tried = 0; }
+        refresh();
+        if (it.z > jmax) {
+            // The smallest key now, and (rows whose rounded keys may stand for the smallest score) what is within the slack of the smallest one of
+            // a row that is not marked.
+            int v[KS], least = ABSENT, key = 0x7fffffff;
             #pragma unroll
             for (int k = 0; k < KS; ++k) {
-                v[k] = max(ra[k], rb[k] + kp);
-                if (!(ra[k] & 1)) least = min(least, v[k]);
+                v[k] = max(ra[k], rb[k] + kpe);
+                key = min(key, v[k]);
+                least = (ra[k] & 1) ? least : min(least, v[k]);
             }
-            const int reach = __reduce_min_sync(FULL_MASK, least) + SLACK;
-            if (reach >= (WHOLE ? RS_ABSENT : RS_CUT)) {   // no row to measure by, or one whose keys are cut
-                const unsigned int before = held_pending();
-                if (__any_sync(FULL_MASK, before != 0)) {
-                    if (!rs_wait(sh, [&] { return __any_sync(FULL_MASK, held_pending() != before) != 0; })) { lost = true; return; }
-                    continue;
+            key = __reduce_min_sync(FULL_MASK, key);
+            const int beyond = LISTS ? min(cut, bound_of(ld_table(table + it.w), kpe)) : cut;
+            if (key > beyond) {    // a row outside the list could do as well, or the keys are cut
+                if (LISTS) {
+                    if (lists_tried < 2) {
+                        ++lists_tried;
+                        next_list(e);
+                        return false;
+                    }
+                } else {
+                    const unsigned int before = held_pending();
+                    if (__any_sync(FULL_MASK, before != 0)) {
+                        if (!rs_wait(sh, [&] { return __any_sync(FULL_MASK, held_pending() != before) != 0; })) { lost = true; return false; }
+                        return false;
+                    }
+                    if (rebase()) return false;
                 }
-                if (!LISTS) break;
-            }
-            if (LISTS && reach >= bound_of(ld_table(table + it.w), kp)) {   // a row outside the list could do as well
-                if (lists_tried == 2) break;
-                ++lists_tried;
-                next_list(e);
-                if (lost) return;
-                continue;
-            }
-            S mine = Scores<WHOLE>::none();
-            int mine_row = NO_ROW;
-            bool wait = false, scan = false;
-            #pragma unroll
-            for (int k = 0; k < KS; ++k) {
-                if (v[k] <= reach && row[k] != NO_ROW) {
-                    const int i = row[k];
-                    if (ld_volatile(rows.pending + i)) wait = true;
-                    else {
+            } else if (key & 1) {    // the best row is marked
+                const unsigned int* word = sh.pending + ((key & K::SLOT) >> 1);
+                if (ld_acquire(word)) {
+                    if (!rs_wait(sh, [&] { return ld_acquire(word) == 0; })) lost = true;
+                    return false;
+                }
+                if (!(__ballot_sync(FULL_MASK, [&] {      // (a far row; but it may just have been folded)
+                        bool far = false;
+                        #pragma unroll
+                        for (int k = 0; k < KS; ++k)
+                            if (tag(k) == (key & K::SLOT)) far = (ld_volatile(rows.state + row(k)) & RS_FAR) != 0;
+                        return far;
+                    }())))
+                    return false;
+            } else if (WHOLE) {
+                return false;
+            } else {
+                const int reach = (__reduce_min_sync(FULL_MASK, least) & ~K::TAGS) + SLACK;
+                S mine = Scores<WHOLE>::none();
+                int mine_tag = NO_ROW;
+                bool scan = false;
+                unsigned int open = 0;
+                #pragma unroll
+                for (int k = 0; k < KS; ++k)
+                    if ((v[k] & ~K::TAGS) <= reach && row(k) != NO_ROW && ld_acquire(sh.pending + 32 * k + lane)) open |= 1u << k;
+                if (__any_sync(FULL_MASK, open != 0)) {
+                    if (!rs_wait(sh, [&] {
+                            bool some = false;
+                            #pragma unroll
+                            for (int k = 0; k < KS; ++k)
+                                if ((open >> k) & 1) some |= ld_acquire(sh.pending + 32 * k + lane) != 0;
+                            return !some;
+                        })) lost = true;
+                    return false;
+                }
+                #pragma unroll
+                for (int k = 0; k < KS; ++k)
+                    if ((v[k] & ~K::TAGS) <= reach && row(k) != NO_ROW) {
+                        const int i = row(k);
                         const unsigned int top = ld_volatile(rows.top + i), jt = ld_volatile(rows.state + i) & RS_JTOP;
-                        const unsigned int tokens = WHOLE ? (unsigned int)ld_volatile2(rows.rec + i).x >> 1 : ld_volatile(rows.tok + i);
                         if (Dc > (int)jt || sc.no_penalty(top, P)) {
-                            const S s = sc.of_peak(tokens, top + (unsigned int)P, P, D);
-                            if (s < mine || (s == mine && i < mine_row)) { mine = s; mine_row = i; }
+                            const S s = sc.of_peak(sc.tokens_of(rows, i), top + (unsigned int)P, P, D);
+                            if (s < mine || (s == mine && tag(k) < mine_tag)) { mine = s; mine_tag = tag(k); }
                         } else scan = true;
+                    }
+                if (!__any_sync(FULL_MASK, scan)) {
+                    const S best = Scores<WHOLE>::warp_min(mine);
+                    const int win = __reduce_min_sync(FULL_MASK, mine == best ? mine_tag : NO_ROW);
+                    if (win != NO_ROW) {
+                        received(win);
+                        tell_slot(e, win, 0u, 0u);
+                        return true;
                     }
                 }
             }
-            if (__any_sync(FULL_MASK, wait)) {
-                if (!rs_wait(sh, [&] {
-                        bool open = false;
-                        #pragma unroll
-                        for (int k = 0; k < KS; ++k)
-                            if (v[k] <= reach && row[k] != NO_ROW) open |= ld_acquire(rows.pending + row[k]) != 0;
-                        return !open;
-                    })) { lost = true; return; }
-                continue;
-            }
-            if (__any_sync(FULL_MASK, scan)) break;
-            const S best = Scores<WHOLE>::warp_min(mine);
-            const int win = __reduce_min_sync(FULL_MASK, mine == best ? mine_row : NO_ROW);
-            if (win >= I) break;
-            received(win);
-            tell(e, win, win, 0u);
-            return;
         }
         auto folding_warps_look = [&](int how) {
             ++looks;
@@ -1409,38 +1548,47 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             if (lane == 0) st_release(&sh.ctl.y, looks);
             if (!rs_wait(sh, [&] { return ld_acquire(&sh.looks_done[lane_f]) == looks; })) lost = true;
         };
-        // A held row takes the arrival without its ramp being known to reach the step of the row's b.
+        // A held row takes the arrival without its ramp being known to reach the step of the row's b, or that fitting into the keys.
         auto received_some = [&](int win) {
             #pragma unroll
             for (int k = 0; k < KS; ++k)
-                if (row[k] == win) { ra[k] = (ra[k] + kpd) | 1; rb[k] = (rb[k] + kpd) | 1; }
+                if (row(k) == win) { ra[k] = (ra[k] + kpde) | 1; rb[k] = (rb[k] + kpde) | 1; }
         };
-        if (!LISTS) {
+        auto received_row = [&](int win) {
+            if (it.z == 0) { received_some(win); return; }
+            #pragma unroll
+            for (int k = 0; k < KS; ++k)
+                if (row(k) == win) received(tag(k));
+        };
+        if (!LISTS && it.z != 0) {
             // ---- short arrivals and rows that are only bounded, among all rows: nothing is waited for but what can be the best
-            while (WHOLE || kp < RS_CUT) {
+            for (;;) {
                 // The rows that can have the smallest score: those whose least value (a held row's keys grow with what it has received,
                 // the drop in its state is that of its last fold or a later one) is within the slack of the smallest one that a row
                 // has at most.
-                int v[KS], least = RS_ABSENT;
+                int v[KS], least = ABSENT;
                 #pragma unroll
                 for (int k = 0; k < KS; ++k) {
-                    int exact, most = max(ra[k], rb[k] + kp);
-                    const int add = sc.key_least(row[k] != NO_ROW ? ld_volatile(rows.state + row[k]) : 0u, kp, Dc, exact);
+                    int exact, most = max(ra[k], rb[k] + kpe);
+                    const int add = sc.key_least(row(k) != NO_ROW ? ld_volatile(rows.state + row(k)) : 0u, kp, Dc, exact);
                     if (ra[k] & 1) {
-                        most = RS_ABSENT;
-                        if (!ld_acquire(rows.pending + row[k])) {
-                            const unsigned int tokens = sc.tokens_of(rows, row[k]);
-                            most = max(sc.key_a(tokens), sc.key_b(tokens, rows.top[row[k]]) + kp);
+                        most = ABSENT;
+                        if (!ld_acquire(sh.pending + 32 * k + lane)) {
+                            const unsigned int tokens = sc.tokens_of(rows, row(k));
+                            most = K::relative(max(sc.key_a(tokens), sc.key_b(tokens, rows.top[row(k)]) + kp), base);
                         }
                     }
-                    v[k] = max(ra[k], rb[k] + add);
-                    least = min(least, most);
+                    v[k] = max(ra[k], rb[k] + K::scaled(max(add, -K::LIMIT / 2))) & ~K::TAGS;
+                    least = min(least, most & ~K::TAGS);
                 }
                 const int reach = __reduce_min_sync(FULL_MASK, least) + SLACK;
-                if (reach >= (WHOLE ? RS_ABSENT : RS_CUT)) {   // no row to measure by, or one whose keys are cut
+                if (reach > cut) {   // no row to measure by, or one whose keys are cut
                     const unsigned int before = held_pending();
-                    if (!__any_sync(FULL_MASK, before != 0)) break;
-                    if (!rs_wait(sh, [&] { return __any_sync(FULL_MASK, held_pending() != before) != 0; })) { lost = true; return; }
+                    if (!__any_sync(FULL_MASK, before != 0)) {
+                        if (rebase()) continue;
+                        break;
+                    }
+                    if (!rs_wait(sh, [&] { return __any_sync(FULL_MASK, held_pending() != before) != 0; })) { lost = true; return false; }
                     refresh();
                     continue;
                 }
@@ -1450,9 +1598,9 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 bool wait = false;
                 #pragma unroll
                 for (int k = 0; k < KS; ++k) {
-                    if (v[k] <= reach && row[k] != NO_ROW) {
-                        const int i = row[k];
-                        if (ld_acquire(rows.pending + i)) wait = true;
+                    if (v[k] <= reach && row(k) != NO_ROW) {
+                        const int i = row(k);
+                        if (ld_acquire(sh.pending + 32 * k + lane)) wait = true;
                         else {
                             const unsigned int top = rows.top[i], jt = rows.state[i] & RS_JTOP;
                             if (Dc > (int)jt) reached |= 1u << k;
@@ -1468,9 +1616,9 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                             bool pending = false;
                             #pragma unroll
                             for (int k = 0; k < KS; ++k)
-                                if (v[k] <= reach && row[k] != NO_ROW) pending |= ld_acquire(rows.pending + row[k]) != 0;
+                                if (v[k] <= reach && row(k) != NO_ROW) pending |= ld_acquire(sh.pending + 32 * k + lane) != 0;
                             return !pending;
-                        })) { lost = true; return; }
+                        })) { lost = true; return false; }
                     refresh();
                     continue;
                 }
@@ -1481,7 +1629,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 if (__any_sync(FULL_MASK, open != 0)) {    // bounded rows that could be better are scanned
                     #pragma unroll 1
                     for (int k = 0; k < KS; ++k) {
-                        const int i = k * 32 + lane;       // (all rows are held: row[k])
+                        const int i = k * 32 + lane;       // (all rows are held)
                         bool todo = ((open >> k) & 1) != 0;
                         unsigned int tokens = 0;
                         if (todo) {
@@ -1495,7 +1643,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                         if (todo) sh.scan_row[slot] = i;
                         if (lane == 0) sh.scan_n = __popc(which);
                         folding_warps_look(RS_SCANS);
-                        if (lost) return;
+                        if (lost) return false;
                         const unsigned int p = todo ? sh.scan_peak[slot] : 0u;
                         const S s = todo ? sc.of_peak(tokens, p, P, D) : Scores<WHOLE>::none();
                         const S smallest = Scores<WHOLE>::warp_min(s);
@@ -1508,45 +1656,56 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                     }
                 }
                 if (win >= I) break;
-                if (!scanned && __any_sync(FULL_MASK, mine_row == win && ((reached >> (win >> 5)) & 1))) received(win);
+                if (!scanned && __any_sync(FULL_MASK, mine_row == win && ((reached >> (win >> 5)) & 1))) received(2 * win);
                 else received_some(win);
-                tell(e, win, scanned ? win | (int)RS_GIVEN : win, peak);
-                return;
+                tell_slot(e, 2 * win, scanned ? RS_GIVEN : 0u, peak);
+                return true;
             }
         }
         // ---- rows outside the list could do as well, or keys are cut: all rows, with every fold done
-        if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return; }
+        if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return false; }
         acquire_cta();
         if (LISTS) {
             int4 k;
             if (I <= RS_OWN_LOOK) k = look.template keys<32, 8>(0, P, D);
             else {
                 folding_warps_look(RS_KEYS);
-                if (lost) return;
+                if (lost) return false;
                 k = look.all_keys();
             }
             if (look.decide(k, kp, P, Dc)) {
-                if (Dc > (int)(rows.state[k.y] & RS_JTOP)) received(k.y);
+                if (Dc > (int)(rows.state[k.y] & RS_JTOP)) received_row(k.y);
                 else received_some(k.y);      // (it pays no penalty)
-                tell(e, k.y, k.y, 0u);
-                return;
+                tell_row(e, k.y, 0u, 0u);
+                return true;
             }
         }
         folding_warps_look(RS_CLOSELY);
-        if (lost) return;
+        if (lost) return false;
         S best;
         int win;
         unsigned int win_peak;
         look.smallest(1, best, win, win_peak);
-        #pragma unroll
-        for (int k = 0; k < KS; ++k)
-            if (row[k] == win) {      // (a lower bound, odd)
-                ra[k] = (min(ra[k] + kpd + 1, RS_CUT) - 1) | 1;
-                rb[k] = (min(rb[k] + kpd + 1, RS_CUT) - 1) | 1;
-            }
-        tell(e, win, win | (int)RS_GIVEN, win_peak);
+        received_some(win);
+        tell_row(e, win, RS_GIVEN, win_peak);
+        return true;
     };
 
+    // ---- the usual way
+    int4 it0, it1, it2, ahead = make_int4(0, 0, 0, 0);     // items e, e + 1, e + 2, the bounds for item e + 1
+    int bound;                                             // for item e: the key that a row outside the list (or a case that is unusual) has at least
+    auto bound_for = [&](const int4& it, const int4& others) {
+        const int b = it.z > jmax ? cut : (int)0x80000001u;
+        return LISTS ? min(b, bound_of(others, it.x)) : b;
+    };
+    auto fetch = [&](unsigned int e) {
+        it0 = ld_table(at_items + 16u * (e % RS_ITEMS));
+        it1 = ld_table(at_items + 16u * ((e + 1) % RS_ITEMS));
+        it2 = ld_table(at_items + 16u * ((e + 2) % RS_ITEMS));
+        int4 now = ahead;
+        if (LISTS) { now = ld_table(table + it0.w); ahead = ld_table(table + it1.w); }
+        bound = bound_for(it0, now);
+    };
     unsigned int e = 0, ready = 0;   // decisions made, items known to be there
     while (!lost) {     // (every way out has published what was decided)
         if (e >= ready) {
@@ -1559,7 +1718,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 break;
             if (ready <= e) break;
         }
-        unsigned int stop = min(ready, e + CHUNK);
+        unsigned int limit = ready;
         if (ADMIT) {
             // Every instance overloaded?  Each decision not folded yet may have taken one more over the level; while fewer of
             // those are under way than rows are known not to be overloaded, the request is routed.
@@ -1575,91 +1734,83 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 if (lane == 0) { sh.blocked = 1; sh.blocked_k = sh.item_at[e % RS_ITEMS]; }
                 break;
             }
-            stop = min(stop, e + (unsigned int)spare);
+            limit = min(limit, e + (unsigned int)spare);
         }
+        const unsigned int stop = min(limit, e + CHUNK);
         refresh();
-        // The usual way.  What was decided at one step is checked and told at the next, while the reduction over its scores is
-        // under way: the branch and the stores would else be waited for (measured in this loop alone, four rows per lane:
-        // 232 cycles with them in the step, 158 with them a step later, four steps per trip and the keys marked in their last bit).
-        int4 it = sh.items[e % RS_ITEMS];
-        int4 others = make_int4(0, 0, 0, 0);
-        if (LISTS) others = ld_table(table + it.w);
-        int w = NONE;        // the decision of the step before; ODD: that was not the usual case
-        auto scores = [&](int kp, int (&v)[KS]) {    // of the rows held; returns the lane's smallest
+        fetch(e);
+        while (e < stop) {
+            int was_a[KS], was_b[KS], key[TRIP], not_usual = 0;
+            const unsigned int at = at_items + 16u * (e % RS_ITEMS);
             #pragma unroll
-            for (int k = 0; k < KS; ++k) v[k] = __viaddmax_s32(rb[k], kp, ra[k]);
-            int least = v[0];
+            for (int k = 0; k < KS; ++k) { was_a[k] = ra[k]; was_b[k] = rb[k]; }
             #pragma unroll
-            for (int k = 1; k + 1 < KS; k += 2) least = __vimin3_s32(least, v[k], v[k + 1]);
-            return KS % 2 ? least : min(least, v[KS - 1]);
-        };
-        // u: e modulo 4 where that is known.  False: the step before was not the usual case, nothing has been done.
-        auto step = [&](unsigned int e, unsigned int trip, int u, bool publishes) -> bool {
-            const int kp = it.x, kpd = it.y, kpb = kpd + kp;
-            int v[KS];
-            const int best = __reduce_min_sync(FULL_MASK, scores(kp, v));
-            if (w == ODD) return false;
-            tell(u > 0 ? trip + u - 1 : e - 1, w, w, 0u);
-            if (publishes) release(e);
-            int bound = it.z > jmax ? (WHOLE ? RS_ABSENT : RS_CUT) : RS_LOWEST;
-            if (LISTS) bound = __vimin3_s32(bound, __viaddmin_s32(others.y, kp, others.x), __viaddmax_s32(others.w, kp, others.z));
-            it = ld_table(at_items + 16u * (u >= 0 && u < 3 ? (trip + u + 1) : (e + 1) % RS_ITEMS));      // (beyond the items that are there: not used)
-            int mine = NO_ROW;
-            if (WHOLE) {
+            for (int u = 0; u < TRIP; ++u) {     // (items from `limit` on are whatever the slots hold: what is done with them is taken back)
+                const int kp = it0.x, kpd = it0.y, kpb = kpd + kp;
+                int v[KS];
                 #pragma unroll
-                for (int k = KS - 1; k >= 0; --k) mine = v[k] == best ? row[k] : mine;
-            } else {     // more than one row that can be the best: not the usual case
-                int many = 0;
+                for (int k = 0; k < KS; ++k) v[k] = __viaddmax_s32(rb[k], kp, ra[k]);
+                int least = bound;
                 #pragma unroll
-                for (int k = KS - 1; k >= 0; --k)
-                    if (v[k] <= best + SLACK) { mine = row[k]; ++many; }
-                if (many > 1) mine = ODD;
-            }
-            if (best + SLACK >= bound || (best & 1)) mine = ODD;
-            w = __reduce_min_sync(FULL_MASK, mine);
-            if (!WHOLE) {
-                const int last = __reduce_max_sync(FULL_MASK, mine == NO_ROW ? ODD : mine);
-                if (last != w) w = ODD;
-            }
-            if (LISTS) others = ld_table(table + it.w);
-            #pragma unroll
-            for (int k = 0; k < KS; ++k)
-                if (row[k] == w) { ra[k] += kpd; rb[k] += kpb; }
-            return true;
-        };
-        // (everything unusual in one place, away from the loop: inlined in it the way around it cost 15 cycles a step)
-        for (;;) {
-            bool usual = true;
-            while (e < stop) {
-                if ((e & 3u) == 0 && e + 4 <= stop) {
-                    const unsigned int trip = e % RS_ITEMS;
-                    usual = step(e, trip, 0, true);
-                    if (!usual) break;
-                    ++e;
-                    usual = step(e, trip, 1, PUBLISH == 1);
-                    if (!usual) break;
-                    ++e;
-                    usual = step(e, trip, 2, PUBLISH <= 2);
-                    if (!usual) break;
-                    ++e;
-                    usual = step(e, trip, 3, PUBLISH == 1);
-                    if (!usual) break;
-                    ++e;
-                } else {
-                    usual = step(e, 0u, -1, true);
-                    if (!usual) break;
-                    ++e;
+                for (int k = 0; k + 1 < KS; k += 2) least = __vimin3_s32(least, v[k], v[k + 1]);
+                if (KS == 1) least = min(least, v[0]);
+                const int best = __reduce_min_sync(FULL_MASK, least);
+                // (while the reduction is under way)
+                it0 = it1; it1 = it2;
+                it2 = ld_table(at + 16u * (u + 3));
+                bound = bound_for(it0, ahead);
+                if (LISTS) ahead = ld_table(table + it1.w);
+                #pragma unroll
+                for (int k = 0; k < KS; ++k)
+                    if (v[k] == best) { ra[k] += kpd; rb[k] += kpb; }
+                key[u] = best;
+                not_usual |= best & 1;
+                if (!WHOLE) {     // another row that can be the best
+                    int next = 0x7fffffff;
+                    #pragma unroll
+                    for (int k = 0; k < KS; ++k) next = min(next, v[k] == best ? 0x7fffffff : v[k]);
+                    next = __reduce_min_sync(FULL_MASK, next);
+                    if (next <= (best | K::TAGS) + SLACK) not_usual |= 2 << u;
                 }
             }
-            if (usual && w != ODD) break;
-            unusual(e - 1);
-            w = NONE;
-            if (lost || e >= stop) break;
-            if (LISTS) others = ld_table(table + it.w);
+            int told = key[0];
+            #pragma unroll
+            for (int u = 1; u < TRIP; ++u) told = lane == u ? key[u] : told;
+            if (not_usual == 0 && e + TRIP <= limit) {
+                tell(e, told, TRIP);
+                e += TRIP;
+                publish(e);
+                continue;
+            }
+            // ---- the first `usual` steps of the trip stand, the others are taken back
+            const int there = (int)min(limit - e, (unsigned int)TRIP);
+            int usual = there;
+            #pragma unroll
+            for (int u = TRIP - 1; u >= 0; --u)
+                if (u < there && ((key[u] & 1) || (not_usual & (2 << u)))) usual = u;
+            #pragma unroll
+            for (int k = 0; k < KS; ++k) { ra[k] = was_a[k]; rb[k] = was_b[k]; }
+            #pragma unroll
+            for (int u = 0; u + 1 < TRIP; ++u) {
+                const int4 it = ld_table(at + 16u * u);
+                const int t = u < usual ? key[u] & K::SLOT : -1;
+                #pragma unroll
+                for (int k = 0; k < KS; ++k) {
+                    ra[k] += tag(k) == t ? it.y : 0;
+                    rb[k] += tag(k) == t ? it.y + it.x : 0;
+                }
+            }
+            tell(e, told, usual);
+            e += usual;
+            if (usual < there) {
+                if (unusual(e)) { ++e; publish(e); }
+                else if (lost) break;
+                else refresh();
+            } else {
+                publish(e);
+            }
+            fetch(e);
         }
-        tell(e - 1, w, w, 0u);
-        if (lost) break;
-        publish(e);
     }
     __syncwarp();
     if (lane == 0) st_release(&sh.ctl.z, 1u);
@@ -1751,21 +1902,22 @@ __device__ __noinline__ void rs_literal(const RouteSumArgs& a, RsShared& sh, lon
 }
 
 // After a wait that was abandoned: the results of the decisions that were told and that the io warp has not written.  A row has
-// at most one decision that is not folded, and as long as it is pending its numbers are those that the decision was made with.
+// at most one decision that is not folded, and as long as it is not its numbers are those that the decision was made with.
 // The maps need nothing: they receive the ramps of every table row that is not marked as applied.  Returns the first item that
 // was not decided (the ones from there on that are malformed or find the table full have their results already, the same
 // as those that were not reached).  (`rows` and `sc` by value: by reference they would live on the stack of every thread.)
-template <bool ADMIT, bool WHOLE>
+template <int FOLD_WARPS, bool LISTS, bool ADMIT, bool WHOLE>
 __device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const Rows rows, const Scores<WHOLE> sc, int waiting) {
     const unsigned int told = sh.ctl.x;
     for (unsigned int e = sh.written + threadIdx.x; e < told; e += blockDim.x) {
         const uint2 job = sh.jobs[e % RS_ITEMS];
         const int2 pd = sh.raw[e % RS_ITEMS];
-        const int w = (int)(job.x & ~RS_GIVEN), k = sh.item_at[e % RS_ITEMS];
+        const int w = job_row<LISTS>(sh, job.x), k = sh.item_at[e % RS_ITEMS];
         const long long at = sh.n0 + e;
-        double s = sh.score[e % RS_ITEMS];
-        if (rows.pending[w])
-            s = summary_score(sc.tokens_of(rows, w), (job.x & RS_GIVEN) ? job.y : rows.top[w] + (unsigned int)pd.x, (double)pd.x + (double)pd.y, a.theta, a.beta);
+        uint2 of = sh.scored[e % RS_ITEMS];
+        if ((int)(sh.done[e % FOLD_WARPS] - e) <= 0)      // (not folded)
+            of = make_uint2(sc.tokens_of(rows, w), (job.x & RS_GIVEN) ? job.y : rows.top[w] + (unsigned int)pd.x);
+        const double s = summary_score(of.x, of.y, (double)pd.x + (double)pd.y, a.theta, a.beta);
         a.prompt[at] = pd.x; a.generated[at] = 0; a.predicted[at] = pd.y; a.instance[at] = w;
         if (ADMIT && k < waiting) a.queue_choice[k] = w;
         else {
@@ -1780,7 +1932,7 @@ __device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const
 
 // Folding and list warps, warps and threads of the instantiations.
 template <bool LISTS, bool ADMIT> struct Shape {
-    static constexpr int FOLD = LISTS ? 6 : 5, LIST = LISTS ? 8 : 0;
+    static constexpr int FOLD = 8, LIST = LISTS ? RS_LIST_WARPS : 0;
     static constexpr int WARPS = 4 * ((FOLD + 1 + LIST + 2) / 3), THREADS = 32 * WARPS;
 };
 
@@ -1795,8 +1947,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     rows.rec = reinterpret_cast<int2*>(rs_smem);
     rows.state = reinterpret_cast<unsigned int*>(rows.rec + I);
     rows.top = rows.state + I;
-    rows.pending = rows.top + I;
-    rows.tok = rows.pending + I;     // (binary64 scores only)
+    rows.tok = rows.top + I;     // (binary64 scores only)
 
     // (the warp's number by a shuffle: the compiler then knows that the roles part between warps and not within one, and
     // leaves out what would bring the lanes of a warp together again: 157 instead of 202 cycles for a step of the deciding warp)
@@ -1812,7 +1963,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
                 rows.rec[i] = make_int2((int)q.x, (int)q.w);
                 rows.top[i] = q.y;
                 rows.state[i] = q.z;
-                rows.pending[i] = (unsigned int)above;
+                sh.pending[i] = (unsigned int)above;
             });
         batch_totals(a, tid, THREADS, sh_guard);
         __syncthreads();
@@ -1837,14 +1988,17 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         sh.n0 = *a.n_requests;
         sh.ctl = make_uint4(0u, 0u, 0u, 0u);
         sh.items_ready = sh.items_end = sh.not_over = sh.jmax = sh.n_far = sh.n_least = sh.written = sh.flush = 0;
-        sh.lists_wanted = sh.lists_ready = sh.list_met = sh.look_met = 0;
+        sh.lists_wanted = sh.lists_ready = sh.look_met = 0;
         sh.list_n[0] = sh.list_n[1] = 0;
         sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0;
         sh.first_bad = sh.first_full = 0x7fffffff;
     }
-    for (int i = tid; i < RS_ITEMS; i += THREADS) sh.items[i] = make_int4(0, 0, 0, 0);    // (an item is fetched before it is known to be there)
+    for (int i = tid; i < RS_ITEMS + RS_AHEAD; i += THREADS) sh.items[i] = make_int4(0, 0, 0, 0);    // (an item is fetched before it is known to be there)
     if (tid < RS_MAX_FOLD_WARPS) { sh.done[tid] = (unsigned int)tid; sh.looks_done[tid] = 0; }
     if (tid < RS_PROBES) sh.probe_t[tid] = 0xffffffffu;
+    if (tid < 32) { sh.bucket_a[tid] = 0xffffffffu; sh.bucket_b[tid] = 0xffffffffu; }
+    if (!alone)
+        for (int i = tid; i < RS_LIST_ROWS; i += THREADS) sh.pending[i] = 0;
     // ADMIT: the requests that were waiting when the call was made come first, then the arrivals
     long long q_head = 0, q_len = 0;
     if (ADMIT && a.queue_capacity > 0) {
@@ -1875,20 +2029,20 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     const unsigned long long mean_l = ramps / (unsigned long long)(n_items > 0 ? n_items : 1);
     const int mean = mean_l < (1ull << 22) ? (int)mean_l : 1 << 22;     // prompt + ramp of a typical request
     Scores<WHOLE> sc;
-    sc.start(a.theta, a.beta, peak_bound, max_pd, max_p, (base_sum + tokens_in) / (unsigned long long)I, mean);
+    sc.start(a.theta, a.beta, peak_bound, max_pd, max_p, (base_sum + tokens_in) / (unsigned long long)I, mean, Held<KS>::ITEM);
     {
         unsigned int jmax = 0, n_far = 0;
         int free_rows = 0;
-        int least[LISTS ? RS_PROBES : 1];      // the smallest value per probe, for the first list
-        if (LISTS)
-            #pragma unroll
-            for (int p = 0; p < RS_PROBES; ++p) least[LISTS ? p : 0] = 0x7f000000;
+        constexpr int PROBES = LISTS ? RS_PROBES : 1;      // (the first one: an empty prompt)
+        int least[PROBES];                     // the smallest value per probe, for the first list
+        #pragma unroll
+        for (int p = 0; p < PROBES; ++p) least[p] = 0x7f000000;
         for (int i = tid; i < I; i += THREADS) {
             uint4 q;
             int above = 0;
             if (alone) {
                 q = make_uint4((unsigned int)rows.rec[i].x, rows.top[i], rows.state[i], (unsigned int)rows.rec[i].y);
-                above = (int)rows.pending[i];
+                above = (int)sh.pending[i];
             } else {
                 q = a.summary0[i];
                 if (ADMIT) above = a.over0[i];
@@ -1903,12 +2057,11 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
             rows.rec[i] = rec;
             rows.state[i] = jtop | (drop << RS_DROP) | (far ? RS_FAR : 0u) | (pays && jtop >= (unsigned int)RS_NEAR ? RS_FULL : 0u) | (not_over ? RS_NOT_OVER : 0u);
             rows.top[i] = q.y;
-            rows.pending[i] = 0;
+            if (alone) sh.pending[i] = 0;
             if (!WHOLE) rows.tok[i] = q.x;
             a.newest[i] = RS_NOBODY;
-            if (LISTS)
-                #pragma unroll
-                for (int p = 0; p < RS_PROBES; ++p) least[LISTS ? p : 0] = min(least[LISTS ? p : 0], max(rec.x, rec.y + sc.key_p(rs_probe(mean, p))));
+            #pragma unroll
+            for (int p = 0; p < PROBES; ++p) least[p] = min(least[p], max(rec.x, rec.y + sc.key_p(rs_probe(mean, p))));
         }
         jmax = __reduce_max_sync(FULL_MASK, jmax);
         if (lane == 0 && jmax) atomicMax(&sh.jmax, jmax);
@@ -1916,12 +2069,11 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
             n_far = __reduce_add_sync(FULL_MASK, n_far);
             if (lane == 0 && n_far) atomicAdd(&sh.n_far, n_far);
         }
-        if (LISTS)
-            #pragma unroll
-            for (int p = 0; p < RS_PROBES; ++p) {
-                const int v = __reduce_min_sync(FULL_MASK, least[LISTS ? p : 0]);
-                if (lane == 0) atomicMin(&sh.probe_t[p], ordered(v));
-            }
+        #pragma unroll
+        for (int p = 0; p < PROBES; ++p) {
+            const int v = __reduce_min_sync(FULL_MASK, least[p]);
+            if (lane == 0) atomicMin(&sh.probe_t[p], ordered(v));
+        }
         if (ADMIT) {
             free_rows = __reduce_add_sync(FULL_MASK, free_rows);
             if (lane == 0 && free_rows) atomicAdd(&sh.not_over, (unsigned int)free_rows);
@@ -1944,13 +2096,13 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     } else if ((warp & 3) != 0) {
         if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, WHOLE, LISTS>(a, sh, rows, sc, role);
         else if (role == Sp::FOLD)
-            rs_io_loop<Sp::FOLD, ADMIT, WHOLE>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
+            rs_io_loop<KS, Sp::FOLD, ADMIT, WHOLE>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
         else if (LISTS && role <= Sp::FOLD + Sp::LIST)
-            rs_list_loop<LISTS ? Sp::LIST : 8, 32 * KS, WHOLE>(sh, rows, sc, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
+            rs_list_loop<LISTS ? Sp::LIST : 8, KS, WHOLE>(sh, rows, sc, a.near, a.far, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
     }
     __syncthreads();
     if (sh.ctl.w) {     // (all threads alike: nobody writes it any more)
-        decided = rs_settle<ADMIT, WHOLE>(a, sh, rows, sc, (int)q_len);
+        decided = rs_settle<Sp::FOLD, LISTS, ADMIT, WHOLE>(a, sh, rows, sc, (int)q_len);
         __syncthreads();
     }
     }
@@ -2073,7 +2225,7 @@ static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* s
     cudaFuncAttributes attr;
     cudaError_t e = cudaFuncGetAttributes(&attr, fn);
     if (e != cudaSuccess) return e;
-    const size_t smem = (size_t)I * (sizeof(int2) + (summaries_whole_numbers(ctx) ? 3 : 4) * sizeof(unsigned int));
+    const size_t smem = (size_t)I * (sizeof(int2) + (summaries_whole_numbers(ctx) ? 2 : 3) * sizeof(unsigned int));
     if (smem + attr.sharedSizeBytes + 256 > limit) return cudaSuccess;   // too many instances
     // (the limit is shared by every context of the process: always the device maximum)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(limit - attr.sharedSizeBytes));
