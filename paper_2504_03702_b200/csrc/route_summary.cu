@@ -51,19 +51,22 @@
 
 namespace {
 
-constexpr int RS_MAX_FOLD_WARPS = 8;
+constexpr int RS_MAX_FOLD_WARPS = 10;
 constexpr int RS_LIST_WARPS = 6;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
 constexpr int RS_AHEAD = 8;                 // items that are fetched beyond the present one, at most
 constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
 constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lane, 8 beyond RS_LONG_LISTS instances)
-constexpr int RS_LONG_LISTS = 2048;
+constexpr int RS_LONG_LISTS = 1024;
 constexpr int RS_NEAR_ROWS = 2304;          // rows the list warps keep for a closer look at once
 constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding warp looks at their keys by itself
 // Beyond RS_DIRECT_ROWS instances two kinds of batches cost this kernel more than the scanning one (which takes 2.4 us an arrival on 1,024 x
 // 1,024 whatever the rows): many far rows that may pay a penalty, whose arrivals need a look at all rows, scans, and folds of
 // whole rows (share of such rows, us: 28 % 2.0, 51 % 4.4, 58 % 5.4; with 512 x 40, 55 %, 1.3 against 2.3); and more rows that
 // share the smallest score than a list holds (empty services; 512 rows 2.7, 4,096 rows 42 against 3.1).
+// And keys in units of more than so many tokens (beta of thousands): 1,024 x 1,024, beta 1,000.5 (16 tokens) 1.5 us an arrival, 100,000.5
+// (2,048 tokens) 9.5, the scanning kernel 2.5.
+constexpr int RS_COARSE_SHIFT = -6;
 constexpr int RS_FAR_SHARE = 3, RS_FAR_STEPS = 256;     // one row in so many, maps of more steps than that
 constexpr int RS_PROBES = 8;                // prompt lengths for which a list has the best rows
 constexpr int RS_NEAR = 64;                 // steps kept exactly; the rest in 32 stretches of whole chunks of as many steps
@@ -536,25 +539,48 @@ template <int KS> struct Held {
     static __device__ __forceinline__ int scaled(int key) { return key * (1 << SLOT_BITS); }
     static __device__ __forceinline__ int relative(int key, int base) { return scaled(min(max(key - base, -LIMIT), LIMIT)); }
 };
+//   RS_HALVES (beta = m / 2^k, m at most 3, k at most 2, and m * theta with a fraction that is neither nearly none nor nearly one): keys in
+//   units of 2^-(k+1) tokens, which decide as the binary64 scores do.  2^k times the score of a row that pays is n + f, of one that does
+//   not 2^k * n, n whole numbers and f = ceil(m * theta) - m * theta for all rows alike, so 2 n + 1 and 2 * 2^k * n have the
+//   order of the scores.  The binary64 scores have it, too: peak - theta is a multiple of theta's last place, and beta times it is exact
+//   while peak - theta is below 1 / m of the power of two above theta (rows whose peak could be larger are taken as far); the token
+//   counts are exact; so a score is the real number rounded once: equal sums stay equal, and the last place of the largest ones, 2^-20,
+//   is less than f / 2^k or (1 - f) / 2^k.
+//   (With rounded keys one arrival in ten had to be compared outside the loop, and its steps had a second reduction: 2,000 x 1,536 in blocks
+//   of 16 tokens, 8,192 arrivals: 1,902 -> 1,200 us.)
+constexpr int RS_ROUNDED = 0, RS_WHOLE = 1, RS_HALVES = 2;
 constexpr int RS_LEAST_SHIFT = -20;
 constexpr int RS_CUT = 1 << 29, RS_ABSENT = 0x60000000, RS_LOWEST = -(1 << 30), RS_TOP_KEY = 0x3ffffffe;
-template <bool WHOLE> struct Scores {
-    static constexpr int SLACK = WHOLE ? 0 : 8;
+template <int KIND> struct Scores {
+    static constexpr bool WHOLE = KIND == RS_WHOLE, HALVES = KIND == RS_HALVES, EXACT = WHOLE || HALVES;
+    static constexpr int SLACK = EXACT ? 0 : 8;
     double theta, beta, unit;
+    long long theta_c;
     int theta_i, beta_i, shift, code_base;
     int slope;           // what a token less at the peak takes from b at most (0: too much)
+    unsigned int far_top;        // (RS_HALVES) a row whose top is not below is far
     unsigned int free_below;     // a row whose top is below pays no penalty, whatever arrival of the batch it gets
     __device__ __forceinline__ void start(double theta_d, double beta_d, unsigned long long peak_bound, unsigned long long max_pd, unsigned long long max_p,
                                           unsigned long long typical_tokens, int mean, int item_limit) {
         theta = theta_d; beta = beta_d;
         beta_i = theta_i = shift = 0;
+        theta_c = 0;
         unit = 1.0;
         if (WHOLE) {
             beta_i = (int)beta_d;
             // a threshold above every peak of the batch is as good as any other: the penalty is never paid
             theta_i = theta_d > (double)peak_bound ? (int)(peak_bound + 1) : (int)theta_d;
             free_below = max_p <= (unsigned long long)theta_i ? (unsigned int)((unsigned long long)theta_i - max_p) + 1 : 0u;
+            far_top = 0xffffffffu;
+        } else if (HALVES) {
+            for (shift = 1, unit = 2.0; beta * unit != 2.0 * floor(0.5 * beta * unit) && shift < 8; ++shift) unit *= 2.0;
+            beta_i = (int)(0.5 * beta * unit);
+            theta_c = (long long)ceil((double)beta_i * theta);
+            const double most = floor(theta) - (double)max_p, far = theta + ldexp(1.0, ilogb(theta) + 1) / (double)beta_i - (double)max_p;
+            free_below = most < 0.0 ? 0u : (unsigned int)most + 1u;
+            far_top = far < 0.0 ? 0u : far >= 4294967294.0 ? 0xffffffffu : (unsigned int)far;
         } else {
+            far_top = 0xffffffffu;
             // seven binary digits, fewer (below none: units of several tokens) for long requests, many tokens or a large beta
             shift = 7;
             unit = 128.0;
@@ -580,10 +606,12 @@ template <bool WHOLE> struct Scores {
     }
     __device__ __forceinline__ int key_b(unsigned int tokens, unsigned int t) const {
         if (WHOLE) return 2 * ((int)tokens + beta_i * ((int)t - theta_i));
+        if (HALVES) return 2 * (int)min(max(2 * (((long long)tokens << (shift - 1)) + (long long)beta_i * t - theta_c) + 1, (long long)(RS_LOWEST / 2)), (long long)(RS_CUT / 2));
         return 2 * min(max(__double2int_rd(((double)tokens + beta * ((double)t - theta)) * unit), RS_LOWEST / 2), RS_CUT / 2);
     }
     __device__ __forceinline__ int key_p(int P) const {      // what a prompt adds to b
         if (WHOLE) return (int)min(2ll * beta_i * P, (long long)RS_TOP_KEY);
+        if (HALVES) return 2 * (int)min(2ll * beta_i * P, (long long)(RS_CUT / 2));
         return 2 * min(__double2int_rd(beta * (double)P * unit), RS_CUT / 2);
     }
     __device__ __forceinline__ int key_pd(int P, int D) const {
@@ -608,6 +636,8 @@ template <bool WHOLE> struct Scores {
         if constexpr (WHOLE) return tokens + (unsigned int)(beta_i * max((int)peak - theta_i, 0));
         else return summary_score(tokens, peak, (double)P + (double)D, theta, beta);
     }
+    // whether a row that may pay is far
+    __device__ __forceinline__ bool far_row(unsigned int top, unsigned int jtop, int H) const { return jtop >= far_from(H) || (HALVES && top >= far_top); }
     __device__ __forceinline__ bool no_penalty(unsigned int top, int P) const { return beta == 0.0 || !((double)(top + (unsigned int)P) > theta); }
     static __device__ __forceinline__ S warp_min(S s) {   // scores are >= 0: ordered by their bits
         if constexpr (WHOLE) return __reduce_min_sync(FULL_MASK, s);
@@ -619,8 +649,8 @@ template <bool WHOLE> struct Scores {
         }
     }
 };
-template <bool WHOLE>
-__device__ __forceinline__ int Scores<WHOLE>::key_least(unsigned int state, int kp, int Dc, int& exact) const {
+template <int KIND>
+__device__ __forceinline__ int Scores<KIND>::key_least(unsigned int state, int kp, int Dc, int& exact) const {
     const int drop = (int)((state >> RS_DROP) & RS_DROP_MAX), jt = (int)(state & RS_JTOP), near = (state & RS_FAR) ? 0 : 1;
     const int no_drop = slope ? (int)RS_DROP_MAX : 0, far_add = Dc >= RS_LIMIT ? kp : RS_LOWEST, jt_max = slope ? RS_NEAR : 0;
     const int by_first = drop < no_drop ? kp - slope * drop : RS_LOWEST;
@@ -639,12 +669,12 @@ __device__ __forceinline__ int job_row(const RsShared& sh, unsigned int job) {
     if (!(job & RS_BY_SLOT)) return (int)(job & ~RS_GIVEN);
     return LISTS ? sh.list_row[(job >> 16) & 1][job_slot(job)] : (int)job_slot(job);
 }
-template <bool ADMIT, bool WHOLE, bool LISTS>
+template <bool ADMIT, int KIND, bool LISTS>
 struct Folder {
     const RouteSumArgs& a;
     RsShared& sh;
     const Rows& rows;
-    const Scores<WHOLE>& sc;
+    const Scores<KIND>& sc;
     int far_steps;      // steps of a stretch
 
     __device__ __forceinline__ void store_numbers(int w, const RowNumbers& n) {
@@ -737,7 +767,7 @@ struct Folder {
             not_over = not_over && !((double)n.above > a.many);
             full = (n.jtop >= (unsigned int)RS_NEAR && n.top >= sc.free_below) || (not_over && (double)most_above(n) > a.many);
         }
-        const bool pays = n.top >= sc.free_below, far = pays && n.jtop >= far_from(H);
+        const bool pays = n.top >= sc.free_below, far = pays && sc.far_row(n.top, n.jtop, H);
         unsigned int key_top = n.top, key_step = n.jtop;
         if (far) key_top = first_top(n.near0, n.near1, H, key_step);
         __syncwarp();   // every lane's cells before the row is handed on
@@ -745,7 +775,7 @@ struct Folder {
             if (pays && key_step > ld_volatile(&sh.jmax)) atomicMax(&sh.jmax, key_step);
             const unsigned int now = tokens + (unsigned int)P + (unsigned int)D;
             rows.top[w] = n.top;
-            if (!WHOLE) rows.tok[w] = now;
+            if (!Scores<KIND>::WHOLE) rows.tok[w] = now;
             rows.rec[w] = make_int2(sc.key_a(now), sc.key_b(now, key_top));
             rows.state[w] = n.jtop | (drop_of(key_top, n.near0) << RS_DROP) | (far ? RS_FAR : 0u) | (full ? RS_FULL : 0u) | (deferred ? RS_DEFERRED : 0u) | (not_over ? RS_NOT_OVER : 0u);
             if (ADMIT && (state & RS_NOT_OVER) && !not_over) atomicSub(&sh.not_over, 1u);
@@ -781,14 +811,14 @@ struct Folder {
 // rounding.  A closer look takes the scores of the rows that can be the best, and scans those that are only bounded.
 // What bounds it: the hand-over and one or two passes over the rows' words in shared memory.  By the deciding warp alone the look at the
 // keys took 3,000 cycles with 4,096 rows, and the closer one, taken for all bounded rows and all binary64 scores, 28,000.
-template <int FOLD_WARPS, bool ADMIT, bool WHOLE, bool LISTS>
+template <int FOLD_WARPS, bool ADMIT, int KIND, bool LISTS>
 struct Look {
-    typedef typename Scores<WHOLE>::S S;
+    typedef typename Scores<KIND>::S S;
     static constexpr int STRIDE = 32 * FOLD_WARPS;
     const RouteSumArgs& a;
     RsShared& sh;
     const Rows& rows;
-    const Scores<WHOLE>& sc;
+    const Scores<KIND>& sc;
     unsigned int met;
 
     // The rows from `start` on, 32 of every EACH: {smallest key, odd if exact; its row; the next smallest key}.
@@ -812,21 +842,21 @@ struct Look {
                 const int add = sc.key_least(st[u], kp, Dc, exact), v = max(r[u].x, r[u].y + add);
                 const int free = ((st[u] & RS_FAR) ? 0 : 1) & (r[u].y + kp <= r[u].x ? 1 : 0);      // (no penalty: the token count)
                 const int key = v | exact | free;
-                if (!WHOLE) next = min(next, max(least, key));
+                if (!Scores<KIND>::EXACT) next = min(next, max(least, key));
                 least_row = key < least ? base + u * EACH : least_row;      // a lane's rows ascend
                 least = min(least, key);
             }
         }
         const int best = __reduce_min_sync(FULL_MASK, least);
         const int win = __reduce_min_sync(FULL_MASK, least == best ? least_row : RS_NO_ROW);
-        if (!WHOLE) next = __reduce_min_sync(FULL_MASK, least_row == win ? next : least);
+        if (!Scores<KIND>::EXACT) next = __reduce_min_sync(FULL_MASK, least_row == win ? next : least);
         return make_int4(best, win, next, 0);
     }
     // Whether such keys decide: a whole-number key that is exact does, one in binary64 if no other is as close as its rounding.
     __device__ __forceinline__ bool decide(const int4& k, int kp, int P, int Dc) const {
         if (!(k.x & 1) || k.y >= a.I) return false;
-        if (WHOLE) return true;
-        if (k.z <= k.x + Scores<WHOLE>::SLACK || k.x >= RS_CUT || kp >= RS_CUT) return false;
+        if (Scores<KIND>::EXACT) return Scores<KIND>::WHOLE || (k.x < RS_CUT && kp < RS_CUT);
+        if (k.z <= k.x + Scores<KIND>::SLACK || k.x >= RS_CUT || kp >= RS_CUT) return false;
         return Dc > (int)(rows.state[k.y] & RS_JTOP) || sc.no_penalty(rows.top[k.y], P);
     }
     // (deciding warp) The keys of all folding warps together.
@@ -865,16 +895,16 @@ struct Look {
     __device__ __forceinline__ void smallest(int stage, S& best, int& win, unsigned int& peak) const {
         const int lane = threadIdx.x & 31, x = lane < FOLD_WARPS ? lane : 0;
         S s;
-        if constexpr (WHOLE) s = (S)sh.look_score[stage][x];
+        if constexpr (Scores<KIND>::WHOLE) s = (S)sh.look_score[stage][x];
         else s = __longlong_as_double((long long)sh.look_score[stage][x]);
         const int r = sh.look_row[stage][x];
-        best = Scores<WHOLE>::warp_min(s);
+        best = Scores<KIND>::warp_min(s);
         win = __reduce_min_sync(FULL_MASK, s == best ? r : RS_NO_ROW);
         peak = __shfl_sync(FULL_MASK, sh.look_peak[stage][x], __ffs(__ballot_sync(FULL_MASK, s == best && r == win)) - 1);
     }
     __device__ __forceinline__ void put(int stage, int me, S best, int win, unsigned int peak) {
         if ((threadIdx.x & 31) != 0) return;
-        if constexpr (WHOLE) sh.look_score[stage][me] = best;
+        if constexpr (Scores<KIND>::WHOLE) sh.look_score[stage][me] = best;
         else sh.look_score[stage][me] = (unsigned long long)__double_as_longlong(best);
         sh.look_row[stage][me] = win;
         sh.look_peak[stage][me] = peak;
@@ -896,8 +926,8 @@ struct Look {
         if (!meet()) return false;
         // (keys that are cut say nothing: then every row counts)
         const int smallest_most = unordered(sh.look_least);
-        const int reach = !WHOLE && (smallest_most >= RS_CUT || kp >= RS_CUT) ? 0x7fffffff : smallest_most + Scores<WHOLE>::SLACK;
-        S mine = Scores<WHOLE>::none();
+        const int reach = !Scores<KIND>::WHOLE && (smallest_most >= RS_CUT || kp >= RS_CUT) ? 0x7fffffff : smallest_most + Scores<KIND>::SLACK;
+        S mine = Scores<KIND>::none();
         int mine_row = RS_NO_ROW, n = 0;
         unsigned int mine_peak = 0;
         unsigned long long open = 0;       // the lane's rows that are only bounded and could have the smallest score
@@ -912,7 +942,7 @@ struct Look {
                 if (s < mine || mine_row == RS_NO_ROW) { mine = s; mine_row = i; mine_peak = top + (unsigned int)P; }
             } else open |= 1ull << n;
         }
-        S best = Scores<WHOLE>::warp_min(mine);
+        S best = Scores<KIND>::warp_min(mine);
         int win = __reduce_min_sync(FULL_MASK, mine == best ? mine_row : RS_NO_ROW);
         unsigned int peak = __shfl_sync(FULL_MASK, mine_peak, __ffs(__ballot_sync(FULL_MASK, mine == best && mine_row == win)) - 1);
         put(0, me, best, win, peak);
@@ -934,7 +964,7 @@ struct Look {
                     const int src = __ffs(which) - 1, w = __shfl_sync(FULL_MASK, i, src);
                     const unsigned int t = __shfl_sync(FULL_MASK, tokens, src);
                     unsigned int p = 0;
-                    Folder<ADMIT, WHOLE, LISTS> f{a, sh, rows, sc, far_chunks(a.H) * RS_NEAR};
+                    Folder<ADMIT, KIND, LISTS> f{a, sh, rows, sc, far_chunks(a.H) * RS_NEAR};
                     if (!f.scan(w, P, Dc, decided, p)) return false;
                     const S s = sc.of_peak(t, p, P, D);
                     if (s < best || (s == best && w < win)) { best = s; win = w; peak = p; }
@@ -947,11 +977,11 @@ struct Look {
     }
 };
 
-template <int FOLD_WARPS, bool ADMIT, bool WHOLE, bool LISTS>
-__device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, int me) {
+template <int FOLD_WARPS, bool ADMIT, int KIND, bool LISTS>
+__device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<KIND>& sc, int me) {
     const int lane = threadIdx.x & 31;
-    Folder<ADMIT, WHOLE, LISTS> f{a, sh, rows, sc, far_chunks(a.H) * RS_NEAR};
-    Look<FOLD_WARPS, ADMIT, WHOLE, LISTS> look{a, sh, rows, sc, 0u};
+    Folder<ADMIT, KIND, LISTS> f{a, sh, rows, sc, far_chunks(a.H) * RS_NEAR};
+    Look<FOLD_WARPS, ADMIT, KIND, LISTS> look{a, sh, rows, sc, 0u};
     unsigned int looks = 0;
     for (unsigned int n = me;;) {
         uint4 ctl;
@@ -990,8 +1020,8 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
 }
 
 // ---- io warp: arrivals ahead of the decisions, results behind the folds
-template <int KS, int FOLD_WARPS, bool ADMIT, bool WHOLE>
-__device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, const Scores<WHOLE>& sc, long long q_head, int waiting, int items, int room) {
+template <int KS, int FOLD_WARPS, bool ADMIT, int KIND>
+__device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, const Scores<KIND>& sc, long long q_head, int waiting, int items, int room) {
     const int lane = threadIdx.x & 31;
     const long long n0 = sh.n0;
     auto put_result = [&](int k, int c, double s) {
@@ -1096,10 +1126,10 @@ __device__ __forceinline__ void prefetch_row(const uint2* near, const unsigned i
     asm volatile("prefetch.global.L1 [%0]; prefetch.global.L1 [%0 + 128]; prefetch.global.L1 [%1];" ::"l"(near + (size_t)row * 32), "l"(far + (size_t)row * 32));
 }
 
-template <int LIST_WARPS, int KS, bool WHOLE>
-__device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc, const uint2* near_cells, const unsigned int* far_cells, int I, int mean, int longest, int t) {
+template <int LIST_WARPS, int KS, int KIND>
+__device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, const Scores<KIND>& sc, const uint2* near_cells, const unsigned int* far_cells, int I, int mean, int longest, int t) {
     constexpr int THREADS = 32 * LIST_WARPS, ROOM = 32 * KS, NEAR_ROOM = RS_NEAR_ROWS / LIST_WARPS;
-    constexpr int FAR_KEY = 0x7f000000, AT_ONCE = 4;      // AT_ONCE: rows a thread has on their way
+    constexpr int FAR_KEY = 0x7f000000, EACH = 4, AT_ONCE = 4;      // AT_ONCE: rows a thread has on their way
     static_assert(NEAR_ROOM >= 2 * 32 * AT_ONCE, "");
     const int lane = threadIdx.x & 31, me = t >> 5;
     const bool leader = t < 32;
@@ -1176,25 +1206,29 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
             int n_near = 0, n_take = 0;
             auto sort_near = [&]() {        // the rows that were not dropped: into the list or into a bucket
                 __syncwarp();
-                // (two rows a lane at once and no branches: what bounds this is the latency of a row's chain)
-                for (int x = lane; x - lane < n_near; x += 64) {
-                    int2 r[2];
-                    bool in[2], take[2], low[2];
-                    int i[2], c[2];
+                // (several rows a lane at once and no branches: what bounds this is the latency of a row's chain)
+                for (int x = lane; x - lane < n_near; x += 32 * EACH) {
+                    int2 r[EACH];
+                    bool in[EACH], take[EACH], low = false;
+                    int i[EACH], c[EACH];
                     #pragma unroll
-                    for (int u = 0; u < 2; ++u) { in[u] = x + 32 * u < n_near; i[u] = near[in[u] ? x + 32 * u : 0]; }
+                    for (int u = 0; u < EACH; ++u) { in[u] = x + 32 * u < n_near; i[u] = near[in[u] ? x + 32 * u : 0]; }
                     #pragma unroll
-                    for (int u = 0; u < 2; ++u) r[u] = ld_volatile2(rows.rec + i[u]);
+                    for (int u = 0; u < EACH; ++u) r[u] = ld_volatile2(rows.rec + i[u]);
                     #pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        take[u] = false;
+                    for (int u = 0; u < EACH; ++u) {
+                        // (the largest limit_b of the probes whose limit_a the row keeps)
+                        int most_b = RS_LOWEST;
                         #pragma unroll
-                        for (int p = 0; p < RS_PROBES; ++p) take[u] |= r[u].x <= limit_a[p] && r[u].y <= limit_b[p];
-                        take[u] &= in[u];
+                        for (int p = RS_PROBES - 1; p >= 0; --p) most_b = r[u].x <= limit_a[p] ? max(most_b, limit_b[p]) : most_b;
+                        take[u] = in[u] && r[u].y <= most_b && most_b != RS_LOWEST;
                         c[u] = sc.row_code(r[u]);
                     }
+                    unsigned int was_a[EACH], was_b[EACH];
                     #pragma unroll
-                    for (int u = 0; u < 2; ++u) {
+                    for (int u = 0; u < EACH; ++u) { was_a[u] = ld_volatile(&sh.bucket_a[c[u]]); was_b[u] = ld_volatile(&sh.bucket_b[c[u]]); }
+                    #pragma unroll
+                    for (int u = 0; u < EACH; ++u) {
                         const unsigned int vote = __ballot_sync(FULL_MASK, take[u]);
                         const int at = n_take + __popc(vote & ((1u << lane) - 1u));
                         if (take[u] && at < ROOM) sh.list_seg[me][at] = (unsigned short)i[u];
@@ -1202,12 +1236,13 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
                         const bool left = in[u] && !take[u], middle = left && c[u] != 0 && c[u] != 31;
                         hot_b = min(hot_b, left && c[u] == 0 ? r[u].y : FAR_KEY);
                         cold_a = min(cold_a, left && c[u] == 31 ? r[u].x : FAR_KEY);
-                        low[u] = middle && (ordered(r[u].x) < ld_volatile(&sh.bucket_a[c[u]]) || ordered(r[u].y) < ld_volatile(&sh.bucket_b[c[u]]));
+                        in[u] = middle && (ordered(r[u].x) < was_a[u] || ordered(r[u].y) < was_b[u]);
+                        low |= in[u];
                     }
-                    if (__any_sync(FULL_MASK, low[0] || low[1])) {      // (most rows change no bucket)
+                    if (__any_sync(FULL_MASK, low)) {      // (most rows change no bucket)
                         #pragma unroll
-                        for (int u = 0; u < 2; ++u)
-                            if (low[u]) {
+                        for (int u = 0; u < EACH; ++u)
+                            if (in[u]) {
                                 atomicMin(&sh.bucket_a[c[u]], ordered(r[u].x));
                                 atomicMin(&sh.bucket_b[c[u]], ordered(r[u].y));
                             }
@@ -1274,7 +1309,7 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
                 // The entries as keys that the deciding warp holds: a row that wins by less than the rounding of its key does not beat them.
                 // (The base is a lower bound of every row's score, so an entry that is cut below is one, too.)
                 const int base = unordered(sh.probe_t[0]) & ~1;
-                auto entry = [&](int key) { return Held<KS>::relative(key, base) - 1 - Held<KS>::scaled(Scores<WHOLE>::SLACK); };
+                auto entry = [&](int key) { return Held<KS>::relative(key, base) - 1 - Held<KS>::scaled(Scores<KIND>::SLACK); };
                 sh.table[now][lane] = make_int4(entry(above_a), entry(below_b), entry(ka), entry(row_b));
                 const int c = sc.code((float)probe_key);
                 const int ex = __shfl_sync(FULL_MASK, above_a, c), ey = __shfl_sync(FULL_MASK, below_b, c), ez = __shfl_sync(FULL_MASK, ka, c), ew = __shfl_sync(FULL_MASK, row_b, c);
@@ -1297,15 +1332,15 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
 // instructions (85 and 130).  So nothing else is in the loop: no branch (one per step cost 50 to 100 cycles; whether all steps were usual
 // is seen once per trip, which is taken back as far as they were not), items and bounds fetched two steps ahead, and what need not
 // be in the chain (scores, token counts, the tables) is done by the folding warps.
-template <int KS, bool LISTS, int FOLD_WARPS, bool ADMIT, bool WHOLE>
-__device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<WHOLE>& sc) {
-    typedef typename Scores<WHOLE>::S S;
+template <int KS, bool LISTS, int FOLD_WARPS, bool ADMIT, int KIND>
+__device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<KIND>& sc) {
+    typedef typename Scores<KIND>::S S;
     typedef Held<KS> K;
-    constexpr int SLACK = Scores<WHOLE>::SLACK * (1 << K::SLOT_BITS);
+    constexpr int SLACK = Scores<KIND>::SLACK * (1 << K::SLOT_BITS);
     // steps of a trip: decisions are made known to the folding warps by trips (few rows: soon)
-    constexpr int TRIP = KS <= 2 ? 2 : 4;
+    constexpr int TRIP = KS == 1 ? 2 : 4;
     // decisions between two looks at items and at the rows that were pending
-    constexpr unsigned int CHUNK = LISTS ? 32 : 4 * KS;
+    constexpr unsigned int CHUNK = LISTS ? 64 : 8 * KS;
     const int lane = threadIdx.x & 31, I = a.I, H = a.H;
     const int lane_f = lane < FOLD_WARPS ? lane : 0;
     unsigned int looks = 0;
@@ -1324,7 +1359,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     int jmax = 0;        // an arrival whose ramp is longer than this reaches the step of every row's b
     auto take_base = [&](int b) {
         base = b;
-        cut = (WHOLE ? K::CUT : min(K::CUT, RS_CUT - b)) * (1 << K::SLOT_BITS) - 1 - SLACK;
+        cut = (Scores<KIND>::WHOLE ? K::CUT : min(K::CUT, RS_CUT - b)) * (1 << K::SLOT_BITS) - 1 - SLACK;
     };
     auto unread = [&]() {        // all rows present are marked, with keys that are below any
         #pragma unroll
@@ -1445,7 +1480,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         const int2 pd = sh.raw[e % RS_ITEMS];
         const int P = pd.x, D = pd.y, Dc = D < H ? D : H, kp = sc.key_p(P), kpe = it.x;
         const int kpde = K::scaled(min(sc.key_pd(P, D), K::ITEM));
-        const Look<FOLD_WARPS, ADMIT, WHOLE, LISTS> look{a, sh, rows, sc, 0u};
+        const Look<FOLD_WARPS, ADMIT, KIND, LISTS> look{a, sh, rows, sc, 0u};
         publish(e);
         auto received = [&](int t) {     // the arrival's ramp reaches the step of the row's b
             #pragma unroll
@@ -1499,11 +1534,11 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                         return far;
                     }())))
                     return false;
-            } else if (WHOLE) {
+            } else if (Scores<KIND>::EXACT) {
                 return false;
             } else {
                 const int reach = (__reduce_min_sync(FULL_MASK, least) & ~K::TAGS) + SLACK;
-                S mine = Scores<WHOLE>::none();
+                S mine = Scores<KIND>::none();
                 int mine_tag = NO_ROW;
                 bool scan = false;
                 unsigned int open = 0;
@@ -1531,7 +1566,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                         } else scan = true;
                     }
                 if (!__any_sync(FULL_MASK, scan)) {
-                    const S best = Scores<WHOLE>::warp_min(mine);
+                    const S best = Scores<KIND>::warp_min(mine);
                     const int win = __reduce_min_sync(FULL_MASK, mine == best ? mine_tag : NO_ROW);
                     if (win != NO_ROW) {
                         received(win);
@@ -1592,7 +1627,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                     refresh();
                     continue;
                 }
-                S mine = Scores<WHOLE>::none();
+                S mine = Scores<KIND>::none();
                 int mine_row = NO_ROW;
                 unsigned int open = 0, reached = 0;     // (of the lane's rows) only bounded; the ramp reaches the step of the top
                 bool wait = false;
@@ -1622,7 +1657,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                     refresh();
                     continue;
                 }
-                S best = Scores<WHOLE>::warp_min(mine);
+                S best = Scores<KIND>::warp_min(mine);
                 int win = __reduce_min_sync(FULL_MASK, mine == best ? mine_row : NO_ROW);
                 unsigned int peak = 0;
                 bool scanned = false;
@@ -1645,8 +1680,8 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                         folding_warps_look(RS_SCANS);
                         if (lost) return false;
                         const unsigned int p = todo ? sh.scan_peak[slot] : 0u;
-                        const S s = todo ? sc.of_peak(tokens, p, P, D) : Scores<WHOLE>::none();
-                        const S smallest = Scores<WHOLE>::warp_min(s);
+                        const S s = todo ? sc.of_peak(tokens, p, P, D) : Scores<KIND>::none();
+                        const S smallest = Scores<KIND>::warp_min(s);
                         const int r = __reduce_min_sync(FULL_MASK, todo && s == smallest ? i : NO_ROW);
                         if (smallest < best || (smallest == best && r < win)) {
                             best = smallest; win = r; scanned = true;
@@ -1708,6 +1743,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     };
     unsigned int e = 0, ready = 0;   // decisions made, items known to be there
     while (!lost) {     // (every way out has published what was decided)
+        ready = __shfl_sync(FULL_MASK, ld_acquire(&sh.items_ready), 0);
         if (e >= ready) {
             bool end = false;
             if (!rs_wait(sh, [&] {
@@ -1739,6 +1775,8 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         const unsigned int stop = min(limit, e + CHUNK);
         refresh();
         fetch(e);
+        unsigned int untold = 0;      // decisions before e that are not told yet (the last trip's: they are while the next reduction is under way)
+        int told = 0;
         while (e < stop) {
             int was_a[KS], was_b[KS], key[TRIP], not_usual = 0;
             const unsigned int at = at_items + 16u * (e % RS_ITEMS);
@@ -1756,6 +1794,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 if (KS == 1) least = min(least, v[0]);
                 const int best = __reduce_min_sync(FULL_MASK, least);
                 // (while the reduction is under way)
+                if (u == 0 && untold) { tell(e - TRIP, told, TRIP); publish(e); }
                 it0 = it1; it1 = it2;
                 it2 = ld_table(at + 16u * (u + 3));
                 bound = bound_for(it0, ahead);
@@ -1765,7 +1804,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                     if (v[k] == best) { ra[k] += kpd; rb[k] += kpb; }
                 key[u] = best;
                 not_usual |= best & 1;
-                if (!WHOLE) {     // another row that can be the best
+                if (!Scores<KIND>::EXACT) {     // another row that can be the best
                     int next = 0x7fffffff;
                     #pragma unroll
                     for (int k = 0; k < KS; ++k) next = min(next, v[k] == best ? 0x7fffffff : v[k]);
@@ -1773,13 +1812,13 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                     if (next <= (best | K::TAGS) + SLACK) not_usual |= 2 << u;
                 }
             }
-            int told = key[0];
+            told = key[0];
             #pragma unroll
             for (int u = 1; u < TRIP; ++u) told = lane == u ? key[u] : told;
+            untold = 0;
             if (not_usual == 0 && e + TRIP <= limit) {
-                tell(e, told, TRIP);
                 e += TRIP;
-                publish(e);
+                untold = TRIP;
                 continue;
             }
             // ---- the first `usual` steps of the trip stand, the others are taken back
@@ -1811,6 +1850,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             }
             fetch(e);
         }
+        if (untold) { tell(e - TRIP, told, TRIP); publish(e); }
     }
     __syncwarp();
     if (lane == 0) st_release(&sh.ctl.z, 1u);
@@ -1906,8 +1946,8 @@ __device__ __noinline__ void rs_literal(const RouteSumArgs& a, RsShared& sh, lon
 // The maps need nothing: they receive the ramps of every table row that is not marked as applied.  Returns the first item that
 // was not decided (the ones from there on that are malformed or find the table full have their results already, the same
 // as those that were not reached).  (`rows` and `sc` by value: by reference they would live on the stack of every thread.)
-template <int FOLD_WARPS, bool LISTS, bool ADMIT, bool WHOLE>
-__device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const Rows rows, const Scores<WHOLE> sc, int waiting) {
+template <int FOLD_WARPS, bool LISTS, bool ADMIT, int KIND>
+__device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const Rows rows, const Scores<KIND> sc, int waiting) {
     const unsigned int told = sh.ctl.x;
     for (unsigned int e = sh.written + threadIdx.x; e < told; e += blockDim.x) {
         const uint2 job = sh.jobs[e % RS_ITEMS];
@@ -1930,15 +1970,19 @@ __device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const
     return sh.items_ready > told ? sh.item_at[told % RS_ITEMS] : sh.cursor;
 }
 
-// Folding and list warps, warps and threads of the instantiations.
-template <bool LISTS, bool ADMIT> struct Shape {
-    static constexpr int FOLD = 8, LIST = LISTS ? RS_LIST_WARPS : 0;
+// Folding and list warps, warps and threads of the instantiations.  (Decisions come every 100 to 150 cycles and a fold takes some 700 from when
+// it is told: fewer warps than that leave the rows pending for longer, and more would leave the deciding warp fewer registers.  Measured
+// on 512 x 1,024 / 4,096 x 2,048, us: 10 and 4 warps 1,036 / 11,141 with 6 and 5, 8 and 6 1,064 / 10,910, 6 and 5 1,080 / 11,279; two folds
+// at once by one warp, or the next one's loads ahead: 1,131 and 1,178, as either makes a single fold take longer.)
+template <int KS, bool LISTS> struct Shape {
+    static constexpr int FOLD = !LISTS ? 8 : KS == 4 ? 10 : 8, LIST = !LISTS ? 0 : KS == 4 ? 4 : 6;
     static constexpr int WARPS = 4 * ((FOLD + 1 + LIST + 2) / 3), THREADS = 32 * WARPS;
+    static_assert(FOLD <= RS_MAX_FOLD_WARPS && LIST <= RS_LIST_WARPS, "");
 };
 
-template <int KS, bool LISTS, bool ADMIT, bool WHOLE>
-__global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_summaries(const __grid_constant__ RouteSumArgs a) {
-    typedef Shape<LISTS, ADMIT> Sp;
+template <int KS, bool LISTS, bool ADMIT, int KIND>
+__global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summaries(const __grid_constant__ RouteSumArgs a) {
+    typedef Shape<KS, LISTS> Sp;
     constexpr int THREADS = Sp::THREADS;
     extern __shared__ __align__(16) unsigned char rs_smem[];
     __shared__ __align__(16) RsShared sh;
@@ -1980,7 +2024,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
         const bool ok = guard[GUARD_BAD] == 0 && peak_bound <= 0xffffffffull && token_bound <= 0xffffffffull &&
                         a.n_arrivals + (ADMIT ? a.queue_capacity : 0) < (1ll << 26);
         // (whole-number scores: the host has seen to beta and theta)
-        const bool exact = !WHOLE || token_bound + max_pd + (unsigned long long)a.beta * (peak_bound + 1) < (1ull << 29);
+        const bool exact = !Scores<KIND>::WHOLE || token_bound + max_pd + (unsigned long long)a.beta * (peak_bound + 1) < (1ull << 29);
         sh.mode = ok && exact ? 1 : 0;
         sh.spin_limit = a.spin_limit;
         sh.idle_limit = max(a.spin_limit < (1u << 27) ? 16u * a.spin_limit : 0xffffffffu, 1u << 22);
@@ -2028,7 +2072,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     } else {
     const unsigned long long mean_l = ramps / (unsigned long long)(n_items > 0 ? n_items : 1);
     const int mean = mean_l < (1ull << 22) ? (int)mean_l : 1 << 22;     // prompt + ramp of a typical request
-    Scores<WHOLE> sc;
+    Scores<KIND> sc;
     sc.start(a.theta, a.beta, peak_bound, max_pd, max_p, (base_sum + tokens_in) / (unsigned long long)I, mean, Held<KS>::ITEM);
     {
         unsigned int jmax = 0, n_far = 0;
@@ -2048,7 +2092,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
                 if (ADMIT) above = a.over0[i];
             }
             const unsigned int jtop = q.z & 0xffffu, step = (q.z >> 16) & 31u, drop = q.z >> 21;
-            const bool pays = q.y >= sc.free_below, far = pays && jtop >= far_from(H);
+            const bool pays = q.y >= sc.free_below, far = pays && sc.far_row(q.y, jtop, H);
             jmax = max(jmax, !pays ? 0u : far ? step : jtop);
             n_far += far;
             const bool not_over = ADMIT && !((double)above > a.many);
@@ -2058,7 +2102,7 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
             rows.state[i] = jtop | (drop << RS_DROP) | (far ? RS_FAR : 0u) | (pays && jtop >= (unsigned int)RS_NEAR ? RS_FULL : 0u) | (not_over ? RS_NOT_OVER : 0u);
             rows.top[i] = q.y;
             if (alone) sh.pending[i] = 0;
-            if (!WHOLE) rows.tok[i] = q.x;
+            if (!Scores<KIND>::WHOLE) rows.tok[i] = q.x;
             a.newest[i] = RS_NOBODY;
             #pragma unroll
             for (int p = 0; p < PROBES; ++p) least[p] = min(least[p], max(rec.x, rec.y + sc.key_p(rs_probe(mean, p))));
@@ -2083,26 +2127,26 @@ __global__ void __launch_bounds__(Shape<LISTS, ADMIT>::THREADS, 1) pre_route_sum
     __syncthreads();
     if (LISTS && a.may_decline) {
         unsigned int n_least = 0;
-        for (int i = tid; i < I; i += THREADS) n_least += max(rows.rec[i].x, rows.rec[i].y) <= unordered(sh.probe_t[0]) + Scores<WHOLE>::SLACK;
+        for (int i = tid; i < I; i += THREADS) n_least += max(rows.rec[i].x, rows.rec[i].y) <= unordered(sh.probe_t[0]) + Scores<KIND>::SLACK;
         n_least = __reduce_add_sync(FULL_MASK, n_least);
         if (lane == 0 && n_least) atomicAdd(&sh.n_least, n_least);
         __syncthreads();
-        if ((H > RS_FAR_STEPS && sh.n_far > (unsigned int)(I / RS_FAR_SHARE)) || sh.n_least > 32u * KS) { decline(); return; }
+        if ((H > RS_FAR_STEPS && sh.n_far > (unsigned int)(I / RS_FAR_SHARE)) || sh.n_least > 32u * KS || sc.shift < RS_COARSE_SHIFT) { decline(); return; }
     }
 
     const int role = (warp >> 2) * 3 + (warp & 3) - 1;      // (of the warps that are not on the deciding warp's scheduler)
     if (warp == 0) {
-        rs_decide_loop<KS, LISTS, Sp::FOLD, ADMIT, WHOLE>(a, sh, rows, sc);
+        rs_decide_loop<KS, LISTS, Sp::FOLD, ADMIT, KIND>(a, sh, rows, sc);
     } else if ((warp & 3) != 0) {
-        if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, WHOLE, LISTS>(a, sh, rows, sc, role);
+        if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, KIND, LISTS>(a, sh, rows, sc, role);
         else if (role == Sp::FOLD)
-            rs_io_loop<KS, Sp::FOLD, ADMIT, WHOLE>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
+            rs_io_loop<KS, Sp::FOLD, ADMIT, KIND>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
         else if (LISTS && role <= Sp::FOLD + Sp::LIST)
-            rs_list_loop<LISTS ? Sp::LIST : 8, KS, WHOLE>(sh, rows, sc, a.near, a.far, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
+            rs_list_loop<LISTS ? Sp::LIST : 4, KS, KIND>(sh, rows, sc, a.near, a.far, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
     }
     __syncthreads();
     if (sh.ctl.w) {     // (all threads alike: nobody writes it any more)
-        decided = rs_settle<Sp::FOLD, LISTS, ADMIT, WHOLE>(a, sh, rows, sc, (int)q_len);
+        decided = rs_settle<Sp::FOLD, LISTS, ADMIT, KIND>(a, sh, rows, sc, (int)q_len);
         __syncthreads();
     }
     }
@@ -2199,21 +2243,32 @@ static bool summaries_whole_numbers(const pre_ctx* ctx) {
     return beta == floor(beta) && theta == floor(theta) && beta <= 1048576.0 && theta < 1073741824.0;
 }
 
+// beta = m / 2^k and m * theta with a fraction: see RS_HALVES.  (Where m is larger or theta small, rows are far whose peaks are ordinary.)
+static bool summaries_halves(const pre_ctx* ctx) {
+    const double beta = ctx->cfg.beta, theta = ctx->theta, least = 1.0 / 65536.0;
+    double m = beta;
+    for (int k = 0; k < 2 && m != floor(m); ++k) m *= 2.0;
+    if (!(m >= 1.0 && m <= 3.0) || m != floor(m)) return false;
+    const double f = m * theta - floor(m * theta);
+    return theta >= 1024.0 && theta < 268435456.0 && f > least && f < 1.0 - least;
+}
+
 // All rows in the deciding warp's registers while that is at most eight per lane, a list of 128 or 256 beyond (a list costs a
 // look at its bounds per arrival and a share of the next list: about what four more rows per lane cost).
-template <bool ADMIT, bool WHOLE>
+template <bool ADMIT, int KIND>
 static const void* summaries_kernel(int I) {
-    if (I <= 32) return (const void*)pre_route_summaries<1, false, ADMIT, WHOLE>;
-    if (I <= 64) return (const void*)pre_route_summaries<2, false, ADMIT, WHOLE>;
-    if (I <= 128) return (const void*)pre_route_summaries<4, false, ADMIT, WHOLE>;
-    if (I <= RS_DIRECT_ROWS) return (const void*)pre_route_summaries<8, false, ADMIT, WHOLE>;
-    if (I <= RS_LONG_LISTS) return (const void*)pre_route_summaries<4, true, ADMIT, WHOLE>;
-    return (const void*)pre_route_summaries<8, true, ADMIT, WHOLE>;
+    if (I <= 32) return (const void*)pre_route_summaries<1, false, ADMIT, KIND>;
+    if (I <= 64) return (const void*)pre_route_summaries<2, false, ADMIT, KIND>;
+    if (I <= 128) return (const void*)pre_route_summaries<4, false, ADMIT, KIND>;
+    if (I <= RS_DIRECT_ROWS) return (const void*)pre_route_summaries<8, false, ADMIT, KIND>;
+    if (I <= RS_LONG_LISTS) return (const void*)pre_route_summaries<4, true, ADMIT, KIND>;
+    return (const void*)pre_route_summaries<8, true, ADMIT, KIND>;
 }
 template <bool ADMIT>
 static const void* summaries_kernel_for(const pre_ctx* ctx) {
     const int I = ctx->cfg.n_instances;
-    return summaries_whole_numbers(ctx) ? summaries_kernel<ADMIT, true>(I) : summaries_kernel<ADMIT, false>(I);
+    return summaries_whole_numbers(ctx) ? summaries_kernel<ADMIT, RS_WHOLE>(I)
+           : summaries_halves(ctx) ? summaries_kernel<ADMIT, RS_HALVES>(I) : summaries_kernel<ADMIT, RS_ROUNDED>(I);
 }
 
 template <bool ADMIT>
@@ -2303,7 +2358,7 @@ static cudaError_t launch_summary_kernels(pre_ctx* ctx, const SumArgs& p, const 
     }
     typedef void (*Kernel)(const RouteSumArgs);
     const Kernel kernel = reinterpret_cast<Kernel>(const_cast<void*>(summaries_kernel_for<ADMIT>(ctx)));
-    const int threads = I > RS_DIRECT_ROWS ? Shape<true, ADMIT>::THREADS : Shape<false, ADMIT>::THREADS;
+    const int threads = I <= RS_DIRECT_ROWS ? Shape<1, false>::THREADS : I <= RS_LONG_LISTS ? Shape<4, true>::THREADS : Shape<8, true>::THREADS;
     const size_t smem = ADMIT ? ctx->route_summary_smem_admit : ctx->route_summary_smem;
     if (a.alone) {
         kernel<<<1, threads, smem, s>>>(a);

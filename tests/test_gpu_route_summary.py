@@ -464,3 +464,18 @@ def test_large_fractional_penalties(n_inst, h, beta):
     ad = rng.integers(1, 2 * h, 500).astype(np.int32)
     wl.max_requests = 10 * n_inst + 500
     route_and_compare(wl, ap, ad, batches=2)
+
+
+@pytest.mark.parametrize("n_inst,h", [(7, 48), (40, 300), (140, 64), (257, 90), (2100, 40)])
+@pytest.mark.parametrize("beta,capacity,t_mem", [(1.0, 1281, 0.8), (1.0, 5003, 0.8), (1.0, 40001, 0.8), (1.0, 20000, 0.812345),
+                                                 (0.75, 2003, 0.8), (0.75, 30002, 0.8), (0.5, 9001, 0.8), (3.0, 7007, 0.8)])
+def test_scores_with_a_fraction_that_all_paying_rows_share(n_inst, h, beta, capacity, t_mem):
+    """beta a small dyadic fraction and a fractional threshold: whole-number keys decide as the binary64 scores do, ties among rows that pay and ties among
+    rows that do not; peaks so far beyond the threshold (the small capacities) that beta times the excess is no longer exact."""
+    wl = W.make_random(640 + n_inst % 83, n_inst, h, 10 * n_inst, 0, max_prompt=600, max_output=h, capacity=capacity, beta=beta)
+    wl.t_mem = t_mem
+    rng = np.random.default_rng(25)
+    ap = rng.choice([40, 41, 300, 2000], 500).astype(np.int32)      # (many equal sums)
+    ad = rng.choice([3, 30, h - 1, 2 * h], 500).astype(np.int32)
+    wl.max_requests = 10 * n_inst + 500
+    route_and_compare(wl, ap, ad, batches=2)
