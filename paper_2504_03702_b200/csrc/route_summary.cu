@@ -27,10 +27,11 @@
 //                        arithmetic stays exact for the whole batch;
 //   pre_route_summaries  routes the batch with ONE block whose warps have different jobs:
 //     deciding warp  takes the arrivals one by one.  It holds rows in registers (two keys each), takes
-//                    every row's score for the arrival, the smallest by two warp reductions, and updates the winner in
+//                    every row's score for the arrival, the smallest and its row by one warp reduction, and updates the winner in
 //                    place: no other warp is in this chain.  Up to 256 instances it holds all rows.  Beyond, it holds
-//                    the at most 128 rows of a list (256 beyond 2,048 instances), and a table that bounds the scores of all other rows from below:
-//                    while the best row of the list beats that bound it is the best row of all.
+//                    the at most 128 rows of a list (256 beyond RS_LONG_LISTS instances), and a table that bounds the scores of all other rows from
+//                    below: while the best row of the list beats that bound it is the best row of all.  Up to 32 instances it folds
+//                    its decisions itself.
 //     list warps     (beyond 256 instances) build the next list while the present one is being used up: the rows
 //                    whose score is within a margin of the smallest one for any of eight prompt lengths, and the
 //                    bounds of the rest.  Scores only grow during a batch, so a list that is a little behind is valid.
@@ -669,17 +670,20 @@ __device__ __forceinline__ int job_row(const RsShared& sh, unsigned int job) {
     if (!(job & RS_BY_SLOT)) return (int)(job & ~RS_GIVEN);
     return LISTS ? sh.list_row[(job >> 16) & 1][job_slot(job)] : (int)job_slot(job);
 }
+struct Cells { uint2* near; unsigned int* far; };      // [I][32] each
 template <bool ADMIT, int KIND, bool LISTS>
 struct Folder {
     const RouteSumArgs& a;
     RsShared& sh;
     const Rows& rows;
     const Scores<KIND>& sc;
+    uint2* near;        // the first cells and the stretches: in device memory, or (rows of the deciding warp alone) in shared
+    unsigned int* far;
     int far_steps;      // steps of a stretch
 
     __device__ __forceinline__ void store_numbers(int w, const RowNumbers& n) {
-        a.near[(size_t)w * 32 + (threadIdx.x & 31)] = make_uint2(n.near0, n.near1);
-        a.far[(size_t)w * 32 + (threadIdx.x & 31)] = n.far;
+        near[(size_t)w * 32 + (threadIdx.x & 31)] = make_uint2(n.near0, n.near1);
+        far[(size_t)w * 32 + (threadIdx.x & 31)] = n.far;
     }
     // At most so many cells are above the overload level: the first ones counted, a stretch whole if its bound is above.
     __device__ __forceinline__ int most_above(const RowNumbers& n) {
@@ -738,8 +742,8 @@ struct Folder {
         const uint2 job = sh.jobs[e % RS_ITEMS];
         const int2 pd = sh.raw[e % RS_ITEMS];
         const int w = job_row<LISTS>(sh, job.x), P = pd.x, D = pd.y, Dc = D < H ? D : H;
-        const uint2 q = a.near[(size_t)w * 32 + lane];      // (on their way before anything else)
-        const unsigned int q_far = a.far[(size_t)w * 32 + lane];
+        const uint2 q = near[(size_t)w * 32 + lane];      // (on their way before anything else)
+        const unsigned int q_far = far[(size_t)w * 32 + lane];
         const unsigned int state = rows.state[w], old_top = rows.top[w];
         const unsigned int tokens = sc.tokens_of(rows, w);
         RowNumbers n;
@@ -767,9 +771,9 @@ struct Folder {
             not_over = not_over && !((double)n.above > a.many);
             full = (n.jtop >= (unsigned int)RS_NEAR && n.top >= sc.free_below) || (not_over && (double)most_above(n) > a.many);
         }
-        const bool pays = n.top >= sc.free_below, far = pays && sc.far_row(n.top, n.jtop, H);
+        const bool pays = n.top >= sc.free_below, is_far = pays && sc.far_row(n.top, n.jtop, H);
         unsigned int key_top = n.top, key_step = n.jtop;
-        if (far) key_top = first_top(n.near0, n.near1, H, key_step);
+        if (is_far) key_top = first_top(n.near0, n.near1, H, key_step);
         __syncwarp();   // every lane's cells before the row is handed on
         if (lane == 0) {
             if (pays && key_step > ld_volatile(&sh.jmax)) atomicMax(&sh.jmax, key_step);
@@ -777,7 +781,7 @@ struct Folder {
             rows.top[w] = n.top;
             if (!Scores<KIND>::WHOLE) rows.tok[w] = now;
             rows.rec[w] = make_int2(sc.key_a(now), sc.key_b(now, key_top));
-            rows.state[w] = n.jtop | (drop_of(key_top, n.near0) << RS_DROP) | (far ? RS_FAR : 0u) | (full ? RS_FULL : 0u) | (deferred ? RS_DEFERRED : 0u) | (not_over ? RS_NOT_OVER : 0u);
+            rows.state[w] = n.jtop | (drop_of(key_top, n.near0) << RS_DROP) | (is_far ? RS_FAR : 0u) | (full ? RS_FULL : 0u) | (deferred ? RS_DEFERRED : 0u) | (not_over ? RS_NOT_OVER : 0u);
             if (ADMIT && (state & RS_NOT_OVER) && !not_over) atomicSub(&sh.not_over, 1u);
             sh.scored[e % RS_ITEMS] = make_uint2(tokens, (job.x & RS_GIVEN) ? job.y : old_top + (unsigned int)P);
             sh.jobs[e % RS_ITEMS].x = (unsigned int)w | (job.x & RS_GIVEN);
@@ -789,9 +793,9 @@ struct Folder {
     __device__ __forceinline__ bool scan(int w, int P, int Dc, unsigned int decided, unsigned int& peak) {
         const int lane = threadIdx.x & 31, H = a.H;
         // the first cells, and what bounds the others: enough when Dc ends among the first and none of the others can be larger
-        const uint2 q = a.near[(size_t)w * 32 + lane];
+        const uint2 q = near[(size_t)w * 32 + lane];
         const int j = 2 * lane, lo = RS_NEAR + lane * far_steps;
-        const unsigned int u = a.far[(size_t)w * 32 + lane];
+        const unsigned int u = far[(size_t)w * 32 + lane];
         peak = __reduce_max_sync(FULL_MASK, max(q.x + (j < Dc ? (unsigned int)(P + j) : 0u), q.y + (j + 1 < Dc ? (unsigned int)(P + j + 1) : 0u)));
         const bool others = Dc > RS_NEAR || u > peak + (unsigned int)(u ? lo : 0);
         if (!__any_sync(FULL_MASK, others)) return true;
@@ -819,6 +823,7 @@ struct Look {
     RsShared& sh;
     const Rows& rows;
     const Scores<KIND>& sc;
+    const Cells& cells;
     unsigned int met;
 
     // The rows from `start` on, 32 of every EACH: {smallest key, odd if exact; its row; the next smallest key}.
@@ -964,7 +969,7 @@ struct Look {
                     const int src = __ffs(which) - 1, w = __shfl_sync(FULL_MASK, i, src);
                     const unsigned int t = __shfl_sync(FULL_MASK, tokens, src);
                     unsigned int p = 0;
-                    Folder<ADMIT, KIND, LISTS> f{a, sh, rows, sc, far_chunks(a.H) * RS_NEAR};
+                    Folder<ADMIT, KIND, LISTS> f{a, sh, rows, sc, cells.near, cells.far, far_chunks(a.H) * RS_NEAR};
                     if (!f.scan(w, P, Dc, decided, p)) return false;
                     const S s = sc.of_peak(t, p, P, D);
                     if (s < best || (s == best && w < win)) { best = s; win = w; peak = p; }
@@ -977,22 +982,23 @@ struct Look {
     }
 };
 
-template <int FOLD_WARPS, bool ADMIT, int KIND, bool LISTS>
-__device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<KIND>& sc, int me) {
+// SELF: the deciding warp folds, these warps only look.
+template <int FOLD_WARPS, bool ADMIT, int KIND, bool LISTS, bool SELF>
+__device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<KIND>& sc, const Cells& cells, int me) {
     const int lane = threadIdx.x & 31;
-    Folder<ADMIT, KIND, LISTS> f{a, sh, rows, sc, far_chunks(a.H) * RS_NEAR};
-    Look<FOLD_WARPS, ADMIT, KIND, LISTS> look{a, sh, rows, sc, 0u};
+    Folder<ADMIT, KIND, LISTS> f{a, sh, rows, sc, cells.near, cells.far, far_chunks(a.H) * RS_NEAR};
+    Look<FOLD_WARPS, ADMIT, KIND, LISTS> look{a, sh, rows, sc, cells, 0u};
     unsigned int looks = 0;
     for (unsigned int n = me;;) {
         uint4 ctl;
         if (!rs_wait<true>(sh, [&] {
                 ctl = ld_volatile4(&sh.ctl);
-                return (int)(ctl.x - n) > 0 || ctl.y != looks || ctl.z != 0;
-            }, LISTS ? 20 : 0))    // (the list warps need the issue slots)
+                return (!SELF && (int)(ctl.x - n) > 0) || ctl.y != looks || ctl.z != 0;
+            }, LISTS || SELF ? 20 : 0))    // (the list warps need the issue slots)
             return;
         acquire_cta();
-        if (__all_sync(FULL_MASK, (int)(ctl.x - n) <= 0)) ctl = ld_volatile4(&sh.ctl);
-        if (__any_sync(FULL_MASK, (int)(ctl.x - n) > 0)) {
+        if (SELF || __all_sync(FULL_MASK, (int)(ctl.x - n) <= 0)) ctl = ld_volatile4(&sh.ctl);
+        if (!SELF && __any_sync(FULL_MASK, (int)(ctl.x - n) > 0)) {
             if (!f.fold(n)) return;
             n += FOLD_WARPS;
             if (lane == 0) st_release(&sh.done[me], n);
@@ -1288,7 +1294,7 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
             for (int x = lane; x < n_take; x += 32) {
                 const int i = sh.list_seg[me][x];
                 sh.list_row[now][before + x] = i;
-                prefetch_row(near_cells, far_cells, i);     // (the folds of its rows: 280 cycles less)
+                prefetch_row(near_cells, far_cells, i);     // (for the folds of its rows)
             }
             if (leader) {
                 // (a key that no row has set is out of reach; rows of code 31 count by their a alone, no b is kept for them)
@@ -1326,23 +1332,36 @@ __device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, con
     }
 }
 
+// Folding and list warps, warps and threads of the instantiations.  (Decisions come every 100 to 150 cycles and a fold takes some 700 from when
+// it is told: fewer warps than that leave the rows pending for longer, and more would leave the deciding warp fewer registers.  Measured
+// on 512 x 1,024 / 4,096 x 2,048, us: 10 and 4 warps 1,036 / 11,141 with 6 and 5, 8 and 6 1,064 / 10,910, 6 and 5 1,080 / 11,279; two folds
+// at once by one warp, or the next one's loads ahead: 1,131 and 1,178, as either makes a single fold take longer.)
+template <int KS, bool LISTS> struct Shape {
+    static constexpr int FOLD = !LISTS ? 8 : KS == 4 ? 10 : 8, LIST = !LISTS ? 0 : KS == 4 ? 4 : 6;
+    static constexpr bool SELF = KS == 1;                  // the deciding warp folds its decisions itself
+    static constexpr int DONE = SELF ? 1 : FOLD;           // warps that fold
+    static constexpr int WARPS = 4 * ((FOLD + 1 + LIST + 2) / 3), THREADS = 32 * WARPS;
+    static_assert(FOLD <= RS_MAX_FOLD_WARPS && LIST <= RS_LIST_WARPS, "");
+};
+
 // ---- deciding warp.  KS: rows per lane.  LISTS: they are a list's, else all rows.
 // What bounds it: the latency of one chain of dependent instructions per arrival (a warp reduction, 23 cycles, and some eight integer
 // operations: 65 cycles with two rows per lane, in a kernel with nothing else) and, with four and eight rows per lane, the number of its
-// instructions (85 and 130).  So nothing else is in the loop: no branch (one per step cost 50 to 100 cycles; whether all steps were usual
+// instructions (85 and 130).  In the kernel a step takes 85, 130 and 160 to 185 cycles.  So nothing else is in the loop: no branch (one per step cost 50 to 100 cycles; whether all steps were usual
 // is seen once per trip, which is taken back as far as they were not), items and bounds fetched two steps ahead, and what need not
 // be in the chain (scores, token counts, the tables) is done by the folding warps.
 template <int KS, bool LISTS, int FOLD_WARPS, bool ADMIT, int KIND>
-__device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<KIND>& sc) {
+__device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<KIND>& sc, const Cells& cells) {
     typedef typename Scores<KIND>::S S;
     typedef Held<KS> K;
     constexpr int SLACK = Scores<KIND>::SLACK * (1 << K::SLOT_BITS);
     // steps of a trip: decisions are made known to the folding warps by trips (few rows: soon)
-    constexpr int TRIP = KS == 1 ? 2 : 4;
+    constexpr int TRIP = 4;
     // decisions between two looks at items and at the rows that were pending
     constexpr unsigned int CHUNK = LISTS ? 64 : 8 * KS;
     const int lane = threadIdx.x & 31, I = a.I, H = a.H;
-    const int lane_f = lane < FOLD_WARPS ? lane : 0;
+    constexpr bool SELF = Shape<KS, LISTS>::SELF;
+    const int lane_f = lane < Shape<KS, LISTS>::DONE ? lane : 0;
     unsigned int looks = 0;
     bool lost = false;
 
@@ -1480,7 +1499,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         const int2 pd = sh.raw[e % RS_ITEMS];
         const int P = pd.x, D = pd.y, Dc = D < H ? D : H, kp = sc.key_p(P), kpe = it.x;
         const int kpde = K::scaled(min(sc.key_pd(P, D), K::ITEM));
-        const Look<FOLD_WARPS, ADMIT, KIND, LISTS> look{a, sh, rows, sc, 0u};
+        const Look<FOLD_WARPS, ADMIT, KIND, LISTS> look{a, sh, rows, sc, cells, 0u};
         publish(e);
         auto received = [&](int t) {     // the arrival's ramp reaches the step of the row's b
             #pragma unroll
@@ -1581,7 +1600,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             if (lane == 0) { sh.look_P = P; sh.look_D = D; sh.look_how = how; sh.look_least = 0xffffffffu; }
             __syncwarp();
             if (lane == 0) st_release(&sh.ctl.y, looks);
-            if (!rs_wait(sh, [&] { return ld_acquire(&sh.looks_done[lane_f]) == looks; })) lost = true;
+            if (!rs_wait(sh, [&] { return ld_acquire(&sh.looks_done[lane < FOLD_WARPS ? lane : 0]) == looks; })) lost = true;
         };
         // A held row takes the arrival without its ramp being known to reach the step of the row's b, or that fitting into the keys.
         auto received_some = [&](int win) {
@@ -1741,6 +1760,113 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         if (LISTS) { now = ld_table(table + it0.w); ahead = ld_table(table + it1.w); }
         bound = bound_for(it0, now);
     };
+    if constexpr (SELF) {
+        // ---- up to 32 rows, one per lane: the deciding warp folds each decision itself, so that no row is ever pending.  With few rows the next
+        // arrival mostly wants the row that was just taken, and waiting for a folding warp took 650 cycles an arrival (8 x 64).  What bounds
+        // it: the chain of an arrival, three reductions and two accesses of shared memory.  (Whole passes: 21 x 60, 14 arrivals 37 -> 30 us; with
+        // more rows the folding warps are ahead: 64 x 256 takes 170 cycles an arrival with them.)
+        Folder<ADMIT, KIND, LISTS> f{a, sh, rows, sc, cells.near, cells.far, far_chunks(H) * RS_NEAR};
+        const int mine = lane < I ? lane : 0, j = 2 * lane, steps = f.far_steps, lo = RS_NEAR + lane * steps;
+        unsigned int state, top, tokens;        // of the lane's row
+        auto own = [&]() { state = ld_volatile(rows.state + mine); top = ld_volatile(rows.top + mine); tokens = sc.tokens_of(rows, mine); };
+        auto publish_folded = [&](unsigned int n) {
+            __syncwarp();
+            if (lane == 0) { st_release(&sh.done[0], n); st_release(&sh.ctl.x, n); }
+        };
+        own();
+        unsigned int e = 0, ready = 0;
+        while (!lost) {
+            ready = __shfl_sync(FULL_MASK, ld_acquire(&sh.items_ready), 0);
+            if (e >= ready) {
+                bool end = false;
+                if (!rs_wait(sh, [&] {
+                        end = __any_sync(FULL_MASK, ld_acquire(&sh.items_end) != 0);    // (before the count: the count is then final)
+                        ready = __shfl_sync(FULL_MASK, ld_acquire(&sh.items_ready), 0);
+                        return ready > e || end;
+                    }))
+                    break;
+                if (ready <= e) break;
+            }
+            const unsigned int stop = min(ready, e + 32);
+            int4 it = ld_table(at_items + 16u * (e % RS_ITEMS));
+            int2 pd = ld_volatile2(sh.raw + e % RS_ITEMS);
+            while (e < stop) {
+                if (ADMIT && ld_volatile(&sh.not_over) == 0) break;
+                const int key = max(rb[0] + it.x, ra[0]);
+                const int best = __reduce_min_sync(FULL_MASK, min(key, it.z > jmax ? cut : (int)0x80000001u));
+                bool usual = (best & 1) == 0;
+                if (!Scores<KIND>::EXACT)
+                    usual = usual && __reduce_min_sync(FULL_MASK, key == best ? 0x7fffffff : key) > (best | K::TAGS) + SLACK;
+                const int P = pd.x, D = pd.y, Dc = D < H ? D : H, w = (best & K::SLOT) >> 1;
+                const unsigned int at = e % RS_ITEMS;
+                if (usual) {
+                    RowNumbers n;
+                    const uint2 q = cells.near[w * 32 + lane];
+                    n.far = cells.far[w * 32 + lane];
+                    const unsigned int w_state = __shfl_sync(FULL_MASK, state, w), w_top = __shfl_sync(FULL_MASK, top, w), w_tokens = __shfl_sync(FULL_MASK, tokens, w);
+                    it = ld_table(at_items + 16u * (at + 1));
+                    pd = ld_volatile2(sh.raw + (e + 1) % RS_ITEMS);
+                    n.near0 = q.x + (j < Dc ? (unsigned int)(P + j) : 0u);
+                    n.near1 = q.y + (j + 1 < Dc ? (unsigned int)(P + j + 1) : 0u);
+                    n.far += lo < Dc ? (unsigned int)(P + min(Dc, lo + steps) - 1) : 0u;
+                    const unsigned int t0 = j < H ? n.near0 + (unsigned int)j : 0u, t = max(t0, j + 1 < H ? n.near1 + (unsigned int)(j + 1) : 0u);
+                    n.top = __reduce_max_sync(FULL_MASK, t);
+                    n.jtop = __reduce_min_sync(FULL_MASK, t == n.top && j < H ? (unsigned int)(t0 == t ? j : j + 1) : 0xffffffffu);
+                    const bool beyond = __any_sync(FULL_MASK, n.far > n.top);
+                    // (a row with RS_FULL, a stretch that may hold the top, a row that may be overloaded now: the general fold)
+                    const bool general = (w_state & RS_FULL) || beyond || (ADMIT && (w_state & RS_NOT_OVER) && (double)f.most_above(n) > a.many);
+                    if (!general) {
+                        f.store_numbers(w, n);
+                        const bool pays = n.top >= sc.free_below, far = pays && sc.far_row(n.top, n.jtop, H);
+                        unsigned int key_top = n.top, step = n.jtop;
+                        if (far) key_top = first_top(n.near0, n.near1, H, step);
+                        if (pays && (int)step > jmax) { jmax = (int)step; if (lane == 0) sh.jmax = step; }
+                        const unsigned int now = w_tokens + (unsigned int)P + (unsigned int)D;
+                        const unsigned int drop = drop_of(key_top, __shfl_sync(FULL_MASK, n.near0, 0));
+                        if (lane == w) {
+                            state = n.jtop | (drop << RS_DROP) | (far ? RS_FAR : 0u) | RS_DEFERRED | (w_state & RS_NOT_OVER);
+                            top = n.top; tokens = now;
+                            const int2 rec = make_int2(sc.key_a(now), sc.key_b(now, key_top));
+                            ra[0] = K::relative(rec.x, base) + tag(0) + (far ? 1 : 0);
+                            rb[0] = K::relative(rec.y, base) + tag(0) + (far ? 1 : 0);
+                            rows.rec[w] = rec; rows.state[w] = state; rows.top[w] = top;
+                            if (!Scores<KIND>::WHOLE) rows.tok[w] = now;
+                            sh.scored[at] = make_uint2(w_tokens, w_top + (unsigned int)P);
+                            sh.jobs[at].x = (unsigned int)w;
+                        }
+                        ++e;
+                        if ((e & 7u) == 0) publish_folded(e);
+                        continue;
+                    }
+                    tell_slot(e, 2 * w, 0u, 0u);
+                    if (lane == w) ra[0] |= 1;
+                    publish_folded(e);
+                } else {
+                    publish_folded(e);
+                    if (!unusual(e)) {
+                        if (lost) break;
+                        refresh();
+                        it = ld_table(at_items + 16u * at);
+                        pd = ld_volatile2(sh.raw + at);
+                        continue;
+                    }
+                }
+                if (!f.fold(e)) { lost = true; break; }
+                __syncwarp();
+                own();
+                refresh();
+                ++e;
+                it = ld_table(at_items + 16u * (e % RS_ITEMS));
+                pd = ld_volatile2(sh.raw + e % RS_ITEMS);
+            }
+            publish_folded(e);
+            if (lost) break;
+            if (ADMIT && e < ready && ld_volatile(&sh.not_over) == 0) {   // every instance overloaded: the batch stops here
+                if (lane == 0) { sh.blocked = 1; sh.blocked_k = sh.item_at[e % RS_ITEMS]; }
+                break;
+            }
+        }
+    } else {
     unsigned int e = 0, ready = 0;   // decisions made, items known to be there
     while (!lost) {     // (every way out has published what was decided)
         ready = __shfl_sync(FULL_MASK, ld_acquire(&sh.items_ready), 0);
@@ -1791,7 +1917,6 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 int least = bound;
                 #pragma unroll
                 for (int k = 0; k + 1 < KS; k += 2) least = __vimin3_s32(least, v[k], v[k + 1]);
-                if (KS == 1) least = min(least, v[0]);
                 const int best = __reduce_min_sync(FULL_MASK, least);
                 // (while the reduction is under way)
                 if (u == 0 && untold) { tell(e - TRIP, told, TRIP); publish(e); }
@@ -1841,16 +1966,19 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             }
             tell(e, told, usual);
             e += usual;
-            if (usual < there) {
-                if (unusual(e)) { ++e; publish(e); }
-                else if (lost) break;
-                else refresh();
-            } else {
-                publish(e);
-            }
-            fetch(e);
+            publish(e);
+            if (usual < there)
+                do {      // (no trip for the next arrival either while it does not reach every row's top)
+                    if (unusual(e)) { ++e; publish(e); }
+                    else if (lost) break;
+                    else refresh();
+                    fetch(e);
+                } while (e < stop && __any_sync(FULL_MASK, bound == (int)0x80000001u));
+            else fetch(e);
+            if (lost) break;
         }
         if (untold) { tell(e - TRIP, told, TRIP); publish(e); }
+    }
     }
     __syncwarp();
     if (lane == 0) st_release(&sh.ctl.z, 1u);
@@ -1970,16 +2098,6 @@ __device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const
     return sh.items_ready > told ? sh.item_at[told % RS_ITEMS] : sh.cursor;
 }
 
-// Folding and list warps, warps and threads of the instantiations.  (Decisions come every 100 to 150 cycles and a fold takes some 700 from when
-// it is told: fewer warps than that leave the rows pending for longer, and more would leave the deciding warp fewer registers.  Measured
-// on 512 x 1,024 / 4,096 x 2,048, us: 10 and 4 warps 1,036 / 11,141 with 6 and 5, 8 and 6 1,064 / 10,910, 6 and 5 1,080 / 11,279; two folds
-// at once by one warp, or the next one's loads ahead: 1,131 and 1,178, as either makes a single fold take longer.)
-template <int KS, bool LISTS> struct Shape {
-    static constexpr int FOLD = !LISTS ? 8 : KS == 4 ? 10 : 8, LIST = !LISTS ? 0 : KS == 4 ? 4 : 6;
-    static constexpr int WARPS = 4 * ((FOLD + 1 + LIST + 2) / 3), THREADS = 32 * WARPS;
-    static_assert(FOLD <= RS_MAX_FOLD_WARPS && LIST <= RS_LIST_WARPS, "");
-};
-
 template <int KS, bool LISTS, bool ADMIT, int KIND>
 __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summaries(const __grid_constant__ RouteSumArgs a) {
     typedef Shape<KS, LISTS> Sp;
@@ -1992,6 +2110,11 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
     rows.state = reinterpret_cast<unsigned int*>(rows.rec + I);
     rows.top = rows.state + I;
     rows.tok = rows.top + I;     // (binary64 scores only)
+    Cells cells{a.near, a.far};
+    if (Sp::SELF) {
+        cells.near = reinterpret_cast<uint2*>(rows.tok + (Scores<KIND>::WHOLE ? 0 : I + (I & 1)));
+        cells.far = reinterpret_cast<unsigned int*>(cells.near + 32 * I);
+    }
 
     // (the warp's number by a shuffle: the compiler then knows that the roles part between warps and not within one, and
     // leaves out what would bring the lanes of a warp together again: 157 instead of 202 cycles for a step of the deciding warp)
@@ -2003,7 +2126,7 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
         if (tid < GUARDS) sh_guard[tid] = 0;
         __syncthreads();
         for (int i = warp; i < I; i += Sp::WARPS)
-            summarise_row(a, i, a.near, a.far, sh_guard, [&](const uint4& q, int above) {
+            summarise_row(a, i, cells.near, cells.far, sh_guard, [&](const uint4& q, int above) {
                 rows.rec[i] = make_int2((int)q.x, (int)q.w);
                 rows.top[i] = q.y;
                 rows.state[i] = q.z;
@@ -2081,6 +2204,8 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
         int least[PROBES];                     // the smallest value per probe, for the first list
         #pragma unroll
         for (int p = 0; p < PROBES; ++p) least[p] = 0x7f000000;
+        if (Sp::SELF && !alone)
+            for (int i = tid; i < 32 * I; i += THREADS) { cells.near[i] = a.near[i]; cells.far[i] = a.far[i]; }
         for (int i = tid; i < I; i += THREADS) {
             uint4 q;
             int above = 0;
@@ -2136,17 +2261,17 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
 
     const int role = (warp >> 2) * 3 + (warp & 3) - 1;      // (of the warps that are not on the deciding warp's scheduler)
     if (warp == 0) {
-        rs_decide_loop<KS, LISTS, Sp::FOLD, ADMIT, KIND>(a, sh, rows, sc);
+        rs_decide_loop<KS, LISTS, Sp::FOLD, ADMIT, KIND>(a, sh, rows, sc, cells);
     } else if ((warp & 3) != 0) {
-        if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, KIND, LISTS>(a, sh, rows, sc, role);
+        if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, KIND, LISTS, Sp::SELF>(a, sh, rows, sc, cells, role);
         else if (role == Sp::FOLD)
-            rs_io_loop<KS, Sp::FOLD, ADMIT, KIND>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
+            rs_io_loop<KS, Sp::DONE, ADMIT, KIND>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
         else if (LISTS && role <= Sp::FOLD + Sp::LIST)
             rs_list_loop<LISTS ? Sp::LIST : 4, KS, KIND>(sh, rows, sc, a.near, a.far, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
     }
     __syncthreads();
     if (sh.ctl.w) {     // (all threads alike: nobody writes it any more)
-        decided = rs_settle<Sp::FOLD, LISTS, ADMIT, KIND>(a, sh, rows, sc, (int)q_len);
+        decided = rs_settle<Sp::DONE, LISTS, ADMIT, KIND>(a, sh, rows, sc, (int)q_len);
         __syncthreads();
     }
     }
@@ -2280,7 +2405,8 @@ static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* s
     cudaFuncAttributes attr;
     cudaError_t e = cudaFuncGetAttributes(&attr, fn);
     if (e != cudaSuccess) return e;
-    const size_t smem = (size_t)I * (sizeof(int2) + (summaries_whole_numbers(ctx) ? 2 : 3) * sizeof(unsigned int));
+    size_t smem = (size_t)I * (sizeof(int2) + (summaries_whole_numbers(ctx) ? 2 : 3) * sizeof(unsigned int));
+    if (I <= 32) smem += sizeof(uint2) + (size_t)I * 32 * (sizeof(uint2) + sizeof(unsigned int));      // (the rows' cells)
     if (smem + attr.sharedSizeBytes + 256 > limit) return cudaSuccess;   // too many instances
     // (the limit is shared by every context of the process: always the device maximum)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(limit - attr.sharedSizeBytes));
