@@ -45,9 +45,9 @@ ROUTE_DRAM_READ = {3: 67322880}
 # profiles/ncu_dram_route_summary_kernels_config3_full_batch.txt: the three kernels of the summary router on the full
 # batch (the traffic does not grow in proportion to the batch, so the figure is used for the full batch only)
 ROUTE_SUMMARY_DRAM_TRAFFIC = {(3, 65536): 67732992 + 165120 + 2322176 + 50707456 + 2891264}
-# warp instructions per arrival of pre_route_summaries (smsp__inst_executed.sum of the 2,048-arrival capture in
-# profiles/ncu_full_step_kernels_config3_2048_arrivals.txt: 1,565,269 / 2,048)
-ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL = {3: 1565269 / 2048}
+# warp instructions per arrival of pre_route_summaries; none of the present kernel have been captured (the capture in
+# profiles/ncu_full_step_kernels_config3_2048_arrivals.txt is of the kernel with two reductions per arrival)
+ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL = {}
 ROUTE_DRAM_WRITE_PER_ARRIVAL = {3: 679168 / 256}
 ANTICIPATE_DRAM_TRAFFIC = {3: 33812992 + 19587328}
 STEP_DRAM_TRAFFIC = {3: 33670144 + 67196928 + 9366528}
