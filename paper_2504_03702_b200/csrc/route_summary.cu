@@ -1632,7 +1632,8 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                             most = K::relative(max(sc.key_a(tokens), sc.key_b(tokens, rows.top[row(k)]) + kp), base);
                         }
                     }
-                    v[k] = max(ra[k], rb[k] + K::scaled(max(add, -K::LIMIT / 2))) & ~K::TAGS;
+                    // (an addition that leaves the range downwards, or of which nothing is known, says nothing: the row is still worth its a)
+                    v[k] = (add > -K::LIMIT / 2 ? max(ra[k], rb[k] + K::scaled(add)) : ra[k]) & ~K::TAGS;
                     least = min(least, most & ~K::TAGS);
                 }
                 const int reach = __reduce_min_sync(FULL_MASK, least) + SLACK;

@@ -479,3 +479,40 @@ def test_scores_with_a_fraction_that_all_paying_rows_share(n_inst, h, beta, capa
     ad = rng.choice([3, 30, h - 1, 2 * h], 500).astype(np.int32)
     wl.max_requests = 10 * n_inst + 500
     route_and_compare(wl, ap, ad, batches=2)
+
+
+def one_request_each(prompt, generated, predicted, horizon, capacity, beta, arrivals):
+    """One request per instance: the map of instance i rises from prompt + generated to its last step, where cell + step is largest."""
+    n_inst = len(prompt)
+    wl = W.make_random(1, n_inst, horizon, 0, 0, capacity=capacity, beta=beta)
+    wl.prompt, wl.generated, wl.predicted = (np.asarray(x, dtype=np.int32) for x in (prompt, generated, predicted))
+    wl.instance = np.arange(n_inst, dtype=np.int32)
+    wl.max_requests = n_inst + arrivals
+    return wl
+
+
+def test_a_short_arrival_on_a_row_whose_top_costs_more_than_half_the_range_of_the_keys():
+    """beta = 100,000: the top of row 150 lies at step 20, and its cells there cost 4 million less than cell + step says."""
+    prompt, predicted = np.full(200, 999), np.full(200, 2)
+    prompt[150], predicted[150] = 974, 22
+    wl = one_request_each(prompt, np.ones(200), predicted, 128, 1000, 1e5, 1)
+    ref = route_and_compare(wl, np.array([1], np.int32), np.array([2], np.int32))
+    assert ref.instance[200] == 150, "the case was meant to go to the row with the far lower peak"
+
+
+@pytest.mark.parametrize("n_inst", [20, 50, 100, 200])
+@pytest.mark.parametrize("h", [40, 128])
+@pytest.mark.parametrize("beta", [17000.0, 1e5, 1e6, 200.5, 2000.5, 1e15])
+def test_short_arrivals_with_large_penalties(n_inst, h, beta):
+    """Peaks within 20 tokens of the threshold, tops at steps up to 60 and as far above it: what such an arrival adds to the key of the
+    top is less than any key holds.  Every sixth row has its top among the first steps, where most arrivals reach it."""
+    rng = np.random.default_rng(int(beta) % 1000 + n_inst + h)
+    step = rng.integers(5, min(h, 61), n_inst)
+    step[::6] = rng.integers(0, 3, len(step[::6]))
+    peak = 200 + rng.integers(-20, 21, n_inst)
+    wl = one_request_each(peak - step - 1, np.ones(n_inst), step + 2, h, 250, beta, 60)
+    ap, ad = rng.integers(0, 5, 60).astype(np.int32), rng.integers(1, 5, 60).astype(np.int32)
+    before = oracle.State.from_workload(wl)
+    before.anticipate()
+    assert ((before.curves + np.arange(h)[None, :]).argmax(axis=1) == step).all() and (before.curves.max(axis=1) == peak).all()
+    route_and_compare(wl, ap, ad, batches=3)
