@@ -516,3 +516,57 @@ def test_short_arrivals_with_large_penalties(n_inst, h, beta):
     before.anticipate()
     assert ((before.curves + np.arange(h)[None, :]).argmax(axis=1) == step).all() and (before.curves.max(axis=1) == peak).all()
     route_and_compare(wl, ap, ad, batches=3)
+
+
+def skewed(n_inst, h, per, n_arr, beta, whole=True):
+    """`per` requests per instance on average, assigned by Zipf: most instances hold a few requests, and the tops of many maps lie far out."""
+    n = n_inst * per
+    prompt, generated, predicted = W._lengths(77, n, 1024, 1.2, 16, 8192, 384, 1.2, 1, 4096, in_flight=True)
+    instance = W._zipf_instances(77, n, n_inst, 1.1)
+    wl = W.make_random(77, n_inst, h, 0, 0, beta=beta, capacity=W._capacity(prompt, generated, instance, n_inst) // 5 * 5 + (0 if whole else 3))
+    wl.prompt, wl.generated, wl.predicted, wl.instance = prompt, generated, predicted, instance
+    ap, _, ad = W._lengths(78, n_arr, 1024, 1.2, 16, 8192, 384, 1.2, 1, 4096, in_flight=False)
+    wl.max_requests = n + n_arr
+    return wl, ap, ad
+
+
+@pytest.mark.parametrize("n_inst,h", [(300, 228), (700, 500), (1054, 228), (2100, 100)])
+@pytest.mark.parametrize("beta,whole", [(1.0, True), (1.0, False), (0.75, False), (0.4, False)])
+def test_far_rows_of_a_list_are_compared_in_place(n_inst, h, beta, whole):
+    wl, ap, ad = skewed(n_inst, h, 20, 400, beta, whole)
+    before = oracle.State.from_workload(wl)
+    before.anticipate()
+    far = (before.curves + np.arange(h)[None, :]).argmax(axis=1) >= 32
+    assert far.mean() > 0.1 and not far.all(), "the case was meant to have far rows and others"
+    route_and_compare(wl, ap, ad, batches=2)
+
+
+def share_of_the_scanning_time(wl, ap, ad):
+    """The library's choice of kernel against the scanning kernel, whose time does not depend on the rows: best of seven calls each."""
+    st = DeviceState.from_workload(wl)
+    p, d = dev(ap), dev(ad)
+    best = {}
+    for path in (B.ROUTE_AUTO, B.ROUTE_SCAN):
+        st.select_router(path)
+        times = []
+        for _ in range(7):
+            st.n_requests.fill_(len(wl.prompt))
+            st.queued_p.zero_()
+            st.anticipate(len(wl.prompt))
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            st.route_batch(p, d)
+            t1.record()
+            torch.cuda.synchronize()
+            times.append(t0.elapsed_time(t1))
+        best[path] = min(times)
+    assert st.status() == B.PRE_OK
+    st.close()
+    return best[B.ROUTE_AUTO] / best[B.ROUTE_SCAN]
+
+
+@pytest.mark.parametrize("beta,whole", [(1.0, True), (1.0, False)])
+def test_arrivals_on_far_rows_do_not_take_a_look_at_all_rows(beta, whole):
+    """Some 0.4 of the scanning kernel's time where a far row that wins is compared among the list's rows, 0.7 and more where each such
+    arrival takes a look at all rows."""
+    assert share_of_the_scanning_time(*skewed(1054, 228, 35, 817, beta, whole)) < 0.6
