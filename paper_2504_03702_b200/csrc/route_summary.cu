@@ -30,8 +30,8 @@
 //                    every row's score for the arrival, the smallest and its row by one warp reduction, and updates the winner in
 //                    place: no other warp is in this chain.  Up to 256 instances it holds all rows.  Beyond, it holds
 //                    the at most 128 rows of a list (256 beyond RS_LONG_LISTS instances), and a table that bounds the scores of all other rows from
-//                    below: while the best row of the list beats that bound it is the best row of all.  Up to 32 instances it folds
-//                    its decisions itself.
+//                    below: while the best row of the list beats that bound it is the best row of all.  Up to RS_SELF_ROWS instances
+//                    it folds its decisions itself.
 //     list warps     (beyond 256 instances) build the next list while the present one is being used up: the rows
 //                    whose score is within a margin of the smallest one for any of eight prompt lengths, and the
 //                    bounds of the rest.  Scores only grow during a batch, so a list that is a little behind is valid.
@@ -56,6 +56,10 @@ constexpr int RS_MAX_FOLD_WARPS = 10;
 constexpr int RS_LIST_WARPS = 6;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
 constexpr int RS_AHEAD = 8;                 // items that are fetched beyond the present one, at most
+// Up to so many rows the deciding warp folds its decisions itself: with few rows the next arrival mostly wants the row that was just taken. us a call,
+// by itself / by the folding warps: 2,000 arrivals on 256 steps, whole-number scores, 1 row 846 / 1,796, 4 rows 575 / 647, 6 rows 618 / 565, 20 rows
+// 561 / 278; fractional 1,028 / 1,957, 755 / 720, 778 / 627, 738 / 341; 32 arrivals on 64 steps: 4 rows 33 / 37, 8 rows 34 / 34, 32 rows 37 / 35.
+constexpr int RS_SELF_ROWS = 4;
 constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
 constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lane, 8 beyond RS_LONG_LISTS instances)
 constexpr int RS_LONG_LISTS = 1024;
@@ -1781,10 +1785,8 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         bound = bound_for(it0, now);
     };
     if constexpr (SELF) {
-        // ---- up to 32 rows, one per lane: the deciding warp folds each decision itself, so that no row is ever pending.  With few rows the next
-        // arrival mostly wants the row that was just taken, and waiting for a folding warp took 650 cycles an arrival (8 x 64).  What bounds
-        // it: the chain of an arrival, three reductions and two accesses of shared memory.  (Whole passes: 21 x 60, 14 arrivals 37 -> 30 us; with
-        // more rows the folding warps are ahead: 64 x 256 takes 170 cycles an arrival with them.)
+        // ---- up to RS_SELF_ROWS rows, one per lane: the deciding warp folds each decision itself, so that no row is ever pending.  What bounds it: the
+        // chain of an arrival, three reductions and two accesses of shared memory.
         Folder<ADMIT, KIND, LISTS> f{a, sh, rows, sc, cells.near, cells.far, far_chunks(H) * RS_NEAR};
         const int mine = lane < I ? lane : 0, j = 2 * lane, steps = f.far_steps, lo = RS_NEAR + lane * steps;
         unsigned int state, top, tokens;        // of the lane's row
@@ -2393,8 +2395,8 @@ static bool summaries_halves(const pre_ctx* ctx) {
     const double beta = ctx->cfg.beta, theta = ctx->theta, least = 1.0 / 65536.0;
     double m = beta;
     for (int k = 0; k < 2 && m != floor(m); ++k) m *= 2.0;
-    // (few rows soon have a backlog whose peaks make them far, and seldom tie: 7 x 108, 1,420 arrivals 679 us with rounded keys in the kernel
-    // before, 1,377 with exact ones)
+    // (few rows soon have a backlog whose peaks make them far, and seldom tie: beta = 0.75, 2,000 arrivals on 256 steps, 6, 20 and 32 rows: 631, 338 and 273 us
+    // with rounded keys, 2,022, 1,210 and 553 with exact ones)
     if (ctx->cfg.n_instances <= 32 || !(m >= 1.0 && m <= 3.0) || m != floor(m)) return false;
     const double f = m * theta - floor(m * theta);
     return theta >= 1024.0 && theta < 268435456.0 && f > least && f < 1.0 - least;
@@ -2404,7 +2406,9 @@ static bool summaries_halves(const pre_ctx* ctx) {
 // look at its bounds per arrival and a share of the next list: about what four more rows per lane cost).
 template <bool ADMIT, int KIND>
 static const void* summaries_kernel(int I) {
-    if (I <= 32) return (const void*)pre_route_summaries<1, false, ADMIT, KIND>;
+    if constexpr (KIND != RS_HALVES) {      // (that kind begins beyond)
+        if (I <= RS_SELF_ROWS) return (const void*)pre_route_summaries<1, false, ADMIT, KIND>;
+    }
     if (I <= 64) return (const void*)pre_route_summaries<2, false, ADMIT, KIND>;
     if (I <= 128) return (const void*)pre_route_summaries<4, false, ADMIT, KIND>;
     if (I <= RS_DIRECT_ROWS) return (const void*)pre_route_summaries<8, false, ADMIT, KIND>;
@@ -2428,7 +2432,7 @@ static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* s
     cudaError_t e = cudaFuncGetAttributes(&attr, fn);
     if (e != cudaSuccess) return e;
     size_t smem = (size_t)I * (sizeof(int2) + (summaries_whole_numbers(ctx) ? 2 : 3) * sizeof(unsigned int));
-    if (I <= 32) smem += sizeof(uint2) + (size_t)I * 32 * (sizeof(uint2) + sizeof(unsigned int));      // (the rows' cells)
+    if (I <= RS_SELF_ROWS) smem += sizeof(uint2) + (size_t)I * 32 * (sizeof(uint2) + sizeof(unsigned int));      // (the rows' cells)
     if (smem + attr.sharedSizeBytes + 256 > limit) return cudaSuccess;   // too many instances
     // (the limit is shared by every context of the process: always the device maximum)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(limit - attr.sharedSizeBytes));

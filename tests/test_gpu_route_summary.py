@@ -570,3 +570,18 @@ def test_arrivals_on_far_rows_do_not_take_a_look_at_all_rows(beta, whole):
     """Some 0.4 of the scanning kernel's time where a far row that wins is compared among the list's rows, 0.7 and more where each such
     arrival takes a look at all rows."""
     assert share_of_the_scanning_time(*skewed(1054, 228, 35, 817, beta, whole)) < 0.6
+
+
+@pytest.mark.parametrize("n_inst", [4, 5, 20, 32, 33])
+@pytest.mark.parametrize("beta,whole", [(1.0, True), (0.75, False)])
+def test_small_services_with_a_long_backlog(n_inst, beta, whole):
+    """Both sides of the rule that leaves the folds to the deciding warp, and of that for exact keys."""
+    wl, ap, ad = skewed(n_inst, 57, 32, 900, beta, whole)
+    route_and_compare(wl, ap, ad, batches=2)
+
+
+@pytest.mark.parametrize("n_inst", [20, 32])
+@pytest.mark.parametrize("beta,whole", [(1.0, True), (0.75, False)])
+def test_backlogs_of_small_services_are_folded_by_the_folding_warps(n_inst, beta, whole):
+    """Less than a tenth of the scanning kernel's time; 0.13 to 0.17 with every fold made by the deciding warp itself."""
+    assert share_of_the_scanning_time(*skewed(n_inst, 256, 128, 2000, beta, whole)) < 0.12

@@ -78,7 +78,7 @@ def test_admission_router_wait_that_runs_out():
 
 
 # (instances, steps, beta): all rows held by the deciding warp, in one launch and in three; lists; binary64 scores
-SUMMARY_SHAPES = [(8, 64, 1.0), (200, 96, 1.0), (600, 64, 1.0), (2100, 40, 1.0), (40, 700, 0.75), (600, 64, 0.75)]
+SUMMARY_SHAPES = [(3, 64, 1.0), (8, 64, 1.0), (200, 96, 1.0), (600, 64, 1.0), (2100, 40, 1.0), (40, 700, 0.75), (600, 64, 0.75)]
 
 
 def summary_case(n_inst, h, beta, seed):
