@@ -126,7 +126,7 @@ int pre_create(const pre_config* cfg, pre_ctx** out) {
     if (e == cudaSuccess) e = pre_route_configure(c);
     if (e == cudaSuccess) e = alloc_zero(&c->d_slots, (size_t)32 * c->route_blocks);
     if (e == cudaSuccess) e = pre_route_summary_configure(c);
-    if (e == cudaSuccess) e = alloc_zero(&c->d_rs_guard, 8);
+    if (e == cudaSuccess) e = alloc_zero(&c->d_rs_guard, 9);
     if (e == cudaSuccess) e = alloc_zero(&c->d_rs_handled, 1);
     if (e == cudaSuccess && c->route_summary_smem) {
         e = alloc_zero(&c->d_rs_summary, (size_t)2 * I);

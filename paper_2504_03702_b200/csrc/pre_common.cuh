@@ -79,7 +79,7 @@ struct pre_ctx {
     unsigned char* d_rs_applied;    // [max_requests] 1: the map has this request of the batch already (zero between calls)
     long long* d_rs_ramps;          // {first table row, rows} whose ramps the maps lack after the routing kernel
     int32_t* d_rs_over;             // [I] steps of a row above the overload level (admission queue)
-    unsigned long long* d_rs_guard; // [8] what the summarising kernel found (largest cell, totals of the batch, ...; zero between calls)
+    unsigned long long* d_rs_guard; // [9] what the summarising kernel found (largest cell, totals of the batch, ...; zero between calls)
     int* d_rs_handled;              // 1 when the summary kernel routed the last batch, 0 when it left it to the scanning kernel
 };
 

@@ -72,6 +72,13 @@ constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding war
 // And keys in units of more than so many tokens (beta of thousands): 1,024 x 1,024, beta 1,000.5 (16 tokens) 1.5 us an arrival, 100,000.5
 // (2,048 tokens) 9.5, the scanning kernel 2.5.
 constexpr int RS_COARSE_SHIFT = -6;
+// Exact keys have a unit of their own, rounded ones the batch's.  A batch is routed with rounded keys where one arrival in RS_LONG_SHARE does not fit the
+// exact ones (it is decided outside the loop, on all rows), or where one row in RS_BEYOND_SHARE will be far by its top alone when half of the batch is
+// routed (RS_HALVES).  Lists of 256 rows become lists of 128, whose keys have a bit more (whole-number scores: exact ones still).  us a call, 2,048
+// arrivals on 512 steps, exact / rounded: beta = 0.75, prompts to 131,072 (median 16,384), 50, 200 and 600 rows 1,258 / 306, 1,396 / 367, 694 / 343;
+// (median 300, a long tail) 2,362 / 432, 6,604 / 631, 4,919 / 762; beta = 100, prompts to 8,192, 200 rows 741 / 599.
+constexpr unsigned long long RS_LONG_SHARE = 32;
+constexpr int RS_BEYOND_SHARE = 8;
 constexpr int RS_FAR_SHARE = 3, RS_FAR_STEPS = 256;     // one row in so many, maps of more steps than that
 constexpr int RS_PROBES = 8;                // prompt lengths for which a list has the best rows
 constexpr int RS_NEAR = 64;                 // steps kept exactly; the rest in 32 stretches of whole chunks of as many steps
@@ -94,7 +101,7 @@ constexpr unsigned int FULL_MASK = 0xffffffffu;
 
 // guard words written by the summarising kernel; the routing kernel clears them for the next call
 constexpr int GUARD_MAX_CELL = 0, GUARD_MAX_BASE = 1, GUARD_BAD = 2, GUARD_SUM_RAMP = 3, GUARD_SUM_TOKENS = 4,
-              GUARD_MAX_PD = 5, GUARD_SUM_BASE = 6, GUARD_MAX_P = 7, GUARDS = 8;
+              GUARD_MAX_PD = 5, GUARD_SUM_BASE = 6, GUARD_MAX_P = 7, GUARD_LONG = 8, GUARDS = 9;
 
 // What a warp finds out about a row in one pass: lane l has cells 2l and 2l+1 of the first 64 and the largest c[j] + j of
 // stretch l (0: no such stretch).
@@ -240,6 +247,7 @@ struct SumArgs {
     const int32_t* queue_predicted;
     const int64_t* queue_state;    // {head, length}
     long long queue_capacity;
+    float long_p, long_d;          // an arrival with P * long_p + D * long_d > 1 is long: it does not fit the exact keys (see Held; 0: rounded keys)
 };
 
 // The largest c[j] + j of the steps below RS_LIMIT, from the first cells, and the step at which it is first taken.
@@ -255,13 +263,14 @@ __device__ __forceinline__ unsigned int first_top(unsigned int near0, unsigned i
 template <typename Args>
 __device__ __forceinline__ void batch_totals(const Args& a, long long first, long long stride, unsigned long long* guard) {
     unsigned long long ramp = 0, tokens = 0;
-    unsigned int max_pd = 0, max_p = 0;
+    unsigned int max_pd = 0, max_p = 0, n_long = 0;
     auto count = [&](int P, int D) {
         if (P < 0 || D < 1 || P > PRE_FIELD_MAX || D > PRE_FIELD_MAX) return;
         ramp += (unsigned long long)P + (unsigned long long)(D < a.H ? D : a.H);
         tokens += (unsigned long long)P + (unsigned long long)D;
         max_pd = max(max_pd, (unsigned int)P + (unsigned int)D);
         max_p = max(max_p, (unsigned int)P);
+        n_long += (float)P * a.long_p + (float)D * a.long_d > 1.0f;
     };
     for (long long k = first; k < a.n_arrivals; k += stride)
         count(a.arr_prompt[k], a.arr_predicted[k]);
@@ -282,11 +291,13 @@ __device__ __forceinline__ void batch_totals(const Args& a, long long first, lon
     }
     max_pd = __reduce_max_sync(FULL_MASK, max_pd);
     max_p = __reduce_max_sync(FULL_MASK, max_p);
+    n_long = __reduce_add_sync(FULL_MASK, n_long);
     if ((threadIdx.x & 31) == 0 && (ramp | tokens)) {
         atomicAdd(guard + GUARD_SUM_RAMP, ramp);
         atomicAdd(guard + GUARD_SUM_TOKENS, tokens);
         atomicMax(guard + GUARD_MAX_PD, (unsigned long long)max_pd);
         atomicMax(guard + GUARD_MAX_P, (unsigned long long)max_p);
+        if (n_long) atomicAdd(guard + GUARD_LONG, (unsigned long long)n_long);
     }
 }
 
@@ -338,7 +349,7 @@ __global__ void __launch_bounds__(SUM_THREADS) pre_summarise_rows(const SumArgs 
         const unsigned long long v = sh_guard[tid];
         if (v) {
             if (tid == GUARD_BAD) atomicOr(a.guard + tid, v);
-            else if (tid == GUARD_SUM_RAMP || tid == GUARD_SUM_TOKENS || tid == GUARD_SUM_BASE) atomicAdd(a.guard + tid, v);
+            else if (tid == GUARD_SUM_RAMP || tid == GUARD_SUM_TOKENS || tid == GUARD_SUM_BASE || tid == GUARD_LONG) atomicAdd(a.guard + tid, v);
             else atomicMax(a.guard + tid, v);
         }
     }
@@ -386,6 +397,7 @@ struct RouteSumArgs {
     long long hot;                 // floor(overload_level * M): a cell counts when it is above
     double many;                   // overload_share * H: overloaded when more cells than this count
     const int32_t* over0;          // [I] steps above the level per row, from the summarising kernel
+    float long_p, long_d;          // as in SumArgs
 };
 
 // What the deciding warp can ask of the folding warps: the peaks of some rows, or a look at all rows.
@@ -439,7 +451,7 @@ struct RsShared {
     int look_row[2][RS_MAX_FOLD_WARPS];                    // the row that has it
     unsigned int look_peak[2][RS_MAX_FOLD_WARPS];          // and its peak
     unsigned int jmax;                      // largest step that a row's b stands for
-    unsigned int n_far, n_least;            // when the batch begins: far rows, rows with the smallest score for an empty prompt
+    unsigned int n_far, n_least, n_beyond;  // when the batch begins: far rows, rows with the smallest score for an empty prompt, rows that would be far by their tops alone
     unsigned int items_ready;               // items written so far
     unsigned int items_end;                 // 1: there will be no more
     unsigned int written;                   // results written so far
@@ -2120,105 +2132,22 @@ __device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const
     return sh.items_ready > told ? sh.item_at[told % RS_ITEMS] : sh.cursor;
 }
 
+// The batch by the block's warps, with the keys of KIND.  False: left to the scanning kernel.
+struct Batch {
+    unsigned long long peak_bound, ramps, tokens_in, max_pd, max_p, base_sum;
+    long long q_head, q_len, n_items;
+    bool alone;
+};
 template <int KS, bool LISTS, bool ADMIT, int KIND>
-__global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summaries(const __grid_constant__ RouteSumArgs a) {
+__device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Cells& cells, const Batch& b, long long& decided) {
     typedef Shape<KS, LISTS> Sp;
     constexpr int THREADS = Sp::THREADS;
-    extern __shared__ __align__(16) unsigned char rs_smem[];
-    __shared__ __align__(16) RsShared sh;
-    const int I = a.I, H = a.H;
-    Rows rows;
-    rows.rec = reinterpret_cast<int2*>(rs_smem);
-    rows.state = reinterpret_cast<unsigned int*>(rows.rec + I);
-    rows.top = rows.state + I;
-    rows.tok = rows.top + I;     // (binary64 scores only)
-    Cells cells{a.near, a.far};
-    if (Sp::SELF) {
-        cells.near = reinterpret_cast<uint2*>(rows.tok + (Scores<KIND>::WHOLE ? 0 : I + (I & 1)));
-        cells.far = reinterpret_cast<unsigned int*>(cells.near + 32 * I);
-    }
-
-    // (the warp's number by a shuffle: the compiler then knows that the roles part between warps and not within one, and
-    // leaves out what would bring the lanes of a warp together again: 157 instead of 202 cycles for a step of the deciding warp)
-    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(FULL_MASK, tid >> 5, 0);
-    __shared__ unsigned long long sh_guard[GUARDS];
-    const bool alone = !LISTS && a.alone;
-    if (!alone) pre_wait_for_previous();
-    if (alone) {     // small shapes: what pre_summarise_rows does (kept in the rows' words until the keys' units are known)
-        if (tid < GUARDS) sh_guard[tid] = 0;
-        __syncthreads();
-        for (int i = warp; i < I; i += Sp::WARPS)
-            summarise_row(a, i, cells.near, cells.far, sh_guard, [&](const uint4& q, int above) {
-                rows.rec[i] = make_int2((int)q.x, (int)q.w);
-                rows.top[i] = q.y;
-                rows.state[i] = q.z;
-                sh.pending[i] = (unsigned int)above;
-            });
-        batch_totals(a, tid, THREADS, sh_guard);
-        __syncthreads();
-    }
-    const unsigned long long* guard = alone ? sh_guard : a.guard;
-    const unsigned long long mc = guard[GUARD_MAX_CELL], mb = guard[GUARD_MAX_BASE], ramps = guard[GUARD_SUM_RAMP],
-                             tokens_in = guard[GUARD_SUM_TOKENS], max_pd = guard[GUARD_MAX_PD], max_p = guard[GUARD_MAX_P], base_sum = guard[GUARD_SUM_BASE];
-    // every cell, every cell + step with a prompt added, and every token count stay below 2^32 all batch long
-    // (the ramps of the batch bound what an arrival that is not routed yet can add, too)
-    const unsigned long long peak_bound = mc + ramps + (unsigned long long)H;
-    if (tid == 0) {
-        const unsigned long long token_bound = mb + tokens_in;
-        // (and the batch is short enough for 32-bit counters)
-        const bool ok = guard[GUARD_BAD] == 0 && peak_bound <= 0xffffffffull && token_bound <= 0xffffffffull &&
-                        a.n_arrivals + (ADMIT ? a.queue_capacity : 0) < (1ll << 26);
-        // (whole-number scores: the host has seen to beta and theta)
-        const bool exact = !Scores<KIND>::WHOLE || token_bound + max_pd + (unsigned long long)a.beta * (peak_bound + 1) < (1ull << 29);
-        sh.mode = ok && exact ? 1 : 0;
-        sh.spin_limit = a.spin_limit;
-        sh.idle_limit = max(a.spin_limit < (1u << 27) ? 16u * a.spin_limit : 0xffffffffu, 1u << 22);
-        sh.cursor = 0; sh.beat = 0;
-        sh.n0 = *a.n_requests;
-        sh.ctl = make_uint4(0u, 0u, 0u, 0u);
-        sh.items_ready = sh.items_end = sh.not_over = sh.jmax = sh.n_far = sh.n_least = sh.written = sh.flush = 0;
-        sh.lists_wanted = sh.lists_ready = sh.look_met = 0;
-        sh.list_n[0] = sh.list_n[1] = 0;
-        sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0;
-        sh.first_bad = sh.first_full = 0x7fffffff;
-    }
-    for (int i = tid; i < RS_ITEMS + RS_AHEAD; i += THREADS) sh.items[i] = make_int4(0, 0, 0, 0);    // (an item is fetched before it is known to be there)
-    if (tid < RS_MAX_FOLD_WARPS) { sh.done[tid] = (unsigned int)tid; sh.looks_done[tid] = 0; }
-    if (tid < RS_PROBES) sh.probe_t[tid] = 0xffffffffu;
-    if (tid < 32) { sh.bucket_a[tid] = 0xffffffffu; sh.bucket_b[tid] = 0xffffffffu; }
-    if (!alone)
-        for (int i = tid; i < RS_LIST_ROWS; i += THREADS) sh.pending[i] = 0;
-    // ADMIT: the requests that were waiting when the call was made come first, then the arrivals
-    long long q_head = 0, q_len = 0;
-    if (ADMIT && a.queue_capacity > 0) {
-        q_head = a.queue_state[0];
-        q_len = a.queue_state[1];
-    }
-    __syncthreads();
-    if (tid < GUARDS && !alone) a.guard[tid] = 0;    // ready for the next call
-    const int mode = __shfl_sync(FULL_MASK, sh.mode, 0);     // (all threads alike, and known to be)
-    auto decline = [&]() {
-        if (tid == 0) {
-            *a.handled = 0;
-            if (ADMIT) { a.queue_entry[0] = a.queue_state[0]; a.queue_entry[1] = a.queue_state[1]; }
-        }
-        if (tid < 3) a.give_up[tid] = 0;
-    };
-    if (mode == 0 && !alone) { decline(); return; }
-    if (ADMIT && a.queue_capacity > 0) {   // kept inside the ring whatever the two words hold
-        if (q_head < 0 || q_head >= a.queue_capacity) q_head = 0;
-        if (q_len < 0) q_len = 0;
-        if (q_len > a.queue_capacity) q_len = a.queue_capacity;
-    }
-    const long long n_items = q_len + a.n_arrivals;
-    long long decided = n_items;     // items from here on were not decided
-    if (mode == 0) {
-        rs_literal<ADMIT>(a, sh, q_head, q_len, n_items);
-    } else {
-    const unsigned long long mean_l = ramps / (unsigned long long)(n_items > 0 ? n_items : 1);
+    const int I = a.I, H = a.H, tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(FULL_MASK, tid >> 5, 0);
+    const bool alone = b.alone;
+    const unsigned long long mean_l = b.ramps / (unsigned long long)(b.n_items > 0 ? b.n_items : 1);
     const int mean = mean_l < (1ull << 22) ? (int)mean_l : 1 << 22;     // prompt + ramp of a typical request
     Scores<KIND> sc;
-    sc.start(a.theta, a.beta, peak_bound, max_pd, max_p, (base_sum + tokens_in) / (unsigned long long)I, mean, Held<KS>::ITEM);
+    sc.start(a.theta, a.beta, b.peak_bound, b.max_pd, b.max_p, (b.base_sum + b.tokens_in) / (unsigned long long)I, mean, Held<KS>::ITEM);
     {
         unsigned int jmax = 0, n_far = 0;
         int free_rows = 0;
@@ -2278,7 +2207,7 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
         n_least = __reduce_add_sync(FULL_MASK, n_least);
         if (lane == 0 && n_least) atomicAdd(&sh.n_least, n_least);
         __syncthreads();
-        if ((H > RS_FAR_STEPS && sh.n_far > (unsigned int)(I / RS_FAR_SHARE)) || sh.n_least > 32u * KS || sc.shift < RS_COARSE_SHIFT) { decline(); return; }
+        if ((H > RS_FAR_STEPS && sh.n_far > (unsigned int)(I / RS_FAR_SHARE)) || sh.n_least > 32u * KS || sc.shift < RS_COARSE_SHIFT) return false;
     }
 
     const int role = (warp >> 2) * 3 + (warp & 3) - 1;      // (of the warps that are not on the deciding warp's scheduler)
@@ -2287,14 +2216,137 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
     } else if ((warp & 3) != 0) {
         if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, KIND, LISTS, Sp::SELF>(a, sh, rows, sc, cells, role);
         else if (role == Sp::FOLD)
-            rs_io_loop<KS, Sp::DONE, ADMIT, KIND>(a, sh, sc, q_head, (int)q_len, (int)n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
+            rs_io_loop<KS, Sp::DONE, ADMIT, KIND>(a, sh, sc, b.q_head, (int)b.q_len, (int)b.n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
         else if (LISTS && role <= Sp::FOLD + Sp::LIST)
-            rs_list_loop<LISTS ? Sp::LIST : 4, KS, KIND>(sh, rows, sc, a.near, a.far, I, mean, sc.key_p(max_pd < (1ull << 29) ? (int)max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
+            rs_list_loop<LISTS ? Sp::LIST : 4, KS, KIND>(sh, rows, sc, a.near, a.far, I, mean, sc.key_p(b.max_pd < (1ull << 29) ? (int)b.max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
     }
     __syncthreads();
     if (sh.ctl.w) {     // (all threads alike: nobody writes it any more)
-        decided = rs_settle<Sp::DONE, LISTS, ADMIT, KIND>(a, sh, rows, sc, (int)q_len);
+        decided = rs_settle<Sp::DONE, LISTS, ADMIT, KIND>(a, sh, rows, sc, (int)b.q_len);
         __syncthreads();
+    }
+    return true;
+}
+
+template <int KS, bool LISTS, bool ADMIT, int KIND>
+__global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summaries(const __grid_constant__ RouteSumArgs a) {
+    typedef Shape<KS, LISTS> Sp;
+    constexpr int THREADS = Sp::THREADS;
+    extern __shared__ __align__(16) unsigned char rs_smem[];
+    __shared__ __align__(16) RsShared sh;
+    const int I = a.I, H = a.H;
+    Rows rows;
+    rows.rec = reinterpret_cast<int2*>(rs_smem);
+    rows.state = reinterpret_cast<unsigned int*>(rows.rec + I);
+    rows.top = rows.state + I;
+    rows.tok = rows.top + I;     // (not for whole-number scores beyond RS_MAX_BINARY64_ROWS instances)
+    Cells cells{a.near, a.far};
+    if (Sp::SELF) {
+        cells.near = reinterpret_cast<uint2*>(rows.tok + I + (I & 1));
+        cells.far = reinterpret_cast<unsigned int*>(cells.near + 32 * I);
+    }
+
+    // (the warp's number by a shuffle: the compiler then knows that the roles part between warps and not within one, and
+    // leaves out what would bring the lanes of a warp together again: 157 instead of 202 cycles for a step of the deciding warp)
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(FULL_MASK, tid >> 5, 0);
+    __shared__ unsigned long long sh_guard[GUARDS];
+    const bool alone = !LISTS && a.alone;
+    if (!alone) pre_wait_for_previous();
+    if (alone) {     // small shapes: what pre_summarise_rows does (kept in the rows' words until the keys' units are known)
+        if (tid < GUARDS) sh_guard[tid] = 0;
+        __syncthreads();
+        for (int i = warp; i < I; i += Sp::WARPS)
+            summarise_row(a, i, cells.near, cells.far, sh_guard, [&](const uint4& q, int above) {
+                rows.rec[i] = make_int2((int)q.x, (int)q.w);
+                rows.top[i] = q.y;
+                rows.state[i] = q.z;
+                sh.pending[i] = (unsigned int)above;
+            });
+        batch_totals(a, tid, THREADS, sh_guard);
+        __syncthreads();
+    }
+    const unsigned long long* guard = alone ? sh_guard : a.guard;
+    const unsigned long long mc = guard[GUARD_MAX_CELL], mb = guard[GUARD_MAX_BASE], ramps = guard[GUARD_SUM_RAMP],
+                             tokens_in = guard[GUARD_SUM_TOKENS], max_pd = guard[GUARD_MAX_PD], max_p = guard[GUARD_MAX_P], base_sum = guard[GUARD_SUM_BASE], n_long = guard[GUARD_LONG];
+    // every cell, every cell + step with a prompt added, and every token count stay below 2^32 all batch long
+    // (the ramps of the batch bound what an arrival that is not routed yet can add, too)
+    const unsigned long long peak_bound = mc + ramps + (unsigned long long)H;
+    if (tid == 0) {
+        const unsigned long long token_bound = mb + tokens_in;
+        // (and the batch is short enough for 32-bit counters)
+        const bool ok = guard[GUARD_BAD] == 0 && peak_bound <= 0xffffffffull && token_bound <= 0xffffffffull &&
+                        a.n_arrivals + (ADMIT ? a.queue_capacity : 0) < (1ll << 26);
+        // (whole-number scores: the host has seen to beta and theta)
+        const bool exact = !Scores<KIND>::WHOLE || token_bound + max_pd + (unsigned long long)a.beta * (peak_bound + 1) < (1ull << 29);
+        sh.mode = ok && exact ? 1 : 0;
+        sh.spin_limit = a.spin_limit;
+        sh.idle_limit = max(a.spin_limit < (1u << 27) ? 16u * a.spin_limit : 0xffffffffu, 1u << 22);
+        sh.cursor = 0; sh.beat = 0;
+        sh.n0 = *a.n_requests;
+        sh.ctl = make_uint4(0u, 0u, 0u, 0u);
+        sh.items_ready = sh.items_end = sh.not_over = sh.jmax = sh.n_far = sh.n_least = sh.n_beyond = sh.written = sh.flush = 0;
+        sh.lists_wanted = sh.lists_ready = sh.look_met = 0;
+        sh.list_n[0] = sh.list_n[1] = 0;
+        sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0;
+        sh.first_bad = sh.first_full = 0x7fffffff;
+    }
+    for (int i = tid; i < RS_ITEMS + RS_AHEAD; i += THREADS) sh.items[i] = make_int4(0, 0, 0, 0);    // (an item is fetched before it is known to be there)
+    if (tid < RS_MAX_FOLD_WARPS) { sh.done[tid] = (unsigned int)tid; sh.looks_done[tid] = 0; }
+    if (tid < RS_PROBES) sh.probe_t[tid] = 0xffffffffu;
+    if (tid < 32) { sh.bucket_a[tid] = 0xffffffffu; sh.bucket_b[tid] = 0xffffffffu; }
+    if (!alone)
+        for (int i = tid; i < RS_LIST_ROWS; i += THREADS) sh.pending[i] = 0;
+    // ADMIT: the requests that were waiting when the call was made come first, then the arrivals
+    long long q_head = 0, q_len = 0;
+    if (ADMIT && a.queue_capacity > 0) {
+        q_head = a.queue_state[0];
+        q_len = a.queue_state[1];
+    }
+    __syncthreads();
+    if (tid < GUARDS && !alone) a.guard[tid] = 0;    // ready for the next call
+    const int mode = __shfl_sync(FULL_MASK, sh.mode, 0);     // (all threads alike, and known to be)
+    auto decline = [&]() {
+        if (tid == 0) {
+            *a.handled = 0;
+            if (ADMIT) { a.queue_entry[0] = a.queue_state[0]; a.queue_entry[1] = a.queue_state[1]; }
+        }
+        if (tid < 3) a.give_up[tid] = 0;
+    };
+    if (mode == 0 && !alone) { decline(); return; }
+    if (ADMIT && a.queue_capacity > 0) {   // kept inside the ring whatever the two words hold
+        if (q_head < 0 || q_head >= a.queue_capacity) q_head = 0;
+        if (q_len < 0) q_len = 0;
+        if (q_len > a.queue_capacity) q_len = a.queue_capacity;
+    }
+    const long long n_items = q_len + a.n_arrivals;
+    long long decided = n_items;     // items from here on were not decided
+    if (mode == 0) {
+        rs_literal<ADMIT>(a, sh, q_head, q_len, n_items);
+    } else {
+    // Which keys: exact ones while the batch fits them (see RS_LONG_SHARE).
+    constexpr int OTHER_KS = LISTS && KS == 8 ? 4 : KS, OTHER = KIND == RS_WHOLE && OTHER_KS != KS ? RS_WHOLE : RS_ROUNDED;
+    static_assert(Shape<OTHER_KS, LISTS>::THREADS == THREADS, "");
+    bool exact = true;
+    if (KIND != RS_ROUNDED && (KIND == RS_HALVES || OTHER == RS_WHOLE || I <= RS_MAX_BINARY64_ROWS)) {
+        exact = n_long <= (unsigned long long)n_items / RS_LONG_SHARE;
+        if (KIND == RS_HALVES) {
+            Scores<KIND> sc;
+            sc.start(a.theta, a.beta, peak_bound, max_pd, max_p, 0ull, 1, Held<KS>::ITEM);
+            const unsigned long long rise = ramps / (2ull * (unsigned long long)I);       // of a row's top until half of the batch is routed
+            unsigned int n_beyond = 0;
+            for (int i = tid; i < I; i += THREADS) n_beyond += (alone ? rows.top[i] : a.summary0[i].y) + rise >= sc.far_top;
+            n_beyond = __reduce_add_sync(FULL_MASK, n_beyond);
+            if (lane == 0 && n_beyond) atomicAdd(&sh.n_beyond, n_beyond);
+            __syncthreads();
+            exact = exact && sh.n_beyond <= (unsigned int)(I / RS_BEYOND_SHARE);
+        }
+        exact = __shfl_sync(FULL_MASK, (int)exact, 0) != 0;     // (all threads alike, and known to be)
+    }
+    const Batch b{peak_bound, ramps, tokens_in, max_pd, max_p, base_sum, q_head, q_len, n_items, alone};
+    if (exact ? !rs_route<KS, LISTS, ADMIT, KIND>(a, sh, rows, cells, b, decided)
+              : !rs_route<KIND == RS_ROUNDED ? KS : OTHER_KS, LISTS, ADMIT, OTHER>(a, sh, rows, cells, b, decided)) {
+        decline();
+        return;
     }
     }
     const bool blocked = ADMIT && sh.blocked, dropped = !blocked && decided < n_items;
@@ -2415,6 +2467,17 @@ static const void* summaries_kernel(int I) {
     if (I <= RS_LONG_LISTS) return (const void*)pre_route_summaries<4, true, ADMIT, KIND>;
     return (const void*)pre_route_summaries<8, true, ADMIT, KIND>;
 }
+// What a token of the prompt and of the response adds to exact keys, as a share of Held::ITEM of the kernel chosen above (0: rounded keys).
+static void summaries_long(const pre_ctx* ctx, float& long_p, float& long_d) {
+    const int I = ctx->cfg.n_instances;
+    const int slot_bits = I <= RS_SELF_ROWS ? 5 : I <= 64 ? 6 : I <= 128 ? 7 : I <= RS_DIRECT_ROWS ? 8 : I <= RS_LONG_LISTS ? 7 : 8;
+    double unit = 0.0;
+    if (summaries_whole_numbers(ctx)) unit = 1.0;
+    else if (summaries_halves(ctx))
+        for (unit = 2.0; ctx->cfg.beta * unit != 2.0 * floor(0.5 * ctx->cfg.beta * unit);) unit *= 2.0;
+    long_d = (float)(2.0 * unit / (double)(1 << (28 - slot_bits)));
+    long_p = (float)((1.0 + ctx->cfg.beta) * 2.0 * unit / (double)(1 << (28 - slot_bits)));
+}
 template <bool ADMIT>
 static const void* summaries_kernel_for(const pre_ctx* ctx) {
     const int I = ctx->cfg.n_instances;
@@ -2431,7 +2494,7 @@ static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* s
     cudaFuncAttributes attr;
     cudaError_t e = cudaFuncGetAttributes(&attr, fn);
     if (e != cudaSuccess) return e;
-    size_t smem = (size_t)I * (sizeof(int2) + (summaries_whole_numbers(ctx) ? 2 : 3) * sizeof(unsigned int));
+    size_t smem = (size_t)I * (sizeof(int2) + (I > RS_MAX_BINARY64_ROWS ? 2 : 3) * sizeof(unsigned int));
     if (I <= RS_SELF_ROWS) smem += sizeof(uint2) + (size_t)I * 32 * (sizeof(uint2) + sizeof(unsigned int));      // (the rows' cells)
     if (smem + attr.sharedSizeBytes + 256 > limit) return cudaSuccess;   // too many instances
     // (the limit is shared by every context of the process: always the device maximum)
@@ -2496,6 +2559,8 @@ static void fill_summary_args(pre_ctx* ctx, SumArgs& p, RouteSumArgs& a, const i
     a.own_ramps = a.alone && (n_arrivals + queue_capacity) * (long long)H <= RS_OWN_RAMP_CELLS ? 1 : 0;
     a.queue_prompt = nullptr; a.queue_predicted = nullptr; a.queue_state = nullptr; a.queue_entry = nullptr;
     a.queue_capacity = 0; a.queue_choice = nullptr; a.hot = 0; a.many = 0.0; a.over0 = nullptr;
+    summaries_long(ctx, p.long_p, p.long_d);
+    a.long_p = p.long_p; a.long_d = p.long_d;
 }
 
 template <bool ADMIT>

@@ -585,3 +585,40 @@ def test_small_services_with_a_long_backlog(n_inst, beta, whole):
 def test_backlogs_of_small_services_are_folded_by_the_folding_warps(n_inst, beta, whole):
     """Less than a tenth of the scanning kernel's time; 0.13 to 0.17 with every fold made by the deciding warp itself."""
     assert share_of_the_scanning_time(*skewed(n_inst, 256, 128, 2000, beta, whole)) < 0.12
+
+
+def long_prompts(n_inst, n_arr, beta, whole, median, sigma, longest):
+    """Log-normal prompts up to `longest` on 512 steps, 64 requests per instance."""
+    n = 64 * n_inst
+    prompt, generated, predicted = W._lengths(79, n, median, sigma, 16, longest, 384, 1.2, 1, 4096, in_flight=True)
+    instance = W._uniform_instances(79, n, n_inst)
+    wl = W.make_random(79, n_inst, 512, 0, 0, beta=beta, capacity=W._capacity(prompt, generated, instance, n_inst) // 5 * 5 + (0 if whole else 3))
+    wl.prompt, wl.generated, wl.predicted, wl.instance = prompt, generated, predicted, instance
+    ap, _, ad = W._lengths(80, n_arr, median, sigma, 16, longest, 384, 1.2, 1, 4096, in_flight=False)
+    wl.max_requests = n + n_arr
+    return wl, ap, ad
+
+
+LONG = {"half of the prompts beyond exact keys": (0.75, False, 65536, 1.2, 131072), "peaks far beyond the threshold": (0.75, False, 300, 2.0, 131072),
+        "large penalty": (100.0, True, 1024, 1.2, 8192), "larger penalty": (700.0, True, 60, 1.2, 1500)}
+
+
+@pytest.mark.parametrize("kind", LONG)
+@pytest.mark.parametrize("n_inst", [3, 40, 100, 200, 300, 1100])
+def test_batches_that_do_not_fit_exact_keys(kind, n_inst):
+    """Whole-number scores and those of fractional thresholds, routed with rounded keys or a shorter list; and where few arrivals are too long, with exact ones."""
+    beta, whole, median, sigma, longest = LONG[kind]
+    wl, ap, ad = long_prompts(n_inst, 250, beta, whole, median, sigma, longest)
+    ap[::3] = np.minimum(ap[::3], 400)
+    route_and_compare(wl, ap, ad, batches=2)
+    few = np.minimum(ap, 300)
+    few[10::100] = longest
+    route_and_compare(wl, few, ad, batches=2)
+
+
+@pytest.mark.parametrize("n_inst,kind,limit", [(50, "peaks far beyond the threshold", 0.2), (100, "peaks far beyond the threshold", 0.2),
+                                               (200, "peaks far beyond the threshold", 0.3), (600, "peaks far beyond the threshold", 0.3),
+                                               (100, "half of the prompts beyond exact keys", 0.15), (2000, "large penalty", 0.2)])
+def test_batches_that_do_not_fit_exact_keys_are_not_decided_one_by_one_on_all_rows(n_inst, kind, limit):
+    """Two thirds of the limit or less; with exact keys (the arrivals that do not fit, or all rows that count as far, outside the loop) well above it."""
+    assert share_of_the_scanning_time(*long_prompts(n_inst, 2048, *LONG[kind])) < limit
