@@ -1371,7 +1371,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     typedef typename Scores<KIND>::S S;
     typedef Held<KS> K;
     constexpr int SLACK = Scores<KIND>::SLACK * (1 << K::SLOT_BITS);
-    // steps of a trip: decisions are made known to the folding warps by trips (few rows: soon)
+    // steps of a trip: decisions are made known to the folding warps by trips, under the next one's first reduction
     constexpr int TRIP = 4;
     // decisions between two looks at items and at the rows that were pending
     constexpr unsigned int CHUNK = LISTS ? 64 : 8 * KS;
@@ -1755,6 +1755,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         // ---- rows outside the list could do as well, or keys are cut: all rows, with every fold done
         if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return false; }
         acquire_cta();
+        refresh();      // (a row that several such arrivals go to in turn would gather their additions)
         if (LISTS) {
             int4 k;
             if (I <= RS_OWN_LOOK) k = look.template keys<32, 8>(0, P, D);
