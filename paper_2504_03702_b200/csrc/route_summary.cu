@@ -62,6 +62,8 @@ constexpr int RS_AHEAD = 8;                 // items that are fetched beyond the
 constexpr int RS_SELF_ROWS = 4;
 constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
 constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lane, 8 beyond RS_LONG_LISTS instances)
+// Lists of 256 / 128 rows, us a call, 8,192 arrivals on 1,024 steps: whole-number scores 1,025 rows 1,064 / 1,112, 1,600 1,005 / 1,095, 2,048 1,253 / 1,408;
+// fractional 1,153 / 1,168, 1,055 / 1,165, 1,328 / 1,464.
 constexpr int RS_LONG_LISTS = 1024;
 constexpr int RS_NEAR_ROWS = 2304;          // rows the list warps keep for a closer look at once
 constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding warp looks at their keys by itself
@@ -419,6 +421,11 @@ struct Rows {
     unsigned int* tok;
 };
 
+struct Batch {
+    unsigned long long peak_bound, ramps, tokens_in, max_pd, max_p, base_sum;
+    long long q_head, q_len, n_items;
+    bool alone;
+};
 struct RsShared {
     // what the deciding warp tells the folding warps and the io warp, read with one access
     uint4 ctl;                              // {decisions made, arrivals for all rows, 1: no more of either, 1: a wait was abandoned}
@@ -465,6 +472,7 @@ struct RsShared {
     int mode;                               // 0: decline the batch
     long long n0;
     int first_bad, first_full;              // the first items dropped as malformed / for a full table
+    Batch batch;                            // (for rs_route_apart)
     int warp_ok[32];                        // (the tail of ADMIT)
     long long joined;
     int any_bad;
@@ -2134,11 +2142,6 @@ __device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const
 }
 
 // The batch by the block's warps, with the keys of KIND.  False: left to the scanning kernel.
-struct Batch {
-    unsigned long long peak_bound, ramps, tokens_in, max_pd, max_p, base_sum;
-    long long q_head, q_len, n_items;
-    bool alone;
-};
 template <int KS, bool LISTS, bool ADMIT, int KIND>
 __device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Cells& cells, const Batch& b, long long& decided) {
     typedef Shape<KS, LISTS> Sp;
@@ -2229,23 +2232,48 @@ __device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, co
     return true;
 }
 
-template <int KS, bool LISTS, bool ADMIT, int KIND>
-__global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summaries(const __grid_constant__ RouteSumArgs a) {
-    typedef Shape<KS, LISTS> Sp;
-    constexpr int THREADS = Sp::THREADS;
-    extern __shared__ __align__(16) unsigned char rs_smem[];
+// What a block has in shared memory: the words of its warps, and behind each other the rows' (and, rows of the deciding warp alone, their cells).
+__device__ __forceinline__ RsShared& rs_block() {
     __shared__ __align__(16) RsShared sh;
-    const int I = a.I, H = a.H;
+    return sh;
+}
+__device__ __forceinline__ Rows rs_rows(int I) {
+    extern __shared__ __align__(16) unsigned char rs_smem[];
     Rows rows;
     rows.rec = reinterpret_cast<int2*>(rs_smem);
     rows.state = reinterpret_cast<unsigned int*>(rows.rec + I);
     rows.top = rows.state + I;
     rows.tok = rows.top + I;     // (not for whole-number scores beyond RS_MAX_BINARY64_ROWS instances)
+    return rows;
+}
+template <bool SELF>
+__device__ __forceinline__ Cells rs_cells(const RouteSumArgs& a, const Rows& rows) {
     Cells cells{a.near, a.far};
-    if (Sp::SELF) {
-        cells.near = reinterpret_cast<uint2*>(rows.tok + I + (I & 1));
-        cells.far = reinterpret_cast<unsigned int*>(cells.near + 32 * I);
+    if (SELF) {
+        cells.near = reinterpret_cast<uint2*>(rows.tok + a.I + (a.I & 1));
+        cells.far = reinterpret_cast<unsigned int*>(cells.near + 32 * a.I);
     }
+    return cells;
+}
+
+// The same with the keys that are not the kernel's usual ones, as a function of its own: in one with the usual way, that lost registers and took 4 % longer
+// (512 x 1,024 with the admission queue 1,205 -> 1,238 us).  -1: left to the scanning kernel.
+template <int KS, bool LISTS, bool ADMIT, int KIND>
+__device__ __noinline__ long long rs_route_apart(const RouteSumArgs& a) {
+    const Rows rows = rs_rows(a.I);
+    const Batch b = rs_block().batch;
+    long long decided = b.n_items;
+    return rs_route<KS, LISTS, ADMIT, KIND>(a, rs_block(), rows, rs_cells<Shape<KS, LISTS>::SELF>(a, rows), b, decided) ? decided : -1;
+}
+
+template <int KS, bool LISTS, bool ADMIT, int KIND>
+__global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summaries(const __grid_constant__ RouteSumArgs a) {
+    typedef Shape<KS, LISTS> Sp;
+    constexpr int THREADS = Sp::THREADS;
+    RsShared& sh = rs_block();
+    const int I = a.I, H = a.H;
+    const Rows rows = rs_rows(I);
+    const Cells cells = rs_cells<Sp::SELF>(a, rows);
 
     // (the warp's number by a shuffle: the compiler then knows that the roles part between warps and not within one, and
     // leaves out what would bring the lanes of a warp together again: 157 instead of 202 cycles for a step of the deciding warp)
@@ -2344,11 +2372,15 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
         exact = __shfl_sync(FULL_MASK, (int)exact, 0) != 0;     // (all threads alike, and known to be)
     }
     const Batch b{peak_bound, ramps, tokens_in, max_pd, max_p, base_sum, q_head, q_len, n_items, alone};
-    if (exact ? !rs_route<KS, LISTS, ADMIT, KIND>(a, sh, rows, cells, b, decided)
-              : !rs_route<KIND == RS_ROUNDED ? KS : OTHER_KS, LISTS, ADMIT, OTHER>(a, sh, rows, cells, b, decided)) {
-        decline();
-        return;
+    bool routed;
+    if (KIND == RS_ROUNDED || exact) routed = rs_route<KS, LISTS, ADMIT, KIND>(a, sh, rows, cells, b, decided);
+    else {
+        if (tid == 0) sh.batch = b;
+        __syncthreads();
+        decided = rs_route_apart<OTHER_KS, LISTS, ADMIT, OTHER>(a);
+        routed = decided >= 0;
     }
+    if (!routed) { decline(); return; }
     }
     const bool blocked = ADMIT && sh.blocked, dropped = !blocked && decided < n_items;
     if (blocked) decided = sh.blocked_k;
