@@ -44,10 +44,10 @@ METRIC_STREAM = "routes/sec over the whole stream (decode step + routing of the 
 ROUTE_DRAM_READ = {3: 67322880}
 # profiles/ncu_dram_route_summary_kernels_config3_full_batch.txt: the three kernels of the summary router on the full
 # batch (the traffic does not grow in proportion to the batch, so the figure is used for the full batch only)
-ROUTE_SUMMARY_DRAM_TRAFFIC = {(3, 65536): 67732992 + 165120 + 2322176 + 50707456 + 2891264}
-# warp instructions per arrival of pre_route_summaries; none of the present kernel have been captured (the capture in
-# profiles/ncu_full_step_kernels_config3_2048_arrivals.txt is of the kernel with two reductions per arrival)
-ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL = {}
+ROUTE_SUMMARY_DRAM_TRAFFIC = {(3, 65536): 67736576 + 381440 + 2255616 + 50708224 + 2829568}
+# warp instructions per arrival of pre_route_summaries (smsp__inst_executed.sum of the 2,048-arrival capture in
+# profiles/ncu_full_step_kernels_config3_2048_arrivals.txt: 987,740 / 2,048)
+ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL = {3: 987740 / 2048}
 ROUTE_DRAM_WRITE_PER_ARRIVAL = {3: 679168 / 256}
 ANTICIPATE_DRAM_TRAFFIC = {3: 33812992 + 19587328}
 STEP_DRAM_TRAFFIC = {3: 33670144 + 67196928 + 9366528}
@@ -674,7 +674,7 @@ def route_summary_roofline(wl, index, t_route_ms, n_arrivals, clocks):
         "us_per_arrival": sec * 1e6 / n_arrivals, "cycles_per_arrival": sec * mhz * 1e6 / n_arrivals,
         "scan_equivalent_gbs": literal / sec / 1e9,
         "hbm_frac_of_captured_traffic": None if traffic is None else traffic / sec / 1e9 / hbm_peak,
-        "limiter": "latency: arrivals are decided one after another by one warp (two warp reductions and some ten dependent "
+        "limiter": "latency: arrivals are decided one after another by one warp (one warp reduction and some eight dependent "
                    "instructions each); neither a memory nor the instruction issue is saturated",
         "note": "decisions are taken from two numbers per row instead of scanning the maps (identical decisions), by ONE block; "
                 "scan_equivalent_gbs is the literal formulation's 8 bytes per cell and arrival over time, a convenience "

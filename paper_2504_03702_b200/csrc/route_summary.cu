@@ -69,10 +69,10 @@ constexpr int RS_NEAR_ROWS = 2304;          // rows the list warps keep for a cl
 constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding warp looks at their keys by itself
 // Beyond RS_DIRECT_ROWS instances two kinds of batches cost this kernel more than the scanning one (which takes 2.4 us an arrival on 1,024 x
 // 1,024 whatever the rows): many far rows that may pay a penalty, whose arrivals need a look at all rows, scans, and folds of
-// whole rows (share of such rows, us: 28 % 2.0, 51 % 4.4, 58 % 5.4; with 512 x 40, 55 %, 1.3 against 2.3); and more rows that
+// whole rows (share of such rows, us: 16 % 1.7, 26 % 3.2, 39 % 3.9, 62 % 7.2; maps of 228 steps, 44 % 2.5, 68 % 5.1); and more rows that
 // share the smallest score than a list holds (empty services; 512 rows 2.7, 4,096 rows 42 against 3.1).
-// And keys in units of more than so many tokens (beta of thousands): 1,024 x 1,024, beta 1,000.5 (16 tokens) 1.5 us an arrival, 100,000.5
-// (2,048 tokens) 9.5, the scanning kernel 2.5.
+// And keys in units of more than 64 tokens (beta of thousands): 1,024 x 1,024, beta 1,000.5 (units of 4 tokens) 1.2 us an arrival, 100,000.5
+// (of 512) 10.4, the scanning kernel 2.4.
 constexpr int RS_COARSE_SHIFT = -6;
 // Exact keys have a unit of their own, rounded ones the batch's.  A batch is routed with rounded keys where one arrival in RS_LONG_SHARE does not fit the
 // exact ones (it is decided outside the loop, on all rows), or where one row in RS_BEYOND_SHARE will be far by its top alone when half of the batch is

@@ -580,11 +580,11 @@ def test_small_services_with_a_long_backlog(n_inst, beta, whole):
     route_and_compare(wl, ap, ad, batches=2)
 
 
-@pytest.mark.parametrize("n_inst", [20, 32])
 @pytest.mark.parametrize("beta,whole", [(1.0, True), (0.75, False)])
-def test_backlogs_of_small_services_are_folded_by_the_folding_warps(n_inst, beta, whole):
-    """Less than a tenth of the scanning kernel's time; 0.13 to 0.17 with every fold made by the deciding warp itself."""
-    assert share_of_the_scanning_time(*skewed(n_inst, 256, 128, 2000, beta, whole)) < 0.12
+def test_backlogs_of_small_services_are_folded_by_the_folding_warps(beta, whole):
+    """32 rows, 2,000 arrivals: 0.05 to 0.07 of the scanning kernel's time, 0.13 to 0.17 with every fold made by the deciding warp itself; the limit lies
+    half as much again above the one and below the other."""
+    assert share_of_the_scanning_time(*skewed(32, 256, 128, 2000, beta, whole)) < 0.1
 
 
 def long_prompts(n_inst, n_arr, beta, whole, median, sigma, longest):
