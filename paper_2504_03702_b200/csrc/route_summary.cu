@@ -1028,7 +1028,7 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
             if (lane == 0) st_release(&sh.done[me], n);
             __syncwarp();
         } else if (__any_sync(FULL_MASK, ctl.y != looks)) {
-            looks = ctl.y;
+            looks = __reduce_max_sync(FULL_MASK, ctl.y);      // (the lanes need not have loaded it at the same time)
             const int how = sh.look_how;
             if (!LISTS && how == RS_SCANS) {
                 const int P = sh.look_P, Dc = sh.look_D < a.H ? sh.look_D : a.H, count = sh.scan_n;
@@ -1431,7 +1431,8 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             ra[k] = read ? key_a : ra[k];
             rb[k] = read ? key_b : rb[k];
         }
-        jmax = (int)ld_volatile(&sh.jmax);    // (after the rows were read)
+        // (after the rows were read; the lanes take the same ways by it, and nothing makes them load it at the same time)
+        jmax = (int)__reduce_max_sync(FULL_MASK, ld_volatile(&sh.jmax));
     };
     auto held_pending = [&]() {
         unsigned int m = 0;
@@ -1562,7 +1563,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 const bool bounded = (key & 1) != 0;      // the best row is marked
                 if (bounded) {
                     const unsigned int* word = sh.pending + ((key & K::SLOT) >> 1);
-                    if (ld_acquire(word)) {
+                    if (__any_sync(FULL_MASK, ld_acquire(word) != 0)) {
                         if (!rs_wait(sh, [&] { return ld_acquire(word) == 0; })) lost = true;
                         return false;
                     }
