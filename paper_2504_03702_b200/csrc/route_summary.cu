@@ -56,6 +56,7 @@ constexpr int RS_MAX_FOLD_WARPS = 10;
 constexpr int RS_LIST_WARPS = 6;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
 constexpr int RS_AHEAD = 8;                 // items that are fetched beyond the present one, at most
+constexpr int RS_READY = 64;                // items made ready for the deciding loop at once, at most
 // Up to so many rows the deciding warp folds its decisions itself: with few rows the next arrival mostly wants the row that was just taken. us a call,
 // by itself / by the folding warps: 2,000 arrivals on 256 steps, whole-number scores, 1 row 846 / 1,796, 4 rows 575 / 647, 6 rows 618 / 565, 20 rows
 // 561 / 278; fractional 1,028 / 1,957, 755 / 720, 778 / 627, 738 / 341; 32 arrivals on 64 steps: 4 rows 33 / 37, 8 rows 34 / 34, 32 rows 37 / 35.
@@ -432,6 +433,8 @@ struct RsShared {
     int4 items[RS_ITEMS + RS_AHEAD];        // of the requests to route, in order: {what P adds to b, P + D as a key and the mark, min(D, H)
                                             // (0: not for the quick way), offset of P's entry in the table}; both keys as in Held; the first ones
                                             // once more behind the last
+    int4 ready[RS_READY + RS_AHEAD];        // (deciding warp) the next items as its loop takes them: {what P adds to b, what the item adds to a and the mark, the
+                                            // key that a row outside the list (or a case that is unusual) has at least, what the item adds to b}
     int2 raw[RS_ITEMS];                     // {P, D}
     int item_at[RS_ITEMS];                  // their indices in the batch
     uint2 jobs[RS_ITEMS];                   // decisions: {row, or until it is folded 2 * slot | list's parity << 16 | RS_BY_SLOT; RS_GIVEN if the peak is
@@ -1370,10 +1373,12 @@ template <int KS, bool LISTS> struct Shape {
 
 // ---- deciding warp.  KS: rows per lane.  LISTS: they are a list's, else all rows.
 // What bounds it: the latency of one chain of dependent instructions per arrival (a warp reduction, 23 cycles, and some eight integer
-// operations: 65 cycles with two rows per lane, in a kernel with nothing else) and, with four and eight rows per lane, the number of its
-// instructions (85 and 130).  In the kernel a step takes 85, 130 and 160 to 185 cycles.  So nothing else is in the loop: no branch (one per step cost 50 to 100 cycles; whether all steps were usual
-// is seen once per trip, which is taken back as far as they were not), items and bounds fetched two steps ahead, and what need not
-// be in the chain (scores, token counts, the tables) is done by the folding warps.
+// operations) and, with four and eight rows per lane, the number of its instructions (an integer instruction takes the warp two cycles): a step takes 52, 77 and
+// 113 cycles with two, four and eight rows per lane.  So nothing else is in the loop: no branch (whether all steps were usual is seen once per
+// trip, which is taken back as far as they were not; a branch around the telling of a trip's decisions cost 20 cycles a step), items with their bounds
+// made ready by all lanes for up to 64 at once (per step: 7 cycles), fetched two steps ahead, and what need not be in the chain (scores, token counts, the
+// tables) is done by the folding warps.
+// us a call with both, before and after: 256 x 100 149 -> 141, 512 x 1,024 425 -> 419, 2,000 x 1,536 580 -> 544.
 template <int KS, bool LISTS, int FOLD_WARPS, bool ADMIT, int KIND>
 __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<KIND>& sc, const Cells& cells) {
     typedef typename Scores<KIND>::S S;
@@ -1381,8 +1386,9 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     constexpr int SLACK = Scores<KIND>::SLACK * (1 << K::SLOT_BITS);
     // steps of a trip: decisions are made known to the folding warps by trips, under the next one's first reduction
     constexpr int TRIP = 4;
-    // decisions between two looks at items and at the rows that were pending
-    constexpr unsigned int CHUNK = LISTS ? 64 : 8 * KS;
+    // decisions between two looks at items and at the rows that were pending; items made ready at once (a trip may begin with the last but one of a
+    // chunk)
+    constexpr unsigned int READY = !LISTS && KS <= 4 ? 32 : RS_READY, CHUNK = !LISTS && KS == 2 ? 16 : READY - TRIP;
     const int lane = threadIdx.x & 31, I = a.I, H = a.H;
     constexpr bool SELF = Shape<KS, LISTS>::SELF;
     const int lane_f = lane < Shape<KS, LISTS>::DONE ? lane : 0;
@@ -1445,9 +1451,10 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         return __all_sync(FULL_MASK, (int)(ld_acquire(&sh.done[lane_f]) - e) >= 0);
     };
     const unsigned int at_pending = smem_u32(sh.pending), at_jobs = smem_u32(sh.jobs), at_items = smem_u32(sh.items);
+    const unsigned int at_ctl = smem_u32(&sh.ctl.x), at_ready = smem_u32(sh.ready);
     auto publish = [&](unsigned int n) {
         __syncwarp();
-        if (lane == 0) st_release(&sh.ctl.x, n);
+        asm volatile("{ .reg .pred p; setp.eq.s32 p, %0, 0; @p st.release.cta.shared.u32 [%1], %2; }" ::"r"(lane), "r"(at_ctl), "r"(n) : "memory");
     };
     unsigned int list = 0;           // the list held
     unsigned int table = smem_u32(sh.table[0]);
@@ -1792,19 +1799,21 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     };
 
     // ---- the usual way
-    int4 it0, it1, it2, ahead = make_int4(0, 0, 0, 0);     // items e, e + 1, e + 2, the bounds for item e + 1
-    int bound;                                             // for item e: the key that a row outside the list (or a case that is unusual) has at least
-    auto bound_for = [&](const int4& it, const int4& others) {
-        const int b = it.z > jmax ? cut : (int)0x80000001u;
-        return LISTS ? min(b, bound_of(others, it.x)) : b;
-    };
+    int4 it0, it1, it2;              // items e, e + 1, e + 2 (see RsShared::ready)
+    unsigned int first = 0;          // the first of the items made ready
     auto fetch = [&](unsigned int e) {
-        it0 = ld_table(at_items + 16u * (e % RS_ITEMS));
-        it1 = ld_table(at_items + 16u * ((e + 1) % RS_ITEMS));
-        it2 = ld_table(at_items + 16u * ((e + 2) % RS_ITEMS));
-        int4 now = ahead;
-        if (LISTS) { now = ld_table(table + it0.w); ahead = ld_table(table + it1.w); }
-        bound = bound_for(it0, now);
+        first = e;
+        __syncwarp();
+        #pragma unroll
+        for (unsigned int x = 0; x < READY; x += 32) {
+            const int4 it = ld_table(at_items + 16u * ((e + x + lane) % RS_ITEMS));
+            const int b = it.z > jmax ? cut : (int)0x80000001u;
+            sh.ready[x + lane] = make_int4(it.x, it.y, LISTS ? min(b, bound_of(ld_table(table + it.w), it.x)) : b, it.x + it.y);
+        }
+        __syncwarp();
+        it0 = ld_table(at_ready);
+        it1 = ld_table(at_ready + 16u);
+        it2 = ld_table(at_ready + 32u);
     };
     if constexpr (SELF) {
         // ---- up to RS_SELF_ROWS rows, one per lane: the deciding warp folds each decision itself, so that no row is ever pending.  What bounds it: the
@@ -1945,29 +1954,27 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         const unsigned int stop = min(limit, e + CHUNK);
         refresh();
         fetch(e);
-        unsigned int untold = 0;      // decisions before e that are not told yet (the last trip's: they are while the next reduction is under way)
+        int untold = 0;               // decisions before e that are not told yet (the last trip's: they are while the next reduction is under way)
         int told = 0;
         while (e < stop) {
             int was_a[KS], was_b[KS], key[TRIP], not_usual = 0;
-            const unsigned int at = at_items + 16u * (e % RS_ITEMS);
+            const unsigned int at = at_ready + 16u * (e - first);
             #pragma unroll
             for (int k = 0; k < KS; ++k) { was_a[k] = ra[k]; was_b[k] = rb[k]; }
             #pragma unroll
             for (int u = 0; u < TRIP; ++u) {     // (items from `limit` on are whatever the slots hold: what is done with them is taken back)
-                const int kp = it0.x, kpd = it0.y, kpb = kpd + kp;
+                const int kp = it0.x, kpd = it0.y, kpb = it0.w;
                 int v[KS];
                 #pragma unroll
                 for (int k = 0; k < KS; ++k) v[k] = __viaddmax_s32(rb[k], kp, ra[k]);
-                int least = bound;
+                int least = it0.z;
                 #pragma unroll
                 for (int k = 0; k + 1 < KS; k += 2) least = __vimin3_s32(least, v[k], v[k + 1]);
                 const int best = __reduce_min_sync(FULL_MASK, least);
                 // (while the reduction is under way)
-                if (u == 0 && untold) { tell(e - TRIP, told, TRIP); publish(e); }
+                if (u == 0) { tell(e - TRIP, told, untold); publish(e); }     // (whether there is anything to tell or not: a branch here cost 20 cycles a step)
                 it0 = it1; it1 = it2;
                 it2 = ld_table(at + 16u * (u + 3));
-                bound = bound_for(it0, ahead);
-                if (LISTS) ahead = ld_table(table + it1.w);
                 #pragma unroll
                 for (int k = 0; k < KS; ++k)
                     if (v[k] == best) { ra[k] += kpd; rb[k] += kpb; }
@@ -2005,7 +2012,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 #pragma unroll
                 for (int k = 0; k < KS; ++k) {
                     ra[k] += tag(k) == t ? it.y : 0;
-                    rb[k] += tag(k) == t ? it.y + it.x : 0;
+                    rb[k] += tag(k) == t ? it.w : 0;
                 }
             }
             tell(e, told, usual);
@@ -2016,12 +2023,12 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                     if (unusual(e)) { ++e; publish(e); }
                     else if (lost) break;
                     else refresh();
-                    fetch(e);
-                } while (e < stop && __any_sync(FULL_MASK, bound == (int)0x80000001u));
-            else fetch(e);
+                } while (e < stop && __any_sync(FULL_MASK, sh.items[e % RS_ITEMS].z <= jmax));
             if (lost) break;
+            fetch(e);
         }
-        if (untold) { tell(e - TRIP, told, TRIP); publish(e); }
+        tell(e - TRIP, told, untold);
+        publish(e);
     }
     }
     __syncwarp();
