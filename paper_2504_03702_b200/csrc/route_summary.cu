@@ -25,16 +25,17 @@
 //   pre_summarise_rows   one pass over the maps: the numbers of every row, the rows' token
 //                        counts (queued_p + current_d) and the guards that tell whether 32-bit
 //                        arithmetic stays exact for the whole batch;
-//   pre_route_summaries  routes the batch with ONE block whose warps have different jobs:
+//   pre_route_summaries  routes the batch with ONE block whose warps have different jobs, and beyond 256 instances a second one on another SM (a cluster of two):
 //     deciding warp  takes the arrivals one by one.  It holds rows in registers (two keys each), takes
 //                    every row's score for the arrival, the smallest and its row by one warp reduction, and updates the winner in
 //                    place: no other warp is in this chain.  Up to 256 instances it holds all rows.  Beyond, it holds
 //                    the at most 128 rows of a list (256 beyond RS_LONG_LISTS instances), and a table that bounds the scores of all other rows from
 //                    below: while the best row of the list beats that bound it is the best row of all.  Up to RS_SELF_ROWS instances
 //                    it folds its decisions itself.
-//     list warps     (beyond 256 instances) build the next list while the present one is being used up: the rows
+//     list block     (beyond 256 instances) builds the next list while the present one is being used up: the rows
 //                    whose score is within a margin of the smallest one for any of eight prompt lengths, and the
-//                    bounds of the rest.  Scores only grow during a batch, so a list that is a little behind is valid.
+//                    bounds of the rest.  Scores only grow during a batch, so a list that is a little behind is valid.  It reads the rows' keys in the routing
+//                    block's shared memory and writes the list there.
 //     folding warps  add each routed request to its row's numbers, one warp per request; they scan single rows for the
 //                    deciding warp, and decide an arrival on all rows together where the rows it holds leave it undecided;
 //     io warp        reads the arrivals ahead of the decisions and writes the results behind them.
@@ -53,7 +54,6 @@
 namespace {
 
 constexpr int RS_MAX_FOLD_WARPS = 10;
-constexpr int RS_LIST_WARPS = 6;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
 constexpr int RS_AHEAD = 8;                 // items that are fetched beyond the present one, at most
 constexpr int RS_READY = 64;                // items made ready for the deciding loop at once, at most
@@ -66,7 +66,6 @@ constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lan
 // Lists of 256 / 128 rows, us a call, 8,192 arrivals on 1,024 steps: whole-number scores 1,025 rows 1,064 / 1,112, 1,600 1,005 / 1,095, 2,048 1,253 / 1,408;
 // fractional 1,153 / 1,168, 1,055 / 1,165, 1,328 / 1,464.
 constexpr int RS_LONG_LISTS = 1024;
-constexpr int RS_NEAR_ROWS = 2304;          // rows the list warps keep for a closer look at once
 constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding warp looks at their keys by itself
 // Beyond RS_DIRECT_ROWS instances two kinds of batches cost this kernel more than the scanning one (which takes 2.4 us an arrival on 1,024 x
 // 1,024 whatever the rows): many far rows that may pay a penalty, whose arrivals need a look at all rows, scans, and folds of
@@ -403,6 +402,10 @@ struct RouteSumArgs {
     float long_p, long_d;          // as in SumArgs
 };
 
+// The list block: its warps, the bins by which it finds how many rows are within a margin, and what the routing block tells it.
+constexpr int RS_LIST_WARPS = 16, RS_LIST_BINS = 64;
+constexpr unsigned int RS_GO_USUAL = 1, RS_GO_APART = 2, RS_GO_LEAVE = 3;
+
 // What the deciding warp can ask of the folding warps: the peaks of some rows, or a look at all rows.
 constexpr int RS_SCANS = 0, RS_KEYS = 1, RS_CLOSELY = 2;
 
@@ -441,15 +444,20 @@ struct RsShared {
                                             // given, peak}
     unsigned int pending[RS_LIST_ROWS];     // by slot of the row held: 1 from the decision for it to the end of its fold; cleared last
     uint2 scored[RS_ITEMS];                 // {token count, peak} of their scores, from the folding warps
+    // from the list block, for the present list and the next one
     int4 table[2][32];                      // by code of the prompt: {bounds of the rows outside the list}
     int list_row[2][RS_LIST_ROWS];
     int list_n[2], list_base[2];
-    unsigned short list_seg[RS_LIST_WARPS][RS_LIST_ROWS];      // (list warps) each one's rows of the list, and their number
-    int list_take[RS_LIST_WARPS];
-    unsigned int bucket_a[32], bucket_b[32];   // (list warps) smallest keys of the rows outside the list
-    unsigned int probe_t[RS_PROBES];        // (list warps) smallest scores at the probes
-    unsigned short near_row[RS_NEAR_ROWS];
-    unsigned int lists_wanted, lists_ready;
+    unsigned int lists_ready;
+    unsigned int least;                     // smallest score of an empty prompt, to begin with
+    // (the list block's own)
+    unsigned int lists_wanted, lists_go;    // the list that is asked for; RS_GO_USUAL, RS_GO_APART, RS_GO_LEAVE
+    unsigned short list_seg[RS_LIST_WARPS][RS_LIST_ROWS];      // each warp's rows of the list, and their number
+    int list_take[RS_LIST_WARPS], list_found[RS_LIST_WARPS];   // (and of the rows that later lists are made of)
+    int probe_w[RS_LIST_WARPS][RS_PROBES];  // smallest scores at the probes, by warp
+    unsigned int list_bin[RS_LIST_BINS];    // rows by how far they are above them
+    unsigned int bucket_a[32], bucket_b[32];   // smallest keys of the rows outside the list
+    unsigned int far_a[32], far_b[32];         // and of those outside the rows that it was made of
     unsigned int done[RS_MAX_FOLD_WARPS];   // the next decision each folding warp will fold
     unsigned int looks_done[RS_MAX_FOLD_WARPS];
     int look_P, look_D, look_how;           // RS_SCANS, RS_KEYS or RS_CLOSELY
@@ -468,6 +476,7 @@ struct RsShared {
     unsigned int flush;                     // ... and as many are asked for
     int cursor;                             // items of the batch that the io warp has looked at (when it has ended)
     unsigned int spin_limit, idle_limit;
+    unsigned int touched[32];               // (see touch_row)
     unsigned int beat;                      // moves while the io warp goes through arrivals
     unsigned int not_over;                  // ADMIT: rows that are not overloaded, as far as folded
     int blocked;                            // ADMIT: a request found every instance overloaded ...
@@ -510,8 +519,49 @@ __device__ __forceinline__ int4 ld_table(unsigned int at) {
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at));
     return v;
 }
+// Words of the other block of a cluster of two: rank 0 routes, rank 1 builds the lists.
+__device__ __forceinline__ unsigned int block_rank() { unsigned int r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ unsigned int other_smem(const void* p, unsigned int rank) {
+    unsigned int v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(v) : "r"(smem_u32(p)), "r"(rank));
+    return v;
+}
+__device__ __forceinline__ unsigned int ld_cluster(unsigned int at) {
+    unsigned int v;
+    asm volatile("ld.relaxed.cluster.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+    return v;
+}
+__device__ __forceinline__ int2 ld_cluster2(unsigned int at) {
+    int2 v;
+    asm volatile("ld.relaxed.cluster.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(at) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned int ld_acquire_cluster(const unsigned int* p) {      // (a word of this block that the other one writes)
+    unsigned int v;
+    asm volatile("ld.acquire.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_cluster(unsigned int at, unsigned int v) { asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory"); }
+__device__ __forceinline__ void st_cluster4(unsigned int at, int4 v) {
+    asm volatile("st.relaxed.cluster.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ void st_release_cluster(unsigned int at, unsigned int v) {
+    asm volatile("fence.acq_rel.cluster; st.release.cluster.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void acquire_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 
+// Polls of a warp that nothing is owed to.
+__device__ __forceinline__ unsigned int rs_idle_limit(unsigned int spin_limit) { return max(spin_limit < (1u << 27) ? 16u * spin_limit : 0xffffffffu, 1u << 22); }
+// The newest list that is there.  No acquire: what is read behind it lies in this block's shared memory and was there before the list block's release, and loads
+// of shared memory are made in order.  An acquire of the cluster empties the SM's L1 of the rows' cells (by every poll of the io warp: a fold's load took 350
+// cycles instead of 80).
+__device__ __forceinline__ unsigned int list_number(const RsShared& sh) {
+    unsigned int v;
+    asm volatile("ld.relaxed.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(&sh.lists_ready)) : "memory");
+    return v;
+}
 // A wait of a whole warp on words that other warps of this block write.  False: abandoned, here or elsewhere.
 // What counts against the limit is time in which nothing moves.  IDLE: nothing is owed to this warp, it waits for work; that
 // there is none as long as the deciding warp gets on without is no reason to give up.
@@ -1021,7 +1071,7 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
         if (!rs_wait<true>(sh, [&] {
                 ctl = ld_volatile4(&sh.ctl);
                 return (!SELF && (int)(ctl.x - n) > 0) || ctl.y != looks || ctl.z != 0;
-            }, LISTS || SELF ? 20 : 0))    // (the list warps need the issue slots)
+            }, LISTS || SELF ? 20 : 0))
             return;
         acquire_cta();
         if (SELF || __all_sync(FULL_MASK, (int)(ctl.x - n) <= 0)) ctl = ld_volatile4(&sh.ctl);
@@ -1053,7 +1103,14 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
 }
 
 // ---- io warp: arrivals ahead of the decisions, results behind the folds
-template <int KS, int FOLD_WARPS, bool ADMIT, int KIND>
+// Brings a row's cells into this SM's L1: the load of a fold that finds them there takes 80 cycles and 350 otherwise, of a fold's 970.
+// (prefetch.global.L1 left them in L2, and loads whose values are not used are not made: the sum goes to a word that nobody reads.)
+__device__ __forceinline__ unsigned int touch_row(const uint2* near, const unsigned int* far, int row) {
+    const unsigned int* cells = reinterpret_cast<const unsigned int*>(near + (size_t)row * 32);
+    return cells[0] ^ cells[32] ^ far[(size_t)row * 32];
+}
+
+template <int KS, bool LISTS, int FOLD_WARPS, bool ADMIT, int KIND>
 __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, const Scores<KIND>& sc, long long q_head, int waiting, int items, int room) {
     const int lane = threadIdx.x & 31;
     const long long n0 = sh.n0;
@@ -1069,7 +1126,19 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
     unsigned int written = 0;       // results written out
     int first_bad = 0x7fffffff, first_full = 0x7fffffff;
     unsigned int quiet = 0, seen = 0;      // rounds of this loop in which nothing has moved
+    unsigned int list = 0;                 // the newest one whose rows are on their way
     for (;;) {
+        if (LISTS) {      // (for the folds of its rows)
+            const unsigned int newest = __reduce_max_sync(FULL_MASK, list_number(sh));
+            if (newest != list) {
+                list = newest;
+                const int n = sh.list_n[list & 1];      // (may be none)
+                unsigned int sum = 0;
+                #pragma unroll 2
+                for (int x = lane; x < n; x += 32) sum ^= touch_row(a.near, a.far, sh.list_row[list & 1][x]);
+                sh.touched[lane] = sum;
+            }
+        }
         while (cursor < items && entered - written <= RS_ITEMS - 32) {
             const int k = cursor + lane;
             int P = -1, D = 0;
@@ -1144,8 +1213,8 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
     if (lane == 0) { sh.first_bad = first_bad; sh.first_full = first_full; sh.cursor = min(cursor, items); }
 }
 
-// ---- list warps.  A list holds the rows whose key value for one of RS_PROBES prompt lengths lies within a margin of the
-// smallest one known for it; the margin follows the list's room.  The other rows are bounded by 32 buckets: bucket x
+// ---- list block.  A list holds the rows whose key value for one of RS_PROBES prompt lengths lies within a margin of the
+// smallest one, as many as there is room for.  The other rows are bounded by 32 buckets: bucket x
 // holds the smallest a and the smallest b of the rows whose row_code is x.  For an arrival of code q the rows
 // of codes above q pay no penalty (value = a), those below q do (value = b + beta * P), and those of code q either
 // (value = the larger, hence at least the larger of the two smallest): four numbers per code.
@@ -1154,221 +1223,225 @@ __device__ __forceinline__ int rs_probe(int mean, int x) {
     const float share[RS_PROBES] = {0.0f, 0.08f, 0.17f, 0.3f, 0.5f, 0.9f, 1.5f, 2.5f};
     return (int)((float)mean * share[x]);
 }
-
-__device__ __forceinline__ void prefetch_row(const uint2* near, const unsigned int* far, int row) {
-    asm volatile("prefetch.global.L1 [%0]; prefetch.global.L1 [%0 + 128]; prefetch.global.L1 [%1];" ::"l"(near + (size_t)row * 32), "l"(far + (size_t)row * 32));
+__device__ __forceinline__ int rs_mean(const Batch& b) {      // prompt + ramp of a typical request
+    const unsigned long long mean = b.ramps / (unsigned long long)(b.n_items > 0 ? b.n_items : 1);
+    return mean < (1ull << 22) ? (int)mean : 1 << 22;
+}
+template <int KS, int KIND>
+__device__ __forceinline__ Scores<KIND> rs_scores(const RouteSumArgs& a, const Batch& b) {
+    Scores<KIND> sc;
+    sc.start(a.theta, a.beta, b.peak_bound, b.max_pd, b.max_p, (b.base_sum + b.tokens_in) / (unsigned long long)a.I, rs_mean(b), Held<KS>::ITEM);
+    return sc;
 }
 
-template <int LIST_WARPS, int KS, int KIND>
-__device__ __forceinline__ void rs_list_loop(RsShared& sh, const Rows& rows, const Scores<KIND>& sc, const uint2* near_cells, const unsigned int* far_cells, int I, int mean, int longest, int t) {
-    constexpr int THREADS = 32 * LIST_WARPS, ROOM = 32 * KS, NEAR_ROOM = RS_NEAR_ROWS / LIST_WARPS;
-    constexpr int FAR_KEY = 0x7f000000, EACH = 4, AT_ONCE = 4;      // AT_ONCE: rows a thread has on their way
-    static_assert(NEAR_ROOM >= 2 * 32 * AT_ONCE, "");
-    const int lane = threadIdx.x & 31, me = t >> 5;
-    const bool leader = t < 32;
-    auto over = [&] { return __any_sync(FULL_MASK, ld_volatile(&sh.ctl.z) != 0); };
-    // The list warps meet at a barrier of their own, and leave together if one of them has seen that the last decision is made.  (Polls of
-    // a counter took 500 cycles a meeting and the other warps' issue slots.)
-    auto meet = [&](bool stop) -> bool {
-        int leave;
-        __syncwarp();
-        asm volatile("{ .reg .pred p, q; setp.ne.s32 p, %1, 0; barrier.cta.red.or.pred q, 1, %2, p; selp.s32 %0, 1, 0, q; }" : "=r"(leave) : "r"((int)stop), "n"(THREADS) : "memory");
-        return leave != 0;
-    };
-    auto empty_buckets = [&] { if (leader) { sh.bucket_a[lane] = 0xffffffffu; sh.bucket_b[lane] = 0xffffffffu; } };
-    int probe_key = 0;
+// The second block of the cluster, on an SM of its own: it takes a copy of the rows' keys from the routing block's shared memory, sorts the rows into the list
+// and the buckets, and writes the list back.  What bounds it: the latency of some ten passes and meetings.  By four to six warps of the routing
+// block, among the warps that fold, a list took 5,000 cycles on 512 rows and 11,400 on 4,096, about as long as one lasts, and the deciding warp waited for
+// lists for 15 to 45 cycles an arrival.
+template <int KS, int KIND>
+__device__ __forceinline__ void rs_build_lists(const RouteSumArgs& a, RsShared& sh, const Rows& rows) {
+    constexpr int ROOM = 32 * KS, FAR_KEY = 0x7f000000, EACH = 4;
+    const int t = threadIdx.x, lane = t & 31, me = __shfl_sync(FULL_MASK, t >> 5, 0), I = a.I;
+    const Batch b = *reinterpret_cast<const Batch*>(__cluster_map_shared_rank(&sh.batch, 0));
+    const Scores<KIND> sc = rs_scores<KS, KIND>(a, b);
+    const int mean = rs_mean(b);
+    const unsigned int at_rec = other_smem(rows.rec, 0), at_ctl = other_smem(&sh.ctl, 0), at_beat = other_smem(&sh.beat, 0);
+    int2* const rec = rows.rec;                                     // this block's copy
+    int* const above = reinterpret_cast<int*>(rows.state);          // how far a row is above the smallest score, at the probe where that is least
+    // Beyond RS_LONG_LISTS instances most lists are made of the rows that were within four margins when all rows were looked at last: scores only grow, so the others
+    // are where they were, or further off.  They are bounded by buckets of their own, and `reach` by probe; when a list's margin passes that, the next
+    // one is made of all rows again.
+    constexpr bool NEAR = KS == 8;
+    unsigned short* const near = reinterpret_cast<unsigned short*>(rows.top);       // (the rows, ascending)
+    unsigned short* const found = near + I;
+    bool all_rows = true;
+    int n_near = 0, reach[RS_PROBES];
+    #pragma unroll
+    for (int p = 0; p < RS_PROBES; ++p) reach[p] = FAR_KEY;
     int bp[RS_PROBES];
     #pragma unroll
-    for (int x = 0; x < RS_PROBES; ++x) {
-        bp[x] = sc.key_p(rs_probe(mean, x));
-        if (lane == x) probe_key = bp[x];
-    }
-    int margin = max(sc.key_a((unsigned int)mean) / 16, 8);
-    const int least_margin = max(sc.key_a(1u), 1);
-    unsigned short* near = sh.near_row + me * NEAR_ROOM;
+    for (int x = 0; x < RS_PROBES; ++x) bp[x] = sc.key_p(rs_probe(mean, x));
+    int width = min(max(max(sc.key_a((unsigned int)mean) / 16, 8) / (RS_LIST_BINS / 2), 1), 1 << 20);      // of a bin (256 of them leave room for keys)
     // (a warp has neighbouring rows: the list is put together in their order)
-    const int share = ((I + THREADS - 1) / THREADS) * 32, first = me * share, end = min(I, first + share);
     for (unsigned int n = 1;; ++n) {
-        bool stop = false;
-        if (leader) {      // (one of them looks for work, the others wait for it)
-            stop = !rs_wait<true>(sh, [&] {
-                const unsigned int last = ld_volatile(&sh.ctl.z);
-                return ld_acquire(&sh.lists_wanted) >= n || last != 0;
-            }, 20);
-            stop = stop || !__any_sync(FULL_MASK, ld_acquire(&sh.lists_wanted) >= n);     // (nothing is asked for after the last decision)
-        }
-        if (meet(stop)) return;
-        const int old = (n + 1) & 1, now = n & 1;
-        // the smallest value known per probe: the rows of the present list, and (kept in probe_t) the others' bound
-        if (n > 1) {   // (the first list: probe_t was set when the rows were loaded)
-            const int old_n = sh.list_n[old];
-            if (t - lane < old_n) {
-                int least[RS_PROBES];
-                #pragma unroll
-                for (int x = 0; x < RS_PROBES; ++x) least[x] = FAR_KEY;
-                for (int x = t; x < old_n; x += THREADS) {
-                    const int2 r = ld_volatile2(rows.rec + sh.list_row[old][x]);
-                    #pragma unroll
-                    for (int p = 0; p < RS_PROBES; ++p) least[p] = min(least[p], max(r.x, r.y + bp[p]));
+        bool leave = false;
+        if (me == 0) {      // (one warp looks for work, the others wait for it; as in rs_wait what counts is time in which the deciding warp does not get on)
+            unsigned int seen = 0, polls = 0;
+            while (__any_sync(FULL_MASK, (int)(ld_acquire_cluster(&sh.lists_wanted) - n) < 0)) {
+                if (__any_sync(FULL_MASK, ld_acquire_cluster(&sh.lists_go) == RS_GO_LEAVE)) { leave = true; break; }
+                if ((++polls & 255u) == 0) {
+                    const unsigned int now = __reduce_max_sync(FULL_MASK, ld_cluster(at_ctl) + ld_cluster(at_beat));
+                    if (now != seen) { seen = now; polls = 0; }
                 }
-                int mine = 0;
-                #pragma unroll
-                for (int p = 0; p < RS_PROBES; ++p) {
-                    const int v = __reduce_min_sync(FULL_MASK, least[p]);
-                    mine = lane == p ? v : mine;
-                }
-                if (lane < RS_PROBES) atomicMin(&sh.probe_t[lane], ordered(mine));
+                if (polls >= sh.idle_limit) { if (lane == 0) st_cluster(at_ctl + 12u, 1u); leave = true; break; }
+                __nanosleep(20);
             }
         }
-        if (meet(over())) return;
-        for (int tries = 0;; ++tries) {
-            // A row is in the list if for some probe its a is at most limit_a and its b at most limit_b.
-            // Rows beyond far_a or far_b are out of reach of this list: the two limits bound them, and they are dropped by
-            // two comparisons.
-            int limit_a[RS_PROBES], limit_b[RS_PROBES];
-            int far_a = RS_LOWEST;
+        if (__syncthreads_or(leave)) return;
+        const int now = n & 1, of = NEAR && !all_rows ? n_near : I;
+        const int share = ((of + 32 * RS_LIST_WARPS - 1) / (32 * RS_LIST_WARPS)) * 32, first = me * share, end = min(of, first + share);
+        auto row_of = [&](int x) { return NEAR && !all_rows ? (int)near[x] : x; };
+        // ---- the rows as they are, and the smallest score at each probe.  (Loops with short bodies: what is unrolled is fetched anew for every list.)
+        #pragma unroll 1
+        for (int base = first + lane; base - lane < end; base += 32 * EACH) {
+            int2 r[EACH];
+            #pragma unroll
+            for (int u = 0; u < EACH; ++u) r[u] = ld_cluster2(at_rec + 8u * (unsigned int)row_of(base + 32 * u < end ? base + 32 * u : first));
+            #pragma unroll
+            for (int u = 0; u < EACH; ++u)
+                if (base + 32 * u < end) rec[base + 32 * u] = r[u];
+        }
+        {
+            int least[RS_PROBES];
+            #pragma unroll
+            for (int p = 0; p < RS_PROBES; ++p) least[p] = FAR_KEY;
+            #pragma unroll 1
+            for (int i = first + lane; i < end; i += 32) {      // (a lane's own rows)
+                const int2 r = rec[i];
+                #pragma unroll
+                for (int p = 0; p < RS_PROBES; ++p) least[p] = min(least[p], __viaddmax_s32(r.y, bp[p], r.x));
+            }
+            int mine = 0;
             #pragma unroll
             for (int p = 0; p < RS_PROBES; ++p) {
-                limit_a[p] = tries < 8 ? unordered(sh.probe_t[p]) + margin : RS_LOWEST;   // (an empty list is a list, too)
-                limit_b[p] = limit_a[p] - bp[p];
-                far_a = max(far_a, limit_a[p]);
+                const int v = __reduce_min_sync(FULL_MASK, least[p]);
+                mine = lane == p ? v : mine;
             }
-            const int far_b = limit_a[0];
-            far_a = (int)min((long long)far_a + longest, (long long)RS_ABSENT);
-            int hot_b = FAR_KEY, cold_a = FAR_KEY;
-            int n_near = 0, n_take = 0;
-            auto sort_near = [&]() {        // the rows that were not dropped: into the list or into a bucket
-                __syncwarp();
-                // (several rows a lane at once and no branches: what bounds this is the latency of a row's chain)
-                for (int x = lane; x - lane < n_near; x += 32 * EACH) {
-                    int2 r[EACH];
-                    bool in[EACH], take[EACH], low = false;
-                    int i[EACH], c[EACH];
-                    #pragma unroll
-                    for (int u = 0; u < EACH; ++u) { in[u] = x + 32 * u < n_near; i[u] = near[in[u] ? x + 32 * u : 0]; }
-                    #pragma unroll
-                    for (int u = 0; u < EACH; ++u) r[u] = ld_volatile2(rows.rec + i[u]);
-                    #pragma unroll
-                    for (int u = 0; u < EACH; ++u) {
-                        // (the largest limit_b of the probes whose limit_a the row keeps)
-                        int most_b = RS_LOWEST;
-                        #pragma unroll
-                        for (int p = RS_PROBES - 1; p >= 0; --p) most_b = r[u].x <= limit_a[p] ? max(most_b, limit_b[p]) : most_b;
-                        take[u] = in[u] && r[u].y <= most_b && most_b != RS_LOWEST;
-                        c[u] = sc.row_code(r[u]);
-                    }
-                    unsigned int was_a[EACH], was_b[EACH];
-                    #pragma unroll
-                    for (int u = 0; u < EACH; ++u) { was_a[u] = ld_volatile(&sh.bucket_a[c[u]]); was_b[u] = ld_volatile(&sh.bucket_b[c[u]]); }
-                    #pragma unroll
-                    for (int u = 0; u < EACH; ++u) {
-                        const unsigned int vote = __ballot_sync(FULL_MASK, take[u]);
-                        const int at = n_take + __popc(vote & ((1u << lane) - 1u));
-                        if (take[u] && at < ROOM) sh.list_seg[me][at] = (unsigned short)i[u];
-                        n_take += __popc(vote);
-                        const bool left = in[u] && !take[u], middle = left && c[u] != 0 && c[u] != 31;
-                        hot_b = min(hot_b, left && c[u] == 0 ? r[u].y : FAR_KEY);
-                        cold_a = min(cold_a, left && c[u] == 31 ? r[u].x : FAR_KEY);
-                        in[u] = middle && (ordered(r[u].x) < was_a[u] || ordered(r[u].y) < was_b[u]);
-                        low |= in[u];
-                    }
-                    if (__any_sync(FULL_MASK, low)) {      // (most rows change no bucket)
-                        #pragma unroll
-                        for (int u = 0; u < EACH; ++u)
-                            if (in[u]) {
-                                atomicMin(&sh.bucket_a[c[u]], ordered(r[u].x));
-                                atomicMin(&sh.bucket_b[c[u]], ordered(r[u].y));
-                            }
-                    }
-                }
-                __syncwarp();
-                n_near = 0;
-            };
-            for (int base = first; base < end; base += AT_ONCE * 32) {
-                int2 r[AT_ONCE];
-                #pragma unroll
-                for (int u = 0; u < AT_ONCE; ++u) {
-                    const int i = base + u * 32 + lane;
-                    r[u] = ld_volatile2(rows.rec + (i < end ? i : first));
-                }
-                const bool enough = over();
-                #pragma unroll
-                for (int u = 0; u < AT_ONCE; ++u) {
-                    const int i = base + u * 32 + lane;
-                    const bool keep = i < end && r[u].y <= far_b && r[u].x <= far_a;
-                    const unsigned int vote = __ballot_sync(FULL_MASK, keep);
-                    if (keep) near[n_near + __popc(vote & ((1u << lane) - 1u))] = (unsigned short)i;
-                    n_near += __popc(vote);
-                }
-                if (enough) break;
-                if (n_near > NEAR_ROOM - AT_ONCE * 32) sort_near();
-            }
-            sort_near();
-            const int hb = __reduce_min_sync(FULL_MASK, hot_b), ca = __reduce_min_sync(FULL_MASK, cold_a);
-            if (lane == 0) { atomicMin(&sh.bucket_b[0], ordered(hb)); atomicMin(&sh.bucket_a[31], ordered(ca)); sh.list_take[me] = n_take; }
-            if (meet(over())) return;
-            const int taken = lane < LIST_WARPS ? sh.list_take[lane] : 0, count = __reduce_add_sync(FULL_MASK, taken);
-            // (the margin that fills four fifths of the list, were its rows spread evenly)
-            const int fitting = (int)((float)margin * fmaxf(0.8f * ROOM / (float)max(count, 1), 0.25f));
-            if (count > ROOM) {
-                margin = max(min(fitting, margin / 2 + margin / 4), least_margin);
-                if (tries > 4) margin = 0;
-                empty_buckets();
-                if (meet(over())) return;
-                continue;
-            }
-            const int before = __reduce_add_sync(FULL_MASK, lane < me ? taken : 0);
-            for (int x = lane; x < n_take; x += 32) {
-                const int i = sh.list_seg[me][x];
-                sh.list_row[now][before + x] = i;
-                prefetch_row(near_cells, far_cells, i);     // (for the folds of its rows)
-            }
-            if (leader) {
-                // (a key that no row has set is out of reach; rows of code 31 count by their a alone, no b is kept for them)
-                const int ka = unordered(min(sh.bucket_a[lane], ordered(RS_ABSENT)));
-                const int kb = unordered(min(sh.bucket_b[lane], ordered(RS_TOP_KEY)));     // (room for beta * P on top)
-                int above_a = min(ka, far_a), below_b = min(kb, far_b);
-                #pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const int x = __shfl_down_sync(FULL_MASK, above_a, off), y = __shfl_up_sync(FULL_MASK, below_b, off);
-                    if (lane + off < 32) above_a = min(above_a, x);
-                    if (lane >= off) below_b = min(below_b, y);
-                }
-                above_a = __shfl_down_sync(FULL_MASK, above_a, 1);
-                below_b = __shfl_up_sync(FULL_MASK, below_b, 1);
-                if (lane == 31) above_a = far_a;
-                if (lane == 0) below_b = far_b;
-                const int row_b = lane == 31 ? RS_LOWEST : kb;
-                // The entries as keys that the deciding warp holds: a row that wins by less than the rounding of its key does not beat them.
-                // (The base is a lower bound of every row's score, so an entry that is cut below is one, too.)
-                const int base = unordered(sh.probe_t[0]) & ~1;
-                auto entry = [&](int key) { return Held<KS>::relative(key, base) - 1 - Held<KS>::scaled(Scores<KIND>::SLACK); };
-                sh.table[now][lane] = make_int4(entry(above_a), entry(below_b), entry(ka), entry(row_b));
-                const int c = sc.code((float)probe_key);
-                const int ex = __shfl_sync(FULL_MASK, above_a, c), ey = __shfl_sync(FULL_MASK, below_b, c), ez = __shfl_sync(FULL_MASK, ka, c), ew = __shfl_sync(FULL_MASK, row_b, c);
-                __syncwarp();
-                if (lane < RS_PROBES) sh.probe_t[lane] = ordered(min(min(ex, ey + probe_key), max(ez, ew + probe_key)));
-                if (lane == 0) { sh.list_n[now] = count; sh.list_base[now] = base; }
-                empty_buckets();
-            }
-            if (meet(over())) return;
-            if (t == 0) st_release(&sh.lists_ready, n);
-            margin = max(min(min(fitting, margin + margin / 2 + 1), 1 << 27), least_margin);
-            break;
+            if (lane < RS_PROBES) sh.probe_w[me][lane] = mine;
         }
+        if (t < RS_LIST_BINS) sh.list_bin[t] = 0;
+        if (t < 32) { sh.bucket_a[t] = 0xffffffffu; sh.bucket_b[t] = 0xffffffffu; }
+        if (NEAR && all_rows && t < 32) { sh.far_a[t] = 0xffffffffu; sh.far_b[t] = 0xffffffffu; }
+        __syncthreads();
+        int smallest[RS_PROBES];
+        {
+            int v = FAR_KEY;
+            #pragma unroll
+            for (int q = 0; q < RS_LIST_WARPS / 4; ++q) v = min(v, sh.probe_w[RS_LIST_WARPS / 4 * (lane >> 3) + q][lane & 7]);
+            v = min(v, __shfl_xor_sync(FULL_MASK, v, 8));
+            v = min(v, __shfl_xor_sync(FULL_MASK, v, 16));
+            #pragma unroll
+            for (int p = 0; p < RS_PROBES; ++p) smallest[p] = min(__shfl_sync(FULL_MASK, v, p), all_rows ? FAR_KEY : reach[p]);
+        }
+        // ---- how far each row is above them, in bins; as many bins are taken as there is room for
+        int bins = 0;
+        auto bin = [&](int d) { return (unsigned int)((float)d * (1.0f / (float)width)); };      // (ascends with d)
+        for (int tries = 0;; ++tries) {
+            #pragma unroll 1
+            for (int i = first + lane; i < end; i += 32) {
+                int d = FAR_KEY;
+                if (tries == 0) {
+                    const int2 r = rec[i];
+                    #pragma unroll
+                    for (int p = 0; p < RS_PROBES; ++p) d = __viaddmin_s32(__viaddmax_s32(r.y, bp[p], r.x), -smallest[p], d);
+                    above[i] = d;
+                } else d = above[i];
+                const unsigned int x = bin(d);
+                if (x < (unsigned int)RS_LIST_BINS) atomicAdd(&sh.list_bin[x], 1u);
+            }
+            __syncthreads();
+            unsigned int lo = sh.list_bin[lane], hi = sh.list_bin[lane + 32];
+            #pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const unsigned int x = __shfl_up_sync(FULL_MASK, lo, off), y = __shfl_up_sync(FULL_MASK, hi, off);
+                if (lane >= off) { lo += x; hi += y; }
+            }
+            hi += __shfl_sync(FULL_MASK, lo, 31);
+            bins = __popc(__ballot_sync(FULL_MASK, lo <= ROOM)) + __popc(__ballot_sync(FULL_MASK, hi <= ROOM));
+            const int all = (int)__shfl_sync(FULL_MASK, hi, 31);
+            const bool finer = bins < RS_LIST_BINS / 8 && width > 1, coarser = bins == RS_LIST_BINS && all < of && all < ROOM / 2 && width < (1 << 19);
+            if (tries >= 8 || !(finer || coarser)) break;
+            __syncthreads();
+            if (t < RS_LIST_BINS) sh.list_bin[t] = 0;
+            width = finer ? max(width / 16, 1) : 4 * width;
+            __syncthreads();
+        }
+        // ---- the list, and the buckets of the others
+        int hot_b = FAR_KEY, cold_a = FAR_KEY, n_take = 0, n_found = 0;
+        const unsigned int near_bins = 4u * (unsigned int)max(bins, 1);
+        #pragma unroll 1
+        for (int x = first + lane; x - lane < end; x += 32) {
+            const bool in = x < end;
+            const int i = row_of(in ? x : first);
+            const int2 r = rec[in ? x : first];
+            const unsigned int b = bin(above[in ? x : first]);
+            const bool take = in && b < (unsigned int)bins, left = in && !take, far = NEAR && all_rows && b >= near_bins;
+            const int c = sc.row_code(r);
+            unsigned int* const bucket_a = far ? sh.far_a : sh.bucket_a, * const bucket_b = far ? sh.far_b : sh.bucket_b;
+            const unsigned int was_a = ld_volatile(bucket_a + c), was_b = ld_volatile(bucket_b + c);
+            const unsigned int vote = __ballot_sync(FULL_MASK, take);
+            const int at = n_take + __popc(vote & ((1u << lane) - 1u));
+            if (take && at < ROOM) sh.list_seg[me][at] = (unsigned short)i;
+            n_take += __popc(vote);
+            if (NEAR && all_rows) {
+                const unsigned int near_vote = __ballot_sync(FULL_MASK, in && !far);
+                if (in && !far) found[first + n_found + __popc(near_vote & ((1u << lane) - 1u))] = (unsigned short)i;
+                n_found += __popc(near_vote);
+            }
+            hot_b = min(hot_b, left && !far && c == 0 ? r.y : FAR_KEY);
+            cold_a = min(cold_a, left && !far && c == 31 ? r.x : FAR_KEY);
+            if (left && (far || (c != 0 && c != 31)) && (ordered(r.x) < was_a || ordered(r.y) < was_b)) {      // (most rows change no bucket)
+                if (c != 0) atomicMin(bucket_a + c, ordered(r.x));
+                if (c != 31) atomicMin(bucket_b + c, ordered(r.y));
+            }
+        }
+        const int hb = __reduce_min_sync(FULL_MASK, hot_b), ca = __reduce_min_sync(FULL_MASK, cold_a);
+        if (lane == 0) { atomicMin(&sh.bucket_b[0], ordered(hb)); atomicMin(&sh.bucket_a[31], ordered(ca)); sh.list_take[me] = n_take; sh.list_found[me] = n_found; }
+        __syncthreads();
+        const int taken = lane < RS_LIST_WARPS ? sh.list_take[lane] : 0, before = __reduce_add_sync(FULL_MASK, lane < me ? taken : 0);
+        const unsigned int at_list = other_smem(sh.list_row[now], 0);
+        for (int x = lane; x < n_take; x += 32) st_cluster(at_list + 4u * (unsigned int)(before + x), sh.list_seg[me][x]);
+        if (me == 0) {
+            // (a key that no row has set is out of reach; rows of code 31 count by their a alone, no b is kept for them)
+            const int ka = unordered(min(min(sh.bucket_a[lane], NEAR ? sh.far_a[lane] : 0xffffffffu), ordered(RS_ABSENT)));
+            const int kb = unordered(min(min(sh.bucket_b[lane], NEAR ? sh.far_b[lane] : 0xffffffffu), ordered(RS_TOP_KEY)));     // (room for beta * P on top)
+            int above_a = ka, below_b = kb;
+            #pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int x = __shfl_down_sync(FULL_MASK, above_a, off), y = __shfl_up_sync(FULL_MASK, below_b, off);
+                if (lane + off < 32) above_a = min(above_a, x);
+                if (lane >= off) below_b = min(below_b, y);
+            }
+            above_a = __shfl_down_sync(FULL_MASK, above_a, 1);
+            below_b = __shfl_up_sync(FULL_MASK, below_b, 1);
+            if (lane == 31) above_a = RS_ABSENT;
+            if (lane == 0) below_b = RS_TOP_KEY;
+            const int row_b = lane == 31 ? RS_LOWEST : kb;
+            // The entries as keys that the deciding warp holds: a row that wins by less than the rounding of its key does not beat them.
+            // (The base is a lower bound of every row's score, so an entry that is cut below is one, too.)
+            const int base = smallest[0] & ~1, count = __reduce_add_sync(FULL_MASK, taken);
+            auto entry = [&](int key) { return Held<KS>::relative(key, base) - 1 - Held<KS>::scaled(Scores<KIND>::SLACK); };
+            st_cluster4(other_smem(&sh.table[now][lane], 0), make_int4(entry(above_a), entry(below_b), entry(ka), entry(row_b)));
+            if (lane == 0) { st_cluster(other_smem(&sh.list_n[now], 0), (unsigned int)count); st_cluster(other_smem(&sh.list_base[now], 0), (unsigned int)base); }
+        }
+        __syncthreads();
+        if (t == 0) st_release_cluster(other_smem(&sh.lists_ready, 0), n);
+        const int margin = bins * width;
+        if (NEAR && all_rows) {
+            const int mine = lane < RS_LIST_WARPS ? sh.list_found[lane] : 0, at = __reduce_add_sync(FULL_MASK, lane < me ? mine : 0);
+            n_near = __reduce_add_sync(FULL_MASK, mine);
+            for (int x = lane; x < n_found; x += 32) near[at + x] = found[first + x];
+            all_rows = n_near > I / 2;      // (nothing is gained)
+            const int off = (int)near_bins * width, sure = off - (off >> 16) - 2;      // (the bins are rounded)
+            #pragma unroll
+            for (int p = 0; p < RS_PROBES; ++p) reach[p] = smallest[p] + sure;
+        } else if (NEAR) {
+            #pragma unroll
+            for (int p = 0; p < RS_PROBES; ++p) all_rows |= smallest[p] + margin > reach[p];
+        }
+        width = min(max(margin / (RS_LIST_BINS / 2), 1), 1 << 20);      // (half of the bins the next time)
     }
 }
 
-// Folding and list warps, warps and threads of the instantiations.  (Decisions come every 100 to 150 cycles and a fold takes some 700 from when
-// it is told: fewer warps than that leave the rows pending for longer, and more would leave the deciding warp fewer registers.  Measured
-// on 512 x 1,024 / 4,096 x 2,048, us: 10 and 4 warps 1,036 / 11,141 with 6 and 5, 8 and 6 1,064 / 10,910, 6 and 5 1,080 / 11,279; two folds
-// at once by one warp, or the next one's loads ahead: 1,131 and 1,178, as either makes a single fold take longer.)
+// Folding warps, warps and threads of the instantiations.  (Decisions come every 100 cycles and a fold takes some 700 from when
+// it is told: fewer warps than that leave the rows pending for longer; two folds at once by one warp, or the next one's loads ahead, make
+// a single fold take longer.)
 template <int KS, bool LISTS> struct Shape {
-    static constexpr int FOLD = !LISTS ? 8 : KS == 4 ? 10 : 8, LIST = !LISTS ? 0 : KS == 4 ? 4 : 6;
+    static constexpr int FOLD = LISTS ? 10 : 8;
     static constexpr bool SELF = KS == 1;                  // the deciding warp folds its decisions itself
     static constexpr int DONE = SELF ? 1 : FOLD;           // warps that fold
-    static constexpr int WARPS = 4 * ((FOLD + 1 + LIST + 2) / 3), THREADS = 32 * WARPS;
-    static_assert(FOLD <= RS_MAX_FOLD_WARPS && LIST <= RS_LIST_WARPS, "");
+    static constexpr int WARPS = 4 * ((FOLD + 1 + 2) / 3), THREADS = 32 * WARPS;
+    static_assert(FOLD <= RS_MAX_FOLD_WARPS && (!LISTS || WARPS == RS_LIST_WARPS), "");
 };
 
 // ---- deciding warp.  KS: rows per lane.  LISTS: they are a list's, else all rows.
@@ -1388,7 +1461,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     constexpr int TRIP = 4;
     // decisions between two looks at items and at the rows that were pending; items made ready at once (a trip may begin with the last but one of a
     // chunk)
-    constexpr unsigned int READY = !LISTS && KS <= 4 ? 32 : RS_READY, CHUNK = !LISTS && KS == 2 ? 16 : READY - TRIP;
+    constexpr unsigned int READY = RS_READY, CHUNK = LISTS ? READY - TRIP : 8 * KS;
     const int lane = threadIdx.x & 31, I = a.I, H = a.H;
     constexpr bool SELF = Shape<KS, LISTS>::SELF;
     const int lane_f = lane < Shape<KS, LISTS>::DONE ? lane : 0;
@@ -1460,12 +1533,12 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     unsigned int table = smem_u32(sh.table[0]);
     bool asked = false;
     auto ask_for_list = [&]() {
-        if (!asked && lane == 0) st_release(&sh.lists_wanted, list + 1);
+        if (!asked && lane == 0) st_cluster(other_smem(&sh.lists_wanted, 1), list + 1);
         asked = true;
     };
     auto next_list = [&](unsigned int e) {
         ask_for_list();
-        if (!rs_wait(sh, [&] { return ld_acquire(&sh.lists_ready) > list; })) { lost = true; return; }
+        if (!rs_wait(sh, [&] { return list_number(sh) > list; })) { lost = true; return; }
         ++list;
         asked = false;
         table = smem_u32(sh.table[list & 1]);
@@ -1498,7 +1571,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     if (LISTS) {
         next_list(0);
     } else {
-        take_base(unordered(sh.probe_t[0]) & ~1);
+        take_base(unordered(sh.least) & ~1);
         unread();
         refresh();
     }
@@ -1523,7 +1596,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         if (t >= 0) tell_slot(e, t, given, peak);
         else if (lane == 0) sh.jobs[e % RS_ITEMS] = make_uint2((unsigned int)w | given, peak);
     };
-    // Everything unusual about item e.  False: not decided, but the keys are such that it may be usual now (or the batch is lost).
+    // Everything unusual about item e.  False: not decided, but the marked rows have been read again, and it may be usual now (or the batch is lost).
     unsigned int tried_at = 0xffffffffu;      // the item for which `lists_tried` lists have been taken
     int lists_tried = 0;
     auto unusual = [&](unsigned int e) -> bool {
@@ -1562,6 +1635,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                     const unsigned int before = held_pending();
                     if (__any_sync(FULL_MASK, before != 0)) {
                         if (!rs_wait(sh, [&] { return __any_sync(FULL_MASK, held_pending() != before) != 0; })) { lost = true; return false; }
+                        refresh();
                         return false;
                     }
                     if (rebase()) return false;
@@ -1572,6 +1646,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                     const unsigned int* word = sh.pending + ((key & K::SLOT) >> 1);
                     if (__any_sync(FULL_MASK, ld_acquire(word) != 0)) {
                         if (!rs_wait(sh, [&] { return ld_acquire(word) == 0; })) lost = true;
+                        refresh();
                         return false;
                     }
                     if (!(__ballot_sync(FULL_MASK, [&] {      // (a far row; but it may just have been folded)
@@ -1580,8 +1655,10 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                             for (int k = 0; k < KS; ++k)
                                 if (tag(k) == (key & K::SLOT)) far = (ld_volatile(rows.state + row(k)) & RS_FAR) != 0;
                             return far;
-                        }())))
+                        }()))) {
+                        refresh();
                         return false;
+                    }
                 } else if (Scores<KIND>::EXACT) return false;
                 if (LISTS || !bounded) {
                     // Compared here: the rows that can be the best by what a row is worth at most, the far ones of a list by what they are worth if the
@@ -1631,6 +1708,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                         }
                         if (__any_sync(FULL_MASK, open >= 0)) {
                             if (!rs_wait(sh, [&] { return open < 0 || ld_acquire(sh.pending + open) == 0; })) lost = true;
+                            refresh();
                             return false;
                         }
                         if (!__any_sync(FULL_MASK, scan)) {
@@ -1799,21 +1877,24 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     };
 
     // ---- the usual way
-    int4 it0, it1, it2;              // items e, e + 1, e + 2 (see RsShared::ready)
-    unsigned int first = 0;          // the first of the items made ready
-    auto fetch = [&](unsigned int e) {
-        first = e;
-        __syncwarp();
-        #pragma unroll
-        for (unsigned int x = 0; x < READY; x += 32) {
-            const int4 it = ld_table(at_items + 16u * ((e + x + lane) % RS_ITEMS));
-            const int b = it.z > jmax ? cut : (int)0x80000001u;
-            sh.ready[x + lane] = make_int4(it.x, it.y, LISTS ? min(b, bound_of(ld_table(table + it.w), it.x)) : b, it.x + it.y);
+    int4 it0, it1, it2;              // items e, e + 1, e + 2 (LISTS: see RsShared::ready)
+    unsigned int first = 0;          // (LISTS) the first of the items made ready
+    auto item_at = [&](unsigned int e, unsigned int x) { return ld_table(LISTS ? at_ready + 16u * (e - first + x) : at_items + 16u * (e % RS_ITEMS + x)); };
+    auto fetch = [&](unsigned int e, unsigned int stop) {
+        if (LISTS) {      // (as many as a chunk up to `stop` needs)
+            first = e;
+            __syncwarp();
+            #pragma unroll 1
+            for (unsigned int x = 0; x < READY && (x == 0 || stop - e > x - TRIP); x += 32) {
+                const int4 it = ld_table(at_items + 16u * ((e + x + lane) % RS_ITEMS));
+                const int b = it.z > jmax ? cut : (int)0x80000001u;
+                sh.ready[x + lane] = make_int4(it.x, it.y, min(b, bound_of(ld_table(table + it.w), it.x)), it.x + it.y);
+            }
+            __syncwarp();
         }
-        __syncwarp();
-        it0 = ld_table(at_ready);
-        it1 = ld_table(at_ready + 16u);
-        it2 = ld_table(at_ready + 32u);
+        it0 = item_at(e, 0);
+        it1 = item_at(e, 1);
+        it2 = item_at(e, 2);
     };
     if constexpr (SELF) {
         // ---- up to RS_SELF_ROWS rows, one per lane: the deciding warp folds each decision itself, so that no row is ever pending.  What bounds it: the
@@ -1920,6 +2001,10 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             }
         }
     } else {
+    // With eight rows per lane and a list, what the steps behind an unusual one have added is taken off again, which asks that a marked row that wins gets nothing
+    // (its tag would become its neighbour's); else the keys from before the trip are kept and put back, which takes 15 cycles a step with eight
+    // rows and 5 with four, as many as not adding to marked rows.  (Without a list the items beyond the last one may have been written over by then.)
+    constexpr bool TAKE_OFF = LISTS && KS == 8;
     unsigned int e = 0, ready = 0;   // decisions made, items known to be there
     while (!lost) {     // (every way out has published what was decided)
         ready = __shfl_sync(FULL_MASK, ld_acquire(&sh.items_ready), 0);
@@ -1953,79 +2038,121 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         }
         const unsigned int stop = min(limit, e + CHUNK);
         refresh();
-        fetch(e);
+        fetch(e, stop);
         int untold = 0;               // decisions before e that are not told yet (the last trip's: they are while the next reduction is under way)
         int told = 0;
         while (e < stop) {
             int was_a[KS], was_b[KS], key[TRIP], not_usual = 0;
-            const unsigned int at = at_ready + 16u * (e - first);
-            #pragma unroll
-            for (int k = 0; k < KS; ++k) { was_a[k] = ra[k]; was_b[k] = rb[k]; }
-            #pragma unroll
-            for (int u = 0; u < TRIP; ++u) {     // (items from `limit` on are whatever the slots hold: what is done with them is taken back)
-                const int kp = it0.x, kpd = it0.y, kpb = it0.w;
-                int v[KS];
-                #pragma unroll
-                for (int k = 0; k < KS; ++k) v[k] = __viaddmax_s32(rb[k], kp, ra[k]);
-                int least = it0.z;
-                #pragma unroll
-                for (int k = 0; k + 1 < KS; k += 2) least = __vimin3_s32(least, v[k], v[k + 1]);
-                const int best = __reduce_min_sync(FULL_MASK, least);
-                // (while the reduction is under way)
-                if (u == 0) { tell(e - TRIP, told, untold); publish(e); }     // (whether there is anything to tell or not: a branch here cost 20 cycles a step)
-                it0 = it1; it1 = it2;
-                it2 = ld_table(at + 16u * (u + 3));
+            bool whole;
+            // (one loop with nothing but the trip: with the ways back from the unusual arrivals to its head a step took 104 cycles instead of 77)
+            #pragma unroll 1
+            do {
+                not_usual = 0;
+                const unsigned int at = LISTS ? at_ready + 16u * (e - first) : at_items + 16u * (e % RS_ITEMS);
                 #pragma unroll
                 for (int k = 0; k < KS; ++k)
-                    if (v[k] == best) { ra[k] += kpd; rb[k] += kpb; }
-                key[u] = best;
-                not_usual |= best & 1;
-                if (!Scores<KIND>::EXACT) {     // another row that can be the best
-                    int next = 0x7fffffff;
+                    if (!TAKE_OFF) { was_a[k] = ra[k]; was_b[k] = rb[k]; }
+                #pragma unroll
+                for (int u = 0; u < TRIP; ++u) {     // (items from `limit` on are whatever the slots hold: what is done with them is taken back)
+                    const int kp = it0.x, kpd = it0.y, kpb = LISTS ? it0.w : it0.x + it0.y;
+                    int v[KS];
                     #pragma unroll
-                    for (int k = 0; k < KS; ++k) next = min(next, v[k] == best ? 0x7fffffff : v[k]);
-                    next = __reduce_min_sync(FULL_MASK, next);
-                    if (next <= (best | K::TAGS) + SLACK) not_usual |= 2 << u;
+                    for (int k = 0; k < KS; ++k) v[k] = __viaddmax_s32(rb[k], kp, ra[k]);
+                    int least = LISTS ? it0.z : it0.z > jmax ? cut : (int)0x80000001u;
+                    #pragma unroll
+                    for (int k = 0; k + 1 < KS; k += 2) least = __vimin3_s32(least, v[k], v[k + 1]);
+                    const int best = __reduce_min_sync(FULL_MASK, least);
+                    // (while the reduction is under way)
+                    if (u == 0) { tell(e - TRIP, told, untold); publish(e); }     // (whether there is anything to tell or not: a branch here cost 20 cycles a step)
+                    it0 = it1; it1 = it2;
+                    it2 = ld_table(at + 16u * (u + 3));
+                    #pragma unroll
+                    for (int k = 0; k < KS; ++k)
+                        if (v[k] == (TAKE_OFF ? best & ~1 : best)) { ra[k] += kpd; rb[k] += kpb; }
+                    key[u] = best;
+                    not_usual |= best & 1;
+                    if (!Scores<KIND>::EXACT) {     // another row that can be the best
+                        int next = 0x7fffffff;
+                        #pragma unroll
+                        for (int k = 0; k < KS; ++k) next = min(next, v[k] == best ? 0x7fffffff : v[k]);
+                        next = __reduce_min_sync(FULL_MASK, next);
+                        if (next <= (best | K::TAGS) + SLACK) not_usual |= 2 << u;
+                    }
                 }
-            }
-            told = key[0];
-            #pragma unroll
-            for (int u = 1; u < TRIP; ++u) told = lane == u ? key[u] : told;
-            untold = 0;
-            if (not_usual == 0 && e + TRIP <= limit) {
-                e += TRIP;
-                untold = TRIP;
-                continue;
-            }
+                told = key[0];
+                #pragma unroll
+                for (int u = 1; u < TRIP; ++u) told = lane == u ? key[u] : told;
+                whole = not_usual == 0 && e + TRIP <= limit;
+                untold = whole ? TRIP : 0;
+                e += untold;
+            } while (whole && e < stop);
+            if (whole) break;
+            const unsigned int at = LISTS ? at_ready + 16u * (e - first) : at_items + 16u * (e % RS_ITEMS);
             // ---- the first `usual` steps of the trip stand, the others are taken back
             const int there = (int)min(limit - e, (unsigned int)TRIP);
             int usual = there;
             #pragma unroll
             for (int u = TRIP - 1; u >= 0; --u)
                 if (u < there && ((key[u] & 1) || (not_usual & (2 << u)))) usual = u;
-            #pragma unroll
-            for (int k = 0; k < KS; ++k) { ra[k] = was_a[k]; rb[k] = was_b[k]; }
-            #pragma unroll
-            for (int u = 0; u + 1 < TRIP; ++u) {
-                const int4 it = ld_table(at + 16u * u);
-                const int t = u < usual ? key[u] & K::SLOT : -1;
+            if (TAKE_OFF) {
                 #pragma unroll
-                for (int k = 0; k < KS; ++k) {
-                    ra[k] += tag(k) == t ? it.y : 0;
-                    rb[k] += tag(k) == t ? it.w : 0;
+                for (int u = 0; u < TRIP; ++u) {
+                    const int4 it = ld_table(at + 16u * u);
+                    const int t = u >= usual && (key[u] & 1) == 0 ? key[u] & K::SLOT : -1;
+                    #pragma unroll
+                    for (int k = 0; k < KS; ++k) {
+                        ra[k] -= tag(k) == t ? it.y : 0;
+                        rb[k] -= tag(k) == t ? it.w : 0;
+                    }
+                }
+            } else {
+                #pragma unroll
+                for (int k = 0; k < KS; ++k) { ra[k] = was_a[k]; rb[k] = was_b[k]; }
+                #pragma unroll
+                for (int u = 0; u + 1 < TRIP; ++u) {
+                    const int4 it = ld_table(at + 16u * u);
+                    const int t = u < usual ? key[u] & K::SLOT : -1;
+                    #pragma unroll
+                    for (int k = 0; k < KS; ++k) {
+                        ra[k] += tag(k) == t ? it.y : 0;
+                        rb[k] += tag(k) == t ? (LISTS ? it.w : it.x + it.y) : 0;
+                    }
                 }
             }
             tell(e, told, usual);
             e += usual;
             publish(e);
-            if (usual < there)
+            if (usual < there) {
+                // The two usual reasons, each without the look at everything: the winner was marked when it was last read, and a row outside the list could do
+                // as well.  (An arrival of 64 x 256 that is not usual: 670 cycles by `unusual` alone.)
+                int won = key[0];
+                #pragma unroll
+                for (int u = 1; u < TRIP; ++u) won = u == usual ? key[u] : won;
+                const int4 it = item_at(e, 0);
+                const int beyond = LISTS ? it.z : it.z > jmax ? cut : (int)0x80000001u;
+                bool again = false;
+                if (won != beyond && (won & 1)) {
+                    const unsigned int* word = sh.pending + ((won & K::SLOT) >> 1);
+                    if (__any_sync(FULL_MASK, ld_acquire(word) != 0) && !rs_wait(sh, [&] { return ld_acquire(word) == 0; })) { lost = true; break; }
+                    refresh();
+                    bool marked = false;
+                    #pragma unroll
+                    for (int k = 0; k < KS; ++k) marked |= tag(k) == (won & K::SLOT) && (ra[k] & 1) != 0;
+                    again = !__any_sync(FULL_MASK, marked);      // (else it is far)
+                } else if (LISTS && won == beyond && won != (int)0x80000001u && won != cut && tried_at != e) {
+                    tried_at = e; lists_tried = 1;
+                    next_list(e);
+                    again = true;
+                }
+                if (lost) break;
+                if (again) { fetch(e, stop); continue; }
                 do {      // (no trip for the next arrival either while it does not reach every row's top)
                     if (unusual(e)) { ++e; publish(e); }
                     else if (lost) break;
-                    else refresh();
                 } while (e < stop && __any_sync(FULL_MASK, sh.items[e % RS_ITEMS].z <= jmax));
+            }
             if (lost) break;
-            fetch(e);
+            fetch(e, stop);
         }
         tell(e - TRIP, told, untold);
         publish(e);
@@ -2151,22 +2278,16 @@ __device__ __noinline__ int rs_settle(const RouteSumArgs& a, RsShared& sh, const
 
 // The batch by the block's warps, with the keys of KIND.  False: left to the scanning kernel.
 template <int KS, bool LISTS, bool ADMIT, int KIND>
-__device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Cells& cells, const Batch& b, long long& decided) {
+__device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Cells& cells, const Batch& b, unsigned int go, long long& decided) {
     typedef Shape<KS, LISTS> Sp;
     constexpr int THREADS = Sp::THREADS;
     const int I = a.I, H = a.H, tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(FULL_MASK, tid >> 5, 0);
     const bool alone = b.alone;
-    const unsigned long long mean_l = b.ramps / (unsigned long long)(b.n_items > 0 ? b.n_items : 1);
-    const int mean = mean_l < (1ull << 22) ? (int)mean_l : 1 << 22;     // prompt + ramp of a typical request
-    Scores<KIND> sc;
-    sc.start(a.theta, a.beta, b.peak_bound, b.max_pd, b.max_p, (b.base_sum + b.tokens_in) / (unsigned long long)I, mean, Held<KS>::ITEM);
+    const Scores<KIND> sc = rs_scores<KS, KIND>(a, b);
     {
         unsigned int jmax = 0, n_far = 0;
         int free_rows = 0;
-        constexpr int PROBES = LISTS ? RS_PROBES : 1;      // (the first one: an empty prompt)
-        int least[PROBES];                     // the smallest value per probe, for the first list
-        #pragma unroll
-        for (int p = 0; p < PROBES; ++p) least[p] = 0x7f000000;
+        int least = 0x7f000000;                // the smallest score of an empty prompt
         if (Sp::SELF && !alone)
             for (int i = tid; i < 32 * I; i += THREADS) { cells.near[i] = a.near[i]; cells.far[i] = a.far[i]; }
         for (int i = tid; i < I; i += THREADS) {
@@ -2192,8 +2313,7 @@ __device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, co
             if (alone) sh.pending[i] = 0;
             if (!Scores<KIND>::WHOLE) rows.tok[i] = q.x;
             a.newest[i] = RS_NOBODY;
-            #pragma unroll
-            for (int p = 0; p < PROBES; ++p) least[p] = min(least[p], max(rec.x, rec.y + sc.key_p(rs_probe(mean, p))));
+            least = min(least, max(rec.x, rec.y));
         }
         jmax = __reduce_max_sync(FULL_MASK, jmax);
         if (lane == 0 && jmax) atomicMax(&sh.jmax, jmax);
@@ -2201,11 +2321,8 @@ __device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, co
             n_far = __reduce_add_sync(FULL_MASK, n_far);
             if (lane == 0 && n_far) atomicAdd(&sh.n_far, n_far);
         }
-        #pragma unroll
-        for (int p = 0; p < PROBES; ++p) {
-            const int v = __reduce_min_sync(FULL_MASK, least[p]);
-            if (lane == 0) atomicMin(&sh.probe_t[p], ordered(v));
-        }
+        least = __reduce_min_sync(FULL_MASK, least);
+        if (lane == 0) atomicMin(&sh.least, ordered(least));
         if (ADMIT) {
             free_rows = __reduce_add_sync(FULL_MASK, free_rows);
             if (lane == 0 && free_rows) atomicAdd(&sh.not_over, (unsigned int)free_rows);
@@ -2215,22 +2332,21 @@ __device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, co
     __syncthreads();
     if (LISTS && a.may_decline) {
         unsigned int n_least = 0;
-        for (int i = tid; i < I; i += THREADS) n_least += max(rows.rec[i].x, rows.rec[i].y) <= unordered(sh.probe_t[0]) + Scores<KIND>::SLACK;
+        for (int i = tid; i < I; i += THREADS) n_least += max(rows.rec[i].x, rows.rec[i].y) <= unordered(sh.least) + Scores<KIND>::SLACK;
         n_least = __reduce_add_sync(FULL_MASK, n_least);
         if (lane == 0 && n_least) atomicAdd(&sh.n_least, n_least);
         __syncthreads();
         if ((H > RS_FAR_STEPS && sh.n_far > (unsigned int)(I / RS_FAR_SHARE)) || sh.n_least > 32u * KS || sc.shift < RS_COARSE_SHIFT) return false;
     }
 
+    if (LISTS && tid == 0) st_release_cluster(other_smem(&sh.lists_go, 1), go);      // (the rows' keys and sh.batch can be read)
     const int role = (warp >> 2) * 3 + (warp & 3) - 1;      // (of the warps that are not on the deciding warp's scheduler)
     if (warp == 0) {
         rs_decide_loop<KS, LISTS, Sp::FOLD, ADMIT, KIND>(a, sh, rows, sc, cells);
     } else if ((warp & 3) != 0) {
         if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, KIND, LISTS, Sp::SELF>(a, sh, rows, sc, cells, role);
         else if (role == Sp::FOLD)
-            rs_io_loop<KS, Sp::DONE, ADMIT, KIND>(a, sh, sc, b.q_head, (int)b.q_len, (int)b.n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
-        else if (LISTS && role <= Sp::FOLD + Sp::LIST)
-            rs_list_loop<LISTS ? Sp::LIST : 4, KS, KIND>(sh, rows, sc, a.near, a.far, I, mean, sc.key_p(b.max_pd < (1ull << 29) ? (int)b.max_pd : 1 << 29), lane + 32 * (role - Sp::FOLD - 1));
+            rs_io_loop<KS, LISTS, Sp::DONE, ADMIT, KIND>(a, sh, sc, b.q_head, (int)b.q_len, (int)b.n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
     }
     __syncthreads();
     if (sh.ctl.w) {     // (all threads alike: nobody writes it any more)
@@ -2271,7 +2387,33 @@ __device__ __noinline__ long long rs_route_apart(const RouteSumArgs& a) {
     const Rows rows = rs_rows(a.I);
     const Batch b = rs_block().batch;
     long long decided = b.n_items;
-    return rs_route<KS, LISTS, ADMIT, KIND>(a, rs_block(), rows, rs_cells<Shape<KS, LISTS>::SELF>(a, rows), b, decided) ? decided : -1;
+    return rs_route<KS, LISTS, ADMIT, KIND>(a, rs_block(), rows, rs_cells<Shape<KS, LISTS>::SELF>(a, rows), b, RS_GO_APART, decided) ? decided : -1;
+}
+
+// What the list block does; it touches no memory but the two blocks' own.
+template <int KS, int KIND, int OTHER_KS, int OTHER>
+__device__ __forceinline__ void rs_list_block(const RouteSumArgs& a, RsShared& sh, const Rows& rows) {
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        sh.lists_wanted = sh.lists_go = 0;
+        sh.idle_limit = rs_idle_limit(a.spin_limit);
+    }
+    __syncthreads();
+    cluster_arrive();
+    cluster_wait();
+    // (What the routing block does until it says what to build ends by itself: no limit is needed here but the one of a warp without work.)
+    unsigned int go = 0;
+    if (tid < 32)
+        for (unsigned int polls = 0; __any_sync(FULL_MASK, (go = ld_acquire_cluster(&sh.lists_go)) == 0) && polls < sh.idle_limit; ++polls) __nanosleep(100);
+    if (tid == 0) sh.list_take[0] = (int)go;
+    __syncthreads();
+    go = (unsigned int)sh.list_take[0];
+    __syncthreads();
+    if (go == RS_GO_USUAL) rs_build_lists<KS, KIND>(a, sh, rows);
+    else if (go == RS_GO_APART && (OTHER != KIND || OTHER_KS != KS)) rs_build_lists<OTHER_KS, OTHER>(a, sh, rows);
+    __syncthreads();
+    cluster_arrive();
+    cluster_wait();
 }
 
 template <int KS, bool LISTS, bool ADMIT, int KIND>
@@ -2286,6 +2428,13 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
     // (the warp's number by a shuffle: the compiler then knows that the roles part between warps and not within one, and
     // leaves out what would bring the lanes of a warp together again: 157 instead of 202 cycles for a step of the deciding warp)
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(FULL_MASK, tid >> 5, 0);
+    // Which keys a batch takes that does not fit the usual ones (see RS_LONG_SHARE).
+    constexpr int OTHER_KS = LISTS && KS == 8 ? 4 : KS, OTHER = KIND == RS_WHOLE && OTHER_KS != KS ? RS_WHOLE : RS_ROUNDED;
+    static_assert(Shape<OTHER_KS, LISTS>::THREADS == THREADS, "");
+    if constexpr (LISTS) {
+        if (block_rank() != 0) { rs_list_block<KS, KIND, OTHER_KS, OTHER>(a, sh, rows); return; }
+        cluster_arrive();
+    }
     __shared__ unsigned long long sh_guard[GUARDS];
     const bool alone = !LISTS && a.alone;
     if (!alone) pre_wait_for_previous();
@@ -2317,20 +2466,19 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
         const bool exact = !Scores<KIND>::WHOLE || token_bound + max_pd + (unsigned long long)a.beta * (peak_bound + 1) < (1ull << 29);
         sh.mode = ok && exact ? 1 : 0;
         sh.spin_limit = a.spin_limit;
-        sh.idle_limit = max(a.spin_limit < (1u << 27) ? 16u * a.spin_limit : 0xffffffffu, 1u << 22);
+        sh.idle_limit = rs_idle_limit(a.spin_limit);
         sh.cursor = 0; sh.beat = 0;
         sh.n0 = *a.n_requests;
         sh.ctl = make_uint4(0u, 0u, 0u, 0u);
         sh.items_ready = sh.items_end = sh.not_over = sh.jmax = sh.n_far = sh.n_least = sh.n_beyond = sh.written = sh.flush = 0;
-        sh.lists_wanted = sh.lists_ready = sh.look_met = 0;
+        sh.lists_ready = sh.look_met = 0;
         sh.list_n[0] = sh.list_n[1] = 0;
+        sh.least = 0xffffffffu;
         sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0;
         sh.first_bad = sh.first_full = 0x7fffffff;
     }
     for (int i = tid; i < RS_ITEMS + RS_AHEAD; i += THREADS) sh.items[i] = make_int4(0, 0, 0, 0);    // (an item is fetched before it is known to be there)
     if (tid < RS_MAX_FOLD_WARPS) { sh.done[tid] = (unsigned int)tid; sh.looks_done[tid] = 0; }
-    if (tid < RS_PROBES) sh.probe_t[tid] = 0xffffffffu;
-    if (tid < 32) { sh.bucket_a[tid] = 0xffffffffu; sh.bucket_b[tid] = 0xffffffffu; }
     if (!alone)
         for (int i = tid; i < RS_LIST_ROWS; i += THREADS) sh.pending[i] = 0;
     // ADMIT: the requests that were waiting when the call was made come first, then the arrivals
@@ -2349,7 +2497,15 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
         }
         if (tid < 3) a.give_up[tid] = 0;
     };
-    if (mode == 0 && !alone) { decline(); return; }
+    // The list block leaves, and does not read this one's words any more.
+    auto part = [&]() {
+        if (!LISTS) return;
+        if (tid == 0) st_cluster(other_smem(&sh.lists_go, 1), RS_GO_LEAVE);
+        cluster_arrive();
+        cluster_wait();
+    };
+    if (LISTS) cluster_wait();      // (the list block's words are there)
+    if (mode == 0 && !alone) { decline(); part(); return; }
     if (ADMIT && a.queue_capacity > 0) {   // kept inside the ring whatever the two words hold
         if (q_head < 0 || q_head >= a.queue_capacity) q_head = 0;
         if (q_len < 0) q_len = 0;
@@ -2360,10 +2516,7 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
     if (mode == 0) {
         rs_literal<ADMIT>(a, sh, q_head, q_len, n_items);
     } else {
-    // Which keys: exact ones while the batch fits them (see RS_LONG_SHARE).
-    constexpr int OTHER_KS = LISTS && KS == 8 ? 4 : KS, OTHER = KIND == RS_WHOLE && OTHER_KS != KS ? RS_WHOLE : RS_ROUNDED;
-    static_assert(Shape<OTHER_KS, LISTS>::THREADS == THREADS, "");
-    bool exact = true;
+    bool exact = true;      // (the batch fits the usual keys)
     if (KIND != RS_ROUNDED && (KIND == RS_HALVES || OTHER == RS_WHOLE || I <= RS_MAX_BINARY64_ROWS)) {
         exact = n_long <= (unsigned long long)n_items / RS_LONG_SHARE;
         if (KIND == RS_HALVES) {
@@ -2380,15 +2533,19 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
         exact = __shfl_sync(FULL_MASK, (int)exact, 0) != 0;     // (all threads alike, and known to be)
     }
     const Batch b{peak_bound, ramps, tokens_in, max_pd, max_p, base_sum, q_head, q_len, n_items, alone};
+    if (tid == 0) sh.batch = b;
+    __syncthreads();
     bool routed;
-    if (KIND == RS_ROUNDED || exact) routed = rs_route<KS, LISTS, ADMIT, KIND>(a, sh, rows, cells, b, decided);
+    if (KIND == RS_ROUNDED || exact) routed = rs_route<KS, LISTS, ADMIT, KIND>(a, sh, rows, cells, b, RS_GO_USUAL, decided);
     else {
-        if (tid == 0) sh.batch = b;
-        __syncthreads();
         decided = rs_route_apart<OTHER_KS, LISTS, ADMIT, OTHER>(a);
         routed = decided >= 0;
     }
-    if (!routed) { decline(); return; }
+    if (!routed) { decline(); part(); return; }
+    }
+    if (LISTS) {
+        if (tid == 0) st_cluster(other_smem(&sh.lists_go, 1), RS_GO_LEAVE);
+        cluster_arrive();
     }
     const bool blocked = ADMIT && sh.blocked, dropped = !blocked && decided < n_items;
     if (blocked) decided = sh.blocked_k;
@@ -2471,6 +2628,7 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
             if (blocked && sh.any_bad) atomicOr(a.status, PRE_ST_BADREQ);
         }
     }
+    if (LISTS) cluster_wait();      // (the list block may read this one's words until then)
 }
 
 }  // namespace
@@ -2540,6 +2698,8 @@ static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* s
     if (smem + attr.sharedSizeBytes + 256 > limit) return cudaSuccess;   // too many instances
     // (the limit is shared by every context of the process: always the device maximum)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(limit - attr.sharedSizeBytes));
+    // As much L1 as that leaves: with shared memory at its maximum the rows' cells miss it (a fold's load 350 cycles instead of 80).
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
     if (e != cudaSuccess) return e;
     *smem_out = smem;
     return cudaSuccess;
@@ -2616,13 +2776,14 @@ static cudaError_t launch_summary_kernels(pre_ctx* ctx, const SumArgs& p, const 
     }
     typedef void (*Kernel)(const RouteSumArgs);
     const Kernel kernel = reinterpret_cast<Kernel>(const_cast<void*>(summaries_kernel_for<ADMIT>(ctx)));
-    const int threads = I <= RS_DIRECT_ROWS ? Shape<1, false>::THREADS : I <= RS_LONG_LISTS ? Shape<4, true>::THREADS : Shape<8, true>::THREADS;
+    const bool lists = I > RS_DIRECT_ROWS;      // (a cluster of two blocks)
+    const int threads = lists ? Shape<4, true>::THREADS : Shape<1, false>::THREADS;
     const size_t smem = ADMIT ? ctx->route_summary_smem_admit : ctx->route_summary_smem;
     if (a.alone) {
         kernel<<<1, threads, smem, s>>>(a);
         e = cudaGetLastError();
     } else {
-        e = pre_launch_behind(kernel, 1, threads, smem, s, a);
+        e = pre_launch_behind_cluster(lists ? 2 : 1, kernel, lists ? 2 : 1, threads, smem, s, a);
     }
     if (e == cudaSuccess && a.alone && !a.own_ramps) e = pre_launch_add_ramps(ctx, a.n_arrivals + a.queue_capacity, a.prompt, a.predicted, a.instance, a.curves, s);
     return e;
