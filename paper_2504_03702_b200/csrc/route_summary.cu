@@ -56,16 +56,16 @@ namespace {
 constexpr int RS_MAX_FOLD_WARPS = 10;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
 constexpr int RS_AHEAD = 8;                 // items that are fetched beyond the present one, at most
-constexpr int RS_READY = 64;                // items made ready for the deciding loop at once, at most
+constexpr int RS_READY = 128;               // items made ready for the deciding loop at once, at most
 // Up to so many rows the deciding warp folds its decisions itself: with few rows the next arrival mostly wants the row that was just taken. us a call,
 // by itself / by the folding warps: 2,000 arrivals on 256 steps, whole-number scores, 1 row 846 / 1,796, 4 rows 575 / 647, 6 rows 618 / 565, 20 rows
 // 561 / 278; fractional 1,028 / 1,957, 755 / 720, 778 / 627, 738 / 341; 32 arrivals on 64 steps: 4 rows 33 / 37, 8 rows 34 / 34, 32 rows 37 / 35.
 constexpr int RS_SELF_ROWS = 4;
 constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
 constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lane, 8 beyond RS_LONG_LISTS instances)
-// Lists of 256 / 128 rows, us a call, 8,192 arrivals on 1,024 steps: whole-number scores 1,025 rows 1,064 / 1,112, 1,600 1,005 / 1,095, 2,048 1,253 / 1,408;
-// fractional 1,153 / 1,168, 1,055 / 1,165, 1,328 / 1,464.
+// Lists of 256 / 128 rows, us a pass: 4,096 x 2,048 with 65,536 arrivals 7,716 / 10,926, 2,000 x 1,536 with 8,192 873 / 933; 1,024 x 1,024 with 4,096 - / 453.
 constexpr int RS_LONG_LISTS = 1024;
+constexpr int RS_FEW = 4;                   // arrivals that no list is built for: each is decided on all rows
 constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding warp looks at their keys by itself
 // Beyond RS_DIRECT_ROWS instances two kinds of batches cost this kernel more than the scanning one (which takes 2.4 us an arrival on 1,024 x
 // 1,024 whatever the rows): many far rows that may pay a penalty, whose arrivals need a look at all rows, scans, and folds of
@@ -476,7 +476,6 @@ struct RsShared {
     unsigned int flush;                     // ... and as many are asked for
     int cursor;                             // items of the batch that the io warp has looked at (when it has ended)
     unsigned int spin_limit, idle_limit;
-    unsigned int touched[32];               // (see touch_row)
     unsigned int beat;                      // moves while the io warp goes through arrivals
     unsigned int not_over;                  // ADMIT: rows that are not overloaded, as far as folded
     int blocked;                            // ADMIT: a request found every instance overloaded ...
@@ -555,8 +554,8 @@ __device__ __forceinline__ void acquire_cta() { asm volatile("fence.acq_rel.cta;
 // Polls of a warp that nothing is owed to.
 __device__ __forceinline__ unsigned int rs_idle_limit(unsigned int spin_limit) { return max(spin_limit < (1u << 27) ? 16u * spin_limit : 0xffffffffu, 1u << 22); }
 // The newest list that is there.  No acquire: what is read behind it lies in this block's shared memory and was there before the list block's release, and loads
-// of shared memory are made in order.  An acquire of the cluster empties the SM's L1 of the rows' cells (by every poll of the io warp: a fold's load took 350
-// cycles instead of 80).
+// of shared memory are made in order.  An acquire of the cluster empties the SM's L1 of the rows' cells (one per poll: a fold's load took 350 cycles instead of
+// 110 to 230).
 __device__ __forceinline__ unsigned int list_number(const RsShared& sh) {
     unsigned int v;
     asm volatile("ld.relaxed.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(&sh.lists_ready)) : "memory");
@@ -1071,7 +1070,7 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
         if (!rs_wait<true>(sh, [&] {
                 ctl = ld_volatile4(&sh.ctl);
                 return (!SELF && (int)(ctl.x - n) > 0) || ctl.y != looks || ctl.z != 0;
-            }, LISTS || SELF ? 20 : 0))
+            }, SELF ? 20 : 0))
             return;
         acquire_cta();
         if (SELF || __all_sync(FULL_MASK, (int)(ctl.x - n) <= 0)) ctl = ld_volatile4(&sh.ctl);
@@ -1103,14 +1102,7 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
 }
 
 // ---- io warp: arrivals ahead of the decisions, results behind the folds
-// Brings a row's cells into this SM's L1: the load of a fold that finds them there takes 80 cycles and 350 otherwise, of a fold's 970.
-// (prefetch.global.L1 left them in L2, and loads whose values are not used are not made: the sum goes to a word that nobody reads.)
-__device__ __forceinline__ unsigned int touch_row(const uint2* near, const unsigned int* far, int row) {
-    const unsigned int* cells = reinterpret_cast<const unsigned int*>(near + (size_t)row * 32);
-    return cells[0] ^ cells[32] ^ far[(size_t)row * 32];
-}
-
-template <int KS, bool LISTS, int FOLD_WARPS, bool ADMIT, int KIND>
+template <int KS, int FOLD_WARPS, bool ADMIT, int KIND>
 __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, const Scores<KIND>& sc, long long q_head, int waiting, int items, int room) {
     const int lane = threadIdx.x & 31;
     const long long n0 = sh.n0;
@@ -1126,19 +1118,7 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
     unsigned int written = 0;       // results written out
     int first_bad = 0x7fffffff, first_full = 0x7fffffff;
     unsigned int quiet = 0, seen = 0;      // rounds of this loop in which nothing has moved
-    unsigned int list = 0;                 // the newest one whose rows are on their way
     for (;;) {
-        if (LISTS) {      // (for the folds of its rows)
-            const unsigned int newest = __reduce_max_sync(FULL_MASK, list_number(sh));
-            if (newest != list) {
-                list = newest;
-                const int n = sh.list_n[list & 1];      // (may be none)
-                unsigned int sum = 0;
-                #pragma unroll 2
-                for (int x = lane; x < n; x += 32) sum ^= touch_row(a.near, a.far, sh.list_row[list & 1][x]);
-                sh.touched[lane] = sum;
-            }
-        }
         while (cursor < items && entered - written <= RS_ITEMS - 32) {
             const int k = cursor + lane;
             int P = -1, D = 0;
@@ -1453,7 +1433,7 @@ template <int KS, bool LISTS> struct Shape {
 // tables) is done by the folding warps.
 // us a call with both, before and after: 256 x 100 149 -> 141, 512 x 1,024 425 -> 419, 2,000 x 1,536 580 -> 544.
 template <int KS, bool LISTS, int FOLD_WARPS, bool ADMIT, int KIND>
-__device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<KIND>& sc, const Cells& cells) {
+__device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& sh, const Rows& rows, const Scores<KIND>& sc, const Cells& cells, bool few) {
     typedef typename Scores<KIND>::S S;
     typedef Held<KS> K;
     constexpr int SLACK = Scores<KIND>::SLACK * (1 << K::SLOT_BITS);
@@ -1461,7 +1441,8 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     constexpr int TRIP = 4;
     // decisions between two looks at items and at the rows that were pending; items made ready at once (a trip may begin with the last but one of a
     // chunk)
-    constexpr unsigned int READY = RS_READY, CHUNK = LISTS ? READY - TRIP : 8 * KS;
+    // (128 items / 64: 4,096 x 2,048 7,555 / 7,716 us, 2,000 x 1,536 866 / 873; lists of 128 rows, which last half as long, 512 x 1,024 861 / 846)
+    constexpr unsigned int READY = KS == 8 ? RS_READY : RS_READY / 2, CHUNK = LISTS ? READY - TRIP : 8 * KS;
     const int lane = threadIdx.x & 31, I = a.I, H = a.H;
     constexpr bool SELF = Shape<KS, LISTS>::SELF;
     const int lane_f = lane < Shape<KS, LISTS>::DONE ? lane : 0;
@@ -1569,7 +1550,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         return true;
     };
     if (LISTS) {
-        next_list(0);
+        if (!few) next_list(0);
     } else {
         take_base(unordered(sh.least) & ~1);
         unread();
@@ -1617,7 +1598,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         };
         if (tried_at != e) { tried_at = e; lists_tried = 0; }
         refresh();
-        if (it.z > jmax) {
+        if (it.z > jmax && !few) {
             // The smallest key now; where that is only a bound, or rounded, the rows that can be the best are compared.
             int key = 0x7fffffff;
             #pragma unroll
@@ -2038,6 +2019,10 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         }
         const unsigned int stop = min(limit, e + CHUNK);
         refresh();
+        if (LISTS && few) {
+            if (unusual(e)) { ++e; publish(e); }
+            continue;
+        }
         fetch(e, stop);
         int untold = 0;               // decisions before e that are not told yet (the last trip's: they are while the next reduction is under way)
         int told = 0;
@@ -2339,14 +2324,14 @@ __device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, co
         if ((H > RS_FAR_STEPS && sh.n_far > (unsigned int)(I / RS_FAR_SHARE)) || sh.n_least > 32u * KS || sc.shift < RS_COARSE_SHIFT) return false;
     }
 
-    if (LISTS && tid == 0) st_release_cluster(other_smem(&sh.lists_go, 1), go);      // (the rows' keys and sh.batch can be read)
+    if (LISTS && tid == 0 && b.n_items > RS_FEW) st_release_cluster(other_smem(&sh.lists_go, 1), go);      // (the rows' keys and sh.batch can be read)
     const int role = (warp >> 2) * 3 + (warp & 3) - 1;      // (of the warps that are not on the deciding warp's scheduler)
     if (warp == 0) {
-        rs_decide_loop<KS, LISTS, Sp::FOLD, ADMIT, KIND>(a, sh, rows, sc, cells);
+        rs_decide_loop<KS, LISTS, Sp::FOLD, ADMIT, KIND>(a, sh, rows, sc, cells, LISTS && b.n_items <= RS_FEW);
     } else if ((warp & 3) != 0) {
         if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, KIND, LISTS, Sp::SELF>(a, sh, rows, sc, cells, role);
         else if (role == Sp::FOLD)
-            rs_io_loop<KS, LISTS, Sp::DONE, ADMIT, KIND>(a, sh, sc, b.q_head, (int)b.q_len, (int)b.n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
+            rs_io_loop<KS, Sp::DONE, ADMIT, KIND>(a, sh, sc, b.q_head, (int)b.q_len, (int)b.n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
     }
     __syncthreads();
     if (sh.ctl.w) {     // (all threads alike: nobody writes it any more)
@@ -2533,8 +2518,10 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
         exact = __shfl_sync(FULL_MASK, (int)exact, 0) != 0;     // (all threads alike, and known to be)
     }
     const Batch b{peak_bound, ramps, tokens_in, max_pd, max_p, base_sum, q_head, q_len, n_items, alone};
-    if (tid == 0) sh.batch = b;
-    __syncthreads();
+    if (LISTS || !exact) {
+        if (tid == 0) sh.batch = b;
+        __syncthreads();
+    }
     bool routed;
     if (KIND == RS_ROUNDED || exact) routed = rs_route<KS, LISTS, ADMIT, KIND>(a, sh, rows, cells, b, RS_GO_USUAL, decided);
     else {
@@ -2698,8 +2685,6 @@ static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* s
     if (smem + attr.sharedSizeBytes + 256 > limit) return cudaSuccess;   // too many instances
     // (the limit is shared by every context of the process: always the device maximum)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(limit - attr.sharedSizeBytes));
-    // As much L1 as that leaves: with shared memory at its maximum the rows' cells miss it (a fold's load 350 cycles instead of 80).
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
     if (e != cudaSuccess) return e;
     *smem_out = smem;
     return cudaSuccess;
