@@ -56,7 +56,7 @@ namespace {
 constexpr int RS_MAX_FOLD_WARPS = 10;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
 constexpr int RS_AHEAD = 8;                 // items that are fetched beyond the present one, at most
-constexpr int RS_READY = 128;               // items made ready for the deciding loop at once, at most
+constexpr int RS_READY = 32;                // items made ready for the deciding loop at once, one per lane
 // Up to so many rows the deciding warp folds its decisions itself: with few rows the next arrival mostly wants the row that was just taken. us a call,
 // by itself / by the folding warps: 2,000 arrivals on 256 steps, whole-number scores, 1 row 846 / 1,796, 4 rows 575 / 647, 6 rows 618 / 565, 20 rows
 // 561 / 278; fractional 1,028 / 1,957, 755 / 720, 778 / 627, 738 / 341; 32 arrivals on 64 steps: 4 rows 33 / 37, 8 rows 34 / 34, 32 rows 37 / 35.
@@ -1441,8 +1441,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     constexpr int TRIP = 4;
     // decisions between two looks at items and at the rows that were pending; items made ready at once (a trip may begin with the last but one of a
     // chunk)
-    // (128 items / 64: 4,096 x 2,048 7,555 / 7,716 us, 2,000 x 1,536 866 / 873; lists of 128 rows, which last half as long, 512 x 1,024 861 / 846)
-    constexpr unsigned int READY = KS == 8 ? RS_READY : RS_READY / 2, CHUNK = LISTS ? READY - TRIP : 8 * KS;
+    constexpr unsigned int CHUNK = LISTS ? 64 : 8 * KS;
     const int lane = threadIdx.x & 31, I = a.I, H = a.H;
     constexpr bool SELF = Shape<KS, LISTS>::SELF;
     const int lane_f = lane < Shape<KS, LISTS>::DONE ? lane : 0;
@@ -1861,16 +1860,13 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     int4 it0, it1, it2;              // items e, e + 1, e + 2 (LISTS: see RsShared::ready)
     unsigned int first = 0;          // (LISTS) the first of the items made ready
     auto item_at = [&](unsigned int e, unsigned int x) { return ld_table(LISTS ? at_ready + 16u * (e - first + x) : at_items + 16u * (e % RS_ITEMS + x)); };
-    auto fetch = [&](unsigned int e, unsigned int stop) {
-        if (LISTS) {      // (as many as a chunk up to `stop` needs)
+    auto fetch = [&](unsigned int e) {
+        if (LISTS) {
             first = e;
             __syncwarp();
-            #pragma unroll 1
-            for (unsigned int x = 0; x < READY && (x == 0 || stop - e > x - TRIP); x += 32) {
-                const int4 it = ld_table(at_items + 16u * ((e + x + lane) % RS_ITEMS));
-                const int b = it.z > jmax ? cut : (int)0x80000001u;
-                sh.ready[x + lane] = make_int4(it.x, it.y, min(b, bound_of(ld_table(table + it.w), it.x)), it.x + it.y);
-            }
+            const int4 it = ld_table(at_items + 16u * ((e + lane) % RS_ITEMS));
+            const int b = it.z > jmax ? cut : (int)0x80000001u;
+            sh.ready[lane] = make_int4(it.x, it.y, min(b, bound_of(ld_table(table + it.w), it.x)), it.x + it.y);
             __syncwarp();
         }
         it0 = item_at(e, 0);
@@ -2023,12 +2019,13 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             if (unusual(e)) { ++e; publish(e); }
             continue;
         }
-        fetch(e, stop);
+        fetch(e);
         int untold = 0;               // decisions before e that are not told yet (the last trip's: they are while the next reduction is under way)
         int told = 0;
         while (e < stop) {
             int was_a[KS], was_b[KS], key[TRIP], not_usual = 0;
             bool whole;
+            const unsigned int until = LISTS ? min(stop, first + (RS_READY - TRIP)) : stop;      // (a trip may begin with the last but one)
             // (one loop with nothing but the trip: with the ways back from the unusual arrivals to its head a step took 104 cycles instead of 77)
             #pragma unroll 1
             do {
@@ -2070,8 +2067,11 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 whole = not_usual == 0 && e + TRIP <= limit;
                 untold = whole ? TRIP : 0;
                 e += untold;
-            } while (whole && e < stop);
-            if (whole) break;
+            } while (whole && e < until);
+            if (whole) {
+                if (LISTS && e < stop) fetch(e);
+                continue;
+            }
             const unsigned int at = LISTS ? at_ready + 16u * (e - first) : at_items + 16u * (e % RS_ITEMS);
             // ---- the first `usual` steps of the trip stand, the others are taken back
             const int there = (int)min(limit - e, (unsigned int)TRIP);
@@ -2108,15 +2108,15 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             e += usual;
             publish(e);
             if (usual < there) {
-                // The two usual reasons, each without the look at everything: the winner was marked when it was last read, and a row outside the list could do
-                // as well.  (An arrival of 64 x 256 that is not usual: 670 cycles by `unusual` alone.)
+                // The usual reason, without the look at everything: the winner was marked when it was last read (all rows held; an arrival of 64 x 256 that is not usual takes 670
+                // cycles by `unusual` alone), or a row outside the list could do as well.  (Lists whose far rows win by the dozen lose by a look at the mark first.)
                 int won = key[0];
                 #pragma unroll
                 for (int u = 1; u < TRIP; ++u) won = u == usual ? key[u] : won;
                 const int4 it = item_at(e, 0);
                 const int beyond = LISTS ? it.z : it.z > jmax ? cut : (int)0x80000001u;
                 bool again = false;
-                if (won != beyond && (won & 1)) {
+                if (!LISTS && won != beyond && (won & 1)) {
                     const unsigned int* word = sh.pending + ((won & K::SLOT) >> 1);
                     if (__any_sync(FULL_MASK, ld_acquire(word) != 0) && !rs_wait(sh, [&] { return ld_acquire(word) == 0; })) { lost = true; break; }
                     refresh();
@@ -2130,14 +2130,14 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                     again = true;
                 }
                 if (lost) break;
-                if (again) { fetch(e, stop); continue; }
+                if (again) { fetch(e); continue; }
                 do {      // (no trip for the next arrival either while it does not reach every row's top)
                     if (unusual(e)) { ++e; publish(e); }
                     else if (lost) break;
                 } while (e < stop && __any_sync(FULL_MASK, sh.items[e % RS_ITEMS].z <= jmax));
             }
             if (lost) break;
-            fetch(e, stop);
+            fetch(e);
         }
         tell(e - TRIP, told, untold);
         publish(e);
@@ -2685,6 +2685,8 @@ static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* s
     if (smem + attr.sharedSizeBytes + 256 > limit) return cudaSuccess;   // too many instances
     // (the limit is shared by every context of the process: always the device maximum)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(limit - attr.sharedSizeBytes));
+    // As much L1 as that leaves, for the rows' cells that the folds read: 512 x 1,024 896 -> 838 us.
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
     if (e != cudaSuccess) return e;
     *smem_out = smem;
     return cudaSuccess;

@@ -622,3 +622,35 @@ def test_batches_that_do_not_fit_exact_keys(kind, n_inst):
 def test_batches_that_do_not_fit_exact_keys_are_not_decided_one_by_one_on_all_rows(n_inst, kind, limit):
     """Two thirds of the limit or less; with exact keys (the arrivals that do not fit, or all rows that count as far, outside the loop) well above it."""
     assert share_of_the_scanning_time(*long_prompts(n_inst, 2048, *LONG[kind])) < limit
+
+
+@pytest.mark.parametrize("n_inst", [257, 300, 1100, 4200])
+@pytest.mark.parametrize("n_arr", [1, 4, 5, 9])
+@pytest.mark.parametrize("beta", [1.0, 0.75])
+def test_a_few_arrivals_on_many_instances(n_inst, n_arr, beta):
+    """Both sides of the line up to which no list is built; several batches, short arrivals among them."""
+    wl = W.make_random(71, n_inst, 40, 12 * n_inst, 0, max_prompt=300, max_output=60, beta=beta)
+    rng = np.random.default_rng(n_arr)
+    ap = rng.integers(0, 300, 3 * n_arr).astype(np.int32)
+    ad = np.where(rng.random(3 * n_arr) < 0.3, rng.integers(1, 8, 3 * n_arr), rng.integers(8, 60, 3 * n_arr)).astype(np.int32)
+    wl.max_requests = 12 * n_inst + 3 * n_arr
+    route_and_compare(wl, ap, ad, batches=3)
+
+
+# the smallest list service, a whole number of passes of the list block and one more, both sides of the line between lists of 128 and of
+# 256 rows (and between lists of all rows and of the near ones)
+@pytest.mark.parametrize("n_inst", [257, 512, 513, 1024, 1025, 2049])
+@pytest.mark.parametrize("beta,t_mem", [(1.0, 0.8), (0.75, 0.8), (0.3, 0.81237)])
+@pytest.mark.parametrize("skew", [False, True])
+def test_many_lists_in_one_batch(n_inst, beta, t_mem, skew):
+    h, n = 40, 24 * n_inst
+    wl = W.make_random(72, n_inst, h, n, 0, max_prompt=400, max_output=h, beta=beta)
+    wl.t_mem = t_mem
+    rng = np.random.default_rng(n_inst)
+    if skew:
+        wl.instance[:] = np.minimum(n_inst * rng.random(n) ** 3, n_inst - 1).astype(np.int32)
+    n_arr = 2200
+    ap = np.where(rng.random(n_arr) < 0.02, rng.integers(3000, 6000, n_arr), rng.integers(1, 400, n_arr)).astype(np.int32)
+    ad = np.where(rng.random(n_arr) < 0.02, 1, rng.integers(1, 2 * h, n_arr)).astype(np.int32)
+    wl.max_requests = n + n_arr
+    route_and_compare(wl, ap, ad)
