@@ -44,10 +44,10 @@ METRIC_STREAM = "routes/sec over the whole stream (decode step + routing of the 
 ROUTE_DRAM_READ = {3: 67322880}
 # profiles/ncu_dram_route_summary_kernels_config3_full_batch.txt: the three kernels of the summary router on the full
 # batch (the traffic does not grow in proportion to the batch, so the figure is used for the full batch only)
-ROUTE_SUMMARY_DRAM_TRAFFIC = {(3, 65536): 67736576 + 381440 + 2255616 + 50708224 + 2829568}
+ROUTE_SUMMARY_DRAM_TRAFFIC = {(3, 65536): 67736576 + 349696 + 2059520 + 50737664 + 2790656}
 # warp instructions per arrival of pre_route_summaries (smsp__inst_executed.sum of the 2,048-arrival capture in
-# profiles/ncu_full_step_kernels_config3_2048_arrivals.txt: 987,740 / 2,048)
-ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL = {3: 987740 / 2048}
+# profiles/ncu_full_step_kernels_config3_2048_arrivals.txt: 1,062,765 / 2,048)
+ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL = {3: 1062765 / 2048}
 ROUTE_DRAM_WRITE_PER_ARRIVAL = {3: 679168 / 256}
 ANTICIPATE_DRAM_TRAFFIC = {3: 33812992 + 19587328}
 STEP_DRAM_TRAFFIC = {3: 33670144 + 67196928 + 9366528}
@@ -658,7 +658,7 @@ def route_scan_roofline(wl, index, t_route_ms, n_arrivals, map_max, layout, rout
 def route_summary_roofline(wl, index, t_route_ms, n_arrivals, clocks):
     """The summary router: rows' numbers, the routing block, the batch's ramps.  The routing block is bound by the chain of
     dependent instructions of its deciding warp, not by any bandwidth; where the instructions per arrival are known from an
-    ncu capture the roof quoted is the instruction issue of the ONE SM the block runs on."""
+    ncu capture the roof quoted is the instruction issue of the SMs its block, and beyond 256 instances the list block, run on."""
     i, h = wl.n_instances, wl.horizon
     mhz = clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or 1965.0
     sec = t_route_ms * 1e-3
@@ -666,8 +666,9 @@ def route_summary_roofline(wl, index, t_route_ms, n_arrivals, clocks):
     traffic = ROUTE_SUMMARY_DRAM_TRAFFIC.get((index, n_arrivals))
     hbm_peak, kind = measured_peak_gbs()
     inst = ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL.get(index)
-    # 4 warp instructions per clock of the SM
-    issue_peak = 4 * mhz * 1e6 / 1e9
+    # 4 warp instructions per clock of an SM
+    sms = 2 if i > 256 else 1
+    issue_peak = sms * 4 * mhz * 1e6 / 1e9
     issued = None if inst is None else inst * n_arrivals / sec / 1e9
     return {
         "traffic": traffic, "kernel": "pre_summarise_rows + pre_route_summaries + pre_route_persistent (ramps)",
@@ -676,13 +677,13 @@ def route_summary_roofline(wl, index, t_route_ms, n_arrivals, clocks):
         "hbm_frac_of_captured_traffic": None if traffic is None else traffic / sec / 1e9 / hbm_peak,
         "limiter": "latency: arrivals are decided one after another by one warp (one warp reduction and some eight dependent "
                    "instructions each); neither a memory nor the instruction issue is saturated",
-        "note": "decisions are taken from two numbers per row instead of scanning the maps (identical decisions), by ONE block; "
+        "note": "decisions are taken from two numbers per row instead of scanning the maps (identical decisions), by one block and one that builds its lists; "
                 "scan_equivalent_gbs is the literal formulation's 8 bytes per cell and arrival over time, a convenience "
                 "number that is not memory traffic; traffic = DRAM bytes of the call's kernels from the ncu capture of this "
                 f"batch ({kind} HBM peak {hbm_peak:.0f} GB/s for hbm_frac_of_captured_traffic)",
         "bound": "alu", "achieved": issued, "peak": issue_peak, "unit": "G warp-instructions/s",
         "frac": None if issued is None else issued / issue_peak,
-        "peak_kind": f"derived: 1 SM x 4 schedulers x 1 warp instruction per clock x {mhz:.0f} MHz (SM clock sampled during "
+        "peak_kind": f"derived: {sms} SM x 4 schedulers x 1 warp instruction per clock x {mhz:.0f} MHz (SM clock sampled during "
                      "the timed region)",
         "warp_instructions_per_arrival": inst}
 
