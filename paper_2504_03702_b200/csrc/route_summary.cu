@@ -56,16 +56,18 @@ namespace {
 constexpr int RS_MAX_FOLD_WARPS = 10;
 constexpr int RS_ITEMS = 256;               // arrivals and decisions between the io warp, the deciding warp and the folding warps
 constexpr int RS_AHEAD = 8;                 // items that are fetched beyond the present one, at most
-constexpr int RS_READY = 32;                // items made ready for the deciding loop at once, one per lane
+constexpr int RS_READY = 64;                // items made ready for the deciding loop at once, at most
 // Up to so many rows the deciding warp folds its decisions itself: with few rows the next arrival mostly wants the row that was just taken. us a call,
 // by itself / by the folding warps: 2,000 arrivals on 256 steps, whole-number scores, 1 row 846 / 1,796, 4 rows 575 / 647, 6 rows 618 / 565, 20 rows
 // 561 / 278; fractional 1,028 / 1,957, 755 / 720, 778 / 627, 738 / 341; 32 arrivals on 64 steps: 4 rows 33 / 37, 8 rows 34 / 34, 32 rows 37 / 35.
 constexpr int RS_SELF_ROWS = 4;
 constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
 constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lane, 8 beyond RS_LONG_LISTS instances)
-// Lists of 256 / 128 rows, us a pass: 4,096 x 2,048 with 65,536 arrivals 7,716 / 10,926, 2,000 x 1,536 with 8,192 873 / 933; 1,024 x 1,024 with 4,096 - / 453.
+// Lists of 256 / 128 rows, us a pass: 4,096 x 2,048 with 65,536 arrivals 7,716 / 10,926, 2,000 x 1,536 with 8,192 873 / 933.
 constexpr int RS_LONG_LISTS = 1024;
-constexpr int RS_FEW = 4;                   // arrivals that no list is built for: each is decided on all rows
+// Arrivals that no list is built for: each is decided on all rows.  us a cycle of four ticks, with lists / so: 1 arrival on 300 rows 157 / 141, on 4,096 245 / 190;
+// 4 arrivals 168 / 163 and 260 / 248, on 1,000 rows 188 / 191.
+constexpr int RS_FEW = 4;
 constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding warp looks at their keys by itself
 // Beyond RS_DIRECT_ROWS instances two kinds of batches cost this kernel more than the scanning one (which takes 2.4 us an arrival on 1,024 x
 // 1,024 whatever the rows): many far rows that may pay a penalty, whose arrivals need a look at all rows, scans, and folds of
@@ -476,6 +478,7 @@ struct RsShared {
     unsigned int flush;                     // ... and as many are asked for
     int cursor;                             // items of the batch that the io warp has looked at (when it has ended)
     unsigned int spin_limit, idle_limit;
+    unsigned int touched[32];               // (see touch_row)
     unsigned int beat;                      // moves while the io warp goes through arrivals
     unsigned int not_over;                  // ADMIT: rows that are not overloaded, as far as folded
     int blocked;                            // ADMIT: a request found every instance overloaded ...
@@ -1102,7 +1105,14 @@ __device__ __forceinline__ void rs_fold_loop(const RouteSumArgs& a, RsShared& sh
 }
 
 // ---- io warp: arrivals ahead of the decisions, results behind the folds
-template <int KS, int FOLD_WARPS, bool ADMIT, int KIND>
+// Brings a row's cells into this SM's L1: the load of a fold that finds them there takes 80 cycles and 350 otherwise, of a fold's 970.
+// (prefetch.global.L1 left them in L2, and loads whose values are not used are not made: the sum goes to a word that nobody reads.)
+__device__ __forceinline__ unsigned int touch_row(const uint2* near, const unsigned int* far, int row) {
+    const unsigned int* cells = reinterpret_cast<const unsigned int*>(near + (size_t)row * 32);
+    return cells[0] ^ cells[32] ^ far[(size_t)row * 32];
+}
+
+template <int KS, bool LISTS, int FOLD_WARPS, bool ADMIT, int KIND>
 __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, const Scores<KIND>& sc, long long q_head, int waiting, int items, int room) {
     const int lane = threadIdx.x & 31;
     const long long n0 = sh.n0;
@@ -1118,7 +1128,19 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
     unsigned int written = 0;       // results written out
     int first_bad = 0x7fffffff, first_full = 0x7fffffff;
     unsigned int quiet = 0, seen = 0;      // rounds of this loop in which nothing has moved
+    unsigned int list = 0;                 // the newest one whose rows are on their way
     for (;;) {
+        if (LISTS) {      // (for the folds of its rows)
+            const unsigned int newest = __reduce_max_sync(FULL_MASK, list_number(sh));
+            if (newest != list) {
+                list = newest;
+                const int n = sh.list_n[list & 1];      // (may be none)
+                unsigned int sum = 0;
+                #pragma unroll 2
+                for (int x = lane; x < n; x += 32) sum ^= touch_row(a.near, a.far, sh.list_row[list & 1][x]);
+                sh.touched[lane] = sum;
+            }
+        }
         while (cursor < items && entered - written <= RS_ITEMS - 32) {
             const int k = cursor + lane;
             int P = -1, D = 0;
@@ -1441,7 +1463,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     constexpr int TRIP = 4;
     // decisions between two looks at items and at the rows that were pending; items made ready at once (a trip may begin with the last but one of a
     // chunk)
-    constexpr unsigned int CHUNK = LISTS ? 64 : 8 * KS;
+    constexpr unsigned int READY = RS_READY, CHUNK = LISTS ? READY - TRIP : 8 * KS;
     const int lane = threadIdx.x & 31, I = a.I, H = a.H;
     constexpr bool SELF = Shape<KS, LISTS>::SELF;
     const int lane_f = lane < Shape<KS, LISTS>::DONE ? lane : 0;
@@ -1860,13 +1882,16 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     int4 it0, it1, it2;              // items e, e + 1, e + 2 (LISTS: see RsShared::ready)
     unsigned int first = 0;          // (LISTS) the first of the items made ready
     auto item_at = [&](unsigned int e, unsigned int x) { return ld_table(LISTS ? at_ready + 16u * (e - first + x) : at_items + 16u * (e % RS_ITEMS + x)); };
-    auto fetch = [&](unsigned int e) {
-        if (LISTS) {
+    auto fetch = [&](unsigned int e, unsigned int stop) {
+        if (LISTS) {      // (as many as a chunk up to `stop` needs)
             first = e;
             __syncwarp();
-            const int4 it = ld_table(at_items + 16u * ((e + lane) % RS_ITEMS));
-            const int b = it.z > jmax ? cut : (int)0x80000001u;
-            sh.ready[lane] = make_int4(it.x, it.y, min(b, bound_of(ld_table(table + it.w), it.x)), it.x + it.y);
+            #pragma unroll 1
+            for (unsigned int x = 0; x < READY && (x == 0 || stop - e > x - TRIP); x += 32) {
+                const int4 it = ld_table(at_items + 16u * ((e + x + lane) % RS_ITEMS));
+                const int b = it.z > jmax ? cut : (int)0x80000001u;
+                sh.ready[x + lane] = make_int4(it.x, it.y, min(b, bound_of(ld_table(table + it.w), it.x)), it.x + it.y);
+            }
             __syncwarp();
         }
         it0 = item_at(e, 0);
@@ -2019,13 +2044,12 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             if (unusual(e)) { ++e; publish(e); }
             continue;
         }
-        fetch(e);
+        fetch(e, stop);
         int untold = 0;               // decisions before e that are not told yet (the last trip's: they are while the next reduction is under way)
         int told = 0;
         while (e < stop) {
             int was_a[KS], was_b[KS], key[TRIP], not_usual = 0;
             bool whole;
-            const unsigned int until = LISTS ? min(stop, first + (RS_READY - TRIP)) : stop;      // (a trip may begin with the last but one)
             // (one loop with nothing but the trip: with the ways back from the unusual arrivals to its head a step took 104 cycles instead of 77)
             #pragma unroll 1
             do {
@@ -2067,11 +2091,8 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 whole = not_usual == 0 && e + TRIP <= limit;
                 untold = whole ? TRIP : 0;
                 e += untold;
-            } while (whole && e < until);
-            if (whole) {
-                if (LISTS && e < stop) fetch(e);
-                continue;
-            }
+            } while (whole && e < stop);
+            if (whole) break;
             const unsigned int at = LISTS ? at_ready + 16u * (e - first) : at_items + 16u * (e % RS_ITEMS);
             // ---- the first `usual` steps of the trip stand, the others are taken back
             const int there = (int)min(limit - e, (unsigned int)TRIP);
@@ -2108,15 +2129,15 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
             e += usual;
             publish(e);
             if (usual < there) {
-                // The usual reason, without the look at everything: the winner was marked when it was last read (all rows held; an arrival of 64 x 256 that is not usual takes 670
-                // cycles by `unusual` alone), or a row outside the list could do as well.  (Lists whose far rows win by the dozen lose by a look at the mark first.)
+                // The two usual reasons, each without the look at everything: the winner was marked when it was last read, and a row outside the list could do
+                // as well.  (An arrival of 64 x 256 that is not usual: 670 cycles by `unusual` alone.)
                 int won = key[0];
                 #pragma unroll
                 for (int u = 1; u < TRIP; ++u) won = u == usual ? key[u] : won;
                 const int4 it = item_at(e, 0);
                 const int beyond = LISTS ? it.z : it.z > jmax ? cut : (int)0x80000001u;
                 bool again = false;
-                if (!LISTS && won != beyond && (won & 1)) {
+                if (won != beyond && (won & 1)) {
                     const unsigned int* word = sh.pending + ((won & K::SLOT) >> 1);
                     if (__any_sync(FULL_MASK, ld_acquire(word) != 0) && !rs_wait(sh, [&] { return ld_acquire(word) == 0; })) { lost = true; break; }
                     refresh();
@@ -2130,14 +2151,14 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                     again = true;
                 }
                 if (lost) break;
-                if (again) { fetch(e); continue; }
+                if (again) { fetch(e, stop); continue; }
                 do {      // (no trip for the next arrival either while it does not reach every row's top)
                     if (unusual(e)) { ++e; publish(e); }
                     else if (lost) break;
                 } while (e < stop && __any_sync(FULL_MASK, sh.items[e % RS_ITEMS].z <= jmax));
             }
             if (lost) break;
-            fetch(e);
+            fetch(e, stop);
         }
         tell(e - TRIP, told, untold);
         publish(e);
@@ -2331,7 +2352,7 @@ __device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, co
     } else if ((warp & 3) != 0) {
         if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, KIND, LISTS, Sp::SELF>(a, sh, rows, sc, cells, role);
         else if (role == Sp::FOLD)
-            rs_io_loop<KS, Sp::DONE, ADMIT, KIND>(a, sh, sc, b.q_head, (int)b.q_len, (int)b.n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
+            rs_io_loop<KS, LISTS, Sp::DONE, ADMIT, KIND>(a, sh, sc, b.q_head, (int)b.q_len, (int)b.n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
     }
     __syncthreads();
     if (sh.ctl.w) {     // (all threads alike: nobody writes it any more)
@@ -2685,7 +2706,7 @@ static cudaError_t summaries_configure_one(pre_ctx* ctx, size_t limit, size_t* s
     if (smem + attr.sharedSizeBytes + 256 > limit) return cudaSuccess;   // too many instances
     // (the limit is shared by every context of the process: always the device maximum)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(limit - attr.sharedSizeBytes));
-    // As much L1 as that leaves, for the rows' cells that the folds read: 512 x 1,024 896 -> 838 us.
+    // As much L1 as that leaves: with shared memory at its maximum the rows' cells miss it (a fold's load 350 cycles instead of 80).
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
     if (e != cudaSuccess) return e;
     *smem_out = smem;
