@@ -175,22 +175,24 @@ __device__ __forceinline__ void pre_flush_counts(const unsigned int* sh, unsigne
 // touches memory.
 __device__ __forceinline__ void pre_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pre_wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-template <typename... Params, typename... Args>
-cudaError_t pre_launch_behind_cluster(int cluster, void (*kernel)(Params...), int grid, int block, size_t smem, cudaStream_t s, Args... args) {
+struct PreBehind {       // (not to be copied: the configuration points to the attributes)
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned int)grid); cfg.blockDim = dim3((unsigned int)block);
-    cfg.dynamicSmemBytes = smem; cfg.stream = s;
     cudaLaunchAttribute attr[2] = {};
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned int)cluster; attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
-}
+    PreBehind(int cluster, int grid, int block, size_t smem, cudaStream_t s) {
+        cfg.gridDim = dim3((unsigned int)grid); cfg.blockDim = dim3((unsigned int)block);
+        cfg.dynamicSmemBytes = smem; cfg.stream = s;
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned int)cluster; attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
+    }
+    PreBehind(const PreBehind&) = delete;
+};
 template <typename... Params, typename... Args>
 cudaError_t pre_launch_behind(void (*kernel)(Params...), int grid, int block, size_t smem, cudaStream_t s, Args... args) {
-    return pre_launch_behind_cluster(1, kernel, grid, block, smem, s, args...);
+    const PreBehind behind(1, grid, block, smem, s);
+    return cudaLaunchKernelEx(&behind.cfg, kernel, Params(args)...);
 }
 
 __device__ __forceinline__ bool pre_request_ok(int32_t P, int32_t g, int32_t D, int32_t inst, int32_t I) {
