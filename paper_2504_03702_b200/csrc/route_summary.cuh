@@ -2017,95 +2017,92 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         }
         const unsigned int stop = min(limit, e + CHUNK);
         refresh();
-        if (LISTS && few) {
-            if (unusual(e)) { ++e; publish(e); }
-            continue;
-        }
-        fetch(e, stop);
+        if (!LISTS || !few) fetch(e, stop);
         int untold = 0;               // decisions before e that are not told yet (the last trip's: they are while the next reduction is under way)
         int told = 0;
         while (e < stop) {
-            int was_a[KS], was_b[KS], key[TRIP], not_usual = 0;
-            bool whole;
-            // (one loop with nothing but the trip: with the ways back from the unusual arrivals to its head a step took 104 cycles instead of 77)
-            #pragma unroll 1
-            do {
-                not_usual = 0;
-                const unsigned int at = LISTS ? at_ready + 16u * (e - first) : at_items + 16u * (e % RS_ITEMS);
-                #pragma unroll
-                for (int k = 0; k < KS; ++k)
-                    if (!TAKE_OFF) { was_a[k] = ra[k]; was_b[k] = rb[k]; }
-                #pragma unroll
-                for (int u = 0; u < TRIP; ++u) {     // (items from `limit` on are whatever the slots hold: what is done with them is taken back)
-                    const int kp = it0.x, kpd = it0.y, kpb = LISTS ? it0.w : it0.x + it0.y;
-                    int v[KS];
-                    #pragma unroll
-                    for (int k = 0; k < KS; ++k) v[k] = __viaddmax_s32(rb[k], kp, ra[k]);
-                    int least = LISTS ? it0.z : it0.z > jmax ? cut : (int)0x80000001u;
-                    #pragma unroll
-                    for (int k = 0; k + 1 < KS; k += 2) least = __vimin3_s32(least, v[k], v[k + 1]);
-                    const int best = __reduce_min_sync(FULL_MASK, least);
-                    // (while the reduction is under way)
-                    if (u == 0) { tell(e - TRIP, told, untold); publish(e); }     // (whether there is anything to tell or not: a branch here cost 20 cycles a step)
-                    it0 = it1; it1 = it2;
-                    it2 = ld_table(at + 16u * (u + 3));
+            if (!LISTS || !few) {
+                int was_a[KS], was_b[KS], key[TRIP], not_usual = 0;
+                bool whole;
+                // (one loop with nothing but the trip: with the ways back from the unusual arrivals to its head a step took 104 cycles instead of 77)
+                #pragma unroll 1
+                do {
+                    not_usual = 0;
+                    const unsigned int at = LISTS ? at_ready + 16u * (e - first) : at_items + 16u * (e % RS_ITEMS);
                     #pragma unroll
                     for (int k = 0; k < KS; ++k)
-                        if (v[k] == (TAKE_OFF ? best & ~1 : best)) { ra[k] += kpd; rb[k] += kpb; }
-                    key[u] = best;
-                    not_usual |= best & 1;
-                    if (!Scores<KIND>::EXACT) {     // another row that can be the best
-                        int next = 0x7fffffff;
+                        if (!TAKE_OFF) { was_a[k] = ra[k]; was_b[k] = rb[k]; }
+                    #pragma unroll
+                    for (int u = 0; u < TRIP; ++u) {     // (items from `limit` on are whatever the slots hold: what is done with them is taken back)
+                        const int kp = it0.x, kpd = it0.y, kpb = LISTS ? it0.w : it0.x + it0.y;
+                        int v[KS];
                         #pragma unroll
-                        for (int k = 0; k < KS; ++k) next = min(next, v[k] == best ? 0x7fffffff : v[k]);
-                        next = __reduce_min_sync(FULL_MASK, next);
-                        if (next <= (best | K::TAGS) + SLACK) not_usual |= 2 << u;
+                        for (int k = 0; k < KS; ++k) v[k] = __viaddmax_s32(rb[k], kp, ra[k]);
+                        int least = LISTS ? it0.z : it0.z > jmax ? cut : (int)0x80000001u;
+                        #pragma unroll
+                        for (int k = 0; k + 1 < KS; k += 2) least = __vimin3_s32(least, v[k], v[k + 1]);
+                        const int best = __reduce_min_sync(FULL_MASK, least);
+                        // (while the reduction is under way)
+                        if (u == 0) { tell(e - TRIP, told, untold); publish(e); }     // (whether there is anything to tell or not: a branch here cost 20 cycles a step)
+                        it0 = it1; it1 = it2;
+                        it2 = ld_table(at + 16u * (u + 3));
+                        #pragma unroll
+                        for (int k = 0; k < KS; ++k)
+                            if (v[k] == (TAKE_OFF ? best & ~1 : best)) { ra[k] += kpd; rb[k] += kpb; }
+                        key[u] = best;
+                        not_usual |= best & 1;
+                        if (!Scores<KIND>::EXACT) {     // another row that can be the best
+                            int next = 0x7fffffff;
+                            #pragma unroll
+                            for (int k = 0; k < KS; ++k) next = min(next, v[k] == best ? 0x7fffffff : v[k]);
+                            next = __reduce_min_sync(FULL_MASK, next);
+                            if (next <= (best | K::TAGS) + SLACK) not_usual |= 2 << u;
+                        }
                     }
-                }
-                told = key[0];
-                #pragma unroll
-                for (int u = 1; u < TRIP; ++u) told = lane == u ? key[u] : told;
-                whole = not_usual == 0 && e + TRIP <= limit;
-                untold = whole ? TRIP : 0;
-                e += untold;
-            } while (whole && e < stop);
-            if (whole) break;
-            const unsigned int at = LISTS ? at_ready + 16u * (e - first) : at_items + 16u * (e % RS_ITEMS);
-            // ---- the first `usual` steps of the trip stand, the others are taken back
-            const int there = (int)min(limit - e, (unsigned int)TRIP);
-            int usual = there;
-            #pragma unroll
-            for (int u = TRIP - 1; u >= 0; --u)
-                if (u < there && ((key[u] & 1) || (not_usual & (2 << u)))) usual = u;
-            if (TAKE_OFF) {
-                #pragma unroll
-                for (int u = 0; u < TRIP; ++u) {
-                    const int4 it = ld_table(at + 16u * u);
-                    const int t = u >= usual && (key[u] & 1) == 0 ? key[u] & K::SLOT : -1;
+                    told = key[0];
                     #pragma unroll
-                    for (int k = 0; k < KS; ++k) {
-                        ra[k] -= tag(k) == t ? it.y : 0;
-                        rb[k] -= tag(k) == t ? it.w : 0;
-                    }
-                }
-            } else {
+                    for (int u = 1; u < TRIP; ++u) told = lane == u ? key[u] : told;
+                    whole = not_usual == 0 && e + TRIP <= limit;
+                    untold = whole ? TRIP : 0;
+                    e += untold;
+                } while (whole && e < stop);
+                if (whole) break;
+                const unsigned int at = LISTS ? at_ready + 16u * (e - first) : at_items + 16u * (e % RS_ITEMS);
+                // ---- the first `usual` steps of the trip stand, the others are taken back
+                const int there = (int)min(limit - e, (unsigned int)TRIP);
+                int usual = there;
                 #pragma unroll
-                for (int k = 0; k < KS; ++k) { ra[k] = was_a[k]; rb[k] = was_b[k]; }
-                #pragma unroll
-                for (int u = 0; u + 1 < TRIP; ++u) {
-                    const int4 it = ld_table(at + 16u * u);
-                    const int t = u < usual ? key[u] & K::SLOT : -1;
+                for (int u = TRIP - 1; u >= 0; --u)
+                    if (u < there && ((key[u] & 1) || (not_usual & (2 << u)))) usual = u;
+                if (TAKE_OFF) {
                     #pragma unroll
-                    for (int k = 0; k < KS; ++k) {
-                        ra[k] += tag(k) == t ? it.y : 0;
-                        rb[k] += tag(k) == t ? (LISTS ? it.w : it.x + it.y) : 0;
+                    for (int u = 0; u < TRIP; ++u) {
+                        const int4 it = ld_table(at + 16u * u);
+                        const int t = u >= usual && (key[u] & 1) == 0 ? key[u] & K::SLOT : -1;
+                        #pragma unroll
+                        for (int k = 0; k < KS; ++k) {
+                            ra[k] -= tag(k) == t ? it.y : 0;
+                            rb[k] -= tag(k) == t ? it.w : 0;
+                        }
+                    }
+                } else {
+                    #pragma unroll
+                    for (int k = 0; k < KS; ++k) { ra[k] = was_a[k]; rb[k] = was_b[k]; }
+                    #pragma unroll
+                    for (int u = 0; u + 1 < TRIP; ++u) {
+                        const int4 it = ld_table(at + 16u * u);
+                        const int t = u < usual ? key[u] & K::SLOT : -1;
+                        #pragma unroll
+                        for (int k = 0; k < KS; ++k) {
+                            ra[k] += tag(k) == t ? it.y : 0;
+                            rb[k] += tag(k) == t ? (LISTS ? it.w : it.x + it.y) : 0;
+                        }
                     }
                 }
-            }
-            tell(e, told, usual);
-            e += usual;
-            publish(e);
-            if (usual < there) {
+                tell(e, told, usual);
+                e += usual;
+                publish(e);
+                if (usual == there) { fetch(e, stop); continue; }
                 // The two usual reasons, each without the look at everything: the winner was marked when it was last read, and a row outside the list could do
                 // as well.  (An arrival of 64 x 256 that is not usual: 670 cycles by `unusual` alone.)
                 int won = key[0];
@@ -2129,13 +2126,15 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 }
                 if (lost) break;
                 if (again) { fetch(e, stop); continue; }
-                do {      // (no trip for the next arrival either while it does not reach every row's top)
-                    if (unusual(e)) { ++e; publish(e); }
-                    else if (lost) break;
-                } while (e < stop && __any_sync(FULL_MASK, sh.items[e % RS_ITEMS].z <= jmax));
             }
+            // (The one call of `unusual`: with a second one the compiler left it a function of its own in eight of the twelve list kernels, with all that the
+            // deciding loop holds on the stack: maps, a step and 8,192 arrivals on 2,000 x 1,536 in blocks of 16 tokens 2,420 us, 893 so.)
+            do {      // (no trip for the next arrival either while it does not reach every row's top)
+                if (unusual(e)) { ++e; publish(e); }
+                else if (lost) break;
+            } while (e < stop && ((LISTS && few) || __any_sync(FULL_MASK, sh.items[e % RS_ITEMS].z <= jmax)));
             if (lost) break;
-            fetch(e, stop);
+            if (!LISTS || !few) fetch(e, stop);
         }
         tell(e - TRIP, told, untold);
         publish(e);
