@@ -424,10 +424,11 @@ struct RsShared {
     unsigned int pending[RS_LIST_ROWS];     // by slot of the row held: 1 from the decision for it to the end of its fold; cleared last
     uint2 scored[RS_ITEMS];                 // {token count, peak} of their scores, from the folding warps
     // from the list block, for the present list and the next one
-    int4 table[2][32];                      // by code of the prompt: {bounds of the rows outside the list}
-    int list_row[2][RS_LIST_ROWS];
-    int list_n[2], list_base[2];
+    int4 table[2][32];                      // by code of the prompt: {bounds of the rows outside the list}, each with the list's number
+    unsigned int list_row[2][RS_LIST_ROWS]; // by slot: {list's number, row}
+    unsigned int list_base[2][2];           // {list's number, half of the base}
     unsigned int lists_ready;
+    unsigned int list_free;                 // the list whose half nobody reads any more, from the deciding warp (in the list block: as passed on)
     unsigned int least;                     // smallest score of an empty prompt, to begin with
     // (the list block's own)
     unsigned int lists_wanted, lists_go;    // the list that is asked for; RS_GO_USUAL, RS_GO_APART, RS_GO_LEAVE
@@ -488,6 +489,7 @@ __device__ __forceinline__ int2 ld_volatile2(const int2* p) {
     asm volatile("ld.volatile.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(smem_u32(p)) : "memory");
     return v;
 }
+__device__ __forceinline__ void st_volatile2(int2* p, int2 v) { asm volatile("st.volatile.shared.v2.u32 [%0], {%1, %2};" ::"r"(smem_u32(p)), "r"(v.x), "r"(v.y) : "memory"); }
 __device__ __forceinline__ uint4 ld_volatile4(const uint4* p) {
     uint4 v;
     asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem_u32(p)) : "memory");
@@ -525,7 +527,7 @@ __device__ __forceinline__ void st_cluster4(unsigned int at, int4 v) {
     asm volatile("st.relaxed.cluster.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 __device__ __forceinline__ void st_release_cluster(unsigned int at, unsigned int v) {
-    asm volatile("fence.acq_rel.cluster; st.release.cluster.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+    asm volatile("st.release.cluster.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
 }
 __device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
@@ -533,14 +535,30 @@ __device__ __forceinline__ void acquire_cta() { asm volatile("fence.acq_rel.cta;
 
 // Polls of a warp that nothing is owed to.
 __device__ __forceinline__ unsigned int rs_idle_limit(unsigned int spin_limit) { return max(spin_limit < (1u << 27) ? 16u * spin_limit : 0xffffffffu, 1u << 22); }
-// The newest list that is there.  No acquire: what is read behind it lies in this block's shared memory and was there before the list block's release, and loads
-// of shared memory are made in order.  An acquire of the cluster empties the SM's L1 of the rows' cells (one per poll: a fold's load took 350 cycles instead of
-// 110 to 230).
-__device__ __forceinline__ unsigned int list_number(const RsShared& sh) {
+// The hand-over of a list from the list block to the routing block, by relaxed operations of the cluster on words that say themselves which list they belong
+// to: a row's word has the list's number above the row, an entry of the table has it in the bits that the entries all have alike, the base is in two words
+// like a row's.  Whoever reads a word that has the number read the list's value; no order between words is relied on.  A folding warp reads a row's word behind the
+// deciding warp (which told it the slot by a release), hence the same value or a later one; and there is none as long as the decision is not folded: a half
+// is written anew when the deciding warp has taken the next list, with every decision of the old one folded.  That is told by a release of its own, which the
+// list block acquires before it writes, not before it begins to build; a warp without other work passes it on to the cluster.
+// (An acquire of the cluster instead, one per list, empties the SM's L1 of the rows' cells, and the folds behind it miss: 512 x 1,024, Zipf, 8,192 arrivals 900 ->
+// 1,015 us a pass, 4,096 x 2,048 7,817 -> 8,986.  A release of the
+// cluster by the deciding warp takes it 0.7 us: 900 -> 935 and 7,817 -> 8,090.)
+__device__ __forceinline__ unsigned int ld_relaxed_cluster(const void* p) {
     unsigned int v;
-    asm volatile("ld.relaxed.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(&sh.lists_ready)) : "memory");
+    asm volatile("ld.relaxed.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
     return v;
 }
+__device__ __forceinline__ int4 ld_relaxed_cluster4(unsigned int at) {
+    int4 v;
+    asm volatile("ld.relaxed.cluster.shared::cta.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+    return v;
+}
+constexpr unsigned int RS_LIST_NOBODY = 0xffffu;      // (a slot without a row)
+__device__ __forceinline__ unsigned int list_word(unsigned int list, unsigned int v) { return list << 16 | v; }
+__device__ __forceinline__ bool of_list(unsigned int word, unsigned int list) { return word >> 16 == (list & 0xffffu); }
+// The newest list that is there, as far as it is known: a hint of when to look at the words.
+__device__ __forceinline__ unsigned int list_number(const RsShared& sh) { return ld_relaxed_cluster(&sh.lists_ready); }
 // A wait of a whole warp on words that other warps of this block write.  False: abandoned, here or elsewhere.
 // What counts against the limit is time in which nothing moves.  IDLE: nothing is owed to this warp, it waits for work; that
 // there is none as long as the deciding warp gets on without is no reason to give up.
@@ -595,6 +613,9 @@ template <int KS> struct Held {
     static constexpr int LIMIT = 1 << (30 - SLOT_BITS), CUT = LIMIT / 2, ITEM = LIMIT / 4;
     static __device__ __forceinline__ int scaled(int key) { return key * (1 << SLOT_BITS); }
     static __device__ __forceinline__ int relative(int key, int base) { return scaled(min(max(key - base, -LIMIT), LIMIT)); }
+    // An entry of the bounds' table: its lowest bits (TAGS), all set, have the list's number instead.
+    static __device__ __forceinline__ int numbered(int entry, unsigned int list) { return (entry & ~TAGS) | (int)(list & (unsigned int)TAGS); }
+    static __device__ __forceinline__ bool of_list(int4 e, unsigned int list) { return (((e.x ^ (int)list) | (e.y ^ (int)list) | (e.z ^ (int)list) | (e.w ^ (int)list)) & TAGS) == 0; }
 };
 //   RS_HALVES (beta = m / 2^k, m at most 3, k at most 2, and m * theta with a fraction that is neither nearly none nor nearly one): keys in
 //   units of 2^-(k+1) tokens, which decide as the binary64 scores do.  2^k times the score of a row that pays is n + f, of one that does
@@ -724,7 +745,7 @@ __device__ __forceinline__ unsigned int job_slot(unsigned int job) { return (job
 template <bool LISTS>
 __device__ __forceinline__ int job_row(const RsShared& sh, unsigned int job) {
     if (!(job & RS_BY_SLOT)) return (int)(job & ~RS_GIVEN);
-    return LISTS ? sh.list_row[(job >> 16) & 1][job_slot(job)] : (int)job_slot(job);
+    return LISTS ? (int)(ld_relaxed_cluster(&sh.list_row[(job >> 16) & 1][job_slot(job)]) & 0xffffu) : (int)job_slot(job);
 }
 struct Cells { uint2* near; unsigned int* far; };      // [I][32] each
 template <bool ADMIT, int KIND, bool LISTS>
@@ -836,7 +857,7 @@ struct Folder {
             const unsigned int now = tokens + (unsigned int)P + (unsigned int)D;
             rows.top[w] = n.top;
             if (!Scores<KIND>::WHOLE) rows.tok[w] = now;
-            rows.rec[w] = make_int2(sc.key_a(now), sc.key_b(now, key_top));
+            st_volatile2(rows.rec + w, make_int2(sc.key_a(now), sc.key_b(now, key_top)));      // (the list block reads it whenever it does)
             rows.state[w] = n.jtop | (drop_of(key_top, n.near0) << RS_DROP) | (is_far ? RS_FAR : 0u) | (full ? RS_FULL : 0u) | (deferred ? RS_DEFERRED : 0u) | (not_over ? RS_NOT_OVER : 0u);
             if (ADMIT && (state & RS_NOT_OVER) && !not_over) atomicSub(&sh.not_over, 1u);
             sh.scored[e % RS_ITEMS] = make_uint2(tokens, (job.x & RS_GIVEN) ? job.y : old_top + (unsigned int)P);
@@ -1111,10 +1132,13 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
             const unsigned int newest = __reduce_max_sync(FULL_MASK, list_number(sh));
             if (newest != list) {
                 list = newest;
-                const int n = sh.list_n[list & 1];      // (may be none)
+                // (This warp has no claim on the list, whose words may be on their way or written anew: any row that there is will do.)
                 unsigned int sum = 0;
                 #pragma unroll 2
-                for (int x = lane; x < n; x += 32) sum ^= touch_row(a.near, a.far, sh.list_row[list & 1][x]);
+                for (int x = lane; x < 32 * KS; x += 32) {
+                    const unsigned int w = ld_relaxed_cluster(&sh.list_row[list & 1][x]) & 0xffffu;
+                    if (w < (unsigned int)a.I) sum ^= touch_row(a.near, a.far, (int)w);
+                }
                 sh.touched[lane] = sum;
             }
         }
@@ -1192,6 +1216,26 @@ __device__ __forceinline__ void rs_io_loop(const RouteSumArgs& a, RsShared& sh, 
     if (lane == 0) { sh.first_bad = first_bad; sh.first_full = first_full; sh.cursor = min(cursor, items); }
 }
 
+// The warp of the routing block that passes on to the list block which half of the lists nobody reads any more (see list_number).
+__device__ __forceinline__ void rs_pass_on(RsShared& sh) {
+    const int lane = threadIdx.x & 31;
+    for (unsigned int passed = 0;;) {
+        unsigned int free = 0;
+        bool end = false;
+        if (!rs_wait<true>(sh, [&] {
+                end = ld_volatile(&sh.ctl.z) != 0;
+                free = ld_volatile(&sh.list_free);
+                return free != passed || end;
+            }, 200))      // (a list takes some 2 us to build: seldom polls leave the scheduler to the folds beside this warp)
+            return;
+        if (__any_sync(FULL_MASK, end)) return;
+        acquire_cta();
+        passed = __reduce_max_sync(FULL_MASK, free);      // (the lanes need not have loaded it at the same time)
+        __syncwarp();
+        if (lane == 0) st_release_cluster(other_smem(&sh.list_free, 1), passed);
+    }
+}
+
 // ---- list block.  A list holds the rows whose key value for one of RS_PROBES prompt lengths lies within a margin of the
 // smallest one, as many as there is room for.  The other rows are bounded by 32 buckets: bucket x
 // holds the smallest a and the smallest b of the rows whose row_code is x.  For an arrival of code q the rows
@@ -1241,22 +1285,23 @@ __device__ __forceinline__ void rs_build_lists(const RouteSumArgs& a, RsShared& 
     #pragma unroll
     for (int x = 0; x < RS_PROBES; ++x) bp[x] = sc.key_p(rs_probe(mean, x));
     int width = min(max(max(sc.key_a((unsigned int)mean) / 16, 8) / (RS_LIST_BINS / 2), 1), 1 << 20);      // of a bin (256 of them leave room for keys)
+    // (By one warp, the others wait for it.  As in rs_wait what counts is time in which the deciding warp does not get on.)  False: no list is wanted any more.
+    auto told = [&](const unsigned int* word, unsigned int n) {
+        unsigned int seen = 0, polls = 0;
+        while (__any_sync(FULL_MASK, (int)(ld_acquire_cluster(word) - n) < 0)) {
+            if (__any_sync(FULL_MASK, ld_acquire_cluster(&sh.lists_go) == RS_GO_LEAVE)) return false;
+            if ((++polls & 255u) == 0) {
+                const unsigned int now = __reduce_max_sync(FULL_MASK, ld_cluster(at_ctl) + ld_cluster(at_beat));
+                if (now != seen) { seen = now; polls = 0; }
+            }
+            if (polls >= sh.idle_limit) { if (lane == 0) st_cluster(at_ctl + 12u, 1u); return false; }
+            __nanosleep(20);
+        }
+        return true;
+    };
     // (a warp has neighbouring rows: the list is put together in their order)
     for (unsigned int n = 1;; ++n) {
-        bool leave = false;
-        if (me == 0) {      // (one warp looks for work, the others wait for it; as in rs_wait what counts is time in which the deciding warp does not get on)
-            unsigned int seen = 0, polls = 0;
-            while (__any_sync(FULL_MASK, (int)(ld_acquire_cluster(&sh.lists_wanted) - n) < 0)) {
-                if (__any_sync(FULL_MASK, ld_acquire_cluster(&sh.lists_go) == RS_GO_LEAVE)) { leave = true; break; }
-                if ((++polls & 255u) == 0) {
-                    const unsigned int now = __reduce_max_sync(FULL_MASK, ld_cluster(at_ctl) + ld_cluster(at_beat));
-                    if (now != seen) { seen = now; polls = 0; }
-                }
-                if (polls >= sh.idle_limit) { if (lane == 0) st_cluster(at_ctl + 12u, 1u); leave = true; break; }
-                __nanosleep(20);
-            }
-        }
-        if (__syncthreads_or(leave)) return;
+        if (__syncthreads_or(me == 0 && !told(&sh.lists_wanted, n))) return;
         const int now = n & 1, of = NEAR && !all_rows ? n_near : I;
         const int share = ((of + 32 * RS_LIST_WARPS - 1) / (32 * RS_LIST_WARPS)) * 32, first = me * share, end = min(of, first + share);
         auto row_of = [&](int x) { return NEAR && !all_rows ? (int)near[x] : x; };
@@ -1366,10 +1411,11 @@ __device__ __forceinline__ void rs_build_lists(const RouteSumArgs& a, RsShared& 
         }
         const int hb = __reduce_min_sync(FULL_MASK, hot_b), ca = __reduce_min_sync(FULL_MASK, cold_a);
         if (lane == 0) { atomicMin(&sh.bucket_b[0], ordered(hb)); atomicMin(&sh.bucket_a[31], ordered(ca)); sh.list_take[me] = n_take; sh.list_found[me] = n_found; }
-        __syncthreads();
+        if (__syncthreads_or(me == 0 && !told(&sh.list_free, n))) return;      // (by now it has been told for long)
         const int taken = lane < RS_LIST_WARPS ? sh.list_take[lane] : 0, before = __reduce_add_sync(FULL_MASK, lane < me ? taken : 0);
         const unsigned int at_list = other_smem(sh.list_row[now], 0);
-        for (int x = lane; x < n_take; x += 32) st_cluster(at_list + 4u * (unsigned int)(before + x), sh.list_seg[me][x]);
+        for (int x = lane; x < n_take; x += 32) st_cluster(at_list + 4u * (unsigned int)(before + x), list_word(n, sh.list_seg[me][x]));
+        for (int x = __reduce_add_sync(FULL_MASK, taken) + t; x < ROOM; x += 32 * RS_LIST_WARPS) st_cluster(at_list + 4u * (unsigned int)x, list_word(n, RS_LIST_NOBODY));
         if (me == 0) {
             // (a key that no row has set is out of reach; rows of code 31 count by their a alone, no b is kept for them)
             const int ka = unordered(min(min(sh.bucket_a[lane], NEAR ? sh.far_a[lane] : 0xffffffffu), ordered(RS_ABSENT)));
@@ -1388,13 +1434,13 @@ __device__ __forceinline__ void rs_build_lists(const RouteSumArgs& a, RsShared& 
             const int row_b = lane == 31 ? RS_LOWEST : kb;
             // The entries as keys that the deciding warp holds: a row that wins by less than the rounding of its key does not beat them.
             // (The base is a lower bound of every row's score, so an entry that is cut below is one, too.)
-            const int base = smallest[0] & ~1, count = __reduce_add_sync(FULL_MASK, taken);
-            auto entry = [&](int key) { return Held<KS>::relative(key, base) - 1 - Held<KS>::scaled(Scores<KIND>::SLACK); };
+            const int base = smallest[0] & ~1;
+            auto entry = [&](int key) { return Held<KS>::numbered(Held<KS>::relative(key, base) - 1 - Held<KS>::scaled(Scores<KIND>::SLACK), n); };
             st_cluster4(other_smem(&sh.table[now][lane], 0), make_int4(entry(above_a), entry(below_b), entry(ka), entry(row_b)));
-            if (lane == 0) { st_cluster(other_smem(&sh.list_n[now], 0), (unsigned int)count); st_cluster(other_smem(&sh.list_base[now], 0), (unsigned int)base); }
+            if (lane < 2) st_cluster(other_smem(&sh.list_base[now][lane], 0), list_word(n, ((unsigned int)base >> (16 * lane)) & 0xffffu));
         }
         __syncthreads();
-        if (t == 0) st_release_cluster(other_smem(&sh.lists_ready, 0), n);
+        if (t == 0) st_cluster(other_smem(&sh.lists_ready, 0), n);
         const int margin = bins * width;
         if (NEAR && all_rows) {
             const int mine = lane < RS_LIST_WARPS ? sh.list_found[lane] : 0, at = __reduce_add_sync(FULL_MASK, lane < me ? mine : 0);
@@ -1512,7 +1558,11 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     unsigned int table = smem_u32(sh.table[0]);
     bool asked = false;
     auto ask_for_list = [&]() {
-        if (!asked && lane == 0) st_cluster(other_smem(&sh.lists_wanted, 1), list + 1);
+        __syncwarp();
+        if (!asked && lane == 0) {
+            st_cluster(other_smem(&sh.lists_wanted, 1), list + 1);
+            st_release(&sh.list_free, list + 1);      // (see list_number)
+        }
         asked = true;
     };
     auto next_list = [&](unsigned int e) {
@@ -1521,11 +1571,20 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         ++list;
         asked = false;
         table = smem_u32(sh.table[list & 1]);
-        const int n = sh.list_n[list & 1];
+        unsigned int word[KS], half[2];
+        if (!rs_wait(sh, [&] {
+                bool there = K::of_list(ld_relaxed_cluster4(table + 16u * lane), list);
+                #pragma unroll
+                for (int k = 0; k < KS; ++k) { word[k] = ld_relaxed_cluster(&sh.list_row[list & 1][k * 32 + lane]); there &= of_list(word[k], list); }
+                #pragma unroll
+                for (int x = 0; x < 2; ++x) { half[x] = ld_relaxed_cluster(&sh.list_base[list & 1][x]); there &= of_list(half[x], list); }
+                return there;
+            })) { lost = true; return; }
+        __syncwarp();      // (any lane reads the table's entries from here on)
         #pragma unroll
-        for (int k = 0; k < KS; ++k) list_row[LISTS ? k : 0] = k * 32 + lane < n ? sh.list_row[list & 1][k * 32 + lane] : NO_ROW;
+        for (int k = 0; k < KS; ++k) list_row[LISTS ? k : 0] = (word[k] & 0xffffu) != RS_LIST_NOBODY ? (int)(word[k] & 0xffffu) : NO_ROW;
         by_slot = RS_BY_SLOT | ((list & 1) << 16);
-        take_base(sh.list_base[list & 1]);
+        take_base((int)((half[1] << 16) | (half[0] & 0xffffu)));
         unread();
         if (!rs_wait(sh, [&] { return all_folded(e); })) { lost = true; return; }
         refresh();
@@ -1555,7 +1614,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         refresh();
     }
     // An entry of the bounds' table, for an arrival that adds kp: no row outside the list has a smaller key.
-    auto bound_of = [&](int4 b, int kp) { return min(__viaddmin_s32(b.y, kp, b.x), __viaddmax_s32(b.w, kp, b.z)); };
+    auto bound_of = [&](int4 b, int kp) { return min(__viaddmin_s32(b.y, kp, b.x), __viaddmax_s32(b.w, kp, b.z)) | K::TAGS; };
     // Decisions told to the folding warps: those of `count` items from e on, lane u's row by the key that has won.
     auto tell = [&](unsigned int e, int key, int count) {
         asm volatile("{ .reg .pred p; setp.lt.s32 p, %0, %1; @p st.shared.u32 [%2], %3; @p st.shared.u32 [%4], 1; }"
@@ -1651,7 +1710,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                         marked |= (ra[k] & 1) ? 1u << k : 0u;
                         least = (ra[k] & 1) ? least : min(least, max(ra[k], rb[k] + kpe));
                     }
-                    auto row_at = [&](int slot) { return LISTS ? sh.list_row[list & 1][slot] : slot; };
+                    auto row_at = [&](int slot) { return LISTS ? min((int)(ld_relaxed_cluster(&sh.list_row[list & 1][slot]) & 0xffffu), I - 1) : slot; };
                     auto tokens_at = [&](int i) { return Scores<KIND>::WHOLE ? (unsigned int)ld_volatile2(rows.rec + i).x >> 1 : ld_volatile(rows.tok + i); };
                     if (LISTS && bounded) {
                         #pragma unroll 1
@@ -2329,6 +2388,7 @@ __device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, co
         if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, KIND, LISTS, Sp::SELF>(a, sh, rows, sc, cells, role);
         else if (role == Sp::FOLD)
             rs_io_loop<KS, LISTS, Sp::DONE, ADMIT, KIND>(a, sh, sc, b.q_head, (int)b.q_len, (int)b.n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
+        else if (LISTS) rs_pass_on(sh);
     }
     __syncthreads();
     if (sh.ctl.w) {     // (all threads alike: nobody writes it any more)
@@ -2377,7 +2437,7 @@ template <int KS, int KIND, int OTHER_KS, int OTHER>
 __device__ __forceinline__ void rs_list_block(const RouteSumArgs& a, RsShared& sh, const Rows& rows) {
     const int tid = threadIdx.x;
     if (tid == 0) {
-        sh.lists_wanted = sh.lists_go = 0;
+        sh.lists_wanted = sh.lists_go = sh.list_free = 0;
         sh.idle_limit = rs_idle_limit(a.spin_limit);
     }
     __syncthreads();
@@ -2453,8 +2513,8 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
         sh.n0 = *a.n_requests;
         sh.ctl = make_uint4(0u, 0u, 0u, 0u);
         sh.items_ready = sh.items_end = sh.not_over = sh.jmax = sh.n_far = sh.n_least = sh.n_beyond = sh.written = sh.flush = 0;
-        sh.lists_ready = sh.look_met = 0;
-        sh.list_n[0] = sh.list_n[1] = 0;
+        sh.lists_ready = sh.list_free = sh.look_met = 0;
+        sh.list_base[0][0] = sh.list_base[0][1] = sh.list_base[1][0] = sh.list_base[1][1] = 0;
         sh.least = 0xffffffffu;
         sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0;
         sh.first_bad = sh.first_full = 0x7fffffff;
@@ -2463,6 +2523,10 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
     if (tid < RS_MAX_FOLD_WARPS) { sh.done[tid] = (unsigned int)tid; sh.looks_done[tid] = 0; }
     if (!alone)
         for (int i = tid; i < RS_LIST_ROWS; i += THREADS) sh.pending[i] = 0;
+    if (LISTS) {      // (of no list yet: they are numbered from 1)
+        for (int i = tid; i < RS_LIST_ROWS; i += THREADS) sh.list_row[0][i] = sh.list_row[1][i] = 0;
+        if (tid < 32) sh.table[0][tid] = sh.table[1][tid] = make_int4(0, 0, 0, 0);
+    }
     // ADMIT: the requests that were waiting when the call was made come first, then the arrivals
     long long q_head = 0, q_len = 0;
     if (ADMIT && a.queue_capacity > 0) {

@@ -1,4 +1,4 @@
-"""What ptxas says of the kernels that the build made (no GPU needed)."""
+"""What can be seen without a GPU of how the kernels were written and built: ptxas' report, and the order of a hand-over in the source."""
 import os
 import re
 
@@ -30,3 +30,32 @@ def test_the_deciding_loop_keeps_nothing_on_the_stack(source):
     assert len(kernels) == (5 if "halves" in source else 6)      # (one per number of rows held; exact fractions begin beyond the smallest)
     assert all(v == (0, 0) for v in kernels.values()), kernels
     assert not [k for k in found if "rs_decide_loop" in k], "a part of the deciding loop is a function of its own"
+
+
+def body(text, opening):
+    """From `opening` to the brace that closes it."""
+    at = text.index(opening)
+    depth, end = 0, at
+    for end in range(text.index("{", at), len(text)):
+        depth += {"{": 1, "}": -1}.get(text[end], 0)
+        if depth == 0:
+            break
+    return text[at:end + 1]
+
+
+def test_the_words_of_a_list_are_read_with_its_number():
+    """The list block writes them from another SM, and nothing orders them behind the word that says a list is there.  No run shows a word that is read too
+    early (shared memory is read in order where it is compiled so), so the source is looked at: the list's words are read by relaxed loads alone, the
+    deciding warp takes none before each has the list's number, and the io warp, which does not look for it, no row that there is not."""
+    text = open(os.path.join(build.CSRC, "route_summary.cuh")).read()
+    code = "\n".join(line.split("//")[0] for line in text.splitlines())
+    for word in ("list_row[", "list_base["):
+        reads = [line for line in code.splitlines() if "sh." + word in line and "other_smem" not in line and not re.search(r"\] = 0;", line)]
+        assert reads and all("ld_relaxed_cluster(&sh." + word in line for line in reads), reads
+    take = body(code, "auto next_list = [&](unsigned int e) {")
+    assert take.index("there = K::of_list(") < take.index("there &= of_list(word[k]") < take.index("there &= of_list(half[x]") < take.index("RS_LIST_NOBODY")
+    asks, builds = body(code, "auto ask_for_list = [&]() {"), body(code, "void rs_build_lists(")
+    assert "st_release(&sh.list_free" in asks and "st_release_cluster(other_smem(&sh.list_free" in body(code, "void rs_pass_on(")
+    assert builds.index("told(&sh.lists_wanted") < builds.index("told(&sh.list_free") < builds.index("st_cluster(at_list")
+    touch = body(code, "void rs_io_loop(")
+    assert touch.index("if (w < (unsigned int)a.I)") < touch.index("touch_row(a.near")
