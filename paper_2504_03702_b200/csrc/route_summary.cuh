@@ -468,6 +468,7 @@ struct RsShared {
     int warp_ok[32];                        // (the tail of ADMIT)
     long long joined;
     int any_bad;
+    int lost;                               // a wait was abandoned before the warps met
 };
 
 __device__ __forceinline__ unsigned int smem_u32(const void* p) { return (unsigned int)__cvta_generic_to_shared(p); }
@@ -2390,8 +2391,10 @@ __device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, co
             rs_io_loop<KS, LISTS, Sp::DONE, ADMIT, KIND>(a, sh, sc, b.q_head, (int)b.q_len, (int)b.n_items, room < 0 ? 0 : (room > 0x7fffffffLL ? 0x7fffffff : (int)room));
         else if (LISTS) rs_pass_on(sh);
     }
-    __syncthreads();
-    if (sh.ctl.w) {     // (all threads alike: nobody writes it any more)
+    // (the list block may still give up and write the word: what counts is what the block saw here, all threads alike)
+    const bool lost = __syncthreads_or(ld_volatile(&sh.ctl.w) != 0) != 0;
+    if (tid == 0) sh.lost = lost;
+    if (lost) {
         decided = rs_settle<Sp::DONE, LISTS, ADMIT, KIND>(a, sh, rows, sc, (int)b.q_len);
         __syncthreads();
     }
@@ -2516,7 +2519,7 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
         sh.lists_ready = sh.list_free = sh.look_met = 0;
         sh.list_base[0][0] = sh.list_base[0][1] = sh.list_base[1][0] = sh.list_base[1][1] = 0;
         sh.least = 0xffffffffu;
-        sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0;
+        sh.blocked = 0; sh.blocked_k = 0; sh.joined = 0; sh.any_bad = 0; sh.lost = 0;
         sh.first_bad = sh.first_full = 0x7fffffff;
     }
     for (int i = tid; i < RS_ITEMS + RS_AHEAD; i += THREADS) sh.items[i] = make_int4(0, 0, 0, 0);    // (an item is fetched before it is known to be there)
@@ -2608,7 +2611,7 @@ __global__ void __launch_bounds__(Shape<KS, LISTS>::THREADS, 1) pre_route_summar
         a.ramps[1] = mode == 0 || a.own_ramps ? 0 : (long long)sh.ctl.x;
         // (what was noted beyond a blocked request is decided again below, what was noted beyond the last decision is dropped: neither
         // counts here)
-        int flags = sh.ctl.w ? PRE_ST_TIMEOUT : 0;
+        int flags = sh.lost ? PRE_ST_TIMEOUT : 0;
         if (sh.first_bad < decided) flags |= PRE_ST_BADREQ;
         if (sh.first_full < decided) flags |= PRE_ST_CAPACITY;
         if (flags) atomicOr(a.status, flags);

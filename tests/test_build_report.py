@@ -59,3 +59,13 @@ def test_the_words_of_a_list_are_read_with_its_number():
     assert builds.index("told(&sh.lists_wanted") < builds.index("told(&sh.list_free") < builds.index("st_cluster(at_list")
     touch = body(code, "void rs_io_loop(")
     assert touch.index("if (w < (unsigned int)a.I)") < touch.index("touch_row(a.near")
+
+
+def test_a_batch_is_given_up_by_the_whole_block():
+    """The list block, on another SM, may store the word that says a wait was abandoned until it is told to leave: the routing block's threads branch on one common
+    look at it (a barrier follows that branch), and the status of the batch is that look's."""
+    text = open(os.path.join(build.CSRC, "route_summary.cuh")).read()
+    code = "\n".join(line.split("//")[0] for line in text.splitlines())
+    route = body(code, "__device__ __forceinline__ bool rs_route(")
+    assert [line.strip() for line in route.splitlines() if "ctl.w" in line] == ["const bool lost = __syncthreads_or(ld_volatile(&sh.ctl.w) != 0) != 0;"]
+    assert "ctl.w" not in body(code, "pre_route_summaries(const __grid_constant__ RouteSumArgs a) {")
