@@ -1609,6 +1609,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
     };
     if (LISTS) {
         if (!few) next_list(0);
+        else unread();      // (no rows)
     } else {
         take_base(unordered(sh.least) & ~1);
         unread();
