@@ -1918,18 +1918,23 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
 
     // ---- the usual way
     int4 it0, it1, it2;              // items e, e + 1, e + 2 (LISTS: see RsShared::ready)
-    unsigned int first = 0;          // (LISTS) the first of the items made ready
+    // (LISTS) the items made ready: the first one, how many, up to which one they were there, and for which jmax and list
+    unsigned int first = 0, made = 0, made_there = 0, made_list = 0;
+    int made_jmax = 0;
     auto item_at = [&](unsigned int e, unsigned int x) { return ld_table(LISTS ? at_ready + 16u * (e - first + x) : at_items + 16u * (e % RS_ITEMS + x)); };
-    auto fetch = [&](unsigned int e, unsigned int stop) {
-        if (LISTS) {      // (as many as a chunk up to `stop` needs)
-            first = e;
+    auto fetch = [&](unsigned int e, unsigned int stop, unsigned int limit, unsigned int there) {
+        // (As many as the trips of a chunk up to `stop` need, of the items there are.  What was made ready holds until jmax or the list is another: made anew
+        // behind each interrupted trip it took 50 to 230 cycles an arrival where most trips are interrupted.)
+        if (LISTS && (made_list != list || made_jmax != jmax || stop - first + TRIP - 1 > made || (int)(min(stop + TRIP - 1, limit) - made_there) > 0)) {
+            first = e; made = 0; made_there = there; made_list = list; made_jmax = jmax;
             __syncwarp();
             #pragma unroll 1
-            for (unsigned int x = 0; x < READY && (x == 0 || stop - e > x - TRIP); x += 32) {
-                const int4 it = ld_table(at_items + 16u * ((e + x + lane) % RS_ITEMS));
+            do {
+                const int4 it = ld_table(at_items + 16u * ((e + made + lane) % RS_ITEMS));
                 const int b = it.z > jmax ? cut : (int)0x80000001u;
-                sh.ready[x + lane] = make_int4(it.x, it.y, min(b, bound_of(ld_table(table + it.w), it.x)), it.x + it.y);
-            }
+                sh.ready[made + lane] = make_int4(it.x, it.y, min(b, bound_of(ld_table(table + it.w), it.x)), it.x + it.y);
+                made += 32;
+            } while (made < READY && stop - e + TRIP - 1 > made);
             __syncwarp();
         }
         it0 = item_at(e, 0);
@@ -2078,7 +2083,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
         }
         const unsigned int stop = min(limit, e + CHUNK);
         refresh();
-        if (!LISTS || !few) fetch(e, stop);
+        if (!LISTS || !few) fetch(e, stop, limit, ready);
         int untold = 0;               // decisions before e that are not told yet (the last trip's: they are while the next reduction is under way)
         int told = 0;
         while (e < stop) {
@@ -2163,7 +2168,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 tell(e, told, usual);
                 e += usual;
                 publish(e);
-                if (usual == there) { fetch(e, stop); continue; }
+                if (usual == there) { fetch(e, stop, limit, ready); continue; }
                 // The two usual reasons, each without the look at everything: the winner was marked when it was last read, and a row outside the list could do
                 // as well.  (An arrival of 64 x 256 that is not usual: 670 cycles by `unusual` alone.)
                 int won = key[0];
@@ -2186,7 +2191,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                     again = true;
                 }
                 if (lost) break;
-                if (again) { fetch(e, stop); continue; }
+                if (again) { fetch(e, stop, limit, ready); continue; }
             }
             // (The one call of `unusual`: with a second one the compiler left it a function of its own in eight of the twelve list kernels, with all that the
             // deciding loop holds on the stack: maps, a step and 8,192 arrivals on 2,000 x 1,536 in blocks of 16 tokens 2,420 us, 893 so.)
@@ -2195,7 +2200,7 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 else if (lost) break;
             } while (e < stop && ((LISTS && few) || __any_sync(FULL_MASK, sh.items[e % RS_ITEMS].z <= jmax)));
             if (lost) break;
-            if (!LISTS || !few) fetch(e, stop);
+            if (!LISTS || !few) fetch(e, stop, limit, ready);
         }
         tell(e - TRIP, told, untold);
         publish(e);
