@@ -2180,11 +2180,12 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 if (won != beyond && (won & 1)) {
                     const unsigned int* word = sh.pending + ((won & K::SLOT) >> 1);
                     if (__any_sync(FULL_MASK, ld_acquire(word) != 0) && !rs_wait(sh, [&] { return ld_acquire(word) == 0; })) { lost = true; break; }
-                    refresh();
-                    bool marked = false;
+                    bool far = false;
                     #pragma unroll
-                    for (int k = 0; k < KS; ++k) marked |= tag(k) == (won & K::SLOT) && (ra[k] & 1) != 0;
-                    again = !__any_sync(FULL_MASK, marked);      // (else it is far)
+                    for (int k = 0; k < KS; ++k)
+                        if (tag(k) == (won & K::SLOT)) far = (ld_volatile(rows.state + row(k)) & RS_FAR) != 0;
+                    again = !__any_sync(FULL_MASK, far);
+                    if (again) refresh();
                 } else if (LISTS && won == beyond && won != (int)0x80000001u && won != cut && tried_at != e) {
                     tried_at = e; lists_tried = 1;
                     next_list(e);
