@@ -654,3 +654,33 @@ def test_many_lists_in_one_batch(n_inst, beta, t_mem, skew):
     ad = np.where(rng.random(n_arr) < 0.02, 1, rng.integers(1, 2 * h, n_arr)).astype(np.int32)
     wl.max_requests = n + n_arr
     route_and_compare(wl, ap, ad)
+
+
+def test_long_prompts_on_thousands_of_rows_find_their_rows_in_the_list():
+    """4,096 rows with a window of 100 steps and a deep backlog, prompts to four times the mean: arrivals with prompts beyond the longest one that lists had
+    rows for took two lists and a look at all rows each (0.18 of the scanning kernel's time; 0.07 where lists have rows for the longest prompt)."""
+    wl = W.make_config(3)
+    ap, ad = (dev(x) for x in wl.ticks[0])
+    n = len(wl.prompt) + len(ap)
+    st = DeviceState(wl.n_instances, 100, wl.capacity_tokens, n + 8192, wl.t_mem, wl.beta, device="cuda:0")
+    st.load_requests(wl.prompt, wl.generated, wl.predicted, wl.instance)
+    st.make_ring(wl.horizon)
+    st.ring_window()
+    choice, _ = st.route_batch(ap, ad)
+    st.ring_fold(ap, ad, choice)
+    queued = st.queued_p.clone()
+    best = {}
+    for path in (B.ROUTE_AUTO, B.ROUTE_SCAN) * 3:
+        st.select_router(path)
+        st.ring_window()
+        st.n_requests.fill_(n)
+        st.queued_p.copy_(queued)
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t0.record()
+        st.route_batch(ap[:8192], ad[:8192])
+        t1.record()
+        torch.cuda.synchronize()
+        best[path] = min(best.get(path, 1e9), t0.elapsed_time(t1))
+    assert st.status() == B.PRE_OK
+    st.close()
+    assert best[B.ROUTE_AUTO] < 0.11 * best[B.ROUTE_SCAN]
