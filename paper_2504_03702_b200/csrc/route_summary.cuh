@@ -2183,12 +2183,13 @@ __device__ __forceinline__ void rs_decide_loop(const RouteSumArgs& a, RsShared& 
                 if (won != beyond && (won & 1)) {
                     const unsigned int* word = sh.pending + ((won & K::SLOT) >> 1);
                     if (__any_sync(FULL_MASK, ld_acquire(word) != 0) && !rs_wait(sh, [&] { return ld_acquire(word) == 0; })) { lost = true; break; }
-                    bool far = false;
+                    bool far = false;      // (a far one stays marked: in a list many are, and are not read again for it)
+                    if (!LISTS) refresh();
                     #pragma unroll
                     for (int k = 0; k < KS; ++k)
-                        if (tag(k) == (won & K::SLOT)) far = (ld_volatile(rows.state + row(k)) & RS_FAR) != 0;
+                        if (tag(k) == (won & K::SLOT)) far = LISTS ? (ld_volatile(rows.state + row(k)) & RS_FAR) != 0 : (ra[k] & 1) != 0;
                     again = !__any_sync(FULL_MASK, far);
-                    if (again) refresh();
+                    if (LISTS && again) refresh();
                 } else if (LISTS && won == beyond && won != (int)0x80000001u && won != cut && tried_at != e) {
                     tried_at = e; lists_tried = 1;
                     next_list(e);
