@@ -64,18 +64,20 @@ constexpr int RS_READY = 64;                // items made ready for the deciding
 constexpr int RS_SELF_ROWS = 4;
 constexpr int RS_DIRECT_ROWS = 256;         // up to this many rows the deciding warp holds them all (8 per lane)
 constexpr int RS_LIST_ROWS = 256;           // rows of a list at most (4 per lane, 8 beyond RS_LONG_LISTS instances)
-// Lists of 256 / 128 rows, us a pass: 4,096 x 2,048 with 65,536 arrivals 7,716 / 10,926, 2,000 x 1,536 with 8,192 873 / 933.
+// Lists of 256 / 128 rows, us a pass: 4,096 x 2,048 with 65,536 arrivals 7,800 / 12,700, 2,000 x 1,536 with 8,192 855 / 1,106.
 constexpr int RS_LONG_LISTS = 1024;
-// Arrivals that no list is built for: each is decided on all rows.  us a cycle of four ticks, with lists / so: 1 arrival on 300 rows 157 / 141, on 4,096 245 / 190;
-// 4 arrivals 168 / 163 and 260 / 248, on 1,000 rows 188 / 191.
-constexpr int RS_FEW = 4;
 constexpr int RS_OWN_LOOK = 2048;           // rows up to which the deciding warp looks at their keys by itself
+// Arrivals that no list is built for: each is decided on all rows.  us a cycle of four ticks of 1 / 2 / 3 / 4 arrivals, with lists and so: 300 rows 164 / 167 / 164 /
+// 164 and 153 / 161 / 168 / 174, 1,000 rows 176 / 180 / 184 / 184 and 165 / 177 / 187 / 192, 2,000 rows 204 / 205 / 209 / 207 and 184 / 200 / 217 / 228, 4,096 rows (looked
+// at by all folding warps) 253 / 250 / 257 / 256 and 207 / 221 / 239 / 254.
+__device__ __forceinline__ int few_for(int I) { return I > RS_OWN_LOOK ? 4 : 2; }
 // Beyond RS_DIRECT_ROWS instances two kinds of batches cost this kernel more than the scanning one (which takes 2.4 us an arrival on 1,024 x
 // 1,024 whatever the rows): many far rows that may pay a penalty, whose arrivals need a look at all rows, scans, and folds of
-// whole rows (share of such rows, us: 16 % 1.7, 26 % 3.2, 39 % 3.9, 62 % 7.2; maps of 228 steps, 44 % 2.5, 68 % 5.1); and more rows that
-// share the smallest score than a list holds (empty services; 512 rows 2.7, 4,096 rows 42 against 3.1).
-// And keys in units of more than 64 tokens (beta of thousands): 1,024 x 1,024, beta 1,000.5 (units of 4 tokens) 1.2 us an arrival, 100,000.5
-// (of 512) 10.4, the scanning kernel 2.4.
+// whole rows (share of such rows, us with whole-number scores / fractional: 512 x 1,024 16 % 1.3 / 1.6, 35 % 2.8 / 3.1, 62 % 4.5 / 5.0; 1,024 x 1,024 18 % 0.95 / 1.2,
+// 45 % 2.7 / 3.1, 66 % 5.3 / 6.1; 2,048 x 512 24 % 1.1 / 1.2, 52 % 3.2 / 3.5); and more rows that share the smallest score than a list holds
+// (empty services; 512 rows 4.9 against 2.7, 4,096 rows 15 against 3.3).
+// And keys in units of more than 64 tokens (beta of thousands): 1,024 x 1,024, beta 1,000.5 (units of 4 tokens) 1.5 us an arrival, 100,000.5
+// (of 512) 9.3, the scanning kernel 2.4.
 constexpr int RS_COARSE_SHIFT = -6;
 // Exact keys have a unit of their own, rounded ones the batch's.  A batch is routed with rounded keys where one arrival in RS_LONG_SHARE does not fit the
 // exact ones (it is decided outside the loop, on all rows), or where one row in RS_BEYOND_SHARE will be far by its top alone when half of the batch is
@@ -1475,8 +1477,8 @@ template <int KS, bool LISTS> struct Shape {
 
 // ---- deciding warp.  KS: rows per lane.  LISTS: they are a list's, else all rows.
 // What bounds it: the latency of one chain of dependent instructions per arrival (a warp reduction, 23 cycles, and some eight integer
-// operations) and, with four and eight rows per lane, the number of its instructions (an integer instruction takes the warp two cycles): a step takes 52, 77 and
-// 113 cycles with two, four and eight rows per lane.  So nothing else is in the loop: no branch (whether all steps were usual is seen once per
+// operations) and, with four and eight rows per lane, the number of its instructions (an integer instruction takes the warp two cycles): a step takes 65, 84 and
+// 120 cycles with two, four and eight rows per lane (clock of the deciding warp around its trips, 64 x 256, 512 x 1,024 and 4,096 x 2,048).  So nothing else is in the loop: no branch (whether all steps were usual is seen once per
 // trip, which is taken back as far as they were not; a branch around the telling of a trip's decisions cost 20 cycles a step), items with their bounds
 // made ready by all lanes for up to 64 at once (per step: 7 cycles), fetched two steps ahead, and what need not be in the chain (scores, token counts, the
 // tables) is done by the folding warps.
@@ -2392,10 +2394,10 @@ __device__ __forceinline__ bool rs_route(const RouteSumArgs& a, RsShared& sh, co
         if ((H > RS_FAR_STEPS && sh.n_far > (unsigned int)(I / RS_FAR_SHARE)) || sh.n_least > 32u * KS || sc.shift < RS_COARSE_SHIFT) return false;
     }
 
-    if (LISTS && tid == 0 && b.n_items > RS_FEW) st_release_cluster(other_smem(&sh.lists_go, 1), go);      // (the rows' keys and sh.batch can be read)
+    if (LISTS && tid == 0 && b.n_items > few_for(I)) st_release_cluster(other_smem(&sh.lists_go, 1), go);      // (the rows' keys and sh.batch can be read)
     const int role = (warp >> 2) * 3 + (warp & 3) - 1;      // (of the warps that are not on the deciding warp's scheduler)
     if (warp == 0) {
-        rs_decide_loop<KS, LISTS, Sp::FOLD, ADMIT, KIND>(a, sh, rows, sc, cells, LISTS && b.n_items <= RS_FEW);
+        rs_decide_loop<KS, LISTS, Sp::FOLD, ADMIT, KIND>(a, sh, rows, sc, cells, LISTS && b.n_items <= few_for(I));
     } else if ((warp & 3) != 0) {
         if (role < Sp::FOLD) rs_fold_loop<Sp::FOLD, ADMIT, KIND, LISTS, Sp::SELF>(a, sh, rows, sc, cells, role);
         else if (role == Sp::FOLD)

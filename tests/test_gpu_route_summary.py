@@ -684,3 +684,15 @@ def test_long_prompts_on_thousands_of_rows_find_their_rows_in_the_list():
     assert st.status() == B.PRE_OK
     st.close()
     assert best[B.ROUTE_AUTO] < 0.11 * best[B.ROUTE_SCAN]
+
+
+# the line up to which no list is built: two arrivals, and four where all folding warps look at the rows
+@pytest.mark.parametrize("n_inst", [257, 2048, 2049])
+@pytest.mark.parametrize("n_arr", [2, 3, 4, 5])
+@pytest.mark.parametrize("beta", [1.0, 0.75])
+def test_arrivals_on_both_sides_of_the_line_for_lists(n_inst, n_arr, beta):
+    wl = W.make_random(73, n_inst, 70, 6 * n_inst, 0, max_prompt=300, max_output=90, beta=beta)
+    rng = np.random.default_rng(n_inst + n_arr)
+    ap, ad = rng.integers(0, 300, 2 * n_arr).astype(np.int32), rng.integers(1, 90, 2 * n_arr).astype(np.int32)
+    wl.max_requests = 6 * n_inst + 2 * n_arr
+    route_and_compare(wl, ap, ad, batches=2)
