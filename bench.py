@@ -44,10 +44,10 @@ METRIC_STREAM = "routes/sec over the whole stream (decode step + routing of the 
 ROUTE_DRAM_READ = {3: 67322880}
 # profiles/ncu_dram_route_summary_kernels_config3_full_batch.txt: the three kernels of the summary router on the full
 # batch (the traffic does not grow in proportion to the batch, so the figure is used for the full batch only)
-ROUTE_SUMMARY_DRAM_TRAFFIC = {(3, 65536): 67736576 + 349696 + 2059520 + 50737664 + 2790656}
+ROUTE_SUMMARY_DRAM_TRAFFIC = {(3, 65536): 67736576 + 295680 + 2358528 + 50721792 + 2772736}
 # warp instructions per arrival of pre_route_summaries (smsp__inst_executed.sum of the 2,048-arrival capture in
-# profiles/ncu_full_step_kernels_config3_2048_arrivals.txt: 1,062,765 / 2,048)
-ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL = {3: 1062765 / 2048}
+# profiles/ncu_full_step_kernels_config3_2048_arrivals.txt: 1,014,988 / 2,048)
+ROUTE_SUMMARY_WARP_INSTRUCTIONS_PER_ARRIVAL = {3: 1014988 / 2048}
 ROUTE_DRAM_WRITE_PER_ARRIVAL = {3: 679168 / 256}
 ANTICIPATE_DRAM_TRAFFIC = {3: 33812992 + 19587328}
 STEP_DRAM_TRAFFIC = {3: 33670144 + 67196928 + 9366528}
@@ -677,7 +677,8 @@ def route_summary_roofline(wl, index, t_route_ms, n_arrivals, clocks):
         "hbm_frac_of_captured_traffic": None if traffic is None else traffic / sec / 1e9 / hbm_peak,
         "limiter": "latency: arrivals are decided one after another by one warp (one warp reduction and some eight dependent "
                    "instructions each); neither a memory nor the instruction issue is saturated",
-        "note": "decisions are taken from two numbers per row instead of scanning the maps (identical decisions), by one block and one that builds its lists; "
+        "note": "decisions are taken from two numbers per row instead of scanning the maps (identical decisions), by one block"
+                f"{' and one that builds its lists' if i > 256 else ''}; "
                 "scan_equivalent_gbs is the literal formulation's 8 bytes per cell and arrival over time, a convenience "
                 "number that is not memory traffic; traffic = DRAM bytes of the call's kernels from the ncu capture of this "
                 f"batch ({kind} HBM peak {hbm_peak:.0f} GB/s for hbm_frac_of_captured_traffic)",

@@ -314,7 +314,8 @@ int pre_last_cuda_error(const pre_ctx* ctx);
  * the summary kernel when the shape fits it, the scanning kernel otherwise or when the summary kernel declines a batch, because
  * a value could leave its numbers or because the rows are such that the scanning kernel is faster), PRE_ROUTE_SCAN
  * (always the scanning kernel), PRE_ROUTE_SUMMARY (the summary kernel whenever its numbers hold the batch; PRE_ESIZE here when the
- * shape does not fit it).  Results do not depend on it. */
+ * shape does not fit it).  Results do not depend on it.  Beyond 256 instances the summary kernel is a cluster of two blocks: it starts when two
+ * SMs of one cluster are free at the same time. */
 #define PRE_ROUTE_AUTO    0
 #define PRE_ROUTE_SCAN    1
 #define PRE_ROUTE_SUMMARY 2
